@@ -152,13 +152,11 @@ static anpd_status model_make_plans(anpd_model* m) {
     m->plain_gemm = std::getenv("ANPD_PLAIN_GEMM") != nullptr;
     size_t ints = 0;
     int max_tiles = 0;
-    m->max_segs = 1;
     for (int k = 0; k < GK_COUNT; ++k) {
         ints += 2 * (size_t)m->plan[k].m_tiles;
         max_tiles = std::max(max_tiles, m->plan[k].m_tiles);
-        m->max_segs = std::max(m->max_segs, m->plan[k].max_segs);
     }
-    ints += 4 * (size_t)max_tiles + (size_t)GK_COUNT * max_tiles;
+    ints += 4 * (size_t)max_tiles + (size_t)GK_COUNT * max_tiles;                   // constants 1..4, then a table per projection
     std::vector<int> host(ints);
     CUDA_TRY(cudaMalloc((void**)&m->d_plan_tables, ints * sizeof(int)));
     size_t off = 0;
@@ -172,12 +170,12 @@ static anpd_status model_make_plans(anpd_model* m) {
     m->d_ones = m->d_plan_tables + off;
     for (int i = 0; i < max_tiles; ++i) host[off + i] = 1;
     m->d_const_segs[0] = m->d_const_segs[1] = m->d_ones;
-    for (int k = 2; k <= 3; ++k) {
+    for (int k = 2; k <= 4; ++k) {
         m->d_const_segs[k] = m->d_plan_tables + off + (size_t)(k - 1) * max_tiles;
         for (int i = 0; i < max_tiles; ++i) host[off + (size_t)(k - 1) * max_tiles + i] = k;
     }
     for (int k = 0; k < GK_COUNT; ++k) {
-        m->d_tail_segs[k] = m->d_plan_tables + off + (size_t)(3 + k) * max_tiles;
+        m->d_tail_segs[k] = m->d_plan_tables + off + (size_t)(4 + k) * max_tiles;
         m->tail_cfg[k] = -1;
     }
     CUDA_TRY(cudaMemcpy(m->d_plan_tables, host.data(), ints * sizeof(int), cudaMemcpyHostToDevice));
@@ -231,9 +229,8 @@ anpd_status anpd_model_create(const anpd_model_config* cfg, const void* const* w
     m->dkv = c.n_kv_heads * c.head_dim;
     m->nqkv = m->dq + 2 * m->dkv;
     const size_t d = c.d_model, F = c.d_ffn, V = c.vocab;
-    // GEMM weights are stored tile by tile (128 output rows x 64 inputs, 16 KB contiguous each, zero
-    // padded at ragged edges) so that every TMA box is one contiguous read; the embedding table stays
-    // row-major because it is only gathered.
+    // Projection weights are stored in the order the decode projections stream them (ClPlan, zero padded at ragged edges);
+    // the embedding table stays row-major because it is only gathered.
     {
         int dev = 0, sms = 0;
         if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
@@ -243,7 +240,14 @@ anpd_status anpd_model_create(const anpd_model_config* cfg, const void* const* w
         m->device = dev;
         const int shapes[GK_COUNT][2] = {{m->nqkv, c.d_model}, {c.d_model, m->dq}, {2 * c.d_ffn, c.d_model}, {c.d_model, c.d_ffn},
                                          {c.vocab, c.d_model}};
-        for (int k = 0; k < GK_COUNT; ++k) gemm_make_plan(&m->plan[k], shapes[k][0], shapes[k][1], sms);
+        const int kinds[GK_COUNT] = {CL_QKV, CL_RESID, CL_GU, CL_RESID, CL_LM}, ncl = cl_clusters();
+        if (ncl < 1) { delete m; return ANPD_ERR_CUDA; }
+        m->cl_all_fused = true;
+        for (int k = 0; k < GK_COUNT; ++k) {
+            gemm_make_plan(&m->plan[k], shapes[k][0], shapes[k][1], sms);
+            cl_make_plan(&m->cl[k], kinds[k], shapes[k][0], shapes[k][1], c.head_dim, c.d_ffn, ncl);
+            m->cl_all_fused = m->cl_all_fused && cl_fused(m->cl[k]);
+        }
         for (int k = 0; k < GK_COUNT; ++k) rr_make_plan(&m->rr[k], shapes[k][0], shapes[k][1], sms);
     }
     m->rr_slab = nullptr;
@@ -253,9 +257,8 @@ anpd_status anpd_model_create(const anpd_model_config* cfg, const void* const* w
     m->rr_ready = std::getenv("ANPD_RR") != nullptr;
     for (int k = 0; k < GK_COUNT; ++k)
         if (m->rr[k].mt > 2) m->rr_ready = false;      // a CTA's feature range must fit two 128-row MMA tiles (very large vocabularies do not)
-    const size_t b_embed = up256(V * d * 2), b_lm = up256(gemm_tiled_elems(m->plan[GK_LM]) * 2),
-                 b_qkv = up256(gemm_tiled_elems(m->plan[GK_QKV]) * 2), b_o = up256(gemm_tiled_elems(m->plan[GK_O]) * 2),
-                 b_gu = up256(gemm_tiled_elems(m->plan[GK_GU]) * 2), b_d = up256(gemm_tiled_elems(m->plan[GK_DOWN]) * 2),
+    const size_t b_embed = up256(V * d * 2), b_lm = cl_storage_bytes(m->cl[GK_LM]), b_qkv = cl_storage_bytes(m->cl[GK_QKV]),
+                 b_o = cl_storage_bytes(m->cl[GK_O]), b_gu = cl_storage_bytes(m->cl[GK_GU]), b_d = cl_storage_bytes(m->cl[GK_DOWN]),
                  b_norm = up256(d * 4);
     m->slab_bytes = b_embed + b_lm + b_norm + c.n_layers * (b_qkv + b_o + b_gu + b_d + 2 * b_norm);
     if (cudaMalloc(&m->slab, m->slab_bytes) != cudaSuccess) { cudaGetLastError(); delete m; return ANPD_ERR_OOM; }
@@ -265,6 +268,15 @@ anpd_status anpd_model_create(const anpd_model_config* cfg, const void* const* w
         rr_total += rr_bytes[k] * (k == GK_LM ? 1 : (size_t)c.n_layers);
     }
     if (m->rr_ready && cudaMalloc(&m->rr_slab, rr_total) != cudaSuccess) { cudaGetLastError(); cudaFree(m->slab); delete m; return ANPD_ERR_OOM; }
+    // ANPD_STEP_KERNEL=1: the persistent step kernel streams a copy of the projections in block storage
+    size_t block_bytes[GK_COUNT], block_total = 0;
+    for (int k = 0; k < GK_COUNT; ++k) {
+        block_bytes[k] = up256(gemm_tiled_elems(m->plan[k]) * 2);
+        block_total += block_bytes[k] * (k == GK_LM ? 1 : (size_t)c.n_layers);
+    }
+    const bool blocks = std::getenv("ANPD_STEP_KERNEL") != nullptr;
+    m->block_slab = nullptr; m->block_lm = nullptr;
+    if (blocks && cudaMalloc(&m->block_slab, block_total) != cudaSuccess) { cudaGetLastError(); cudaFree(m->rr_slab); cudaFree(m->slab); delete m; return ANPD_ERR_OOM; }
     m->streamed_bytes = 2.0 * ((double)c.n_layers * ((double)m->nqkv * d + (double)d * m->dq + 3.0 * F * d) + (double)V * d);
 
     char* p = (char*)m->slab;
@@ -275,17 +287,19 @@ anpd_status anpd_model_create(const anpd_model_config* cfg, const void* const* w
     // staging for host-side sources: the largest matrix in its source type
     void* stage = nullptr;
     const size_t max_elems = std::max(std::max((size_t)V * d, F * d), std::max((size_t)m->dq * d, d * F));
-    if (!dev && cudaMalloc(&stage, max_elems * (bf ? 2 : 4)) != cudaSuccess) { cudaGetLastError(); cudaFree(m->rr_slab); cudaFree(m->slab); delete m; return ANPD_ERR_OOM; }
+    if (!dev && cudaMalloc(&stage, max_elems * (bf ? 2 : 4)) != cudaSuccess) { cudaGetLastError(); cudaFree(m->block_slab); cudaFree(m->rr_slab); cudaFree(m->slab); delete m; return ANPD_ERR_OOM; }
+    if (blocks && cudaMemsetAsync(m->block_slab, 0, block_total, st) != cudaSuccess) rc = ANPD_ERR_CUDA;
     if (cudaMemsetAsync(m->slab, 0, m->slab_bytes, st) != cudaSuccess) rc = ANPD_ERR_CUDA;
     if (m->rr_ready && cudaMemsetAsync(m->rr_slab, 0, rr_total, st) != cudaSuccess) rc = ANPD_ERR_CUDA;
     unsigned char* rp = (unsigned char*)m->rr_slab;     // next free byte of the row-range storage
+    unsigned char* bp = (unsigned char*)m->block_slab;  // next free byte of the block storage
     auto put = [&](const void* src, size_t n, bool as_bf16, size_t bytes) -> void* {
         void* dst = p;
         p += bytes;
         if (rc == ANPD_OK) rc = upload(dst, src, n, as_bf16, bf, dev, st, tmp, nullptr, 0);
         return dst;
     };
-    // rows [row_off, row_off + rows) of a tiled [*, K] matrix at dst, and of its row-range copy at rdst
+    // rows [row_off, row_off + rows) of a stored [*, K] matrix at dst, of its row-range copy at rdst and its block copy at bp
     auto put_tiled = [&](int kind, const void* src, int rows, int K, int row_off, void* dst, unsigned char* rdst) {
         if (rc != ANPD_OK) return;
         const void* dsrc = src;
@@ -294,7 +308,8 @@ anpd_status anpd_model_create(const anpd_model_config* cfg, const void* const* w
                 cudaStreamSynchronize(st) != cudaSuccess) { anpd_note_cuda_error(cudaGetLastError(), __FILE__, __LINE__); rc = ANPD_ERR_CUDA; return; }
             dsrc = stage;
         }
-        rc = gemm_retile_enqueue(m->plan[kind], dsrc, !bf, rows, row_off, (bf16*)dst, st);
+        rc = cl_retile_enqueue(m->cl[kind], dsrc, !bf, rows, row_off, (unsigned char*)dst, st);
+        if (rc == ANPD_OK && blocks) rc = gemm_retile_enqueue(m->plan[kind], dsrc, !bf, rows, row_off, (bf16*)bp, st);
         if (rc == ANPD_OK && m->rr_ready) {
             const int map = kind == GK_QKV ? RR_MAP_HEADS : kind == GK_GU ? RR_MAP_GATE_UP : RR_MAP_IDENTITY;
             rc = rr_retile_enqueue(m->rr[kind], dsrc, !bf, rows, row_off, map, c.head_dim, c.d_ffn, rdst, st);
@@ -305,42 +320,49 @@ anpd_status anpd_model_create(const anpd_model_config* cfg, const void* const* w
     m->embed = (const bf16*)put(weights[t++], V * d, true, b_embed);
     m->layers.resize(c.n_layers);
     m->rr_layers.resize(c.n_layers);
+    m->block_layers.resize(blocks ? c.n_layers : 0);
+    auto block_next = [&](int kind) { const bf16* at = (const bf16*)bp; if (blocks) bp += block_bytes[kind]; return at; };
     for (int l = 0; l < c.n_layers; ++l) {
         LayerW& w = m->layers[l];
         anpd_model::LayerRR& r = m->rr_layers[l];
         w.attn_norm = (const float*)put(weights[t++], d, false, b_norm);
         // q, k and v rows form one matrix so that one GEMM produces all three
-        w.wqkv = (const bf16*)p;
+        w.wqkv = (const unsigned char*)p;
         r.wqkv = rp;
         put_tiled(GK_QKV, weights[t++], m->dq, (int)d, 0, p, rp);
         put_tiled(GK_QKV, weights[t++], m->dkv, (int)d, m->dq, p, rp);
         put_tiled(GK_QKV, weights[t++], m->dkv, (int)d, m->dq + m->dkv, p, rp);
+        if (blocks) m->block_layers[l].wqkv = block_next(GK_QKV);
         p += b_qkv; rp += rr_bytes[GK_QKV];
-        w.wo = (const bf16*)p;
+        w.wo = (const unsigned char*)p;
         r.wo = rp;
         put_tiled(GK_O, weights[t++], (int)d, m->dq, 0, p, rp);
+        if (blocks) m->block_layers[l].wo = block_next(GK_O);
         p += b_o; rp += rr_bytes[GK_O];
         w.ffn_norm = (const float*)put(weights[t++], d, false, b_norm);
-        w.wgu = (const bf16*)p;
+        w.wgu = (const unsigned char*)p;
         r.wgu = rp;
         put_tiled(GK_GU, weights[t++], (int)F, (int)d, 0, p, rp);
         put_tiled(GK_GU, weights[t++], (int)F, (int)d, (int)F, p, rp);
+        if (blocks) m->block_layers[l].wgu = block_next(GK_GU);
         p += b_gu; rp += rr_bytes[GK_GU];
-        w.wd = (const bf16*)p;
+        w.wd = (const unsigned char*)p;
         r.wd = rp;
         put_tiled(GK_DOWN, weights[t++], (int)d, (int)F, 0, p, rp);
+        if (blocks) m->block_layers[l].wd = block_next(GK_DOWN);
         p += b_d; rp += rr_bytes[GK_DOWN];
     }
     m->final_norm = (const float*)put(weights[t++], d, false, b_norm);
-    m->lm_head = (const bf16*)p;
+    m->lm_head = (const unsigned char*)p;
     m->rr_lm = rp;
     put_tiled(GK_LM, weights[t++], (int)V, (int)d, 0, p, rp);
+    m->block_lm = block_next(GK_LM);
     p += b_lm;
     if (rc == ANPD_OK && cudaStreamSynchronize(st) != cudaSuccess) { anpd_note_cuda_error(cudaGetLastError(), __FILE__, __LINE__); rc = ANPD_ERR_CUDA; }
     if (stage) cudaFree(stage);
     m->d_plan_tables = nullptr;
     if (rc == ANPD_OK) rc = model_make_plans(m);
-    if (rc != ANPD_OK) { cudaFree(m->d_plan_tables); cudaFree(m->rr_slab); cudaFree(m->slab); delete m; return rc; }
+    if (rc != ANPD_OK) { cudaFree(m->d_plan_tables); cudaFree(m->block_slab); cudaFree(m->rr_slab); cudaFree(m->slab); delete m; return rc; }
     *out = m;
     return ANPD_OK;
 }
@@ -349,6 +371,7 @@ anpd_status anpd_model_destroy(anpd_model* m) {
     if (!m) return ANPD_ERR_ARG;
     cudaStreamSynchronize(m->stream);
     cudaFree(m->d_plan_tables);
+    cudaFree(m->block_slab);
     cudaFree(m->rr_slab);
     cudaFree(m->slab);
     delete m;
@@ -391,11 +414,11 @@ anpd_status anpd_kv_create(const anpd_model* cm, int max_len, int batch, int shu
     ws.prefill_rows = std::min(PREFILL_ROWS_MAX, (kv->max_len + 255) / 256 * 256);
     ws.r_max = std::max(ws.prefill_rows, batch * ANPD_ROWS);
     ws.n_max_out = (std::max(std::max(m->nqkv, 2 * c.d_ffn), std::max(c.d_model, c.vocab)) + 127) / 128 * 128;
-    ws.splits_max = m->max_segs;
     ws.amax_blocks = (c.vocab + 1023) / 1024;
     const size_t R = ws.r_max, d = c.d_model, F = c.d_ffn, V = c.vocab, hd = c.head_dim, half = hd / 2;
     const size_t pool = (size_t)c.n_layers * kv->total_pages * c.n_kv_heads * KV_PAGE * hd * 2;
     const size_t n_part = (size_t)R * c.n_q_heads * kv->pages_per_seq;
+    const int S = batch * ANPD_ROWS;                   // rows of a decode step
     struct Item { void** ptr; size_t bytes; };
     std::vector<Item> items = {
         {(void**)&kv->kpool, pool}, {(void**)&kv->vpool, pool},
@@ -408,8 +431,7 @@ anpd_status anpd_kv_create(const anpd_model* cm, int max_len, int batch, int shu
         {(void**)&ws.x, R * d * 4}, {(void**)&ws.h_hi, R * d * 2}, {(void**)&ws.h_lo, R * d * 2},
         {(void**)&ws.ao_hi, R * m->dq * 2}, {(void**)&ws.ao_lo, R * m->dq * 2},
         {(void**)&ws.act_hi, R * F * 2}, {(void**)&ws.act_lo, R * F * 2},
-        // decode steps leave up to splits_max partial sums per output, prompt passes up to three (their cut along K)
-        {(void**)&ws.part, std::max((size_t)ws.splits_max * batch * ANPD_ROWS, 3 * R) * ws.n_max_out * 4},
+        {(void**)&ws.part, 3 * R * ws.n_max_out * 4},    // prompt passes leave up to three partial sums per output (their cut along K)
         {(void**)&ws.q_hi, R * m->dq * 2}, {(void**)&ws.q_lo, R * m->dq * 2},
         {(void**)&ws.attn_m, n_part * 4}, {(void**)&ws.attn_l, n_part * 4}, {(void**)&ws.attn_o, n_part * hd * 4},
         {(void**)&ws.logits, (size_t)batch * ANPD_ROWS * V * 4},
@@ -417,6 +439,10 @@ anpd_status anpd_kv_create(const anpd_model* cm, int max_len, int batch, int shu
         {(void**)&ws.gemm_err, 256}, {(void**)&kv->loop_steps_left, 256},
         {(void**)&ws.img_h, act_img_bytes(c.d_model)}, {(void**)&ws.img_h2, act_img_bytes(c.d_model)},
         {(void**)&ws.img_ao, act_img_bytes(m->dq)}, {(void**)&ws.img_act, act_img_bytes(c.d_ffn)},
+        {(void**)&ws.ci_h, cl_img_bytes(S, c.d_model)}, {(void**)&ws.ci_h2, cl_img_bytes(S, c.d_model)},
+        {(void**)&ws.ci_ao, cl_img_bytes(S, m->dq)}, {(void**)&ws.ci_act, cl_img_bytes(S, c.d_ffn)},
+        {(void**)&ws.ss_cl_a, (size_t)cl_parts(m->cl[GK_DOWN]) * ANPD_ROWS * 4}, {(void**)&ws.ss_cl_b, (size_t)cl_parts(m->cl[GK_O]) * ANPD_ROWS * 4},
+        {(void**)&ws.amax_val_cl, (size_t)cl_parts(m->cl[GK_LM]) * ANPD_ROWS * 4}, {(void**)&ws.amax_idx_cl, (size_t)cl_parts(m->cl[GK_LM]) * ANPD_ROWS * 4},
         {(void**)&ws.ss_a, (size_t)m->num_sms * ANPD_ROWS * 4}, {(void**)&ws.ss_b, (size_t)m->num_sms * ANPD_ROWS * 4},
         {(void**)&ws.amax_val_rr, (size_t)m->num_sms * ANPD_ROWS * 4}, {(void**)&ws.amax_idx_rr, (size_t)m->num_sms * ANPD_ROWS * 4},
     };
@@ -431,20 +457,14 @@ anpd_status anpd_kv_create(const anpd_model* cm, int max_len, int batch, int shu
     if (cudaMallocHost((void**)&kv->h_seq, pinned_bytes) != cudaSuccess) { cudaGetLastError(); cudaFree(kv->slab); delete kv; return ANPD_ERR_OOM; }
     kv->h_small = (int*)((char*)kv->h_seq + sizeof(SeqState) * (size_t)batch);
 
-    // TMA views of the GEMM inputs: decode rows (batch * 8) and prefill rows, each padded to the MMA's N
+    // TMA views of the inputs of the prompt passes' projections (rows beyond the tensor's extent are zero-filled by the copy engine)
     {
-        const int mode_rows[2] = {batch * ANPD_ROWS, ws.prefill_rows};
         anpd_status rc = ANPD_OK;
-        for (int md = 0; md < 2 && rc == ANPD_OK; ++md) {
-            const int rows = mode_rows[md], nb = md == 0 ? (rows + 15) / 16 * 16 : 128;
-            ws.nb[md] = nb;
-            struct { CUtensorMap* maps; const bf16* hi; const bf16* lo; int K; } bufs[3] = {
-                {ws.map_h[md], ws.h_hi, ws.h_lo, c.d_model}, {ws.map_ao[md], ws.ao_hi, ws.ao_lo, m->dq}, {ws.map_act[md], ws.act_hi, ws.act_lo, c.d_ffn}};
-            for (auto& bdesc : bufs) {
-                // rows beyond the tensor's extent are zero-filled by the copy engine
-                if (rc == ANPD_OK) rc = make_tmap_bf16(&bdesc.maps[0], bdesc.hi, rows, bdesc.K, nb, false);
-                if (rc == ANPD_OK) rc = make_tmap_bf16(&bdesc.maps[1], bdesc.lo, rows, bdesc.K, nb, false);
-            }
+        struct { CUtensorMap* maps; const bf16* hi; const bf16* lo; int K; } bufs[3] = {
+            {ws.map_h, ws.h_hi, ws.h_lo, c.d_model}, {ws.map_ao, ws.ao_hi, ws.ao_lo, m->dq}, {ws.map_act, ws.act_hi, ws.act_lo, c.d_ffn}};
+        for (auto& bdesc : bufs) {
+            if (rc == ANPD_OK) rc = make_tmap_bf16(&bdesc.maps[0], bdesc.hi, ws.prefill_rows, bdesc.K, 128, false);
+            if (rc == ANPD_OK) rc = make_tmap_bf16(&bdesc.maps[1], bdesc.lo, ws.prefill_rows, bdesc.K, 128, false);
         }
         if (rc != ANPD_OK) { cudaFreeHost(kv->h_seq); cudaFree(kv->slab); delete kv; return rc; }
     }
@@ -452,11 +472,18 @@ anpd_status anpd_kv_create(const anpd_model* cm, int max_len, int batch, int shu
     // TMA views of the K and V pools for the tensor-core attention: every page of every layer and kv head is 128 rows of hd
     kv->attn_tc = (c.head_dim == 128) && std::getenv("ANPD_ATTN_MMA_SYNC") == nullptr;
     kv->attn_pf = std::getenv("ANPD_ATTN_PROMPT_TILE16") == nullptr;
+    if (c.head_dim == 64) {
+        const long long page_heads = (long long)c.n_layers * kv->total_pages * c.n_kv_heads;
+        anpd_status rc = page_heads * KV_PAGE < (1ll << 31) ? ANPD_OK : ANPD_ERR_CAPACITY;
+        if (rc == ANPD_OK) rc = make_tmap_bf16(&kv->map_k, kv->kpool, (int)(page_heads * KV_PAGE), c.head_dim, KV_PAGE, true);
+        if (rc == ANPD_OK) rc = make_tmap_bf16(&kv->map_v, kv->vpool, (int)(page_heads * c.head_dim), KV_PAGE, c.head_dim, true);
+        if (rc != ANPD_OK) { cudaFreeHost(kv->h_seq); cudaFree(kv->slab); delete kv; return rc; }
+    }
     if (kv->attn_tc) {
         const long long pool_rows = (long long)c.n_layers * kv->total_pages * c.n_kv_heads * KV_PAGE;
         anpd_status rc = pool_rows < (1ll << 31) ? ANPD_OK : ANPD_ERR_CAPACITY;
         if (rc == ANPD_OK) rc = make_tmap_bf16(&kv->map_k, kv->kpool, (int)pool_rows, c.head_dim, KV_PAGE, true);
-        if (rc == ANPD_OK) rc = make_tmap_bf16(&kv->map_v, kv->vpool, (int)pool_rows, c.head_dim, KV_PAGE, true);
+        if (rc == ANPD_OK) rc = make_tmap_bf16(&kv->map_v, kv->vpool, (int)pool_rows, KV_PAGE, c.head_dim, true);
         if (rc == ANPD_OK) rc = make_tmap_bf16(&ws.map_q[0], ws.q_hi, ws.r_max, m->dq, 128, false);
         if (rc == ANPD_OK) rc = make_tmap_bf16(&ws.map_q[1], ws.q_lo, ws.r_max, m->dq, 128, false);
         if (rc != ANPD_OK) { cudaFreeHost(kv->h_seq); cudaFree(kv->slab); delete kv; return rc; }
@@ -578,7 +605,7 @@ static anpd_status read_seqs(anpd_kv* kv) {
     CUDA_TRY(cudaStreamSynchronize(kv->m->stream));
     for (int b = 0; b < kv->batch; ++b) { kv->h_kv_len[b] = kv->h_seq[b].kv_len; kv->h_len_stale[b] = 0; }
     if (*h_err != 0) {
-        std::snprintf(g_last_error, sizeof(g_last_error), "a kernel gave up waiting on a barrier (code %d: 201 GEMM, 202 attention, 204 step kernel)", *h_err);
+        std::snprintf(g_last_error, sizeof(g_last_error), "a kernel gave up waiting on a barrier (code %d: 201 GEMM, 202 attention, 204 step kernel, 205 prompt GEMM, 206 prompt attention, 207 decode projection, 208 decode attention)", *h_err);
         return ANPD_ERR_CUDA;
     }
     return ANPD_OK;
@@ -1025,16 +1052,69 @@ static anpd_status debug_gemm_row_range(const uint16_t* w_bf16, int N, int K, co
     return rc;
 }
 
+// The product through the decode projection (a cluster of CTAs per range of features), plain epilogue.
+static anpd_status debug_gemm_cluster(const uint16_t* w_bf16, int N, int K, const float* a, int rows, float* out) {
+    ClPlan plan;
+    const int ncl = cl_clusters();
+    if (ncl < 1) return ANPD_ERR_CUDA;
+    cl_make_plan(&plan, CL_RAW, N, K, 0, 0, ncl);
+    const size_t wb = up256(cl_storage_bytes(plan)), ib = up256(cl_img_bytes(rows, K)), sb = up256((size_t)N * K * 2),
+                 ab = up256((size_t)rows * K * 4), ob = up256((size_t)CL_CTAS * rows * N * 4);
+    const int parts = rows == ANPD_ROWS && cl_fused(plan) ? 1 : CL_CTAS;
+    char* slab = nullptr;
+    if (cudaMalloc((void**)&slab, wb + ib + sb + ab + ob + 256) != cudaSuccess) { cudaGetLastError(); return ANPD_ERR_OOM; }
+    unsigned char* dW = (unsigned char*)slab;
+    unsigned char* dimg = dW + wb;
+    void* dsrc = dimg + ib;
+    float* da = (float*)((char*)dsrc + sb);
+    float* dout = (float*)((char*)da + ab);
+    int* derr = (int*)((char*)dout + ob);
+    auto body = [&]() -> anpd_status {
+        CUDA_TRY(cudaMemset(slab, 0, wb + ib));
+        CUDA_TRY(cudaMemset(dout, 0, ob + 256));
+        CUDA_TRY(cudaMemcpy(dsrc, w_bf16, (size_t)N * K * 2, cudaMemcpyHostToDevice));
+        CUDA_TRY(cudaMemcpy(da, a, (size_t)rows * K * 4, cudaMemcpyHostToDevice));
+        ANPD_TRY(cl_retile_enqueue(plan, dsrc, false, N, 0, dW, 0));
+        ANPD_TRY(cl_image_enqueue(da, rows, K, dimg, 0));
+        CUDA_TRY(cudaDeviceSynchronize());
+        if (rows == ANPD_ROWS && cl_fused(plan)) {
+            ClEpilogue e;
+            e.out = dout;
+            ANPD_TRY(cl_enqueue(plan, dW, dimg, e, derr, 0, nullptr));
+        } else {
+            ANPD_TRY(cl_partial_enqueue(plan, dW, dimg, rows, dout, (size_t)rows * N, N, nullptr, nullptr, 0, 0, derr, 0, nullptr));
+        }
+        CUDA_TRY(cudaDeviceSynchronize());
+        int err = 0;
+        CUDA_TRY(cudaMemcpy(&err, derr, 4, cudaMemcpyDeviceToHost));
+        if (err) { std::snprintf(g_last_error, sizeof(g_last_error), "GEMM kernel gave up waiting (code %d)", err); return ANPD_ERR_CUDA; }
+        std::vector<float> part((size_t)parts * rows * N);
+        CUDA_TRY(cudaMemcpy(part.data(), dout, part.size() * 4, cudaMemcpyDeviceToHost));
+        for (size_t i = 0; i < (size_t)rows * N; ++i) {
+            float acc = part[i];
+            for (int k = 1; k < parts; ++k) acc += part[(size_t)k * rows * N + i];
+            out[i] = acc;
+        }
+        return ANPD_OK;
+    };
+    const anpd_status rc = body();
+    cudaFree(slab);
+    return rc;
+}
+
 anpd_status anpd_debug_gemm(const uint16_t* w_bf16, int N, int K, const float* a, int rows, float* out, int plain) {
     if (!w_bf16 || !a || !out || N < 1 || K < 8 || K % 8 || rows < 8 || rows % 8 || rows > 128) return ANPD_ERR_ARG;
     if (plain == 2 && rows != ANPD_ROWS) return ANPD_ERR_ARG;
     if (!have_device()) return ANPD_ERR_CUDA;
     if (plain == 2) return debug_gemm_row_range(w_bf16, N, K, a, out);
+    if (plain == 3) return debug_gemm_cluster(w_bf16, N, K, a, rows, out);
     int dev = 0, sms = 0;
     CUDA_TRY(cudaGetDevice(&dev));
     CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     GemmPlan plan;
     gemm_make_plan(&plan, N, K, sms);
+    ClPlan rows_plan;                                   // the plain kernel reads the decode projections' storage
+    cl_make_plan(&rows_plan, CL_RAW, N, K, 0, 0, 32);
     const int NB = (rows + 15) / 16 * 16;
     const int segs = plain ? 1 : plan.max_segs;
     std::vector<uint16_t> hi((size_t)rows * K), lo((size_t)rows * K);
@@ -1044,7 +1124,7 @@ anpd_status anpd_debug_gemm(const uint16_t* w_bf16, int N, int K, const float* a
         float h; std::memcpy(&h, &u, 4);
         lo[i] = f32_to_bf16_host(a[i] - h);
     }
-    const size_t wb = up256(gemm_tiled_elems(plan) * 2), ab = up256((size_t)rows * K * 2), pb = up256((size_t)segs * rows * N * 4),
+    const size_t wb = std::max(up256(gemm_tiled_elems(plan) * 2), up256(cl_storage_bytes(rows_plan))), ab = up256((size_t)rows * K * 2), pb = up256((size_t)segs * rows * N * 4),
                  tb = up256((size_t)plan.m_tiles * 4), sb = up256((size_t)N * K * 2);
     char* slab = nullptr;
     if (cudaMalloc((void**)&slab, wb + 2 * ab + pb + tb + 256 + sb) != cudaSuccess) { cudaGetLastError(); return ANPD_ERR_OOM; }
@@ -1059,12 +1139,13 @@ anpd_status anpd_debug_gemm(const uint16_t* w_bf16, int N, int K, const float* a
         CUDA_TRY(cudaMemset(slab, 0, wb));
         CUDA_TRY(cudaMemset(slab + wb + 2 * ab, 0, pb + tb + 256));
         CUDA_TRY(cudaMemcpy(dsrc, w_bf16, (size_t)N * K * 2, cudaMemcpyHostToDevice));
-        ANPD_TRY(gemm_retile_enqueue(plan, dsrc, false, N, 0, dW, 0));
+        if (plain) ANPD_TRY(cl_retile_enqueue(rows_plan, dsrc, false, N, 0, (unsigned char*)dW, 0));
+        else ANPD_TRY(gemm_retile_enqueue(plan, dsrc, false, N, 0, dW, 0));
         CUDA_TRY(cudaMemcpy(dhi, hi.data(), hi.size() * 2, cudaMemcpyHostToDevice));
         CUDA_TRY(cudaMemcpy(dlo, lo.data(), lo.size() * 2, cudaMemcpyHostToDevice));
         CUDA_TRY(cudaMemcpy(dfirst, plan.first_cta.data(), (size_t)plan.m_tiles * 4, cudaMemcpyHostToDevice));
         if (plain) {
-            ANPD_TRY(gemm_plain_enqueue(plan, dW, dhi, dlo, rows, dpart, N, 0, nullptr));
+            ANPD_TRY(gemm_plain_enqueue(rows_plan, (const unsigned char*)dW, dhi, dlo, rows, dpart, N, 0, nullptr));
         } else {
             CUtensorMap mh, ml;
             ANPD_TRY(make_tmap_bf16(&mh, dhi, rows, K, NB, false));

@@ -1,0 +1,435 @@
+// Attention of a decode step, complete in one kernel: the 8 rows of a sequence's step (x the query heads of one kv head) against
+// the paged cache, softmax, and the result as the O projection's operand image.
+//
+// What bounds it: the cache's pages from HBM at long contexts; at short ones a memory round trip, the merge and the launch.  The
+// pages of one kv head of one sequence are dealt to VR shares: share v takes the pages p with (p / PG) mod VR == v.  A step of few
+// (sequence, head) pairs gives every share a CTA of its own, VR of them forming a cluster; a step of many has one CTA take the
+// shares one after the other.  A producer thread brings pages in through a ring of TMA copies (those no kernel of this step
+// writes before the dependency wait); sixteen warps compute, each on 16 keys at a time: block b of a share belongs to key slot
+// b mod KW and to the MT warps of that slot, one per 16-row tile of query vectors.
+//
+// Order.  A slot takes its blocks in ascending order with a running maximum; the slots of a share are merged in slot order, the
+// shares in share order, each into the running result.  All of it depends on absolute key positions and head counts only, and a
+// masked key contributes an exact zero, so a row's result does not depend on the rows it shares the step with, on the batch, on
+// who computes a share, or on how far the cache reaches behind the row.
+//
+// mma.sync m16n8k16 (bf16, fp32 sums): with 8 to 64 query vectors per kv head the products are small beside the loads.  Queries
+// and weights enter as two bf16 terms; with one query head per kv head the two terms of the 8 rows are the tile's 16 rows.
+#include "internal.h"
+#include "tc_ptx.cuh"
+
+#include <math_constants.h>
+
+#include <algorithm>
+
+typedef __nv_bfloat16 bf16;
+
+namespace {
+
+using namespace tc;
+
+constexpr int AD_WARPS = 16;             // compute warps; one more loads
+constexpr int AD_THREADS = 32 * (AD_WARPS + 1);
+constexpr int AD_COMPUTE = 32 * AD_WARPS;
+constexpr int AD_KEYS = 16;              // keys per block
+constexpr int AD_MAX_STAGES = 6;
+constexpr int AD_ERR_TIMEOUT = 208;
+
+template <int HD, int G> struct AdCfg {
+    static constexpr bool STACK = G == 1;                    // hi and lo terms of the 8 vectors share a tile
+    static constexpr int NV = STACK ? 8 : 16;                // query vectors per tile
+    static constexpr int Q = 8 * G;                          // query vectors per kv head
+    static constexpr int MT = Q / NV;                        // tiles (= warps per key slot)
+    static constexpr int KW = AD_WARPS / MT;                 // key slots of a share: 16, 16, 8, 4
+    static constexpr int PG = KW > 8 ? 2 : 1;                // neighbouring pages of a share
+    static constexpr int VR = G <= 2 ? 4 : 8;                // shares
+    static constexpr int VO = Q / VR;                        // vectors a CTA of a cluster finishes
+    static constexpr int OP = HD + 4;                        // padded row
+    static constexpr int QP = HD * 2 + 16;                   // bytes per staged query row
+    static constexpr int QROWS = STACK ? 16 : 32 * MT;
+    static constexpr int V4 = HD / 4;
+    static constexpr int ITEMS = (Q * V4 + AD_COMPUTE - 1) / AD_COMPUTE;      // 4-dimension pieces of the result per thread
+    static constexpr int PAGE_BYTES = 2 * KV_PAGE * HD * 2;  // K and V^T
+    static constexpr int REST = 1024 + AD_WARPS * NV * OP * 4 + Q * HD * 4 + 2 * AD_WARPS * NV * 4 + 2 * Q * 4 + QROWS * QP;
+    static constexpr int STAGES_MAX = (225 * 1024 - REST) / PAGE_BYTES;
+    static constexpr int STAGES = STAGES_MAX < AD_MAX_STAGES ? STAGES_MAX : AD_MAX_STAGES;
+    static constexpr size_t SMEM = (size_t)STAGES * PAGE_BYTES + REST;
+};
+
+struct AdArgs {
+    const bf16 *q_hi, *q_lo;
+    const int *page_table, *row_pos, *row_seq, *row_slot, *hole_lo, *hole_hi;      // row_slot and the holes: null outside two-candidate steps
+    int pages_per_seq, Hkv, rows, layer_page0, cluster;       // cluster: VR or 1
+    unsigned char* img;
+    int* err;
+};
+
+__device__ __forceinline__ void ad_mma(float* c, const uint32_t* a, uint32_t b0, uint32_t b1) {
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ void ad_ldm4(uint32_t addr, uint32_t* r) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ uint32_t ad_split(float x, float y, uint32_t& lo) {
+    const bf16 hx = __float2bfloat16_rn(x), hy = __float2bfloat16_rn(y);
+    const bf16 lx = __float2bfloat16_rn(x - __bfloat162float(hx)), ly = __float2bfloat16_rn(y - __bfloat162float(hy));
+    lo = (uint32_t)__bfloat16_as_ushort(lx) | ((uint32_t)__bfloat16_as_ushort(ly) << 16);
+    return (uint32_t)__bfloat16_as_ushort(hx) | ((uint32_t)__bfloat16_as_ushort(hy) << 16);
+}
+__device__ __forceinline__ uint32_t ad_map(const void* p, uint32_t cta) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_u32(p)), "r"(cta));
+    return r;
+}
+__device__ __forceinline__ void ad_bar() { asm volatile("bar.sync 1, %0;" ::"n"(AD_COMPUTE) : "memory"); }
+
+// a part (maximum pm, sum pl, values p) into the running result
+__device__ __forceinline__ void ad_fold(float& m, float& l, float4& a, float pm, float pl, float4 p) {
+    const float mn = fmaxf(m, pm);
+    const float so = m == -CUDART_INF_F ? 0.0f : exp2f(m - mn), sp = pm == -CUDART_INF_F ? 0.0f : exp2f(pm - mn);
+    a.x = fmaf(p.x, sp, a.x * so); a.y = fmaf(p.y, sp, a.y * so); a.z = fmaf(p.z, sp, a.z * so); a.w = fmaf(p.w, sp, a.w * so);
+    l = fmaf(pl, sp, l * so);
+    m = mn;
+}
+
+template <int HD, int G>
+__global__ void __launch_bounds__(AD_THREADS, 1) attn_dec_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v, const AdArgs g) {
+    typedef AdCfg<HD, G> Cfg;
+    constexpr bool STACK = Cfg::STACK;
+    constexpr int NV = Cfg::NV, MT = Cfg::MT, KW = Cfg::KW, PG = Cfg::PG, VR = Cfg::VR, VO = Cfg::VO, OP = Cfg::OP, QP = Cfg::QP, V4 = Cfg::V4;
+    constexpr int KS = HD / 16, DT = HD / 8, NR = STACK ? 1 : 2, STAGES = Cfg::STAGES;      // NR: query vectors per thread
+    constexpr int KV_BYTES = KV_PAGE * HD * 2;
+    extern __shared__ __align__(1024) unsigned char ad_smem[];
+    __shared__ uint64_t full_k[STAGES], full_v[STAGES], empty[STAGES];
+    __shared__ int abort_flag, s_issued;
+    unsigned char* ring = ad_smem + ((1024u - (smem_u32(ad_smem) & 1023u)) & 1023u);
+    float* sm_o = (float*)(ring + (size_t)STAGES * Cfg::PAGE_BYTES);       // [warp][NV][OP]
+    float* recv = sm_o + AD_WARPS * NV * OP;                // cluster: [share][VO][HD], the shares of this CTA's vectors
+    float* sm_m = recv + Cfg::Q * HD;                       // [warp][NV]
+    float* sm_l = sm_m + AD_WARPS * NV;
+    float* rc_m = sm_l + AD_WARPS * NV;                     // [share][VO]
+    float* rc_l = rc_m + Cfg::Q;
+    unsigned char* Qs = (unsigned char*)(rc_l + Cfg::Q);
+
+    pdl_trigger();
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");          // waited for before the first remote store: every CTA runs then
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int rank = blockIdx.x, kvh = blockIdx.y, r0 = blockIdx.z * ANPD_ROWS;
+    const int v_lo = g.cluster == 1 ? 0 : rank, v_hi = g.cluster == 1 ? VR : rank + 1;       // this CTA's shares
+    // The row plan is older than the kernel before this one (the embedding kernel lets its successors start only after its own
+    // dependency wait), so it may be read at once; so may pages below the first position this launch writes - the group's own
+    // first, or the first of all rows where they are one sequence's (a prompt as short as a step of the batch).
+    const int seq = g.row_seq[r0];
+    const int first_new = g.row_pos[gridDim.z > 1 && g.row_seq[0] == g.row_seq[ANPD_ROWS] ? 0 : r0];
+    const int pos_lo = g.row_pos[r0], pos_hi = (g.row_slot ? g.row_slot : g.row_pos)[r0 + ANPD_ROWS - 1];
+    const int n_pages = pos_hi / KV_PAGE + 1;
+    volatile int* abortp = &abort_flag;
+
+    if (warp == AD_WARPS) {
+        if (elect_one()) {
+            abort_flag = 0; s_issued = 0;
+#pragma unroll
+            for (int s = 0; s < STAGES; ++s) { mbar_init(&full_k[s], 1); mbar_init(&full_v[s], 1); mbar_init(&empty[s], PG == 2 ? AD_WARPS / 2 : AD_WARPS); }
+            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        }
+        __syncwarp();
+    }
+    __syncthreads();
+
+    if (warp == AD_WARPS) {
+        // ---------------- pages ----------------
+        if (elect_one()) {
+            const uint64_t pol = policy_evict_first();
+            const int* pages = g.page_table + (size_t)seq * g.pages_per_seq;
+            int stage = 0, count = 0;
+            uint32_t phase = 1;
+            bool waited = false, ok = true;
+            for (int v = v_lo; v < v_hi && ok; ++v)
+                for (int p0 = v * PG; p0 < n_pages && ok; p0 += VR * PG)
+                    for (int p = p0; p < min(p0 + PG, n_pages); ++p) {
+                        if (!waited && (p + 1) * KV_PAGE > first_new) { pdl_wait(); waited = true; }       // holds rows the kernel before writes
+                        if (count >= STAGES) ok = mbar_wait(&empty[stage], phase, abortp);
+                        if (!ok) break;
+                        const int row = (g.layer_page0 + pages[p]) * g.Hkv + kvh;
+                        unsigned char* kb = ring + (size_t)stage * Cfg::PAGE_BYTES;
+                        mbar_expect_tx(&full_k[stage], KV_BYTES);
+#pragma unroll
+                        for (int s = 0; s < HD / 64; ++s) tma_load_2d(kb + s * (KV_PAGE * 128), &map_k, s * 64, row * KV_PAGE, &full_k[stage], pol);
+                        mbar_expect_tx(&full_v[stage], KV_BYTES);
+#pragma unroll
+                        for (int s = 0; s < 2; ++s) tma_load_2d(kb + KV_BYTES + s * (HD * 128), &map_v, s * 64, row * HD, &full_v[stage], pol);
+                        ++count;
+                        if (++stage == STAGES) { stage = 0; phase ^= 1u; }
+                    }
+            s_issued = count;
+        }
+        __syncwarp();
+    } else {
+        const int gid = lane >> 2, t = lane & 3, mt = warp % MT, ks = warp / MT;
+        pdl_wait();                                         // the queries come from the kernel before
+        for (int idx = threadIdx.x; idx < Cfg::QROWS * (HD / 8); idx += AD_COMPUTE) {
+            const int row = idx / (HD / 8), c = idx % (HD / 8);
+            const bool lo = STACK ? row >= 8 : (row & 31) >= 16;
+            const int vec = STACK ? row & 7 : (row >> 5) * 16 + (row & 15);
+            const bf16* src = (lo ? g.q_lo : g.q_hi) + ((size_t)(r0 + vec / G) * g.Hkv * G + kvh * G + vec % G) * HD + c * 8;
+            *(uint4*)(Qs + row * QP + c * 16) = *(const uint4*)src;
+        }
+        int qpos[NR], qhl[NR], qhh[NR];
+#pragma unroll
+        for (int h = 0; h < NR; ++h) {
+            const int r = (STACK ? gid : mt * 16 + gid + 8 * h) / G;
+            qpos[h] = g.row_slot ? g.row_slot[r0 + r] : pos_lo + r;
+            qhl[h] = g.row_slot ? g.hole_lo[r0 + r] : 0;
+            qhh[h] = g.row_slot ? g.hole_hi[r0 + r] : 0;
+        }
+        ad_bar();
+        // lane offsets of the ldmatrix addresses: matrix (lane / 8) of four
+        const int mi = lane >> 3, lr = lane & 7;
+        const uint32_t q_addr = smem_u32(Qs) + (uint32_t)(((STACK ? 0 : mt * 32) + lr + 8 * (mi & 1)) * QP + (mi >> 1) * 16);
+        const uint32_t kv_off = (uint32_t)((lr + 8 * (mi >> 1)) * 128), chunk0 = (uint32_t)(mi & 1);
+        const uint32_t ring_addr = smem_u32(ring);
+
+        float m_run[NR], l_run[NR], o[DT][4];
+        auto block = [&](uint32_t kb, int key_page, int p, uint32_t par, int stage) {       // keys key_page .. + 15 of page p
+            float c[2][4];
+#pragma unroll
+            for (int j = 0; j < 2; ++j) { c[j][0] = 0.f; c[j][1] = 0.f; c[j][2] = 0.f; c[j][3] = 0.f; }
+            const uint32_t kr = kb + kv_off + (uint32_t)key_page * 128u;
+#pragma unroll
+            for (int k = 0; k < KS; ++k) {
+                uint32_t b[4], a[4];
+                ad_ldm4(kr + (uint32_t)((k >> 2) * (KV_PAGE * 128)) + ((((uint32_t)((k & 3) * 2) + chunk0) ^ (uint32_t)lr) << 4), b);
+                ad_ldm4(q_addr + (uint32_t)(k * 32), a);
+                ad_mma(c[0], a, b[0], b[1]);
+                ad_mma(c[1], a, b[2], b[3]);
+                if (!STACK) {
+                    ad_ldm4(q_addr + (uint32_t)(16 * QP + k * 32), a);
+                    ad_mma(c[0], a, b[0], b[1]);
+                    ad_mma(c[1], a, b[2], b[3]);
+                }
+            }
+            uint32_t ph[4], pl[4];
+            float resc[NR];
+#pragma unroll
+            for (int h = 0; h < NR; ++h) {
+                float w[2][2], mx = -CUDART_INF_F;
+#pragma unroll
+                for (int j = 0; j < 2; ++j)
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        const int key = p * KV_PAGE + key_page + 8 * j + 2 * t + e;
+                        const float s = STACK ? c[j][e] + c[j][2 + e] : c[j][2 * h + e];
+                        w[j][e] = (key <= qpos[h] && !(key >= qhl[h] && key < qhh[h])) ? s : -CUDART_INF_F;
+                        mx = fmaxf(mx, w[j][e]);
+                    }
+                mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+                mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+                const float m_new = fmaxf(m_run[h], mx);
+                const bool none = m_new == -CUDART_INF_F;
+                resc[h] = none ? 1.0f : exp2f(m_run[h] - m_new);
+                float sum = 0.0f;
+#pragma unroll
+                for (int j = 0; j < 2; ++j)
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) { w[j][e] = none ? 0.0f : exp2f(w[j][e] - m_new); sum += w[j][e]; }
+                l_run[h] = l_run[h] * resc[h] + sum;        // this lane's keys; the four lanes of a row are added at the end
+                m_run[h] = m_new;
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    uint32_t lo;
+                    const uint32_t hi = ad_split(w[j][0], w[j][1], lo);
+                    if (STACK) { ph[2 * j] = hi; ph[2 * j + 1] = lo; }       // rows gid: hi terms, rows gid + 8: lo terms
+                    else { ph[2 * j + h] = hi; pl[2 * j + h] = lo; }
+                }
+            }
+            const float ra = resc[0], rb = resc[NR - 1];
+            if (__any_sync(0xffffffffu, ra != 1.0f || rb != 1.0f)) {        // multiplying by 1 changes nothing
+#pragma unroll
+                for (int d = 0; d < DT; ++d) { o[d][0] *= ra; o[d][1] *= ra; o[d][2] *= rb; o[d][3] *= rb; }
+            }
+            mbar_wait(&full_v[stage], par, abortp);
+            const uint32_t vr = kb + KV_BYTES + kv_off + (uint32_t)((key_page >> 6) * (HD * 128)) + ((((uint32_t)((key_page & 63) >> 3) + chunk0) ^ (uint32_t)lr) << 4);
+#pragma unroll
+            for (int d = 0; d < DT / 2; ++d) {
+                uint32_t b[4];
+                ad_ldm4(vr + (uint32_t)(d * 16 * 128), b);
+                ad_mma(o[2 * d], ph, b[0], b[1]);
+                ad_mma(o[2 * d + 1], ph, b[2], b[3]);
+                if (!STACK) { ad_mma(o[2 * d], pl, b[0], b[1]); ad_mma(o[2 * d + 1], pl, b[2], b[3]); }
+            }
+        };
+
+        float R_m[Cfg::ITEMS], R_l[Cfg::ITEMS];             // one CTA for all shares: the running result of this thread's pieces
+        float4 R_a[Cfg::ITEMS];
+#pragma unroll
+        for (int i = 0; i < Cfg::ITEMS; ++i) { R_m[i] = -CUDART_INF_F; R_l[i] = 0.0f; R_a[i] = make_float4(0.f, 0.f, 0.f, 0.f); }
+        int stage = 0;
+        uint32_t par = 0;
+        bool cluster_ready = false;
+        for (int v = v_lo; v < v_hi; ++v) {
+            if (g.cluster == 1 && v * PG >= n_pages) break;  // the remaining shares hold nothing
+#pragma unroll
+            for (int h = 0; h < NR; ++h) { m_run[h] = -CUDART_INF_F; l_run[h] = 0.0f; }
+#pragma unroll
+            for (int d = 0; d < DT; ++d) { o[d][0] = 0.f; o[d][1] = 0.f; o[d][2] = 0.f; o[d][3] = 0.f; }
+            for (int p0 = v * PG; p0 < n_pages; p0 += VR * PG)
+                for (int i = 0; i < PG; ++i) {
+                    const int p = p0 + i;
+                    if (p >= n_pages) break;
+                    if (PG == 1 || (ks >> 3) == i) {
+                        mbar_wait(&full_k[stage], par, abortp);
+                        const uint32_t kb = ring_addr + (uint32_t)stage * (uint32_t)Cfg::PAGE_BYTES;
+#pragma unroll 1
+                        for (int b = KW >= 8 ? ks & 7 : ks; b < KV_PAGE / AD_KEYS; b += (KW >= 8 ? 8 : KW))
+                            if (p * KV_PAGE + b * AD_KEYS <= pos_hi) block(kb, b * AD_KEYS, p, par, stage);
+                        mbar_wait(&full_v[stage], par, abortp);
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(&empty[stage]);
+                    }
+                    if (++stage == STAGES) { stage = 0; par ^= 1u; }
+                }
+            // ---- the share's key slots, in slot order ----
+#pragma unroll
+            for (int h = 0; h < NR; ++h) {
+                l_run[h] += __shfl_xor_sync(0xffffffffu, l_run[h], 1);
+                l_run[h] += __shfl_xor_sync(0xffffffffu, l_run[h], 2);
+                if (t == 0) { sm_m[warp * NV + gid + 8 * h] = m_run[h]; sm_l[warp * NV + gid + 8 * h] = l_run[h]; }
+            }
+            float* mine = sm_o + (size_t)warp * NV * OP;
+#pragma unroll
+            for (int d = 0; d < DT; ++d) {
+                if (STACK) *(float2*)(mine + gid * OP + 8 * d + 2 * t) = make_float2(o[d][0] + o[d][2], o[d][1] + o[d][3]);
+                else {
+                    *(float2*)(mine + gid * OP + 8 * d + 2 * t) = make_float2(o[d][0], o[d][1]);
+                    *(float2*)(mine + (gid + 8) * OP + 8 * d + 2 * t) = make_float2(o[d][2], o[d][3]);
+                }
+            }
+            ad_bar();
+            if (g.cluster > 1 && !cluster_ready) { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); cluster_ready = true; }
+#pragma unroll
+            for (int i = 0; i < Cfg::ITEMS; ++i) {
+                const int idx = threadIdx.x + i * AD_COMPUTE;
+                if (idx < Cfg::Q * V4) {
+                    const int vec = idx / V4, d4 = idx % V4, tile = vec / NV, vi = vec % NV;
+                    float mx = -CUDART_INF_F;
+#pragma unroll
+                    for (int k = 0; k < KW; ++k) mx = fmaxf(mx, sm_m[(k * MT + tile) * NV + vi]);
+                    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+                    float l = 0.0f;
+#pragma unroll
+                    for (int k = 0; k < KW; ++k) {
+                        const int w = k * MT + tile;
+                        const float m = sm_m[w * NV + vi], s = m == -CUDART_INF_F ? 0.0f : exp2f(m - mx);
+                        const float4 x = *(const float4*)(sm_o + (size_t)(w * NV + vi) * OP + 4 * d4);
+                        a.x = fmaf(x.x, s, a.x); a.y = fmaf(x.y, s, a.y); a.z = fmaf(x.z, s, a.z); a.w = fmaf(x.w, s, a.w);
+                        l = fmaf(sm_l[w * NV + vi], s, l);
+                    }
+                    if (g.cluster == 1) ad_fold(R_m[i], R_l[i], R_a[i], mx, l, a);
+                    else {
+                        const int owner = vec / VO, at = v * VO + vec % VO;
+                        asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(ad_map(recv + at * HD + 4 * d4, owner)), "f"(a.x), "f"(a.y), "f"(a.z), "f"(a.w) : "memory");
+                        if (d4 == 0) {
+                            asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(ad_map(rc_m + at, owner)), "f"(mx) : "memory");
+                            asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(ad_map(rc_l + at, owner)), "f"(l) : "memory");
+                        }
+                    }
+                }
+            }
+            if (v + 1 < v_hi) ad_bar();                      // the slots' results may be overwritten
+        }
+        // ---- the result, as hi + lo terms in the O projection's operand image ----
+        auto store = [&](int vec, int d4, float l, float4 a) {
+            const int row = r0 + vec / G, k = (kvh * G + vec % G) * HD + 4 * d4;
+            uint2 hi, lo;
+            hi.x = ad_split(a.x / l, a.y / l, lo.x);
+            hi.y = ad_split(a.z / l, a.w / l, lo.y);
+            *(uint2*)(g.img + cl_img_offset(g.rows, row, k)) = hi;
+            *(uint2*)(g.img + cl_img_offset(g.rows, g.rows + row, k)) = lo;
+        };
+        if (g.cluster == 1) {
+#pragma unroll
+            for (int i = 0; i < Cfg::ITEMS; ++i) {
+                const int idx = threadIdx.x + i * AD_COMPUTE;
+                if (idx < Cfg::Q * V4) store(idx / V4, idx % V4, R_l[i], R_a[i]);
+            }
+        } else {
+            asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+            for (int idx = threadIdx.x; idx < VO * V4; idx += AD_COMPUTE) {
+                const int vo = idx / V4, d4 = idx % V4;
+                float m = -CUDART_INF_F, l = 0.0f;
+                float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                for (int k = 0; k < VR; ++k)
+                    ad_fold(m, l, a, rc_m[k * VO + vo], rc_l[k * VO + vo], *(const float4*)(recv + (k * VO + vo) * HD + 4 * d4));
+                store(rank * VO + vo, d4, l, a);
+            }
+        }
+    }
+    // the loading warp and a CTA that is its own cluster take part in the cluster barriers too
+    if (g.cluster == 1) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+    else if (warp == AD_WARPS) {
+        asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+        asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+    }
+    __syncthreads();
+    if (threadIdx.x == 0 && abort_flag) {
+        // gave up somewhere: let every copy already requested land before the CTA may exit
+        for (int i = max(0, s_issued - STAGES); i < s_issued; ++i) {
+            for (unsigned spin = 0; spin < WAIT_LIMIT && !mbar_try_wait(&full_k[i % STAGES], (uint32_t)((i / STAGES) & 1)); ++spin) {}
+            for (unsigned spin = 0; spin < WAIT_LIMIT && !mbar_try_wait(&full_v[i % STAGES], (uint32_t)((i / STAGES) & 1)); ++spin) {}
+        }
+        atomicExch(g.err, AD_ERR_TIMEOUT);
+    }
+}
+
+template <int HD, int G>
+anpd_status launch_attn_dec(anpd_model* m, anpd_kv* kv, AdArgs& a) {
+    typedef AdCfg<HD, G> Cfg;
+    static bool attr_set[64] = {false};
+    if (first_call_on_device(attr_set)) CUDA_TRY(cudaFuncSetAttribute(attn_dec_kernel<HD, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::SMEM));
+    // A CTA per share or one per head, whichever takes fewer rounds of a share's work: about 7/8 of the SMs can hold clusters.
+    const int heads = a.Hkv * kv->batch, resident = std::max(1, m->num_sms * 7 / 8 / Cfg::VR);
+    a.cluster = (heads + resident - 1) / resident < Cfg::VR * ((heads + m->num_sms - 1) / m->num_sms) ? Cfg::VR : 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(a.cluster, a.Hkv, kv->batch); cfg.blockDim = dim3(AD_THREADS); cfg.dynamicSmemBytes = Cfg::SMEM; cfg.stream = m->stream;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = a.cluster; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = (g_use_pdl && !t_no_pdl) ? 2 : 1;
+    LAUNCH(&m->prof, m->stream, KC_ATTN, 0, (cudaLaunchKernelEx(&cfg, attn_dec_kernel<HD, G>, kv->map_k, kv->map_v, (const AdArgs)a)));
+    CUDA_TRY(cudaGetLastError());
+    return ANPD_OK;
+}
+
+}  // namespace
+
+bool attn_dec_supported(const anpd_model* m) {
+    const int G = m->cfg.n_q_heads / m->cfg.n_kv_heads;
+    return m->cfg.head_dim == 64 || G == 1;
+}
+
+anpd_status attn_dec_enqueue(anpd_model* m, anpd_kv* kv, int layer, bool tree) {
+    const anpd_model_config& c = m->cfg;
+    Workspace& ws = kv->ws;
+    AdArgs a;
+    a.q_hi = ws.q_hi; a.q_lo = ws.q_lo;
+    a.page_table = kv->page_table; a.row_pos = ws.row_pos; a.row_seq = ws.row_seq;
+    a.row_slot = tree ? ws.row_slot : nullptr; a.hole_lo = tree ? ws.row_hole_lo : nullptr; a.hole_hi = tree ? ws.row_hole_hi : nullptr;
+    a.pages_per_seq = kv->pages_per_seq; a.Hkv = c.n_kv_heads; a.rows = kv->batch * ANPD_ROWS;
+    a.layer_page0 = layer * kv->total_pages;
+    a.img = ws.ci_ao; a.err = ws.gemm_err;
+    switch (c.head_dim * 16 + c.n_q_heads / c.n_kv_heads) {
+        case 64 * 16 + 1: return launch_attn_dec<64, 1>(m, kv, a);
+        case 64 * 16 + 2: return launch_attn_dec<64, 2>(m, kv, a);
+        case 64 * 16 + 4: return launch_attn_dec<64, 4>(m, kv, a);
+        case 64 * 16 + 8: return launch_attn_dec<64, 8>(m, kv, a);
+        case 128 * 16 + 1: return launch_attn_dec<128, 1>(m, kv, a);
+    }
+    return ANPD_ERR_ARG;
+}

@@ -99,9 +99,12 @@ __device__ __forceinline__ void store_split4(const float4 v, bf16* hi_ptr, bf16*
 
 __global__ void __launch_bounds__(NORM_THREADS) embed_norm_kernel(const bf16* __restrict__ embed, const int* __restrict__ row_tok,
                                                                   const float* __restrict__ gain, float eps, int d,
-                                                                  float* __restrict__ x, bf16* __restrict__ h_hi, bf16* __restrict__ h_lo) {
-    pdl_trigger();
+                                                                  float* __restrict__ x, bf16* __restrict__ h_hi, bf16* __restrict__ h_lo,
+                                                                  unsigned char* __restrict__ img) {
+    // img: a decode step's operand image of gridDim.x rows instead of h_hi and h_lo.  The trigger comes after the wait here:
+    // whatever starts behind this kernel may then read the row plan at once.
     pdl_wait();
+    pdl_trigger();
     __shared__ float red[32];
     const int row = blockIdx.x, chunks = d >> 2;
     const bf16* e = embed + (size_t)row_tok[row] * d;
@@ -126,9 +129,36 @@ __global__ void __launch_bounds__(NORM_THREADS) embed_norm_kernel(const bf16* __
         if (c < chunks) {
             const float4 g = *(const float4*)(gain + 4 * c);
             store_split4(make_float4(v[u].x * rstd * g.x, v[u].y * rstd * g.y, v[u].z * rstd * g.z, v[u].w * rstd * g.w),
-                         h_hi + (size_t)row * d + 4 * c, h_lo + (size_t)row * d + 4 * c);
+                         img ? (bf16*)(img + cl_img_offset(gridDim.x, row, 4 * c)) : h_hi + (size_t)row * d + 4 * c,
+                         img ? (bf16*)(img + cl_img_offset(gridDim.x, gridDim.x + row, 4 * c)) : h_lo + (size_t)row * d + 4 * c);
         }
     }
+}
+
+// Decode steps: x = E[tok]; the first projection's operand image receives x * gain as hi + lo terms, un-normalised (the consumer
+// applies 1 / RMS); the row's sum of squares goes to ss[row] (one part).
+__global__ void __launch_bounds__(NORM_THREADS) embed_cl_kernel(const bf16* __restrict__ embed, const int* __restrict__ row_tok,
+                                                                const float* __restrict__ gain, int d, float* __restrict__ x,
+                                                                unsigned char* __restrict__ img, int img_rows, float* __restrict__ ss) {
+    // The trigger comes after the wait here: whatever starts behind this kernel may then read the row plan at once.
+    pdl_wait();
+    pdl_trigger();
+    __shared__ float red[32];
+    const int row = blockIdx.x, chunks = d >> 2;
+    const bf16* e = embed + (size_t)row_tok[row] * d;
+    float acc = 0.0f;
+    for (int c = threadIdx.x; c < chunks; c += NORM_THREADS) {
+        const uint2 raw = *(const uint2*)(e + 4 * c);
+        const bf16* b = (const bf16*)&raw;
+        const float4 g = *(const float4*)(gain + 4 * c);
+        const float4 v = make_float4(__bfloat162float(b[0]), __bfloat162float(b[1]), __bfloat162float(b[2]), __bfloat162float(b[3]));
+        *(float4*)(x + (size_t)row * d + 4 * c) = v;
+        store_split4(make_float4(v.x * g.x, v.y * g.y, v.z * g.z, v.w * g.w), (bf16*)(img + cl_img_offset(img_rows, row, 4 * c)),
+                     (bf16*)(img + cl_img_offset(img_rows, img_rows + row, 4 * c)));        // 4 elements never straddle a 16-byte chunk
+        acc += v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
+    }
+    const float t = block_sum_1024(acc, red);
+    if (threadIdx.x == 0) ss[row] = t;
 }
 
 // Single-sequence steps (row-range projections): x = E[tok]; the first projection's operand image receives
@@ -163,7 +193,9 @@ __global__ void __launch_bounds__(NORM_THREADS) embed_img_kernel(const bf16* __r
 __global__ void __launch_bounds__(NORM_THREADS) resid_norm_kernel(float* __restrict__ x, const float* __restrict__ part,
                                                                   const int* __restrict__ seg_count, size_t split_stride, int ld_part,
                                                                   const float* __restrict__ gain, float eps, int d,
-                                                                  bf16* __restrict__ h_hi, bf16* __restrict__ h_lo, int ns_max) {
+                                                                  bf16* __restrict__ h_hi, bf16* __restrict__ h_lo, int ns_max,
+                                                                  unsigned char* __restrict__ img) {
+    // img: a decode step's operand image of gridDim.x rows instead of h_hi and h_lo.
     // ns_max: the most partial sums any tile of this projection has.  The loads cover that many slabs whatever the tile's own
     // count (slabs beyond it hold older sums: read, never added), so they do not wait for the count to arrive.
     pdl_trigger();
@@ -207,7 +239,8 @@ __global__ void __launch_bounds__(NORM_THREADS) resid_norm_kernel(float* __restr
         if (c < chunks) {
             const float4 g = gn[u];
             store_split4(make_float4(v[u].x * rstd * g.x, v[u].y * rstd * g.y, v[u].z * rstd * g.z, v[u].w * rstd * g.w),
-                         h_hi + (size_t)row * d + 4 * c, h_lo + (size_t)row * d + 4 * c);
+                         img ? (bf16*)(img + cl_img_offset(gridDim.x, row, 4 * c)) : h_hi + (size_t)row * d + 4 * c,
+                         img ? (bf16*)(img + cl_img_offset(gridDim.x, gridDim.x + row, 4 * c)) : h_lo + (size_t)row * d + 4 * c);
         }
     }
 }
@@ -606,7 +639,7 @@ constexpr int COMBINE_SLICES = 4;
 constexpr int COMBINE_MAX_PAGES = 256;
 __global__ void attn_combine_kernel(const float* __restrict__ pm, const float* __restrict__ pl, const float* __restrict__ po,
                                     const int* __restrict__ row_pos, int Hq, int hd, int pages_per_seq,
-                                    bf16* __restrict__ ao_hi, bf16* __restrict__ ao_lo, unsigned char* __restrict__ img) {
+                                    bf16* __restrict__ ao_hi, bf16* __restrict__ ao_lo, unsigned char* __restrict__ img, int img_rows) {
     // row_pos: the rows' cache slots (= positions outside two-candidate steps)
     pdl_trigger();
     pdl_wait();
@@ -651,7 +684,10 @@ __global__ void attn_combine_kernel(const float* __restrict__ pm, const float* _
         for (int k = 1; k < COMBINE_SLICES; ++k) t += s_o[k][dim];
         bf16 hi, lo;
         split_bf16(t / s_L, hi, lo);
-        if (img) {                                        // single-sequence step: straight into the O projection's operand image
+        if (img_rows > 0) {                               // straight into the O projection's operand image
+            *(bf16*)(img + cl_img_offset(img_rows, row, head * hd + dim)) = hi;
+            *(bf16*)(img + cl_img_offset(img_rows, img_rows + row, head * hd + dim)) = lo;
+        } else if (img) {                                 // the same for the row-range projections
             *(bf16*)(img + act_img_offset(row, head * hd + dim)) = hi;
             *(bf16*)(img + act_img_offset(ANPD_ROWS + row, head * hd + dim)) = lo;
         } else {
@@ -669,7 +705,7 @@ template <int VEC>
 __global__ void __launch_bounds__(32 * COMBINE_SLICES) attn_combine_wide_kernel(const float* __restrict__ pm, const float* __restrict__ pl,
                                                                                const float* __restrict__ po, const int* __restrict__ row_pos,
                                                                                int Hq, int pages_per_seq, bf16* __restrict__ ao_hi,
-                                                                               bf16* __restrict__ ao_lo) {
+                                                                               bf16* __restrict__ ao_lo, unsigned char* __restrict__ img, int img_rows) {
     pdl_trigger();
     pdl_wait();
     constexpr int hd = 32 * VEC;
@@ -703,6 +739,9 @@ __global__ void __launch_bounds__(32 * COMBINE_SLICES) attn_combine_wide_kernel(
     __syncthreads();
     if (slice == 0) {
         const size_t out = (size_t)row * Hq * hd + head * hd + lane * VEC;
+        const int k = head * hd + lane * VEC;
+        bf16* dst_hi = img_rows > 0 ? (bf16*)(img + cl_img_offset(img_rows, row, k)) : ao_hi + out;       // VEC elements never straddle a 16-byte chunk
+        bf16* dst_lo = img_rows > 0 ? (bf16*)(img + cl_img_offset(img_rows, img_rows + row, k)) : ao_lo + out;
         bf16 h[VEC], l[VEC];
 #pragma unroll
         for (int e = 0; e < VEC; ++e) {
@@ -710,8 +749,8 @@ __global__ void __launch_bounds__(32 * COMBINE_SLICES) attn_combine_wide_kernel(
             for (int k = 1; k < COMBINE_SLICES; ++k) t += s_o[k][lane * VEC + e];
             split_bf16(t / L, h[e], l[e]);
         }
-        if (VEC == 4) { *(uint2*)(ao_hi + out) = *(const uint2*)h; *(uint2*)(ao_lo + out) = *(const uint2*)l; }
-        else { *(uint32_t*)(ao_hi + out) = *(const uint32_t*)h; *(uint32_t*)(ao_lo + out) = *(const uint32_t*)l; }
+        if (VEC == 4) { *(uint2*)dst_hi = *(const uint2*)h; *(uint2*)dst_lo = *(const uint2*)l; }
+        else { *(uint32_t*)dst_hi = *(const uint32_t*)h; *(uint32_t*)dst_lo = *(const uint32_t*)l; }
     }
 }
 
@@ -719,7 +758,8 @@ __global__ void __launch_bounds__(32 * COMBINE_SLICES) attn_combine_wide_kernel(
 // SwiGLU epilogue of the gate/up projection
 // ---------------------------------------------------------------------------------------------
 __global__ void swiglu_kernel(const float* __restrict__ part, const int* __restrict__ seg_count, size_t split_stride, int ld_part, int F,
-                              bf16* __restrict__ act_hi, bf16* __restrict__ act_lo, int ns_max) {
+                              bf16* __restrict__ act_hi, bf16* __restrict__ act_lo, int ns_max, unsigned char* __restrict__ img) {
+    // img: a decode step's operand image of gridDim.y rows instead of act_hi and act_lo
     pdl_trigger();
     pdl_wait();
     const int row = blockIdx.y, j = blockIdx.x * blockDim.x + threadIdx.x;
@@ -733,7 +773,7 @@ __global__ void swiglu_kernel(const float* __restrict__ part, const int* __restr
         pg[s] = (s < ns_max) ? pr[s * split_stride + j] : 0.0f;
         pu[s] = (s < ns_max) ? pr[s * split_stride + F + j] : 0.0f;
     }
-    const int ng = seg_count[j >> 7], nu = seg_count[(F + j) >> 7];
+    const int ng = seg_count[j >> 6], nu = ng;          // a 128-position storage tile holds 64 gate features and their up features
 #pragma unroll
     for (int s = 0; s < 4; ++s) { if (s < ng) gte += pg[s]; if (s < nu) up += pu[s]; }
     for (int s = 4; s < ng; ++s) gte += pr[s * split_stride + j];
@@ -741,6 +781,11 @@ __global__ void swiglu_kernel(const float* __restrict__ part, const int* __restr
     const float v = gte / (1.0f + expf(-gte)) * up;
     bf16 hi, lo;
     split_bf16(v, hi, lo);
+    if (img) {
+        *(bf16*)(img + cl_img_offset(gridDim.y, row, j)) = hi;
+        *(bf16*)(img + cl_img_offset(gridDim.y, gridDim.y + row, j)) = lo;
+        return;
+    }
     act_hi[(size_t)row * F + j] = hi;
     act_lo[(size_t)row * F + j] = lo;
 }
@@ -748,7 +793,7 @@ __global__ void swiglu_kernel(const float* __restrict__ part, const int* __restr
 // The same for many rows (prefill passes): a thread owns four consecutive features, so the partial sums come in
 // 16-byte loads.  Per element the arithmetic is that of swiglu_kernel, in the same order.
 __global__ void swiglu_wide_kernel(const float* __restrict__ part, const int* __restrict__ seg_count, size_t split_stride, int ld_part, int F,
-                                   bf16* __restrict__ act_hi, bf16* __restrict__ act_lo) {
+                                   bf16* __restrict__ act_hi, bf16* __restrict__ act_lo, unsigned char* __restrict__ img) {
     pdl_trigger();
     pdl_wait();
     // two chunks of four features per thread (a block's width apart); every output has at least one partial sum, so the
@@ -767,8 +812,7 @@ __global__ void swiglu_wide_kernel(const float* __restrict__ part, const int* __
         if (live[c]) {
             g4[c] = *(const float4*)(pr + j);
             u4[c] = *(const float4*)(pr + F + j);
-            ng[c] = seg_count[j >> 7];
-            nu[c] = seg_count[(F + j) >> 7];
+            ng[c] = nu[c] = seg_count[j >> 6];               // a 128-position storage tile holds 64 gate features and their up features
         }
     }
 #pragma unroll
@@ -781,8 +825,8 @@ __global__ void swiglu_wide_kernel(const float* __restrict__ part, const int* __
         bf16 hi[4], lo[4];
 #pragma unroll
         for (int e = 0; e < 4; ++e) split_bf16(gte[e] / (1.0f + expf(-gte[e])) * up[e], hi[e], lo[e]);
-        *(uint2*)(act_hi + (size_t)row * F + j) = *(const uint2*)hi;
-        *(uint2*)(act_lo + (size_t)row * F + j) = *(const uint2*)lo;
+        *(uint2*)(img ? (bf16*)(img + cl_img_offset(gridDim.y, row, j)) : act_hi + (size_t)row * F + j) = *(const uint2*)hi;
+        *(uint2*)(img ? (bf16*)(img + cl_img_offset(gridDim.y, gridDim.y + row, j)) : act_lo + (size_t)row * F + j) = *(const uint2*)lo;
     }
 }
 
@@ -936,20 +980,19 @@ __global__ void kv_move_kernel(const SeqState* __restrict__ seqs, const int* __r
 // weight-streaming GEMM, plain version: one warp per output feature, 8 rows at a time
 //   part[0][row][n] = sum_k W[n][k] * (a_hi[row][k] + a_lo[row][k])
 // ---------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) gemm_rows8_kernel(const bf16* __restrict__ W, const bf16* __restrict__ a_hi,
-                                                         const bf16* __restrict__ a_lo, int rows, int N, int K, long long total, int G,
+__global__ void __launch_bounds__(256) gemm_rows8_kernel(const unsigned char* __restrict__ W, const bf16* __restrict__ a_hi,
+                                                         const bf16* __restrict__ a_lo, int rows, const ClPlan plan,
                                                          float* __restrict__ part, int ld_part) {
     pdl_trigger();
     pdl_wait();
     const int n = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    const int N = plan.N, K = plan.K;
     if (n >= N) return;
-    // block storage: logical block (n / 128, k / 64) is 128 x 64 contiguous at its slot
-    const int k_blocks = (K + 63) / 64;
+    const int pos = cl_position(plan, n);
     for (int r0 = 0; r0 < rows; r0 += 8) {
         float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
         for (int k0 = lane * 8; k0 < K; k0 += 256) {
-            const long long slot = gemm_block_slot((long long)(n >> 7) * k_blocks + (k0 >> 6), total, G);
-            const uint4 wv = *(const uint4*)(W + gemm_block_elem(slot, n & 127, k0 & 63));
+            const uint4 wv = *(const uint4*)(W + cl_weight_offset(plan, pos, k0));
             const bf16* w8 = (const bf16*)&wv;
             float wf[8];
 #pragma unroll
@@ -986,6 +1029,18 @@ __global__ void fill_tail_segs_kernel(int* segs, int m_tiles, int first_cut, int
     if (i < m_tiles) segs[i] = i >= first_cut ? parts : 1;
 }
 
+// rows [from, from + 8) of the normalised activations -> rows 0-7 of a decode step's operand image
+__global__ void rows_to_image_kernel(const bf16* __restrict__ h_hi, const bf16* __restrict__ h_lo, int from, int d, unsigned char* __restrict__ img,
+                                     int img_rows) {
+    pdl_trigger();
+    pdl_wait();
+    const int r = blockIdx.x;
+    for (int i = threadIdx.x; i < d / 8; i += blockDim.x) {
+        *(uint4*)(img + cl_img_offset(img_rows, r, 8 * i)) = ((const uint4*)(h_hi + (size_t)(from + r) * d))[i];
+        *(uint4*)(img + cl_img_offset(img_rows, img_rows + r, 8 * i)) = ((const uint4*)(h_lo + (size_t)(from + r) * d))[i];
+    }
+}
+
 // rows [from, from + 8) of the normalised activations -> rows [0, 8)
 __global__ void move_rows_kernel(bf16* __restrict__ h_hi, bf16* __restrict__ h_lo, int from, int d) {
     pdl_trigger();
@@ -998,52 +1053,55 @@ __global__ void move_rows_kernel(bf16* __restrict__ h_hi, bf16* __restrict__ h_l
     }
 }
 
-// One projection of the forward.  Returns the per-tile segment counts its consumer must use.
-anpd_status gemm_enqueue(anpd_model* m, anpd_kv* kv, int kind, int layer, int rows, const int** seg_count_out, int* seg_max_out = nullptr) {
-    int seg_max_dummy;
-    if (!seg_max_out) seg_max_out = &seg_max_dummy;
+// One projection of a prompt pass, of a step of several sequences or, with the plain GEMM, of any forward.  Returns the number
+// of partial sums per 128-feature storage tile its consumer must add.
+anpd_status gemm_enqueue(anpd_model* m, anpd_kv* kv, int kind, int layer, int rows, const int** seg_count_out, int* seg_max_out) {
     Workspace& ws = kv->ws;
-    const GemmPlan& plan = m->plan[kind];
-    const int mode = (rows == kv->batch * ANPD_ROWS) ? 0 : 1;
-    const bf16* W = kind == GK_LM ? m->lm_head : (kind == GK_QKV ? m->layers[layer].wqkv : kind == GK_O ? m->layers[layer].wo
-                                                 : kind == GK_GU ? m->layers[layer].wgu : m->layers[layer].wd);
+    const ClPlan& plan = m->cl[kind];
+    const unsigned char* W = kind == GK_LM ? m->lm_head : (kind == GK_QKV ? m->layers[layer].wqkv : kind == GK_O ? m->layers[layer].wo
+                                                          : kind == GK_GU ? m->layers[layer].wgu : m->layers[layer].wd);
     const bf16 *a_hi = ws.h_hi, *a_lo = ws.h_lo;
-    const CUtensorMap* maps = ws.map_h[mode];
-    if (kind == GK_O) { a_hi = ws.ao_hi; a_lo = ws.ao_lo; maps = ws.map_ao[mode]; }
-    if (kind == GK_DOWN) { a_hi = ws.act_hi; a_lo = ws.act_lo; maps = ws.map_act[mode]; }
+    const CUtensorMap* maps = ws.map_h;
+    if (kind == GK_O) { a_hi = ws.ao_hi; a_lo = ws.ao_lo; maps = ws.map_ao; }
+    if (kind == GK_DOWN) { a_hi = ws.act_hi; a_lo = ws.act_lo; maps = ws.map_act; }
     if (m->plain_gemm) {
         *seg_count_out = m->d_ones;
         *seg_max_out = 1;
         return gemm_plain_enqueue(plan, W, a_hi, a_lo, rows, ws.part, ws.n_max_out, m->stream, &m->prof);
     }
-    if (mode == 1) {                                   // a prompt pass: complete sums, one per output
-        const int n_ft = (plan.m_tiles + 1) / 2, n_tt = (rows + 255) / 256;
-        const PfSchedule sched = gemm_pf_schedule(n_ft, n_tt, plan.k_blocks, m->num_sms);
-        if (sched.tail_split > 1) {                    // feature tiles from `first` on come in tail_split parts, the others in one
-            const int first = 2 * (sched.tail_from / n_tt), cfg = first * 4 + sched.tail_split;
-            if (m->tail_cfg[kind] != cfg) {
-                LAUNCH(&m->prof, m->stream, KC_OTHER, 0,
-                       (launch_k(fill_tail_segs_kernel, (plan.m_tiles + 127) / 128, 128, 0, m->stream, m->d_tail_segs[kind], plan.m_tiles, first,
-                                 sched.tail_split)));
-                m->tail_cfg[kind] = cfg;
-            }
-            *seg_count_out = m->d_tail_segs[kind];
-        } else {
-            *seg_count_out = m->d_const_segs[sched.ksplit];
-        }
-        *seg_max_out = std::max(sched.ksplit, sched.tail_split);
-        return gemm_pf_enqueue(plan, W, maps[0], maps[1], rows, ws.part, ws.n_max_out, (size_t)ws.r_max * ws.n_max_out, sched, m->num_sms,
-                               ws.gemm_err, m->stream, &m->prof);
+    if (rows == kv->batch * ANPD_ROWS) {               // a decode step: a partial sum per CTA of a cluster
+        const unsigned char* act = kind == GK_O ? ws.ci_ao : kind == GK_DOWN ? ws.ci_act : ws.ci_h;
+        *seg_count_out = m->d_const_segs[CL_CTAS];
+        *seg_max_out = CL_CTAS;
+        // the projection after this one, whose first weights are fetched into L2 under the small kernels between the two
+        const bool last = layer + 1 == m->cfg.n_layers;
+        const int next = kind == GK_QKV ? GK_O : kind == GK_O ? GK_GU : kind == GK_GU ? GK_DOWN : last ? GK_LM : GK_QKV;
+        const LayerW& lw = m->layers[layer];
+        const unsigned char* next_w = kind == GK_QKV ? lw.wo : kind == GK_O ? lw.wgu : kind == GK_GU ? lw.wd : last ? m->lm_head : m->layers[layer + 1].wqkv;
+        return cl_partial_enqueue(plan, W, act, rows, ws.part, (size_t)rows * ws.n_max_out, ws.n_max_out, kind == GK_LM ? nullptr : &m->cl[next], next_w,
+                                  CL_LEAD, kind == GK_QKV && layer == 0 ? 0 : CL_LEAD, ws.gemm_err, m->stream, &m->prof);
     }
-    ANPD_TRY(gemm_tc_enqueue(plan, W, maps[0], maps[1], rows, ws.nb[mode], ws.part, (size_t)kv->batch * ANPD_ROWS * ws.n_max_out,
-                             ws.n_max_out, ws.gemm_err, m->stream, &m->prof));
-    *seg_count_out = plan.d_seg_count;
-    *seg_max_out = plan.max_segs;
-    return ANPD_OK;
+    // a prompt pass: complete sums, or up to three per output
+    const int m_tiles = m->plan[kind].m_tiles, n_ft = (m_tiles + 1) / 2, n_tt = (rows + 255) / 256;
+    const PfSchedule sched = gemm_pf_schedule(n_ft, n_tt, plan.kb, m->num_sms);
+    if (sched.tail_split > 1) {                        // feature tiles from `first` on come in tail_split parts, the others in one
+        const int first = 2 * (sched.tail_from / n_tt), cfg = first * 4 + sched.tail_split;
+        if (m->tail_cfg[kind] != cfg) {
+            LAUNCH(&m->prof, m->stream, KC_OTHER, 0,
+                   (launch_k(fill_tail_segs_kernel, (m_tiles + 127) / 128, 128, 0, m->stream, m->d_tail_segs[kind], m_tiles, first, sched.tail_split)));
+            m->tail_cfg[kind] = cfg;
+        }
+        *seg_count_out = m->d_tail_segs[kind];
+    } else {
+        *seg_count_out = m->d_const_segs[sched.ksplit];
+    }
+    *seg_max_out = std::max(sched.ksplit, sched.tail_split);
+    return gemm_pf_enqueue(plan, W, maps[0], maps[1], rows, ws.part, ws.n_max_out, (size_t)ws.r_max * ws.n_max_out, sched, m->num_sms,
+                           ws.gemm_err, m->stream, &m->prof);
 }
 
 template <int HD>
-anpd_status attn_enqueue(anpd_model* m, anpd_kv* kv, int layer, int rows, int max_pos, unsigned char* img = nullptr, bool tree = false) {
+anpd_status attn_enqueue(anpd_model* m, anpd_kv* kv, int layer, int rows, int max_pos, unsigned char* img = nullptr, bool tree = false, int img_rows = 0) {
     const anpd_model_config& c = m->cfg;
     Workspace& ws = kv->ws;
     const size_t layer_elems = (size_t)kv->total_pages * c.n_kv_heads * KV_PAGE * HD;
@@ -1069,20 +1127,19 @@ anpd_status attn_enqueue(anpd_model* m, anpd_kv* kv, int layer, int rows, int ma
     }
     if (rows >= 64) LAUNCH(&m->prof, m->stream, KC_ATTN, 0,
            (launch_k(attn_combine_wide_kernel<HD / 32>, dim3(rows, c.n_q_heads), 32 * COMBINE_SLICES, 0, m->stream, ws.attn_m, ws.attn_l, ws.attn_o,
-                     tree ? ws.row_slot : ws.row_pos, c.n_q_heads, kv->pages_per_seq, ws.ao_hi, ws.ao_lo)));
+                     tree ? ws.row_slot : ws.row_pos, c.n_q_heads, kv->pages_per_seq, ws.ao_hi, ws.ao_lo, img, img_rows)));
     else LAUNCH(&m->prof, m->stream, KC_ATTN, 0,
            (launch_k(attn_combine_kernel, dim3(rows, c.n_q_heads), HD * COMBINE_SLICES, 0, m->stream, ws.attn_m, ws.attn_l, ws.attn_o, tree ? ws.row_slot : ws.row_pos, c.n_q_heads,
-                                                                              HD, kv->pages_per_seq, ws.ao_hi, ws.ao_lo, img)));
+                                                                              HD, kv->pages_per_seq, ws.ao_hi, ws.ao_lo, img, img_rows)));
     return ANPD_OK;
 }
 
 }  // namespace
 
-anpd_status gemm_plain_enqueue(const GemmPlan& p, const bf16* W, const bf16* a_hi, const bf16* a_lo, int rows, float* part, int ld_part,
+anpd_status gemm_plain_enqueue(const ClPlan& p, const unsigned char* W, const bf16* a_hi, const bf16* a_lo, int rows, float* part, int ld_part,
                                cudaStream_t st, Profiler* prof) {
     LAUNCH(prof, st, KC_GEMM, 2.0 * (double)p.N * (double)p.K,
-           (launch_k(gemm_rows8_kernel, (p.N + 7) / 8, 256, 0, st, W, a_hi, a_lo, rows, p.N, p.K, (long long)p.m_tiles * p.k_blocks, p.grid,
-                                                           part, ld_part)));
+           (launch_k(gemm_rows8_kernel, (p.N + 7) / 8, 256, 0, st, W, a_hi, a_lo, rows, p, part, ld_part)));
     CUDA_TRY(cudaGetLastError());
     return ANPD_OK;
 }
@@ -1170,10 +1227,77 @@ static anpd_status forward_rr_enqueue(anpd_model* m, anpd_kv* kv, int max_pos, b
     return ANPD_OK;
 }
 
+// The vocabulary projection of the 8 rows whose operand image is ws.ci_h, and its argmax candidates.
+static anpd_status lm_head_cl_enqueue(anpd_model* m, anpd_kv* kv, const float* ss, int n_parts, bool want_logits, unsigned own_lead = 0) {
+    const anpd_model_config& c = m->cfg;
+    Workspace& ws = kv->ws;
+    ClEpilogue lm;
+    lm.ss_in = ss; lm.n_parts = n_parts; lm.inv_d = 1.0f / (float)c.d_model; lm.eps = c.rms_eps;
+    lm.own_lead = own_lead;
+    lm.out = want_logits ? ws.logits : nullptr; lm.amax_val = ws.amax_val_cl; lm.amax_idx = ws.amax_idx_cl;
+    ANPD_TRY(cl_enqueue(m->cl[GK_LM], m->lm_head, ws.ci_h, lm, ws.gemm_err, m->stream, &m->prof));
+    ws.amax_nblk = cl_parts(m->cl[GK_LM]);
+    ws.amax_val_use = ws.amax_val_cl;
+    ws.amax_idx_use = ws.amax_idx_cl;
+    return ANPD_OK;
+}
+
+// The forward of a single sequence's step: per layer QKV (+ rotary, append), attention, O (+ residual), gate/up (+ SwiGLU), down
+// (+ residual); then the LM head (+ argmax).  Every projection finishes its own results (gemm_cl.cu).
+static anpd_status forward_cl_enqueue(anpd_model* m, anpd_kv* kv, int max_pos, bool want_logits, bool two_candidates) {
+    const anpd_model_config& c = m->cfg;
+    Workspace& ws = kv->ws;
+    cudaStream_t st = m->stream;
+    Profiler* pf = &m->prof;
+    const int d = c.d_model, hd = c.head_dim, rows = ANPD_ROWS;
+    const size_t layer_elems = (size_t)kv->total_pages * c.n_kv_heads * KV_PAGE * hd;
+    LAUNCH(pf, st, KC_OTHER, 0, (launch_k(embed_cl_kernel, rows, NORM_THREADS, 0, st, m->embed, ws.row_tok, m->layers[0].attn_norm, d, ws.x,
+                                          ws.ci_h, rows, ws.ss_cl_a)));
+    int parts_a = 1;                                   // sums of squares behind ci_h: one after the embedding, then the down projection's
+    // Each projection brings the first weights of the next one into L2 while its own tail and the hand-over leave HBM idle.
+    auto chain = [&](ClEpilogue& e, unsigned own, int next, const unsigned char* w) {
+        e.own_lead = own; e.next = &m->cl[next]; e.next_w = w; e.next_lead = CL_LEAD;
+    };
+    for (int l = 0; l < c.n_layers; ++l) {
+        const LayerW& w = m->layers[l];
+        ClEpilogue q;
+        q.ss_in = ws.ss_cl_a; q.n_parts = parts_a; q.inv_d = 1.0f / (float)d; q.eps = c.rms_eps;
+        q.row_pos = ws.row_pos; q.row_slot = ws.row_slot; q.row_seq = ws.row_seq; q.row_ok = ws.row_ok;
+        q.rope_cos = kv->rope_cos; q.rope_sin = kv->rope_sin; q.page_table = kv->page_table; q.pages_per_seq = kv->pages_per_seq;
+        q.Hq = c.n_q_heads; q.Hkv = c.n_kv_heads; q.hd = hd; q.q_scale = 1.4426950408889634f / sqrtf((float)hd);
+        q.q_hi = ws.q_hi; q.q_lo = ws.q_lo; q.kpool_l = kv->kpool + l * layer_elems; q.vpool_l = kv->vpool + l * layer_elems;
+        chain(q, l ? CL_LEAD : 0, GK_O, w.wo);
+        ANPD_TRY(cl_enqueue(m->cl[GK_QKV], w.wqkv, ws.ci_h, q, ws.gemm_err, st, pf));
+        if (attn_dec_supported(m) && (hd == 64 || kv->attn_tc)) ANPD_TRY(attn_dec_enqueue(m, kv, l, two_candidates));
+        else if (hd == 128) ANPD_TRY(attn_enqueue<128>(m, kv, l, rows, max_pos, ws.ci_ao, two_candidates, rows));
+        else ANPD_TRY(attn_enqueue<64>(m, kv, l, rows, max_pos, ws.ci_ao, two_candidates, rows));
+        ClEpilogue o;
+        o.x = ws.x; o.gain = w.ffn_norm; o.ss_out = ws.ss_cl_b; o.d = d; o.act_out = ws.ci_h2;
+        chain(o, CL_LEAD, GK_GU, w.wgu);
+        ANPD_TRY(cl_enqueue(m->cl[GK_O], w.wo, ws.ci_ao, o, ws.gemm_err, st, pf));
+        ClEpilogue gu;
+        gu.ss_in = ws.ss_cl_b; gu.n_parts = cl_parts(m->cl[GK_O]); gu.inv_d = 1.0f / (float)d; gu.eps = c.rms_eps; gu.act_out = ws.ci_act;
+        chain(gu, CL_LEAD, GK_DOWN, w.wd);
+        ANPD_TRY(cl_enqueue(m->cl[GK_GU], w.wgu, ws.ci_h2, gu, ws.gemm_err, st, pf));
+        ClEpilogue dn;
+        dn.x = ws.x; dn.gain = (l + 1 < c.n_layers) ? m->layers[l + 1].attn_norm : m->final_norm; dn.ss_out = ws.ss_cl_a; dn.d = d;
+        dn.act_out = ws.ci_h;
+        const bool last = l + 1 == c.n_layers;
+        chain(dn, CL_LEAD, last ? GK_LM : GK_QKV, last ? m->lm_head : m->layers[l + 1].wqkv);
+        ANPD_TRY(cl_enqueue(m->cl[GK_DOWN], w.wd, ws.ci_act, dn, ws.gemm_err, st, pf));
+        parts_a = cl_parts(m->cl[GK_DOWN]);
+    }
+    ANPD_TRY(lm_head_cl_enqueue(m, kv, ws.ss_cl_a, parts_a, want_logits, CL_LEAD));
+    CUDA_TRY(cudaGetLastError());
+    return ANPD_OK;
+}
+
 anpd_status forward_enqueue(anpd_model* m, anpd_kv* kv, int rows, int max_pos, bool head, bool want_logits, int head_row, bool two_candidates) {
     // the two fused variants know nothing of a second candidate's cache slots and mask
     if (m->rr_ready && kv->batch == 1 && rows == ANPD_ROWS && head && !m->plain_gemm && !two_candidates) return forward_rr_enqueue(m, kv, max_pos, want_logits);
     if (kv->step_ready && rows == kv->batch * ANPD_ROWS && head && !m->prof.on && !two_candidates) return step_kernel_enqueue(m, kv, max_pos, want_logits);
+    const bool decode = rows == kv->batch * ANPD_ROWS && !m->plain_gemm;           // (or a prompt pass of as many rows)
+    if (decode && kv->batch == 1 && head && m->cl_all_fused) return forward_cl_enqueue(m, kv, max_pos, want_logits, two_candidates);
     const anpd_model_config& c = m->cfg;
     kv->ws.amax_nblk = kv->ws.amax_blocks;
     kv->ws.amax_val_use = kv->ws.amax_val;
@@ -1182,14 +1306,13 @@ anpd_status forward_enqueue(anpd_model* m, anpd_kv* kv, int rows, int max_pos, b
     cudaStream_t st = m->stream;
     Profiler* pf = &m->prof;
     const int d = c.d_model, F = c.d_ffn, hd = c.head_dim, V = c.vocab;
-    // between the partial sums of an output: the segments of a decode step, the K parts of a prompt pass
-    const size_t sstride = (rows == kv->batch * ANPD_ROWS) ? (size_t)kv->batch * ANPD_ROWS * ws.n_max_out : (size_t)ws.r_max * ws.n_max_out;
+    const size_t sstride = (size_t)(decode ? rows : ws.r_max) * ws.n_max_out;      // between the partial sums of an output (the K parts of a projection)
     const size_t layer_elems = (size_t)kv->total_pages * c.n_kv_heads * KV_PAGE * hd;
     const int* segs = nullptr;
     int seg_max = 1;                                   // the most partial sums a tile of the last projection has
 
     LAUNCH(pf, st, KC_OTHER, 0, (launch_k(embed_norm_kernel, rows, NORM_THREADS, 0, st, m->embed, ws.row_tok, m->layers[0].attn_norm, c.rms_eps, d,
-                                                                      ws.x, ws.h_hi, ws.h_lo)));
+                                                                      ws.x, ws.h_hi, ws.h_lo, decode ? ws.ci_h : nullptr)));
     const bool many_rows = rows >= 64;                 // prefill passes: throughput-shaped launches of the small kernels
     const int rope_hpb = many_rows ? 256 / (hd / 2) : 1;            // heads per block of the rotary kernel
     for (int l = 0; l < c.n_layers; ++l) {
@@ -1212,38 +1335,45 @@ anpd_status forward_enqueue(anpd_model* m, anpd_kv* kv, int rows, int max_pos, b
                    ws.part, segs, sstride, ws.n_max_out, ws.row_pos, ws.row_slot, ws.row_seq, ws.row_ok, kv->rope_cos, kv->rope_sin,
                    kv->page_table, kv->pages_per_seq, c.n_q_heads, c.n_kv_heads, hd, 1.4426950408889634f / sqrtf((float)hd), ws.q_hi,
                    ws.q_lo, kv->kpool + l * layer_elems, kv->vpool + l * layer_elems, seg_max)));
-        if (hd == 128) ANPD_TRY(attn_enqueue<128>(m, kv, l, rows, max_pos, nullptr, two_candidates));
-        else ANPD_TRY(attn_enqueue<64>(m, kv, l, rows, max_pos, nullptr, two_candidates));
+        unsigned char* ao_img = decode ? ws.ci_ao : nullptr;
+        const int ao_rows = decode ? rows : 0;
+        if (decode && hd == 64) ANPD_TRY(attn_dec_enqueue(m, kv, l, two_candidates));
+        else if (hd == 128) ANPD_TRY(attn_enqueue<128>(m, kv, l, rows, max_pos, ao_img, two_candidates, ao_rows));
+        else ANPD_TRY(attn_enqueue<64>(m, kv, l, rows, max_pos, ao_img, two_candidates, ao_rows));
         ANPD_TRY(gemm_enqueue(m, kv, GK_O, l, rows, &segs, &seg_max));
         LAUNCH(pf, st, KC_OTHER, 0,
                (launch_k(resid_norm_kernel, rows, NORM_THREADS, 0, st, ws.x, ws.part, segs, sstride, ws.n_max_out, w.ffn_norm, c.rms_eps, d,
-                                                       ws.h_hi, ws.h_lo, seg_max)));
+                                                       ws.h_hi, ws.h_lo, seg_max, decode ? ws.ci_h : nullptr)));
         ANPD_TRY(gemm_enqueue(m, kv, GK_GU, l, rows, &segs, &seg_max));
         if (many_rows) LAUNCH(pf, st, KC_OTHER, 0,
                (launch_k(swiglu_wide_kernel, dim3((F / 4 + 511) / 512, rows), 256, 0, st, ws.part, segs, sstride, ws.n_max_out, F, ws.act_hi,
-                         ws.act_lo)));
+                         ws.act_lo, decode ? ws.ci_act : nullptr)));
         else LAUNCH(pf, st, KC_OTHER, 0,
                (launch_k(swiglu_kernel, dim3((F + 255) / 256, rows), 256, 0, st, ws.part, segs, sstride, ws.n_max_out, F, ws.act_hi,
-                                                                          ws.act_lo, seg_max)));
+                                                                          ws.act_lo, seg_max, decode ? ws.ci_act : nullptr)));
         ANPD_TRY(gemm_enqueue(m, kv, GK_DOWN, l, rows, &segs, &seg_max));
         const float* next_gain = (l + 1 < c.n_layers) ? m->layers[l + 1].attn_norm : m->final_norm;
         LAUNCH(pf, st, KC_OTHER, 0,
                (launch_k(resid_norm_kernel, rows, NORM_THREADS, 0, st, ws.x, ws.part, segs, sstride, ws.n_max_out, next_gain, c.rms_eps, d,
-                                                       ws.h_hi, ws.h_lo, seg_max)));
+                                                       ws.h_hi, ws.h_lo, seg_max, decode ? ws.ci_h : nullptr)));
     }
     if (!head) { CUDA_TRY(cudaGetLastError()); return ANPD_OK; }
-    int head_rows = rows;
-    if (rows != kv->batch * ANPD_ROWS) {
-        // A prompt pass needs the LM head for its last token only: the group of 8 rows that holds it moves to rows 0-7 and
-        // goes through the decode projection (the other rows of that launch are whatever the buffer holds; rows are independent).
-        head_rows = kv->batch * ANPD_ROWS;
+    // A prompt pass needs the LM head for its last token only: the group of 8 rows that holds it becomes rows 0-7 of a decode
+    // projection (the other rows of that launch, if any, are whatever the buffer holds; rows are independent).
+    const int group = (head_row / ANPD_ROWS) * ANPD_ROWS;
+    const bool prompt = rows != kv->batch * ANPD_ROWS;
+    if (prompt && !m->plain_gemm) {
+        const int img_rows = cl_fused(m->cl[GK_LM]) ? ANPD_ROWS : kv->batch * ANPD_ROWS;
         LAUNCH(pf, st, KC_OTHER, 0,
-               (launch_k(move_rows_kernel, ANPD_ROWS, 256, 0, st, ws.h_hi, ws.h_lo, (head_row / ANPD_ROWS) * ANPD_ROWS, d)));
+               (launch_k(rows_to_image_kernel, ANPD_ROWS, 256, 0, st, ws.h_hi, ws.h_lo, group, d, ws.ci_h, img_rows)));
+        if (cl_fused(m->cl[GK_LM])) return lm_head_cl_enqueue(m, kv, nullptr, 0, want_logits);
+    } else if (prompt) {
+        LAUNCH(pf, st, KC_OTHER, 0, (launch_k(move_rows_kernel, ANPD_ROWS, 256, 0, st, ws.h_hi, ws.h_lo, group, d)));
     }
-    ANPD_TRY(gemm_enqueue(m, kv, GK_LM, 0, head_rows, &segs));
-    rows = head_rows;
+    rows = kv->batch * ANPD_ROWS;
+    ANPD_TRY(gemm_enqueue(m, kv, GK_LM, 0, rows, &segs, &seg_max));
     LAUNCH(pf, st, KC_OTHER, 0,
-           (launch_k(argmax_partial_kernel, dim3(ws.amax_blocks, rows), 256, 0, st, ws.part, segs, (size_t)kv->batch * ANPD_ROWS * ws.n_max_out, ws.n_max_out, V,
+           (launch_k(argmax_partial_kernel, dim3(ws.amax_blocks, rows), 256, 0, st, ws.part, segs, (size_t)rows * ws.n_max_out, ws.n_max_out, V,
                                                                              want_logits ? ws.logits : nullptr, ws.amax_val,
                                                                              ws.amax_idx, ws.amax_blocks)));
     CUDA_TRY(cudaGetLastError());

@@ -2,8 +2,8 @@
 // bound by the tensor cores, not by reading the weights:  out[row][n] = sum_k W[n][k] * (a_hi[row][k] + a_lo[row][k]).
 //
 // A CTA owns an output tile of 256 features x 256 rows and walks the whole contraction dimension.  Per 64-wide k-block it
-// brings two 128-feature weight blocks (the same pre-swizzled 16 KB blocks the decode GEMM streams, any block is addressable
-// through gemm_block_slot) and the 256 rows' hi and lo activation tiles (four TMA boxes of 128 rows) into shared memory -
+// brings two 128-feature weight blocks (the storage the decode projections stream, see ClPlan: the 256 features are neighbours
+// in storage order, one linear copy per cluster they belong to) and the 256 rows' hi and lo activation tiles (four TMA boxes of 128 rows) into shared memory -
 // 96 KB for sixteen 128 x 256 x 16 MMAs - and accumulates W0 x hi, W0 x lo into one 256-column accumulator in tensor
 // memory and W1 x hi, W1 x lo into a second one: every activation byte is used against 256 features, every weight byte
 // against 256 rows.  Tiles that share a weight pair run on neighbouring CTAs at the same time, so a weight block crosses HBM
@@ -33,13 +33,15 @@ constexpr int PF_ERR_TIMEOUT = 205;
 
 struct PfArgs {
     float* out; int ld;
-    int N, rows;
-    int m_tiles, k_blocks, n_ft, n_tt, ksplit;
+    int rows;
+    int k_blocks, n_ft, n_tt, ksplit;
     int tail_from, tail_split;         // output tiles from tail_from on are cut into tail_split parts instead of ksplit
     size_t seg_stride;                 // elements between the partial-sum slabs of two K parts
-    long long total; int G;
+    ClPlan plan;
     int* err;
 };
+
+constexpr int PF_GROUPS = PF_BLOCK * 2 / 1024;           // groups of 8 features per output tile
 
 // work item -> (output tile, K part, parts of that tile); K part fastest
 __device__ __forceinline__ void pf_item(const PfArgs& g, int item, int& ot, int& ks, int& parts) {
@@ -49,12 +51,14 @@ __device__ __forceinline__ void pf_item(const PfArgs& g, int item, int& ot, int&
 }
 
 __global__ void __launch_bounds__(PF_THREADS, 1)
-gemm_pf_kernel(const bf16* __restrict__ w_blocks, const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ CUtensorMap map_lo,
-               const PfArgs g) {
+gemm_pf_kernel(const unsigned char* __restrict__ w, const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ CUtensorMap map_lo,
+               const __grid_constant__ PfArgs g) {
     extern __shared__ __align__(1024) unsigned char pf_smem_raw[];
     __shared__ uint64_t bar_full[PF_STAGES], bar_empty[PF_STAGES], bar_acc_full, bar_acc_empty;
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
+    __shared__ const unsigned char* piece_src[PF_GROUPS];             // the tile's groups as runs inside one cluster's storage
+    __shared__ int piece_step[PF_GROUPS], piece_at[PF_GROUPS], piece_bytes[PF_GROUPS];
 
     pdl_trigger();
     unsigned char* smem = pf_smem_raw + ((1024u - (smem_u32(pf_smem_raw) & 1023u)) & 1023u);
@@ -91,16 +95,26 @@ gemm_pf_kernel(const bf16* __restrict__ w_blocks, const __grid_constant__ CUtens
                 int ot, ks, parts;
                 pf_item(g, tile, ot, ks, parts);
                 const int ft = ot / g.n_tt, tt = ot - ft * g.n_tt;
-                const int t0 = 2 * ft, t1 = min(2 * ft + 1, g.m_tiles - 1);      // an odd tile count: the last pair repeats its tile
                 const int row0 = tt * PF_TILE_TOK;
+                const int g_begin = ft * PF_GROUPS, g_end = min(g_begin + PF_GROUPS, g.plan.n_units * g.plan.gpu);
+                int pieces = 0;
+                for (int grp = g_begin; grp < g_end; ++pieces) {
+                    const int c = cl_owner(g.plan, grp), c0 = cl_first_group(g.plan, c), c1 = cl_first_group(g.plan, c + 1), e = min(c1, g_end);
+                    piece_src[pieces] = w + ((size_t)c0 * g.k_blocks + (grp - c0)) * 1024;
+                    piece_step[pieces] = (c1 - c0) * 1024;
+                    piece_at[pieces] = (grp - g_begin) * 1024;
+                    piece_bytes[pieces] = (e - grp) * 1024;
+                    grp = e;
+                }
+                const uint32_t stage_bytes = (uint32_t)((g_end - g_begin) * 1024 + 4 * PF_BLOCK);
                 const int kb_end = (int)((long long)(ks + 1) * g.k_blocks / parts);
                 for (int kb = (int)((long long)ks * g.k_blocks / parts); kb < kb_end; ++kb) {
                     ok = mbar_wait(&bar_empty[stage], phase ^ 1u, abortp);
                     if (!ok) break;
                     unsigned char* st = smem + (size_t)stage * PF_STAGE;
-                    mbar_expect_tx(&bar_full[stage], (uint32_t)PF_STAGE);
-                    bulk_load(st, w_blocks + (size_t)gemm_block_slot((long long)t0 * g.k_blocks + kb, g.total, g.G) * (128 * 64), PF_BLOCK, &bar_full[stage], pol_w);
-                    bulk_load(st + PF_BLOCK, w_blocks + (size_t)gemm_block_slot((long long)t1 * g.k_blocks + kb, g.total, g.G) * (128 * 64), PF_BLOCK, &bar_full[stage], pol_w);
+                    mbar_expect_tx(&bar_full[stage], stage_bytes);
+                    for (int i = 0; i < pieces; ++i)
+                        bulk_load(st + piece_at[i], piece_src[i] + (size_t)kb * piece_step[i], (uint32_t)piece_bytes[i], &bar_full[stage], pol_w);
                     tma_load_2d(st + 2 * PF_BLOCK, &map_hi, kb * 64, row0, &bar_full[stage], pol_a);
                     tma_load_2d(st + 3 * PF_BLOCK, &map_hi, kb * 64, row0 + 128, &bar_full[stage], pol_a);
                     tma_load_2d(st + 4 * PF_BLOCK, &map_lo, kb * 64, row0, &bar_full[stage], pol_a);
@@ -174,15 +188,16 @@ gemm_pf_kernel(const bf16* __restrict__ w_blocks, const __grid_constant__ CUtens
             const int row0 = tt * PF_TILE_TOK;
 #pragma unroll 1
             for (int j = 0; j < 2; ++j) {
-                const int t = 2 * ft + j;
-                if (t >= g.m_tiles) break;
-                const int n = t * 128 + quad * 32 + lane;
+                const int pos0 = (2 * ft + j) * 128, n_pos = g.plan.n_units * g.plan.gpu * 8;
+                if (pos0 >= n_pos) break;
+                const int pos = pos0 + quad * 32 + lane;
+                const int n = pos < n_pos ? cl_feature(g.plan, pos) : g.plan.N;
 #pragma unroll 1
                 for (int c0 = 0; c0 < PF_TILE_TOK; c0 += 16) {
                     if (row0 + c0 >= g.rows) break;
                     float v[16];
                     tc_ld16(tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(j * 256 + c0), v);
-                    if (n < g.N) {
+                    if (n < g.plan.N) {
                         float* out = g.out + (size_t)ks * g.seg_stride + (size_t)(row0 + c0) * g.ld + n;
 #pragma unroll
                         for (int r = 0; r < 16; ++r)
@@ -244,7 +259,7 @@ PfSchedule gemm_pf_schedule(int n_ft, int n_tt, int k_blocks, int num_sms) {
     return best;
 }
 
-anpd_status gemm_pf_enqueue(const GemmPlan& plan, const bf16* w_blocks, const CUtensorMap& map_hi, const CUtensorMap& map_lo, int rows,
+anpd_status gemm_pf_enqueue(const ClPlan& plan, const unsigned char* w, const CUtensorMap& map_hi, const CUtensorMap& map_lo, int rows,
                             float* out, int ld, size_t seg_stride, PfSchedule sched, int num_sms, int* err, cudaStream_t st, Profiler* prof) {
     constexpr int smem = PF_STAGES * PF_STAGE + 1024;
     static bool attr_set[64] = {false};
@@ -252,17 +267,15 @@ anpd_status gemm_pf_enqueue(const GemmPlan& plan, const bf16* w_blocks, const CU
         CUDA_TRY(cudaFuncSetAttribute(gemm_pf_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     }
     PfArgs g;
-    g.out = out; g.ld = ld; g.N = plan.N; g.rows = rows;
-    g.m_tiles = plan.m_tiles; g.k_blocks = plan.k_blocks;
-    g.n_ft = (plan.m_tiles + 1) / 2;
+    g.out = out; g.ld = ld; g.rows = rows;
+    g.plan = plan; g.k_blocks = plan.kb;
+    g.n_ft = (plan.n_units * plan.gpu + PF_GROUPS - 1) / PF_GROUPS;
     g.n_tt = (rows + PF_TILE_TOK - 1) / PF_TILE_TOK;
-    g.total = (long long)plan.m_tiles * plan.k_blocks;
-    g.G = plan.grid;
     g.ksplit = sched.ksplit; g.tail_from = sched.tail_from; g.tail_split = sched.tail_split; g.seg_stride = seg_stride;
     g.err = err;
     const int grid = std::min(num_sms, sched.tail_from * sched.ksplit + (g.n_ft * g.n_tt - sched.tail_from) * sched.tail_split);
     LAUNCH(prof, st, KC_GEMM, 2.0 * (double)plan.N * (double)plan.K,
-           (launch_k(gemm_pf_kernel, grid, PF_THREADS, (size_t)smem, st, w_blocks, map_hi, map_lo, g)));
+           (launch_k(gemm_pf_kernel, grid, PF_THREADS, (size_t)smem, st, w, map_hi, map_lo, g)));
     CUDA_TRY(cudaGetLastError());
     return ANPD_OK;
 }

@@ -227,6 +227,78 @@ anpd_status rr_enqueue(int epi, const RRPlan& p, const unsigned char* w, const u
                        cudaStream_t st, Profiler* prof);
 
 // ---------------------------------------------------------------------------------------------
+// weight storage and decode projections (gemm_cl.cu)
+// ---------------------------------------------------------------------------------------------
+// What a projection does with its results: plain output, rotary embedding + append, residual add, SwiGLU, vocabulary argmax.
+enum ClKind { CL_RAW = 0, CL_QKV = 1, CL_RESID = 2, CL_GU = 3, CL_LM = 4 };
+constexpr int CL_CTAS = 4;             // CTAs per cluster
+// Bytes per CTA fetched into L2 ahead of the next projection, while the tail of this one, the hand-over and what lies between
+// leave HBM idle.  7B, four projections per layer in sequence: 78.8 us without, 76.4 at 64 KB, 77.5 at 128 KB and 84 at 512 KB
+// (the prefetches of CTAs that are through then delay the others' last copies).  13B, eight sequences: no gain beyond 64 KB.
+constexpr unsigned CL_LEAD = 64 * 1024;
+// Storage of an [N][K] weight matrix and its cut over the clusters of a decode projection.  The features are kept in an order
+// in which those that make one result together are neighbours: eight rotary pairs (dimensions i.., then i + hd/2..) or eight
+// gate features and their eight up features make a unit of two groups of 8; elsewhere a unit is one group.  Cluster c owns the
+// units [c * n_units / ncl, (c + 1) * n_units / ncl) and stores them as [k-block of 64][group], 1 KB per group and k-block: 8
+// rows of 128 bytes, 16-byte chunk c of row r at chunk position c ^ r, the shared-memory image the MMA reads (128-byte
+// swizzle).  So a run of groups of one k-block is one linear copy, for the decode kernel and for the prompt kernel alike.
+struct ClPlan { int kind, N, K, hd, F, gpu, n_units, kb, ncl, u_max; };
+// storage position of feature n (position = 8 * group + row of the group), and the feature at a position
+__host__ __device__ inline int cl_position(const ClPlan& p, int n) {
+    if (p.kind == CL_QKV) {
+        const int half = p.hd >> 1, head = n / p.hd, i = n % p.hd, side = i >= half ? 1 : 0, j = i - side * half;
+        return head * p.hd + (j >> 3) * 16 + side * 8 + (j & 7);
+    }
+    if (p.kind == CL_GU) { const int side = n >= p.F ? 1 : 0, j = n - side * p.F; return (j >> 3) * 16 + side * 8 + (j & 7); }
+    return n;
+}
+__host__ __device__ inline int cl_feature(const ClPlan& p, int pos) {
+    if (p.kind == CL_QKV) { const int head = pos / p.hd, i = pos % p.hd; return head * p.hd + (i >> 4) * 8 + ((i >> 3) & 1) * (p.hd >> 1) + (i & 7); }
+    if (p.kind == CL_GU) return ((pos >> 3) & 1) * p.F + (pos >> 4) * 8 + (pos & 7);
+    return pos;
+}
+__host__ __device__ inline int cl_owner(const ClPlan& p, int group) {                    // the cluster that owns a group
+    return (int)(((long long)(group / p.gpu + 1) * p.ncl - 1) / p.n_units);
+}
+__host__ __device__ inline int cl_first_group(const ClPlan& p, int cluster) { return (int)((long long)cluster * p.n_units / p.ncl) * p.gpu; }
+__host__ __device__ inline size_t cl_weight_offset(const ClPlan& p, int pos, int k) {   // byte offset of element (position, k)
+    const int grp = pos >> 3, r = pos & 7, c = cl_owner(p, grp), g0 = cl_first_group(p, c), gc = cl_first_group(p, c + 1) - g0;
+    return ((size_t)g0 * p.kb + (size_t)gc * (k >> 6) + (grp - g0)) * 1024 + (size_t)r * 128 + (size_t)((((k >> 3) & 7) ^ r) << 4) + (size_t)(k & 7) * 2;
+}
+// Operand image of the activations of a decode step: per 64-wide k-block 2 * rows operand rows of 128 bytes (hi parts of the
+// step's rows, then lo parts), 128-byte-swizzled.  Byte offset of element (operand row, k):
+__host__ __device__ inline size_t cl_img_offset(int rows, int r, int k) {
+    return (size_t)(k >> 6) * (size_t)(rows * 256) + (size_t)(r >> 3) * 1024 + (size_t)(r & 7) * 128 + (size_t)((((k >> 3) & 7) ^ (r & 7)) << 4) + (size_t)(k & 7) * 2;
+}
+inline size_t cl_img_bytes(int rows, int K) { return (size_t)((K + 63) / 64) * rows * 256; }
+struct ClEpilogue {                    // only the fields of the projection's kind are read
+    const float* ss_in = nullptr; int n_parts = 0; float inv_d = 0, eps = 0;            // n_parts = 0: the input is normalised already
+    const int *row_pos = nullptr, *row_slot = nullptr, *row_seq = nullptr, *row_ok = nullptr;
+    const float *rope_cos = nullptr, *rope_sin = nullptr; const int* page_table = nullptr;
+    int pages_per_seq = 0, Hq = 0, Hkv = 0, hd = 0; float q_scale = 0;
+    __nv_bfloat16 *q_hi = nullptr, *q_lo = nullptr, *kpool_l = nullptr, *vpool_l = nullptr;
+    float* x = nullptr; const float* gain = nullptr; float* ss_out = nullptr; int d = 0;
+    unsigned char* act_out = nullptr;
+    float* out = nullptr; float* amax_val = nullptr; int* amax_idx = nullptr;
+    // weights the projection fetches into L2 for the one after it, per CTA, and what was fetched for it the same way
+    const ClPlan* next = nullptr; const unsigned char* next_w = nullptr; unsigned next_lead = 0, own_lead = 0;
+};
+int cl_clusters();                      // clusters the current device runs at once, at most 32 (0: none, or no device)
+void cl_make_plan(ClPlan* p, int kind, int N, int K, int hd, int F, int ncl);
+size_t cl_storage_bytes(const ClPlan& p);
+bool cl_fused(const ClPlan& p);         // a single sequence's rows fit one pass, so that the projection can finish its results itself
+int cl_parts(const ClPlan& p);          // sums of squares / argmax candidates per row such a projection leaves, [row][part]
+// rows [row_off, row_off + rows) of a row-major source (bf16, or fp32 rounded to bf16); the storage must be zero before
+anpd_status cl_retile_enqueue(const ClPlan& p, const void* src, bool src_is_f32, int rows, int row_off, unsigned char* dst, cudaStream_t st);
+anpd_status cl_image_enqueue(const float* a_dev, int rows, int K, unsigned char* img, cudaStream_t st);
+// one sequence's 8 rows, with the epilogue of the plan's kind
+anpd_status cl_enqueue(const ClPlan& p, const unsigned char* w, const unsigned char* act, const ClEpilogue& e, int* err, cudaStream_t st, Profiler* prof);
+// any number of rows (a multiple of 8, at most 128): CL_CTAS partial sums per output, part[k][row][feature], added by the consumer
+anpd_status cl_partial_enqueue(const ClPlan& p, const unsigned char* w, const unsigned char* act, int rows, float* part, size_t part_stride, int ld_part,
+                               const ClPlan* next, const unsigned char* next_w, unsigned next_lead, unsigned own_lead, int* err, cudaStream_t st,
+                               Profiler* prof);
+
+// ---------------------------------------------------------------------------------------------
 // model, KV cache and workspace
 // ---------------------------------------------------------------------------------------------
 constexpr int KV_PAGE = 128;          // positions per KV page (= key chunk of one attention block)
@@ -245,11 +317,11 @@ struct GemmPlan {
 enum GemmKind { GK_QKV = 0, GK_O = 1, GK_GU = 2, GK_DOWN = 3, GK_LM = 4, GK_COUNT = 5 };
 
 struct LayerW {
-    // all four matrices in tiled storage (see gemm_tiled_elems)
-    const __nv_bfloat16* wqkv;        // [(Hq + 2 Hkv) * hd, d]  (q rows, then k rows, then v rows)
-    const __nv_bfloat16* wo;          // [d, Hq * hd]
-    const __nv_bfloat16* wgu;         // [2 F, d]  (gate rows, then up rows)
-    const __nv_bfloat16* wd;          // [d, F]
+    // all four matrices in cluster storage (see ClPlan)
+    const unsigned char* wqkv;        // [(Hq + 2 Hkv) * hd, d]  (q rows, then k rows, then v rows)
+    const unsigned char* wo;          // [d, Hq * hd]
+    const unsigned char* wgu;         // [2 F, d]  (gate rows, then up rows)
+    const unsigned char* wd;          // [d, F]
     const float* attn_norm;           // [d]
     const float* ffn_norm;            // [d]
 };
@@ -259,19 +331,25 @@ struct anpd_model {
     cudaStream_t stream;
     int dq, dkv, nqkv;
     const __nv_bfloat16* embed;       // [V, d]
-    const __nv_bfloat16* lm_head;     // [V, d], tiled storage
+    const unsigned char* lm_head;     // [V, d], cluster storage
     const float* final_norm;          // [d]
     std::vector<LayerW> layers;
     void* slab;
     size_t slab_bytes;
     double streamed_bytes;            // weight bytes one forward reads
+    ClPlan cl[GK_COUNT];
+    bool cl_all_fused;                // every projection of a single-sequence step finishes its own results
     GemmPlan plan[GK_COUNT];
+    // second copy of the projections in the block storage of gemm_tc.cu, for the persistent step kernel only (opt-in)
+    struct LayerBlocks { const __nv_bfloat16 *wqkv, *wo, *wgu, *wd; };
+    std::vector<LayerBlocks> block_layers;
+    const __nv_bfloat16* block_lm;
+    void* block_slab;
     int* d_plan_tables;               // device copies of the plans' tables
-    int* d_ones;                      // [tiles] all 1: segment counts of the plain GEMM
-    int* d_const_segs[4];             // [tiles] all k (k = 1..3): segment counts of a prompt-pass GEMM cut into k parts along K
+    int* d_ones;                      // [tiles] all 1: partial sums per tile of a projection that is not cut along K
+    int* d_const_segs[5];             // [tiles] all k (k = 1..4): partial sums per tile of a projection cut into k parts along K
     int* d_tail_segs[GK_COUNT];       // [tiles] segment counts of a prompt-pass GEMM whose last tiles alone are cut (PfSchedule)
     int tail_cfg[GK_COUNT];           // what d_tail_segs[kind] holds: first cut feature tile * 4 + parts, -1 = nothing yet
-    int max_segs;
     bool plain_gemm;                  // debugging aid: route GEMMs through the plain kernel
     // second copy of the projections in row-range storage, used by single-sequence steps (proj_rr.cu)
     RRPlan rr[GK_COUNT];
@@ -289,7 +367,6 @@ struct Workspace {
     int r_max;                        // rows any forward may use
     int prefill_rows;                 // rows of one prompt pass (a multiple of 256)
     int n_max_out;                    // widest GEMM output (max of nqkv, 2F, d, V)
-    int splits_max;
     int* row_tok; int* row_pos; int* row_seq; int* row_ok;    // [r_max]
     // two-candidate mode: the cache slot a row's K/V go to (its position otherwise) and a range of slots it must not see
     int* row_slot; int* row_hole_lo; int* row_hole_hi;          // [r_max]
@@ -297,7 +374,7 @@ struct Workspace {
     __nv_bfloat16 *h_hi, *h_lo;       // [r_max, d]   normalised input of QKV / gate-up / LM head
     __nv_bfloat16 *ao_hi, *ao_lo;     // [r_max, dq]  attention output, input of the O projection
     __nv_bfloat16 *act_hi, *act_lo;   // [r_max, F]   SwiGLU output, input of the down projection
-    float* part;                      // [splits_max, r_max, n_max_out] GEMM partial sums
+    float* part;                      // [3, r_max, n_max_out] partial sums of a prompt pass's projection
     __nv_bfloat16 *q_hi, *q_lo;       // [r_max, dq] rotated queries x log2(e)/sqrt(hd), as two bf16 terms
     float *attn_m, *attn_l, *attn_o;  // per (row, q head, key chunk): max, sum, weighted values
     float* logits;                    // [r_max, V]
@@ -308,13 +385,17 @@ struct Workspace {
     unsigned char *img_h, *img_h2, *img_ao, *img_act;
     float *ss_a, *ss_b;
     float* amax_val_rr; int* amax_idx_rr;
+    // decode steps: operand images of the four projection inputs, sums of squares per row of the residual stream (one per CTA
+    // and pass of the projection that left it; a: embedding or down, b: O), argmax candidates
+    unsigned char *ci_h, *ci_h2, *ci_ao, *ci_act;
+    float *ss_cl_a, *ss_cl_b;
+    float* amax_val_cl; int* amax_idx_cl;
     int amax_nblk;                    // argmax candidates per row left by the last forward (depends on the path it took)
     float* amax_val_use; int* amax_idx_use;   // ... and the arrays that hold them
     int* gemm_err;                    // device flag set by a GEMM kernel that gave up waiting
-    // TMA views of the activation buffers: [0] decode (batch*8 rows), [1] prompt passes (prefill_rows rows, boxes of 128 rows)
-    CUtensorMap map_h[2][2], map_ao[2][2], map_act[2][2];     // [mode][hi/lo]
+    // TMA views of the activation buffers of the prompt passes (prefill_rows rows, boxes of 128 rows)
+    CUtensorMap map_h[2], map_ao[2], map_act[2];              // [hi/lo]
     CUtensorMap map_q[2];             // the queries of a prompt pass (hi, lo) through boxes of 64 columns x 128 rows (head dimension 128)
-    int nb[2];                        // MMA N per mode (rows padded to a multiple of 16)
 };
 
 // Arguments of the persistent step kernel (step_kernel.cu), fixed for a (model, cache) pair.
@@ -361,7 +442,7 @@ struct anpd_kv {
     anpd_model* m;
     int batch, max_len, pages_per_seq, total_pages;
     __nv_bfloat16 *kpool, *vpool;     // per layer and page: K [Hkv][KV_PAGE][hd]; V transposed [Hkv][hd][KV_PAGE]
-    CUtensorMap map_k, map_v;         // TMA views of the two pools as [all page rows][hd] matrices (head dimension 128 only)
+    CUtensorMap map_k, map_v;         // TMA views of the two pools: K as [all page positions][hd], V as [all page dims][KV_PAGE]
     bool attn_tc;                     // attention on tcgen05 (head dimension 128); otherwise the mma.sync kernel
     bool attn_pf;                     // prompt passes: the 128-row kernel (attn_pf.cu); otherwise the 16-row kernel of attn_tc.cu
     int* page_table;                  // device [batch][pages_per_seq]
@@ -424,6 +505,9 @@ anpd_status accept_enqueue(anpd_model* m, anpd_kv* kv, int mode, const NgramDev*
 // attn_tc.cu: per-page attention partials for head dimension 128 (same outputs as the mma.sync kernel in forward.cu)
 // tree: the rows carry cache slots and hidden slot ranges of their own (two-candidate steps)
 anpd_status attn_tc_enqueue(anpd_model* m, anpd_kv* kv, int layer, int rows, int max_pos, bool tree = false);
+// attn_dec.cu: attention of a decode step, written straight to the O projection's operand image
+bool attn_dec_supported(const anpd_model* m);                // head dimension 64, or one query head per kv head
+anpd_status attn_dec_enqueue(anpd_model* m, anpd_kv* kv, int layer, bool tree);
 // attn_pf.cu: attention of a prompt pass with 128 query rows per CTA (head dimension 128, one query head per kv head)
 anpd_status attn_pf_enqueue(anpd_model* m, anpd_kv* kv, int layer, int rows);
 // attention of a prompt pass (one query head per kv head), written straight to the O projection's input
@@ -460,8 +544,8 @@ anpd_status gemm_tc_enqueue(const GemmPlan& plan, const __nv_bfloat16* w_blocks,
 // row tile count, so that a feature tile has one part count for all its rows).
 struct PfSchedule { int ksplit, tail_from, tail_split; };
 PfSchedule gemm_pf_schedule(int n_ft, int n_tt, int k_blocks, int num_sms);
-anpd_status gemm_pf_enqueue(const GemmPlan& plan, const __nv_bfloat16* w_blocks, const CUtensorMap& map_hi, const CUtensorMap& map_lo, int rows,
+anpd_status gemm_pf_enqueue(const ClPlan& plan, const unsigned char* w, const CUtensorMap& map_hi, const CUtensorMap& map_lo, int rows,
                             float* out, int ld, size_t seg_stride, PfSchedule sched, int num_sms, int* err, cudaStream_t st, Profiler* prof);
 // forward.cu: the plain (one warp per output feature) GEMM, kept as a cross-check
-anpd_status gemm_plain_enqueue(const GemmPlan& p, const __nv_bfloat16* W, const __nv_bfloat16* a_hi, const __nv_bfloat16* a_lo, int rows,
+anpd_status gemm_plain_enqueue(const ClPlan& p, const unsigned char* W, const __nv_bfloat16* a_hi, const __nv_bfloat16* a_lo, int rows,
                                float* part, int ld_part, cudaStream_t st, Profiler* prof);

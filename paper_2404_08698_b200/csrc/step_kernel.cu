@@ -4,7 +4,7 @@
 // The step is bound by reading every weight once, so the design goal is that the weight stream never stops.  Every CTA
 // walks the same program - per layer: QKV projection, attention, O projection, gate/up projection, down projection;
 // then the LM head - and its share of each projection is a fixed range of 16 KB weight blocks (the same ranges and the
-// same block storage as the stand-alone GEMM kernel, see gemm_block_slot).  Inside a CTA four roles run decoupled:
+// block storage of gemm_tc.cu, see gemm_block_slot).  Inside a CTA four roles run decoupled:
 //
 //   weight producer (1 thread)   walks the whole step's list of weight blocks and attention pages and keeps a deep
 //                                shared-memory ring full; it depends on nothing but free ring slots (only a KV page that
@@ -953,7 +953,7 @@ bool step_kernel_eligible(const anpd_model* m, const anpd_kv* kv) {
     // of kernels - handing a projection's result to the next one through global memory (partial sums, arrival counter,
     // tail, phase counter, operand fetch: five to seven dependent round trips, each slow while the rings prefetch) costs
     // more than the kernel boundaries it replaces.
-    if (std::getenv("ANPD_STEP_KERNEL") == nullptr || m->plain_gemm) return false;
+    if (std::getenv("ANPD_STEP_KERNEL") == nullptr || m->block_slab == nullptr || m->plain_gemm) return false;
     if (c.head_dim != 128 || c.n_q_heads != c.n_kv_heads) return false;
     if (c.d_model % TILE || c.d_ffn % TILE) return false;
     if (kv->batch * ANPD_ROWS > 64 || kv->pages_per_seq > ST_MAX_PAGES) return false;
@@ -1039,14 +1039,14 @@ anpd_status step_kernel_setup(anpd_model* m, anpd_kv* kv) {
     p.trace_cta = want_trace ? std::max(0, std::min(m->num_sms - 1, std::atoi(std::getenv("ANPD_STEP_TRACE")))) : 0;
     std::vector<StepLayer> hl(c.n_layers);
     for (int l = 0; l < c.n_layers; ++l) {
-        const LayerW& w = m->layers[l];
-        hl[l] = StepLayer{w.wqkv, w.wo, w.wgu, w.wd, w.attn_norm, w.ffn_norm};
+        const anpd_model::LayerBlocks& w = m->block_layers[l];
+        hl[l] = StepLayer{w.wqkv, w.wo, w.wgu, w.wd, m->layers[l].attn_norm, m->layers[l].ffn_norm};
     }
     CUDA_TRY(cudaMemcpyAsync(d_layers, hl.data(), sizeof(StepLayer) * hl.size(), cudaMemcpyHostToDevice, m->stream));
     CUDA_TRY(cudaStreamSynchronize(m->stream));
     p.layers = d_layers;
     p.map_k = kv->map_k; p.map_v = kv->map_v;
-    p.embed = m->embed; p.lm_head = m->lm_head; p.final_norm = m->final_norm;
+    p.embed = m->embed; p.lm_head = m->block_lm; p.final_norm = m->final_norm;
     p.L = c.n_layers; p.d = c.d_model; p.F = c.d_ffn; p.V = c.vocab; p.Hq = c.n_q_heads; p.Hkv = c.n_kv_heads; p.hd = c.head_dim;
     p.dq = m->dq; p.rows = rows; p.stages = stages;
     p.eps = c.rms_eps; p.q_scale = 1.4426950408889634f / sqrtf((float)c.head_dim);
