@@ -2,7 +2,7 @@
 // the paged cache, softmax, and the result as the O projection's operand image.
 //
 // What bounds it: the cache's pages from HBM at long contexts; at short ones a memory round trip, the merge and the launch.  The
-// pages of one kv head of one sequence are dealt to VR shares: share v takes the pages p with (p / PG) mod VR == v.  A step of few
+// pages of one kv head of one sequence are dealt to VR shares: share v takes the pages p with p mod VR == v.  A step of few
 // (sequence, head) pairs gives every share a CTA of its own, VR of them forming a cluster; a step of many has one CTA take the
 // shares one after the other.  A producer thread brings pages in through a ring of TMA copies (those no kernel of this step
 // writes before the dependency wait); sixteen warps compute, each on 16 keys at a time: block b of a share belongs to key slot
@@ -28,11 +28,11 @@ namespace {
 
 using namespace tc;
 
-constexpr int AD_WARPS = 16;             // compute warps; one more loads
-constexpr int AD_THREADS = 32 * (AD_WARPS + 1);
-constexpr int AD_COMPUTE = 32 * AD_WARPS;
 constexpr int AD_KEYS = 16;              // keys per block
-constexpr int AD_MAX_STAGES = 6;
+constexpr int AD_BLOCKS = KV_PAGE / AD_KEYS;
+constexpr int AD_MAX_CHUNKS = 6;
+constexpr int AD_SMEM_MAX = 216 * 1024;
+constexpr int AD_SMEM_PAIR = 111 * 1024; // two CTAs share an SM: another one of these, or one of the projection before or after
 constexpr int AD_ERR_TIMEOUT = 208;
 
 template <int HD, int G> struct AdCfg {
@@ -40,26 +40,38 @@ template <int HD, int G> struct AdCfg {
     static constexpr int NV = STACK ? 8 : 16;                // query vectors per tile
     static constexpr int Q = 8 * G;                          // query vectors per kv head
     static constexpr int MT = Q / NV;                        // tiles (= warps per key slot)
-    static constexpr int KW = AD_WARPS / MT;                 // key slots of a share: 16, 16, 8, 4
-    static constexpr int PG = KW > 8 ? 2 : 1;                // neighbouring pages of a share
+    static constexpr bool PAIR = G <= 2;
+    static constexpr int WARPS = PAIR ? 8 : 16;            // compute warps; one more loads
+    static constexpr int COMPUTE = 32 * WARPS, THREADS = COMPUTE + 32;
+    static constexpr int REGS = PAIR ? 104 : 96;
+    static constexpr int KW = WARPS / MT;                    // key slots of a share: 8, 8, 8, 4
     static constexpr int VR = G <= 2 ? 4 : 8;                // shares
     static constexpr int VO = Q / VR;                        // vectors a CTA of a cluster finishes
     static constexpr int OP = HD + 4;                        // padded row
     static constexpr int QP = HD * 2 + 16;                   // bytes per staged query row
     static constexpr int QROWS = STACK ? 16 : 32 * MT;
     static constexpr int V4 = HD / 4;
-    static constexpr int ITEMS = (Q * V4 + AD_COMPUTE - 1) / AD_COMPUTE;      // 4-dimension pieces of the result per thread
-    static constexpr int PAGE_BYTES = 2 * KV_PAGE * HD * 2;  // K and V^T
-    static constexpr int REST = 1024 + AD_WARPS * NV * OP * 4 + Q * HD * 4 + 2 * AD_WARPS * NV * 4 + 2 * Q * 4 + QROWS * QP;
-    static constexpr int STAGES_MAX = (225 * 1024 - REST) / PAGE_BYTES;
-    static constexpr int STAGES = STAGES_MAX < AD_MAX_STAGES ? STAGES_MAX : AD_MAX_STAGES;
-    static constexpr size_t SMEM = (size_t)STAGES * PAGE_BYTES + REST;
+    static constexpr int ITEMS = (Q * V4 + COMPUTE - 1) / COMPUTE;            // 4-dimension pieces of the result per thread
+    static constexpr int CHUNK = KV_PAGE * HD * 2;           // one copy: the page's K or its V^T
+    static constexpr int SLOTS = WARPS * NV * OP * 4;        // the slots' results
+    static constexpr int REST = 1024 + Q * HD * 4 + 2 * WARPS * NV * 4 + 2 * Q * 4 + QROWS * QP;
+    // PAIR (the steps with many kv heads, whose clusters fill the device): half an SM per CTA, in registers too, so that it starts
+    // beside a CTA of the projection before it and lets the next one start beside it, and 40 heads are resident at once.  7B, step
+    // of a short context 2.80 -> 2.69 ms, at 4096 keys 3.25 -> 3.14; one 13B sequence at 1024 keys 5.64 -> 5.35.  A CTA with one
+    // share has read its last page when the slots' results are written: they take the ring's place.  With 4 or 8 query heads per
+    // kv head few CTAs run and twice the warps serve better (1.1B: 881 us per step, with half the warps 908).
+    static constexpr int chunks(bool cluster) {
+        const int room = (PAIR ? AD_SMEM_PAIR : AD_SMEM_MAX) - REST - (PAIR && cluster ? 0 : SLOTS);
+        return room / CHUNK < AD_MAX_CHUNKS ? room / CHUNK : AD_MAX_CHUNKS;
+    }
+    static constexpr int ring(bool cluster) { return PAIR && cluster && chunks(true) * CHUNK < SLOTS ? SLOTS : chunks(cluster) * CHUNK; }
+    static constexpr int smem(bool cluster) { return REST + ring(cluster) + (PAIR && cluster ? 0 : SLOTS); }
 };
 
 struct AdArgs {
     const bf16 *q_hi, *q_lo;
     const int *page_table, *row_pos, *row_seq, *row_slot, *hole_lo, *hole_hi;      // row_slot and the holes: null outside two-candidate steps
-    int pages_per_seq, Hkv, rows, layer_page0, cluster;       // cluster: VR or 1
+    int pages_per_seq, Hkv, rows, layer_page0, cluster, chunks, ring_bytes;       // cluster: VR or 1
     unsigned char* img;
     int* err;
 };
@@ -83,7 +95,7 @@ __device__ __forceinline__ uint32_t ad_map(const void* p, uint32_t cta) {
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_u32(p)), "r"(cta));
     return r;
 }
-__device__ __forceinline__ void ad_bar() { asm volatile("bar.sync 1, %0;" ::"n"(AD_COMPUTE) : "memory"); }
+template <int N> __device__ __forceinline__ void ad_bar() { asm volatile("bar.sync 1, %0;" ::"n"(N) : "memory"); }
 
 // a part (maximum pm, sum pl, values p) into the running result
 __device__ __forceinline__ void ad_fold(float& m, float& l, float4& a, float pm, float pl, float4 p) {
@@ -95,23 +107,23 @@ __device__ __forceinline__ void ad_fold(float& m, float& l, float4& a, float pm,
 }
 
 template <int HD, int G>
-__global__ void __launch_bounds__(AD_THREADS, 1) attn_dec_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v, const AdArgs g) {
+__global__ void __launch_bounds__((AdCfg<HD, G>::THREADS)) __maxnreg__((AdCfg<HD, G>::REGS)) attn_dec_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v, const AdArgs g) {
     typedef AdCfg<HD, G> Cfg;
     constexpr bool STACK = Cfg::STACK;
-    constexpr int NV = Cfg::NV, MT = Cfg::MT, KW = Cfg::KW, PG = Cfg::PG, VR = Cfg::VR, VO = Cfg::VO, OP = Cfg::OP, QP = Cfg::QP, V4 = Cfg::V4;
-    constexpr int KS = HD / 16, DT = HD / 8, NR = STACK ? 1 : 2, STAGES = Cfg::STAGES;      // NR: query vectors per thread
-    constexpr int KV_BYTES = KV_PAGE * HD * 2;
+    constexpr int NV = Cfg::NV, MT = Cfg::MT, KW = Cfg::KW, VR = Cfg::VR, WARPS = Cfg::WARPS, COMPUTE = Cfg::COMPUTE, VO = Cfg::VO, OP = Cfg::OP, QP = Cfg::QP, V4 = Cfg::V4;
+    constexpr int KS = HD / 16, DT = HD / 8, NR = STACK ? 1 : 2;      // NR: query vectors per thread
+    constexpr int CHUNK = Cfg::CHUNK;
     extern __shared__ __align__(1024) unsigned char ad_smem[];
-    __shared__ uint64_t full_k[STAGES], full_v[STAGES], empty[STAGES];
+    __shared__ uint64_t full[AD_MAX_CHUNKS], empty[AD_MAX_CHUNKS];
     __shared__ int abort_flag, s_issued;
     unsigned char* ring = ad_smem + ((1024u - (smem_u32(ad_smem) & 1023u)) & 1023u);
-    float* sm_o = (float*)(ring + (size_t)STAGES * Cfg::PAGE_BYTES);       // [warp][NV][OP]
-    float* recv = sm_o + AD_WARPS * NV * OP;                // cluster: [share][VO][HD], the shares of this CTA's vectors
+    float* recv = (float*)(ring + g.ring_bytes);            // cluster: [share][VO][HD], the shares of this CTA's vectors
     float* sm_m = recv + Cfg::Q * HD;                       // [warp][NV]
-    float* sm_l = sm_m + AD_WARPS * NV;
-    float* rc_m = sm_l + AD_WARPS * NV;                     // [share][VO]
+    float* sm_l = sm_m + WARPS * NV;
+    float* rc_m = sm_l + WARPS * NV;                        // [share][VO]
     float* rc_l = rc_m + Cfg::Q;
     unsigned char* Qs = (unsigned char*)(rc_l + Cfg::Q);
+    float* sm_o = Cfg::PAIR && g.cluster > 1 ? (float*)ring : (float*)(Qs + Cfg::QROWS * QP);       // [warp][NV][OP]
 
     pdl_trigger();
     asm volatile("barrier.cluster.arrive.release;" ::: "memory");          // waited for before the first remote store: every CTA runs then
@@ -127,11 +139,11 @@ __global__ void __launch_bounds__(AD_THREADS, 1) attn_dec_kernel(const __grid_co
     const int n_pages = pos_hi / KV_PAGE + 1;
     volatile int* abortp = &abort_flag;
 
-    if (warp == AD_WARPS) {
+    if (warp == WARPS) {
         if (elect_one()) {
             abort_flag = 0; s_issued = 0;
 #pragma unroll
-            for (int s = 0; s < STAGES; ++s) { mbar_init(&full_k[s], 1); mbar_init(&full_v[s], 1); mbar_init(&empty[s], PG == 2 ? AD_WARPS / 2 : AD_WARPS); }
+            for (int s = 0; s < AD_MAX_CHUNKS; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], WARPS); }
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         }
@@ -139,7 +151,7 @@ __global__ void __launch_bounds__(AD_THREADS, 1) attn_dec_kernel(const __grid_co
     }
     __syncthreads();
 
-    if (warp == AD_WARPS) {
+    if (warp == WARPS) {
         // ---------------- pages ----------------
         if (elect_one()) {
             const uint64_t pol = policy_evict_first();
@@ -148,29 +160,33 @@ __global__ void __launch_bounds__(AD_THREADS, 1) attn_dec_kernel(const __grid_co
             uint32_t phase = 1;
             bool waited = false, ok = true;
             for (int v = v_lo; v < v_hi && ok; ++v)
-                for (int p0 = v * PG; p0 < n_pages && ok; p0 += VR * PG)
-                    for (int p = p0; p < min(p0 + PG, n_pages); ++p) {
-                        if (!waited && (p + 1) * KV_PAGE > first_new) { pdl_wait(); waited = true; }       // holds rows the kernel before writes
-                        if (count >= STAGES) ok = mbar_wait(&empty[stage], phase, abortp);
+                for (int p = v; p < n_pages && ok; p += VR) {
+                    const int row = (g.layer_page0 + pages[p]) * g.Hkv + kvh;
+                    if (!waited && (p + 1) * KV_PAGE > first_new) { pdl_wait(); waited = true; }       // holds rows the kernel before writes
+#pragma unroll
+                    for (int half = 0; half < 2; ++half) {
+                        if (count >= g.chunks && ok) ok = mbar_wait(&empty[stage], phase, abortp);
                         if (!ok) break;
-                        const int row = (g.layer_page0 + pages[p]) * g.Hkv + kvh;
-                        unsigned char* kb = ring + (size_t)stage * Cfg::PAGE_BYTES;
-                        mbar_expect_tx(&full_k[stage], KV_BYTES);
+                        unsigned char* dst = ring + (size_t)stage * CHUNK;
+                        mbar_expect_tx(&full[stage], CHUNK);
+                        if (half == 0) {
 #pragma unroll
-                        for (int s = 0; s < HD / 64; ++s) tma_load_2d(kb + s * (KV_PAGE * 128), &map_k, s * 64, row * KV_PAGE, &full_k[stage], pol);
-                        mbar_expect_tx(&full_v[stage], KV_BYTES);
+                            for (int s = 0; s < HD / 64; ++s) tma_load_2d(dst + s * (KV_PAGE * 128), &map_k, s * 64, row * KV_PAGE, &full[stage], pol);
+                        } else {
 #pragma unroll
-                        for (int s = 0; s < 2; ++s) tma_load_2d(kb + KV_BYTES + s * (HD * 128), &map_v, s * 64, row * HD, &full_v[stage], pol);
+                            for (int s = 0; s < 2; ++s) tma_load_2d(dst + s * (HD * 128), &map_v, s * 64, row * HD, &full[stage], pol);
+                        }
                         ++count;
-                        if (++stage == STAGES) { stage = 0; phase ^= 1u; }
+                        if (++stage == g.chunks) { stage = 0; phase ^= 1u; }
                     }
+                }
             s_issued = count;
         }
         __syncwarp();
     } else {
         const int gid = lane >> 2, t = lane & 3, mt = warp % MT, ks = warp / MT;
         pdl_wait();                                         // the queries come from the kernel before
-        for (int idx = threadIdx.x; idx < Cfg::QROWS * (HD / 8); idx += AD_COMPUTE) {
+        for (int idx = threadIdx.x; idx < Cfg::QROWS * (HD / 8); idx += COMPUTE) {
             const int row = idx / (HD / 8), c = idx % (HD / 8);
             const bool lo = STACK ? row >= 8 : (row & 31) >= 16;
             const int vec = STACK ? row & 7 : (row >> 5) * 16 + (row & 15);
@@ -185,7 +201,7 @@ __global__ void __launch_bounds__(AD_THREADS, 1) attn_dec_kernel(const __grid_co
             qhl[h] = g.row_slot ? g.hole_lo[r0 + r] : 0;
             qhh[h] = g.row_slot ? g.hole_hi[r0 + r] : 0;
         }
-        ad_bar();
+        ad_bar<COMPUTE>();
         // lane offsets of the ldmatrix addresses: matrix (lane / 8) of four
         const int mi = lane >> 3, lr = lane & 7;
         const uint32_t q_addr = smem_u32(Qs) + (uint32_t)(((STACK ? 0 : mt * 32) + lr + 8 * (mi & 1)) * QP + (mi >> 1) * 16);
@@ -193,11 +209,12 @@ __global__ void __launch_bounds__(AD_THREADS, 1) attn_dec_kernel(const __grid_co
         const uint32_t ring_addr = smem_u32(ring);
 
         float m_run[NR], l_run[NR], o[DT][4];
-        auto block = [&](uint32_t kb, int key_page, int p, uint32_t par, int stage) {       // keys key_page .. + 15 of page p
+        // keys key_page .. + 15 of page p: its K chunk (given back after the last block's scores), its V chunk
+        auto block = [&](int ck, int cv, uint32_t par_v, int key_page, int p, bool last) {
             float c[2][4];
 #pragma unroll
             for (int j = 0; j < 2; ++j) { c[j][0] = 0.f; c[j][1] = 0.f; c[j][2] = 0.f; c[j][3] = 0.f; }
-            const uint32_t kr = kb + kv_off + (uint32_t)key_page * 128u;
+            const uint32_t kr = ring_addr + (uint32_t)ck * (uint32_t)CHUNK + kv_off + (uint32_t)key_page * 128u;
 #pragma unroll
             for (int k = 0; k < KS; ++k) {
                 uint32_t b[4], a[4];
@@ -211,6 +228,7 @@ __global__ void __launch_bounds__(AD_THREADS, 1) attn_dec_kernel(const __grid_co
                     ad_mma(c[1], a, b[2], b[3]);
                 }
             }
+            if (Cfg::PAIR && last) { __syncwarp(); if (lane == 0) mbar_arrive(&empty[ck]); }       // the short ring waits for it
             uint32_t ph[4], pl[4];
             float resc[NR];
 #pragma unroll
@@ -250,8 +268,8 @@ __global__ void __launch_bounds__(AD_THREADS, 1) attn_dec_kernel(const __grid_co
 #pragma unroll
                 for (int d = 0; d < DT; ++d) { o[d][0] *= ra; o[d][1] *= ra; o[d][2] *= rb; o[d][3] *= rb; }
             }
-            mbar_wait(&full_v[stage], par, abortp);
-            const uint32_t vr = kb + KV_BYTES + kv_off + (uint32_t)((key_page >> 6) * (HD * 128)) + ((((uint32_t)((key_page & 63) >> 3) + chunk0) ^ (uint32_t)lr) << 4);
+            mbar_wait(&full[cv], par_v, abortp);
+            const uint32_t vr = ring_addr + (uint32_t)cv * (uint32_t)CHUNK + kv_off + (uint32_t)((key_page >> 6) * (HD * 128)) + ((((uint32_t)((key_page & 63) >> 3) + chunk0) ^ (uint32_t)lr) << 4);
 #pragma unroll
             for (int d = 0; d < DT / 2; ++d) {
                 uint32_t b[4];
@@ -270,27 +288,28 @@ __global__ void __launch_bounds__(AD_THREADS, 1) attn_dec_kernel(const __grid_co
         uint32_t par = 0;
         bool cluster_ready = false;
         for (int v = v_lo; v < v_hi; ++v) {
-            if (g.cluster == 1 && v * PG >= n_pages) break;  // the remaining shares hold nothing
+            if (g.cluster == 1 && v >= n_pages) break;   // the remaining shares hold nothing
 #pragma unroll
             for (int h = 0; h < NR; ++h) { m_run[h] = -CUDART_INF_F; l_run[h] = 0.0f; }
 #pragma unroll
             for (int d = 0; d < DT; ++d) { o[d][0] = 0.f; o[d][1] = 0.f; o[d][2] = 0.f; o[d][3] = 0.f; }
-            for (int p0 = v * PG; p0 < n_pages; p0 += VR * PG)
-                for (int i = 0; i < PG; ++i) {
-                    const int p = p0 + i;
-                    if (p >= n_pages) break;
-                    if (PG == 1 || (ks >> 3) == i) {
-                        mbar_wait(&full_k[stage], par, abortp);
-                        const uint32_t kb = ring_addr + (uint32_t)stage * (uint32_t)Cfg::PAGE_BYTES;
+            for (int p = v; p < n_pages; p += VR) {
+                const int ck = stage;
+                const uint32_t par_k = par;
+                if (++stage == g.chunks) { stage = 0; par ^= 1u; }
+                const int cv = stage;
+                const uint32_t par_v = par;
+                if (++stage == g.chunks) { stage = 0; par ^= 1u; }
+                mbar_wait(&full[ck], par_k, abortp);
+                bool freed = false;
 #pragma unroll 1
-                        for (int b = KW >= 8 ? ks & 7 : ks; b < KV_PAGE / AD_KEYS; b += (KW >= 8 ? 8 : KW))
-                            if (p * KV_PAGE + b * AD_KEYS <= pos_hi) block(kb, b * AD_KEYS, p, par, stage);
-                        mbar_wait(&full_v[stage], par, abortp);
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(&empty[stage]);
-                    }
-                    if (++stage == STAGES) { stage = 0; par ^= 1u; }
-                }
+                for (int b = ks; b < AD_BLOCKS; b += KW)
+                    if (p * KV_PAGE + b * AD_KEYS <= pos_hi) { freed = Cfg::PAIR && b + KW >= AD_BLOCKS; block(ck, cv, par_v, b * AD_KEYS, p, freed); }
+                mbar_wait(&full[cv], par_v, abortp);
+                __syncwarp();
+                if (lane == 0) { if (!freed) mbar_arrive(&empty[ck]); mbar_arrive(&empty[cv]); }
+            }
+            if (Cfg::PAIR && g.cluster > 1) ad_bar<COMPUTE>();            // the slots' results go where the pages were
             // ---- the share's key slots, in slot order ----
 #pragma unroll
             for (int h = 0; h < NR; ++h) {
@@ -307,11 +326,11 @@ __global__ void __launch_bounds__(AD_THREADS, 1) attn_dec_kernel(const __grid_co
                     *(float2*)(mine + (gid + 8) * OP + 8 * d + 2 * t) = make_float2(o[d][2], o[d][3]);
                 }
             }
-            ad_bar();
+            ad_bar<COMPUTE>();
             if (g.cluster > 1 && !cluster_ready) { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); cluster_ready = true; }
 #pragma unroll
             for (int i = 0; i < Cfg::ITEMS; ++i) {
-                const int idx = threadIdx.x + i * AD_COMPUTE;
+                const int idx = threadIdx.x + i * COMPUTE;
                 if (idx < Cfg::Q * V4) {
                     const int vec = idx / V4, d4 = idx % V4, tile = vec / NV, vi = vec % NV;
                     float mx = -CUDART_INF_F;
@@ -338,7 +357,7 @@ __global__ void __launch_bounds__(AD_THREADS, 1) attn_dec_kernel(const __grid_co
                     }
                 }
             }
-            if (v + 1 < v_hi) ad_bar();                      // the slots' results may be overwritten
+            if (v + 1 < v_hi) ad_bar<COMPUTE>();                      // the slots' results may be overwritten
         }
         // ---- the result, as hi + lo terms in the O projection's operand image ----
         auto store = [&](int vec, int d4, float l, float4 a) {
@@ -352,12 +371,12 @@ __global__ void __launch_bounds__(AD_THREADS, 1) attn_dec_kernel(const __grid_co
         if (g.cluster == 1) {
 #pragma unroll
             for (int i = 0; i < Cfg::ITEMS; ++i) {
-                const int idx = threadIdx.x + i * AD_COMPUTE;
+                const int idx = threadIdx.x + i * COMPUTE;
                 if (idx < Cfg::Q * V4) store(idx / V4, idx % V4, R_l[i], R_a[i]);
             }
         } else {
             asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
-            for (int idx = threadIdx.x; idx < VO * V4; idx += AD_COMPUTE) {
+            for (int idx = threadIdx.x; idx < VO * V4; idx += COMPUTE) {
                 const int vo = idx / V4, d4 = idx % V4;
                 float m = -CUDART_INF_F, l = 0.0f;
                 float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -370,17 +389,15 @@ __global__ void __launch_bounds__(AD_THREADS, 1) attn_dec_kernel(const __grid_co
     }
     // the loading warp and a CTA that is its own cluster take part in the cluster barriers too
     if (g.cluster == 1) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
-    else if (warp == AD_WARPS) {
+    else if (warp == WARPS) {
         asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
         asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
     }
     __syncthreads();
     if (threadIdx.x == 0 && abort_flag) {
         // gave up somewhere: let every copy already requested land before the CTA may exit
-        for (int i = max(0, s_issued - STAGES); i < s_issued; ++i) {
-            for (unsigned spin = 0; spin < WAIT_LIMIT && !mbar_try_wait(&full_k[i % STAGES], (uint32_t)((i / STAGES) & 1)); ++spin) {}
-            for (unsigned spin = 0; spin < WAIT_LIMIT && !mbar_try_wait(&full_v[i % STAGES], (uint32_t)((i / STAGES) & 1)); ++spin) {}
-        }
+        for (int i = max(0, s_issued - g.chunks); i < s_issued; ++i)
+            for (unsigned spin = 0; spin < WAIT_LIMIT && !mbar_try_wait(&full[i % g.chunks], (uint32_t)((i / g.chunks) & 1)); ++spin) {}
         atomicExch(g.err, AD_ERR_TIMEOUT);
     }
 }
@@ -389,12 +406,13 @@ template <int HD, int G>
 anpd_status launch_attn_dec(anpd_model* m, anpd_kv* kv, AdArgs& a) {
     typedef AdCfg<HD, G> Cfg;
     static bool attr_set[64] = {false};
-    if (first_call_on_device(attr_set)) CUDA_TRY(cudaFuncSetAttribute(attn_dec_kernel<HD, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::SMEM));
+    if (first_call_on_device(attr_set)) CUDA_TRY(cudaFuncSetAttribute(attn_dec_kernel<HD, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, std::max(Cfg::smem(true), Cfg::smem(false))));
     // A CTA per share or one per head, whichever takes fewer rounds of a share's work: about 7/8 of the SMs can hold clusters.
-    const int heads = a.Hkv * kv->batch, resident = std::max(1, m->num_sms * 7 / 8 / Cfg::VR);
-    a.cluster = (heads + resident - 1) / resident < Cfg::VR * ((heads + m->num_sms - 1) / m->num_sms) ? Cfg::VR : 1;
+    const int heads = a.Hkv * kv->batch, per_sm = Cfg::PAIR ? 2 : 1, resident = std::max(1, m->num_sms * 7 / 8 * per_sm / Cfg::VR);
+    a.cluster = (heads + resident - 1) / resident < Cfg::VR * ((heads + m->num_sms * per_sm - 1) / (m->num_sms * per_sm)) ? Cfg::VR : 1;
+    a.chunks = Cfg::chunks(a.cluster > 1); a.ring_bytes = Cfg::ring(a.cluster > 1);
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(a.cluster, a.Hkv, kv->batch); cfg.blockDim = dim3(AD_THREADS); cfg.dynamicSmemBytes = Cfg::SMEM; cfg.stream = m->stream;
+    cfg.gridDim = dim3(a.cluster, a.Hkv, kv->batch); cfg.blockDim = dim3(Cfg::THREADS); cfg.dynamicSmemBytes = Cfg::smem(a.cluster > 1); cfg.stream = m->stream;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = a.cluster; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
