@@ -156,7 +156,7 @@ static anpd_status model_make_plans(anpd_model* m) {
         ints += 2 * (size_t)m->plan[k].m_tiles;
         max_tiles = std::max(max_tiles, m->plan[k].m_tiles);
     }
-    ints += 4 * (size_t)max_tiles + (size_t)GK_COUNT * max_tiles;                   // constants 1..4, then a table per projection
+    ints += PF_MAX_PARTS * (size_t)max_tiles + (size_t)GK_COUNT * max_tiles;        // constants 1..8, then a table per projection
     std::vector<int> host(ints);
     CUDA_TRY(cudaMalloc((void**)&m->d_plan_tables, ints * sizeof(int)));
     size_t off = 0;
@@ -170,12 +170,12 @@ static anpd_status model_make_plans(anpd_model* m) {
     m->d_ones = m->d_plan_tables + off;
     for (int i = 0; i < max_tiles; ++i) host[off + i] = 1;
     m->d_const_segs[0] = m->d_const_segs[1] = m->d_ones;
-    for (int k = 2; k <= 4; ++k) {
+    for (int k = 2; k <= PF_MAX_PARTS; ++k) {
         m->d_const_segs[k] = m->d_plan_tables + off + (size_t)(k - 1) * max_tiles;
         for (int i = 0; i < max_tiles; ++i) host[off + (size_t)(k - 1) * max_tiles + i] = k;
     }
     for (int k = 0; k < GK_COUNT; ++k) {
-        m->d_tail_segs[k] = m->d_plan_tables + off + (size_t)(4 + k) * max_tiles;
+        m->d_tail_segs[k] = m->d_plan_tables + off + (size_t)(PF_MAX_PARTS + k) * max_tiles;
         m->tail_cfg[k] = -1;
     }
     CUDA_TRY(cudaMemcpy(m->d_plan_tables, host.data(), ints * sizeof(int), cudaMemcpyHostToDevice));
@@ -412,13 +412,14 @@ anpd_status anpd_kv_create(const anpd_model* cm, int max_len, int batch, int shu
     kv->h_len_stale.assign(batch, 0);
     Workspace& ws = kv->ws;
     ws.prefill_rows = std::min(PREFILL_ROWS_MAX, (kv->max_len + 255) / 256 * 256);
+    ws.pf_rows = 0;
     ws.r_max = std::max(ws.prefill_rows, batch * ANPD_ROWS);
     ws.n_max_out = (std::max(std::max(m->nqkv, 2 * c.d_ffn), std::max(c.d_model, c.vocab)) + 127) / 128 * 128;
     ws.amax_blocks = (c.vocab + 1023) / 1024;
     const size_t R = ws.r_max, d = c.d_model, F = c.d_ffn, V = c.vocab, hd = c.head_dim, half = hd / 2;
     const size_t pool = (size_t)c.n_layers * kv->total_pages * c.n_kv_heads * KV_PAGE * hd * 2;
     const size_t n_part = (size_t)R * c.n_q_heads * kv->pages_per_seq;
-    const int S = batch * ANPD_ROWS;                   // rows of a decode step
+    const int S = std::max(batch * ANPD_ROWS, CL_PROMPT_ROWS);      // rows of an operand image: a decode step's or a short prompt pass's
     struct Item { void** ptr; size_t bytes; };
     std::vector<Item> items = {
         {(void**)&kv->kpool, pool}, {(void**)&kv->vpool, pool},
@@ -431,7 +432,7 @@ anpd_status anpd_kv_create(const anpd_model* cm, int max_len, int batch, int shu
         {(void**)&ws.x, R * d * 4}, {(void**)&ws.h_hi, R * d * 2}, {(void**)&ws.h_lo, R * d * 2},
         {(void**)&ws.ao_hi, R * m->dq * 2}, {(void**)&ws.ao_lo, R * m->dq * 2},
         {(void**)&ws.act_hi, R * F * 2}, {(void**)&ws.act_lo, R * F * 2},
-        {(void**)&ws.part, 3 * R * ws.n_max_out * 4},    // prompt passes leave up to three partial sums per output (their cut along K)
+        {(void**)&ws.part, 3 * R * ws.n_max_out * 4},    // three partial sums per output, more where fewer rows are used
         {(void**)&ws.q_hi, R * m->dq * 2}, {(void**)&ws.q_lo, R * m->dq * 2},
         {(void**)&ws.attn_m, n_part * 4}, {(void**)&ws.attn_l, n_part * 4}, {(void**)&ws.attn_o, n_part * hd * 4},
         {(void**)&ws.logits, (size_t)batch * ANPD_ROWS * V * 4},
@@ -463,8 +464,8 @@ anpd_status anpd_kv_create(const anpd_model* cm, int max_len, int batch, int shu
         struct { CUtensorMap* maps; const bf16* hi; const bf16* lo; int K; } bufs[3] = {
             {ws.map_h, ws.h_hi, ws.h_lo, c.d_model}, {ws.map_ao, ws.ao_hi, ws.ao_lo, m->dq}, {ws.map_act, ws.act_hi, ws.act_lo, c.d_ffn}};
         for (auto& bdesc : bufs) {
-            if (rc == ANPD_OK) rc = make_tmap_bf16(&bdesc.maps[0], bdesc.hi, ws.prefill_rows, bdesc.K, 128, false);
-            if (rc == ANPD_OK) rc = make_tmap_bf16(&bdesc.maps[1], bdesc.lo, ws.prefill_rows, bdesc.K, 128, false);
+            if (rc == ANPD_OK) rc = make_tmap_bf16(&bdesc.maps[0], bdesc.hi, ws.prefill_rows, bdesc.K, 64, false);
+            if (rc == ANPD_OK) rc = make_tmap_bf16(&bdesc.maps[1], bdesc.lo, ws.prefill_rows, bdesc.K, 64, false);
         }
         if (rc != ANPD_OK) { cudaFreeHost(kv->h_seq); cudaFree(kv->slab); delete kv; return rc; }
     }

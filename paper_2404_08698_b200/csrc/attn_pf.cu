@@ -50,6 +50,7 @@ struct FaArgs {
     const int* row_pos; const int* row_seq;
     int H, Hkv, layer_row0, rows, n_row_tiles;      // query heads, kv heads (H a multiple of Hkv)
     bf16* ao_hi; bf16* ao_lo;
+    unsigned char* img;                     // the O projection's operand image (few rows) instead of ao_hi and ao_lo
     int* err;
 };
 
@@ -331,8 +332,9 @@ attn_pf_kernel(const __grid_constant__ CUtensorMap map_qh, const __grid_constant
                     const size_t out = (size_t)row * g.H * FA_HD + (size_t)h * FA_HD + half * 64 + ch * 32;
 #pragma unroll
                     for (int u = 0; u < 4; ++u) {
-                        *(uint4*)(g.ao_hi + out + 8 * u) = *(const uint4*)(hh + 4 * u);
-                        *(uint4*)(g.ao_lo + out + 8 * u) = *(const uint4*)(ll + 4 * u);
+                        const int k = h * FA_HD + half * 64 + ch * 32 + 8 * u;
+                        *(uint4*)(g.img ? (bf16*)(g.img + cl_img_offset(g.rows, row, k)) : g.ao_hi + out + 8 * u) = *(const uint4*)(hh + 4 * u);
+                        *(uint4*)(g.img ? (bf16*)(g.img + cl_img_offset(g.rows, g.rows + row, k)) : g.ao_lo + out + 8 * u) = *(const uint4*)(ll + 4 * u);
                     }
                 }
             }
@@ -356,7 +358,7 @@ attn_pf_kernel(const __grid_constant__ CUtensorMap map_qh, const __grid_constant
 
 // Attention of a prompt pass over `rows` rows (a multiple of 8; the row plan covers the padding) of sequence row_seq[0].
 // map_qh / map_ql: the pass's queries [rows][H * 128] seen through boxes of 64 columns x 128 rows.
-anpd_status attn_pf_enqueue(anpd_model* m, anpd_kv* kv, int layer, int rows) {
+anpd_status attn_pf_enqueue(anpd_model* m, anpd_kv* kv, int layer, int rows, unsigned char* img) {
     const anpd_model_config& c = m->cfg;
     Workspace& ws = kv->ws;
     static bool attr_set[64] = {false};
@@ -370,7 +372,7 @@ anpd_status attn_pf_enqueue(anpd_model* m, anpd_kv* kv, int layer, int rows) {
     g.layer_row0 = layer * kv->total_pages * c.n_kv_heads * KV_PAGE;
     g.rows = rows;
     g.n_row_tiles = (rows + FA_ROWS - 1) / FA_ROWS;
-    g.ao_hi = ws.ao_hi; g.ao_lo = ws.ao_lo;
+    g.ao_hi = ws.ao_hi; g.ao_lo = ws.ao_lo; g.img = img;
     g.err = ws.gemm_err;
     const int grid = std::min(m->num_sms, g.n_row_tiles * g.H);
     LAUNCH(&m->prof, m->stream, KC_ATTN, 0,

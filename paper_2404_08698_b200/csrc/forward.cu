@@ -1053,6 +1053,14 @@ __global__ void move_rows_kernel(bf16* __restrict__ h_hi, bf16* __restrict__ h_l
     }
 }
 
+// Whether the projections of a forward of `rows` rows run on the decode kernel (weights streamed once, four partial sums per
+// output, operand images): decode steps, and prompt passes of up to CL_PROMPT_ROWS rows - as many as the tensor memory holds for
+// it.  There the weights bound a pass and this kernel streams them better: 7B, pass of 77 tokens 8.7 -> 4.7 ms, of 128 5.5 ms,
+// where 129 on the prompt GEMM take 5.9.
+static bool cl_rows(const anpd_model* m, const anpd_kv* kv, int rows) {
+    return !m->plain_gemm && (rows == kv->batch * ANPD_ROWS || rows <= CL_PROMPT_ROWS);
+}
+
 // One projection of a prompt pass, of a step of several sequences or, with the plain GEMM, of any forward.  Returns the number
 // of partial sums per 128-feature storage tile its consumer must add.
 anpd_status gemm_enqueue(anpd_model* m, anpd_kv* kv, int kind, int layer, int rows, const int** seg_count_out, int* seg_max_out) {
@@ -1069,7 +1077,7 @@ anpd_status gemm_enqueue(anpd_model* m, anpd_kv* kv, int kind, int layer, int ro
         *seg_max_out = 1;
         return gemm_plain_enqueue(plan, W, a_hi, a_lo, rows, ws.part, ws.n_max_out, m->stream, &m->prof);
     }
-    if (rows == kv->batch * ANPD_ROWS) {               // a decode step: a partial sum per CTA of a cluster
+    if (cl_rows(m, kv, rows)) {                        // a partial sum per CTA of a cluster
         const unsigned char* act = kind == GK_O ? ws.ci_ao : kind == GK_DOWN ? ws.ci_act : ws.ci_h;
         *seg_count_out = m->d_const_segs[CL_CTAS];
         *seg_max_out = CL_CTAS;
@@ -1078,14 +1086,19 @@ anpd_status gemm_enqueue(anpd_model* m, anpd_kv* kv, int kind, int layer, int ro
         const int next = kind == GK_QKV ? GK_O : kind == GK_O ? GK_GU : kind == GK_GU ? GK_DOWN : last ? GK_LM : GK_QKV;
         const LayerW& lw = m->layers[layer];
         const unsigned char* next_w = kind == GK_QKV ? lw.wo : kind == GK_O ? lw.wgu : kind == GK_GU ? lw.wd : last ? m->lm_head : m->layers[layer + 1].wqkv;
-        return cl_partial_enqueue(plan, W, act, rows, ws.part, (size_t)rows * ws.n_max_out, ws.n_max_out, kind == GK_LM ? nullptr : &m->cl[next], next_w,
+        return cl_partial_enqueue(plan, W, act, rows, ws.part, (size_t)rows * ws.n_max_out, ws.n_max_out, kind == GK_LM || (next == GK_LM && rows != kv->batch * ANPD_ROWS) ? nullptr : &m->cl[next], next_w,
                                   CL_LEAD, kind == GK_QKV && layer == 0 ? 0 : CL_LEAD, ws.gemm_err, m->stream, &m->prof);
     }
-    // a prompt pass: complete sums, or up to three per output
-    const int m_tiles = m->plan[kind].m_tiles, n_ft = (m_tiles + 1) / 2, n_tt = (rows + 255) / 256;
-    const PfSchedule sched = gemm_pf_schedule(n_ft, n_tt, plan.kb, m->num_sms);
+    // a prompt pass: complete sums, or several per output
+    const int m_tiles = m->plan[kind].m_tiles;
+    if (ws.pf_rows != rows) {
+        for (int k = 0; k < GK_LM; ++k)
+            ws.pf_sched[k] = gemm_pf_schedule((m->plan[k].m_tiles + 1) / 2, rows, m->cl[k].kb, m->num_sms, std::min(PF_MAX_PARTS, 3 * ws.r_max / rows));
+        ws.pf_rows = rows;
+    }
+    const PfSchedule sched = ws.pf_sched[kind];
     if (sched.tail_split > 1) {                        // feature tiles from `first` on come in tail_split parts, the others in one
-        const int first = 2 * (sched.tail_from / n_tt), cfg = first * 4 + sched.tail_split;
+        const int first = 2 * (sched.tail_from / sched.n_tt), cfg = first * PF_MAX_PARTS + sched.tail_split;
         if (m->tail_cfg[kind] != cfg) {
             LAUNCH(&m->prof, m->stream, KC_OTHER, 0,
                    (launch_k(fill_tail_segs_kernel, (m_tiles + 127) / 128, 128, 0, m->stream, m->d_tail_segs[kind], m_tiles, first, sched.tail_split)));
@@ -1096,7 +1109,7 @@ anpd_status gemm_enqueue(anpd_model* m, anpd_kv* kv, int kind, int layer, int ro
         *seg_count_out = m->d_const_segs[sched.ksplit];
     }
     *seg_max_out = std::max(sched.ksplit, sched.tail_split);
-    return gemm_pf_enqueue(plan, W, maps[0], maps[1], rows, ws.part, ws.n_max_out, (size_t)ws.r_max * ws.n_max_out, sched, m->num_sms,
+    return gemm_pf_enqueue(plan, W, maps[0], maps[1], rows, ws.part, ws.n_max_out, (size_t)rows * ws.n_max_out, sched, m->num_sms,
                            ws.gemm_err, m->stream, &m->prof);
 }
 
@@ -1113,8 +1126,12 @@ anpd_status attn_enqueue(anpd_model* m, anpd_kv* kv, int layer, int rows, int ma
         CUDA_TRY(cudaFuncSetAttribute(attn_partial_kernel<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     }
     // a prompt pass: pages are folded in the kernel, nothing to merge (the older 16-row kernel knows one query head per kv head only)
-    if (HD == 128 && kv->attn_tc && rows != kv->batch * ANPD_ROWS && kv->attn_pf) return attn_pf_enqueue(m, kv, layer, rows);
-    if (HD == 128 && kv->attn_tc && rows != kv->batch * ANPD_ROWS && c.n_q_heads == c.n_kv_heads) return attn_prompt_enqueue(m, kv, layer, rows);
+    if (HD == 128 && kv->attn_tc && rows != kv->batch * ANPD_ROWS && kv->attn_pf) return attn_pf_enqueue(m, kv, layer, rows, img);
+    if (HD == 128 && kv->attn_tc && rows != kv->batch * ANPD_ROWS && c.n_q_heads == c.n_kv_heads) {
+        ANPD_TRY(attn_prompt_enqueue(m, kv, layer, rows));
+        if (img) LAUNCH(&m->prof, m->stream, KC_ATTN, 0, (launch_k(rows_to_image_kernel, rows, 256, 0, m->stream, ws.ao_hi, ws.ao_lo, 0, m->dq, img, rows)));
+        return ANPD_OK;
+    }
     if (HD == 128 && kv->attn_tc) {
         ANPD_TRY(attn_tc_enqueue(m, kv, layer, rows, max_pos, tree));
     } else {
@@ -1297,6 +1314,7 @@ anpd_status forward_enqueue(anpd_model* m, anpd_kv* kv, int rows, int max_pos, b
     if (m->rr_ready && kv->batch == 1 && rows == ANPD_ROWS && head && !m->plain_gemm && !two_candidates) return forward_rr_enqueue(m, kv, max_pos, want_logits);
     if (kv->step_ready && rows == kv->batch * ANPD_ROWS && head && !m->prof.on && !two_candidates) return step_kernel_enqueue(m, kv, max_pos, want_logits);
     const bool decode = rows == kv->batch * ANPD_ROWS && !m->plain_gemm;           // (or a prompt pass of as many rows)
+    const bool slab = cl_rows(m, kv, rows);
     if (decode && kv->batch == 1 && head && m->cl_all_fused) return forward_cl_enqueue(m, kv, max_pos, want_logits, two_candidates);
     const anpd_model_config& c = m->cfg;
     kv->ws.amax_nblk = kv->ws.amax_blocks;
@@ -1306,13 +1324,13 @@ anpd_status forward_enqueue(anpd_model* m, anpd_kv* kv, int rows, int max_pos, b
     cudaStream_t st = m->stream;
     Profiler* pf = &m->prof;
     const int d = c.d_model, F = c.d_ffn, hd = c.head_dim, V = c.vocab;
-    const size_t sstride = (size_t)(decode ? rows : ws.r_max) * ws.n_max_out;      // between the partial sums of an output (the K parts of a projection)
+    const size_t sstride = (size_t)rows * ws.n_max_out;                            // between the partial sums of an output (the K parts of a projection)
     const size_t layer_elems = (size_t)kv->total_pages * c.n_kv_heads * KV_PAGE * hd;
     const int* segs = nullptr;
     int seg_max = 1;                                   // the most partial sums a tile of the last projection has
 
     LAUNCH(pf, st, KC_OTHER, 0, (launch_k(embed_norm_kernel, rows, NORM_THREADS, 0, st, m->embed, ws.row_tok, m->layers[0].attn_norm, c.rms_eps, d,
-                                                                      ws.x, ws.h_hi, ws.h_lo, decode ? ws.ci_h : nullptr)));
+                                                                      ws.x, ws.h_hi, ws.h_lo, slab ? ws.ci_h : nullptr)));
     const bool many_rows = rows >= 64;                 // prefill passes: throughput-shaped launches of the small kernels
     const int rope_hpb = many_rows ? 256 / (hd / 2) : 1;            // heads per block of the rotary kernel
     for (int l = 0; l < c.n_layers; ++l) {
@@ -1335,27 +1353,27 @@ anpd_status forward_enqueue(anpd_model* m, anpd_kv* kv, int rows, int max_pos, b
                    ws.part, segs, sstride, ws.n_max_out, ws.row_pos, ws.row_slot, ws.row_seq, ws.row_ok, kv->rope_cos, kv->rope_sin,
                    kv->page_table, kv->pages_per_seq, c.n_q_heads, c.n_kv_heads, hd, 1.4426950408889634f / sqrtf((float)hd), ws.q_hi,
                    ws.q_lo, kv->kpool + l * layer_elems, kv->vpool + l * layer_elems, seg_max)));
-        unsigned char* ao_img = decode ? ws.ci_ao : nullptr;
-        const int ao_rows = decode ? rows : 0;
+        unsigned char* ao_img = slab ? ws.ci_ao : nullptr;
+        const int ao_rows = slab ? rows : 0;
         if (decode && hd == 64) ANPD_TRY(attn_dec_enqueue(m, kv, l, two_candidates));
         else if (hd == 128) ANPD_TRY(attn_enqueue<128>(m, kv, l, rows, max_pos, ao_img, two_candidates, ao_rows));
         else ANPD_TRY(attn_enqueue<64>(m, kv, l, rows, max_pos, ao_img, two_candidates, ao_rows));
         ANPD_TRY(gemm_enqueue(m, kv, GK_O, l, rows, &segs, &seg_max));
         LAUNCH(pf, st, KC_OTHER, 0,
                (launch_k(resid_norm_kernel, rows, NORM_THREADS, 0, st, ws.x, ws.part, segs, sstride, ws.n_max_out, w.ffn_norm, c.rms_eps, d,
-                                                       ws.h_hi, ws.h_lo, seg_max, decode ? ws.ci_h : nullptr)));
+                                                       ws.h_hi, ws.h_lo, seg_max, slab ? ws.ci_h : nullptr)));
         ANPD_TRY(gemm_enqueue(m, kv, GK_GU, l, rows, &segs, &seg_max));
         if (many_rows) LAUNCH(pf, st, KC_OTHER, 0,
                (launch_k(swiglu_wide_kernel, dim3((F / 4 + 511) / 512, rows), 256, 0, st, ws.part, segs, sstride, ws.n_max_out, F, ws.act_hi,
-                         ws.act_lo, decode ? ws.ci_act : nullptr)));
+                         ws.act_lo, slab ? ws.ci_act : nullptr)));
         else LAUNCH(pf, st, KC_OTHER, 0,
                (launch_k(swiglu_kernel, dim3((F + 255) / 256, rows), 256, 0, st, ws.part, segs, sstride, ws.n_max_out, F, ws.act_hi,
-                                                                          ws.act_lo, seg_max, decode ? ws.ci_act : nullptr)));
+                                                                          ws.act_lo, seg_max, slab ? ws.ci_act : nullptr)));
         ANPD_TRY(gemm_enqueue(m, kv, GK_DOWN, l, rows, &segs, &seg_max));
         const float* next_gain = (l + 1 < c.n_layers) ? m->layers[l + 1].attn_norm : m->final_norm;
         LAUNCH(pf, st, KC_OTHER, 0,
                (launch_k(resid_norm_kernel, rows, NORM_THREADS, 0, st, ws.x, ws.part, segs, sstride, ws.n_max_out, next_gain, c.rms_eps, d,
-                                                       ws.h_hi, ws.h_lo, seg_max, decode ? ws.ci_h : nullptr)));
+                                                       ws.h_hi, ws.h_lo, seg_max, decode || (slab && l + 1 < c.n_layers) ? ws.ci_h : nullptr)));
     }
     if (!head) { CUDA_TRY(cudaGetLastError()); return ANPD_OK; }
     // A prompt pass needs the LM head for its last token only: the group of 8 rows that holds it becomes rows 0-7 of a decode

@@ -1,17 +1,21 @@
 // Projection GEMM for prompt passes (Algorithm 1's LLM(prompt)): hundreds to thousands of rows at once, so the product is
 // bound by the tensor cores, not by reading the weights:  out[row][n] = sum_k W[n][k] * (a_hi[row][k] + a_lo[row][k]).
 //
-// A CTA owns an output tile of 256 features x 256 rows and walks the whole contraction dimension.  Per 64-wide k-block it
-// brings two 128-feature weight blocks (the storage the decode projections stream, see ClPlan: the 256 features are neighbours
-// in storage order, one linear copy per cluster they belong to) and the 256 rows' hi and lo activation tiles (four TMA boxes of 128 rows) into shared memory -
-// 96 KB for sixteen 128 x 256 x 16 MMAs - and accumulates W0 x hi, W0 x lo into one 256-column accumulator in tensor
-// memory and W1 x hi, W1 x lo into a second one: every activation byte is used against 256 features, every weight byte
-// against 256 rows.  Tiles that share a weight pair run on neighbouring CTAs at the same time, so a weight block crosses HBM
-// once per prompt pass and is served from L2 otherwise.  A projection with fewer tiles than would keep every SM busy is also cut
-// along K into `ksplit` equal parts (the same cut for every tile): part s leaves its sums in partial-sum slab s and the
-// consumers add the slabs in order, as they add the decode GEMM's segments.  A projection whose tiles fill some rounds of
-// CTAs and a fraction of one more has the tiles of that last round alone cut into 2 or 3 parts, so that the round takes a
-// half or a third of a tile's time on all SMs instead of a whole tile's time on some.
+// A CTA owns an output tile of 256 features x T rows and walks the whole contraction dimension; T is the pass's rows cut into
+// equal tiles of at most 256.  Per 64-wide k-block it brings two 128-feature weight blocks (the storage the decode projections
+// stream, see ClPlan: the 256 features are neighbours in storage order, one linear copy per cluster they belong to) and the T
+// rows' hi and lo activation tiles (TMA boxes of 64 rows) into shared memory - 96 KB for sixteen 128 x 256 x 16 MMAs at T = 256 -
+// and accumulates W0 x hi, W0 x lo into one 256-column accumulator in tensor memory and W1 x hi, W1 x lo into a second one:
+// every activation byte is used against 256 features, every weight byte against T rows.  The first weight blocks are requested
+// while the kernel before is still running.  Tiles that share a weight pair run on neighbouring CTAs at the same time, so a
+// weight block crosses HBM once per prompt pass and is served from L2 otherwise.  A projection with fewer tiles than would keep
+// every SM busy is also cut along K into `ksplit` equal parts (the same cut for every tile): part s leaves its sums in
+// partial-sum slab s and the consumers add the slabs in order, as they add the decode projections' parts.  A projection whose
+// tiles fill some rounds of CTAs and a fraction of one more has the tiles of that last round alone cut, so that the round takes
+// a fraction of a tile's time on all SMs instead of a whole tile's time on some.
+//
+// Measured per launch (tiles of 256 rows and up to three parts before): 7B down, 250 rows 87 -> 43 us; 1.1B, 333 rows: QKV 27 ->
+// 17, O 27 -> 16, gate-up 48 -> 33, down 52 -> 28; 7B at 1536 rows 199 + 91 + 346 + 185 us, 1.50 PFLOP/s over the layer.
 #include "internal.h"
 #include "tc_ptx.cuh"
 
@@ -26,15 +30,20 @@ using namespace tc;
 
 constexpr int PF_TILE_TOK = 256;
 constexpr int PF_THREADS = 192;          // warp 0: producer, warp 1: MMA issuer + tensor-memory owner, warps 2-5: epilogue
-constexpr int PF_BLOCK = 16384;          // one 128 x 64 bf16 operand tile
-constexpr int PF_STAGE = 6 * PF_BLOCK;   // W0, W1, hi rows 0-127, hi rows 128-255, lo rows 0-127, lo rows 128-255
-constexpr int PF_STAGES = 2;
+constexpr int PF_BLOCK = 16384;          // one 128 x 64 bf16 weight tile
+constexpr int PF_BOX = 8192;             // 64 rows x 64 bf16 of the activations
+constexpr int PF_SMEM = 224 * 1024;
+constexpr int PF_MAX_STAGES = 4;
 constexpr int PF_ERR_TIMEOUT = 205;
+
+// a k-block of a tile: W0, W1, the rows' hi boxes, their lo boxes
+__host__ __device__ constexpr int pf_stage_bytes(int boxes) { return 2 * PF_BLOCK + 2 * boxes * PF_BOX; }
 
 struct PfArgs {
     float* out; int ld;
     int rows;
     int k_blocks, n_ft, n_tt, ksplit;
+    int tile_rows, boxes, stages;
     int tail_from, tail_split;         // output tiles from tail_from on are cut into tail_split parts instead of ksplit
     size_t seg_stride;                 // elements between the partial-sum slabs of two K parts
     ClPlan plan;
@@ -42,6 +51,10 @@ struct PfArgs {
 };
 
 constexpr int PF_GROUPS = PF_BLOCK * 2 / 1024;           // groups of 8 features per output tile
+constexpr int PF_TILE_FT = 8 * PF_GROUPS;
+
+// rows of a tile when the pass is cut into n_tt: a multiple of 16 (the products' N)
+int pf_tile_rows(int rows, int n_tt) { return ((rows + n_tt - 1) / n_tt + 15) / 16 * 16; }
 
 // work item -> (output tile, K part, parts of that tile); K part fastest
 __device__ __forceinline__ void pf_item(const PfArgs& g, int item, int& ot, int& ks, int& parts) {
@@ -54,7 +67,7 @@ __global__ void __launch_bounds__(PF_THREADS, 1)
 gemm_pf_kernel(const unsigned char* __restrict__ w, const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ CUtensorMap map_lo,
                const __grid_constant__ PfArgs g) {
     extern __shared__ __align__(1024) unsigned char pf_smem_raw[];
-    __shared__ uint64_t bar_full[PF_STAGES], bar_empty[PF_STAGES], bar_acc_full, bar_acc_empty;
+    __shared__ uint64_t bar_full[PF_MAX_STAGES], bar_empty[PF_MAX_STAGES], bar_acc_full, bar_acc_empty;
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
     __shared__ const unsigned char* piece_src[PF_GROUPS];             // the tile's groups as runs inside one cluster's storage
@@ -67,7 +80,7 @@ gemm_pf_kernel(const unsigned char* __restrict__ w, const __grid_constant__ CUte
 
     if (threadIdx.x == 0) {
         abort_flag = 0;
-        for (int s = 0; s < PF_STAGES; ++s) { mbar_init(&bar_full[s], 1); mbar_init(&bar_empty[s], 1); }
+        for (int s = 0; s < PF_MAX_STAGES; ++s) { mbar_init(&bar_full[s], 1); mbar_init(&bar_empty[s], 1); }
         mbar_init(&bar_acc_full, 1); mbar_init(&bar_acc_empty, 4);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -82,20 +95,19 @@ gemm_pf_kernel(const unsigned char* __restrict__ w, const __grid_constant__ CUte
     const uint32_t tmem_base = *((volatile uint32_t*)&tmem_slot);
     volatile int* abortp = &abort_flag;
 
-    pdl_wait();                                        // the activations come from the kernel before
+    const int stage_size = pf_stage_bytes(g.boxes);
 
     if (warp == 0) {
-        if (lane == 0) {
+        if (elect_one()) {
             const uint64_t pol_w = policy_evict_last(), pol_a = policy_evict_last();    // both are re-read by other CTAs: keep them in L2
-            int stage = 0;
+            int stage = 0, issued = 0, ahead = 0;          // ahead: steps of the first item whose weights are already on their way
             uint32_t phase = 0;
-            long long issued = 0;
             bool ok = true;
             for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x) {
                 int ot, ks, parts;
                 pf_item(g, tile, ot, ks, parts);
                 const int ft = ot / g.n_tt, tt = ot - ft * g.n_tt;
-                const int row0 = tt * PF_TILE_TOK;
+                const int row0 = tt * g.tile_rows;
                 const int g_begin = ft * PF_GROUPS, g_end = min(g_begin + PF_GROUPS, g.plan.n_units * g.plan.gpu);
                 int pieces = 0;
                 for (int grp = g_begin; grp < g_end; ++pieces) {
@@ -106,38 +118,43 @@ gemm_pf_kernel(const unsigned char* __restrict__ w, const __grid_constant__ CUte
                     piece_bytes[pieces] = (e - grp) * 1024;
                     grp = e;
                 }
-                const uint32_t stage_bytes = (uint32_t)((g_end - g_begin) * 1024 + 4 * PF_BLOCK);
-                const int kb_end = (int)((long long)(ks + 1) * g.k_blocks / parts);
-                for (int kb = (int)((long long)ks * g.k_blocks / parts); kb < kb_end; ++kb) {
-                    ok = mbar_wait(&bar_empty[stage], phase ^ 1u, abortp);
-                    if (!ok) break;
-                    unsigned char* st = smem + (size_t)stage * PF_STAGE;
-                    mbar_expect_tx(&bar_full[stage], stage_bytes);
+                const uint32_t stage_bytes = (uint32_t)((g_end - g_begin) * 1024 + 2 * g.boxes * PF_BOX);
+                const int kb_begin = ks * g.k_blocks / parts, kb_end = (ks + 1) * g.k_blocks / parts;
+                auto weights = [&](int kb, int s) {
+                    unsigned char* st = smem + (size_t)s * stage_size;
+                    mbar_expect_tx(&bar_full[s], stage_bytes);
                     for (int i = 0; i < pieces; ++i)
-                        bulk_load(st + piece_at[i], piece_src[i] + (size_t)kb * piece_step[i], (uint32_t)piece_bytes[i], &bar_full[stage], pol_w);
-                    tma_load_2d(st + 2 * PF_BLOCK, &map_hi, kb * 64, row0, &bar_full[stage], pol_a);
-                    tma_load_2d(st + 3 * PF_BLOCK, &map_hi, kb * 64, row0 + 128, &bar_full[stage], pol_a);
-                    tma_load_2d(st + 4 * PF_BLOCK, &map_lo, kb * 64, row0, &bar_full[stage], pol_a);
-                    tma_load_2d(st + 5 * PF_BLOCK, &map_lo, kb * 64, row0 + 128, &bar_full[stage], pol_a);
+                        bulk_load(st + piece_at[i], piece_src[i] + (size_t)kb * piece_step[i], (uint32_t)piece_bytes[i], &bar_full[s], pol_w);
+                };
+                if (issued == 0) {
+                    for (; ahead < min(g.stages, kb_end - kb_begin); ++ahead) weights(kb_begin + ahead, ahead);
+                    pdl_wait();                            // the activations come from the kernel before
+                }
+                for (int kb = kb_begin; kb < kb_end; ++kb) {
+                    if (issued >= ahead) {
+                        ok = mbar_wait(&bar_empty[stage], phase ^ 1u, abortp);
+                        if (!ok) break;
+                        weights(kb, stage);
+                    }
+                    unsigned char* act = smem + (size_t)stage * stage_size + 2 * PF_BLOCK;
+                    for (int i = 0; i < g.boxes; ++i) {
+                        tma_load_2d(act + i * PF_BOX, &map_hi, kb * 64, row0 + 64 * i, &bar_full[stage], pol_a);
+                        tma_load_2d(act + (g.boxes + i) * PF_BOX, &map_lo, kb * 64, row0 + 64 * i, &bar_full[stage], pol_a);
+                    }
                     ++issued;
-                    if (++stage == PF_STAGES) { stage = 0; phase ^= 1u; }
+                    if (++stage == g.stages) { stage = 0; phase ^= 1u; }
                 }
             }
             if (!ok) {
                 // gave up: let every copy already issued land before the CTA may exit
-                const long long n = issued < PF_STAGES ? issued : PF_STAGES;
-                for (long long i = 0; i < n; ++i) {
-                    const long long idx = issued - 1 - i;
-                    const int s = (int)(idx % PF_STAGES);
-                    const uint32_t ph = (uint32_t)((idx / PF_STAGES) & 1);
-                    for (unsigned spin = 0; spin < WAIT_LIMIT && !mbar_try_wait(&bar_full[s], ph); ++spin) {}
-                }
+                for (int i = max(0, issued - g.stages); i < issued; ++i)
+                    for (unsigned spin = 0; spin < WAIT_LIMIT && !mbar_try_wait(&bar_full[i % g.stages], (uint32_t)((i / g.stages) & 1)); ++spin) {}
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            // fp32 accumulate, bf16 x bf16, both operands K-major, M = 128 (weight features), N = 256 (rows)
-            const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(256 >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+        if (elect_one()) {
+            // fp32 accumulate, bf16 x bf16, both operands K-major, M = 128 (weight features), N = the tile's rows
+            const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(g.tile_rows >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
             int stage = 0;
             uint32_t phase = 0;
             int done_tiles = 0;
@@ -148,18 +165,18 @@ gemm_pf_kernel(const unsigned char* __restrict__ w, const __grid_constant__ CUte
                 tc_fence_after();
                 int ot, ks, parts;
                 pf_item(g, tile, ot, ks, parts);
-                const int kb_begin = (int)((long long)ks * g.k_blocks / parts), kb_end = (int)((long long)(ks + 1) * g.k_blocks / parts);
+                const int kb_begin = ks * g.k_blocks / parts, kb_end = (ks + 1) * g.k_blocks / parts;
                 for (int kb = kb_begin; kb < kb_end; ++kb) {
                     ok = mbar_wait(&bar_full[stage], phase, abortp);
                     if (!ok) break;
                     tc_fence_after();
-                    const uint32_t sb = smem_u32(smem + (size_t)stage * PF_STAGE);
+                    const uint32_t sb = smem_u32(smem + (size_t)stage * stage_size);
 #pragma unroll
                     for (int j = 0; j < 2; ++j) {
                         const uint64_t dw = make_smem_desc(sb + j * PF_BLOCK);
 #pragma unroll
                         for (int half = 0; half < 2; ++half) {
-                            const uint64_t da = make_smem_desc(sb + (2 + 2 * half) * PF_BLOCK);     // 256 rows: two boxes, one after the other
+                            const uint64_t da = make_smem_desc(sb + 2 * PF_BLOCK + half * g.boxes * PF_BOX);       // the boxes lie one after the other
 #pragma unroll
                             for (int k16 = 0; k16 < 4; ++k16) {
                                 const uint64_t adv = (uint64_t)(k16 * 2);
@@ -168,7 +185,7 @@ gemm_pf_kernel(const unsigned char* __restrict__ w, const __grid_constant__ CUte
                         }
                     }
                     tc_commit(&bar_empty[stage]);
-                    if (++stage == PF_STAGES) { stage = 0; phase ^= 1u; }
+                    if (++stage == g.stages) { stage = 0; phase ^= 1u; }
                 }
                 if (!ok) break;
                 tc_commit(&bar_acc_full);
@@ -178,6 +195,7 @@ gemm_pf_kernel(const unsigned char* __restrict__ w, const __grid_constant__ CUte
         const int quad = warp & 3;
         int done_tiles = 0;
         bool ok = true;
+        pdl_wait();                                        // the sums of the projection before have been read
         for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x, ++done_tiles) {
             int ot, ks, parts;
             pf_item(g, tile, ot, ks, parts);
@@ -185,7 +203,7 @@ gemm_pf_kernel(const unsigned char* __restrict__ w, const __grid_constant__ CUte
             ok = mbar_wait(&bar_acc_full, (uint32_t)(done_tiles & 1), abortp);
             if (!ok) break;
             tc_fence_after();
-            const int row0 = tt * PF_TILE_TOK;
+            const int row0 = tt * g.tile_rows;
 #pragma unroll 1
             for (int j = 0; j < 2; ++j) {
                 const int pos0 = (2 * ft + j) * 128, n_pos = g.plan.n_units * g.plan.gpu * 8;
@@ -193,7 +211,7 @@ gemm_pf_kernel(const unsigned char* __restrict__ w, const __grid_constant__ CUte
                 const int pos = pos0 + quad * 32 + lane;
                 const int n = pos < n_pos ? cl_feature(g.plan, pos) : g.plan.N;
 #pragma unroll 1
-                for (int c0 = 0; c0 < PF_TILE_TOK; c0 += 16) {
+                for (int c0 = 0; c0 < g.tile_rows; c0 += 16) {
                     if (row0 + c0 >= g.rows) break;
                     float v[16];
                     tc_ld16(tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(j * 256 + c0), v);
@@ -223,54 +241,59 @@ gemm_pf_kernel(const unsigned char* __restrict__ w, const __grid_constant__ CUte
 
 }  // namespace
 
-// Steps on the busiest CTA when the work items go to the CTAs round robin (a tile's epilogue counts as about six steps).
-static long long pf_cost(int n_ot, int k_blocks, int num_sms, const PfSchedule& s) {
-    const int uniform = s.tail_from * s.ksplit;
-    const int n_items = uniform + (n_ot - s.tail_from) * s.tail_split;
-    const int grid = std::min(num_sms, n_items);
-    std::vector<long long> load((size_t)grid, 0);
-    for (int it = 0; it < n_items; ++it) {
-        const int parts = it < uniform ? s.ksplit : s.tail_split;
-        load[(size_t)(it % grid)] += (k_blocks + parts - 1) / parts + 6;
+// Cycles on the busiest CTA when the work items go to the CTAs round robin, and of the partial sums' way through memory.
+static long long pf_cost(int n_ft, int rows, int k_blocks, int num_sms, const PfSchedule& s) {
+    const int T = pf_tile_rows(rows, s.n_tt), n_ot = n_ft * s.n_tt, boxes = (T + 63) / 64;
+    // a k-block: 16 products of T / 2 cycles, or its bytes at about 48 a cycle and SM; an item: its epilogue and about a microsecond
+    const int step = std::max(8 * T, pf_stage_bytes(boxes) / 48), item = 48 * T + 2000;
+    const int uniform = s.tail_from * s.ksplit, tail = (n_ot - s.tail_from) * s.tail_split, grid = std::min(num_sms, uniform + tail);
+    const long long a = (long long)((k_blocks + s.ksplit - 1) / s.ksplit) * step + item;
+    const long long b = (long long)((k_blocks + s.tail_split - 1) / s.tail_split) * step + item;
+    long long worst = 0;
+    for (int i = 0; i < grid; ++i) {
+        const int nu = (uniform - i + grid - 1) / grid, n = (uniform + tail - i + grid - 1) / grid;
+        worst = std::max(worst, nu * a + (n - nu) * b);
     }
-    return *std::max_element(load.begin(), load.end());
+    // a sum is written, read and added: 8 bytes at about 3000 a cycle for the device
+    const long long sums = (long long)rows * PF_TILE_FT * ((long long)uniform + tail) / std::max(1, s.n_tt) * 8 / 3000;
+    return worst + sums;
 }
 
-// The cut along K with the fewest steps on the busiest SM: every tile in 1, 2 or 3 parts, or the tiles of the last, partly
-// filled round alone in 2 or 3 parts.
-PfSchedule gemm_pf_schedule(int n_ft, int n_tt, int k_blocks, int num_sms) {
-    const int n_ot = n_ft * n_tt;
-    PfSchedule best{1, n_ot, 1};
-    long long best_cost = pf_cost(n_ot, k_blocks, num_sms, best);
-    for (int s = 2; s <= 3; ++s) {
-        const PfSchedule c{s, n_ot, 1};
-        const long long cost = pf_cost(n_ot, k_blocks, num_sms, c);
-        if (cost < best_cost) { best = c; best_cost = cost; }
-    }
-    const int full = n_ot / num_sms;
-    if (full >= 1 && n_ot % num_sms != 0) {
-        const int from = (full * num_sms / n_tt) * n_tt;            // whole feature pairs stay uncut
-        for (int s = 2; s <= 3 && from > 0; ++s) {
-            const PfSchedule c{1, from, s};
-            const long long cost = pf_cost(n_ot, k_blocks, num_sms, c);
-            if (cost < best_cost) { best = c; best_cost = cost; }
-        }
+// The rows' tiles and the cut along K with the least cost: every tile in up to max_parts parts, or the tiles of the last, partly
+// filled round alone in 2 to 4.
+PfSchedule gemm_pf_schedule(int n_ft, int rows, int k_blocks, int num_sms, int max_parts) {
+    PfSchedule best{1, n_ft, 1, 1};
+    long long best_cost = -1;
+    const int least = (rows + PF_TILE_TOK - 1) / PF_TILE_TOK;
+    for (int n_tt = least; n_tt <= least + 1; ++n_tt) {
+        const int n_ot = n_ft * n_tt, full = n_ot / num_sms;
+        auto consider = [&](PfSchedule c) {
+            const long long cost = pf_cost(n_ft, rows, k_blocks, num_sms, c);
+            if (best_cost < 0 || cost < best_cost) { best = c; best_cost = cost; }
+        };
+        for (int s = 1; s <= std::min(max_parts, k_blocks); ++s) consider({s, n_ot, 1, n_tt});
+        const int from = (full * num_sms / n_tt) * n_tt;                // whole feature pairs stay uncut
+        if (from > 0 && from < n_ot)
+            for (int s = 2; s <= std::min(std::min(max_parts, 4), k_blocks); ++s) consider({1, from, s, n_tt});
     }
     return best;
 }
 
 anpd_status gemm_pf_enqueue(const ClPlan& plan, const unsigned char* w, const CUtensorMap& map_hi, const CUtensorMap& map_lo, int rows,
                             float* out, int ld, size_t seg_stride, PfSchedule sched, int num_sms, int* err, cudaStream_t st, Profiler* prof) {
-    constexpr int smem = PF_STAGES * PF_STAGE + 1024;
     static bool attr_set[64] = {false};
     if (first_call_on_device(attr_set)) {
-        CUDA_TRY(cudaFuncSetAttribute(gemm_pf_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+        CUDA_TRY(cudaFuncSetAttribute(gemm_pf_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, PF_SMEM));
     }
     PfArgs g;
     g.out = out; g.ld = ld; g.rows = rows;
     g.plan = plan; g.k_blocks = plan.kb;
     g.n_ft = (plan.n_units * plan.gpu + PF_GROUPS - 1) / PF_GROUPS;
-    g.n_tt = (rows + PF_TILE_TOK - 1) / PF_TILE_TOK;
+    g.n_tt = sched.n_tt;
+    g.tile_rows = pf_tile_rows(rows, g.n_tt);
+    g.boxes = (g.tile_rows + 63) / 64;
+    g.stages = std::min(PF_MAX_STAGES, (PF_SMEM - 1024) / pf_stage_bytes(g.boxes));
+    const int smem = g.stages * pf_stage_bytes(g.boxes) + 1024;
     g.ksplit = sched.ksplit; g.tail_from = sched.tail_from; g.tail_split = sched.tail_split; g.seg_stride = seg_stride;
     g.err = err;
     const int grid = std::min(num_sms, sched.tail_from * sched.ksplit + (g.n_ft * g.n_tt - sched.tail_from) * sched.tail_split);

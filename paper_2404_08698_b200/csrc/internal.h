@@ -235,6 +235,7 @@ constexpr int CL_CTAS = 4;             // CTAs per cluster
 // Bytes per CTA fetched into L2 ahead of the next projection, while the tail of this one, the hand-over and what lies between
 // leave HBM idle.  7B, four projections per layer in sequence: 78.8 us without, 76.4 at 64 KB, 77.5 at 128 KB and 84 at 512 KB
 // (the prefetches of CTAs that are through then delay the others' last copies).  13B, eight sequences: no gain beyond 64 KB.
+constexpr int CL_PROMPT_ROWS = 128;       // prompt passes of up to this many rows use the decode projections
 constexpr unsigned CL_LEAD = 64 * 1024;
 // Storage of an [N][K] weight matrix and its cut over the clusters of a decode projection.  The features are kept in an order
 // in which those that make one result together are neighbours: eight rotary pairs (dimensions i.., then i + hd/2..) or eight
@@ -347,9 +348,9 @@ struct anpd_model {
     void* block_slab;
     int* d_plan_tables;               // device copies of the plans' tables
     int* d_ones;                      // [tiles] all 1: partial sums per tile of a projection that is not cut along K
-    int* d_const_segs[5];             // [tiles] all k (k = 1..4): partial sums per tile of a projection cut into k parts along K
+    int* d_const_segs[9];             // [tiles] all k (k = 1..8): partial sums per tile of a projection cut into k parts along K
     int* d_tail_segs[GK_COUNT];       // [tiles] segment counts of a prompt-pass GEMM whose last tiles alone are cut (PfSchedule)
-    int tail_cfg[GK_COUNT];           // what d_tail_segs[kind] holds: first cut feature tile * 4 + parts, -1 = nothing yet
+    int tail_cfg[GK_COUNT];           // what d_tail_segs[kind] holds: first cut feature tile * 8 + parts, -1 = nothing yet
     bool plain_gemm;                  // debugging aid: route GEMMs through the plain kernel
     // second copy of the projections in row-range storage, used by single-sequence steps (proj_rr.cu)
     RRPlan rr[GK_COUNT];
@@ -363,6 +364,9 @@ struct anpd_model {
     Profiler prof;
 };
 
+// How a prompt pass's projection is cut: row tiles, parts along K of the output tiles before tail_from and from it on.
+struct PfSchedule { int ksplit, tail_from, tail_split, n_tt; };
+
 struct Workspace {
     int r_max;                        // rows any forward may use
     int prefill_rows;                 // rows of one prompt pass (a multiple of 256)
@@ -374,7 +378,9 @@ struct Workspace {
     __nv_bfloat16 *h_hi, *h_lo;       // [r_max, d]   normalised input of QKV / gate-up / LM head
     __nv_bfloat16 *ao_hi, *ao_lo;     // [r_max, dq]  attention output, input of the O projection
     __nv_bfloat16 *act_hi, *act_lo;   // [r_max, F]   SwiGLU output, input of the down projection
-    float* part;                      // [3, r_max, n_max_out] partial sums of a prompt pass's projection
+    float* part;                      // 3 * r_max * n_max_out partial sums of a projection: slabs of [rows][n_max_out]
+    int pf_rows;                      // the prompt pass pf_sched was made for (0: none yet)
+    PfSchedule pf_sched[GK_COUNT];
     __nv_bfloat16 *q_hi, *q_lo;       // [r_max, dq] rotated queries x log2(e)/sqrt(hd), as two bf16 terms
     float *attn_m, *attn_l, *attn_o;  // per (row, q head, key chunk): max, sum, weighted values
     float* logits;                    // [r_max, V]
@@ -509,7 +515,7 @@ anpd_status attn_tc_enqueue(anpd_model* m, anpd_kv* kv, int layer, int rows, int
 bool attn_dec_supported(const anpd_model* m);                // head dimension 64, or one query head per kv head
 anpd_status attn_dec_enqueue(anpd_model* m, anpd_kv* kv, int layer, bool tree);
 // attn_pf.cu: attention of a prompt pass with 128 query rows per CTA (head dimension 128, one query head per kv head)
-anpd_status attn_pf_enqueue(anpd_model* m, anpd_kv* kv, int layer, int rows);
+anpd_status attn_pf_enqueue(anpd_model* m, anpd_kv* kv, int layer, int rows, unsigned char* img);
 // attention of a prompt pass (one query head per kv head), written straight to the O projection's input
 anpd_status attn_prompt_enqueue(anpd_model* m, anpd_kv* kv, int layer, int rows);
 
@@ -542,8 +548,8 @@ anpd_status gemm_tc_enqueue(const GemmPlan& plan, const __nv_bfloat16* w_blocks,
 // tile fastest) are cut along K: tiles [0, tail_from) into `ksplit` equal parts each, tiles [tail_from, end) - those that would
 // form a last, partly filled round of CTAs - into `tail_split` parts (tail_from == tile count: no such tail; a multiple of the
 // row tile count, so that a feature tile has one part count for all its rows).
-struct PfSchedule { int ksplit, tail_from, tail_split; };
-PfSchedule gemm_pf_schedule(int n_ft, int n_tt, int k_blocks, int num_sms);
+PfSchedule gemm_pf_schedule(int n_ft, int rows, int k_blocks, int num_sms, int max_parts);
+constexpr int PF_MAX_PARTS = 8;
 anpd_status gemm_pf_enqueue(const ClPlan& plan, const unsigned char* w, const CUtensorMap& map_hi, const CUtensorMap& map_lo, int rows,
                             float* out, int ld, size_t seg_stride, PfSchedule sched, int num_sms, int* err, cudaStream_t st, Profiler* prof);
 // forward.cu: the plain (one warp per output feature) GEMM, kept as a cross-check

@@ -1,0 +1,50 @@
+"""Prompt passes at the row counts where their kernels change: the decode projections up to 128 rows, above that row tiles cut into
+equal multiples of 16 and up to eight parts along K."""
+import pytest
+import torch
+
+from helpers import as_bf16_values, gpu_model, new_stream, require_gpu, top2_margin
+from oracle.anpd import argmax_lowest
+from oracle.decoder import Decoder
+from workloads import ModelShape, make_weights, markov_prompt
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def A():
+    require_gpu()
+    from paper_2404_08698_b200 import binding
+    return binding
+
+
+@pytest.fixture(scope="module", params=[ModelShape(2, 1024, 8, 8, 128, 2816, 1000), ModelShape(2, 1024, 16, 2, 64, 1400, 1000)], ids=["hd128", "hd64g8"])
+def rig(A, request):
+    shape = request.param
+    w = make_weights(shape, 23, False, std=0.025)
+    m = gpu_model(A, shape, w, new_stream())
+    kv = A.anpd_kv_create(m, 640)
+    yield shape, m, kv, Decoder(shape, as_bf16_values(w), torch.float64, kv_dtype=torch.bfloat16)
+    A.anpd_kv_destroy(kv)
+    A.anpd_model_destroy(m)
+
+
+# 9: two groups of 8; 121 / 129: 128 rows on the decode projections, 136 on the prompt GEMM; 257: two tiles of 144 rows where one of
+# 256 would be a row short; 513: three; one handle for all, so that every cut follows another
+@pytest.mark.parametrize("plen", [9, 64, 121, 128, 129, 200, 256, 257, 513, 15])
+def test_prompt_logits_at_row_tile_edges(A, rig, plen):
+    shape, m, kv, dec = rig
+    prompt = markov_prompt(plen, shape.vocab, 2, 300 + plen).tolist()
+    draft = [int(t) for t in markov_prompt(7, shape.vocab, 2, 301 + plen)]
+    A.anpd_kv_truncate(kv, 0, 0)
+    first = A.anpd_prefill(m, kv, prompt)
+    got = torch.from_numpy(A.anpd_verify_logits(m, kv, first, draft, shape.vocab)).double()
+    cache = dec.new_cache()
+    lp = dec.forward(prompt, cache)
+    if top2_margin(lp[-1]) > 5e-2:
+        assert first == argmax_lowest(lp[-1])
+    want = dec.forward([first] + draft, cache)
+    # the two sides round the same cache to bf16; what is left is fp32 sums of two-term products (2^-17 of a term) and cache
+    # entries that round the other way (2^-9 of an entry, one in hundreds): well below 2^-9 of the logits' scale
+    err = float((got - want).abs().max())
+    assert err <= 2 ** -8 * max(1.0, float(want.abs().max())), err
