@@ -1275,6 +1275,10 @@ static anpd_status forward_cl_enqueue(anpd_model* m, anpd_kv* kv, int max_pos, b
     auto chain = [&](ClEpilogue& e, unsigned own, int next, const unsigned char* w) {
         e.own_lead = own; e.next = &m->cl[next]; e.next_w = w; e.next_lead = CL_LEAD;
     };
+    // Where the O projection's weights fit its first ring of copies, HBM has nothing left to read when the gate-up CTAs start
+    // beside it: these then fetch more of their own weights at once (1.1B: 885 -> 853 us per step; the 7B model, whose O
+    // projection still streams at that point, lost 20 of 2850 us by the same).
+    const bool o_in_ring = cl_storage_bytes(m->cl[GK_O]) <= CL_RING_SHARE * CL_CTAS * m->cl[GK_O].ncl;
     for (int l = 0; l < c.n_layers; ++l) {
         const LayerW& w = m->layers[l];
         ClEpilogue q;
@@ -1295,6 +1299,7 @@ static anpd_status forward_cl_enqueue(anpd_model* m, anpd_kv* kv, int max_pos, b
         ClEpilogue gu;
         gu.ss_in = ws.ss_cl_b; gu.n_parts = cl_parts(m->cl[GK_O]); gu.inv_d = 1.0f / (float)d; gu.eps = c.rms_eps; gu.act_out = ws.ci_act;
         chain(gu, CL_LEAD, GK_DOWN, w.wd);
+        gu.own_burst = o_in_ring ? CL_BURST : 0;
         ANPD_TRY(cl_enqueue(m->cl[GK_GU], w.wgu, ws.ci_h2, gu, ws.gemm_err, st, pf));
         ClEpilogue dn;
         dn.x = ws.x; dn.gain = (l + 1 < c.n_layers) ? m->layers[l + 1].attn_norm : m->final_norm; dn.ss_out = ws.ss_cl_a; dn.d = d;

@@ -59,7 +59,7 @@ struct ClArgs {
     // the projection after this one: its storage and cut, and how many bytes per CTA are fetched into L2 ahead (own: already done)
     const unsigned char* next_w;
     int next_kb, next_gpu, next_units, next_passes;
-    unsigned own_lead, next_lead;
+    unsigned own_lead, own_burst, next_lead;
     // RMSNorm of the input
     const float* ss_in; int n_parts; float inv_d, eps;
     // rotary + append
@@ -277,6 +277,7 @@ __global__ void __launch_bounds__(cl_threads(R), 1) gemm_cl_kernel(const __grid_
                 }
             };
             for (int i = 0; i < w_count; ++i) ahead((unsigned)g.stage_bytes);
+            for (unsigned b = 0; b < g.own_burst && cur < end; b += g.stage_bytes) ahead((unsigned)g.stage_bytes);
             while (w_p < passes) {
                 if (!mbar_wait(&w_empty[stage], phase, abortp)) break;
                 w_issue(stage);
@@ -833,7 +834,7 @@ anpd_status cl_enqueue(const ClPlan& p, const unsigned char* w, const unsigned c
     g.x = e.x; g.gain = e.gain; g.ss_out = e.ss_out; g.d = e.d; g.act_out = e.act_out;
     g.out = e.out; g.amax_val = e.amax_val; g.amax_idx = e.amax_idx;
     if (e.next) { g.next_w = e.next_w; g.next_kb = e.next->kb; g.next_gpu = e.next->gpu; g.next_units = e.next->n_units; g.next_passes = 1; g.next_lead = e.next_lead; }
-    g.own_lead = e.own_lead;
+    g.own_lead = e.own_lead; g.own_burst = e.own_burst;
     g.err = err;
     const double bytes = 2.0 * (double)p.N * (double)p.K;
     switch (p.kind) {
@@ -853,7 +854,7 @@ anpd_status cl_partial_enqueue(const ClPlan& p, const unsigned char* w, const un
     int smem = 0;
     ANPD_TRY(cl_args(&g, p, w, act, rows, cl_passes(p, rows), 0, &smem));
     if (next) { g.next_w = next_w; g.next_kb = next->kb; g.next_gpu = next->gpu; g.next_units = next->n_units; g.next_passes = cl_passes(*next, rows); g.next_lead = next_lead; }
-    g.own_lead = own_lead;
+    g.own_lead = own_lead; g.own_burst = 0;
     g.part = part; g.part_stride = part_stride; g.ld_part = ld_part; g.plan = p;
     g.err = err;
     return launch_cl<CL_RAW, 0>(g, smem, st, prof, 2.0 * (double)p.N * (double)p.K);

@@ -237,6 +237,8 @@ constexpr int CL_CTAS = 4;             // CTAs per cluster
 // (the prefetches of CTAs that are through then delay the others' last copies).  13B, eight sequences: no gain beyond 64 KB.
 constexpr int CL_PROMPT_ROWS = 128;       // prompt passes of up to this many rows use the decode projections
 constexpr unsigned CL_LEAD = 64 * 1024;
+constexpr unsigned CL_BURST = 128 * 1024;
+constexpr size_t CL_RING_SHARE = 96 * 1024;       // a CTA's weights that go out with the first ring of copies
 // Storage of an [N][K] weight matrix and its cut over the clusters of a decode projection.  The features are kept in an order
 // in which those that make one result together are neighbours: eight rotary pairs (dimensions i.., then i + hd/2..) or eight
 // gate features and their eight up features make a unit of two groups of 8; elsewhere a unit is one group.  Cluster c owns the
@@ -283,6 +285,7 @@ struct ClEpilogue {                    // only the fields of the projection's ki
     float* out = nullptr; float* amax_val = nullptr; int* amax_idx = nullptr;
     // weights the projection fetches into L2 for the one after it, per CTA, and what was fetched for it the same way
     const ClPlan* next = nullptr; const unsigned char* next_w = nullptr; unsigned next_lead = 0, own_lead = 0;
+    unsigned own_burst = 0;             // what the projection fetches into L2 of its own weights at its start, beyond that
 };
 int cl_clusters();                      // clusters the current device runs at once, at most 32 (0: none, or no device)
 void cl_make_plan(ClPlan* p, int kind, int N, int K, int hd, int F, int ncl);
