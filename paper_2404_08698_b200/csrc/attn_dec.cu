@@ -2,16 +2,16 @@
 // the paged cache, softmax, and the result as the O projection's operand image.
 //
 // What bounds it: the cache's pages from HBM at long contexts; at short ones a memory round trip, the merge and the launch.  The
-// pages of one kv head of one sequence are dealt to VR shares: share v takes the pages p with p mod VR == v.  A step of few
-// (sequence, head) pairs gives every share a CTA of its own, VR of them forming a cluster; a step of many has one CTA take the
-// shares one after the other.  A producer thread brings pages in through a ring of TMA copies (those no kernel of this step
-// writes before the dependency wait); sixteen warps compute, each on 16 keys at a time: block b of a share belongs to key slot
-// b mod KW and to the MT warps of that slot, one per 16-row tile of query vectors.
+// pages of one kv head of one sequence are dealt to the CTAs of a cluster: CTA v of C takes the pages p with p mod C == v, C (1, 2,
+// 4, and 8 with 4 or 8 query heads per kv head) being as many as the device holds at once.  A producer thread brings pages in
+// through a ring of TMA copies (those no kernel of this step writes before the dependency wait); eight or sixteen warps compute,
+// each on 16 keys at a time: block b of a page belongs to key slot b mod KW and to the MT warps of that slot, one per 16-row tile
+// of query vectors.
 //
-// Order.  A slot takes its blocks in ascending order with a running maximum; the slots of a share are merged in slot order, the
-// shares in share order, each into the running result.  All of it depends on absolute key positions and head counts only, and a
-// masked key contributes an exact zero, so a row's result does not depend on the rows it shares the step with, on the batch, on
-// who computes a share, or on how far the cache reaches behind the row.
+// Order.  A slot takes its blocks in ascending order with a running maximum; the slots of a CTA are merged in slot order, the
+// CTAs in rank order, each into the running result.  All of it depends on absolute key positions and on the handle (heads and
+// sequences) only, and a masked key contributes an exact zero, so a row's result does not depend on the rows it shares the step
+// with or on how far the cache reaches behind the row.
 //
 // mma.sync m16n8k16 (bf16, fp32 sums): with 8 to 64 query vectors per kv head the products are small beside the loads.  Queries
 // and weights enter as two bf16 terms; with one query head per kv head the two terms of the 8 rows are the tile's 16 rows.
@@ -45,33 +45,29 @@ template <int HD, int G> struct AdCfg {
     static constexpr int COMPUTE = 32 * WARPS, THREADS = COMPUTE + 32;
     static constexpr int REGS = PAIR ? 104 : 96;
     static constexpr int KW = WARPS / MT;                    // key slots of a share: 8, 8, 8, 4
-    static constexpr int VR = G <= 2 ? 4 : 8;                // shares
-    static constexpr int VO = Q / VR;                        // vectors a CTA of a cluster finishes
+    static constexpr int C_MAX = PAIR ? 4 : 8;               // CTAs of a cluster
     static constexpr int OP = HD + 4;                        // padded row
     static constexpr int QP = HD * 2 + 16;                   // bytes per staged query row
     static constexpr int QROWS = STACK ? 16 : 32 * MT;
     static constexpr int V4 = HD / 4;
-    static constexpr int ITEMS = (Q * V4 + COMPUTE - 1) / COMPUTE;            // 4-dimension pieces of the result per thread
     static constexpr int CHUNK = KV_PAGE * HD * 2;           // one copy: the page's K or its V^T
     static constexpr int SLOTS = WARPS * NV * OP * 4;        // the slots' results
     static constexpr int REST = 1024 + Q * HD * 4 + 2 * WARPS * NV * 4 + 2 * Q * 4 + QROWS * QP;
     // PAIR (the steps with many kv heads, whose clusters fill the device): half an SM per CTA, in registers too, so that it starts
     // beside a CTA of the projection before it and lets the next one start beside it, and 40 heads are resident at once.  7B, step
-    // of a short context 2.80 -> 2.69 ms, at 4096 keys 3.25 -> 3.14; one 13B sequence at 1024 keys 5.64 -> 5.35.  A CTA with one
-    // share has read its last page when the slots' results are written: they take the ring's place.  With 4 or 8 query heads per
-    // kv head few CTAs run and twice the warps serve better (1.1B: 881 us per step, with half the warps 908).
-    static constexpr int chunks(bool cluster) {
-        const int room = (PAIR ? AD_SMEM_PAIR : AD_SMEM_MAX) - REST - (PAIR && cluster ? 0 : SLOTS);
-        return room / CHUNK < AD_MAX_CHUNKS ? room / CHUNK : AD_MAX_CHUNKS;
-    }
-    static constexpr int ring(bool cluster) { return PAIR && cluster && chunks(true) * CHUNK < SLOTS ? SLOTS : chunks(cluster) * CHUNK; }
-    static constexpr int smem(bool cluster) { return REST + ring(cluster) + (PAIR && cluster ? 0 : SLOTS); }
+    // of a short context 2.80 -> 2.69 ms, at 4096 keys 3.25 -> 3.14; one 13B sequence at 1024 keys 5.64 -> 5.35.  The CTA has read
+    // its last page when the slots' results are written: they take the ring's place.  With 4 or 8 query heads per kv head few CTAs
+    // run and twice the warps serve better (1.1B: 881 us per step, with half the warps 908).
+    static constexpr int ROOM = (PAIR ? AD_SMEM_PAIR : AD_SMEM_MAX) - REST - (PAIR ? 0 : SLOTS);
+    static constexpr int CHUNKS = ROOM / CHUNK < AD_MAX_CHUNKS ? ROOM / CHUNK : AD_MAX_CHUNKS;
+    static constexpr int RING = PAIR && CHUNKS * CHUNK < SLOTS ? SLOTS : CHUNKS * CHUNK;
+    static constexpr int SMEM = REST + RING + (PAIR ? 0 : SLOTS);
 };
 
 struct AdArgs {
     const bf16 *q_hi, *q_lo;
     const int *page_table, *row_pos, *row_seq, *row_slot, *hole_lo, *hole_hi;      // row_slot and the holes: null outside two-candidate steps
-    int pages_per_seq, Hkv, rows, layer_page0, cluster, chunks, ring_bytes;       // cluster: VR or 1
+    int pages_per_seq, Hkv, rows, layer_page0;
     unsigned char* img;
     int* err;
 };
@@ -110,26 +106,25 @@ template <int HD, int G>
 __global__ void __launch_bounds__((AdCfg<HD, G>::THREADS)) __maxnreg__((AdCfg<HD, G>::REGS)) attn_dec_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v, const AdArgs g) {
     typedef AdCfg<HD, G> Cfg;
     constexpr bool STACK = Cfg::STACK;
-    constexpr int NV = Cfg::NV, MT = Cfg::MT, KW = Cfg::KW, VR = Cfg::VR, WARPS = Cfg::WARPS, COMPUTE = Cfg::COMPUTE, VO = Cfg::VO, OP = Cfg::OP, QP = Cfg::QP, V4 = Cfg::V4;
+    constexpr int NV = Cfg::NV, MT = Cfg::MT, KW = Cfg::KW, WARPS = Cfg::WARPS, COMPUTE = Cfg::COMPUTE, CHUNKS = Cfg::CHUNKS, OP = Cfg::OP, QP = Cfg::QP, V4 = Cfg::V4;
     constexpr int KS = HD / 16, DT = HD / 8, NR = STACK ? 1 : 2;      // NR: query vectors per thread
     constexpr int CHUNK = Cfg::CHUNK;
     extern __shared__ __align__(1024) unsigned char ad_smem[];
     __shared__ uint64_t full[AD_MAX_CHUNKS], empty[AD_MAX_CHUNKS];
     __shared__ int abort_flag, s_issued;
     unsigned char* ring = ad_smem + ((1024u - (smem_u32(ad_smem) & 1023u)) & 1023u);
-    float* recv = (float*)(ring + g.ring_bytes);            // cluster: [share][VO][HD], the shares of this CTA's vectors
+    float* recv = (float*)(ring + Cfg::RING);               // [CTA][VO][HD], the cluster's parts of this CTA's vectors
     float* sm_m = recv + Cfg::Q * HD;                       // [warp][NV]
     float* sm_l = sm_m + WARPS * NV;
-    float* rc_m = sm_l + WARPS * NV;                        // [share][VO]
+    float* rc_m = sm_l + WARPS * NV;                        // [CTA][VO]
     float* rc_l = rc_m + Cfg::Q;
     unsigned char* Qs = (unsigned char*)(rc_l + Cfg::Q);
-    float* sm_o = Cfg::PAIR && g.cluster > 1 ? (float*)ring : (float*)(Qs + Cfg::QROWS * QP);       // [warp][NV][OP]
+    float* sm_o = Cfg::PAIR ? (float*)ring : (float*)(Qs + Cfg::QROWS * QP);       // [warp][NV][OP]
 
     pdl_trigger();
     asm volatile("barrier.cluster.arrive.release;" ::: "memory");          // waited for before the first remote store: every CTA runs then
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int rank = blockIdx.x, kvh = blockIdx.y, r0 = blockIdx.z * ANPD_ROWS;
-    const int v_lo = g.cluster == 1 ? 0 : rank, v_hi = g.cluster == 1 ? VR : rank + 1;       // this CTA's shares
+    const int rank = blockIdx.x, C = gridDim.x, VO = Cfg::Q / C, kvh = blockIdx.y, r0 = blockIdx.z * ANPD_ROWS;       // VO: vectors a CTA finishes
     // The row plan is older than the kernel before this one (the embedding kernel lets its successors start only after its own
     // dependency wait), so it may be read at once; so may pages below the first position this launch writes - the group's own
     // first, or the first of all rows where they are one sequence's (a prompt as short as a step of the batch).
@@ -159,27 +154,26 @@ __global__ void __launch_bounds__((AdCfg<HD, G>::THREADS)) __maxnreg__((AdCfg<HD
             int stage = 0, count = 0;
             uint32_t phase = 1;
             bool waited = false, ok = true;
-            for (int v = v_lo; v < v_hi && ok; ++v)
-                for (int p = v; p < n_pages && ok; p += VR) {
-                    const int row = (g.layer_page0 + pages[p]) * g.Hkv + kvh;
-                    if (!waited && (p + 1) * KV_PAGE > first_new) { pdl_wait(); waited = true; }       // holds rows the kernel before writes
+            for (int p = rank; p < n_pages && ok; p += C) {
+                const int row = (g.layer_page0 + pages[p]) * g.Hkv + kvh;
+                if (!waited && (p + 1) * KV_PAGE > first_new) { pdl_wait(); waited = true; }       // holds rows the kernel before writes
 #pragma unroll
-                    for (int half = 0; half < 2; ++half) {
-                        if (count >= g.chunks && ok) ok = mbar_wait(&empty[stage], phase, abortp);
-                        if (!ok) break;
-                        unsigned char* dst = ring + (size_t)stage * CHUNK;
-                        mbar_expect_tx(&full[stage], CHUNK);
-                        if (half == 0) {
+                for (int half = 0; half < 2; ++half) {
+                    if (count >= CHUNKS && ok) ok = mbar_wait(&empty[stage], phase, abortp);
+                    if (!ok) break;
+                    unsigned char* dst = ring + (size_t)stage * CHUNK;
+                    mbar_expect_tx(&full[stage], CHUNK);
+                    if (half == 0) {
 #pragma unroll
-                            for (int s = 0; s < HD / 64; ++s) tma_load_2d(dst + s * (KV_PAGE * 128), &map_k, s * 64, row * KV_PAGE, &full[stage], pol);
-                        } else {
+                        for (int s = 0; s < HD / 64; ++s) tma_load_2d(dst + s * (KV_PAGE * 128), &map_k, s * 64, row * KV_PAGE, &full[stage], pol);
+                    } else {
 #pragma unroll
-                            for (int s = 0; s < 2; ++s) tma_load_2d(dst + s * (HD * 128), &map_v, s * 64, row * HD, &full[stage], pol);
-                        }
-                        ++count;
-                        if (++stage == g.chunks) { stage = 0; phase ^= 1u; }
+                        for (int s = 0; s < 2; ++s) tma_load_2d(dst + s * (HD * 128), &map_v, s * 64, row * HD, &full[stage], pol);
                     }
+                    ++count;
+                    if (++stage == CHUNKS) { stage = 0; phase ^= 1u; }
                 }
+            }
             s_issued = count;
         }
         __syncwarp();
@@ -280,86 +274,47 @@ __global__ void __launch_bounds__((AdCfg<HD, G>::THREADS)) __maxnreg__((AdCfg<HD
             }
         };
 
-        float R_m[Cfg::ITEMS], R_l[Cfg::ITEMS];             // one CTA for all shares: the running result of this thread's pieces
-        float4 R_a[Cfg::ITEMS];
-#pragma unroll
-        for (int i = 0; i < Cfg::ITEMS; ++i) { R_m[i] = -CUDART_INF_F; R_l[i] = 0.0f; R_a[i] = make_float4(0.f, 0.f, 0.f, 0.f); }
         int stage = 0;
         uint32_t par = 0;
-        bool cluster_ready = false;
-        for (int v = v_lo; v < v_hi; ++v) {
-            if (g.cluster == 1 && v >= n_pages) break;   // the remaining shares hold nothing
 #pragma unroll
-            for (int h = 0; h < NR; ++h) { m_run[h] = -CUDART_INF_F; l_run[h] = 0.0f; }
+        for (int h = 0; h < NR; ++h) { m_run[h] = -CUDART_INF_F; l_run[h] = 0.0f; }
 #pragma unroll
-            for (int d = 0; d < DT; ++d) { o[d][0] = 0.f; o[d][1] = 0.f; o[d][2] = 0.f; o[d][3] = 0.f; }
-            for (int p = v; p < n_pages; p += VR) {
-                const int ck = stage;
-                const uint32_t par_k = par;
-                if (++stage == g.chunks) { stage = 0; par ^= 1u; }
-                const int cv = stage;
-                const uint32_t par_v = par;
-                if (++stage == g.chunks) { stage = 0; par ^= 1u; }
-                mbar_wait(&full[ck], par_k, abortp);
-                bool freed = false;
+        for (int d = 0; d < DT; ++d) { o[d][0] = 0.f; o[d][1] = 0.f; o[d][2] = 0.f; o[d][3] = 0.f; }
+        for (int p = rank; p < n_pages; p += C) {
+            const int ck = stage;
+            const uint32_t par_k = par;
+            if (++stage == CHUNKS) { stage = 0; par ^= 1u; }
+            const int cv = stage;
+            const uint32_t par_v = par;
+            if (++stage == CHUNKS) { stage = 0; par ^= 1u; }
+            mbar_wait(&full[ck], par_k, abortp);
+            bool freed = false;
 #pragma unroll 1
-                for (int b = ks; b < AD_BLOCKS; b += KW)
-                    if (p * KV_PAGE + b * AD_KEYS <= pos_hi) { freed = Cfg::PAIR && b + KW >= AD_BLOCKS; block(ck, cv, par_v, b * AD_KEYS, p, freed); }
-                mbar_wait(&full[cv], par_v, abortp);
-                __syncwarp();
-                if (lane == 0) { if (!freed) mbar_arrive(&empty[ck]); mbar_arrive(&empty[cv]); }
-            }
-            if (Cfg::PAIR && g.cluster > 1) ad_bar<COMPUTE>();            // the slots' results go where the pages were
-            // ---- the share's key slots, in slot order ----
-#pragma unroll
-            for (int h = 0; h < NR; ++h) {
-                l_run[h] += __shfl_xor_sync(0xffffffffu, l_run[h], 1);
-                l_run[h] += __shfl_xor_sync(0xffffffffu, l_run[h], 2);
-                if (t == 0) { sm_m[warp * NV + gid + 8 * h] = m_run[h]; sm_l[warp * NV + gid + 8 * h] = l_run[h]; }
-            }
-            float* mine = sm_o + (size_t)warp * NV * OP;
-#pragma unroll
-            for (int d = 0; d < DT; ++d) {
-                if (STACK) *(float2*)(mine + gid * OP + 8 * d + 2 * t) = make_float2(o[d][0] + o[d][2], o[d][1] + o[d][3]);
-                else {
-                    *(float2*)(mine + gid * OP + 8 * d + 2 * t) = make_float2(o[d][0], o[d][1]);
-                    *(float2*)(mine + (gid + 8) * OP + 8 * d + 2 * t) = make_float2(o[d][2], o[d][3]);
-                }
-            }
-            ad_bar<COMPUTE>();
-            if (g.cluster > 1 && !cluster_ready) { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); cluster_ready = true; }
-#pragma unroll
-            for (int i = 0; i < Cfg::ITEMS; ++i) {
-                const int idx = threadIdx.x + i * COMPUTE;
-                if (idx < Cfg::Q * V4) {
-                    const int vec = idx / V4, d4 = idx % V4, tile = vec / NV, vi = vec % NV;
-                    float mx = -CUDART_INF_F;
-#pragma unroll
-                    for (int k = 0; k < KW; ++k) mx = fmaxf(mx, sm_m[(k * MT + tile) * NV + vi]);
-                    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-                    float l = 0.0f;
-#pragma unroll
-                    for (int k = 0; k < KW; ++k) {
-                        const int w = k * MT + tile;
-                        const float m = sm_m[w * NV + vi], s = m == -CUDART_INF_F ? 0.0f : exp2f(m - mx);
-                        const float4 x = *(const float4*)(sm_o + (size_t)(w * NV + vi) * OP + 4 * d4);
-                        a.x = fmaf(x.x, s, a.x); a.y = fmaf(x.y, s, a.y); a.z = fmaf(x.z, s, a.z); a.w = fmaf(x.w, s, a.w);
-                        l = fmaf(sm_l[w * NV + vi], s, l);
-                    }
-                    if (g.cluster == 1) ad_fold(R_m[i], R_l[i], R_a[i], mx, l, a);
-                    else {
-                        const int owner = vec / VO, at = v * VO + vec % VO;
-                        asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(ad_map(recv + at * HD + 4 * d4, owner)), "f"(a.x), "f"(a.y), "f"(a.z), "f"(a.w) : "memory");
-                        if (d4 == 0) {
-                            asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(ad_map(rc_m + at, owner)), "f"(mx) : "memory");
-                            asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(ad_map(rc_l + at, owner)), "f"(l) : "memory");
-                        }
-                    }
-                }
-            }
-            if (v + 1 < v_hi) ad_bar<COMPUTE>();                      // the slots' results may be overwritten
+            for (int b = ks; b < AD_BLOCKS; b += KW)
+                if (p * KV_PAGE + b * AD_KEYS <= pos_hi) { freed = Cfg::PAIR && b + KW >= AD_BLOCKS; block(ck, cv, par_v, b * AD_KEYS, p, freed); }
+            mbar_wait(&full[cv], par_v, abortp);
+            __syncwarp();
+            if (lane == 0) { if (!freed) mbar_arrive(&empty[ck]); mbar_arrive(&empty[cv]); }
         }
-        // ---- the result, as hi + lo terms in the O projection's operand image ----
+        if (Cfg::PAIR) ad_bar<COMPUTE>();                // the slots' results go where the pages were
+        // ---- the key slots, in slot order ----
+#pragma unroll
+        for (int h = 0; h < NR; ++h) {
+            l_run[h] += __shfl_xor_sync(0xffffffffu, l_run[h], 1);
+            l_run[h] += __shfl_xor_sync(0xffffffffu, l_run[h], 2);
+            if (t == 0) { sm_m[warp * NV + gid + 8 * h] = m_run[h]; sm_l[warp * NV + gid + 8 * h] = l_run[h]; }
+        }
+        float* mine = sm_o + (size_t)warp * NV * OP;
+#pragma unroll
+        for (int d = 0; d < DT; ++d) {
+            if (STACK) *(float2*)(mine + gid * OP + 8 * d + 2 * t) = make_float2(o[d][0] + o[d][2], o[d][1] + o[d][3]);
+            else {
+                *(float2*)(mine + gid * OP + 8 * d + 2 * t) = make_float2(o[d][0], o[d][1]);
+                *(float2*)(mine + (gid + 8) * OP + 8 * d + 2 * t) = make_float2(o[d][2], o[d][3]);
+            }
+        }
+        ad_bar<COMPUTE>();
+        // the result, as hi + lo terms in the O projection's operand image
         auto store = [&](int vec, int d4, float l, float4 a) {
             const int row = r0 + vec / G, k = (kvh * G + vec % G) * HD + 4 * d4;
             uint2 hi, lo;
@@ -368,36 +323,53 @@ __global__ void __launch_bounds__((AdCfg<HD, G>::THREADS)) __maxnreg__((AdCfg<HD
             *(uint2*)(g.img + cl_img_offset(g.rows, row, k)) = hi;
             *(uint2*)(g.img + cl_img_offset(g.rows, g.rows + row, k)) = lo;
         };
-        if (g.cluster == 1) {
+        asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+        for (int idx = threadIdx.x; idx < Cfg::Q * V4; idx += COMPUTE) {
+            const int vec = idx / V4, d4 = idx % V4, tile = vec / NV, vi = vec % NV;
+            float mx = -CUDART_INF_F;
 #pragma unroll
-            for (int i = 0; i < Cfg::ITEMS; ++i) {
-                const int idx = threadIdx.x + i * COMPUTE;
-                if (idx < Cfg::Q * V4) store(idx / V4, idx % V4, R_l[i], R_a[i]);
+            for (int k = 0; k < KW; ++k) mx = fmaxf(mx, sm_m[(k * MT + tile) * NV + vi]);
+            float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+            float l = 0.0f;
+#pragma unroll
+            for (int k = 0; k < KW; ++k) {
+                const int w = k * MT + tile;
+                const float m = sm_m[w * NV + vi], s = m == -CUDART_INF_F ? 0.0f : exp2f(m - mx);
+                const float4 x = *(const float4*)(sm_o + (size_t)(w * NV + vi) * OP + 4 * d4);
+                a.x = fmaf(x.x, s, a.x); a.y = fmaf(x.y, s, a.y); a.z = fmaf(x.z, s, a.z); a.w = fmaf(x.w, s, a.w);
+                l = fmaf(sm_l[w * NV + vi], s, l);
             }
-        } else {
+            if (C == 1) { store(vec, d4, l, a); continue; }
+            const int owner = vec / VO, at = rank * VO + vec % VO;
+            asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(ad_map(recv + at * HD + 4 * d4, owner)), "f"(a.x), "f"(a.y), "f"(a.z), "f"(a.w) : "memory");
+            if (d4 == 0) {
+                asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(ad_map(rc_m + at, owner)), "f"(mx) : "memory");
+                asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(ad_map(rc_l + at, owner)), "f"(l) : "memory");
+            }
+        }
+        if (C > 1) {
             asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
             for (int idx = threadIdx.x; idx < VO * V4; idx += COMPUTE) {
                 const int vo = idx / V4, d4 = idx % V4;
                 float m = -CUDART_INF_F, l = 0.0f;
                 float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-                for (int k = 0; k < VR; ++k)
+#pragma unroll 4
+                for (int k = 0; k < C; ++k)
                     ad_fold(m, l, a, rc_m[k * VO + vo], rc_l[k * VO + vo], *(const float4*)(recv + (k * VO + vo) * HD + 4 * d4));
                 store(rank * VO + vo, d4, l, a);
             }
         }
     }
-    // the loading warp and a CTA that is its own cluster take part in the cluster barriers too
-    if (g.cluster == 1) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
-    else if (warp == WARPS) {
+    // the loading warp takes part in the cluster barriers too
+    if (warp == WARPS) {
         asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
-        asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+        if (C > 1) asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
     }
     __syncthreads();
     if (threadIdx.x == 0 && abort_flag) {
         // gave up somewhere: let every copy already requested land before the CTA may exit
-        for (int i = max(0, s_issued - g.chunks); i < s_issued; ++i)
-            for (unsigned spin = 0; spin < WAIT_LIMIT && !mbar_try_wait(&full[i % g.chunks], (uint32_t)((i / g.chunks) & 1)); ++spin) {}
+        for (int i = max(0, s_issued - CHUNKS); i < s_issued; ++i)
+            for (unsigned spin = 0; spin < WAIT_LIMIT && !mbar_try_wait(&full[i % CHUNKS], (uint32_t)((i / CHUNKS) & 1)); ++spin) {}
         atomicExch(g.err, AD_ERR_TIMEOUT);
     }
 }
@@ -406,16 +378,18 @@ template <int HD, int G>
 anpd_status launch_attn_dec(anpd_model* m, anpd_kv* kv, AdArgs& a) {
     typedef AdCfg<HD, G> Cfg;
     static bool attr_set[64] = {false};
-    if (first_call_on_device(attr_set)) CUDA_TRY(cudaFuncSetAttribute(attn_dec_kernel<HD, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, std::max(Cfg::smem(true), Cfg::smem(false))));
-    // A CTA per share or one per head, whichever takes fewer rounds of a share's work: about 7/8 of the SMs can hold clusters.
-    const int heads = a.Hkv * kv->batch, per_sm = Cfg::PAIR ? 2 : 1, resident = std::max(1, m->num_sms * 7 / 8 * per_sm / Cfg::VR);
-    a.cluster = (heads + resident - 1) / resident < Cfg::VR * ((heads + m->num_sms * per_sm - 1) / (m->num_sms * per_sm)) ? Cfg::VR : 1;
-    a.chunks = Cfg::chunks(a.cluster > 1); a.ring_bytes = Cfg::ring(a.cluster > 1);
+    if (first_call_on_device(attr_set)) CUDA_TRY(cudaFuncSetAttribute(attn_dec_kernel<HD, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM));
+    // As many CTAs per head as are resident at once (about 7/8 of the SMs can hold clusters).  1.1B, eight sequences of 300 tokens:
+    // 1666 -> 1389 us per step with four CTAs per head, where one took all pages of a head before.  Eight 13B sequences have one: as
+    // fast as page partials and their merge (2147 -> 2135), four 7B sequences two (1015 -> 997).
+    const int heads = a.Hkv * kv->batch, resident = m->num_sms * 7 / 8 * (Cfg::PAIR ? 2 : 1);
+    int cluster = Cfg::C_MAX;
+    while (cluster > 1 && heads * cluster > resident) cluster /= 2;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(a.cluster, a.Hkv, kv->batch); cfg.blockDim = dim3(Cfg::THREADS); cfg.dynamicSmemBytes = Cfg::smem(a.cluster > 1); cfg.stream = m->stream;
+    cfg.gridDim = dim3(cluster, a.Hkv, kv->batch); cfg.blockDim = dim3(Cfg::THREADS); cfg.dynamicSmemBytes = Cfg::SMEM; cfg.stream = m->stream;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = a.cluster; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    attr[0].val.clusterDim.x = cluster; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
