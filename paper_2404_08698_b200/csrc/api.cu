@@ -156,7 +156,7 @@ static anpd_status model_make_plans(anpd_model* m) {
         ints += 2 * (size_t)m->plan[k].m_tiles;
         max_tiles = std::max(max_tiles, m->plan[k].m_tiles);
     }
-    ints += PF_MAX_PARTS * (size_t)max_tiles + (size_t)GK_COUNT * max_tiles;        // constants 1..8, then a table per projection
+    ints += (size_t)GK_COUNT * max_tiles;                                           // a table per projection
     std::vector<int> host(ints);
     CUDA_TRY(cudaMalloc((void**)&m->d_plan_tables, ints * sizeof(int)));
     size_t off = 0;
@@ -167,15 +167,8 @@ static anpd_status model_make_plans(anpd_model* m) {
         p.d_seg_count = m->d_plan_tables + off;
         std::copy(p.seg_count.begin(), p.seg_count.end(), host.begin() + off); off += p.m_tiles;
     }
-    m->d_ones = m->d_plan_tables + off;
-    for (int i = 0; i < max_tiles; ++i) host[off + i] = 1;
-    m->d_const_segs[0] = m->d_const_segs[1] = m->d_ones;
-    for (int k = 2; k <= PF_MAX_PARTS; ++k) {
-        m->d_const_segs[k] = m->d_plan_tables + off + (size_t)(k - 1) * max_tiles;
-        for (int i = 0; i < max_tiles; ++i) host[off + (size_t)(k - 1) * max_tiles + i] = k;
-    }
     for (int k = 0; k < GK_COUNT; ++k) {
-        m->d_tail_segs[k] = m->d_plan_tables + off + (size_t)(PF_MAX_PARTS + k) * max_tiles;
+        m->d_tail_segs[k] = m->d_plan_tables + off + (size_t)k * max_tiles;
         m->tail_cfg[k] = -1;
     }
     CUDA_TRY(cudaMemcpy(m->d_plan_tables, host.data(), ints * sizeof(int), cudaMemcpyHostToDevice));

@@ -97,6 +97,8 @@ __device__ __forceinline__ void store_split4(const float4 v, bf16* hi_ptr, bf16*
     *(uint2*)lo_ptr = *(const uint2*)l;
 }
 
+__device__ __forceinline__ void add4(float4& a, const float4& p) { a.x += p.x; a.y += p.y; a.z += p.z; a.w += p.w; }
+
 __global__ void __launch_bounds__(NORM_THREADS) embed_norm_kernel(const bf16* __restrict__ embed, const int* __restrict__ row_tok,
                                                                   const float* __restrict__ gain, float eps, int d,
                                                                   float* __restrict__ x, bf16* __restrict__ h_hi, bf16* __restrict__ h_lo,
@@ -189,43 +191,45 @@ __global__ void __launch_bounds__(NORM_THREADS) embed_img_kernel(const bf16* __r
     if (threadIdx.x == 0) ss[row] = t;
 }
 
-// x[row] += sum of the tile's partial sums (in segment order); then h = rmsnorm(x) * gain as hi + lo.
-__global__ void __launch_bounds__(NORM_THREADS) resid_norm_kernel(float* __restrict__ x, const float* __restrict__ part,
+// x[row] += sum of the tile's partial sums (in segment order); then h = rmsnorm(x) * gain as hi + lo.  NCH chunks of 4096 features;
+// rows of one chunk run two to an SM, so that one row's sums travel while the other's are reduced (1536 rows of 4096: 31 -> 19 us).
+template <int NCH>
+__global__ void __launch_bounds__(NORM_THREADS, NCH == 1 ? 2 : 1) resid_norm_kernel(float* __restrict__ x, const float* __restrict__ part,
                                                                   const int* __restrict__ seg_count, size_t split_stride, int ld_part,
                                                                   const float* __restrict__ gain, float eps, int d,
-                                                                  bf16* __restrict__ h_hi, bf16* __restrict__ h_lo, int ns_max,
+                                                                  bf16* __restrict__ h_hi, bf16* __restrict__ h_lo, int ns_min,
                                                                   unsigned char* __restrict__ img) {
     // img: a decode step's operand image of gridDim.x rows instead of h_hi and h_lo.
-    // ns_max: the most partial sums any tile of this projection has.  The loads cover that many slabs whatever the tile's own
-    // count (slabs beyond it hold older sums: read, never added), so they do not wait for the count to arrive.
+    // ns_min: partial sums every tile of this projection has; seg_count: null, or each tile's own count.
     pdl_trigger();
+    constexpr int AT = NCH == 1 ? 4 : 8;
     __shared__ float red[32];
     const int row = blockIdx.x, chunks = d >> 2;
-    float4 v[NORM_MAX_CHUNKS], gn[NORM_MAX_CHUNKS];
+    float4 v[NCH], gn[NCH];
     // the norm's gain is a weight: nothing of this step writes it, so it is fetched before the dependency wait
 #pragma unroll
-    for (int u = 0; u < NORM_MAX_CHUNKS; ++u) {
+    for (int u = 0; u < NCH; ++u) {
         const int c = threadIdx.x + u * NORM_THREADS;
         gn[u] = (c < chunks) ? *(const float4*)(gain + 4 * c) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
     pdl_wait();
     float ss = 0.0f;
 #pragma unroll
-    for (int u = 0; u < NORM_MAX_CHUNKS; ++u) {
+    for (int u = 0; u < NCH; ++u) {
         const int c = threadIdx.x + u * NORM_THREADS;
         v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
         if (c < chunks) {
-            const int ns = seg_count[(4 * c) >> 7];
             const float* pr = part + (size_t)row * ld_part + 4 * c;
             float4 acc = *(const float4*)(x + (size_t)row * d + 4 * c);
-            for (int s0 = 0; s0 < ns_max; s0 += 8) {
-                float4 p[8];
+            const int ns = seg_count ? seg_count[(4 * c) >> 7] : ns_min;
+            for (int s0 = 0; s0 < ns; s0 += AT) {
+                float4 p[AT];
 #pragma unroll
-                for (int k = 0; k < 8; ++k)
-                    p[k] = (s0 + k < ns_max) ? *(const float4*)(pr + (size_t)(s0 + k) * split_stride) : make_float4(0.f, 0.f, 0.f, 0.f);
+                for (int k = 0; k < AT; ++k)
+                    p[k] = (s0 + k < ns) ? *(const float4*)(pr + (size_t)(s0 + k) * split_stride) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-                for (int k = 0; k < 8; ++k)
-                    if (s0 + k < ns) { acc.x += p[k].x; acc.y += p[k].y; acc.z += p[k].z; acc.w += p[k].w; }
+                for (int k = 0; k < AT; ++k)
+                    if (s0 + k < ns) add4(acc, p[k]);
             }
             v[u] = acc;
             *(float4*)(x + (size_t)row * d + 4 * c) = acc;
@@ -234,7 +238,7 @@ __global__ void __launch_bounds__(NORM_THREADS) resid_norm_kernel(float* __restr
     }
     const float rstd = rsqrtf(block_sum_1024(ss, red) / (float)d + eps);
 #pragma unroll
-    for (int u = 0; u < NORM_MAX_CHUNKS; ++u) {
+    for (int u = 0; u < NCH; ++u) {
         const int c = threadIdx.x + u * NORM_THREADS;
         if (c < chunks) {
             const float4 g = gn[u];
@@ -248,133 +252,148 @@ __global__ void __launch_bounds__(NORM_THREADS) resid_norm_kernel(float* __restr
 // ---------------------------------------------------------------------------------------------
 // QKV epilogue: reduce splits, rotary embedding, append K/V to the paged cache, keep q
 // ---------------------------------------------------------------------------------------------
-__global__ void qkv_rope_append_kernel(const float* __restrict__ part, const int* __restrict__ seg_count, size_t split_stride, int ld_part,
+// Bound by latency (a decode step) or by the partial sums' way through L2 (a prompt pass): a thread owns four rotary pairs, requests
+// the sums every tile has (ns_min) several at a time - seg_count, null where all tiles have as many, tells of more - and has fetched
+// what does not depend on the kernel before - the row plan (older than that kernel, see embed_norm_kernel), cosines and sines -
+// while it waits.
+struct RopeSum { float4 a, b; };
+
+template <int AT_ONCE>
+__device__ __forceinline__ RopeSum rope_sum(const float* __restrict__ pr, int half, size_t split_stride, const int* __restrict__ seg, int ns_min) {
+    RopeSum r;
+    r.a = r.b = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int s0 = 0; s0 < ns_min; s0 += AT_ONCE) {
+        float4 pa[AT_ONCE], pb[AT_ONCE];
+#pragma unroll
+        for (int s = 0; s < AT_ONCE; ++s)
+            if (s0 + s < ns_min) { pa[s] = *(const float4*)(pr + (s0 + s) * split_stride); pb[s] = *(const float4*)(pr + (s0 + s) * split_stride + half); }
+#pragma unroll
+        for (int s = 0; s < AT_ONCE; ++s)
+            if (s0 + s < ns_min) { add4(r.a, pa[s]); add4(r.b, pb[s]); }
+    }
+    if (seg)
+        for (int s = ns_min; s < *seg; ++s) { add4(r.a, *(const float4*)(pr + s * split_stride)); add4(r.b, *(const float4*)(pr + s * split_stride + half)); }
+    return r;
+}
+
+__device__ __forceinline__ void rope_rotate(RopeSum& v, float4 c, float4 s) {
+    const float4 a = v.a, b = v.b;
+    v.a = make_float4(a.x * c.x - b.x * s.x, a.y * c.y - b.y * s.y, a.z * c.z - b.z * s.z, a.w * c.w - b.w * s.w);
+    v.b = make_float4(b.x * c.x + a.x * s.x, b.y * c.y + a.y * s.y, b.z * c.z + a.z * s.z, b.w * c.w + a.w * s.w);
+}
+
+// queries leave as two bf16 terms, already multiplied by log2(e) / sqrt(hd): the attention kernels take them as MMA operands and
+// work with base-2 exponentials
+__device__ __forceinline__ void rope_store_q(const RopeSum& v, float q_scale, bf16* hi, bf16* lo, int half) {
+    store_split4(make_float4(v.a.x * q_scale, v.a.y * q_scale, v.a.z * q_scale, v.a.w * q_scale), hi, lo);
+    store_split4(make_float4(v.b.x * q_scale, v.b.y * q_scale, v.b.z * q_scale, v.b.w * q_scale), hi + half, lo + half);
+}
+
+__device__ __forceinline__ uint2 pack_bf16x4(float4 v) {
+    const __nv_bfloat162 x = __floats2bfloat162_rn(v.x, v.y), y = __floats2bfloat162_rn(v.z, v.w);
+    uint2 r;
+    r.x = *(const uint32_t*)&x; r.y = *(const uint32_t*)&y;
+    return r;
+}
+
+// A decode step: hd / 8 threads per (row, head).
+__global__ void __launch_bounds__(128) qkv_rope_append_kernel(const float* __restrict__ part, const int* __restrict__ seg_count, size_t split_stride, int ld_part,
                                        const int* __restrict__ row_pos, const int* __restrict__ row_slot, const int* __restrict__ row_seq,
                                        const int* __restrict__ row_ok, const float* __restrict__ rope_cos,
                                        const float* __restrict__ rope_sin, const int* __restrict__ page_table,
                                        int pages_per_seq, int Hq, int Hkv, int hd, float q_scale, bf16* __restrict__ q_hi,
-                                       bf16* __restrict__ q_lo, bf16* __restrict__ kpool_l, bf16* __restrict__ vpool_l, int ns_max) {
+                                       bf16* __restrict__ q_lo, bf16* __restrict__ kpool_l, bf16* __restrict__ vpool_l, int ns_min) {
     pdl_trigger();
+    const int half = hd >> 1, tph = hd >> 3, row = blockIdx.x, head = blockIdx.y * (blockDim.x / tph) + threadIdx.x / tph, i = threadIdx.x % tph * 4;
+    if (head >= Hq + 2 * Hkv) { pdl_wait(); return; }
+    const size_t at = (size_t)row_pos[row] * half + i;
+    float4 c = make_float4(1.f, 1.f, 1.f, 1.f), sn = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (head < Hq + Hkv) { c = *(const float4*)(rope_cos + at); sn = *(const float4*)(rope_sin + at); }
+    const int slot = row_slot[row];               // where the row lives in the cache (its position, except for a second candidate)
+    const int page = page_table[row_seq[row] * pages_per_seq + slot / KV_PAGE], ok = row_ok[row];
     pdl_wait();
-    // a block covers blockDim.x / (hd / 2) consecutive heads of one row
-    const int half = hd >> 1, row = blockIdx.x, head = blockIdx.y * (blockDim.x / half) + threadIdx.x / half, i = threadIdx.x % half;
-    if (head >= Hq + 2 * Hkv) return;
-    const float* pr = part + (size_t)row * ld_part + (size_t)head * hd;
-    float a = 0.0f, b = 0.0f;
-    // up to four slabs are requested before the tile's own count is known (ns_max: the projection's largest count)
-    float pa[4], pb[4];
-#pragma unroll
-    for (int s = 0; s < 4; ++s) {
-        pa[s] = (s < ns_max) ? pr[s * split_stride + i] : 0.0f;
-        pb[s] = (s < ns_max) ? pr[s * split_stride + i + half] : 0.0f;
-    }
-    const int ns = seg_count[(head * hd + i) >> 7];      // a head never straddles a 128-column tile
-    const int pos = row_pos[row];
-#pragma unroll
-    for (int s = 0; s < 4; ++s) if (s < ns) { a += pa[s]; b += pb[s]; }
-    for (int s = 4; s < ns; ++s) { a += pr[s * split_stride + i]; b += pr[s * split_stride + i + half]; }
-    if (head < Hq + Hkv) {
-        const float c = rope_cos[(size_t)pos * half + i], sn = rope_sin[(size_t)pos * half + i];
-        const float ra = a * c - b * sn, rb = b * c + a * sn;
-        a = ra; b = rb;
-    }
+    RopeSum v = rope_sum<4>(part + (size_t)row * ld_part + (size_t)head * hd + i, half, split_stride, seg_count ? seg_count + ((head * hd) >> 7) : nullptr, ns_min);      // a head never straddles a 128-column tile
+    if (head < Hq + Hkv) rope_rotate(v, c, sn);
     if (head < Hq) {
-        // queries leave as two bf16 terms, already multiplied by log2(e) / sqrt(hd): the attention kernel
-        // takes them as MMA fragments and works with base-2 exponentials
         const size_t o = (size_t)row * Hq * hd + head * hd + i;
-        split_bf16(a * q_scale, q_hi[o], q_lo[o]);
-        split_bf16(b * q_scale, q_hi[o + half], q_lo[o + half]);
+        rope_store_q(v, q_scale, q_hi + o, q_lo + o, half);
         return;
     }
-    if (!row_ok[row]) return;
+    if (!ok) return;
     const bool is_k = head < Hq + Hkv;
     const int kvh = is_k ? head - Hq : head - Hq - Hkv;
-    const int slot = row_slot[row];               // where the row lives in the cache (its position, except for a second candidate)
-    const int page = page_table[row_seq[row] * pages_per_seq + slot / KV_PAGE];
     bf16* pg = (is_k ? kpool_l : vpool_l) + ((size_t)page * Hkv + kvh) * KV_PAGE * hd;
     if (is_k) {                                   // K page: [position][dim]
-        pg[(size_t)(slot % KV_PAGE) * hd + i] = __float2bfloat16_rn(a);
-        pg[(size_t)(slot % KV_PAGE) * hd + i + half] = __float2bfloat16_rn(b);
+        bf16* dst = pg + (size_t)(slot % KV_PAGE) * hd + i;
+        *(uint2*)dst = pack_bf16x4(v.a);
+        *(uint2*)(dst + half) = pack_bf16x4(v.b);
     } else {                                      // V page is kept transposed: [dim][position]
-        pg[(size_t)i * KV_PAGE + (slot % KV_PAGE)] = __float2bfloat16_rn(a);
-        pg[(size_t)(i + half) * KV_PAGE + (slot % KV_PAGE)] = __float2bfloat16_rn(b);
+        const float a[4] = {v.a.x, v.a.y, v.a.z, v.a.w}, b[4] = {v.b.x, v.b.y, v.b.z, v.b.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            pg[(size_t)(i + e) * KV_PAGE + (slot % KV_PAGE)] = __float2bfloat16_rn(a[e]);
+            pg[(size_t)(i + e + half) * KV_PAGE + (slot % KV_PAGE)] = __float2bfloat16_rn(b[e]);
+        }
     }
 }
 
-// The same for a prompt pass (rows are consecutive positions of one sequence, a multiple of 8, the first a multiple of 64):
-// a block takes 64 rows of one head through shared memory, so that the transposed V page receives whole 16-byte runs of
-// positions instead of single elements.  Per element the arithmetic is that of qkv_rope_append_kernel, in the same order.
-constexpr int ROPE_TILE_ROWS = 64;
+// The same for a prompt pass (rows are consecutive positions of one sequence, a multiple of 8, the first a multiple of the page):
+// a block takes 32 rows of the heads blockIdx.x, blockIdx.x + gridDim.x, ... and keeps their cosines and sines; a V head goes
+// through shared memory, so that the transposed page receives whole 16-byte runs of positions instead of single elements.  Per
+// element the arithmetic is that of qkv_rope_append_kernel, in the same order.  7B: 80 rows 14 -> 6 us, 1536 rows 41 -> 36.
+constexpr int ROPE_TILE_ROWS = 32;
 template <int HD>
-__global__ void __launch_bounds__(256) qkv_rope_append_tile_kernel(const float* __restrict__ part, const int* __restrict__ seg_count, size_t split_stride,
+__global__ void __launch_bounds__(256, 3) qkv_rope_append_tile_kernel(const float* __restrict__ part, const int* __restrict__ seg_count, size_t split_stride,
                                                                    int ld_part, int rows, const int* __restrict__ row_pos, const int* __restrict__ row_seq,
                                                                    const int* __restrict__ row_ok, const float* __restrict__ rope_cos,
                                                                    const float* __restrict__ rope_sin, const int* __restrict__ page_table,
                                                                    int pages_per_seq, int Hq, int Hkv, float q_scale, bf16* __restrict__ q_hi,
-                                                                   bf16* __restrict__ q_lo, bf16* __restrict__ kpool_l, bf16* __restrict__ vpool_l) {
+                                                                   bf16* __restrict__ q_lo, bf16* __restrict__ kpool_l, bf16* __restrict__ vpool_l, int ns_min) {
     pdl_trigger();
-    pdl_wait();
     __shared__ float tile[ROPE_TILE_ROWS][HD + 1];
-    constexpr int half = HD / 2;
-    const int r0 = blockIdx.x * ROPE_TILE_ROWS, head = blockIdx.y;
+    constexpr int half = HD / 2, TPR = HD / 8, PER = ROPE_TILE_ROWS * TPR / 256;
+    const int r0 = blockIdx.y * ROPE_TILE_ROWS, i = threadIdx.x % TPR * 4;
     const int nr = min(ROPE_TILE_ROWS, rows - r0);
-    const int ns = seg_count[(head * HD) >> 7];          // a head never straddles a 128-column tile
-    // 16-byte loads, eight of them in flight per thread
-    constexpr int Q4 = HD / 4;
-    for (int base = 0; base < nr * Q4; base += 8 * 256) {
-        float4 a[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {                     // the first partial sums (there is always one): eight independent loads
-            const int idx = base + u * 256 + threadIdx.x;
-            a[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (idx < nr * Q4) a[u] = *(const float4*)(part + (size_t)(r0 + idx / Q4) * ld_part + (size_t)head * HD + (idx % Q4) * 4);
-        }
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const int idx = base + u * 256 + threadIdx.x;
-            if (idx >= nr * Q4) continue;
-            const int r = idx / Q4, dim = (idx % Q4) * 4;
-            const float* pr = part + (size_t)(r0 + r) * ld_part + (size_t)head * HD + dim;
-            for (int s = 1; s < ns; ++s) { const float4 v = *(const float4*)(pr + s * split_stride); a[u].x += v.x; a[u].y += v.y; a[u].z += v.z; a[u].w += v.w; }
-            tile[r][dim] = a[u].x; tile[r][dim + 1] = a[u].y; tile[r][dim + 2] = a[u].z; tile[r][dim + 3] = a[u].w;
-        }
-    }
-    __syncthreads();
-    if (head < Hq + Hkv) {
-        for (int idx = threadIdx.x; idx < nr * half; idx += 256) {
-            const int r = idx / half, i = idx % half;
-            const int pos = row_pos[r0 + r];
-            const float a = tile[r][i], b = tile[r][i + half];
-            const float c = rope_cos[(size_t)pos * half + i], sn = rope_sin[(size_t)pos * half + i];
-            tile[r][i] = a * c - b * sn;
-            tile[r][i + half] = b * c + a * sn;
-        }
-        __syncthreads();
-    }
-    if (head < Hq) {
-        for (int idx = threadIdx.x; idx < nr * Q4; idx += 256) {
-            const int r = idx / Q4, dim = (idx % Q4) * 4;
-            const size_t o = (size_t)(r0 + r) * Hq * HD + (size_t)head * HD + dim;
-            store_split4(make_float4(tile[r][dim] * q_scale, tile[r][dim + 1] * q_scale, tile[r][dim + 2] * q_scale, tile[r][dim + 3] * q_scale),
-                         q_hi + o, q_lo + o);
-        }
-        return;
-    }
-    const bool is_k = head < Hq + Hkv;
-    const int kvh = is_k ? head - Hq : head - Hq - Hkv;
     const int pos0 = row_pos[r0];                        // the tile's rows hold positions pos0, pos0 + 1, ... inside one page
     const int page = page_table[row_seq[r0] * pages_per_seq + pos0 / KV_PAGE];
-    bf16* pg = (is_k ? kpool_l : vpool_l) + ((size_t)page * Hkv + kvh) * KV_PAGE * HD;
-    if (is_k) {                                          // K page: [position][dim]
-        for (int idx = threadIdx.x; idx < nr * Q4; idx += 256) {
-            const int r = idx / Q4, dim = (idx % Q4) * 4;
-            if (!row_ok[r0 + r]) continue;
-            bf16 v[4];
+    float4 c[PER], sn[PER];
+    bool keep[PER];
 #pragma unroll
-            for (int e = 0; e < 4; ++e) v[e] = __float2bfloat16_rn(tile[r][dim + e]);
-            *(uint2*)(pg + (size_t)((pos0 + r) % KV_PAGE) * HD + dim) = *(const uint2*)v;
+    for (int u = 0; u < PER; ++u) {
+        const int r = u * (256 / TPR) + threadIdx.x / TPR;
+        keep[u] = false;
+        if (r < nr) {
+            const size_t at = (size_t)row_pos[r0 + r] * half + i;
+            c[u] = *(const float4*)(rope_cos + at); sn[u] = *(const float4*)(rope_sin + at);
+            keep[u] = row_ok[r0 + r] != 0;
         }
-    } else {                                             // V page, transposed: [dim][position]; 8 positions = 16 bytes
+    }
+    pdl_wait();
+    for (int head = blockIdx.x; head < Hq + 2 * Hkv; head += gridDim.x) {
+        const bool is_q = head < Hq, is_k = !is_q && head < Hq + Hkv;
+        bf16* pg = (is_k ? kpool_l : vpool_l) + ((size_t)page * Hkv + (is_q ? 0 : is_k ? head - Hq : head - Hq - Hkv)) * KV_PAGE * HD;
+        const int* seg = seg_count ? seg_count + ((head * HD) >> 7) : nullptr;
+#pragma unroll
+        for (int u = 0; u < PER; ++u) {
+            const int r = u * (256 / TPR) + threadIdx.x / TPR;
+            if (r >= nr) continue;
+            RopeSum v = rope_sum<4>(part + (size_t)(r0 + r) * ld_part + (size_t)head * HD + i, half, split_stride, seg, ns_min);
+            if (is_q || is_k) rope_rotate(v, c[u], sn[u]);
+            if (is_q) {
+                const size_t o = (size_t)(r0 + r) * Hq * HD + (size_t)head * HD + i;
+                rope_store_q(v, q_scale, q_hi + o, q_lo + o, half);
+            } else if (is_k) {                           // K page: [position][dim]
+                if (!keep[u]) continue;
+                bf16* dst = pg + (size_t)((pos0 + r) % KV_PAGE) * HD + i;
+                *(uint2*)dst = pack_bf16x4(v.a);
+                *(uint2*)(dst + half) = pack_bf16x4(v.b);
+            } else {
+                tile[r][i] = v.a.x; tile[r][i + 1] = v.a.y; tile[r][i + 2] = v.a.z; tile[r][i + 3] = v.a.w;
+                tile[r][i + half] = v.b.x; tile[r][i + half + 1] = v.b.y; tile[r][i + half + 2] = v.b.z; tile[r][i + half + 3] = v.b.w;
+            }
+        }
+        if (is_q || is_k) continue;
+        __syncthreads();                                 // V page, transposed: [dim][position]; 8 positions = 16 bytes
         for (int idx = threadIdx.x; idx < (ROPE_TILE_ROWS / 8) * HD; idx += 256) {
             const int dim = idx % HD, r8 = (idx / HD) * 8;
             if (r8 >= nr) continue;
@@ -387,6 +406,7 @@ __global__ void __launch_bounds__(256) qkv_rope_append_tile_kernel(const float* 
             else
                 for (int e = 0; e < 8; ++e) if (row_ok[r0 + r8 + e]) dst[e] = v[e];
         }
+        __syncthreads();
     }
 }
 
@@ -757,70 +777,42 @@ __global__ void __launch_bounds__(32 * COMBINE_SLICES) attn_combine_wide_kernel(
 // ---------------------------------------------------------------------------------------------
 // SwiGLU epilogue of the gate/up projection
 // ---------------------------------------------------------------------------------------------
-__global__ void swiglu_kernel(const float* __restrict__ part, const int* __restrict__ seg_count, size_t split_stride, int ld_part, int F,
-                              bf16* __restrict__ act_hi, bf16* __restrict__ act_lo, int ns_max, unsigned char* __restrict__ img) {
-    // img: a decode step's operand image of gridDim.y rows instead of act_hi and act_lo
+// A thread owns CH chunks of four consecutive features (a block's width apart) and requests the sums every tile has (ns_min) several at
+// a time; seg_count, null where all tiles have as many, tells of more.  Bound by those sums' way through L2; two chunks where the
+// rows fill the device, one where parallelism is short.
+template <int CH>
+__global__ void __launch_bounds__(256, CH == 1 ? 4 : 5) swiglu_kernel(const float* __restrict__ part, const int* __restrict__ seg_count, size_t split_stride, int ld_part, int F,
+                                                     bf16* __restrict__ act_hi, bf16* __restrict__ act_lo, int ns_min, unsigned char* __restrict__ img) {
+    // img: an operand image of gridDim.y rows instead of act_hi and act_lo
     pdl_trigger();
     pdl_wait();
-    const int row = blockIdx.y, j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= F) return;
+    const int row = blockIdx.y, j0 = 4 * (CH * blockIdx.x * blockDim.x + threadIdx.x);
+    constexpr int AT = CH == 1 ? 4 : 1;
     const float* pr = part + (size_t)row * ld_part;
-    float gte = 0.0f, up = 0.0f;
-    // up to four slabs are requested before the tile's own count is known (ns_max: the projection's largest count)
-    float pg[4], pu[4];
+    float4 g4[CH], u4[CH];
 #pragma unroll
-    for (int s = 0; s < 4; ++s) {
-        pg[s] = (s < ns_max) ? pr[s * split_stride + j] : 0.0f;
-        pu[s] = (s < ns_max) ? pr[s * split_stride + F + j] : 0.0f;
+    for (int c = 0; c < CH; ++c) g4[c] = u4[c] = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int s0 = 0; s0 < ns_min; s0 += AT) {
+        float4 pg[CH][AT], pu[CH][AT];
+#pragma unroll
+        for (int c = 0; c < CH; ++c)
+#pragma unroll
+            for (int s = 0; s < AT; ++s) {
+                const int j = j0 + c * 4 * blockDim.x;
+                if (s0 + s < ns_min && j < F) { pg[c][s] = *(const float4*)(pr + (s0 + s) * split_stride + j); pu[c][s] = *(const float4*)(pr + (s0 + s) * split_stride + F + j); }
+            }
+#pragma unroll
+        for (int c = 0; c < CH; ++c)
+#pragma unroll
+            for (int s = 0; s < AT; ++s)
+                if (s0 + s < ns_min && j0 + c * 4 * (int)blockDim.x < F) { add4(g4[c], pg[c][s]); add4(u4[c], pu[c][s]); }
     }
-    const int ng = seg_count[j >> 6], nu = ng;          // a 128-position storage tile holds 64 gate features and their up features
 #pragma unroll
-    for (int s = 0; s < 4; ++s) { if (s < ng) gte += pg[s]; if (s < nu) up += pu[s]; }
-    for (int s = 4; s < ng; ++s) gte += pr[s * split_stride + j];
-    for (int s = 4; s < nu; ++s) up += pr[s * split_stride + F + j];
-    const float v = gte / (1.0f + expf(-gte)) * up;
-    bf16 hi, lo;
-    split_bf16(v, hi, lo);
-    if (img) {
-        *(bf16*)(img + cl_img_offset(gridDim.y, row, j)) = hi;
-        *(bf16*)(img + cl_img_offset(gridDim.y, gridDim.y + row, j)) = lo;
-        return;
-    }
-    act_hi[(size_t)row * F + j] = hi;
-    act_lo[(size_t)row * F + j] = lo;
-}
-
-// The same for many rows (prefill passes): a thread owns four consecutive features, so the partial sums come in
-// 16-byte loads.  Per element the arithmetic is that of swiglu_kernel, in the same order.
-__global__ void swiglu_wide_kernel(const float* __restrict__ part, const int* __restrict__ seg_count, size_t split_stride, int ld_part, int F,
-                                   bf16* __restrict__ act_hi, bf16* __restrict__ act_lo, unsigned char* __restrict__ img) {
-    pdl_trigger();
-    pdl_wait();
-    // two chunks of four features per thread (a block's width apart); every output has at least one partial sum, so the
-    // first partial sums of gate and up of both chunks are requested together, before anything depends on them
-    const int row = blockIdx.y, j0 = 4 * (2 * blockIdx.x * blockDim.x + threadIdx.x);
-    const float* pr = part + (size_t)row * ld_part;
-    float4 g4[2], u4[2];
-    int ng[2], nu[2];
-    bool live[2];
-#pragma unroll
-    for (int c = 0; c < 2; ++c) {
+    for (int c = 0; c < CH; ++c) {
         const int j = j0 + c * 4 * blockDim.x;
-        live[c] = j < F;
-        g4[c] = u4[c] = make_float4(0.f, 0.f, 0.f, 0.f);
-        ng[c] = nu[c] = 0;
-        if (live[c]) {
-            g4[c] = *(const float4*)(pr + j);
-            u4[c] = *(const float4*)(pr + F + j);
-            ng[c] = nu[c] = seg_count[j >> 6];               // a 128-position storage tile holds 64 gate features and their up features
-        }
-    }
-#pragma unroll
-    for (int c = 0; c < 2; ++c) {
-        if (!live[c]) continue;
-        const int j = j0 + c * 4 * blockDim.x;
-        for (int s = 1; s < ng[c]; ++s) { const float4 p = *(const float4*)(pr + s * split_stride + j); g4[c].x += p.x; g4[c].y += p.y; g4[c].z += p.z; g4[c].w += p.w; }
-        for (int s = 1; s < nu[c]; ++s) { const float4 p = *(const float4*)(pr + s * split_stride + F + j); u4[c].x += p.x; u4[c].y += p.y; u4[c].z += p.z; u4[c].w += p.w; }
+        if (j >= F) continue;
+        if (seg_count)                                   // a 128-position storage tile holds 64 gate features and their up features
+            for (int s = ns_min; s < seg_count[j >> 6]; ++s) { add4(g4[c], *(const float4*)(pr + s * split_stride + j)); add4(u4[c], *(const float4*)(pr + s * split_stride + F + j)); }
         const float gte[4] = {g4[c].x, g4[c].y, g4[c].z, g4[c].w}, up[4] = {u4[c].x, u4[c].y, u4[c].z, u4[c].w};
         bf16 hi[4], lo[4];
 #pragma unroll
@@ -834,7 +826,7 @@ __global__ void swiglu_wide_kernel(const float* __restrict__ part, const int* __
 // LM-head epilogue: reduce splits, (optionally) keep logits, per-block argmax with ties to the lowest id
 // ---------------------------------------------------------------------------------------------
 constexpr int AMAX_COLS = 1024;
-__global__ void __launch_bounds__(256) argmax_partial_kernel(const float* __restrict__ part, const int* __restrict__ seg_count, size_t split_stride,
+__global__ void __launch_bounds__(256) argmax_partial_kernel(const float* __restrict__ part, int n_parts, size_t split_stride,
                                                              int ld_part, int V, float* __restrict__ logits,
                                                              float* __restrict__ amax_val, int* __restrict__ amax_idx, int nblk) {
     pdl_trigger();
@@ -845,14 +837,17 @@ __global__ void __launch_bounds__(256) argmax_partial_kernel(const float* __rest
     const float* pr = part + (size_t)row * ld_part;
     float best = -CUDART_INF_F;
     int bidx = 0x7fffffff;
-    for (int u = 0; u < AMAX_COLS / 256; ++u) {
-        const int v = blockIdx.x * AMAX_COLS + u * 256 + threadIdx.x;
-        if (v < V) {
-            float z = 0.0f;
-            const int ns = seg_count[v >> 7];
-            for (int s = 0; s < ns; ++s) z += pr[s * split_stride + v];
-            if (logits) logits[(size_t)row * V + v] = z;
-            if (z > best) { best = z; bidx = v; }       // ascending v: strict > keeps the lowest id
+    const int v = blockIdx.x * AMAX_COLS + 4 * threadIdx.x;              // four consecutive features (the slabs' rows are padded)
+    if (v < V) {
+        float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
+        for (int s = 0; s < n_parts; ++s) add4(z4, *(const float4*)(pr + s * split_stride + v));
+        const float z[4] = {z4.x, z4.y, z4.z, z4.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            if (v + e >= V) break;
+            if (logits) logits[(size_t)row * V + v + e] = z[e];
+            if (z[e] > best) { best = z[e]; bidx = v + e; }     // ascending: strict > keeps the lowest id
         }
     }
     for (int o = 16; o > 0; o >>= 1) {
@@ -1061,9 +1056,9 @@ static bool cl_rows(const anpd_model* m, const anpd_kv* kv, int rows) {
     return !m->plain_gemm && (rows == kv->batch * ANPD_ROWS || rows <= CL_PROMPT_ROWS);
 }
 
-// One projection of a prompt pass, of a step of several sequences or, with the plain GEMM, of any forward.  Returns the number
-// of partial sums per 128-feature storage tile its consumer must add.
-anpd_status gemm_enqueue(anpd_model* m, anpd_kv* kv, int kind, int layer, int rows, const int** seg_count_out, int* seg_max_out) {
+// One projection of a prompt pass, of a step of several sequences or, with the plain GEMM, of any forward.  Returns how many
+// partial sums every output has and, where some 128-feature storage tiles have more, all tiles' counts.
+anpd_status gemm_enqueue(anpd_model* m, anpd_kv* kv, int kind, int layer, int rows, const int** seg_count_out, int* seg_min_out) {
     Workspace& ws = kv->ws;
     const ClPlan& plan = m->cl[kind];
     const unsigned char* W = kind == GK_LM ? m->lm_head : (kind == GK_QKV ? m->layers[layer].wqkv : kind == GK_O ? m->layers[layer].wo
@@ -1073,14 +1068,14 @@ anpd_status gemm_enqueue(anpd_model* m, anpd_kv* kv, int kind, int layer, int ro
     if (kind == GK_O) { a_hi = ws.ao_hi; a_lo = ws.ao_lo; maps = ws.map_ao; }
     if (kind == GK_DOWN) { a_hi = ws.act_hi; a_lo = ws.act_lo; maps = ws.map_act; }
     if (m->plain_gemm) {
-        *seg_count_out = m->d_ones;
-        *seg_max_out = 1;
+        *seg_count_out = nullptr;
+        *seg_min_out = 1;
         return gemm_plain_enqueue(plan, W, a_hi, a_lo, rows, ws.part, ws.n_max_out, m->stream, &m->prof);
     }
     if (cl_rows(m, kv, rows)) {                        // a partial sum per CTA of a cluster
         const unsigned char* act = kind == GK_O ? ws.ci_ao : kind == GK_DOWN ? ws.ci_act : ws.ci_h;
-        *seg_count_out = m->d_const_segs[CL_CTAS];
-        *seg_max_out = CL_CTAS;
+        *seg_count_out = nullptr;
+        *seg_min_out = CL_CTAS;
         // the projection after this one, whose first weights are fetched into L2 under the small kernels between the two
         const bool last = layer + 1 == m->cfg.n_layers;
         const int next = kind == GK_QKV ? GK_O : kind == GK_O ? GK_GU : kind == GK_GU ? GK_DOWN : last ? GK_LM : GK_QKV;
@@ -1106,9 +1101,9 @@ anpd_status gemm_enqueue(anpd_model* m, anpd_kv* kv, int kind, int layer, int ro
         }
         *seg_count_out = m->d_tail_segs[kind];
     } else {
-        *seg_count_out = m->d_const_segs[sched.ksplit];
+        *seg_count_out = nullptr;
     }
-    *seg_max_out = std::max(sched.ksplit, sched.tail_split);
+    *seg_min_out = sched.ksplit;
     return gemm_pf_enqueue(plan, W, maps[0], maps[1], rows, ws.part, ws.n_max_out, (size_t)rows * ws.n_max_out, sched, m->num_sms,
                            ws.gemm_err, m->stream, &m->prof);
 }
@@ -1319,6 +1314,7 @@ anpd_status forward_enqueue(anpd_model* m, anpd_kv* kv, int rows, int max_pos, b
     if (m->rr_ready && kv->batch == 1 && rows == ANPD_ROWS && head && !m->plain_gemm && !two_candidates) return forward_rr_enqueue(m, kv, max_pos, want_logits);
     if (kv->step_ready && rows == kv->batch * ANPD_ROWS && head && !m->prof.on && !two_candidates) return step_kernel_enqueue(m, kv, max_pos, want_logits);
     const bool decode = rows == kv->batch * ANPD_ROWS && !m->plain_gemm;           // (or a prompt pass of as many rows)
+    const auto resid_norm = m->cfg.d_model <= 4 * NORM_THREADS ? resid_norm_kernel<1> : m->cfg.d_model <= 8 * NORM_THREADS ? resid_norm_kernel<2> : resid_norm_kernel<NORM_MAX_CHUNKS>;
     const bool slab = cl_rows(m, kv, rows);
     if (decode && kv->batch == 1 && head && m->cl_all_fused) return forward_cl_enqueue(m, kv, max_pos, want_logits, two_candidates);
     const anpd_model_config& c = m->cfg;
@@ -1332,53 +1328,53 @@ anpd_status forward_enqueue(anpd_model* m, anpd_kv* kv, int rows, int max_pos, b
     const size_t sstride = (size_t)rows * ws.n_max_out;                            // between the partial sums of an output (the K parts of a projection)
     const size_t layer_elems = (size_t)kv->total_pages * c.n_kv_heads * KV_PAGE * hd;
     const int* segs = nullptr;
-    int seg_max = 1;                                   // the most partial sums a tile of the last projection has
+    int seg_min = 1;                                   // partial sums every tile of the last projection has
 
     LAUNCH(pf, st, KC_OTHER, 0, (launch_k(embed_norm_kernel, rows, NORM_THREADS, 0, st, m->embed, ws.row_tok, m->layers[0].attn_norm, c.rms_eps, d,
                                                                       ws.x, ws.h_hi, ws.h_lo, slab ? ws.ci_h : nullptr)));
-    const bool many_rows = rows >= 64;                 // prefill passes: throughput-shaped launches of the small kernels
-    const int rope_hpb = many_rows ? 256 / (hd / 2) : 1;            // heads per block of the rotary kernel
     for (int l = 0; l < c.n_layers; ++l) {
         const LayerW& w = m->layers[l];
-        ANPD_TRY(gemm_enqueue(m, kv, GK_QKV, l, rows, &segs, &seg_max));
+        ANPD_TRY(gemm_enqueue(m, kv, GK_QKV, l, rows, &segs, &seg_min));
         if (rows != kv->batch * ANPD_ROWS) {            // a prompt pass
-            const dim3 grid((rows + ROPE_TILE_ROWS - 1) / ROPE_TILE_ROWS, c.n_q_heads + 2 * c.n_kv_heads);
+            // as many heads at once as keep every SM's 2048 threads busy, the others by the same blocks
+            const int tiles = (rows + ROPE_TILE_ROWS - 1) / ROPE_TILE_ROWS;
+            const dim3 grid(std::min(c.n_q_heads + 2 * c.n_kv_heads, std::max(1, m->num_sms * 8 / tiles)), tiles);
             const float qs = 1.4426950408889634f / sqrtf((float)hd);
             if (hd == 128) LAUNCH(pf, st, KC_OTHER, 0,
                    (launch_k(qkv_rope_append_tile_kernel<128>, grid, 256, 0, st, ws.part, segs, sstride, ws.n_max_out, rows, ws.row_pos, ws.row_seq, ws.row_ok,
                              kv->rope_cos, kv->rope_sin, kv->page_table, kv->pages_per_seq, c.n_q_heads, c.n_kv_heads, qs, ws.q_hi, ws.q_lo,
-                             kv->kpool + l * layer_elems, kv->vpool + l * layer_elems)));
+                             kv->kpool + l * layer_elems, kv->vpool + l * layer_elems, seg_min)));
             else LAUNCH(pf, st, KC_OTHER, 0,
                    (launch_k(qkv_rope_append_tile_kernel<64>, grid, 256, 0, st, ws.part, segs, sstride, ws.n_max_out, rows, ws.row_pos, ws.row_seq, ws.row_ok,
                              kv->rope_cos, kv->rope_sin, kv->page_table, kv->pages_per_seq, c.n_q_heads, c.n_kv_heads, qs, ws.q_hi, ws.q_lo,
-                             kv->kpool + l * layer_elems, kv->vpool + l * layer_elems)));
+                             kv->kpool + l * layer_elems, kv->vpool + l * layer_elems, seg_min)));
         } else
         LAUNCH(pf, st, KC_OTHER, 0,
-               (launch_k(qkv_rope_append_kernel, dim3(rows, (c.n_q_heads + 2 * c.n_kv_heads + rope_hpb - 1) / rope_hpb), rope_hpb * (hd / 2), 0, st, 
+               (launch_k(qkv_rope_append_kernel, dim3(rows, (c.n_q_heads + 2 * c.n_kv_heads + 1024 / hd - 1) / (1024 / hd)), 128, 0, st,
                    ws.part, segs, sstride, ws.n_max_out, ws.row_pos, ws.row_slot, ws.row_seq, ws.row_ok, kv->rope_cos, kv->rope_sin,
                    kv->page_table, kv->pages_per_seq, c.n_q_heads, c.n_kv_heads, hd, 1.4426950408889634f / sqrtf((float)hd), ws.q_hi,
-                   ws.q_lo, kv->kpool + l * layer_elems, kv->vpool + l * layer_elems, seg_max)));
+                   ws.q_lo, kv->kpool + l * layer_elems, kv->vpool + l * layer_elems, seg_min)));
         unsigned char* ao_img = slab ? ws.ci_ao : nullptr;
         const int ao_rows = slab ? rows : 0;
-        if (decode && hd == 64) ANPD_TRY(attn_dec_enqueue(m, kv, l, two_candidates));
+        if (decode && attn_dec_supported(m) && (hd == 64 || kv->attn_tc)) ANPD_TRY(attn_dec_enqueue(m, kv, l, two_candidates));
         else if (hd == 128) ANPD_TRY(attn_enqueue<128>(m, kv, l, rows, max_pos, ao_img, two_candidates, ao_rows));
         else ANPD_TRY(attn_enqueue<64>(m, kv, l, rows, max_pos, ao_img, two_candidates, ao_rows));
-        ANPD_TRY(gemm_enqueue(m, kv, GK_O, l, rows, &segs, &seg_max));
+        ANPD_TRY(gemm_enqueue(m, kv, GK_O, l, rows, &segs, &seg_min));
         LAUNCH(pf, st, KC_OTHER, 0,
-               (launch_k(resid_norm_kernel, rows, NORM_THREADS, 0, st, ws.x, ws.part, segs, sstride, ws.n_max_out, w.ffn_norm, c.rms_eps, d,
-                                                       ws.h_hi, ws.h_lo, seg_max, slab ? ws.ci_h : nullptr)));
-        ANPD_TRY(gemm_enqueue(m, kv, GK_GU, l, rows, &segs, &seg_max));
-        if (many_rows) LAUNCH(pf, st, KC_OTHER, 0,
-               (launch_k(swiglu_wide_kernel, dim3((F / 4 + 511) / 512, rows), 256, 0, st, ws.part, segs, sstride, ws.n_max_out, F, ws.act_hi,
-                         ws.act_lo, slab ? ws.ci_act : nullptr)));
+               (launch_k(resid_norm, rows, NORM_THREADS, 0, st, ws.x, ws.part, segs, sstride, ws.n_max_out, w.ffn_norm, c.rms_eps, d,
+                                                       ws.h_hi, ws.h_lo, seg_min, slab ? ws.ci_h : nullptr)));
+        ANPD_TRY(gemm_enqueue(m, kv, GK_GU, l, rows, &segs, &seg_min));
+        if (rows >= 256) LAUNCH(pf, st, KC_OTHER, 0,
+               (launch_k(swiglu_kernel<2>, dim3((F / 4 + 511) / 512, rows), 256, 0, st, ws.part, segs, sstride, ws.n_max_out, F, ws.act_hi, ws.act_lo,
+                         seg_min, slab ? ws.ci_act : nullptr)));
         else LAUNCH(pf, st, KC_OTHER, 0,
-               (launch_k(swiglu_kernel, dim3((F + 255) / 256, rows), 256, 0, st, ws.part, segs, sstride, ws.n_max_out, F, ws.act_hi,
-                                                                          ws.act_lo, seg_max, slab ? ws.ci_act : nullptr)));
-        ANPD_TRY(gemm_enqueue(m, kv, GK_DOWN, l, rows, &segs, &seg_max));
+               (launch_k(swiglu_kernel<1>, dim3((F / 4 + 255) / 256, rows), 256, 0, st, ws.part, segs, sstride, ws.n_max_out, F, ws.act_hi, ws.act_lo,
+                         seg_min, slab ? ws.ci_act : nullptr)));
+        ANPD_TRY(gemm_enqueue(m, kv, GK_DOWN, l, rows, &segs, &seg_min));
         const float* next_gain = (l + 1 < c.n_layers) ? m->layers[l + 1].attn_norm : m->final_norm;
         LAUNCH(pf, st, KC_OTHER, 0,
-               (launch_k(resid_norm_kernel, rows, NORM_THREADS, 0, st, ws.x, ws.part, segs, sstride, ws.n_max_out, next_gain, c.rms_eps, d,
-                                                       ws.h_hi, ws.h_lo, seg_max, decode || (slab && l + 1 < c.n_layers) ? ws.ci_h : nullptr)));
+               (launch_k(resid_norm, rows, NORM_THREADS, 0, st, ws.x, ws.part, segs, sstride, ws.n_max_out, next_gain, c.rms_eps, d,
+                                                       ws.h_hi, ws.h_lo, seg_min, decode || (slab && l + 1 < c.n_layers) ? ws.ci_h : nullptr)));
     }
     if (!head) { CUDA_TRY(cudaGetLastError()); return ANPD_OK; }
     // A prompt pass needs the LM head for its last token only: the group of 8 rows that holds it becomes rows 0-7 of a decode
@@ -1394,9 +1390,9 @@ anpd_status forward_enqueue(anpd_model* m, anpd_kv* kv, int rows, int max_pos, b
         LAUNCH(pf, st, KC_OTHER, 0, (launch_k(move_rows_kernel, ANPD_ROWS, 256, 0, st, ws.h_hi, ws.h_lo, group, d)));
     }
     rows = kv->batch * ANPD_ROWS;
-    ANPD_TRY(gemm_enqueue(m, kv, GK_LM, 0, rows, &segs, &seg_max));
+    ANPD_TRY(gemm_enqueue(m, kv, GK_LM, 0, rows, &segs, &seg_min));
     LAUNCH(pf, st, KC_OTHER, 0,
-           (launch_k(argmax_partial_kernel, dim3(ws.amax_blocks, rows), 256, 0, st, ws.part, segs, (size_t)rows * ws.n_max_out, ws.n_max_out, V,
+           (launch_k(argmax_partial_kernel, dim3(ws.amax_blocks, rows), 256, 0, st, ws.part, seg_min, (size_t)rows * ws.n_max_out, ws.n_max_out, V,
                                                                              want_logits ? ws.logits : nullptr, ws.amax_val,
                                                                              ws.amax_idx, ws.amax_blocks)));
     CUDA_TRY(cudaGetLastError());

@@ -350,8 +350,6 @@ struct anpd_model {
     const __nv_bfloat16* block_lm;
     void* block_slab;
     int* d_plan_tables;               // device copies of the plans' tables
-    int* d_ones;                      // [tiles] all 1: partial sums per tile of a projection that is not cut along K
-    int* d_const_segs[9];             // [tiles] all k (k = 1..8): partial sums per tile of a projection cut into k parts along K
     int* d_tail_segs[GK_COUNT];       // [tiles] segment counts of a prompt-pass GEMM whose last tiles alone are cut (PfSchedule)
     int tail_cfg[GK_COUNT];           // what d_tail_segs[kind] holds: first cut feature tile * 8 + parts, -1 = nothing yet
     bool plain_gemm;                  // debugging aid: route GEMMs through the plain kernel
