@@ -1,4 +1,4 @@
-// Causal attention of a prompt pass (Algorithm 1's LLM(prompt)) for head dimension 128, with the query rows on the
+// Causal attention of a prompt pass (Algorithm 1's LLM(prompt)) for head dimensions 64 and 128, with the query rows on the
 // tensor-memory lanes: a CTA takes 128 consecutive rows of one query head through all the pages (of its kv head) those rows
 // may see.
 //
@@ -10,15 +10,20 @@
 //
 // A row's scores live in the two threads that share the row (both read all 128 scores of a page and find the same maximum;
 // each turns 64 of them into weights), so maxima need no exchange between threads and the sums one per tile.  Roles: one thread requests
-// the Q tiles and the K / V^T pages (TMA, a ring of three page buffers filled in the order the products use them: K0, K1, V0,
+// the Q tiles and the K / V^T pages (TMA, a ring of page buffers filled in the order the products use them: K0, K1, V0,
 // K2, V1, ...), one thread issues the products (S of page c+1 before O of page c, so that the tensor core works on the next
 // scores while the softmax threads work on these), 256 threads do the softmax, the rescaling and the epilogue.  Two score
 // accumulators alternate.  Pages are visited in ascending order and a row's result depends on its own position and inputs
 // only.  The queries carry log2(e) / sqrt(hd), as everywhere.  Every wait is bounded and reports through the error flag.
+//
+// Bound by the softmax threads (about 2000 cycles per page and row tile) from a few hundred rows on, by its chain of loads, product,
+// softmax, product below.  Head dimension 64, 8 query heads per kv head (page partials on mma.sync and a merging kernel before):
+// 333 rows 31 -> 14 us, 1024 rows 105 -> 26 us per layer; 1.1B prompt pass of 1024 tokens 6.8 -> 5.0 ms, of 333 tokens 2.8 -> 2.4.
 #include "internal.h"
 #include "tc_ptx.cuh"
 
 #include <algorithm>
+#include <type_traits>
 #include <math_constants.h>
 
 typedef __nv_bfloat16 bf16;
@@ -27,13 +32,15 @@ namespace {
 
 using namespace tc;
 
-constexpr int FA_HD = 128;
 constexpr int FA_ROWS = 128;
 constexpr int FA_ATOM = 16384;               // 128 rows x 64 bf16, 128-byte swizzle (one TMA box)
 constexpr int FA_OPER = 2 * FA_ATOM;         // a 128 x 128 bf16 operand: two boxes
-constexpr int FA_RING = 3;
 constexpr int FA_THREADS = 320;              // warp 0: loads, warp 1: products + tensor-memory owner, warps 2-9: softmax (two threads per row)
-constexpr int FA_SMEM = (4 + FA_RING) * FA_OPER + 1024;      // Q hi, Q lo, P hi, P lo, three page buffers
+template <int HD> struct FaCfg {
+    static constexpr int PAGE = HD * 256;    // a page's K (128 rows of HD) or V^T (HD rows of 128, as two boxes of 64 keys); also the Q tile's hi or lo terms
+    static constexpr int RING = HD == 64 ? 5 : 3;            // page buffers
+    static constexpr int SMEM = (2 + RING) * PAGE + 2 * FA_OPER + 1024;      // Q hi, Q lo, P hi, P lo, the page buffers
+};
 constexpr int FA_ERR_TIMEOUT = 206;
 constexpr float FA_LAZY = 8.0f;             // base-2 exponent by which a page's maximum must exceed the reference to move it
 
@@ -45,18 +52,22 @@ __device__ __forceinline__ int fa_offset(int row, int k) {
     return (k >> 6) * FA_ATOM + (row >> 3) * 1024 + (row & 7) * 128 + (((kk >> 3) ^ (row & 7)) << 4) + (kk & 7) * 2;
 }
 
+template <int V> using FaInt = std::integral_constant<int, V>;
+
 struct FaArgs {
     const int* page_table; int pages_per_seq;
     const int* row_pos; const int* row_seq;
-    int H, Hkv, layer_row0, rows, n_row_tiles;      // query heads, kv heads (H a multiple of Hkv)
+    int H, Hkv, layer_page0, rows, n_row_tiles;     // query heads, kv heads (H a multiple of Hkv)
     bf16* ao_hi; bf16* ao_lo;
     unsigned char* img;                     // the O projection's operand image (few rows) instead of ao_hi and ao_lo
     int* err;
 };
 
+template <int HD>
 __global__ void __launch_bounds__(FA_THREADS, 1)
 attn_pf_kernel(const __grid_constant__ CUtensorMap map_qh, const __grid_constant__ CUtensorMap map_ql,
                const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v, const FaArgs g) {
+    constexpr int FA_RING = FaCfg<HD>::RING, PAGE = FaCfg<HD>::PAGE;
     extern __shared__ __align__(1024) unsigned char fa_smem_raw[];
     __shared__ uint64_t q_full, q_empty, ring_full[FA_RING], ring_empty[FA_RING], s_full[2], s_empty[2], p_full, o_done, o_free;
     __shared__ uint32_t tmem_slot;
@@ -66,10 +77,10 @@ attn_pf_kernel(const __grid_constant__ CUtensorMap map_qh, const __grid_constant
     pdl_trigger();
     unsigned char* smem = fa_smem_raw + ((1024u - (smem_u32(fa_smem_raw) & 1023u)) & 1023u);
     unsigned char* Qh = smem;
-    unsigned char* Ql = smem + FA_OPER;
-    unsigned char* Ph = smem + 2 * FA_OPER;
-    unsigned char* Pl = smem + 3 * FA_OPER;
-    unsigned char* ring = smem + 4 * FA_OPER;
+    unsigned char* Ql = smem + PAGE;                       // 128 rows of HD: as large as a page's K
+    unsigned char* Ph = smem + 2 * PAGE;
+    unsigned char* Pl = Ph + FA_OPER;
+    unsigned char* ring = Pl + FA_OPER;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
     if (threadIdx.x == 0) {
@@ -114,7 +125,7 @@ attn_pf_kernel(const __grid_constant__ CUtensorMap map_qh, const __grid_constant
 
     if (warp == 0) {
         // ---------------- loads ----------------
-        if (lane == 0) {
+        if (elect_one()) {
             const uint64_t pol = policy_evict_last();               // a page is read by every row tile behind it
             uint32_t tq = 0, li = 0;                                // tiles begun, page loads issued so far
             bool ok = true;
@@ -123,11 +134,13 @@ attn_pf_kernel(const __grid_constant__ CUtensorMap map_qh, const __grid_constant
                 item(it, r0, h, n_pages, seq, pos_lo);
                 ok = mbar_wait(&q_empty, (tq & 1u) ^ 1u, abortp);
                 if (!ok) break;
-                mbar_expect_tx(&q_full, 2 * FA_OPER);
-                tma_load_2d(Qh, &map_qh, h * FA_HD, r0, &q_full, pol);
-                tma_load_2d(Qh + FA_ATOM, &map_qh, h * FA_HD + 64, r0, &q_full, pol);
-                tma_load_2d(Ql, &map_ql, h * FA_HD, r0, &q_full, pol);
-                tma_load_2d(Ql + FA_ATOM, &map_ql, h * FA_HD + 64, r0, &q_full, pol);
+                mbar_expect_tx(&q_full, 2 * PAGE);
+#pragma unroll
+                for (int a = 0; a < HD / 64; ++a) {
+                    tma_load_2d(Qh + a * FA_ATOM, &map_qh, h * HD + 64 * a, r0, &q_full, pol);
+                    tma_load_2d(Ql + a * FA_ATOM, &map_ql, h * HD + 64 * a, r0, &q_full, pol);
+                }
+                const int kvh = h / (g.H / g.Hkv);
                 // K0, then for every page c: K(c+1) if there is one, V(c)
                 for (int j = 0; j < 2 * n_pages && ok; ++j, ++li) {
                     // j = 0: K0; odd j: K((j+1)/2) while it exists; even j > 0: V(j/2 - 1); the tail: V(n-1)
@@ -140,11 +153,16 @@ attn_pf_kernel(const __grid_constant__ CUtensorMap map_qh, const __grid_constant
                     const uint32_t slot = li % FA_RING, use = li / FA_RING;
                     ok = mbar_wait(&ring_empty[slot], (use & 1u) ^ 1u, abortp);
                     if (!ok) break;
-                    const int row = g.layer_row0 + (g.page_table[seq * g.pages_per_seq + c] * g.Hkv + h / (g.H / g.Hkv)) * KV_PAGE;
-                    unsigned char* dst = ring + (size_t)slot * FA_OPER;
-                    mbar_expect_tx(&ring_full[slot], FA_OPER);
-                    tma_load_2d(dst, kk ? &map_k : &map_v, 0, row, &ring_full[slot], pol);
-                    tma_load_2d(dst + FA_ATOM, kk ? &map_k : &map_v, 64, row, &ring_full[slot], pol);
+                    const int page = (g.layer_page0 + g.page_table[seq * g.pages_per_seq + c]) * g.Hkv + kvh;
+                    unsigned char* dst = ring + (size_t)slot * PAGE;
+                    mbar_expect_tx(&ring_full[slot], PAGE);
+                    if (kk) {
+#pragma unroll
+                        for (int a = 0; a < HD / 64; ++a) tma_load_2d(dst + a * FA_ATOM, &map_k, 64 * a, page * KV_PAGE, &ring_full[slot], pol);
+                    } else {
+#pragma unroll
+                        for (int a = 0; a < 2; ++a) tma_load_2d(dst + a * HD * 128, &map_v, 64 * a, page * HD, &ring_full[slot], pol);
+                    }
                 }
             }
             if (!ok) {
@@ -158,22 +176,23 @@ attn_pf_kernel(const __grid_constant__ CUtensorMap map_qh, const __grid_constant
         }
     } else if (warp == 1) {
         // ---------------- products ----------------
-        if (lane == 0) {
-            // fp32 accumulate, bf16 x bf16, both operands K-major, M = 128, N = 128
-            const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(128 >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+        if (elect_one()) {
+            // fp32 accumulate, bf16 x bf16, both operands K-major, M = 128 rows, N = 128 keys or HD dimensions
+            constexpr uint32_t idesc0 = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(128 >> 4) << 24);
             uint32_t tq = 0, li = 0, pc = 0;                        // tiles, page loads consumed, pages whose S was issued
             uint32_t pv = 0;                                        // pages whose O product was issued
             bool ok = true;
-            auto product = [&](uint32_t d_tmem, const unsigned char* a_hi, const unsigned char* a_lo, const unsigned char* b, uint32_t acc) {
-                // D (+)= A_hi B^T + A_lo B^T over the 128-wide contraction: 8 steps of 16 per term
+            // D (+)= A_hi B^T + A_lo B^T over `steps` x 16 of the contraction, N columns; b_atom: bytes of 64 of it in B
+            auto product = [&](auto steps, auto N, auto b_atom, uint32_t d_tmem, const unsigned char* a_hi, const unsigned char* a_lo, const unsigned char* b, uint32_t acc) {
+                constexpr uint32_t idesc = idesc0 | ((uint32_t)(decltype(N)::value >> 3) << 17);
 #pragma unroll
                 for (int term = 0; term < 2; ++term) {
                     const unsigned char* a = term ? a_lo : a_hi;
 #pragma unroll
-                    for (int k16 = 0; k16 < 8; ++k16) {
+                    for (int k16 = 0; k16 < decltype(steps)::value; ++k16) {
                         const uint64_t adv = (uint64_t)((k16 & 3) * 2);
                         tc_mma_bf16(d_tmem, make_smem_desc(smem_u32(a + (k16 >> 2) * FA_ATOM)) + adv,
-                                    make_smem_desc(smem_u32(b + (k16 >> 2) * FA_ATOM)) + adv, idesc, (acc | term | k16) ? 1u : 0u);
+                                    make_smem_desc(smem_u32(b + (k16 >> 2) * decltype(b_atom)::value)) + adv, idesc, (acc | term | k16) ? 1u : 0u);
                     }
                 }
             };
@@ -187,7 +206,7 @@ attn_pf_kernel(const __grid_constant__ CUtensorMap map_qh, const __grid_constant
                     if (!mbar_wait(&ring_full[slot], use & 1u, abortp)) return false;
                     if (!mbar_wait(&s_empty[b], ((pc >> 1) & 1u) ^ 1u, abortp)) return false;
                     tc_fence_after();
-                    product(tm_s0 + b * 128u, Qh, Ql, ring + (size_t)slot * FA_OPER, 0u);
+                    product(FaInt<HD / 16>(), FaInt<KV_PAGE>(), FaInt<FA_ATOM>(), tm_s0 + b * 128u, Qh, Ql, ring + (size_t)slot * PAGE, 0u);
                     tc_commit(&ring_empty[slot]);
                     tc_commit(&s_full[b]);
                     ++li; ++pc;
@@ -203,7 +222,7 @@ attn_pf_kernel(const __grid_constant__ CUtensorMap map_qh, const __grid_constant
                     ok = mbar_wait(&p_full, pv & 1u, abortp);
                     if (!ok) break;
                     tc_fence_after();
-                    product(tm_o, Ph, Pl, ring + (size_t)slot * FA_OPER, c > 0 ? 1u : 0u);
+                    product(FaInt<KV_PAGE / 16>(), FaInt<HD>(), FaInt<HD * 128>(), tm_o, Ph, Pl, ring + (size_t)slot * PAGE, c > 0 ? 1u : 0u);
                     tc_commit(&ring_empty[slot]);
                     tc_commit(&o_done);
                     ++li; ++pv;
@@ -214,7 +233,7 @@ attn_pf_kernel(const __grid_constant__ CUtensorMap map_qh, const __grid_constant
     } else {
         // ---------------- softmax, rescaling, epilogue: two threads per row ----------------
         // Both threads of a row read all its 128 scores and find the same maximum; each then turns its own 64 keys into
-        // weights, rescales and finally writes its own 64 output dimensions; the two halves of the weights' sum meet once
+        // weights, rescales and finally writes its own half of the output dimensions; the two halves of the weights' sum meet once
         // per tile.
         const int quad = warp & 3;                        // a warp may only touch tensor-memory lanes 32 * (warp % 4) .. + 31
         const int half = (warp - 2) >> 2;                 // warps 2-5: keys / dimensions 0-63, warps 6-9: 64-127
@@ -267,12 +286,12 @@ attn_pf_kernel(const __grid_constant__ CUtensorMap map_qh, const __grid_constant
                     tc_fence_after();
                     if (__any_sync(0xffffffffu, scale != 1.0f)) {
 #pragma unroll 1
-                        for (int ch = 0; ch < 2; ++ch) {
+                        for (int ch = 0; ch < HD / 64; ++ch) {
                             float o[32];
-                            tc_ld32(tm_o + lane_addr + (uint32_t)(half * 64 + ch * 32), o);
+                            tc_ld32(tm_o + lane_addr + (uint32_t)(half * (HD / 2) + ch * 32), o);
 #pragma unroll
                             for (int i = 0; i < 32; ++i) o[i] *= scale;
-                            tc_st32(tm_o + lane_addr + (uint32_t)(half * 64 + ch * 32), o);
+                            tc_st32(tm_o + lane_addr + (uint32_t)(half * (HD / 2) + ch * 32), o);
                         }
                     }
                 }
@@ -317,9 +336,9 @@ attn_pf_kernel(const __grid_constant__ CUtensorMap map_qh, const __grid_constant
             if (!ok) break;
             tc_fence_after();
 #pragma unroll 1
-            for (int ch = 0; ch < 2; ++ch) {
+            for (int ch = 0; ch < HD / 64; ++ch) {
                 float o[32];
-                tc_ld32(tm_o + lane_addr + (uint32_t)(half * 64 + ch * 32), o);
+                tc_ld32(tm_o + lane_addr + (uint32_t)(half * (HD / 2) + ch * 32), o);
                 if (row < g.rows) {
                     __nv_bfloat162 hh[16], ll[16];
 #pragma unroll
@@ -329,10 +348,10 @@ attn_pf_kernel(const __grid_constant__ CUtensorMap map_qh, const __grid_constant
                         const float2 back = __bfloat1622float2(hh[i >> 1]);
                         ll[i >> 1] = __floats2bfloat162_rn(t0 - back.x, t1 - back.y);
                     }
-                    const size_t out = (size_t)row * g.H * FA_HD + (size_t)h * FA_HD + half * 64 + ch * 32;
+                    const size_t out = (size_t)row * g.H * HD + (size_t)h * HD + half * (HD / 2) + ch * 32;
 #pragma unroll
                     for (int u = 0; u < 4; ++u) {
-                        const int k = h * FA_HD + half * 64 + ch * 32 + 8 * u;
+                        const int k = h * HD + half * (HD / 2) + ch * 32 + 8 * u;
                         *(uint4*)(g.img ? (bf16*)(g.img + cl_img_offset(g.rows, row, k)) : g.ao_hi + out + 8 * u) = *(const uint4*)(hh + 4 * u);
                         *(uint4*)(g.img ? (bf16*)(g.img + cl_img_offset(g.rows, g.rows + row, k)) : g.ao_lo + out + 8 * u) = *(const uint4*)(ll + 4 * u);
                     }
@@ -357,26 +376,29 @@ attn_pf_kernel(const __grid_constant__ CUtensorMap map_qh, const __grid_constant
 }  // namespace
 
 // Attention of a prompt pass over `rows` rows (a multiple of 8; the row plan covers the padding) of sequence row_seq[0].
-// map_qh / map_ql: the pass's queries [rows][H * 128] seen through boxes of 64 columns x 128 rows.
+// map_q: the pass's queries [rows][H * hd] seen through boxes of 64 columns x 128 rows.
+template <int HD>
+static anpd_status launch_attn_pf(anpd_model* m, anpd_kv* kv, const FaArgs& g) {
+    static bool attr_set[64] = {false};
+    if (first_call_on_device(attr_set)) CUDA_TRY(cudaFuncSetAttribute(attn_pf_kernel<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, FaCfg<HD>::SMEM));
+    const int grid = std::min(m->num_sms, g.n_row_tiles * g.H);
+    LAUNCH(&m->prof, m->stream, KC_ATTN, 0,
+           (launch_k(attn_pf_kernel<HD>, grid, FA_THREADS, (size_t)FaCfg<HD>::SMEM, m->stream, kv->ws.map_q[0], kv->ws.map_q[1], kv->map_k, kv->map_v, g)));
+    CUDA_TRY(cudaGetLastError());
+    return ANPD_OK;
+}
+
 anpd_status attn_pf_enqueue(anpd_model* m, anpd_kv* kv, int layer, int rows, unsigned char* img) {
     const anpd_model_config& c = m->cfg;
     Workspace& ws = kv->ws;
-    static bool attr_set[64] = {false};
-    if (first_call_on_device(attr_set)) {
-        CUDA_TRY(cudaFuncSetAttribute(attn_pf_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FA_SMEM));
-    }
     FaArgs g;
     g.page_table = kv->page_table; g.pages_per_seq = kv->pages_per_seq;
     g.row_pos = ws.row_pos; g.row_seq = ws.row_seq;
     g.H = c.n_q_heads; g.Hkv = c.n_kv_heads;
-    g.layer_row0 = layer * kv->total_pages * c.n_kv_heads * KV_PAGE;
+    g.layer_page0 = layer * kv->total_pages;
     g.rows = rows;
     g.n_row_tiles = (rows + FA_ROWS - 1) / FA_ROWS;
     g.ao_hi = ws.ao_hi; g.ao_lo = ws.ao_lo; g.img = img;
     g.err = ws.gemm_err;
-    const int grid = std::min(m->num_sms, g.n_row_tiles * g.H);
-    LAUNCH(&m->prof, m->stream, KC_ATTN, 0,
-           (launch_k(attn_pf_kernel, grid, FA_THREADS, (size_t)FA_SMEM, m->stream, ws.map_q[0], ws.map_q[1], kv->map_k, kv->map_v, g)));
-    CUDA_TRY(cudaGetLastError());
-    return ANPD_OK;
+    return c.head_dim == 64 ? launch_attn_pf<64>(m, kv, g) : launch_attn_pf<128>(m, kv, g);
 }

@@ -1121,7 +1121,7 @@ anpd_status attn_enqueue(anpd_model* m, anpd_kv* kv, int layer, int rows, int ma
         CUDA_TRY(cudaFuncSetAttribute(attn_partial_kernel<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     }
     // a prompt pass: pages are folded in the kernel, nothing to merge (the older 16-row kernel knows one query head per kv head only)
-    if (HD == 128 && kv->attn_tc && rows != kv->batch * ANPD_ROWS && kv->attn_pf) return attn_pf_enqueue(m, kv, layer, rows, img);
+    if (rows != kv->batch * ANPD_ROWS && kv->attn_pf) return attn_pf_enqueue(m, kv, layer, rows, img);
     if (HD == 128 && kv->attn_tc && rows != kv->batch * ANPD_ROWS && c.n_q_heads == c.n_kv_heads) {
         ANPD_TRY(attn_prompt_enqueue(m, kv, layer, rows));
         if (img) LAUNCH(&m->prof, m->stream, KC_ATTN, 0, (launch_k(rows_to_image_kernel, rows, 256, 0, m->stream, ws.ao_hi, ws.ao_lo, 0, m->dq, img, rows)));
