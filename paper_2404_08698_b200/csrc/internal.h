@@ -162,11 +162,11 @@ struct NgramDev {
 
 struct anpd_ngram {
     NgramDev h;            // host copy of the descriptor (device pointers inside)
-    NgramDev* d;           // device copy, for kernels that take an array of descriptors
     cudaStream_t stream;
     int n_tokens;          // host mirror, valid whenever no asynchronous loop is running
     int n_folded;          // host mirror of state[1]: tokens below it are in the tables
-    int* pinned;           // small pinned staging buffer
+    int* pinned;           // host memory a call's kernel leaves its results in
+    int ticket;            // the last call's
     void* slab;            // all tables, one allocation
     size_t slab_bytes;
 };
