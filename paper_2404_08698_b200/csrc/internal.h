@@ -171,6 +171,7 @@ struct anpd_ngram {
     size_t slab_bytes;
 };
 
+anpd_status ngram_reset_enqueue(anpd_ngram* ctx);
 // on: the stream to launch on (null: the context's own)
 anpd_status ngram_enqueue_bulk(anpd_ngram* ctx, int from, int to, Profiler* prof, cudaStream_t on = nullptr);
 // One fused launch for `batch` sequences: folds tokens [state[1], state[0]) of each, then drafts
@@ -445,6 +446,8 @@ struct StepParams {
     int trace_cta;
 };
 
+constexpr int LOGIT_PIECES = 4;
+
 struct anpd_kv {
     anpd_model* m;
     int batch, max_len, pages_per_seq, total_pages;
@@ -459,6 +462,8 @@ struct anpd_kv {
     int* d_prompt;                    // device [max_len]
     NgramDev* d_ctxs;                 // device [batch]: descriptors of the sequences' n-gram contexts
     int* h_small;                     // pinned, a few ints
+    float* h_logits;                  // pinned, [ANPD_ROWS][vocab]: logits on their way to the caller (one sequence only)
+    cudaEvent_t ev_logits[LOGIT_PIECES];
     std::vector<int> h_kv_len;        // host mirror of the sequences' lengths
     std::vector<char> h_len_stale;    // a committing step was enqueued and its outcome not read yet: the mirror is behind
     Workspace ws;

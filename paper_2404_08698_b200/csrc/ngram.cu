@@ -304,6 +304,13 @@ anpd_status ngram_enqueue_step(const NgramDev* d_ctxs, SeqState* d_seq, int batc
     return ANPD_OK;
 }
 
+anpd_status ngram_reset_enqueue(anpd_ngram* c) {
+    CUDA_TRY(cudaMemsetAsync(c->slab, 0, c->slab_bytes, c->stream));
+    c->n_tokens = 0;
+    c->n_folded = 0;
+    return ANPD_OK;
+}
+
 // ---------------------------------------------------------------------------------------------
 // boundary
 // ---------------------------------------------------------------------------------------------
@@ -351,10 +358,8 @@ anpd_status anpd_ngram_create(const anpd_ngram_config* cfg, void* cuda_stream, a
 
 anpd_status anpd_ngram_reset(anpd_ngram* c) {
     if (!c) return ANPD_ERR_ARG;
-    CUDA_TRY(cudaMemsetAsync(c->slab, 0, c->slab_bytes, c->stream));
+    ANPD_TRY(ngram_reset_enqueue(c));
     CUDA_TRY(cudaStreamSynchronize(c->stream));
-    c->n_tokens = 0;
-    c->n_folded = 0;
     return ANPD_OK;
 }
 
