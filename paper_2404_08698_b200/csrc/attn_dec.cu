@@ -1,20 +1,22 @@
-// Attention of a decode step, complete in one kernel: the 8 rows of a sequence's step (x the query heads of one kv head) against
-// the paged cache, softmax, and the result as the O projection's operand image.
+// Attention of a decode step, complete in one kernel: the 8 rows of a sequence's step against the paged cache, softmax, and the
+// result as the O projection's operand image.
 //
-// What bounds it: the cache's pages from HBM at long contexts; at short ones a memory round trip, the merge and the launch.  The
-// pages of one kv head of one sequence are dealt to the CTAs of a cluster: CTA v of C takes the pages p with p mod C == v, C (1, 2,
-// 4, and 8 with 4 or 8 query heads per kv head) being as many as the device holds at once.  A producer thread brings pages in
-// through a ring of TMA copies (those no kernel of this step writes before the dependency wait); eight or sixteen warps compute,
-// each on 16 keys at a time: block b of a page belongs to key slot b mod KW and to the MT warps of that slot, one per 16-row tile
-// of query vectors.
+// What bounds it: the cache's pages from HBM at long contexts; at short ones a memory round trip, the merge and the launch.  A
+// cluster of C CTAs takes one query head (or two that share a kv head) of one sequence: CTA v takes the pages p with p mod C == v.
+// A producer thread brings pages in through a ring of TMA copies (those no kernel of this step writes before the dependency
+// wait); eight warps compute, each on its 16 keys of every page.  Where more than two query heads share a kv head, several
+// clusters read its pages (from L2 but for the first) and each computes a part of the heads.  One cluster of eight CTAs per kv head
+// with four times the rows and twice the warps was slower, its chain of products per page being four times as long: 1.1B (8 query
+// heads per kv head), per step, 827 -> 800 us at 512 keys, 891 -> 839 at 1400, 1024 -> 937 at 4000.
 //
-// Order.  A slot takes its blocks in ascending order with a running maximum; the slots of a CTA are merged in slot order, the
+// Order.  A warp takes its blocks in ascending order with a running maximum; the warps of a CTA are merged in warp order, the
 // CTAs in rank order, each into the running result.  All of it depends on absolute key positions and on the handle (heads and
 // sequences) only, and a masked key contributes an exact zero, so a row's result does not depend on the rows it shares the step
 // with or on how far the cache reaches behind the row.
 //
-// mma.sync m16n8k16 (bf16, fp32 sums): with 8 to 64 query vectors per kv head the products are small beside the loads.  Queries
-// and weights enter as two bf16 terms; with one query head per kv head the two terms of the 8 rows are the tile's 16 rows.
+// mma.sync m16n8k16 (bf16, fp32 sums): with 8 or 16 query vectors the products are small beside the loads.  Queries and weights
+// enter as two bf16 terms; with one query head the two terms of the 8 rows are the tile's 16 rows.  The scores are summed in two
+// chains, which halves the wait for the products (7B at 1536 keys: 1104 -> 1089 us for 12 layers and the head).
 #include "internal.h"
 #include "tc_ptx.cuh"
 
@@ -29,45 +31,38 @@ namespace {
 using namespace tc;
 
 constexpr int AD_KEYS = 16;              // keys per block
-constexpr int AD_BLOCKS = KV_PAGE / AD_KEYS;
 constexpr int AD_MAX_CHUNKS = 6;
-constexpr int AD_SMEM_MAX = 216 * 1024;
 constexpr int AD_SMEM_PAIR = 111 * 1024; // two CTAs share an SM: another one of these, or one of the projection before or after
 constexpr int AD_ERR_TIMEOUT = 208;
 
+// HD: head dimension, G: query heads a CTA takes (1 or 2 of those that share a kv head)
 template <int HD, int G> struct AdCfg {
     static constexpr bool STACK = G == 1;                    // hi and lo terms of the 8 vectors share a tile
-    static constexpr int NV = STACK ? 8 : 16;                // query vectors per tile
-    static constexpr int Q = 8 * G;                          // query vectors per kv head
-    static constexpr int MT = Q / NV;                        // tiles (= warps per key slot)
-    static constexpr bool PAIR = G <= 2;
-    static constexpr int WARPS = PAIR ? 8 : 16;            // compute warps; one more loads
+    static constexpr int NV = STACK ? 8 : 16;                // query vectors of the CTA: one tile
+    static constexpr int WARPS = 8;                          // compute warps, each with 16 keys of a page; one more loads
     static constexpr int COMPUTE = 32 * WARPS, THREADS = COMPUTE + 32;
-    static constexpr int REGS = PAIR ? 104 : 96;
-    static constexpr int KW = WARPS / MT;                    // key slots of a share: 8, 8, 8, 4
-    static constexpr int C_MAX = PAIR ? 4 : 8;               // CTAs of a cluster
+    static constexpr int REGS = 112;
+    static constexpr int C_MAX = 4;                          // CTAs of a cluster
     static constexpr int OP = HD + 4;                        // padded row
     static constexpr int QP = HD * 2 + 16;                   // bytes per staged query row
-    static constexpr int QROWS = STACK ? 16 : 32 * MT;
+    static constexpr int QROWS = STACK ? 16 : 32;
     static constexpr int V4 = HD / 4;
     static constexpr int CHUNK = KV_PAGE * HD * 2;           // one copy: the page's K or its V^T
-    static constexpr int SLOTS = WARPS * NV * OP * 4;        // the slots' results
-    static constexpr int REST = 1024 + Q * HD * 4 + 2 * WARPS * NV * 4 + 2 * Q * 4 + QROWS * QP;
-    // PAIR (the steps with many kv heads, whose clusters fill the device): half an SM per CTA, in registers too, so that it starts
-    // beside a CTA of the projection before it and lets the next one start beside it, and 40 heads are resident at once.  7B, step
-    // of a short context 2.80 -> 2.69 ms, at 4096 keys 3.25 -> 3.14; one 13B sequence at 1024 keys 5.64 -> 5.35.  The CTA has read
-    // its last page when the slots' results are written: they take the ring's place.  With 4 or 8 query heads per kv head few CTAs
-    // run and twice the warps serve better (1.1B: 881 us per step, with half the warps 908).
-    static constexpr int ROOM = (PAIR ? AD_SMEM_PAIR : AD_SMEM_MAX) - REST - (PAIR ? 0 : SLOTS);
+    static constexpr int SLOTS = WARPS * NV * OP * 4;        // the warps' results
+    static constexpr int REST = 1024 + NV * HD * 4 + 2 * WARPS * NV * 4 + 2 * NV * 4 + QROWS * QP;
+    // Half an SM per CTA, in registers too, so that it starts beside a CTA of the projection before it and lets the next one start
+    // beside it.  7B, step of a short context 2.80 -> 2.69 ms, at 4096 keys 3.25 -> 3.14.  The CTA has read its last page when the
+    // warps' results are written: they take the ring's place.
+    static constexpr int ROOM = AD_SMEM_PAIR - REST;
     static constexpr int CHUNKS = ROOM / CHUNK < AD_MAX_CHUNKS ? ROOM / CHUNK : AD_MAX_CHUNKS;
-    static constexpr int RING = PAIR && CHUNKS * CHUNK < SLOTS ? SLOTS : CHUNKS * CHUNK;
-    static constexpr int SMEM = REST + RING + (PAIR ? 0 : SLOTS);
+    static constexpr int RING = CHUNKS * CHUNK < SLOTS ? SLOTS : CHUNKS * CHUNK;
+    static constexpr int SMEM = REST + RING;
 };
 
 struct AdArgs {
     const bf16 *q_hi, *q_lo;
     const int *page_table, *row_pos, *row_seq, *row_slot, *hole_lo, *hole_hi;      // row_slot and the holes: null outside two-candidate steps
-    int pages_per_seq, Hkv, rows, layer_page0;
+    int pages_per_seq, Hkv, split, rows, layer_page0;      // split: CTA clusters that share a kv head, G of its query heads each
     unsigned char* img;
     int* err;
 };
@@ -106,7 +101,7 @@ template <int HD, int G>
 __global__ void __launch_bounds__((AdCfg<HD, G>::THREADS)) __maxnreg__((AdCfg<HD, G>::REGS)) attn_dec_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v, const AdArgs g) {
     typedef AdCfg<HD, G> Cfg;
     constexpr bool STACK = Cfg::STACK;
-    constexpr int NV = Cfg::NV, MT = Cfg::MT, KW = Cfg::KW, WARPS = Cfg::WARPS, COMPUTE = Cfg::COMPUTE, CHUNKS = Cfg::CHUNKS, OP = Cfg::OP, QP = Cfg::QP, V4 = Cfg::V4;
+    constexpr int NV = Cfg::NV, WARPS = Cfg::WARPS, COMPUTE = Cfg::COMPUTE, CHUNKS = Cfg::CHUNKS, OP = Cfg::OP, QP = Cfg::QP, V4 = Cfg::V4;
     constexpr int KS = HD / 16, DT = HD / 8, NR = STACK ? 1 : 2;      // NR: query vectors per thread
     constexpr int CHUNK = Cfg::CHUNK;
     extern __shared__ __align__(1024) unsigned char ad_smem[];
@@ -114,17 +109,17 @@ __global__ void __launch_bounds__((AdCfg<HD, G>::THREADS)) __maxnreg__((AdCfg<HD
     __shared__ int abort_flag, s_issued;
     unsigned char* ring = ad_smem + ((1024u - (smem_u32(ad_smem) & 1023u)) & 1023u);
     float* recv = (float*)(ring + Cfg::RING);               // [CTA][VO][HD], the cluster's parts of this CTA's vectors
-    float* sm_m = recv + Cfg::Q * HD;                       // [warp][NV]
+    float* sm_m = recv + NV * HD;                       // [warp][NV]
     float* sm_l = sm_m + WARPS * NV;
     float* rc_m = sm_l + WARPS * NV;                        // [CTA][VO]
-    float* rc_l = rc_m + Cfg::Q;
-    unsigned char* Qs = (unsigned char*)(rc_l + Cfg::Q);
-    float* sm_o = Cfg::PAIR ? (float*)ring : (float*)(Qs + Cfg::QROWS * QP);       // [warp][NV][OP]
+    float* rc_l = rc_m + NV;
+    unsigned char* Qs = (unsigned char*)(rc_l + NV);
+    float* sm_o = (float*)ring;                             // [warp][NV][OP]
 
     pdl_trigger();
     asm volatile("barrier.cluster.arrive.release;" ::: "memory");          // waited for before the first remote store: every CTA runs then
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int rank = blockIdx.x, C = gridDim.x, VO = Cfg::Q / C, kvh = blockIdx.y, r0 = blockIdx.z * ANPD_ROWS;       // VO: vectors a CTA finishes
+    const int rank = blockIdx.x, C = gridDim.x, VO = NV / C, hv = blockIdx.y, kvh = hv / g.split, r0 = blockIdx.z * ANPD_ROWS;       // VO: vectors a CTA finishes
     // The row plan is older than the kernel before this one (the embedding kernel lets its successors start only after its own
     // dependency wait), so it may be read at once; so may pages below the first position this launch writes - the group's own
     // first, or the first of all rows where they are one sequence's (a prompt as short as a step of the batch).
@@ -149,7 +144,7 @@ __global__ void __launch_bounds__((AdCfg<HD, G>::THREADS)) __maxnreg__((AdCfg<HD
     if (warp == WARPS) {
         // ---------------- pages ----------------
         if (elect_one()) {
-            const uint64_t pol = policy_evict_first();
+            const uint64_t pol = g.split > 1 ? policy_evict_last() : policy_evict_first();       // read again by the clusters that share the head
             const int* pages = g.page_table + (size_t)seq * g.pages_per_seq;
             int stage = 0, count = 0;
             uint32_t phase = 1;
@@ -178,19 +173,18 @@ __global__ void __launch_bounds__((AdCfg<HD, G>::THREADS)) __maxnreg__((AdCfg<HD
         }
         __syncwarp();
     } else {
-        const int gid = lane >> 2, t = lane & 3, mt = warp % MT, ks = warp / MT;
+        const int gid = lane >> 2, t = lane & 3;
         pdl_wait();                                         // the queries come from the kernel before
         for (int idx = threadIdx.x; idx < Cfg::QROWS * (HD / 8); idx += COMPUTE) {
             const int row = idx / (HD / 8), c = idx % (HD / 8);
-            const bool lo = STACK ? row >= 8 : (row & 31) >= 16;
-            const int vec = STACK ? row & 7 : (row >> 5) * 16 + (row & 15);
-            const bf16* src = (lo ? g.q_lo : g.q_hi) + ((size_t)(r0 + vec / G) * g.Hkv * G + kvh * G + vec % G) * HD + c * 8;
+            const int vec = row & (NV - 1);
+            const bf16* src = (row >= NV ? g.q_lo : g.q_hi) + ((size_t)(r0 + vec / G) * gridDim.y * G + hv * G + vec % G) * HD + c * 8;
             *(uint4*)(Qs + row * QP + c * 16) = *(const uint4*)src;
         }
         int qpos[NR], qhl[NR], qhh[NR];
 #pragma unroll
         for (int h = 0; h < NR; ++h) {
-            const int r = (STACK ? gid : mt * 16 + gid + 8 * h) / G;
+            const int r = (gid + 8 * h) / G;
             qpos[h] = g.row_slot ? g.row_slot[r0 + r] : pos_lo + r;
             qhl[h] = g.row_slot ? g.hole_lo[r0 + r] : 0;
             qhh[h] = g.row_slot ? g.hole_hi[r0 + r] : 0;
@@ -198,31 +192,39 @@ __global__ void __launch_bounds__((AdCfg<HD, G>::THREADS)) __maxnreg__((AdCfg<HD
         ad_bar<COMPUTE>();
         // lane offsets of the ldmatrix addresses: matrix (lane / 8) of four
         const int mi = lane >> 3, lr = lane & 7;
-        const uint32_t q_addr = smem_u32(Qs) + (uint32_t)(((STACK ? 0 : mt * 32) + lr + 8 * (mi & 1)) * QP + (mi >> 1) * 16);
+        const uint32_t q_addr = smem_u32(Qs) + (uint32_t)((lr + 8 * (mi & 1)) * QP + (mi >> 1) * 16);
         const uint32_t kv_off = (uint32_t)((lr + 8 * (mi >> 1)) * 128), chunk0 = (uint32_t)(mi & 1);
         const uint32_t ring_addr = smem_u32(ring);
 
         float m_run[NR], l_run[NR], o[DT][4];
         // keys key_page .. + 15 of page p: its K chunk (given back after the last block's scores), its V chunk
-        auto block = [&](int ck, int cv, uint32_t par_v, int key_page, int p, bool last) {
-            float c[2][4];
+        auto block = [&](int ck, int cv, uint32_t par_v, int key_page, int p) {
+            // two chains of products, added at the end: even and odd steps, or hi and lo terms
+            float c[2][4], c2[2][4];
 #pragma unroll
-            for (int j = 0; j < 2; ++j) { c[j][0] = 0.f; c[j][1] = 0.f; c[j][2] = 0.f; c[j][3] = 0.f; }
+            for (int j = 0; j < 2; ++j)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) { c[j][e] = 0.f; c2[j][e] = 0.f; }
             const uint32_t kr = ring_addr + (uint32_t)ck * (uint32_t)CHUNK + kv_off + (uint32_t)key_page * 128u;
 #pragma unroll
             for (int k = 0; k < KS; ++k) {
                 uint32_t b[4], a[4];
                 ad_ldm4(kr + (uint32_t)((k >> 2) * (KV_PAGE * 128)) + ((((uint32_t)((k & 3) * 2) + chunk0) ^ (uint32_t)lr) << 4), b);
                 ad_ldm4(q_addr + (uint32_t)(k * 32), a);
-                ad_mma(c[0], a, b[0], b[1]);
-                ad_mma(c[1], a, b[2], b[3]);
+                ad_mma(STACK && (k & 1) ? c2[0] : c[0], a, b[0], b[1]);
+                ad_mma(STACK && (k & 1) ? c2[1] : c[1], a, b[2], b[3]);
                 if (!STACK) {
                     ad_ldm4(q_addr + (uint32_t)(16 * QP + k * 32), a);
-                    ad_mma(c[0], a, b[0], b[1]);
-                    ad_mma(c[1], a, b[2], b[3]);
+                    ad_mma(c2[0], a, b[0], b[1]);
+                    ad_mma(c2[1], a, b[2], b[3]);
                 }
             }
-            if (Cfg::PAIR && last) { __syncwarp(); if (lane == 0) mbar_arrive(&empty[ck]); }       // the short ring waits for it
+#pragma unroll
+            for (int j = 0; j < 2; ++j)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) c[j][e] += c2[j][e];
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&empty[ck]);         // the short ring waits for it
             uint32_t ph[4], pl[4];
             float resc[NR];
 #pragma unroll
@@ -288,15 +290,12 @@ __global__ void __launch_bounds__((AdCfg<HD, G>::THREADS)) __maxnreg__((AdCfg<HD
             const uint32_t par_v = par;
             if (++stage == CHUNKS) { stage = 0; par ^= 1u; }
             mbar_wait(&full[ck], par_k, abortp);
-            bool freed = false;
-#pragma unroll 1
-            for (int b = ks; b < AD_BLOCKS; b += KW)
-                if (p * KV_PAGE + b * AD_KEYS <= pos_hi) { freed = Cfg::PAIR && b + KW >= AD_BLOCKS; block(ck, cv, par_v, b * AD_KEYS, p, freed); }
-            mbar_wait(&full[cv], par_v, abortp);
+            if (p * KV_PAGE + warp * AD_KEYS <= pos_hi) block(ck, cv, par_v, warp * AD_KEYS, p);
+            else { if (lane == 0) mbar_arrive(&empty[ck]); mbar_wait(&full[cv], par_v, abortp); }
             __syncwarp();
-            if (lane == 0) { if (!freed) mbar_arrive(&empty[ck]); mbar_arrive(&empty[cv]); }
+            if (lane == 0) mbar_arrive(&empty[cv]);
         }
-        if (Cfg::PAIR) ad_bar<COMPUTE>();                // the slots' results go where the pages were
+        ad_bar<COMPUTE>();                               // the slots' results go where the pages were
         // ---- the key slots, in slot order ----
 #pragma unroll
         for (int h = 0; h < NR; ++h) {
@@ -316,7 +315,7 @@ __global__ void __launch_bounds__((AdCfg<HD, G>::THREADS)) __maxnreg__((AdCfg<HD
         ad_bar<COMPUTE>();
         // the result, as hi + lo terms in the O projection's operand image
         auto store = [&](int vec, int d4, float l, float4 a) {
-            const int row = r0 + vec / G, k = (kvh * G + vec % G) * HD + 4 * d4;
+            const int row = r0 + vec / G, k = (hv * G + vec % G) * HD + 4 * d4;
             uint2 hi, lo;
             hi.x = ad_split(a.x / l, a.y / l, lo.x);
             hi.y = ad_split(a.z / l, a.w / l, lo.y);
@@ -324,20 +323,19 @@ __global__ void __launch_bounds__((AdCfg<HD, G>::THREADS)) __maxnreg__((AdCfg<HD
             *(uint2*)(g.img + cl_img_offset(g.rows, g.rows + row, k)) = lo;
         };
         asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
-        for (int idx = threadIdx.x; idx < Cfg::Q * V4; idx += COMPUTE) {
-            const int vec = idx / V4, d4 = idx % V4, tile = vec / NV, vi = vec % NV;
+        for (int idx = threadIdx.x; idx < NV * V4; idx += COMPUTE) {
+            const int vec = idx / V4, d4 = idx % V4;
             float mx = -CUDART_INF_F;
 #pragma unroll
-            for (int k = 0; k < KW; ++k) mx = fmaxf(mx, sm_m[(k * MT + tile) * NV + vi]);
+            for (int w = 0; w < WARPS; ++w) mx = fmaxf(mx, sm_m[w * NV + vec]);
             float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
             float l = 0.0f;
 #pragma unroll
-            for (int k = 0; k < KW; ++k) {
-                const int w = k * MT + tile;
-                const float m = sm_m[w * NV + vi], s = m == -CUDART_INF_F ? 0.0f : exp2f(m - mx);
-                const float4 x = *(const float4*)(sm_o + (size_t)(w * NV + vi) * OP + 4 * d4);
+            for (int w = 0; w < WARPS; ++w) {
+                const float m = sm_m[w * NV + vec], s = m == -CUDART_INF_F ? 0.0f : exp2f(m - mx);
+                const float4 x = *(const float4*)(sm_o + (size_t)(w * NV + vec) * OP + 4 * d4);
                 a.x = fmaf(x.x, s, a.x); a.y = fmaf(x.y, s, a.y); a.z = fmaf(x.z, s, a.z); a.w = fmaf(x.w, s, a.w);
-                l = fmaf(sm_l[w * NV + vi], s, l);
+                l = fmaf(sm_l[w * NV + vec], s, l);
             }
             if (C == 1) { store(vec, d4, l, a); continue; }
             const int owner = vec / VO, at = rank * VO + vec % VO;
@@ -379,14 +377,16 @@ anpd_status launch_attn_dec(anpd_model* m, anpd_kv* kv, AdArgs& a) {
     typedef AdCfg<HD, G> Cfg;
     static bool attr_set[64] = {false};
     if (first_call_on_device(attr_set)) CUDA_TRY(cudaFuncSetAttribute(attn_dec_kernel<HD, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM));
-    // As many CTAs per head as are resident at once (about 7/8 of the SMs can hold clusters).  1.1B, eight sequences of 300 tokens:
-    // 1666 -> 1389 us per step with four CTAs per head, where one took all pages of a head before.  Eight 13B sequences have one: as
-    // fast as page partials and their merge (2147 -> 2135), four 7B sequences two (1015 -> 997).
-    const int heads = a.Hkv * kv->batch, resident = m->num_sms * 7 / 8 * (Cfg::PAIR ? 2 : 1);
+    // As many CTAs per head as find an SM each (about 7/8 of the SMs can hold clusters).  Two to an SM leave no room for the next
+    // projection's CTAs, whose first weights then come late: one 13B sequence of 1000 tokens (8 layers and the head) 1098 us per
+    // step with four CTAs per head, 1072 with two; at 4000 tokens 1255 and 1223; eight 1.1B sequences 1337 and 1230 (two, one); four
+    // 7B sequences of 600 tokens (8 layers) 915 and 880, of 2000 tokens 1088 and 1040.  Never more than four: sixteen clusters of
+    // eight crowd the O projection out (1.1B at 512 keys: 894, with four 800).
+    const int heads = a.Hkv * a.split * kv->batch, resident = m->num_sms * 7 / 8;
     int cluster = Cfg::C_MAX;
     while (cluster > 1 && heads * cluster > resident) cluster /= 2;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(cluster, a.Hkv, kv->batch); cfg.blockDim = dim3(Cfg::THREADS); cfg.dynamicSmemBytes = Cfg::SMEM; cfg.stream = m->stream;
+    cfg.gridDim = dim3(cluster, a.Hkv * a.split, kv->batch); cfg.blockDim = dim3(Cfg::THREADS); cfg.dynamicSmemBytes = Cfg::SMEM; cfg.stream = m->stream;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = cluster; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
@@ -417,11 +417,11 @@ anpd_status attn_dec_enqueue(anpd_model* m, anpd_kv* kv, int layer, bool tree) {
     a.layer_page0 = layer * kv->total_pages;
     a.img = ws.ci_ao; a.err = ws.gemm_err;
     switch (c.head_dim * 16 + c.n_q_heads / c.n_kv_heads) {
-        case 64 * 16 + 1: return launch_attn_dec<64, 1>(m, kv, a);
-        case 64 * 16 + 2: return launch_attn_dec<64, 2>(m, kv, a);
-        case 64 * 16 + 4: return launch_attn_dec<64, 4>(m, kv, a);
-        case 64 * 16 + 8: return launch_attn_dec<64, 8>(m, kv, a);
-        case 128 * 16 + 1: return launch_attn_dec<128, 1>(m, kv, a);
+        case 64 * 16 + 1: a.split = 1; return launch_attn_dec<64, 1>(m, kv, a);
+        case 64 * 16 + 2: a.split = 1; return launch_attn_dec<64, 2>(m, kv, a);
+        case 64 * 16 + 4: a.split = 2; return launch_attn_dec<64, 2>(m, kv, a);
+        case 64 * 16 + 8: a.split = 4; return launch_attn_dec<64, 2>(m, kv, a);
+        case 128 * 16 + 1: a.split = 1; return launch_attn_dec<128, 1>(m, kv, a);
     }
     return ANPD_ERR_ARG;
 }
