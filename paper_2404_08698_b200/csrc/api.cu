@@ -404,7 +404,7 @@ anpd_status anpd_kv_create(const anpd_model* cm, int max_len, int batch, int shu
     kv->h_kv_len.assign(batch, 0);
     kv->h_len_stale.assign(batch, 0);
     Workspace& ws = kv->ws;
-    ws.prefill_rows = std::min(PREFILL_ROWS_MAX, (kv->max_len + 255) / 256 * 256);
+    ws.prefill_rows = (int)std::min<long long>(PREFILL_ROWS_MAX, ((long long)kv->max_len * batch + 255) / 256 * 256);      // several sequences' prompts in one pass
     ws.pf_rows = 0;
     ws.r_max = std::max(ws.prefill_rows, batch * ANPD_ROWS);
     ws.n_max_out = (std::max(std::max(m->nqkv, 2 * c.d_ffn), std::max(c.d_model, c.vocab)) + 127) / 128 * 128;
@@ -418,7 +418,7 @@ anpd_status anpd_kv_create(const anpd_model* cm, int max_len, int batch, int shu
         {(void**)&kv->kpool, pool}, {(void**)&kv->vpool, pool},
         {(void**)&kv->page_table, (size_t)kv->total_pages * 4},
         {(void**)&kv->rope_cos, (size_t)kv->max_len * half * 4}, {(void**)&kv->rope_sin, (size_t)kv->max_len * half * 4},
-        {(void**)&kv->seq, sizeof(SeqState) * (size_t)batch}, {(void**)&kv->d_prompt, (size_t)kv->max_len * 4},
+        {(void**)&kv->seq, sizeof(SeqState) * (size_t)batch}, {(void**)&kv->d_prompt, (size_t)kv->max_len * batch * 4},
         {(void**)&kv->d_ctxs, sizeof(NgramDev) * (size_t)batch},
         {(void**)&ws.row_tok, R * 4}, {(void**)&ws.row_pos, R * 4}, {(void**)&ws.row_seq, R * 4}, {(void**)&ws.row_ok, R * 4},
         {(void**)&ws.row_slot, R * 4}, {(void**)&ws.row_hole_lo, R * 4}, {(void**)&ws.row_hole_hi, R * 4},
@@ -601,6 +601,32 @@ static anpd_status prefill_enqueue(anpd_model* m, anpd_kv* kv, int seq, const in
         ANPD_TRY(forward_enqueue(m, kv, rows, std::min(start + rows - 1, kv->max_len - 1), last, false, last_row));
         // the LM head of a prompt pass runs on the last token's group of 8 rows, moved to rows 0-7
         if (last) ANPD_TRY(accept_enqueue(m, kv, ACCEPT_PREFILL, d_ctxs, seq, rows == kv->batch * ANPD_ROWS ? last_row : last_row % ANPD_ROWS, prompt_len));
+    }
+    return ANPD_OK;
+}
+
+// The prompts of all sequences.  As many as fit share a pass: the weights cross HBM once for them, and row tiles and SMs fill up.
+// Eight sequences, a pass each before: 1.1B, 300 tokens 18.3 -> 11.2 ms; 7B (8 layers) 17.6 -> 13.4; 13B (10 layers), 512 tokens
+// 43.8 -> 41.0.
+static anpd_status prefill_all_enqueue(anpd_model* m, anpd_kv* kv, const int32_t* prompts, int prompt_len, const NgramDev* d_ctxs) {
+    const int B = kv->batch, seg0 = (prompt_len + ANPD_ROWS - 1) / ANPD_ROWS * ANPD_ROWS;
+    // (the cross-check variants of the kernels take one sequence at a time)
+    const int fit = m->plain_gemm || !kv->attn_pf || kv->step_ready ? 1 : kv->ws.prefill_rows / seg0;
+    for (int b = 0; b < B;) {
+        const int n = std::min(fit, B - b);
+        // a pass of exactly batch * 8 rows would be taken for a step
+        const int seg = n * seg0 == B * ANPD_ROWS ? seg0 + ANPD_ROWS : seg0, rows = n * seg;
+        const int32_t* prompt = prompts + (size_t)b * prompt_len;
+        if (n < 2 || rows > kv->ws.prefill_rows) {
+            ANPD_TRY(prefill_enqueue(m, kv, b, prompt, prompt_len, d_ctxs));
+            ++b;
+            continue;
+        }
+        CUDA_TRY(cudaMemcpyAsync(kv->d_prompt, prompt, sizeof(int) * (size_t)n * prompt_len, cudaMemcpyDefault, m->stream));
+        ANPD_TRY(plan_prefill_enqueue(m, kv, b, 0, prompt_len, std::min((rows + 63) / 64 * 64, kv->ws.r_max), n, seg));
+        ANPD_TRY(forward_enqueue(m, kv, rows, std::min(seg, kv->max_len) - 1, true, false, prompt_len - 1, false, n));
+        ANPD_TRY(accept_enqueue(m, kv, ACCEPT_PREFILL, d_ctxs, b, (prompt_len - 1) % ANPD_ROWS, prompt_len, false, n));
+        b += n;
     }
     return ANPD_OK;
 }
@@ -944,7 +970,7 @@ static anpd_status generate_core(anpd_model* m, anpd_kv* kv, anpd_ngram* const* 
             for (int b = 0; b < B; ++b) ANPD_TRY(ngram_enqueue_bulk(ctxs[b], 0, prompt_len, &m->prof));
         }
         // LLM(prompt): the first token lands in the context as its first uncounted token
-        for (int b = 0; b < B; ++b) ANPD_TRY(prefill_enqueue(m, kv, b, prompts + (size_t)b * prompt_len, prompt_len, kv->d_ctxs));
+        ANPD_TRY(prefill_all_enqueue(m, kv, prompts, prompt_len, kv->d_ctxs));
         if (K > 0 && kv->side_stream) CUDA_TRY(cudaStreamWaitEvent(st, kv->ev_join, 0));
         CUDA_TRY(cudaEventRecord(e1, st));
         ANPD_TRY(read_seqs(kv));

@@ -57,7 +57,8 @@ template <int V> using FaInt = std::integral_constant<int, V>;
 struct FaArgs {
     const int* page_table; int pages_per_seq;
     const int* row_pos; const int* row_seq;
-    int H, Hkv, layer_page0, rows, n_row_tiles;     // query heads, kv heads (H a multiple of Hkv)
+    int H, Hkv, layer_page0, n_row_tiles;           // query heads, kv heads (H a multiple of Hkv)
+    int rows, n_seq, seg;                           // n_seq sequences of seg rows each
     bf16* ao_hi; bf16* ao_lo;
     unsigned char* img;                     // the O projection's operand image (few rows) instead of ao_hi and ao_lo
     int* err;
@@ -113,12 +114,12 @@ attn_pf_kernel(const __grid_constant__ CUtensorMap map_qh, const __grid_constant
         const int G = (int)gridDim.x;
         return k * G + ((k & 1) ? G - 1 - (int)blockIdx.x : (int)blockIdx.x);
     };
-    auto item = [&](int it, int& r0, int& h, int& n_pages, int& seq, int& pos_lo) {
-        const int rt = g.n_row_tiles - 1 - it / g.H;
+    auto item = [&](int it, int& r0, int& r_end, int& h, int& n_pages, int& seq) {
+        const int t = it / g.H, rt = (g.n_row_tiles - 1 - t) / g.n_seq, s0 = t % g.n_seq * g.seg;      // a tile's rows are one sequence's
         h = it % g.H;
-        r0 = rt * FA_ROWS;
-        const int last = min(r0 + FA_ROWS, g.rows) - 1;
-        pos_lo = g.row_pos[r0];
+        r0 = s0 + rt * FA_ROWS;
+        r_end = s0 + g.seg;
+        const int last = min(r0 + FA_ROWS, r_end) - 1;
         n_pages = g.row_pos[last] / KV_PAGE + 1;
         seq = g.row_seq[r0];
     };
@@ -130,8 +131,8 @@ attn_pf_kernel(const __grid_constant__ CUtensorMap map_qh, const __grid_constant
             uint32_t tq = 0, li = 0;                                // tiles begun, page loads issued so far
             bool ok = true;
             for (int k = 0, it = nth(0); it < n_items && ok; ++k, it = nth(k), ++tq) {
-                int r0, h, n_pages, seq, pos_lo;
-                item(it, r0, h, n_pages, seq, pos_lo);
+                int r0, r_end, h, n_pages, seq;
+                item(it, r0, r_end, h, n_pages, seq);
                 ok = mbar_wait(&q_empty, (tq & 1u) ^ 1u, abortp);
                 if (!ok) break;
                 mbar_expect_tx(&q_full, 2 * PAGE);
@@ -197,8 +198,8 @@ attn_pf_kernel(const __grid_constant__ CUtensorMap map_qh, const __grid_constant
                 }
             };
             for (int k = 0, it = nth(0); it < n_items && ok; ++k, it = nth(k), ++tq) {
-                int r0, h, n_pages, seq, pos_lo;
-                item(it, r0, h, n_pages, seq, pos_lo);
+                int r0, r_end, h, n_pages, seq;
+                item(it, r0, r_end, h, n_pages, seq);
                 ok = mbar_wait(&q_full, tq & 1u, abortp);
                 if (!ok) break;
                 auto scores = [&]() -> bool {                       // S of the next page in line
@@ -242,10 +243,10 @@ attn_pf_kernel(const __grid_constant__ CUtensorMap map_qh, const __grid_constant
         uint32_t pc = 0, od = 0;                          // pages begun, completions of the O product consumed
         bool ok = true;
         for (int k = 0, it = nth(0); it < n_items && ok; ++k, it = nth(k)) {
-            int r0, h, n_pages, seq, pos_lo;
-            item(it, r0, h, n_pages, seq, pos_lo);
+            int r0, r_end, h, n_pages, seq;
+            item(it, r0, r_end, h, n_pages, seq);
             const int row = r0 + r;
-            const int pos = row < g.rows ? g.row_pos[row] : -1;         // -1: a padding row sees no key
+            const int pos = row < r_end ? g.row_pos[row] : -1;         // -1: a padding row sees no key
             float m_run = -CUDART_INF_F, l_run = 0.0f;
             for (int c = 0; c < n_pages && ok; ++c, ++pc) {
                 const uint32_t b = pc & 1u;
@@ -339,7 +340,7 @@ attn_pf_kernel(const __grid_constant__ CUtensorMap map_qh, const __grid_constant
             for (int ch = 0; ch < HD / 64; ++ch) {
                 float o[32];
                 tc_ld32(tm_o + lane_addr + (uint32_t)(half * (HD / 2) + ch * 32), o);
-                if (row < g.rows) {
+                if (row < r_end) {
                     __nv_bfloat162 hh[16], ll[16];
 #pragma unroll
                     for (int i = 0; i < 32; i += 2) {
@@ -375,7 +376,7 @@ attn_pf_kernel(const __grid_constant__ CUtensorMap map_qh, const __grid_constant
 
 }  // namespace
 
-// Attention of a prompt pass over `rows` rows (a multiple of 8; the row plan covers the padding) of sequence row_seq[0].
+// Attention of a prompt pass over `rows` rows: n_seq sequences of rows / n_seq rows each (a multiple of 8; the row plan covers the padding).
 // map_q: the pass's queries [rows][H * hd] seen through boxes of 64 columns x 128 rows.
 template <int HD>
 static anpd_status launch_attn_pf(anpd_model* m, anpd_kv* kv, const FaArgs& g) {
@@ -388,7 +389,7 @@ static anpd_status launch_attn_pf(anpd_model* m, anpd_kv* kv, const FaArgs& g) {
     return ANPD_OK;
 }
 
-anpd_status attn_pf_enqueue(anpd_model* m, anpd_kv* kv, int layer, int rows, unsigned char* img) {
+anpd_status attn_pf_enqueue(anpd_model* m, anpd_kv* kv, int layer, int rows, unsigned char* img, int n_seq) {
     const anpd_model_config& c = m->cfg;
     Workspace& ws = kv->ws;
     FaArgs g;
@@ -396,8 +397,8 @@ anpd_status attn_pf_enqueue(anpd_model* m, anpd_kv* kv, int layer, int rows, uns
     g.row_pos = ws.row_pos; g.row_seq = ws.row_seq;
     g.H = c.n_q_heads; g.Hkv = c.n_kv_heads;
     g.layer_page0 = layer * kv->total_pages;
-    g.rows = rows;
-    g.n_row_tiles = (rows + FA_ROWS - 1) / FA_ROWS;
+    g.rows = rows; g.n_seq = n_seq; g.seg = rows / n_seq;
+    g.n_row_tiles = n_seq * ((g.seg + FA_ROWS - 1) / FA_ROWS);
     g.ao_hi = ws.ao_hi; g.ao_lo = ws.ao_lo; g.img = img;
     g.err = ws.gemm_err;
     return c.head_dim == 64 ? launch_attn_pf<64>(m, kv, g) : launch_attn_pf<128>(m, kv, g);

@@ -52,19 +52,20 @@ __global__ void plan_decode_kernel(SeqState* seqs, int* row_tok, int* row_pos, i
     row_hole_hi[i] = (r > ka && real) ? s.kv_len + ka + 1 : 0;
 }
 
-__global__ void plan_prefill_kernel(const int* prompt, int seq, int start, int prompt_len, int rows,
+// Rows of a prompt pass: n_seq sequences from `seq` on, `seg` rows each, positions from `start` on; prompts one behind the other.
+__global__ void plan_prefill_kernel(const int* prompt, int seq, int start, int prompt_len, int rows, int n_seq, int seg,
                                     int* row_tok, int* row_pos, int* row_seq, int* row_ok, int* row_slot, int* row_hole_lo,
                                     int* row_hole_hi, int vocab, int max_len, SeqState* seqs) {
     pdl_trigger();
     pdl_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= rows) return;
-    const int p = start + i;
-    int tok = (p < prompt_len) ? prompt[p] : 0;
-    if (tok < 0 || tok >= vocab) { atomicExch(&seqs[seq].error, ERR_TOKEN_RANGE); tok = 0; }
+    const int s = min(i / seg, n_seq - 1), p = start + i - s * seg;
+    int tok = (p < prompt_len) ? prompt[s * prompt_len + p] : 0;
+    if (tok < 0 || tok >= vocab) { atomicExch(&seqs[seq + s].error, ERR_TOKEN_RANGE); tok = 0; }
     row_tok[i] = tok;
     row_pos[i] = min(p, max_len - 1);
-    row_seq[i] = seq;
+    row_seq[i] = seq + s;
     row_ok[i] = (p < max_len && p < prompt_len) ? 1 : 0;
     row_slot[i] = min(p, max_len - 1);
     row_hole_lo[i] = 0;
@@ -337,14 +338,14 @@ __global__ void __launch_bounds__(128) qkv_rope_append_kernel(const float* __res
     }
 }
 
-// The same for a prompt pass (rows are consecutive positions of one sequence, a multiple of 8, the first a multiple of the page):
+// The same for a prompt pass (every `seg` rows are consecutive positions of one sequence, a multiple of 8, the first a multiple of the page):
 // a block takes 32 rows of the heads blockIdx.x, blockIdx.x + gridDim.x, ... and keeps their cosines and sines; a V head goes
 // through shared memory, so that the transposed page receives whole 16-byte runs of positions instead of single elements.  Per
 // element the arithmetic is that of qkv_rope_append_kernel, in the same order.  7B: 80 rows 14 -> 6 us, 1536 rows 41 -> 36.
 constexpr int ROPE_TILE_ROWS = 32;
 template <int HD>
 __global__ void __launch_bounds__(256, 3) qkv_rope_append_tile_kernel(const float* __restrict__ part, const int* __restrict__ seg_count, size_t split_stride,
-                                                                   int ld_part, int rows, const int* __restrict__ row_pos, const int* __restrict__ row_seq,
+                                                                   int ld_part, int seg, const int* __restrict__ row_pos, const int* __restrict__ row_seq,
                                                                    const int* __restrict__ row_ok, const float* __restrict__ rope_cos,
                                                                    const float* __restrict__ rope_sin, const int* __restrict__ page_table,
                                                                    int pages_per_seq, int Hq, int Hkv, float q_scale, bf16* __restrict__ q_hi,
@@ -352,8 +353,9 @@ __global__ void __launch_bounds__(256, 3) qkv_rope_append_tile_kernel(const floa
     pdl_trigger();
     __shared__ float tile[ROPE_TILE_ROWS][HD + 1];
     constexpr int half = HD / 2, TPR = HD / 8, PER = ROPE_TILE_ROWS * TPR / 256;
-    const int r0 = blockIdx.y * ROPE_TILE_ROWS, i = threadIdx.x % TPR * 4;
-    const int nr = min(ROPE_TILE_ROWS, rows - r0);
+    const int tiles = (seg + ROPE_TILE_ROWS - 1) / ROPE_TILE_ROWS, tile0 = blockIdx.y % tiles * ROPE_TILE_ROWS;
+    const int r0 = blockIdx.y / tiles * seg + tile0, i = threadIdx.x % TPR * 4;
+    const int nr = min(ROPE_TILE_ROWS, seg - tile0);
     const int pos0 = row_pos[r0];                        // the tile's rows hold positions pos0, pos0 + 1, ... inside one page
     const int page = page_table[row_seq[r0] * pages_per_seq + pos0 / KV_PAGE];
     float4 c[PER], sn[PER];
@@ -372,12 +374,12 @@ __global__ void __launch_bounds__(256, 3) qkv_rope_append_tile_kernel(const floa
     for (int head = blockIdx.x; head < Hq + 2 * Hkv; head += gridDim.x) {
         const bool is_q = head < Hq, is_k = !is_q && head < Hq + Hkv;
         bf16* pg = (is_k ? kpool_l : vpool_l) + ((size_t)page * Hkv + (is_q ? 0 : is_k ? head - Hq : head - Hq - Hkv)) * KV_PAGE * HD;
-        const int* seg = seg_count ? seg_count + ((head * HD) >> 7) : nullptr;
+        const int* count = seg_count ? seg_count + ((head * HD) >> 7) : nullptr;
 #pragma unroll
         for (int u = 0; u < PER; ++u) {
             const int r = u * (256 / TPR) + threadIdx.x / TPR;
             if (r >= nr) continue;
-            RopeSum v = rope_sum<4>(part + (size_t)(r0 + r) * ld_part + (size_t)head * HD + i, half, split_stride, seg, ns_min);
+            RopeSum v = rope_sum<4>(part + (size_t)(r0 + r) * ld_part + (size_t)head * HD + i, half, split_stride, count, ns_min);
             if (is_q || is_k) rope_rotate(v, c[u], sn[u]);
             if (is_q) {
                 const size_t o = (size_t)(r0 + r) * Hq * HD + (size_t)head * HD + i;
@@ -869,13 +871,14 @@ __global__ void __launch_bounds__(256) argmax_partial_kernel(const float* __rest
 __global__ void __launch_bounds__(256) accept_kernel(SeqState* seqs, const float* __restrict__ amax_val,
                                                      const int* __restrict__ amax_idx, int nblk, int mode,
                                                      const NgramDev* ctxs, int seq_arg, int last_row, int prompt_len, int two) {
+    // a prompt pass: block b takes sequence seq_arg + b, whose last token's row is last_row + 8 b
     pdl_trigger();
     pdl_wait();
     __shared__ int pred[ANPD_ROWS];
-    const int b = (mode == ACCEPT_PREFILL) ? seq_arg : blockIdx.x;
+    const int b = (mode == ACCEPT_PREFILL ? seq_arg : 0) + blockIdx.x;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     {
-        const int row = (mode == ACCEPT_PREFILL) ? (last_row / ANPD_ROWS) * ANPD_ROWS + warp : b * ANPD_ROWS + warp;
+        const int row = (mode == ACCEPT_PREFILL) ? (last_row / ANPD_ROWS + blockIdx.x) * ANPD_ROWS + warp : b * ANPD_ROWS + warp;
         float best = -CUDART_INF_F;
         int bidx = 0x7fffffff;
         for (int i = lane; i < nblk; i += 32) {
@@ -1024,15 +1027,16 @@ __global__ void fill_tail_segs_kernel(int* segs, int m_tiles, int first_cut, int
     if (i < m_tiles) segs[i] = i >= first_cut ? parts : 1;
 }
 
-// rows [from, from + 8) of the normalised activations -> rows 0-7 of a decode step's operand image
-__global__ void rows_to_image_kernel(const bf16* __restrict__ h_hi, const bf16* __restrict__ h_lo, int from, int d, unsigned char* __restrict__ img,
+// groups of 8 rows, `step` rows apart, from row `from` of the normalised activations on -> rows 0, 1, ... of a decode step's operand image
+__global__ void rows_to_image_kernel(const bf16* __restrict__ h_hi, const bf16* __restrict__ h_lo, int from, int step, int d, unsigned char* __restrict__ img,
                                      int img_rows) {
     pdl_trigger();
     pdl_wait();
     const int r = blockIdx.x;
+    const size_t src = (size_t)(from + r / ANPD_ROWS * step + r % ANPD_ROWS) * d;
     for (int i = threadIdx.x; i < d / 8; i += blockDim.x) {
-        *(uint4*)(img + cl_img_offset(img_rows, r, 8 * i)) = ((const uint4*)(h_hi + (size_t)(from + r) * d))[i];
-        *(uint4*)(img + cl_img_offset(img_rows, img_rows + r, 8 * i)) = ((const uint4*)(h_lo + (size_t)(from + r) * d))[i];
+        *(uint4*)(img + cl_img_offset(img_rows, r, 8 * i)) = ((const uint4*)(h_hi + src))[i];
+        *(uint4*)(img + cl_img_offset(img_rows, img_rows + r, 8 * i)) = ((const uint4*)(h_lo + src))[i];
     }
 }
 
@@ -1109,7 +1113,7 @@ anpd_status gemm_enqueue(anpd_model* m, anpd_kv* kv, int kind, int layer, int ro
 }
 
 template <int HD>
-anpd_status attn_enqueue(anpd_model* m, anpd_kv* kv, int layer, int rows, int max_pos, unsigned char* img = nullptr, bool tree = false, int img_rows = 0) {
+anpd_status attn_enqueue(anpd_model* m, anpd_kv* kv, int layer, int rows, int max_pos, unsigned char* img = nullptr, bool tree = false, int img_rows = 0, int n_seq = 1) {
     const anpd_model_config& c = m->cfg;
     Workspace& ws = kv->ws;
     const size_t layer_elems = (size_t)kv->total_pages * c.n_kv_heads * KV_PAGE * HD;
@@ -1121,10 +1125,10 @@ anpd_status attn_enqueue(anpd_model* m, anpd_kv* kv, int layer, int rows, int ma
         CUDA_TRY(cudaFuncSetAttribute(attn_partial_kernel<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     }
     // a prompt pass: pages are folded in the kernel, nothing to merge (the older 16-row kernel knows one query head per kv head only)
-    if (rows != kv->batch * ANPD_ROWS && kv->attn_pf) return attn_pf_enqueue(m, kv, layer, rows, img);
+    if (rows != kv->batch * ANPD_ROWS && kv->attn_pf) return attn_pf_enqueue(m, kv, layer, rows, img, n_seq);
     if (HD == 128 && kv->attn_tc && rows != kv->batch * ANPD_ROWS && c.n_q_heads == c.n_kv_heads) {
         ANPD_TRY(attn_prompt_enqueue(m, kv, layer, rows));
-        if (img) LAUNCH(&m->prof, m->stream, KC_ATTN, 0, (launch_k(rows_to_image_kernel, rows, 256, 0, m->stream, ws.ao_hi, ws.ao_lo, 0, m->dq, img, rows)));
+        if (img) LAUNCH(&m->prof, m->stream, KC_ATTN, 0, (launch_k(rows_to_image_kernel, rows, 256, 0, m->stream, ws.ao_hi, ws.ao_lo, 0, ANPD_ROWS, m->dq, img, rows)));
         return ANPD_OK;
     }
     if (HD == 128 && kv->attn_tc) {
@@ -1166,19 +1170,19 @@ anpd_status plan_decode_enqueue(anpd_model* m, anpd_kv* kv, bool two_candidates)
     return ANPD_OK;
 }
 
-anpd_status plan_prefill_enqueue(anpd_model* m, anpd_kv* kv, int seq, int start, int prompt_len, int rows) {
+anpd_status plan_prefill_enqueue(anpd_model* m, anpd_kv* kv, int seq, int start, int prompt_len, int rows, int n_seq, int seg) {
     Workspace& ws = kv->ws;
     LAUNCH(&m->prof, m->stream, KC_OTHER, 0,
-           (launch_k(plan_prefill_kernel, (rows + 127) / 128, 128, 0, m->stream, kv->d_prompt, seq, start, prompt_len, rows, ws.row_tok,
+           (launch_k(plan_prefill_kernel, (rows + 127) / 128, 128, 0, m->stream, kv->d_prompt, seq, start, prompt_len, rows, n_seq, seg, ws.row_tok,
                                                                           ws.row_pos, ws.row_seq, ws.row_ok, ws.row_slot, ws.row_hole_lo,
                                                                           ws.row_hole_hi, m->cfg.vocab, kv->max_len, kv->seq)));
     CUDA_TRY(cudaGetLastError());
     return ANPD_OK;
 }
 
-anpd_status accept_enqueue(anpd_model* m, anpd_kv* kv, int mode, const NgramDev* d_ctxs, int seq, int last_row, int prompt_len, bool two_candidates) {
+anpd_status accept_enqueue(anpd_model* m, anpd_kv* kv, int mode, const NgramDev* d_ctxs, int seq, int last_row, int prompt_len, bool two_candidates, int n_seq) {
     Workspace& ws = kv->ws;
-    const int blocks = (mode == ACCEPT_PREFILL) ? 1 : kv->batch;
+    const int blocks = (mode == ACCEPT_PREFILL) ? n_seq : kv->batch;
     LAUNCH(&m->prof, m->stream, KC_OTHER, 0,
            (launch_k(accept_kernel, blocks, 256, 0, m->stream, kv->seq, ws.amax_val_use, ws.amax_idx_use,
                      ws.amax_nblk, mode, d_ctxs, seq, last_row, prompt_len, two_candidates ? 1 : 0)));
@@ -1309,7 +1313,7 @@ static anpd_status forward_cl_enqueue(anpd_model* m, anpd_kv* kv, int max_pos, b
     return ANPD_OK;
 }
 
-anpd_status forward_enqueue(anpd_model* m, anpd_kv* kv, int rows, int max_pos, bool head, bool want_logits, int head_row, bool two_candidates) {
+anpd_status forward_enqueue(anpd_model* m, anpd_kv* kv, int rows, int max_pos, bool head, bool want_logits, int head_row, bool two_candidates, int n_seq) {
     // the two fused variants know nothing of a second candidate's cache slots and mask
     if (m->rr_ready && kv->batch == 1 && rows == ANPD_ROWS && head && !m->plain_gemm && !two_candidates) return forward_rr_enqueue(m, kv, max_pos, want_logits);
     if (kv->step_ready && rows == kv->batch * ANPD_ROWS && head && !m->prof.on && !two_candidates) return step_kernel_enqueue(m, kv, max_pos, want_logits);
@@ -1337,15 +1341,15 @@ anpd_status forward_enqueue(anpd_model* m, anpd_kv* kv, int rows, int max_pos, b
         ANPD_TRY(gemm_enqueue(m, kv, GK_QKV, l, rows, &segs, &seg_min));
         if (rows != kv->batch * ANPD_ROWS) {            // a prompt pass
             // as many heads at once as keep every SM's 2048 threads busy, the others by the same blocks
-            const int tiles = (rows + ROPE_TILE_ROWS - 1) / ROPE_TILE_ROWS;
+            const int seg = rows / n_seq, tiles = n_seq * ((seg + ROPE_TILE_ROWS - 1) / ROPE_TILE_ROWS);
             const dim3 grid(std::min(c.n_q_heads + 2 * c.n_kv_heads, std::max(1, m->num_sms * 8 / tiles)), tiles);
             const float qs = 1.4426950408889634f / sqrtf((float)hd);
             if (hd == 128) LAUNCH(pf, st, KC_OTHER, 0,
-                   (launch_k(qkv_rope_append_tile_kernel<128>, grid, 256, 0, st, ws.part, segs, sstride, ws.n_max_out, rows, ws.row_pos, ws.row_seq, ws.row_ok,
+                   (launch_k(qkv_rope_append_tile_kernel<128>, grid, 256, 0, st, ws.part, segs, sstride, ws.n_max_out, seg, ws.row_pos, ws.row_seq, ws.row_ok,
                              kv->rope_cos, kv->rope_sin, kv->page_table, kv->pages_per_seq, c.n_q_heads, c.n_kv_heads, qs, ws.q_hi, ws.q_lo,
                              kv->kpool + l * layer_elems, kv->vpool + l * layer_elems, seg_min)));
             else LAUNCH(pf, st, KC_OTHER, 0,
-                   (launch_k(qkv_rope_append_tile_kernel<64>, grid, 256, 0, st, ws.part, segs, sstride, ws.n_max_out, rows, ws.row_pos, ws.row_seq, ws.row_ok,
+                   (launch_k(qkv_rope_append_tile_kernel<64>, grid, 256, 0, st, ws.part, segs, sstride, ws.n_max_out, seg, ws.row_pos, ws.row_seq, ws.row_ok,
                              kv->rope_cos, kv->rope_sin, kv->page_table, kv->pages_per_seq, c.n_q_heads, c.n_kv_heads, qs, ws.q_hi, ws.q_lo,
                              kv->kpool + l * layer_elems, kv->vpool + l * layer_elems, seg_min)));
         } else
@@ -1357,8 +1361,8 @@ anpd_status forward_enqueue(anpd_model* m, anpd_kv* kv, int rows, int max_pos, b
         unsigned char* ao_img = slab ? ws.ci_ao : nullptr;
         const int ao_rows = slab ? rows : 0;
         if (decode && attn_dec_supported(m) && (hd == 64 || kv->attn_tc)) ANPD_TRY(attn_dec_enqueue(m, kv, l, two_candidates));
-        else if (hd == 128) ANPD_TRY(attn_enqueue<128>(m, kv, l, rows, max_pos, ao_img, two_candidates, ao_rows));
-        else ANPD_TRY(attn_enqueue<64>(m, kv, l, rows, max_pos, ao_img, two_candidates, ao_rows));
+        else if (hd == 128) ANPD_TRY(attn_enqueue<128>(m, kv, l, rows, max_pos, ao_img, two_candidates, ao_rows, n_seq));
+        else ANPD_TRY(attn_enqueue<64>(m, kv, l, rows, max_pos, ao_img, two_candidates, ao_rows, n_seq));
         ANPD_TRY(gemm_enqueue(m, kv, GK_O, l, rows, &segs, &seg_min));
         LAUNCH(pf, st, KC_OTHER, 0,
                (launch_k(resid_norm, rows, NORM_THREADS, 0, st, ws.x, ws.part, segs, sstride, ws.n_max_out, w.ffn_norm, c.rms_eps, d,
@@ -1377,15 +1381,16 @@ anpd_status forward_enqueue(anpd_model* m, anpd_kv* kv, int rows, int max_pos, b
                                                        ws.h_hi, ws.h_lo, seg_min, decode || (slab && l + 1 < c.n_layers) ? ws.ci_h : nullptr)));
     }
     if (!head) { CUDA_TRY(cudaGetLastError()); return ANPD_OK; }
-    // A prompt pass needs the LM head for its last token only: the group of 8 rows that holds it becomes rows 0-7 of a decode
+    // A prompt pass needs the LM head for each sequence's last token only: the groups of 8 rows that hold them become the first rows of a decode
     // projection (the other rows of that launch, if any, are whatever the buffer holds; rows are independent).
     const int group = (head_row / ANPD_ROWS) * ANPD_ROWS;
     const bool prompt = rows != kv->batch * ANPD_ROWS;
     if (prompt && !m->plain_gemm) {
-        const int img_rows = cl_fused(m->cl[GK_LM]) ? ANPD_ROWS : kv->batch * ANPD_ROWS;
+        const bool one = n_seq == 1 && cl_fused(m->cl[GK_LM]);
+        const int img_rows = one ? ANPD_ROWS : kv->batch * ANPD_ROWS;
         LAUNCH(pf, st, KC_OTHER, 0,
-               (launch_k(rows_to_image_kernel, ANPD_ROWS, 256, 0, st, ws.h_hi, ws.h_lo, group, d, ws.ci_h, img_rows)));
-        if (cl_fused(m->cl[GK_LM])) return lm_head_cl_enqueue(m, kv, nullptr, 0, want_logits);
+               (launch_k(rows_to_image_kernel, n_seq * ANPD_ROWS, 256, 0, st, ws.h_hi, ws.h_lo, group, rows / n_seq, d, ws.ci_h, img_rows)));
+        if (one) return lm_head_cl_enqueue(m, kv, nullptr, 0, want_logits);
     } else if (prompt) {
         LAUNCH(pf, st, KC_OTHER, 0, (launch_k(move_rows_kernel, ANPD_ROWS, 256, 0, st, ws.h_hi, ws.h_lo, group, d)));
     }

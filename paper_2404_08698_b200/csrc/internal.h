@@ -459,7 +459,7 @@ struct anpd_kv {
     float *rope_cos, *rope_sin;       // [max_len][hd/2]
     SeqState* seq;                    // device [batch]
     SeqState* h_seq;                  // pinned host staging [batch]
-    int* d_prompt;                    // device [max_len]
+    int* d_prompt;                    // device [batch][max_len]
     NgramDev* d_ctxs;                 // device [batch]: descriptors of the sequences' n-gram contexts
     int* h_small;                     // pinned, a few ints
     float* h_logits;                  // pinned, [ANPD_ROWS][vocab]: logits on their way to the caller (one sequence only)
@@ -497,7 +497,8 @@ struct anpd_kv {
 // max_pos: an upper bound of the largest position any row holds (sizes the attention grid).
 // head: also run the LM head and the per-block argmax (false for all but the last prefill pass).
 // head_row: in a prompt pass, the row whose next token is wanted (the LM head runs for its group of 8 rows only).
-anpd_status forward_enqueue(anpd_model* m, anpd_kv* kv, int rows, int max_pos, bool head, bool want_logits, int head_row = 0, bool two_candidates = false);
+anpd_status forward_enqueue(anpd_model* m, anpd_kv* kv, int rows, int max_pos, bool head, bool want_logits, int head_row = 0, bool two_candidates = false,
+                            int n_seq = 1);
 
 // step_kernel.cu: the whole forward of a decode step as ONE persistent kernel (one CTA per SM).  True if this model / cache
 // pair can take that path (head dimension 128, one query head per kv head, dimensions that are multiples of 128).
@@ -508,11 +509,12 @@ void step_kernel_trace_dump(anpd_kv* kv);
 
 enum AcceptMode { ACCEPT_COMMIT = 0, ACCEPT_PEEK = 1, ACCEPT_PREFILL = 2 };
 anpd_status plan_decode_enqueue(anpd_model* m, anpd_kv* kv, bool two_candidates = false);
-anpd_status plan_prefill_enqueue(anpd_model* m, anpd_kv* kv, int seq, int start, int prompt_len, int rows);
+anpd_status plan_prefill_enqueue(anpd_model* m, anpd_kv* kv, int seq, int start, int prompt_len, int rows, int n_seq = 1, int seg = 1 << 30);
 // mode COMMIT/PEEK: one block per sequence over its 8 rows.  PREFILL: `last_row` of sequence
 // `seq` gives the first generated token, kv_len becomes prompt_len.  d_ctxs may be null; otherwise
 // accepted tokens and the next token are appended to the sequences' token buffers.
-anpd_status accept_enqueue(anpd_model* m, anpd_kv* kv, int mode, const NgramDev* d_ctxs, int seq, int last_row, int prompt_len, bool two_candidates = false);
+anpd_status accept_enqueue(anpd_model* m, anpd_kv* kv, int mode, const NgramDev* d_ctxs, int seq, int last_row, int prompt_len, bool two_candidates = false,
+                           int n_seq = 1);
 
 // attn_tc.cu: per-page attention partials for head dimension 128 (same outputs as the mma.sync kernel in forward.cu)
 // tree: the rows carry cache slots and hidden slot ranges of their own (two-candidate steps)
@@ -521,7 +523,7 @@ anpd_status attn_tc_enqueue(anpd_model* m, anpd_kv* kv, int layer, int rows, int
 bool attn_dec_supported(const anpd_model* m);                // head dimension 64, or one query head per kv head
 anpd_status attn_dec_enqueue(anpd_model* m, anpd_kv* kv, int layer, bool tree);
 // attn_pf.cu: attention of a prompt pass with 128 query rows per CTA (head dimension 128, one query head per kv head)
-anpd_status attn_pf_enqueue(anpd_model* m, anpd_kv* kv, int layer, int rows, unsigned char* img);
+anpd_status attn_pf_enqueue(anpd_model* m, anpd_kv* kv, int layer, int rows, unsigned char* img, int n_seq);
 // attention of a prompt pass (one query head per kv head), written straight to the O projection's input
 anpd_status attn_prompt_enqueue(anpd_model* m, anpd_kv* kv, int layer, int rows);
 

@@ -1,9 +1,10 @@
 """Prompt passes at the row counts where their kernels change: the decode projections up to 128 rows, above that row tiles cut into
 equal multiples of 16 and up to eight parts along K."""
+import numpy as np
 import pytest
 import torch
 
-from helpers import as_bf16_values, gpu_model, new_stream, require_gpu, top2_margin
+from helpers import as_bf16_values, check_stream_against_oracle, gpu_model, new_stream, require_gpu, top2_margin
 from oracle.anpd import argmax_lowest
 from oracle.decoder import Decoder
 from workloads import ModelShape, make_weights, markov_prompt
@@ -48,3 +49,29 @@ def test_prompt_logits_at_row_tile_edges(A, rig, plen):
     # entries that round the other way (2^-9 of an entry, one in hundreds): well below 2^-9 of the logits' scale
     err = float((got - want).abs().max())
     assert err <= 2 ** -8 * max(1.0, float(want.abs().max())), err
+
+
+# rows per sequence: a group of 8 (as many rows as a step has: not to be taken for one), over it, over a tile of 32 and of 128 rows;
+# five sequences of 600 do not fit one pass of 2048 rows, three of 1030 take a pass each
+@pytest.mark.parametrize("hd,group", [(64, 4), (128, 1)])
+@pytest.mark.parametrize("batch,plen", [(3, 5), (4, 16), (8, 8), (2, 41), (5, 139), (5, 600), (3, 1030)])
+def test_prompts_of_several_sequences_share_a_pass(A, batch, plen, hd, group):
+    shape = ModelShape(2, 256, 2 * group, 2, hd, 520, 300)
+    w = make_weights(shape, 29, False, std=0.04)
+    st = new_stream()
+    m = gpu_model(A, shape, w, st)
+    kv = A.anpd_kv_create(m, plen + 24, batch, 1)
+    ctxs = [A.anpd_ngram_create(2, 3, plen + 24, 0, st) for _ in range(batch)]
+    dec = Decoder(shape, as_bf16_values(w), torch.float64, kv_dtype=torch.bfloat16)
+    prompts = np.stack([markov_prompt(plen, shape.vocab, 2, 400 + plen + b) for b in range(batch)])
+    try:
+        out, _ = A.anpd_generate_batch(m, kv, ctxs, prompts, 4, 3)
+        greedy, _ = A.anpd_generate_batch(m, kv, ctxs, prompts, 4, 0)
+        assert np.array_equal(out, greedy)
+        checked = sum(check_stream_against_oracle(dec, prompts[b].tolist(), out[b].tolist()) for b in range(batch))
+        assert checked >= 2
+    finally:
+        for c in ctxs:
+            A.anpd_ngram_destroy(c)
+        A.anpd_kv_destroy(kv)
+        A.anpd_model_destroy(m)
