@@ -790,8 +790,16 @@ static anpd_status cl_args(ClArgs* g, const ClPlan& p, const unsigned char* w, c
     const int up_max = (p.u_max + passes - 1) / passes, groups = up_max * p.gpu;
     const int tiles = one || groups <= 16 ? (groups + 15) / 16 : (groups + 31) / 32 * 2;
     // a cluster with few features: several k-blocks of its one tile make one copy
+    const int nk = (p.kb + CL_CTAS - 1) / CL_CTAS;      // k-blocks of a CTA, at most
     g->kps = (passes == 1 && tiles == 1) ? std::max(1, std::min(std::min(4, 16 / groups), 64 / rows)) : 1;
     if (g->kps == 3) g->kps = 2;                        // a step never straddles two activation slots
+    // A wait, a commit and the turn to the next activation slot cost the issuing thread as much as three to eight products.  So a CTA
+    // of a sequence's step whose k-blocks fit one activation slot takes them in one, and one whose weights all fit the ring beside
+    // another CTA has four k-blocks behind each wait.  1.1B (8 k-blocks: QKV, O, gate-up; ring: QKV, O): 807 -> 791 us per step at 512
+    // keys, 941 -> 922 at 4000; the slot alone 800, the ring alone 799.
+    const bool one_slot = one && nk > 4 && nk <= 8;
+    const bool in_ring = one_slot && tiles == 1 && 8 * groups * 1024 + 8 * rows * 256 + red_bytes + 1024 <= CL_SMEM_PAIR;
+    if (in_ring) g->kps = 4;
     g->two = tiles > 1 && !one;
     g->copies = g->two ? tiles / 2 : tiles;
     g->stage_bytes = tiles == 1 ? groups * g->kps * 1024 : (groups + g->copies - 1) / g->copies * 1024;
@@ -800,14 +808,14 @@ static anpd_status cl_args(ClArgs* g, const ClPlan& p, const unsigned char* w, c
     g->tmem_cols = 32;
     while (g->tmem_cols < g->acc_bufs * g->acc_cols) g->tmem_cols <<= 1;
     // activation slots of 8 KB (one sequence) to 32 KB, a whole number of steps each
-    g->akb = std::max(g->kps, std::min(4, 128 / rows));
+    g->akb = one_slot ? 8 : std::max(g->kps, std::min(4, 128 / rows));
     const int act_slot = g->akb * rows * 256;
-    g->act_slots = std::max(2, std::min(CL_MAX_ACT, (one ? 24 : 96) * 1024 / act_slot));
+    g->act_slots = one_slot ? 1 : std::max(2, std::min(CL_MAX_ACT, (one ? 24 : 96) * 1024 / act_slot));
     const int rest = g->act_slots * act_slot + red_bytes + 1024;
     // Two CTAs of one sequence's projections share an SM where five copies in flight fit beside the rest: the next kernel's first
     // ring is then requested long before its turn.  With fewer in flight the stream itself is slower than that gain (7B, QKV
     // alone: 4 in flight 20.6 us, 8 and no second CTA 18.7), so such a projection takes the SM for itself.
-    const bool pair = one && rest + 5 * g->stage_bytes <= CL_SMEM_PAIR;
+    const bool pair = in_ring || (one && rest + 5 * g->stage_bytes <= CL_SMEM_PAIR);
     const int room = (pair ? CL_SMEM_PAIR : CL_SMEM_MAX) - rest;
     g->stages = std::min(CL_MAX_STAGES, std::min(room, CL_RING_BYTES) / g->stage_bytes);
     if (g->stages < 2) return ANPD_ERR_CAPACITY;
