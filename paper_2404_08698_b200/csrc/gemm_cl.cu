@@ -323,8 +323,10 @@ __global__ void __launch_bounds__(cl_threads(R), 1) gemm_cl_kernel(const __grid_
             const uint32_t stage_step = (uint32_t)g.stage_bytes >> 4, act_step = (uint32_t)act_slot >> 4, kb_step = (uint32_t)(rows * 256) >> 4;
             const uint32_t full0 = smem_u32(&w_full[0]), empty_off = smem_u32(&w_empty[0]) - full0, full_end = full0 + 8u * (uint32_t)g.stages;
             uint32_t full = full0, wph = 0, w_lo = ring_lo;
-            int slot = 0, buf = 0;
-            uint32_t aph = 0, eph = 1, a_lo = act_lo;
+            const uint32_t af0 = smem_u32(&a_full[0]), aempty_off = smem_u32(&a_empty[0]) - af0, af_end = af0 + 8u * (uint32_t)g.act_slots;
+            const int akb = g.akb, kps = g.kps;
+            int buf = 0;
+            uint32_t afull = af0, aph = 0, eph = 1, a_lo = act_lo;
             // A wait that gave up has set the abort flag; the loops run on with whatever the buffers hold (every later wait is
             // short then), so that their trip counts depend on nothing the thread has to test.
             auto next_stage = [&]() {
@@ -342,9 +344,9 @@ __global__ void __launch_bounds__(cl_threads(R), 1) gemm_cl_kernel(const __grid_
                 const uint32_t d0 = tmem_base + (uint32_t)(buf * g.acc_cols);
                 uint32_t acc = 0;
                 const int k_end = T > 0 ? nk : 0;
-                for (int k0 = 0; k0 < k_end; k0 += g.akb) {
-                    mbar_wait(&a_full[slot], aph, abortp);
-                    const int kend = min(g.akb, nk - k0);
+                for (int k0 = 0; k0 < k_end; k0 += akb) {
+                    mbar_wait_at(afull, aph, abortp);
+                    const int kend = min(akb, nk - k0);
                     uint32_t a = a_lo;
                     // a tile of fewer than 16 groups: the instruction reads whatever follows for the rows beyond, whose lanes nobody reads
                     if (!R && g.two) {                                  // two tiles of one k-block per stage
@@ -378,7 +380,7 @@ __global__ void __launch_bounds__(cl_threads(R), 1) gemm_cl_kernel(const __grid_
                             a += kb_step;
                         }
                     } else {                                            // kps k-blocks of the only tile per stage
-                        for (int k = 0; k < kend; k += g.kps) {
+                        for (int k = 0; k < kend; k += kps) {
                             mbar_wait_at(full, wph, abortp);
                             tc_fence_after();
                             tc_mma_k64(d0, w_lo, a, idesc, acc);
@@ -386,7 +388,7 @@ __global__ void __launch_bounds__(cl_threads(R), 1) gemm_cl_kernel(const __grid_
                             a += kb_step;
                             uint32_t w = w_lo;
 #pragma unroll 1
-                            for (int j = min(g.kps, kend - k); j > 1; --j) {
+                            for (int j = min(kps, kend - k); j > 1; --j) {
                                 w += (uint32_t)(G << 6);
                                 tc_mma_k64(d0, w, a, idesc, 1u);
                                 a += kb_step;
@@ -394,9 +396,10 @@ __global__ void __launch_bounds__(cl_threads(R), 1) gemm_cl_kernel(const __grid_
                             next_stage();
                         }
                     }
-                    tc_commit(&a_empty[slot]);
+                    tc_commit_at(afull + aempty_off);
                     a_lo += act_step;
-                    if (++slot == g.act_slots) { slot = 0; aph ^= 1u; a_lo = act_lo; }
+                    afull += 8u;
+                    if (afull == af_end) { afull = af0; aph ^= 1u; a_lo = act_lo; }
                 }
                 tc_commit(&acc_full[buf]);
                 if (++buf == g.acc_bufs) { buf = 0; eph ^= 1u; }
@@ -808,14 +811,17 @@ static anpd_status cl_args(ClArgs* g, const ClPlan& p, const unsigned char* w, c
     g->tmem_cols = 32;
     while (g->tmem_cols < g->acc_bufs * g->acc_cols) g->tmem_cols <<= 1;
     // activation slots of 8 KB (one sequence) to 32 KB, a whole number of steps each
-    g->akb = one_slot ? 8 : std::max(g->kps, std::min(4, 128 / rows));
-    const int act_slot = g->akb * rows * 256;
-    g->act_slots = one_slot ? 1 : std::max(2, std::min(CL_MAX_ACT, (one ? 24 : 96) * 1024 / act_slot));
-    const int rest = g->act_slots * act_slot + red_bytes + 1024;
+    int rest = 0;
+    auto act_ring = [&](int akb, int slots) { g->akb = akb; g->act_slots = slots; rest = slots * akb * rows * 256 + red_bytes + 1024; };
+    const int akb = std::max(g->kps, std::min(4, 128 / rows));
+    if (one_slot) act_ring(8, 1);
+    else act_ring(akb, std::max(2, std::min(CL_MAX_ACT, (one ? 24 : 96) * 1024 / (akb * rows * 256))));
     // Two CTAs of one sequence's projections share an SM where five copies in flight fit beside the rest: the next kernel's first
     // ring is then requested long before its turn.  With fewer in flight the stream itself is slower than that gain (7B, QKV
     // alone: 4 in flight 20.6 us, 8 and no second CTA 18.7), so such a projection takes the SM for itself.
     const bool pair = in_ring || (one && rest + 5 * g->stage_bytes <= CL_SMEM_PAIR);
+    // with the SM to itself: half as many turns to the next slot (7B at 77 keys, 12 layers and the head: 1048.5 -> 1046.8)
+    if (one && !pair && akb == 4) act_ring(8, one_slot ? 1 : 3);
     const int room = (pair ? CL_SMEM_PAIR : CL_SMEM_MAX) - rest;
     g->stages = std::min(CL_MAX_STAGES, std::min(room, CL_RING_BYTES) / g->stage_bytes);
     if (g->stages < 2) return ANPD_ERR_CAPACITY;
