@@ -822,6 +822,9 @@ static anpd_status cl_args(ClArgs* g, const ClPlan& p, const unsigned char* w, c
     const bool pair = in_ring || (one && rest + 5 * g->stage_bytes <= CL_SMEM_PAIR);
     // with the SM to itself: half as many turns to the next slot (7B at 77 keys, 12 layers and the head: 1048.5 -> 1046.8)
     if (one && !pair && akb == 4) act_ring(8, one_slot ? 1 : 3);
+    // beside another CTA: the same 24 KB as two slots of six k-blocks instead of three of four (1.1B, down projection, 22 k-blocks: 785 ->
+    // 778 us per step); a step of kps k-blocks must not straddle two slots
+    if (pair && nk > 8 && akb == 4 && g->kps <= 2) act_ring(6, 2);
     const int room = (pair ? CL_SMEM_PAIR : CL_SMEM_MAX) - rest;
     g->stages = std::min(CL_MAX_STAGES, std::min(room, CL_RING_BYTES) / g->stage_bytes);
     if (g->stages < 2) return ANPD_ERR_CAPACITY;

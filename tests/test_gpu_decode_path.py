@@ -39,8 +39,8 @@ def test_projection_matches_fp64_product(A, N, K, rows):
 
 
 # one sequence, 5 to 8 k-blocks per CTA (one activation slot; all weights in the ring with few features), 4 and 9 beside them;
-# an SM of its own (many features) with more k-blocks than one slot of 8 holds
-@pytest.mark.parametrize("N,K", [(64, 1024), (64, 1088), (300, 1344), (2560, 2048), (2816, 2000), (5640, 2048), (700, 2056), (12296, 2200)])
+# an SM of its own (many features) with more k-blocks than one slot of 8 holds; half an SM with more than 8, steps of 4, 2 and 1 k-blocks
+@pytest.mark.parametrize("N,K", [(64, 1024), (64, 1088), (300, 1344), (2560, 2048), (2816, 2000), (5640, 2048), (700, 2056), (12296, 2200), (1000, 2600), (2048, 5632), (4096, 4104)])
 def test_projection_slots_of_one_sequence(A, N, K):
     test_projection_matches_fp64_product(A, N, K, 8)
 
