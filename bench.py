@@ -374,7 +374,7 @@ def gemm_traffic_per_launch(wl) -> float | None:
     if wl.shape.d_model != 4096 or wl.shape.d_ffn != 11008 or wl.shape.vocab != 32000:
         return None
     try:
-        text = open(os.path.join(ROOT, "profiles", "gemm_tc_kernel_7B_2layer_ncu.md")).read()
+        text = open(os.path.join(ROOT, "profiles", "gemm_cl_kernel_7B_2layer_ncu.md")).read()
         def row(name):
             line = next(l for l in text.splitlines() if l.startswith(name))
             return [float(x) for x in line.split(":", 1)[1].split(",")]
