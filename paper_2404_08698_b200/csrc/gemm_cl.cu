@@ -671,7 +671,9 @@ __global__ void __launch_bounds__(cl_threads(R), 1) gemm_cl_kernel(const __grid_
 
 // Rows [row_off, row_off + rows) of a row-major [rows][K] source into the storage of the plan's matrix: a block takes a row at a
 // time (its place is found once), a thread eight inputs at a time; eight threads write the row's 128 bytes of a k-block.
-template <typename T>
+// WIDE: eight bf16 inputs in one load.  The source is the caller's and may start at any element (a tensor inside a larger buffer),
+// so that takes a source on a 16-byte boundary (its rows are multiples of 16 bytes).
+template <typename T, bool WIDE>
 __global__ void __launch_bounds__(256) cl_retile_kernel(const T* __restrict__ src, int rows, int row_off, const ClPlan p, unsigned char* __restrict__ dst) {
     for (int r = blockIdx.x; r < rows; r += gridDim.x) {
         const int pos = cl_position(p, row_off + r), grp = pos >> 3, c = cl_owner(p, grp), g0 = cl_first_group(p, c);
@@ -680,7 +682,7 @@ __global__ void __launch_bounds__(256) cl_retile_kernel(const T* __restrict__ sr
         for (int k8 = threadIdx.x; k8 < p.K / 8; k8 += blockDim.x) {
             const T* in = src + (size_t)r * p.K + 8 * k8;
             bf16 v[8];
-            if (sizeof(T) == 2) *(uint4*)v = *(const uint4*)in;
+            if (WIDE) *(uint4*)v = *(const uint4*)in;
             else {
 #pragma unroll
                 for (int e = 0; e < 8; ++e) v[e] = (bf16)in[e];
@@ -763,8 +765,9 @@ int cl_parts(const ClPlan& p) { return p.ncl * CL_CTAS; }
 
 anpd_status cl_retile_enqueue(const ClPlan& p, const void* src, bool src_is_f32, int rows, int row_off, unsigned char* dst, cudaStream_t st) {
     const int blocks = std::min(rows, 148 * 16);
-    if (src_is_f32) cl_retile_kernel<float><<<blocks, 256, 0, st>>>((const float*)src, rows, row_off, p, dst);
-    else cl_retile_kernel<bf16><<<blocks, 256, 0, st>>>((const bf16*)src, rows, row_off, p, dst);
+    if (src_is_f32) cl_retile_kernel<float, false><<<blocks, 256, 0, st>>>((const float*)src, rows, row_off, p, dst);
+    else if ((uintptr_t)src % 16 == 0) cl_retile_kernel<bf16, true><<<blocks, 256, 0, st>>>((const bf16*)src, rows, row_off, p, dst);
+    else cl_retile_kernel<bf16, false><<<blocks, 256, 0, st>>>((const bf16*)src, rows, row_off, p, dst);
     CUDA_TRY(cudaGetLastError());
     return ANPD_OK;
 }

@@ -1,0 +1,51 @@
+"""Forms of a call that the boundary accepts and that depend on where or when it is made: weights anywhere in a larger buffer."""
+import numpy as np
+import pytest
+import torch
+
+from helpers import gpu_model, new_stream, require_gpu
+from workloads import ModelShape, make_weights, markov_prompt
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def A():
+    require_gpu()
+    from paper_2404_08698_b200 import binding
+    return binding
+
+
+def _prompt_and_logits(A, shape, m, kv, n=40):
+    prompt = markov_prompt(n, shape.vocab, 2, 31).tolist()
+    A.anpd_kv_truncate(kv, 0, 0)
+    first = A.anpd_prefill(m, kv, prompt)
+    return first, A.anpd_verify_logits(m, kv, first, [3, 9, 4], shape.vocab)
+
+
+# device matrices at 2, 8 and 14 bytes behind a 16-byte boundary; 0 beside them
+@pytest.mark.parametrize("bf16", [True, False])
+@pytest.mark.parametrize("offset", [0, 1, 4, 7])
+def test_device_weights_at_any_element_of_a_buffer(A, offset, bf16):
+    shape = ModelShape(2, 64, 2, 1, 64, 96, 160)
+    w = make_weights(shape, 3, bf16, std=0.08)
+
+    def inside(t):
+        if t.dim() != 2:
+            return t.cuda()
+        flat = torch.zeros(t.numel() + 16, dtype=t.dtype, device="cuda")
+        at = flat[offset:offset + t.numel()].view(t.shape)
+        at.copy_(t)
+        assert (at.data_ptr() - offset * t.element_size()) % 16 == 0
+        return at
+
+    got = []
+    for form in ({k: v.cuda() for k, v in w.items()}, {k: inside(v) for k, v in w.items()}):
+        torch.cuda.synchronize()
+        m = gpu_model(A, shape, form, new_stream())
+        kv = A.anpd_kv_create(m, 128)
+        got.append(_prompt_and_logits(A, shape, m, kv))
+        A.anpd_kv_destroy(kv)
+        A.anpd_model_destroy(m)
+    assert got[0][0] == got[1][0]
+    assert np.array_equal(got[0][1], got[1][1])
