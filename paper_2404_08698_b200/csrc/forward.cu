@@ -125,6 +125,7 @@ __global__ void __launch_bounds__(NORM_THREADS) embed_norm_kernel(const bf16* __
             ss += v[u].x * v[u].x + v[u].y * v[u].y + v[u].z * v[u].z + v[u].w * v[u].w;
         }
     }
+    cl_img_clear_row_tail(img, gridDim.x, row, d);
     const float rstd = rsqrtf(block_sum_1024(ss, red) / (float)d + eps);
 #pragma unroll
     for (int u = 0; u < NORM_MAX_CHUNKS; ++u) {
@@ -160,6 +161,7 @@ __global__ void __launch_bounds__(NORM_THREADS) embed_cl_kernel(const bf16* __re
                      (bf16*)(img + cl_img_offset(img_rows, img_rows + row, 4 * c)));        // 4 elements never straddle a 16-byte chunk
         acc += v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
     }
+    cl_img_clear_row_tail(img, img_rows, row, d);
     const float t = block_sum_1024(acc, red);
     if (threadIdx.x == 0) ss[row] = t;
 }
@@ -237,6 +239,7 @@ __global__ void __launch_bounds__(NORM_THREADS, NCH == 1 ? 2 : 1) resid_norm_ker
             ss += acc.x * acc.x + acc.y * acc.y + acc.z * acc.z + acc.w * acc.w;
         }
     }
+    cl_img_clear_row_tail(img, gridDim.x, row, d);
     const float rstd = rsqrtf(block_sum_1024(ss, red) / (float)d + eps);
 #pragma unroll
     for (int u = 0; u < NCH; ++u) {
@@ -791,6 +794,7 @@ __global__ void __launch_bounds__(256, CH == 1 ? 4 : 5) swiglu_kernel(const floa
     const int row = blockIdx.y, j0 = 4 * (CH * blockIdx.x * blockDim.x + threadIdx.x);
     constexpr int AT = CH == 1 ? 4 : 1;
     const float* pr = part + (size_t)row * ld_part;
+    if (blockIdx.x == 0) cl_img_clear_row_tail(img, gridDim.y, row, F);
     float4 g4[CH], u4[CH];
 #pragma unroll
     for (int c = 0; c < CH; ++c) g4[c] = u4[c] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -1034,6 +1038,7 @@ __global__ void rows_to_image_kernel(const bf16* __restrict__ h_hi, const bf16* 
     pdl_wait();
     const int r = blockIdx.x;
     const size_t src = (size_t)(from + r / ANPD_ROWS * step + r % ANPD_ROWS) * d;
+    cl_img_clear_row_tail(img, img_rows, r, d);
     for (int i = threadIdx.x; i < d / 8; i += blockDim.x) {
         *(uint4*)(img + cl_img_offset(img_rows, r, 8 * i)) = ((const uint4*)(h_hi + src))[i];
         *(uint4*)(img + cl_img_offset(img_rows, img_rows + r, 8 * i)) = ((const uint4*)(h_lo + src))[i];

@@ -496,6 +496,10 @@ __global__ void __launch_bounds__(cl_threads(R), 1) gemm_cl_kernel(const __grid_
         cluster_arrive();                               // nothing leaves for another CTA after the push
         mbar_wait_cluster(&red_full, 0, abortp);
         const int part_step = g.f_own_max * 8;
+        if (EPI == CL_RESID || EPI == CL_GU) {          // the image's columns behind the last feature: one CTA
+            const int k_out = EPI == CL_RESID ? g.d : g.n_out >> 1;
+            if ((k_out & 63) && blockIdx.x == 0 && ft < 128) cl_img_clear_tail(g.act_out, rows, ft >> 3, k_out, ft & 7);
+        }
         auto sum = [&](int f) {                         // feature f of this CTA's share, this thread's row, parts in CTA order
             const float* s = red + f * 8 + row;
             return ((s[0] + s[part_step]) + s[2 * part_step]) + s[3 * part_step];

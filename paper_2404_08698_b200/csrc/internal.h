@@ -274,6 +274,18 @@ __host__ __device__ inline size_t cl_weight_offset(const ClPlan& p, int pos, int
 __host__ __device__ inline size_t cl_img_offset(int rows, int r, int k) {
     return (size_t)(k >> 6) * (size_t)(rows * 256) + (size_t)(r >> 3) * 1024 + (size_t)(r & 7) * 128 + (size_t)((((k >> 3) & 7) ^ (r & 7)) << 4) + (size_t)(k & 7) * 2;
 }
+#ifdef __CUDACC__
+// Where K is no multiple of 64, the columns behind it in the last k-block meet zero weights, so any finite number may stand there -
+// but an image of another row count, made before, may have left an infinity or a NaN there, and 0 x NaN is NaN.  Whoever writes an
+// image clears them: 16-byte chunk `chunk` (0 .. 7) of operand row r, if it lies behind K.
+__device__ __forceinline__ void cl_img_clear_tail(unsigned char* img, int rows, int r, int K, int chunk) {
+    if (8 * chunk >= (K & 63)) *(uint4*)(img + cl_img_offset(rows, r, (K & ~63) + 8 * chunk)) = make_uint4(0u, 0u, 0u, 0u);
+}
+// the same by the block that writes row `row` of the image, hi and lo terms
+__device__ __forceinline__ void cl_img_clear_row_tail(unsigned char* img, int rows, int row, int K) {
+    if (img && (K & 63) && threadIdx.x < 16) cl_img_clear_tail(img, rows, row + (int)(threadIdx.x >> 3) * rows, K, threadIdx.x & 7);
+}
+#endif
 inline size_t cl_img_bytes(int rows, int K) { return (size_t)((K + 63) / 64) * rows * 256; }
 struct ClEpilogue {                    // only the fields of the projection's kind are read
     const float* ss_in = nullptr; int n_parts = 0; float inv_d = 0, eps = 0;            // n_parts = 0: the input is normalised already

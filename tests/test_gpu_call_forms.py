@@ -1,4 +1,5 @@
-"""Forms of a call that the boundary accepts and that depend on where or when it is made: weights anywhere in a larger buffer."""
+"""Forms of a call that the boundary accepts and that depend on where or when it is made: weights anywhere in a larger buffer, a
+handle that has seen other calls."""
 import numpy as np
 import pytest
 import torch
@@ -49,3 +50,35 @@ def test_device_weights_at_any_element_of_a_buffer(A, offset, bf16):
         A.anpd_model_destroy(m)
     assert got[0][0] == got[1][0]
     assert np.array_equal(got[0][1], got[1][1])
+
+
+# widths whose last k-block of 64 is part empty: the residual stream's, the FFN's, both
+@pytest.mark.parametrize("d,f", [(72, 128), (64, 96), (72, 96)])
+def test_an_overflow_stays_with_its_call(A, d, f):
+    """A prompt with a token whose FFN activations overflow, then ordinary calls of other row counts on the same handle: bit for bit
+    what a handle gives that has not seen it.  The token's keys and values are overwritten by the second prompt."""
+    shape = ModelShape(2, d, 1, 1, 64, f, 160)
+    w = make_weights(shape, 7, False, std=0.08)
+    bad, dim = 100, 5
+    w["embed"][:, dim] = 0.0
+    w["embed"][bad, dim] = 1.0
+    w["l0.wo"][dim] = 0.0                                       # the dimension is the token's alone where layer 0 reads it
+    w["l0.w_gate"][:, dim] = 1e25
+    w["l0.w_up"][:, dim] = 1e25
+    good = [t if t != bad else 3 for t in markov_prompt(80, shape.vocab, 2, 12).tolist()]
+    m = gpu_model(A, shape, w, new_stream())
+    used, fresh = A.anpd_kv_create(m, 128), A.anpd_kv_create(m, 128)
+    try:
+        A.anpd_prefill(m, used, good[:3] + [bad] + good[4:])    # 80 rows
+        assert not np.isfinite(A.anpd_verify_logits(m, used, 3, [5], shape.vocab)).all()
+        got = []
+        for kv in (used, fresh):
+            A.anpd_kv_truncate(kv, 0, 0)
+            first = A.anpd_prefill(m, kv, good[:40])            # 40 rows
+            got.append((first, A.anpd_verify_logits(m, kv, 3, [5, 9], shape.vocab)))
+        assert np.isfinite(got[1][1]).all()
+        assert got[0][0] == got[1][0] and np.array_equal(got[0][1], got[1][1])
+    finally:
+        A.anpd_kv_destroy(used)
+        A.anpd_kv_destroy(fresh)
+        A.anpd_model_destroy(m)
