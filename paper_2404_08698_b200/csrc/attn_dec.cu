@@ -7,7 +7,10 @@
 // wait); eight warps compute, each on its 16 keys of every page.  Where more than two query heads share a kv head, several
 // clusters read its pages (from L2 but for the first) and each computes a part of the heads.  One cluster of eight CTAs per kv head
 // with four times the rows and twice the warps was slower, its chain of products per page being four times as long: 1.1B (8 query
-// heads per kv head), per step, 827 -> 800 us at 512 keys, 891 -> 839 at 1400, 1024 -> 937 at 4000.
+// heads per kv head), per step, 827 -> 800 us at 512 keys, 891 -> 839 at 1400, 1024 -> 937 at 4000.  Head dimension 128 takes a
+// cluster per query head whatever the group: 32 query heads, 8 layers and the head, 300 keys, against page partials on the tensor
+// cores and a merging kernel: 16 / 8 / 4 kv heads 745 / 781 / 950 -> 698 / 684 / 683 us per step, at 4000 keys 850 / 871 / 997 ->
+// 793 / 801 / 793.
 //
 // Order.  A warp takes its blocks in ascending order with a running maximum; the warps of a CTA are merged in warp order, the
 // CTAs in rank order, each into the running result.  All of it depends on absolute key positions and on the handle (heads and
@@ -401,11 +404,6 @@ anpd_status launch_attn_dec(anpd_model* m, anpd_kv* kv, AdArgs& a) {
 
 }  // namespace
 
-bool attn_dec_supported(const anpd_model* m) {
-    const int G = m->cfg.n_q_heads / m->cfg.n_kv_heads;
-    return m->cfg.head_dim == 64 || G == 1;
-}
-
 anpd_status attn_dec_enqueue(anpd_model* m, anpd_kv* kv, int layer, bool tree) {
     const anpd_model_config& c = m->cfg;
     Workspace& ws = kv->ws;
@@ -422,6 +420,9 @@ anpd_status attn_dec_enqueue(anpd_model* m, anpd_kv* kv, int layer, bool tree) {
         case 64 * 16 + 4: a.split = 2; return launch_attn_dec<64, 2>(m, kv, a);
         case 64 * 16 + 8: a.split = 4; return launch_attn_dec<64, 2>(m, kv, a);
         case 128 * 16 + 1: a.split = 1; return launch_attn_dec<128, 1>(m, kv, a);
+        case 128 * 16 + 2: a.split = 2; return launch_attn_dec<128, 1>(m, kv, a);
+        case 128 * 16 + 4: a.split = 4; return launch_attn_dec<128, 1>(m, kv, a);
+        case 128 * 16 + 8: a.split = 8; return launch_attn_dec<128, 1>(m, kv, a);
     }
     return ANPD_ERR_ARG;
 }

@@ -528,11 +528,11 @@ anpd_status plan_prefill_enqueue(anpd_model* m, anpd_kv* kv, int seq, int start,
 anpd_status accept_enqueue(anpd_model* m, anpd_kv* kv, int mode, const NgramDev* d_ctxs, int seq, int last_row, int prompt_len, bool two_candidates = false,
                            int n_seq = 1);
 
-// attn_tc.cu: per-page attention partials for head dimension 128 (same outputs as the mma.sync kernel in forward.cu)
+// attn_tc.cu: per-page attention partials for head dimension 128 (same outputs as the mma.sync kernel in forward.cu); the row-range
+// projections' steps and the plain GEMM's take it
 // tree: the rows carry cache slots and hidden slot ranges of their own (two-candidate steps)
 anpd_status attn_tc_enqueue(anpd_model* m, anpd_kv* kv, int layer, int rows, int max_pos, bool tree = false);
 // attn_dec.cu: attention of a decode step, written straight to the O projection's operand image
-bool attn_dec_supported(const anpd_model* m);                // head dimension 64, or one query head per kv head
 anpd_status attn_dec_enqueue(anpd_model* m, anpd_kv* kv, int layer, bool tree);
 // attn_pf.cu: attention of a prompt pass with 128 query rows per CTA (head dimension 128, one query head per kv head)
 anpd_status attn_pf_enqueue(anpd_model* m, anpd_kv* kv, int layer, int rows, unsigned char* img, int n_seq);
