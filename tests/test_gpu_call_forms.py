@@ -1,5 +1,5 @@
 """Forms of a call that the boundary accepts and that depend on where or when it is made: weights anywhere in a larger buffer, a
-handle that has seen other calls."""
+handle that has seen other calls, n-gram calls behind a greedy loop."""
 import numpy as np
 import pytest
 import torch
@@ -81,4 +81,38 @@ def test_an_overflow_stays_with_its_call(A, d, f):
     finally:
         A.anpd_kv_destroy(used)
         A.anpd_kv_destroy(fresh)
+        A.anpd_model_destroy(m)
+
+
+# the first call after a greedy loop finds prompt and output unfolded: more than a call's one block takes
+@pytest.mark.parametrize("first", ["update", "draft"])
+def test_ngram_calls_after_a_greedy_loop(A, first):
+    shape = ModelShape(1, 64, 1, 1, 64, 96, 160)
+    st = new_stream()
+    m = gpu_model(A, shape, make_weights(shape, 9, False, std=0.08), st)
+    n, new = 700, 20
+    kv = A.anpd_kv_create(m, n + new + 32)
+    got, want = (A.anpd_ngram_create(2, 5, n + new + 64, 0, st) for _ in range(2))
+    prompt = markov_prompt(n, shape.vocab, 2, 44)
+    more = [7, 8, 9]
+    try:
+        tokens = np.append(prompt, A.anpd_generate(m, kv, want, prompt, new + 1, 0)[0])
+        A.anpd_generate(m, kv, got, prompt, new, 0)             # its context ends with the token behind the output
+        assert A.anpd_ngram_len(got) == len(tokens)
+        A.anpd_launch_count(True)
+        d = A.anpd_ngram_draft(got, 5) if first == "draft" else A.anpd_ngram_update(got, more)
+        assert A.anpd_launch_count() == 3                       # the two bulk passes, and the call's kernel
+        A.anpd_ngram_reset(want)
+        A.anpd_ngram_update(want, tokens)
+        if first == "draft":
+            assert A.anpd_ngram_draft(want, 5) == d
+            A.anpd_ngram_update(got, more)
+        A.anpd_ngram_update(want, more)
+        for level in range(2, 6):
+            assert A.anpd_ngram_dump(want, level) == A.anpd_ngram_dump(got, level)
+            assert A.anpd_ngram_dump_best(want, level) == A.anpd_ngram_dump_best(got, level)
+    finally:
+        for c in (got, want):
+            A.anpd_ngram_destroy(c)
+        A.anpd_kv_destroy(kv)
         A.anpd_model_destroy(m)
