@@ -134,7 +134,9 @@ anpd_status anpd_model_destroy(anpd_model* m);
 /* ---- KV cache ------------------------------------------------------------------------
  * Paged bf16 cache for `batch` independent sequences of at most max_len positions each
  * (max_len <= 32768 is rounded up to whole pages, batch <= 16; a step needs kv_len + 8 <= max_len).  Also holds the
- * activation buffers of a forward, so a kv handle is tied to the model it was created for.
+ * activation buffers of a forward, so a kv handle is tied to the model it was created for.  Several sequences' prompts
+ * (anpd_generate_batch) share passes of up to 2048 rows, for which the handle holds activations and partial sums; where the
+ * device has no room for them, every prompt takes passes of its own.
  * shuffle_pages != 0 permutes the physical page order (results must not change). */
 anpd_status anpd_kv_create(const anpd_model* m, int max_len, int batch, int shuffle_pages, anpd_kv** out);
 anpd_status anpd_kv_destroy(anpd_kv* kv);

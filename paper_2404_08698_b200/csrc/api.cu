@@ -146,6 +146,23 @@ bool have_device() {
 
 }  // namespace
 
+// Room for the partial sums of the projections: every row count a step or a prompt pass can have, with the cut it gets.
+static size_t part_elems(const anpd_model* m, Workspace& ws, int batch) {
+    const size_t step = (size_t)batch * ANPD_ROWS, few = std::max(step, (size_t)CL_PROMPT_ROWS);
+    size_t n = 0;
+    for (int k = 0; k < GK_COUNT; ++k) {
+        const size_t ld = ws.ld[k];
+        n = std::max(n, CL_CTAS * (k == GK_LM ? step : few) * ld);
+        if (m->plain_gemm) n = std::max(n, (k == GK_LM ? step : (size_t)ws.r_max) * ld);
+    }
+    for (int rows = CL_PROMPT_ROWS + ANPD_ROWS; rows <= ws.prefill_rows; rows += ANPD_ROWS)
+        for (int k = 0; k < GK_LM; ++k) {
+            const PfSchedule c = prompt_schedule(m, ws, k, rows);
+            n = std::max(n, (size_t)std::max(c.ksplit, c.tail_split) * rows * ws.ld[k]);
+        }
+    return n;
+}
+
 // GEMM plans (how each matrix shape is cut across the SMs) and the TMA views of the weights.
 static anpd_status model_make_plans(anpd_model* m) {
     const anpd_model_config& c = m->cfg;
@@ -404,49 +421,61 @@ anpd_status anpd_kv_create(const anpd_model* cm, int max_len, int batch, int shu
     kv->h_kv_len.assign(batch, 0);
     kv->h_len_stale.assign(batch, 0);
     Workspace& ws = kv->ws;
-    ws.prefill_rows = (int)std::min<long long>(PREFILL_ROWS_MAX, ((long long)kv->max_len * batch + 255) / 256 * 256);      // several sequences' prompts in one pass
+    kv->attn_tc = (c.head_dim == 128) && std::getenv("ANPD_ATTN_MMA_SYNC") == nullptr;
+    kv->attn_pf = std::getenv("ANPD_ATTN_MMA_SYNC") == nullptr && std::getenv("ANPD_ATTN_PROMPT_TILE16") == nullptr;
+    for (int k = 0; k < GK_COUNT; ++k) ws.ld[k] = (m->plan[k].N + 127) / 128 * 128;
     ws.pf_rows = 0;
-    ws.r_max = std::max(ws.prefill_rows, batch * ANPD_ROWS);
-    ws.n_max_out = (std::max(std::max(m->nqkv, 2 * c.d_ffn), std::max(c.d_model, c.vocab)) + 127) / 128 * 128;
-    ws.amax_blocks = (c.vocab + 1023) / 1024;
-    const size_t R = ws.r_max, d = c.d_model, F = c.d_ffn, V = c.vocab, hd = c.head_dim, half = hd / 2;
+    ws.amax_nblk = ws.amax_blocks = (c.vocab + 1023) / 1024;
+    const size_t d = c.d_model, F = c.d_ffn, V = c.vocab, hd = c.head_dim, half = hd / 2;
     const size_t pool = (size_t)c.n_layers * kv->total_pages * c.n_kv_heads * KV_PAGE * hd * 2;
-    const size_t n_part = (size_t)R * c.n_q_heads * kv->pages_per_seq;
     const int S = std::max(batch * ANPD_ROWS, CL_PROMPT_ROWS);      // rows of an operand image: a decode step's or a short prompt pass's
     struct Item { void** ptr; size_t bytes; };
-    std::vector<Item> items = {
-        {(void**)&kv->kpool, pool}, {(void**)&kv->vpool, pool},
-        {(void**)&kv->page_table, (size_t)kv->total_pages * 4},
-        {(void**)&kv->rope_cos, (size_t)kv->max_len * half * 4}, {(void**)&kv->rope_sin, (size_t)kv->max_len * half * 4},
-        {(void**)&kv->seq, sizeof(SeqState) * (size_t)batch}, {(void**)&kv->d_prompt, (size_t)kv->max_len * batch * 4},
-        {(void**)&kv->d_ctxs, sizeof(NgramDev) * (size_t)batch},
-        {(void**)&ws.row_tok, R * 4}, {(void**)&ws.row_pos, R * 4}, {(void**)&ws.row_seq, R * 4}, {(void**)&ws.row_ok, R * 4},
-        {(void**)&ws.row_slot, R * 4}, {(void**)&ws.row_hole_lo, R * 4}, {(void**)&ws.row_hole_hi, R * 4},
-        {(void**)&ws.x, R * d * 4}, {(void**)&ws.h_hi, R * d * 2}, {(void**)&ws.h_lo, R * d * 2},
-        {(void**)&ws.ao_hi, R * m->dq * 2}, {(void**)&ws.ao_lo, R * m->dq * 2},
-        {(void**)&ws.act_hi, R * F * 2}, {(void**)&ws.act_lo, R * F * 2},
-        {(void**)&ws.part, 3 * R * ws.n_max_out * 4},    // three partial sums per output, more where fewer rows are used
-        {(void**)&ws.q_hi, R * m->dq * 2}, {(void**)&ws.q_lo, R * m->dq * 2},
-        {(void**)&ws.attn_m, n_part * 4}, {(void**)&ws.attn_l, n_part * 4}, {(void**)&ws.attn_o, n_part * hd * 4},
-        {(void**)&ws.logits, (size_t)batch * ANPD_ROWS * V * 4},
-        {(void**)&ws.amax_val, R * ws.amax_blocks * 4}, {(void**)&ws.amax_idx, R * ws.amax_blocks * 4},
-        {(void**)&ws.gemm_err, 256}, {(void**)&kv->loop_steps_left, 256},
-        {(void**)&ws.img_h, act_img_bytes(c.d_model)}, {(void**)&ws.img_h2, act_img_bytes(c.d_model)},
-        {(void**)&ws.img_ao, act_img_bytes(m->dq)}, {(void**)&ws.img_act, act_img_bytes(c.d_ffn)},
-        {(void**)&ws.ci_h, cl_img_bytes(S, c.d_model)}, {(void**)&ws.ci_h2, cl_img_bytes(S, c.d_model)},
-        {(void**)&ws.ci_ao, cl_img_bytes(S, m->dq)}, {(void**)&ws.ci_act, cl_img_bytes(S, c.d_ffn)},
-        {(void**)&ws.ss_cl_a, (size_t)cl_parts(m->cl[GK_DOWN]) * ANPD_ROWS * 4}, {(void**)&ws.ss_cl_b, (size_t)cl_parts(m->cl[GK_O]) * ANPD_ROWS * 4},
-        {(void**)&ws.amax_val_cl, (size_t)cl_parts(m->cl[GK_LM]) * ANPD_ROWS * 4}, {(void**)&ws.amax_idx_cl, (size_t)cl_parts(m->cl[GK_LM]) * ANPD_ROWS * 4},
-        {(void**)&ws.ss_a, (size_t)m->num_sms * ANPD_ROWS * 4}, {(void**)&ws.ss_b, (size_t)m->num_sms * ANPD_ROWS * 4},
-        {(void**)&ws.amax_val_rr, (size_t)m->num_sms * ANPD_ROWS * 4}, {(void**)&ws.amax_idx_rr, (size_t)m->num_sms * ANPD_ROWS * 4},
-    };
-    ws.amax_nblk = ws.amax_blocks;
-    size_t total = 0;
-    for (const Item& it : items) total += up256(it.bytes);
-    kv->slab_bytes = total;
-    if (cudaMalloc(&kv->slab, total) != cudaSuccess) { cudaGetLastError(); delete kv; return ANPD_ERR_OOM; }
-    char* p = (char*)kv->slab;
-    for (const Item& it : items) { *it.ptr = p; p += up256(it.bytes); }
+    // Rows of a prompt pass: of several sequences' prompts at once or, where the device has no room for that, of one.
+    const long long want[2] = {std::min<long long>(PREFILL_ROWS_MAX, ((long long)kv->max_len * batch + 255) / 256 * 256),
+                               std::min<long long>(PREFILL_ROWS_MAX, (kv->max_len + 255) / 256 * 256)};
+    for (int attempt = 0;; ++attempt) {
+        ws.prefill_rows = (int)want[attempt];
+        ws.r_max = std::max(ws.prefill_rows, batch * ANPD_ROWS);
+        const size_t R = ws.r_max;
+        // page partials are left by the kernels that know no other way: those of steps and, as a cross-check, of prompt passes
+        const size_t n_part = (size_t)(kv->attn_pf ? batch * ANPD_ROWS : ws.r_max) * c.n_q_heads * kv->pages_per_seq;
+        std::vector<Item> items = {
+            {(void**)&kv->kpool, pool}, {(void**)&kv->vpool, pool},
+            {(void**)&kv->page_table, (size_t)kv->total_pages * 4},
+            {(void**)&kv->rope_cos, (size_t)kv->max_len * half * 4}, {(void**)&kv->rope_sin, (size_t)kv->max_len * half * 4},
+            {(void**)&kv->seq, sizeof(SeqState) * (size_t)batch}, {(void**)&kv->d_prompt, (size_t)kv->max_len * batch * 4},
+            {(void**)&kv->d_ctxs, sizeof(NgramDev) * (size_t)batch},
+            {(void**)&ws.row_tok, R * 4}, {(void**)&ws.row_pos, R * 4}, {(void**)&ws.row_seq, R * 4}, {(void**)&ws.row_ok, R * 4},
+            {(void**)&ws.row_slot, R * 4}, {(void**)&ws.row_hole_lo, R * 4}, {(void**)&ws.row_hole_hi, R * 4},
+            {(void**)&ws.x, R * d * 4}, {(void**)&ws.h_hi, R * d * 2}, {(void**)&ws.h_lo, R * d * 2},
+            {(void**)&ws.ao_hi, R * m->dq * 2}, {(void**)&ws.ao_lo, R * m->dq * 2},
+            {(void**)&ws.act_hi, R * F * 2}, {(void**)&ws.act_lo, R * F * 2},
+            {(void**)&ws.part, part_elems(m, ws, batch) * 4},
+            {(void**)&ws.q_hi, R * m->dq * 2}, {(void**)&ws.q_lo, R * m->dq * 2},
+            {(void**)&ws.attn_m, n_part * 4}, {(void**)&ws.attn_l, n_part * 4}, {(void**)&ws.attn_o, n_part * hd * 4},
+            {(void**)&ws.logits, (size_t)batch * ANPD_ROWS * V * 4},
+            {(void**)&ws.amax_val, R * ws.amax_blocks * 4}, {(void**)&ws.amax_idx, R * ws.amax_blocks * 4},
+            {(void**)&ws.gemm_err, 256}, {(void**)&kv->loop_steps_left, 256},
+            {(void**)&ws.img_h, act_img_bytes(c.d_model)}, {(void**)&ws.img_h2, act_img_bytes(c.d_model)},
+            {(void**)&ws.img_ao, act_img_bytes(m->dq)}, {(void**)&ws.img_act, act_img_bytes(c.d_ffn)},
+            {(void**)&ws.ci_h, cl_img_bytes(S, c.d_model)}, {(void**)&ws.ci_h2, cl_img_bytes(S, c.d_model)},
+            {(void**)&ws.ci_ao, cl_img_bytes(S, m->dq)}, {(void**)&ws.ci_act, cl_img_bytes(S, c.d_ffn)},
+            {(void**)&ws.ss_cl_a, (size_t)cl_parts(m->cl[GK_DOWN]) * ANPD_ROWS * 4}, {(void**)&ws.ss_cl_b, (size_t)cl_parts(m->cl[GK_O]) * ANPD_ROWS * 4},
+            {(void**)&ws.amax_val_cl, (size_t)cl_parts(m->cl[GK_LM]) * ANPD_ROWS * 4}, {(void**)&ws.amax_idx_cl, (size_t)cl_parts(m->cl[GK_LM]) * ANPD_ROWS * 4},
+            {(void**)&ws.ss_a, (size_t)m->num_sms * ANPD_ROWS * 4}, {(void**)&ws.ss_b, (size_t)m->num_sms * ANPD_ROWS * 4},
+            {(void**)&ws.amax_val_rr, (size_t)m->num_sms * ANPD_ROWS * 4}, {(void**)&ws.amax_idx_rr, (size_t)m->num_sms * ANPD_ROWS * 4},
+        };
+        size_t total = 0;
+        for (const Item& it : items) total += up256(it.bytes);
+        kv->slab_bytes = total;
+        if (cudaMalloc(&kv->slab, total) == cudaSuccess) {
+            char* p = (char*)kv->slab;
+            for (const Item& it : items) { *it.ptr = p; p += up256(it.bytes); }
+            break;
+        }
+        cudaGetLastError();
+        if (attempt == 1 || want[1] == want[0]) { delete kv; return ANPD_ERR_OOM; }
+    }
     const size_t small_bytes = up256(sizeof(SeqState) * (size_t)batch + 64 * sizeof(int) * (size_t)batch + 256);
     const size_t pinned_bytes = small_bytes + (batch == 1 ? sizeof(float) * ANPD_ROWS * V : 0);       // calls that return logits take one sequence
     if (cudaMallocHost((void**)&kv->h_seq, pinned_bytes) != cudaSuccess) { cudaGetLastError(); cudaFree(kv->slab); delete kv; return ANPD_ERR_OOM; }
@@ -466,8 +495,6 @@ anpd_status anpd_kv_create(const anpd_model* cm, int max_len, int batch, int shu
     }
 
     // TMA views of the K and V pools for the tensor-core attention: every page of every layer and kv head is 128 rows of hd
-    kv->attn_tc = (c.head_dim == 128) && std::getenv("ANPD_ATTN_MMA_SYNC") == nullptr;
-    kv->attn_pf = std::getenv("ANPD_ATTN_MMA_SYNC") == nullptr && std::getenv("ANPD_ATTN_PROMPT_TILE16") == nullptr;
     {
         anpd_status rc = make_tmap_bf16(&ws.map_q[0], ws.q_hi, ws.r_max, m->dq, 128, false);
         if (rc == ANPD_OK) rc = make_tmap_bf16(&ws.map_q[1], ws.q_lo, ws.r_max, m->dq, 128, false);
@@ -515,7 +542,7 @@ anpd_status anpd_kv_create(const anpd_model* cm, int max_len, int batch, int shu
         }
     }
     cudaStream_t st = m->stream;
-    bool ok = cudaMemsetAsync(kv->slab, 0, total, st) == cudaSuccess;
+    bool ok = cudaMemsetAsync(kv->slab, 0, kv->slab_bytes, st) == cudaSuccess;
     ok = ok && cudaMemcpyAsync(kv->page_table, pt.data(), pt.size() * 4, cudaMemcpyHostToDevice, st) == cudaSuccess;
     ok = ok && cudaMemcpyAsync(kv->rope_cos, hc.data(), hc.size() * 4, cudaMemcpyHostToDevice, st) == cudaSuccess;
     ok = ok && cudaMemcpyAsync(kv->rope_sin, hs.data(), hs.size() * 4, cudaMemcpyHostToDevice, st) == cudaSuccess;

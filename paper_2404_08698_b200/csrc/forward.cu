@@ -1079,7 +1079,7 @@ anpd_status gemm_enqueue(anpd_model* m, anpd_kv* kv, int kind, int layer, int ro
     if (m->plain_gemm) {
         *seg_count_out = nullptr;
         *seg_min_out = 1;
-        return gemm_plain_enqueue(plan, W, a_hi, a_lo, rows, ws.part, ws.n_max_out, m->stream, &m->prof);
+        return gemm_plain_enqueue(plan, W, a_hi, a_lo, rows, ws.part, ws.ld[kind], m->stream, &m->prof);
     }
     if (cl_rows(m, kv, rows)) {                        // a partial sum per CTA of a cluster
         const unsigned char* act = kind == GK_O ? ws.ci_ao : kind == GK_DOWN ? ws.ci_act : ws.ci_h;
@@ -1090,14 +1090,14 @@ anpd_status gemm_enqueue(anpd_model* m, anpd_kv* kv, int kind, int layer, int ro
         const int next = kind == GK_QKV ? GK_O : kind == GK_O ? GK_GU : kind == GK_GU ? GK_DOWN : last ? GK_LM : GK_QKV;
         const LayerW& lw = m->layers[layer];
         const unsigned char* next_w = kind == GK_QKV ? lw.wo : kind == GK_O ? lw.wgu : kind == GK_GU ? lw.wd : last ? m->lm_head : m->layers[layer + 1].wqkv;
-        return cl_partial_enqueue(plan, W, act, rows, ws.part, (size_t)rows * ws.n_max_out, ws.n_max_out, kind == GK_LM || (next == GK_LM && rows != kv->batch * ANPD_ROWS) ? nullptr : &m->cl[next], next_w,
+        return cl_partial_enqueue(plan, W, act, rows, ws.part, (size_t)rows * ws.ld[kind], ws.ld[kind], kind == GK_LM || (next == GK_LM && rows != kv->batch * ANPD_ROWS) ? nullptr : &m->cl[next], next_w,
                                   CL_LEAD, kind == GK_QKV && layer == 0 ? 0 : CL_LEAD, ws.gemm_err, m->stream, &m->prof);
     }
     // a prompt pass: complete sums, or several per output
     const int m_tiles = m->plan[kind].m_tiles;
     if (ws.pf_rows != rows) {
         for (int k = 0; k < GK_LM; ++k)
-            ws.pf_sched[k] = gemm_pf_schedule((m->plan[k].m_tiles + 1) / 2, rows, m->cl[k].kb, m->num_sms, std::min(PF_MAX_PARTS, 3 * ws.r_max / rows));
+            ws.pf_sched[k] = prompt_schedule(m, ws, k, rows);
         ws.pf_rows = rows;
     }
     const PfSchedule sched = ws.pf_sched[kind];
@@ -1113,7 +1113,7 @@ anpd_status gemm_enqueue(anpd_model* m, anpd_kv* kv, int kind, int layer, int ro
         *seg_count_out = nullptr;
     }
     *seg_min_out = sched.ksplit;
-    return gemm_pf_enqueue(plan, W, maps[0], maps[1], rows, ws.part, ws.n_max_out, (size_t)rows * ws.n_max_out, sched, m->num_sms,
+    return gemm_pf_enqueue(plan, W, maps[0], maps[1], rows, ws.part, ws.ld[kind], (size_t)rows * ws.ld[kind], sched, m->num_sms,
                            ws.gemm_err, m->stream, &m->prof);
 }
 
@@ -1334,7 +1334,7 @@ anpd_status forward_enqueue(anpd_model* m, anpd_kv* kv, int rows, int max_pos, b
     cudaStream_t st = m->stream;
     Profiler* pf = &m->prof;
     const int d = c.d_model, F = c.d_ffn, hd = c.head_dim, V = c.vocab;
-    const size_t sstride = (size_t)rows * ws.n_max_out;                            // between the partial sums of an output (the K parts of a projection)
+    auto sstride = [&](int kind) { return (size_t)rows * ws.ld[kind]; };           // between the partial sums of an output (the K parts of a projection)
     const size_t layer_elems = (size_t)kv->total_pages * c.n_kv_heads * KV_PAGE * hd;
     const int* segs = nullptr;
     int seg_min = 1;                                   // partial sums every tile of the last projection has
@@ -1350,17 +1350,17 @@ anpd_status forward_enqueue(anpd_model* m, anpd_kv* kv, int rows, int max_pos, b
             const dim3 grid(std::min(c.n_q_heads + 2 * c.n_kv_heads, std::max(1, m->num_sms * 8 / tiles)), tiles);
             const float qs = 1.4426950408889634f / sqrtf((float)hd);
             if (hd == 128) LAUNCH(pf, st, KC_OTHER, 0,
-                   (launch_k(qkv_rope_append_tile_kernel<128>, grid, 256, 0, st, ws.part, segs, sstride, ws.n_max_out, seg, ws.row_pos, ws.row_seq, ws.row_ok,
+                   (launch_k(qkv_rope_append_tile_kernel<128>, grid, 256, 0, st, ws.part, segs, sstride(GK_QKV), ws.ld[GK_QKV], seg, ws.row_pos, ws.row_seq, ws.row_ok,
                              kv->rope_cos, kv->rope_sin, kv->page_table, kv->pages_per_seq, c.n_q_heads, c.n_kv_heads, qs, ws.q_hi, ws.q_lo,
                              kv->kpool + l * layer_elems, kv->vpool + l * layer_elems, seg_min)));
             else LAUNCH(pf, st, KC_OTHER, 0,
-                   (launch_k(qkv_rope_append_tile_kernel<64>, grid, 256, 0, st, ws.part, segs, sstride, ws.n_max_out, seg, ws.row_pos, ws.row_seq, ws.row_ok,
+                   (launch_k(qkv_rope_append_tile_kernel<64>, grid, 256, 0, st, ws.part, segs, sstride(GK_QKV), ws.ld[GK_QKV], seg, ws.row_pos, ws.row_seq, ws.row_ok,
                              kv->rope_cos, kv->rope_sin, kv->page_table, kv->pages_per_seq, c.n_q_heads, c.n_kv_heads, qs, ws.q_hi, ws.q_lo,
                              kv->kpool + l * layer_elems, kv->vpool + l * layer_elems, seg_min)));
         } else
         LAUNCH(pf, st, KC_OTHER, 0,
                (launch_k(qkv_rope_append_kernel, dim3(rows, (c.n_q_heads + 2 * c.n_kv_heads + 1024 / hd - 1) / (1024 / hd)), 128, 0, st,
-                   ws.part, segs, sstride, ws.n_max_out, ws.row_pos, ws.row_slot, ws.row_seq, ws.row_ok, kv->rope_cos, kv->rope_sin,
+                   ws.part, segs, sstride(GK_QKV), ws.ld[GK_QKV], ws.row_pos, ws.row_slot, ws.row_seq, ws.row_ok, kv->rope_cos, kv->rope_sin,
                    kv->page_table, kv->pages_per_seq, c.n_q_heads, c.n_kv_heads, hd, 1.4426950408889634f / sqrtf((float)hd), ws.q_hi,
                    ws.q_lo, kv->kpool + l * layer_elems, kv->vpool + l * layer_elems, seg_min)));
         unsigned char* ao_img = slab ? ws.ci_ao : nullptr;
@@ -1370,19 +1370,19 @@ anpd_status forward_enqueue(anpd_model* m, anpd_kv* kv, int rows, int max_pos, b
         else ANPD_TRY(attn_enqueue<64>(m, kv, l, rows, max_pos, ao_img, two_candidates, ao_rows, n_seq));
         ANPD_TRY(gemm_enqueue(m, kv, GK_O, l, rows, &segs, &seg_min));
         LAUNCH(pf, st, KC_OTHER, 0,
-               (launch_k(resid_norm, rows, NORM_THREADS, 0, st, ws.x, ws.part, segs, sstride, ws.n_max_out, w.ffn_norm, c.rms_eps, d,
+               (launch_k(resid_norm, rows, NORM_THREADS, 0, st, ws.x, ws.part, segs, sstride(GK_O), ws.ld[GK_O], w.ffn_norm, c.rms_eps, d,
                                                        ws.h_hi, ws.h_lo, seg_min, slab ? ws.ci_h : nullptr)));
         ANPD_TRY(gemm_enqueue(m, kv, GK_GU, l, rows, &segs, &seg_min));
         if (rows >= 256) LAUNCH(pf, st, KC_OTHER, 0,
-               (launch_k(swiglu_kernel<2>, dim3((F / 4 + 511) / 512, rows), 256, 0, st, ws.part, segs, sstride, ws.n_max_out, F, ws.act_hi, ws.act_lo,
+               (launch_k(swiglu_kernel<2>, dim3((F / 4 + 511) / 512, rows), 256, 0, st, ws.part, segs, sstride(GK_GU), ws.ld[GK_GU], F, ws.act_hi, ws.act_lo,
                          seg_min, slab ? ws.ci_act : nullptr)));
         else LAUNCH(pf, st, KC_OTHER, 0,
-               (launch_k(swiglu_kernel<1>, dim3((F / 4 + 255) / 256, rows), 256, 0, st, ws.part, segs, sstride, ws.n_max_out, F, ws.act_hi, ws.act_lo,
+               (launch_k(swiglu_kernel<1>, dim3((F / 4 + 255) / 256, rows), 256, 0, st, ws.part, segs, sstride(GK_GU), ws.ld[GK_GU], F, ws.act_hi, ws.act_lo,
                          seg_min, slab ? ws.ci_act : nullptr)));
         ANPD_TRY(gemm_enqueue(m, kv, GK_DOWN, l, rows, &segs, &seg_min));
         const float* next_gain = (l + 1 < c.n_layers) ? m->layers[l + 1].attn_norm : m->final_norm;
         LAUNCH(pf, st, KC_OTHER, 0,
-               (launch_k(resid_norm, rows, NORM_THREADS, 0, st, ws.x, ws.part, segs, sstride, ws.n_max_out, next_gain, c.rms_eps, d,
+               (launch_k(resid_norm, rows, NORM_THREADS, 0, st, ws.x, ws.part, segs, sstride(GK_DOWN), ws.ld[GK_DOWN], next_gain, c.rms_eps, d,
                                                        ws.h_hi, ws.h_lo, seg_min, decode || (slab && l + 1 < c.n_layers) ? ws.ci_h : nullptr)));
     }
     if (!head) { CUDA_TRY(cudaGetLastError()); return ANPD_OK; }
@@ -1402,7 +1402,7 @@ anpd_status forward_enqueue(anpd_model* m, anpd_kv* kv, int rows, int max_pos, b
     rows = kv->batch * ANPD_ROWS;
     ANPD_TRY(gemm_enqueue(m, kv, GK_LM, 0, rows, &segs, &seg_min));
     LAUNCH(pf, st, KC_OTHER, 0,
-           (launch_k(argmax_partial_kernel, dim3(ws.amax_blocks, rows), 256, 0, st, ws.part, seg_min, (size_t)rows * ws.n_max_out, ws.n_max_out, V,
+           (launch_k(argmax_partial_kernel, dim3(ws.amax_blocks, rows), 256, 0, st, ws.part, seg_min, sstride(GK_LM), ws.ld[GK_LM], V,
                                                                              want_logits ? ws.logits : nullptr, ws.amax_val,
                                                                              ws.amax_idx, ws.amax_blocks)));
     CUDA_TRY(cudaGetLastError());

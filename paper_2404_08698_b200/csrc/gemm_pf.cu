@@ -249,8 +249,9 @@ static long long pf_cost(int n_ft, int rows, int k_blocks, int num_sms, const Pf
     const int uniform = s.tail_from * s.ksplit, tail = (n_ot - s.tail_from) * s.tail_split, grid = std::min(num_sms, uniform + tail);
     const long long a = (long long)((k_blocks + s.ksplit - 1) / s.ksplit) * step + item;
     const long long b = (long long)((k_blocks + s.tail_split - 1) / s.tail_split) * step + item;
+    // CTA i gets every grid-th item from i on: the counts of both kinds change at two places only
     long long worst = 0;
-    for (int i = 0; i < grid; ++i) {
+    for (int i : {0, uniform % grid, (uniform + tail) % grid}) {
         const int nu = (uniform - i + grid - 1) / grid, n = (uniform + tail - i + grid - 1) / grid;
         worst = std::max(worst, nu * a + (n - nu) * b);
     }
@@ -277,6 +278,10 @@ PfSchedule gemm_pf_schedule(int n_ft, int rows, int k_blocks, int num_sms, int m
             for (int s = 2; s <= std::min(std::min(max_parts, 4), k_blocks); ++s) consider({1, from, s, n_tt});
     }
     return best;
+}
+
+PfSchedule prompt_schedule(const anpd_model* m, const Workspace& ws, int kind, int rows) {
+    return gemm_pf_schedule((m->plan[kind].m_tiles + 1) / 2, rows, m->cl[kind].kb, m->num_sms, std::min(PF_MAX_PARTS, 3 * ws.r_max / rows));
 }
 
 anpd_status gemm_pf_enqueue(const ClPlan& plan, const unsigned char* w, const CUtensorMap& map_hi, const CUtensorMap& map_lo, int rows,

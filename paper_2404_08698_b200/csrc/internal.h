@@ -384,7 +384,7 @@ struct PfSchedule { int ksplit, tail_from, tail_split, n_tt; };
 struct Workspace {
     int r_max;                        // rows any forward may use
     int prefill_rows;                 // rows of one prompt pass (a multiple of 256)
-    int n_max_out;                    // widest GEMM output (max of nqkv, 2F, d, V)
+    int ld[GK_COUNT];                 // row stride of a projection's partial sums: its features, rounded up to 128
     int* row_tok; int* row_pos; int* row_seq; int* row_ok;    // [r_max]
     // two-candidate mode: the cache slot a row's K/V go to (its position otherwise) and a range of slots it must not see
     int* row_slot; int* row_hole_lo; int* row_hole_hi;          // [r_max]
@@ -392,7 +392,7 @@ struct Workspace {
     __nv_bfloat16 *h_hi, *h_lo;       // [r_max, d]   normalised input of QKV / gate-up / LM head
     __nv_bfloat16 *ao_hi, *ao_lo;     // [r_max, dq]  attention output, input of the O projection
     __nv_bfloat16 *act_hi, *act_lo;   // [r_max, F]   SwiGLU output, input of the down projection
-    float* part;                      // 3 * r_max * n_max_out partial sums of a projection: slabs of [rows][n_max_out]
+    float* part;                      // partial sums of a projection: slabs of [rows][ld]
     int pf_rows;                      // the prompt pass pf_sched was made for (0: none yet)
     PfSchedule pf_sched[GK_COUNT];
     __nv_bfloat16 *q_hi, *q_lo;       // [r_max, dq] rotated queries x log2(e)/sqrt(hd), as two bf16 terms
@@ -569,6 +569,7 @@ anpd_status gemm_tc_enqueue(const GemmPlan& plan, const __nv_bfloat16* w_blocks,
 // form a last, partly filled round of CTAs - into `tail_split` parts (tail_from == tile count: no such tail; a multiple of the
 // row tile count, so that a feature tile has one part count for all its rows).
 PfSchedule gemm_pf_schedule(int n_ft, int rows, int k_blocks, int num_sms, int max_parts);
+PfSchedule prompt_schedule(const anpd_model* m, const Workspace& ws, int kind, int rows);       // the cut a prompt pass of `rows` rows gets
 constexpr int PF_MAX_PARTS = 8;
 anpd_status gemm_pf_enqueue(const ClPlan& plan, const unsigned char* w, const CUtensorMap& map_hi, const CUtensorMap& map_lo, int rows,
                             float* out, int ld, size_t seg_stride, PfSchedule sched, int num_sms, int* err, cudaStream_t st, Profiler* prof);
