@@ -421,8 +421,9 @@ anpd_status anpd_kv_create(const anpd_model* cm, int max_len, int batch, int shu
     kv->h_kv_len.assign(batch, 0);
     kv->h_len_stale.assign(batch, 0);
     Workspace& ws = kv->ws;
-    kv->attn_tc = (c.head_dim == 128) && std::getenv("ANPD_ATTN_MMA_SYNC") == nullptr;
-    kv->attn_pf = std::getenv("ANPD_ATTN_MMA_SYNC") == nullptr && std::getenv("ANPD_ATTN_PROMPT_TILE16") == nullptr;
+    kv->attn_dec = std::getenv("ANPD_ATTN_MMA_SYNC") == nullptr;
+    kv->attn_tc = kv->attn_dec && c.head_dim == 128;
+    kv->attn_pf = kv->attn_dec && std::getenv("ANPD_ATTN_PROMPT_TILE16") == nullptr;
     for (int k = 0; k < GK_COUNT; ++k) ws.ld[k] = (m->plan[k].N + 127) / 128 * 128;
     ws.pf_rows = 0;
     ws.amax_nblk = ws.amax_blocks = (c.vocab + 1023) / 1024;

@@ -1293,7 +1293,7 @@ static anpd_status forward_cl_enqueue(anpd_model* m, anpd_kv* kv, int max_pos, b
         q.q_hi = ws.q_hi; q.q_lo = ws.q_lo; q.kpool_l = kv->kpool + l * layer_elems; q.vpool_l = kv->vpool + l * layer_elems;
         chain(q, l ? CL_LEAD : 0, GK_O, w.wo);
         ANPD_TRY(cl_enqueue(m->cl[GK_QKV], w.wqkv, ws.ci_h, q, ws.gemm_err, st, pf));
-        if (hd == 64 || kv->attn_tc) ANPD_TRY(attn_dec_enqueue(m, kv, l, two_candidates));
+        if (kv->attn_dec) ANPD_TRY(attn_dec_enqueue(m, kv, l, two_candidates));
         else if (hd == 128) ANPD_TRY(attn_enqueue<128>(m, kv, l, rows, max_pos, ws.ci_ao, two_candidates, rows));
         else ANPD_TRY(attn_enqueue<64>(m, kv, l, rows, max_pos, ws.ci_ao, two_candidates, rows));
         ClEpilogue o;
@@ -1365,7 +1365,7 @@ anpd_status forward_enqueue(anpd_model* m, anpd_kv* kv, int rows, int max_pos, b
                    ws.q_lo, kv->kpool + l * layer_elems, kv->vpool + l * layer_elems, seg_min)));
         unsigned char* ao_img = slab ? ws.ci_ao : nullptr;
         const int ao_rows = slab ? rows : 0;
-        if (decode && (hd == 64 || kv->attn_tc)) ANPD_TRY(attn_dec_enqueue(m, kv, l, two_candidates));
+        if (decode && kv->attn_dec) ANPD_TRY(attn_dec_enqueue(m, kv, l, two_candidates));
         else if (hd == 128) ANPD_TRY(attn_enqueue<128>(m, kv, l, rows, max_pos, ao_img, two_candidates, ao_rows, n_seq));
         else ANPD_TRY(attn_enqueue<64>(m, kv, l, rows, max_pos, ao_img, two_candidates, ao_rows, n_seq));
         ANPD_TRY(gemm_enqueue(m, kv, GK_O, l, rows, &segs, &seg_min));

@@ -465,7 +465,8 @@ struct anpd_kv {
     int batch, max_len, pages_per_seq, total_pages;
     __nv_bfloat16 *kpool, *vpool;     // per layer and page: K [Hkv][KV_PAGE][hd]; V transposed [Hkv][hd][KV_PAGE]
     CUtensorMap map_k, map_v;         // TMA views of the two pools: K as [all page positions][hd], V as [all page dims][KV_PAGE]
-    bool attn_tc;                     // attention on tcgen05 (head dimension 128); otherwise the mma.sync kernel
+    bool attn_dec;                    // attention of steps complete in one kernel (attn_dec.cu); otherwise page partials and a merge
+    bool attn_tc;                     // page partials on tcgen05 (head dimension 128); otherwise the mma.sync kernel
     bool attn_pf;                     // prompt passes: the 128-row kernel (attn_pf.cu); otherwise the 16-row kernel of attn_tc.cu
     int* page_table;                  // device [batch][pages_per_seq]
     float *rope_cos, *rope_sin;       // [max_len][hd/2]

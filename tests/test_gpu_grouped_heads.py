@@ -68,3 +68,28 @@ def test_streams_against_the_oracle(A, hkv, group, batch):
             A.anpd_ngram_destroy(c)
         A.anpd_kv_destroy(kv)
         A.anpd_model_destroy(m)
+
+
+@pytest.mark.parametrize("hd,group", [(64, 1), (64, 2), (64, 8), (128, 1), (128, 4)])
+def test_page_partials_on_mma_sync_cross_check_the_step_kernel(A, monkeypatch, hd, group):
+    """The same step through the page-wise kernel and its merge (one launch more per layer).  One layer: both read the same cache."""
+    shape = ModelShape(1, 64, 2 * group, 2, hd, 96, 160)
+    w = make_weights(shape, 8, False, std=0.08)
+    m = gpu_model(A, shape, w, new_stream())
+    prompt = markov_prompt(300, shape.vocab, 2, 18).tolist()
+    got, launches = [], []
+    try:
+        for sync in (False, True):
+            if sync:
+                monkeypatch.setenv("ANPD_ATTN_MMA_SYNC", "1")
+            kv = A.anpd_kv_create(m, 400, 1, 1)
+            A.anpd_prefill(m, kv, prompt)
+            A.anpd_launch_count(True)
+            got.append(A.anpd_verify_logits(m, kv, 3, [5, 9, 2, 7], shape.vocab))
+            launches.append(A.anpd_launch_count())
+            A.anpd_kv_destroy(kv)
+    finally:
+        A.anpd_model_destroy(m)
+    assert launches[1] == launches[0] + 1
+    # fp32 sums of two-term products (2^-17 of a term) in another order, through one layer
+    assert float(np.abs(got[0] - got[1]).max()) <= 2.0 ** -12 * max(1.0, float(np.abs(got[0]).max()))
