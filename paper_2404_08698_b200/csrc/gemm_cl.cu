@@ -54,6 +54,7 @@ struct ClArgs {
     const unsigned char* w;              // see ClPlan
     const unsigned char* act;            // operand image [k-block][2 * rows][64]
     int kb, gpu, n_units, ncl;
+    int seg, next_seg;                   // segments of the storage: ncl or 1
     int rows, passes, copies, two, kps, stages, stage_bytes, akb, act_slots, tmem_cols, acc_bufs, acc_cols;
     int f_own_max;
     // the projection after this one: its storage and cut, and how many bytes per CTA are fetched into L2 ahead (own: already done)
@@ -165,6 +166,7 @@ __global__ void __launch_bounds__(cl_threads(R), 1) gemm_cl_kernel(const __grid_
     const int rank = (int)blockIdx.x % C, cluster = (int)blockIdx.x / C;            // a cluster is C consecutive CTAs
     const int ulo = (int)((long long)cluster * g.n_units / g.ncl), uhi = (int)((long long)(cluster + 1) * g.n_units / g.ncl);
     const int Uc = uhi - ulo, Gc = Uc * g.gpu;                                      // units and groups of the cluster
+    const int GS = g.seg == 1 ? g.n_units * g.gpu : Gc;                             // groups of a k-block in its segment
     const int kb_lo = rank * g.kb / C, nk = (rank + 1) * g.kb / C - kb_lo;          // this CTA's k-blocks
 
     // Units [u0, u0 + up) of pass p (relative to the cluster), up * gpu groups in T copies per k-block: the first `rem` of them
@@ -190,21 +192,21 @@ __global__ void __launch_bounds__(cl_threads(R), 1) gemm_cl_kernel(const __grid_
             if (w_T == 0 || nk == 0) continue;
             w_base = w_G / w_T; w_rem = w_G - w_base * w_T;
             w_k = 0; w_t = 0;
-            w_src = g.w + ((size_t)ulo * g.gpu * g.kb + (size_t)Gc * kb_lo + (size_t)u0 * g.gpu) * 1024;
+            w_src = g.w + ((size_t)ulo * g.gpu * (g.seg == 1 ? 1 : g.kb) + (size_t)GS * kb_lo + (size_t)u0 * g.gpu) * 1024;
             return;
         }
     };
     const uint64_t pol_w = policy_evict_first();
     auto w_issue = [&](int stage) {                     // load the current item into `stage` and move on
         const int n = min(g.kps, nk - w_k);
-        const uint32_t bytes = (uint32_t)(n * (w_base + (w_t < w_rem ? 1 : 0))) << 10;      // n > 1 only where one tile holds all of the cluster's groups
+        const uint32_t bytes = (uint32_t)(n * (w_base + (w_t < w_rem ? 1 : 0))) << 10;      // n > 1 only where one tile holds all of the segment's groups
         mbar_expect_tx(&w_full[stage], bytes);
         bulk_load(ring + stage * g.stage_bytes, w_src, bytes, &w_full[stage], pol_w);
         w_src += bytes;
         if (++w_t == w_T) {
             w_t = 0;
             w_k += n;
-            w_src += (size_t)(Gc - w_G) << 10;          // the other passes' groups of the k-block
+            w_src += (size_t)(GS - w_G) << 10;          // the k-block's other groups
             if (w_k >= nk) { ++w_p; w_enter(); }
         }
     };
@@ -254,22 +256,32 @@ __global__ void __launch_bounds__(cl_threads(R), 1) gemm_cl_kernel(const __grid_
             uint32_t phase = 0;
             // L2 prefetch: through this CTA's own weights (where one pass reads them in storage order), then its share of the next
             // projection's first pass, k-block by k-block
-            const unsigned char* own = g.w + ((size_t)ulo * g.gpu * g.kb + (size_t)Gc * kb_lo) * 1024;
-            const unsigned end = passes == 1 ? (unsigned)(Gc * nk) << 10 : 0u;
-            unsigned cur = g.own_lead, left = 0, nxt_piece = 0, nxt_done = 0;
-            const unsigned char* nxt = nullptr;
+            const unsigned end = passes == 1 ? (unsigned)(Gc * nk) << 10 : 0u, own_piece = g.seg == 1 ? (unsigned)Gc << 10 : end;      // piece: contiguous
+            unsigned cur = g.own_lead, left = 0, own_done = 0, nxt_piece = 0, nxt_done = 0;
+            const unsigned char *own = nullptr, *nxt = nullptr;
             size_t nxt_step = 0;
+            if (cur < end) {
+                const unsigned k = cur / own_piece;
+                own_done = cur - k * own_piece;
+                own = g.w + ((size_t)ulo * g.gpu * (g.seg == 1 ? 1 : g.kb) + (size_t)GS * (kb_lo + (int)k)) * 1024;
+            }
             if (g.next_w) {
                 const int nu0 = (int)((long long)cluster * g.next_units / g.ncl), nu1 = (int)((long long)(cluster + 1) * g.next_units / g.ncl);
-                const int ng = (nu1 - nu0) * g.next_gpu, ng0 = (nu1 - nu0) / g.next_passes * g.next_gpu;
+                const int ng0 = (nu1 - nu0) / g.next_passes * g.next_gpu, ns = (g.next_seg == 1 ? g.next_units : nu1 - nu0) * g.next_gpu;
                 const int k0 = rank * g.next_kb / C, k1 = (rank + 1) * g.next_kb / C;
-                nxt = g.next_w + ((size_t)nu0 * g.next_gpu * g.next_kb + (size_t)ng * k0) * 1024;
-                nxt_piece = (unsigned)ng0 << 10; nxt_step = (size_t)ng << 10;
+                nxt = g.next_w + ((size_t)nu0 * g.next_gpu * (g.next_seg == 1 ? 1 : g.next_kb) + (size_t)ns * k0) * 1024;
+                nxt_piece = (unsigned)ng0 << 10; nxt_step = (size_t)ns << 10;
                 left = min(g.next_lead, (unsigned)(ng0 * (k1 - k0)) << 10);
             }
             auto ahead = [&](unsigned bytes) {
-                if (cur < end) { const unsigned n = min(bytes, end - cur); l2_prefetch(own + cur, n); cur += n; }
-                else if (left) {
+                if (cur < end) {
+                    while (bytes > 0 && cur < end) {
+                        const unsigned n = min(bytes, own_piece - own_done);
+                        l2_prefetch(own + own_done, n);
+                        cur += n; own_done += n; bytes -= n;
+                        if (own_done == own_piece) { own_done = 0; own += (size_t)GS << 10; }
+                    }
+                } else if (left) {
                     const unsigned n = min(min(bytes, left), nxt_piece - nxt_done);
                     l2_prefetch(nxt + nxt_done, n);
                     left -= n; nxt_done += n;
@@ -467,6 +479,10 @@ __global__ void __launch_bounds__(cl_threads(R), 1) gemm_cl_kernel(const __grid_
                 pg = *(const float2*)(g.gain + n);
             }
         }
+        if (EPI == CL_RESID || EPI == CL_GU) {          // the image's columns behind the last feature: one CTA, under the weight stream
+            const int k_out = EPI == CL_RESID ? g.d : g.n_out >> 1;
+            if ((k_out & 63) && blockIdx.x == 0 && ft < 128) cl_img_clear_tail(g.act_out, rows, ft >> 3, k_out, ft & 7);
+        }
         cluster_wait();
 
         if (pushes) {
@@ -496,10 +512,6 @@ __global__ void __launch_bounds__(cl_threads(R), 1) gemm_cl_kernel(const __grid_
         cluster_arrive();                               // nothing leaves for another CTA after the push
         mbar_wait_cluster(&red_full, 0, abortp);
         const int part_step = g.f_own_max * 8;
-        if (EPI == CL_RESID || EPI == CL_GU) {          // the image's columns behind the last feature: one CTA
-            const int k_out = EPI == CL_RESID ? g.d : g.n_out >> 1;
-            if ((k_out & 63) && blockIdx.x == 0 && ft < 128) cl_img_clear_tail(g.act_out, rows, ft >> 3, k_out, ft & 7);
-        }
         auto sum = [&](int f) {                         // feature f of this CTA's share, this thread's row, parts in CTA order
             const float* s = red + f * 8 + row;
             return ((s[0] + s[part_step]) + s[2 * part_step]) + s[3 * part_step];
@@ -680,9 +692,10 @@ __global__ void __launch_bounds__(cl_threads(R), 1) gemm_cl_kernel(const __grid_
 template <typename T, bool WIDE>
 __global__ void __launch_bounds__(256) cl_retile_kernel(const T* __restrict__ src, int rows, int row_off, const ClPlan p, unsigned char* __restrict__ dst) {
     for (int r = blockIdx.x; r < rows; r += gridDim.x) {
-        const int pos = cl_position(p, row_off + r), grp = pos >> 3, c = cl_owner(p, grp), g0 = cl_first_group(p, c);
-        const size_t step = (size_t)(cl_first_group(p, c + 1) - g0) * 1024;            // one k-block of the cluster
-        unsigned char* out = dst + (size_t)g0 * p.kb * 1024 + (size_t)(grp - g0) * 1024 + (size_t)(pos & 7) * 128;
+        const int pos = cl_position(p, row_off + r);
+        const ClRun run = cl_run(p, pos >> 3, 0);
+        const size_t step = (size_t)run.step * 1024;                                   // one k-block of the segment
+        unsigned char* out = dst + run.at + (size_t)(pos & 7) * 128;
         for (int k8 = threadIdx.x; k8 < p.K / 8; k8 += blockDim.x) {
             const T* in = src + (size_t)r * p.K + 8 * k8;
             bf16 v[8];
@@ -759,6 +772,12 @@ void cl_make_plan(ClPlan* p, int kind, int N, int K, int hd, int F, int ncl) {
     p->kb = (K + 63) / 64;
     p->ncl = ncl;
     p->u_max = (p->n_units + ncl - 1) / ncl;
+    // One segment where the contraction is long and a cluster's tiles are (nearly) full: CTAs side by side read one window, and a
+    // kernel that cuts the matrix its own way finds few seams (a stream-K cut over 148 CTAs, 13B width, 128 rows: gate-up 67.9 -> 63.7 us).
+    // Per step of 7B, 8 layers: one sequence 733 -> 727 us, two 792 -> 774.  Short contractions and smaller tiles lost 1 to 2 % by it
+    // (2560 wide 619 -> 630 us, 1.1B 793 -> 801): the weight thread then has more and smaller pieces to request.
+    const int groups = p->n_units / ncl * p->gpu, tiles = (p->u_max * p->gpu + 15) / 16;
+    p->seg = p->kb >= 64 && groups >= 13 * tiles ? 1 : ncl;
 }
 
 size_t cl_storage_bytes(const ClPlan& p) { return (size_t)p.n_units * p.gpu * p.kb * 1024; }
@@ -801,14 +820,15 @@ static anpd_status cl_args(ClArgs* g, const ClPlan& p, const unsigned char* w, c
     const int tiles = one || groups <= 16 ? (groups + 15) / 16 : (groups + 31) / 32 * 2;
     // a cluster with few features: several k-blocks of its one tile make one copy
     const int nk = (p.kb + CL_CTAS - 1) / CL_CTAS;      // k-blocks of a CTA, at most
-    g->kps = (passes == 1 && tiles == 1) ? std::max(1, std::min(std::min(4, 16 / groups), 64 / rows)) : 1;
+    g->seg = p.seg;
+    g->kps = (passes == 1 && tiles == 1 && p.seg == p.ncl) ? std::max(1, std::min(std::min(4, 16 / groups), 64 / rows)) : 1;
     if (g->kps == 3) g->kps = 2;                        // a step never straddles two activation slots
     // A wait, a commit and the turn to the next activation slot cost the issuing thread as much as three to eight products.  So a CTA
     // of a sequence's step whose k-blocks fit one activation slot takes them in one, and one whose weights all fit the ring beside
     // another CTA has four k-blocks behind each wait.  1.1B (8 k-blocks: QKV, O, gate-up; ring: QKV, O): 807 -> 791 us per step at 512
     // keys, 941 -> 922 at 4000; the slot alone 800, the ring alone 799.
     const bool one_slot = one && nk > 4 && nk <= 8;
-    const bool in_ring = one_slot && tiles == 1 && 8 * groups * 1024 + 8 * rows * 256 + red_bytes + 1024 <= CL_SMEM_PAIR;
+    const bool in_ring = one_slot && p.seg == p.ncl && tiles == 1 && 8 * groups * 1024 + 8 * rows * 256 + red_bytes + 1024 <= CL_SMEM_PAIR;
     if (in_ring) g->kps = 4;
     g->two = tiles > 1 && !one;
     g->copies = g->two ? tiles / 2 : tiles;
@@ -857,7 +877,7 @@ anpd_status cl_enqueue(const ClPlan& p, const unsigned char* w, const unsigned c
     g.q_hi = e.q_hi; g.q_lo = e.q_lo; g.kpool = e.kpool_l; g.vpool = e.vpool_l;
     g.x = e.x; g.gain = e.gain; g.ss_out = e.ss_out; g.d = e.d; g.act_out = e.act_out;
     g.out = e.out; g.amax_val = e.amax_val; g.amax_idx = e.amax_idx;
-    if (e.next) { g.next_w = e.next_w; g.next_kb = e.next->kb; g.next_gpu = e.next->gpu; g.next_units = e.next->n_units; g.next_passes = 1; g.next_lead = e.next_lead; }
+    if (e.next) { g.next_w = e.next_w; g.next_kb = e.next->kb; g.next_gpu = e.next->gpu; g.next_units = e.next->n_units; g.next_passes = 1; g.next_seg = e.next->seg; g.next_lead = e.next_lead; }
     g.own_lead = e.own_lead; g.own_burst = e.own_burst;
     g.err = err;
     const double bytes = 2.0 * (double)p.N * (double)p.K;
@@ -877,7 +897,7 @@ anpd_status cl_partial_enqueue(const ClPlan& p, const unsigned char* w, const un
     ClArgs g;
     int smem = 0;
     ANPD_TRY(cl_args(&g, p, w, act, rows, cl_passes(p, rows), 0, &smem));
-    if (next) { g.next_w = next_w; g.next_kb = next->kb; g.next_gpu = next->gpu; g.next_units = next->n_units; g.next_passes = cl_passes(*next, rows); g.next_lead = next_lead; }
+    if (next) { g.next_w = next_w; g.next_kb = next->kb; g.next_gpu = next->gpu; g.next_units = next->n_units; g.next_passes = cl_passes(*next, rows); g.next_seg = next->seg; g.next_lead = next_lead; }
     g.own_lead = own_lead; g.own_burst = 0;
     g.part = part; g.part_stride = part_stride; g.ld_part = ld_part; g.plan = p;
     g.err = err;

@@ -3,7 +3,7 @@
 //
 // A CTA owns an output tile of 256 features x T rows and walks the whole contraction dimension; T is the pass's rows cut into
 // equal tiles of at most 256.  Per 64-wide k-block it brings two 128-feature weight blocks (the storage the decode projections
-// stream, see ClPlan: the 256 features are neighbours in storage order, one linear copy per cluster they belong to) and the T
+// stream, see ClPlan: the 256 features are neighbours in storage order, one linear copy per segment they belong to) and the T
 // rows' hi and lo activation tiles (TMA boxes of 64 rows) into shared memory - 96 KB for sixteen 128 x 256 x 16 MMAs at T = 256 -
 // and accumulates W0 x hi, W0 x lo into one 256-column accumulator in tensor memory and W1 x hi, W1 x lo into a second one:
 // every activation byte is used against 256 features, every weight byte against T rows.  The first weight blocks are requested
@@ -70,7 +70,7 @@ gemm_pf_kernel(const unsigned char* __restrict__ w, const __grid_constant__ CUte
     __shared__ uint64_t bar_full[PF_MAX_STAGES], bar_empty[PF_MAX_STAGES], bar_acc_full, bar_acc_empty;
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
-    __shared__ const unsigned char* piece_src[PF_GROUPS];             // the tile's groups as runs inside one cluster's storage
+    __shared__ const unsigned char* piece_src[PF_GROUPS];             // the tile's groups as runs inside one segment
     __shared__ int piece_step[PF_GROUPS], piece_at[PF_GROUPS], piece_bytes[PF_GROUPS];
 
     pdl_trigger();
@@ -108,15 +108,16 @@ gemm_pf_kernel(const unsigned char* __restrict__ w, const __grid_constant__ CUte
                 pf_item(g, tile, ot, ks, parts);
                 const int ft = ot / g.n_tt, tt = ot - ft * g.n_tt;
                 const int row0 = tt * g.tile_rows;
-                const int g_begin = ft * PF_GROUPS, g_end = min(g_begin + PF_GROUPS, g.plan.n_units * g.plan.gpu);
+                const int g_begin = ft * PF_GROUPS, g_end = min(g_begin + PF_GROUPS, cl_groups(g.plan));
                 int pieces = 0;
                 for (int grp = g_begin; grp < g_end; ++pieces) {
-                    const int c = cl_owner(g.plan, grp), c0 = cl_first_group(g.plan, c), c1 = cl_first_group(g.plan, c + 1), e = min(c1, g_end);
-                    piece_src[pieces] = w + ((size_t)c0 * g.k_blocks + (grp - c0)) * 1024;
-                    piece_step[pieces] = (c1 - c0) * 1024;
+                    const ClRun r = cl_run(g.plan, grp, 0);
+                    const int n = min(r.run, g_end - grp);
+                    piece_src[pieces] = w + r.at;
+                    piece_step[pieces] = r.step * 1024;
                     piece_at[pieces] = (grp - g_begin) * 1024;
-                    piece_bytes[pieces] = (e - grp) * 1024;
-                    grp = e;
+                    piece_bytes[pieces] = n * 1024;
+                    grp += n;
                 }
                 const uint32_t stage_bytes = (uint32_t)((g_end - g_begin) * 1024 + 2 * g.boxes * PF_BOX);
                 const int kb_begin = ks * g.k_blocks / parts, kb_end = (ks + 1) * g.k_blocks / parts;
@@ -206,7 +207,7 @@ gemm_pf_kernel(const unsigned char* __restrict__ w, const __grid_constant__ CUte
             const int row0 = tt * g.tile_rows;
 #pragma unroll 1
             for (int j = 0; j < 2; ++j) {
-                const int pos0 = (2 * ft + j) * 128, n_pos = g.plan.n_units * g.plan.gpu * 8;
+                const int pos0 = (2 * ft + j) * 128, n_pos = cl_groups(g.plan) * 8;
                 if (pos0 >= n_pos) break;
                 const int pos = pos0 + quad * 32 + lane;
                 const int n = pos < n_pos ? cl_feature(g.plan, pos) : g.plan.N;

@@ -243,10 +243,10 @@ constexpr size_t CL_RING_SHARE = 96 * 1024;       // a CTA's weights that go out
 // Storage of an [N][K] weight matrix and its cut over the clusters of a decode projection.  The features are kept in an order
 // in which those that make one result together are neighbours: eight rotary pairs (dimensions i.., then i + hd/2..) or eight
 // gate features and their eight up features make a unit of two groups of 8; elsewhere a unit is one group.  Cluster c owns the
-// units [c * n_units / ncl, (c + 1) * n_units / ncl) and stores them as [k-block of 64][group], 1 KB per group and k-block: 8
-// rows of 128 bytes, 16-byte chunk c of row r at chunk position c ^ r, the shared-memory image the MMA reads (128-byte
-// swizzle).  So a run of groups of one k-block is one linear copy, for the decode kernel and for the prompt kernel alike.
-struct ClPlan { int kind, N, K, hd, F, gpu, n_units, kb, ncl, u_max; };
+// units [c * n_units / ncl, (c + 1) * n_units / ncl).  The matrix is stored in `seg` segments cut the same way, each as
+// [k-block of 64][group], 1 KB per group and k-block: 8 rows of 128 bytes, 16-byte chunk c of row r at chunk position c ^ r, the
+// shared-memory image the MMA reads (128-byte swizzle).  So a run of a segment's groups of one k-block is one linear copy.
+struct ClPlan { int kind, N, K, hd, F, gpu, n_units, kb, ncl, u_max, seg; };
 // storage position of feature n (position = 8 * group + row of the group), and the feature at a position
 __host__ __device__ inline int cl_position(const ClPlan& p, int n) {
     if (p.kind == CL_QKV) {
@@ -261,13 +261,21 @@ __host__ __device__ inline int cl_feature(const ClPlan& p, int pos) {
     if (p.kind == CL_GU) return ((pos >> 3) & 1) * p.F + (pos >> 4) * 8 + (pos & 7);
     return pos;
 }
-__host__ __device__ inline int cl_owner(const ClPlan& p, int group) {                    // the cluster that owns a group
-    return (int)(((long long)(group / p.gpu + 1) * p.ncl - 1) / p.n_units);
+__host__ __device__ inline int cl_groups(const ClPlan& p) { return p.n_units * p.gpu; }
+// the segment that holds a group, and a segment's first group (32-bit products: at most 32 n_units)
+__host__ __device__ inline int cl_segment(const ClPlan& p, int group) {
+    return p.seg == 1 ? 0 : (int)(((unsigned)((group >> (p.gpu - 1)) + 1) * (unsigned)p.seg - 1u) / (unsigned)p.n_units);
 }
-__host__ __device__ inline int cl_first_group(const ClPlan& p, int cluster) { return (int)((long long)cluster * p.n_units / p.ncl) * p.gpu; }
+__host__ __device__ inline int cl_segment_start(const ClPlan& p, int s) { return p.seg == 1 ? s * cl_groups(p) : (int)((unsigned)s * (unsigned)p.n_units / (unsigned)p.seg) * p.gpu; }
+// k-block kb of the groups from `group` on: where it lies, how many groups the segment still has (run), 1 KB units to the next k-block
+struct ClRun { size_t at; int run, step; };
+__host__ __device__ inline ClRun cl_run(const ClPlan& p, int group, int kb) {
+    const int s = cl_segment(p, group), g0 = cl_segment_start(p, s), g1 = cl_segment_start(p, s + 1);
+    return {((size_t)g0 * p.kb + (size_t)(g1 - g0) * kb + (group - g0)) * 1024, g1 - group, g1 - g0};
+}
 __host__ __device__ inline size_t cl_weight_offset(const ClPlan& p, int pos, int k) {   // byte offset of element (position, k)
-    const int grp = pos >> 3, r = pos & 7, c = cl_owner(p, grp), g0 = cl_first_group(p, c), gc = cl_first_group(p, c + 1) - g0;
-    return ((size_t)g0 * p.kb + (size_t)gc * (k >> 6) + (grp - g0)) * 1024 + (size_t)r * 128 + (size_t)((((k >> 3) & 7) ^ r) << 4) + (size_t)(k & 7) * 2;
+    const int r = pos & 7;
+    return cl_run(p, pos >> 3, k >> 6).at + (size_t)r * 128 + (size_t)((((k >> 3) & 7) ^ r) << 4) + (size_t)(k & 7) * 2;
 }
 // Operand image of the activations of a decode step: per 64-wide k-block 2 * rows operand rows of 128 bytes (hi parts of the
 // step's rows, then lo parts), 128-byte-swizzled.  Byte offset of element (operand row, k):
