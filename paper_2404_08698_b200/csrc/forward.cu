@@ -257,26 +257,23 @@ __global__ void __launch_bounds__(NORM_THREADS, NCH == 1 ? 2 : 1) resid_norm_ker
 // QKV epilogue: reduce splits, rotary embedding, append K/V to the paged cache, keep q
 // ---------------------------------------------------------------------------------------------
 // Bound by latency (a decode step) or by the partial sums' way through L2 (a prompt pass): a thread owns four rotary pairs, requests
-// the sums every tile has (ns_min) several at a time - seg_count, null where all tiles have as many, tells of more - and has fetched
-// what does not depend on the kernel before - the row plan (older than that kernel, see embed_norm_kernel), cosines and sines -
-// while it waits.
+// the sums several at a time, and has fetched what does not depend on the kernel before - the row plan (older than that kernel, see
+// embed_norm_kernel), cosines and sines - while it waits.
 struct RopeSum { float4 a, b; };
 
 template <int AT_ONCE>
-__device__ __forceinline__ RopeSum rope_sum(const float* __restrict__ pr, int half, size_t split_stride, const int* __restrict__ seg, int ns_min) {
+__device__ __forceinline__ RopeSum rope_sum(const float* __restrict__ pr, int half, size_t split_stride, int ns) {
     RopeSum r;
     r.a = r.b = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int s0 = 0; s0 < ns_min; s0 += AT_ONCE) {
+    for (int s0 = 0; s0 < ns; s0 += AT_ONCE) {
         float4 pa[AT_ONCE], pb[AT_ONCE];
 #pragma unroll
         for (int s = 0; s < AT_ONCE; ++s)
-            if (s0 + s < ns_min) { pa[s] = *(const float4*)(pr + (s0 + s) * split_stride); pb[s] = *(const float4*)(pr + (s0 + s) * split_stride + half); }
+            if (s0 + s < ns) { pa[s] = *(const float4*)(pr + (s0 + s) * split_stride); pb[s] = *(const float4*)(pr + (s0 + s) * split_stride + half); }
 #pragma unroll
         for (int s = 0; s < AT_ONCE; ++s)
-            if (s0 + s < ns_min) { add4(r.a, pa[s]); add4(r.b, pb[s]); }
+            if (s0 + s < ns) { add4(r.a, pa[s]); add4(r.b, pb[s]); }
     }
-    if (seg)
-        for (int s = ns_min; s < *seg; ++s) { add4(r.a, *(const float4*)(pr + s * split_stride)); add4(r.b, *(const float4*)(pr + s * split_stride + half)); }
     return r;
 }
 
@@ -300,43 +297,51 @@ __device__ __forceinline__ uint2 pack_bf16x4(float4 v) {
     return r;
 }
 
-// A decode step: hd / 8 threads per (row, head).
-__global__ void __launch_bounds__(128) qkv_rope_append_kernel(const float* __restrict__ part, const int* __restrict__ seg_count, size_t split_stride, int ld_part,
+// A step: a block takes the 8 rows of one sequence through the heads blockIdx.x, blockIdx.x + gridDim.x, ..., hd / 8 threads per
+// row.  A V head goes through shared memory, so that eight lanes write the rows' eight positions of a dimension of the transposed
+// page: single elements, a page row apart, were most of the kernel's time (7B, 16 sequences: 14.9 -> 8.5 us, 8: 9.0 -> 6.4).
+// seg_count is fixed by the model here and read before the wait.
+template <int HD>
+__global__ void __launch_bounds__(HD) qkv_rope_append_kernel(const float* __restrict__ part, const int* __restrict__ seg_count, size_t split_stride, int ld_part,
                                        const int* __restrict__ row_pos, const int* __restrict__ row_slot, const int* __restrict__ row_seq,
                                        const int* __restrict__ row_ok, const float* __restrict__ rope_cos,
                                        const float* __restrict__ rope_sin, const int* __restrict__ page_table,
-                                       int pages_per_seq, int Hq, int Hkv, int hd, float q_scale, bf16* __restrict__ q_hi,
+                                       int pages_per_seq, int Hq, int Hkv, float q_scale, bf16* __restrict__ q_hi,
                                        bf16* __restrict__ q_lo, bf16* __restrict__ kpool_l, bf16* __restrict__ vpool_l, int ns_min) {
     pdl_trigger();
-    const int half = hd >> 1, tph = hd >> 3, row = blockIdx.x, head = blockIdx.y * (blockDim.x / tph) + threadIdx.x / tph, i = threadIdx.x % tph * 4;
-    if (head >= Hq + 2 * Hkv) { pdl_wait(); return; }
+    constexpr int half = HD / 2, TPR = HD / 8;
+    __shared__ float tile[ANPD_ROWS][HD + 1];
+    __shared__ int s_page[ANPD_ROWS], s_slot[ANPD_ROWS];
+    const int r = threadIdx.x / TPR, i = threadIdx.x % TPR * 4, row = blockIdx.y * ANPD_ROWS + r;
     const size_t at = (size_t)row_pos[row] * half + i;
-    float4 c = make_float4(1.f, 1.f, 1.f, 1.f), sn = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (head < Hq + Hkv) { c = *(const float4*)(rope_cos + at); sn = *(const float4*)(rope_sin + at); }
+    const float4 c = *(const float4*)(rope_cos + at), sn = *(const float4*)(rope_sin + at);
     const int slot = row_slot[row];               // where the row lives in the cache (its position, except for a second candidate)
     const int page = page_table[row_seq[row] * pages_per_seq + slot / KV_PAGE], ok = row_ok[row];
+    if (i == 0) { s_page[r] = ok ? page : -1; s_slot[r] = slot % KV_PAGE; }
+    int ns = seg_count ? seg_count[(blockIdx.x * HD) >> 7] : ns_min;          // a head never straddles a 128-column tile
     pdl_wait();
-    RopeSum v = rope_sum<4>(part + (size_t)row * ld_part + (size_t)head * hd + i, half, split_stride, seg_count ? seg_count + ((head * hd) >> 7) : nullptr, ns_min);      // a head never straddles a 128-column tile
-    if (head < Hq + Hkv) rope_rotate(v, c, sn);
-    if (head < Hq) {
-        const size_t o = (size_t)row * Hq * hd + head * hd + i;
-        rope_store_q(v, q_scale, q_hi + o, q_lo + o, half);
-        return;
-    }
-    if (!ok) return;
-    const bool is_k = head < Hq + Hkv;
-    const int kvh = is_k ? head - Hq : head - Hq - Hkv;
-    bf16* pg = (is_k ? kpool_l : vpool_l) + ((size_t)page * Hkv + kvh) * KV_PAGE * hd;
-    if (is_k) {                                   // K page: [position][dim]
-        bf16* dst = pg + (size_t)(slot % KV_PAGE) * hd + i;
-        *(uint2*)dst = pack_bf16x4(v.a);
-        *(uint2*)(dst + half) = pack_bf16x4(v.b);
-    } else {                                      // V page is kept transposed: [dim][position]
-        const float a[4] = {v.a.x, v.a.y, v.a.z, v.a.w}, b[4] = {v.b.x, v.b.y, v.b.z, v.b.w};
+    for (int head = blockIdx.x; head < Hq + 2 * Hkv; head += gridDim.x) {
+        if (seg_count && head != (int)blockIdx.x) ns = seg_count[(head * HD) >> 7];
+        RopeSum v = rope_sum<4>(part + (size_t)row * ld_part + (size_t)head * HD + i, half, split_stride, ns);
+        if (head < Hq + Hkv) rope_rotate(v, c, sn);
+        if (head < Hq) {
+            const size_t o = (size_t)row * Hq * HD + head * HD + i;
+            rope_store_q(v, q_scale, q_hi + o, q_lo + o, half);
+        } else if (head < Hq + Hkv) {             // K page: [position][dim]
+            if (!ok) continue;
+            bf16* dst = kpool_l + (((size_t)page * Hkv + head - Hq) * KV_PAGE + slot % KV_PAGE) * HD + i;
+            *(uint2*)dst = pack_bf16x4(v.a);
+            *(uint2*)(dst + half) = pack_bf16x4(v.b);
+        } else {                                  // V page is kept transposed: [dim][position]
+            __syncthreads();
+            tile[r][i] = v.a.x; tile[r][i + 1] = v.a.y; tile[r][i + 2] = v.a.z; tile[r][i + 3] = v.a.w;
+            tile[r][i + half] = v.b.x; tile[r][i + half + 1] = v.b.y; tile[r][i + half + 2] = v.b.z; tile[r][i + half + 3] = v.b.w;
+            __syncthreads();
+            const int wr = threadIdx.x & (ANPD_ROWS - 1), pg = s_page[wr];
+            if (pg < 0) continue;
+            bf16* dst = vpool_l + ((size_t)pg * Hkv + head - Hq - Hkv) * KV_PAGE * HD + s_slot[wr];
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            pg[(size_t)(i + e) * KV_PAGE + (slot % KV_PAGE)] = __float2bfloat16_rn(a[e]);
-            pg[(size_t)(i + e + half) * KV_PAGE + (slot % KV_PAGE)] = __float2bfloat16_rn(b[e]);
+            for (int dim = threadIdx.x / ANPD_ROWS; dim < HD; dim += HD / ANPD_ROWS) dst[(size_t)dim * KV_PAGE] = __float2bfloat16_rn(tile[wr][dim]);
         }
     }
 }
@@ -346,6 +351,7 @@ __global__ void __launch_bounds__(128) qkv_rope_append_kernel(const float* __res
 // through shared memory, so that the transposed page receives whole 16-byte runs of positions instead of single elements.  Per
 // element the arithmetic is that of qkv_rope_append_kernel, in the same order.  7B: 80 rows 14 -> 6 us, 1536 rows 41 -> 36.
 constexpr int ROPE_TILE_ROWS = 32;
+constexpr int ROPE_BLOCKS = 12;                  // a step's blocks per SM
 template <int HD>
 __global__ void __launch_bounds__(256, 3) qkv_rope_append_tile_kernel(const float* __restrict__ part, const int* __restrict__ seg_count, size_t split_stride,
                                                                    int ld_part, int seg, const int* __restrict__ row_pos, const int* __restrict__ row_seq,
@@ -377,12 +383,12 @@ __global__ void __launch_bounds__(256, 3) qkv_rope_append_tile_kernel(const floa
     for (int head = blockIdx.x; head < Hq + 2 * Hkv; head += gridDim.x) {
         const bool is_q = head < Hq, is_k = !is_q && head < Hq + Hkv;
         bf16* pg = (is_k ? kpool_l : vpool_l) + ((size_t)page * Hkv + (is_q ? 0 : is_k ? head - Hq : head - Hq - Hkv)) * KV_PAGE * HD;
-        const int* count = seg_count ? seg_count + ((head * HD) >> 7) : nullptr;
+        const int count = seg_count ? seg_count[(head * HD) >> 7] : ns_min;
 #pragma unroll
         for (int u = 0; u < PER; ++u) {
             const int r = u * (256 / TPR) + threadIdx.x / TPR;
             if (r >= nr) continue;
-            RopeSum v = rope_sum<4>(part + (size_t)(r0 + r) * ld_part + (size_t)head * HD + i, half, split_stride, count, ns_min);
+            RopeSum v = rope_sum<4>(part + (size_t)(r0 + r) * ld_part + (size_t)head * HD + i, half, split_stride, count);
             if (is_q || is_k) rope_rotate(v, c[u], sn[u]);
             if (is_q) {
                 const size_t o = (size_t)(r0 + r) * Hq * HD + (size_t)head * HD + i;
@@ -1358,11 +1364,14 @@ anpd_status forward_enqueue(anpd_model* m, anpd_kv* kv, int rows, int max_pos, b
                              kv->rope_cos, kv->rope_sin, kv->page_table, kv->pages_per_seq, c.n_q_heads, c.n_kv_heads, qs, ws.q_hi, ws.q_lo,
                              kv->kpool + l * layer_elems, kv->vpool + l * layer_elems, seg_min)));
         } else
-        LAUNCH(pf, st, KC_OTHER, 0,
-               (launch_k(qkv_rope_append_kernel, dim3(rows, (c.n_q_heads + 2 * c.n_kv_heads + 1024 / hd - 1) / (1024 / hd)), 128, 0, st,
-                   ws.part, segs, sstride(GK_QKV), ws.ld[GK_QKV], ws.row_pos, ws.row_slot, ws.row_seq, ws.row_ok, kv->rope_cos, kv->rope_sin,
-                   kv->page_table, kv->pages_per_seq, c.n_q_heads, c.n_kv_heads, hd, 1.4426950408889634f / sqrtf((float)hd), ws.q_hi,
-                   ws.q_lo, kv->kpool + l * layer_elems, kv->vpool + l * layer_elems, seg_min)));
+        {
+            const float qs = 1.4426950408889634f / sqrtf((float)hd);
+            const dim3 grid(std::min(c.n_q_heads + 2 * c.n_kv_heads, std::max(1, m->num_sms * ROPE_BLOCKS / kv->batch)), kv->batch);
+            LAUNCH(pf, st, KC_OTHER, 0,
+                   (launch_k(hd == 128 ? qkv_rope_append_kernel<128> : qkv_rope_append_kernel<64>, grid, hd, 0, st, ws.part, segs, sstride(GK_QKV), ws.ld[GK_QKV],
+                             ws.row_pos, ws.row_slot, ws.row_seq, ws.row_ok, kv->rope_cos, kv->rope_sin, kv->page_table, kv->pages_per_seq, c.n_q_heads,
+                             c.n_kv_heads, qs, ws.q_hi, ws.q_lo, kv->kpool + l * layer_elems, kv->vpool + l * layer_elems, seg_min)));
+        }
         unsigned char* ao_img = slab ? ws.ci_ao : nullptr;
         const int ao_rows = slab ? rows : 0;
         if (decode && kv->attn_dec) ANPD_TRY(attn_dec_enqueue(m, kv, l, two_candidates));
