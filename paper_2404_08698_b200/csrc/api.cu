@@ -152,7 +152,10 @@ static size_t part_elems(const anpd_model* m, Workspace& ws, int batch) {
     size_t n = 0;
     for (int k = 0; k < GK_COUNT; ++k) {
         const size_t ld = ws.ld[k];
-        n = std::max(n, CL_CTAS * (k == GK_LM ? step : few) * ld);
+        for (size_t rows = ANPD_ROWS; rows <= (k == GK_LM ? step : few); rows += ANPD_ROWS) {
+            const GemmPlan* tc = tc_model_plan(m, k, (int)rows);
+            n = std::max(n, (tc ? tc->max_segs : CL_CTAS) * rows * ld);
+        }
         if (m->plain_gemm) n = std::max(n, (k == GK_LM ? step : (size_t)ws.r_max) * ld);
     }
     for (int rows = CL_PROMPT_ROWS + ANPD_ROWS; rows <= ws.prefill_rows; rows += ANPD_ROWS)
@@ -1124,35 +1127,46 @@ static anpd_status debug_gemm_row_range(const uint16_t* w_bf16, int N, int K, co
     return rc;
 }
 
-// The product through the decode projection (a cluster of CTAs per range of features), plain epilogue.
-static anpd_status debug_gemm_cluster(const uint16_t* w_bf16, int N, int K, const float* a, int rows, float* out) {
+// The product through the projections of a step, plain epilogue: one sequence's rows on clusters, more of them as partial sums.
+static anpd_status debug_gemm_step(const uint16_t* w_bf16, int N, int K, const float* a, int rows, float* out) {
     ClPlan plan;
+    GemmPlan tc;
     const int ncl = cl_clusters();
     if (ncl < 1) return ANPD_ERR_CUDA;
+    int dev = 0, sms = 0;
+    CUDA_TRY(cudaGetDevice(&dev));
+    CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     cl_make_plan(&plan, CL_RAW, N, K, 0, 0, ncl);
+    gemm_make_plan(&tc, N, K, sms);
+    const bool fused = rows == ANPD_ROWS && cl_fused(plan), sweep = !fused && tc_model_fits(tc, rows);
+    const int parts = fused ? 1 : sweep ? tc.max_segs : CL_CTAS;
     const size_t wb = up256(cl_storage_bytes(plan)), ib = up256(cl_img_bytes(rows, K)), sb = up256((size_t)N * K * 2),
-                 ab = up256((size_t)rows * K * 4), ob = up256((size_t)CL_CTAS * rows * N * 4);
-    const int parts = rows == ANPD_ROWS && cl_fused(plan) ? 1 : CL_CTAS;
+                 ab = up256((size_t)rows * K * 4), ob = up256((size_t)parts * rows * N * 4), tb = up256((tc.first_cta.size() + tc.seg_count.size()) * 4);
     char* slab = nullptr;
-    if (cudaMalloc((void**)&slab, wb + ib + sb + ab + ob + 256) != cudaSuccess) { cudaGetLastError(); return ANPD_ERR_OOM; }
+    if (cudaMalloc((void**)&slab, wb + ib + sb + ab + ob + tb + 256) != cudaSuccess) { cudaGetLastError(); return ANPD_ERR_OOM; }
     unsigned char* dW = (unsigned char*)slab;
     unsigned char* dimg = dW + wb;
     void* dsrc = dimg + ib;
     float* da = (float*)((char*)dsrc + sb);
     float* dout = (float*)((char*)da + ab);
-    int* derr = (int*)((char*)dout + ob);
+    tc.d_first_cta = (int*)((char*)dout + ob);
+    tc.d_seg_count = tc.d_first_cta + tc.first_cta.size();
+    int* derr = (int*)((char*)dout + ob + tb);
     auto body = [&]() -> anpd_status {
         CUDA_TRY(cudaMemset(slab, 0, wb + ib));
-        CUDA_TRY(cudaMemset(dout, 0, ob + 256));
+        CUDA_TRY(cudaMemset(dout, 0, ob + tb + 256));
+        CUDA_TRY(cudaMemcpy(tc.d_first_cta, tc.first_cta.data(), tc.first_cta.size() * 4, cudaMemcpyHostToDevice));
         CUDA_TRY(cudaMemcpy(dsrc, w_bf16, (size_t)N * K * 2, cudaMemcpyHostToDevice));
         CUDA_TRY(cudaMemcpy(da, a, (size_t)rows * K * 4, cudaMemcpyHostToDevice));
         ANPD_TRY(cl_retile_enqueue(plan, dsrc, false, N, 0, dW, 0));
         ANPD_TRY(cl_image_enqueue(da, rows, K, dimg, 0));
         CUDA_TRY(cudaDeviceSynchronize());
-        if (rows == ANPD_ROWS && cl_fused(plan)) {
+        if (fused) {
             ClEpilogue e;
             e.out = dout;
             ANPD_TRY(cl_enqueue(plan, dW, dimg, e, derr, 0, nullptr));
+        } else if (sweep) {
+            ANPD_TRY(gemm_tc_model_enqueue(tc, plan, dW, dimg, rows, dout, (size_t)rows * N, N, derr, 0, nullptr));
         } else {
             ANPD_TRY(cl_partial_enqueue(plan, dW, dimg, rows, dout, (size_t)rows * N, N, nullptr, nullptr, 0, 0, derr, 0, nullptr));
         }
@@ -1163,8 +1177,9 @@ static anpd_status debug_gemm_cluster(const uint16_t* w_bf16, int N, int K, cons
         std::vector<float> part((size_t)parts * rows * N);
         CUDA_TRY(cudaMemcpy(part.data(), dout, part.size() * 4, cudaMemcpyDeviceToHost));
         for (size_t i = 0; i < (size_t)rows * N; ++i) {
+            const int n = sweep ? tc.seg_count[(i % N) >> 7] : parts;
             float acc = part[i];
-            for (int k = 1; k < parts; ++k) acc += part[(size_t)k * rows * N + i];
+            for (int k = 1; k < n; ++k) acc += part[(size_t)k * rows * N + i];
             out[i] = acc;
         }
         return ANPD_OK;
@@ -1179,7 +1194,7 @@ anpd_status anpd_debug_gemm(const uint16_t* w_bf16, int N, int K, const float* a
     if (plain == 2 && rows != ANPD_ROWS) return ANPD_ERR_ARG;
     if (!have_device()) return ANPD_ERR_CUDA;
     if (plain == 2) return debug_gemm_row_range(w_bf16, N, K, a, out);
-    if (plain == 3) return debug_gemm_cluster(w_bf16, N, K, a, rows, out);
+    if (plain == 3) return debug_gemm_step(w_bf16, N, K, a, rows, out);
     int dev = 0, sms = 0;
     CUDA_TRY(cudaGetDevice(&dev));
     CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));

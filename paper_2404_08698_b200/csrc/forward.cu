@@ -838,7 +838,7 @@ __global__ void __launch_bounds__(256, CH == 1 ? 4 : 5) swiglu_kernel(const floa
 // LM-head epilogue: reduce splits, (optionally) keep logits, per-block argmax with ties to the lowest id
 // ---------------------------------------------------------------------------------------------
 constexpr int AMAX_COLS = 1024;
-__global__ void __launch_bounds__(256) argmax_partial_kernel(const float* __restrict__ part, int n_parts, size_t split_stride,
+__global__ void __launch_bounds__(256) argmax_partial_kernel(const float* __restrict__ part, const int* __restrict__ seg_count, int n_parts, size_t split_stride,
                                                              int ld_part, int V, float* __restrict__ logits,
                                                              float* __restrict__ amax_val, int* __restrict__ amax_idx, int nblk) {
     pdl_trigger();
@@ -852,8 +852,9 @@ __global__ void __launch_bounds__(256) argmax_partial_kernel(const float* __rest
     const int v = blockIdx.x * AMAX_COLS + 4 * threadIdx.x;              // four consecutive features (the slabs' rows are padded)
     if (v < V) {
         float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
+        const int ns = seg_count ? seg_count[v >> 7] : n_parts;
 #pragma unroll 4
-        for (int s = 0; s < n_parts; ++s) add4(z4, *(const float4*)(pr + s * split_stride + v));
+        for (int s = 0; s < ns; ++s) add4(z4, *(const float4*)(pr + s * split_stride + v));
         const float z[4] = {z4.x, z4.y, z4.z, z4.w};
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
@@ -1063,7 +1064,7 @@ __global__ void move_rows_kernel(bf16* __restrict__ h_hi, bf16* __restrict__ h_l
     }
 }
 
-// Whether the projections of a forward of `rows` rows run on the decode kernel (weights streamed once, four partial sums per
+// Whether the projections of a forward of `rows` rows run on the decode kernels (weights streamed once, several partial sums per
 // output, operand images): decode steps, and prompt passes of up to CL_PROMPT_ROWS rows - as many as the tensor memory holds for
 // it.  There the weights bound a pass and this kernel streams them better: 7B, pass of 77 tokens 8.7 -> 4.7 ms, of 128 5.5 ms,
 // where 129 on the prompt GEMM take 5.9.
@@ -1089,6 +1090,11 @@ anpd_status gemm_enqueue(anpd_model* m, anpd_kv* kv, int kind, int layer, int ro
     }
     if (cl_rows(m, kv, rows)) {                        // a partial sum per CTA of a cluster
         const unsigned char* act = kind == GK_O ? ws.ci_ao : kind == GK_DOWN ? ws.ci_act : ws.ci_h;
+        if (const GemmPlan* tc = tc_model_plan(m, kind, rows)) {
+            *seg_count_out = tc->d_seg_count;
+            *seg_min_out = tc->min_segs;
+            return gemm_tc_model_enqueue(*tc, plan, W, act, rows, ws.part, (size_t)rows * ws.ld[kind], ws.ld[kind], ws.gemm_err, m->stream, &m->prof);
+        }
         *seg_count_out = nullptr;
         *seg_min_out = CL_CTAS;
         // the projection after this one, whose first weights are fetched into L2 under the small kernels between the two
@@ -1162,6 +1168,14 @@ anpd_status attn_enqueue(anpd_model* m, anpd_kv* kv, int layer, int rows, int ma
 }
 
 }  // namespace
+
+// Where the projections of several sequences' steps run as one stream-K sweep over all SMs and not on clusters.  The cluster form
+// re-reads its activations once per pass and leaves four sums per value, which costs more the more rows there are; the sweep's
+// sums are one more than a tile has CTAs, which a narrow or short matrix pays for.  us per step, cluster form and sweep: 13B (10
+// layers) 16 sequences 2733 and 2409, 12 2345 and 2069, 8 1760 and 1749, 6 1606 and 1559; 7B (8 layers) 16 1460 and 1415, 12 1240 and
+// 1168, 8 1000 and 998, 4 817 and 803, but 2 sequences 771 and 783; 1.1B, 8 sequences 1241 and 1341.
+bool tc_model_fits(const GemmPlan& p, int rows) { return rows >= 32 && p.k_blocks >= 64 && p.max_segs <= 6; }
+const GemmPlan* tc_model_plan(const anpd_model* m, int kind, int rows) { return tc_model_fits(m->plan[kind], rows) ? &m->plan[kind] : nullptr; }
 
 anpd_status gemm_plain_enqueue(const ClPlan& p, const unsigned char* W, const bf16* a_hi, const bf16* a_lo, int rows, float* part, int ld_part,
                                cudaStream_t st, Profiler* prof) {
@@ -1411,7 +1425,7 @@ anpd_status forward_enqueue(anpd_model* m, anpd_kv* kv, int rows, int max_pos, b
     rows = kv->batch * ANPD_ROWS;
     ANPD_TRY(gemm_enqueue(m, kv, GK_LM, 0, rows, &segs, &seg_min));
     LAUNCH(pf, st, KC_OTHER, 0,
-           (launch_k(argmax_partial_kernel, dim3(ws.amax_blocks, rows), 256, 0, st, ws.part, seg_min, sstride(GK_LM), ws.ld[GK_LM], V,
+           (launch_k(argmax_partial_kernel, dim3(ws.amax_blocks, rows), 256, 0, st, ws.part, segs, seg_min, sstride(GK_LM), ws.ld[GK_LM], V,
                                                                              want_logits ? ws.logits : nullptr, ws.amax_val,
                                                                              ws.amax_idx, ws.amax_blocks)));
     CUDA_TRY(cudaGetLastError());

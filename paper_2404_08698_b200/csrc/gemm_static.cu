@@ -103,7 +103,7 @@ extern "C" anpd_status anpd_gemm_static(const uint16_t* w_bf16_dev, int N, int K
     plan.N = N; plan.K = K; plan.m_tiles = m_tiles; plan.k_blocks = k_blocks;
     plan.grid = (int)(total < sms ? total : sms);
     plan.max_count = (int)((total + plan.grid - 1) / plan.grid);
-    plan.max_segs = 0;
+    plan.max_segs = plan.min_segs = 0;
     plan.d_first_cta = (int*)(scratch + OFF_FIRST);
     plan.d_seg_count = (int*)(scratch + OFF_SEGS);
     if ((long long)plan.max_count * plan.grid > MAX_SLOTS) return ANPD_ERR_CAPACITY;

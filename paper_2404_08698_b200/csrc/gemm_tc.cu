@@ -44,31 +44,40 @@ struct GemmArgs {
     size_t seg_stride;      // elements between segment slabs
     int ld_part;
     int N, rows;            // valid output features / valid rows (stores are clipped to these)
-    int NB;                 // MMA N: rows padded to a multiple of 16
+    int NB;                 // MMA N: rows padded to a multiple of 16 (operand image: the rows themselves)
     int m_tiles, k_blocks;
     int stages;
     int tmem_cols;          // power of two >= 4 * NB (two accumulators of 2 * NB columns: W x hi and W x lo side by side)
     const int* first_cta;   // [m_tiles] CTA that owns the first k-block of a tile
+    const unsigned char* act;   // MODEL: the operand image
+    ClPlan plan;            // MODEL: the weights' storage
     int* err;
 };
 
+constexpr int TILE_GROUPS = TILE_M / 8;
+// A tile's groups as runs inside one segment of the storage each
+struct TileRuns { const unsigned char* src[TILE_GROUPS]; uint32_t step[TILE_GROUPS], bytes[TILE_GROUPS]; int n; };
+
+// MODEL: the weights in the model's storage (see ClPlan; a tile is 16 groups in storage order) and the activations an operand
+// image; otherwise blocks of 16 KB in the order the CTAs read them and row-major activations.
+template <bool MODEL>
 __global__ void __launch_bounds__(GEMM_THREADS, 1)
-gemm_tc_kernel(const bf16* __restrict__ w_blocks, const __grid_constant__ CUtensorMap map_hi,
-               const __grid_constant__ CUtensorMap map_lo, const GemmArgs g) {
+gemm_tc_kernel(const unsigned char* __restrict__ w_blocks, const __grid_constant__ CUtensorMap map_hi,
+               const __grid_constant__ CUtensorMap map_lo, const __grid_constant__ GemmArgs g) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     __shared__ uint64_t bar_full[MAX_STAGES], bar_empty[MAX_STAGES], bar_acc_full[2], bar_acc_empty[2];
     __shared__ uint32_t tmem_base_slot;
     __shared__ int abort_flag;
+    __shared__ TileRuns runs;                               // the producer's
 
     // the swizzled tiles need 1024-byte alignment in the shared address space
-    pdl_trigger();
     unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
-    const int stage_bytes = A_BYTES + 2 * g.NB * 128;
+    const int act_bytes = 2 * g.NB * 128, stage_bytes = A_BYTES + act_bytes;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
     // this CTA's contiguous range of (m_tile, k_block) pairs
     const long long total = (long long)g.m_tiles * g.k_blocks;
-    const long long lo = (long long)blockIdx.x * total / gridDim.x, hi = (long long)(blockIdx.x + 1) * total / gridDim.x;
+    const int lo = (int)(blockIdx.x * total / gridDim.x), hi = (int)((blockIdx.x + 1) * total / gridDim.x);
 
     if (threadIdx.x == 0) {
         abort_flag = 0;
@@ -84,117 +93,130 @@ gemm_tc_kernel(const bf16* __restrict__ w_blocks, const __grid_constant__ CUtens
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    // Only now may the next kernels start beside this one: their tensor-memory allocations must not come before this CTA's.
+    pdl_trigger();
     const uint32_t tmem_base = *((volatile uint32_t*)&tmem_base_slot);
     volatile int* abortp = &abort_flag;
 
     if (warp == 0) {
         // ---------------- producer ----------------
-        if (lane == 0) {
+        if (elect_one()) {
             const uint64_t pol_w = policy_evict_first(), pol_a = policy_evict_last();
-            int stage = 0;
-            uint32_t phase = 0;
-            long long issued = 0;
-            bool ok = true;
+            int tile = lo / g.k_blocks, kb = lo - tile * g.k_blocks;                    // the next block to load; advanced without divisions
+            int akb = kb;                                   // k-block of the next activation load
+            uint32_t tile_bytes = A_BYTES;
+            auto enter_tile = [&]() {
+                const int g0 = tile * TILE_GROUPS, g1 = min(g0 + TILE_GROUPS, cl_groups(g.plan));
+                int n = 0;
+                for (int grp = g0; grp < g1; ++n) {
+                    const ClRun r = cl_run(g.plan, grp, 0);
+                    const int len = min(r.run, g1 - grp);
+                    runs.src[n] = w_blocks + r.at;
+                    runs.step[n] = (uint32_t)r.step << 10;
+                    runs.bytes[n] = (uint32_t)len << 10;
+                    grp += len;
+                }
+                runs.n = n;
+                tile_bytes = (uint32_t)(g1 - g0) << 10;     // a last tile of fewer groups: nobody reads the other lanes
+            };
+            if (MODEL) enter_tile();
+            auto weights = [&](int i, unsigned char* dst, uint64_t* bar) {              // the i-th block of this CTA; moves to the next one
+                mbar_expect_tx(bar, tile_bytes + (uint32_t)act_bytes);
+                if (MODEL) {
+                    for (int r = 0; r < runs.n; ++r) {
+                        bulk_load(dst, runs.src[r] + (size_t)kb * runs.step[r], runs.bytes[r], bar, pol_w);
+                        dst += runs.bytes[r];
+                    }
+                    if (++kb == g.k_blocks) { kb = 0; ++tile; if (tile < g.m_tiles) enter_tile(); }
+                } else                                                                  // this CTA's slot of the step's window
+                    bulk_load(dst, w_blocks + ((size_t)i * gridDim.x + blockIdx.x) * A_BYTES, A_BYTES, bar, pol_w);
+            };
+            auto activations = [&](unsigned char* dst, uint64_t* bar) {
+                if (MODEL) bulk_load(dst, g.act + (size_t)akb * act_bytes, (uint32_t)act_bytes, bar, pol_a);
+                else {
+                    tma_load_2d(dst, &map_hi, akb * TILE_K, 0, bar, pol_a);
+                    tma_load_2d(dst + g.NB * 128, &map_lo, akb * TILE_K, 0, bar, pol_a);
+                }
+                if (++akb == g.k_blocks) akb = 0;
+            };
             // The weights do not depend on the previous kernel: request the first ring of weight tiles at
             // once, and only then wait for the kernel that produces this GEMM's activations.
-            const long long ahead = min((long long)g.stages, hi - lo);
-            for (long long i = 0; i < ahead; ++i) {
-                unsigned char* sa = smem + (size_t)i * stage_bytes;
-                mbar_expect_tx(&bar_full[i], (uint32_t)stage_bytes);
-                bulk_load(sa, w_blocks + (size_t)(i * gridDim.x + blockIdx.x) * (TILE_M * TILE_K), A_BYTES, &bar_full[i], pol_w);
-            }
+            const int ahead = min(g.stages, hi - lo);
+            for (int i = 0; i < ahead; ++i) weights(i, smem + (size_t)i * stage_bytes, &bar_full[i]);
             pdl_wait();
-            int kb = (int)(lo % g.k_blocks);            // k-block of the next activation load; advanced without divisions
-            for (long long i = 0; i < ahead; ++i) {
-                unsigned char* sa = smem + (size_t)i * stage_bytes;
-                tma_load_2d(sa + A_BYTES, &map_hi, kb * TILE_K, 0, &bar_full[i], pol_a);
-                tma_load_2d(sa + A_BYTES + g.NB * 128, &map_lo, kb * TILE_K, 0, &bar_full[i], pol_a);
-                if (++kb == g.k_blocks) kb = 0;
-            }
-            issued = ahead;
-            stage = (int)(ahead % g.stages);
-            phase = (ahead == g.stages) ? 1u : 0u;
-            for (long long blk = lo + ahead; blk < hi && ok; ++blk) {
+            for (int i = 0; i < ahead; ++i) activations(smem + (size_t)i * stage_bytes + A_BYTES, &bar_full[i]);
+            int issued = ahead, stage = ahead % g.stages;
+            uint32_t phase = (ahead == g.stages) ? 1u : 0u;
+            bool ok = true;
+            for (; issued < hi - lo; ++issued) {
                 ok = mbar_wait(&bar_empty[stage], phase ^ 1u, abortp);
                 if (!ok) break;
                 unsigned char* sa = smem + (size_t)stage * stage_bytes;
-                mbar_expect_tx(&bar_full[stage], (uint32_t)stage_bytes);
-                bulk_load(sa, w_blocks + (size_t)((blk - lo) * gridDim.x + blockIdx.x) * (TILE_M * TILE_K), A_BYTES, &bar_full[stage], pol_w);   // this CTA's slot of the step's window
-                tma_load_2d(sa + A_BYTES, &map_hi, kb * TILE_K, 0, &bar_full[stage], pol_a);
-                tma_load_2d(sa + A_BYTES + g.NB * 128, &map_lo, kb * TILE_K, 0, &bar_full[stage], pol_a);
-                if (++kb == g.k_blocks) kb = 0;
-                ++issued;
+                weights(issued, sa, &bar_full[stage]);
+                activations(sa + A_BYTES, &bar_full[stage]);
                 if (++stage == g.stages) { stage = 0; phase ^= 1u; }
             }
             if (!ok) {
                 // gave up: let every copy already issued land before the CTA may exit
-                const long long n = issued < g.stages ? issued : g.stages;
-                for (long long i = 0; i < n; ++i) {
-                    const long long idx = issued - 1 - i;
-                    const int s = (int)(idx % g.stages);
-                    const uint32_t ph = (uint32_t)((idx / g.stages) & 1);
-                    for (unsigned spin = 0; spin < WAIT_LIMIT && !mbar_try_wait(&bar_full[s], ph); ++spin) {}
-                }
+                for (int i = max(0, issued - g.stages); i < issued; ++i)
+                    for (unsigned spin = 0; spin < WAIT_LIMIT && !mbar_try_wait(&bar_full[i % g.stages], (uint32_t)((i / g.stages) & 1)); ++spin) {}
             }
         }
+        __syncwarp();
     } else if (warp == 1) {
         // ---------------- MMA issuer ----------------
-        pdl_wait();
-        if (lane == 0) {
+        if (elect_one()) {
             // fp32 accumulate, bf16 x bf16, both operands K-major, N = 2 * NB (hi rows then lo rows), M = 128
             const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)((2 * g.NB) >> 3) << 17) | ((uint32_t)(TILE_M >> 4) << 24);
-            int stage = 0;
-            uint32_t phase = 0;
-            int seg = 0;
+            const uint32_t w0 = smem_desc_lo(smem_u32(smem)), step = (uint32_t)stage_bytes >> 4, a_off = (uint32_t)A_BYTES >> 4;
+            const uint32_t full0 = smem_u32(&bar_full[0]), empty_off = smem_u32(&bar_empty[0]) - full0, full_end = full0 + 8u * (uint32_t)g.stages;
+            uint32_t full = full0, phase = 0, w = w0;
+            int seg = 0, left = hi - lo, n = min(left, (lo / g.k_blocks + 1) * g.k_blocks - lo);
             bool ok = true;
-            long long blk = lo;
-            while (blk < hi && ok) {
-                const int tile = (int)(blk / g.k_blocks);
-                const long long seg_end = min(hi, (long long)(tile + 1) * g.k_blocks);
+            while (left > 0 && ok) {
                 const int buf = seg & 1;
                 ok = mbar_wait(&bar_acc_empty[buf], (uint32_t)(((seg >> 1) & 1) ^ 1), abortp);
                 if (!ok) break;
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_base + (uint32_t)(buf * 2 * g.NB);
                 uint32_t acc = 0;
-                for (; blk < seg_end; ++blk) {
-                    ok = mbar_wait(&bar_full[stage], phase, abortp);
+                for (int i = n; i > 0; --i) {
+                    ok = mbar_wait_at(full, phase, abortp);
                     if (!ok) break;
                     tc_fence_after();
-                    const uint32_t sa = smem_u32(smem + (size_t)stage * stage_bytes);
                     // the lo rows follow the hi rows in the stage, so one descriptor spans both: one MMA reads the
                     // weight slice from shared memory once and yields W x hi in columns [0, NB) and W x lo in [NB, 2 NB)
-                    const uint64_t da = make_smem_desc(sa), db = make_smem_desc(sa + A_BYTES);
-#pragma unroll
-                    for (int k16 = 0; k16 < TILE_K / 16; ++k16) {
-                        const uint64_t adv = (uint64_t)(k16 * 32 >> 4);     // 16 bf16 = 32 bytes along K inside the swizzle row
-                        tc_mma_bf16(d_tmem, da + adv, db + adv, idesc, acc);
-                        acc = 1;
-                    }
-                    tc_commit(&bar_empty[stage]);        // frees the stage once these MMAs have read it
-                    if (++stage == g.stages) { stage = 0; phase ^= 1u; }
+                    tc_mma_k64(d_tmem, w, w + a_off, idesc, acc);
+                    acc = 1;
+                    tc_commit_at(full + empty_off);      // frees the stage once these MMAs have read it
+                    w += step;
+                    full += 8u;
+                    if (full == full_end) { full = full0; phase ^= 1u; w = w0; }
                 }
                 if (!ok) break;
                 tc_commit(&bar_acc_full[buf]);           // accumulator complete
                 ++seg;
+                left -= n;
+                n = min(left, g.k_blocks);
             }
         }
+        __syncwarp();
     } else {
         // ---------------- epilogue: TMEM -> registers -> partial sums in global memory ----------------
         pdl_wait();                                       // the partial-sum buffer may still be read by the previous kernel
         const int quad = warp & 3;                        // a warp may only touch TMEM lanes 32*(warp%4)..+31
         int seg = 0;
         bool ok = true;
-        long long blk = lo;
+        int blk = lo;
         while (blk < hi && ok) {
-            const int tile = (int)(blk / g.k_blocks);
-            const long long seg_end = min(hi, (long long)(tile + 1) * g.k_blocks);
+            const int tile = blk / g.k_blocks, seg_end = min(hi, (tile + 1) * g.k_blocks);
             const int buf = seg & 1;
             ok = mbar_wait(&bar_acc_full[buf], (uint32_t)((seg >> 1) & 1), abortp);
             if (!ok) break;
             tc_fence_after();
             const int ordinal = (int)blockIdx.x - g.first_cta[tile];      // position of this segment in the tile's K order
-            const int n = tile * TILE_M + quad * 32 + lane;
+            int n = tile * TILE_M + quad * 32 + lane;
+            if (MODEL) n = n < cl_groups(g.plan) * 8 ? cl_feature(g.plan, n) : g.N;
             float* out = g.part + (size_t)ordinal * g.seg_stride + n;
             for (int c0 = 0; c0 < g.NB; c0 += 16) {
                 float v[16], w[16];
@@ -306,7 +328,8 @@ void gemm_make_plan(GemmPlan* p, int N, int K, int num_sms) {
             p->seg_count[t] += 1;
         }
     }
-    for (int t = 0; t < p->m_tiles; ++t) p->max_segs = std::max(p->max_segs, p->seg_count[t]);
+    p->min_segs = p->seg_count[0];
+    for (int t = 0; t < p->m_tiles; ++t) { p->max_segs = std::max(p->max_segs, p->seg_count[t]); p->min_segs = std::min(p->min_segs, p->seg_count[t]); }
     p->d_first_cta = nullptr;
     p->d_seg_count = nullptr;
 }
@@ -320,25 +343,39 @@ int gemm_smem_bytes(int NB, int* stages_out) {
     return stages * stage_bytes + 1024;
 }
 
-anpd_status gemm_tc_enqueue(const GemmPlan& plan, const bf16* w_blocks, const CUtensorMap& map_hi, const CUtensorMap& map_lo,
-                            int rows, int NB, float* part, size_t seg_stride, int ld_part, int* err, cudaStream_t st,
-                            Profiler* prof) {
+template <bool MODEL>
+static anpd_status launch_tc(const GemmPlan& plan, const void* w, const CUtensorMap& map_hi, const CUtensorMap& map_lo, GemmArgs& g,
+                             float* part, size_t seg_stride, int ld_part, int* err, cudaStream_t st, Profiler* prof) {
     static bool attr_set[64] = {false};
     if (first_call_on_device(attr_set)) {
-        CUDA_TRY(cudaFuncSetAttribute(gemm_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
+        CUDA_TRY(cudaFuncSetAttribute(gemm_tc_kernel<MODEL>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
     }
-    GemmArgs g;
     g.part = part; g.seg_stride = seg_stride; g.ld_part = ld_part;
-    g.N = plan.N; g.rows = rows; g.NB = NB;
+    g.N = plan.N;
     g.m_tiles = plan.m_tiles; g.k_blocks = plan.k_blocks;
-    const int smem = gemm_smem_bytes(NB, &g.stages);
-    int cols = 32;
-    while (cols < 4 * NB) cols <<= 1;
-    g.tmem_cols = cols;
+    const int smem = gemm_smem_bytes(g.NB, &g.stages);
+    g.tmem_cols = 32;
+    while (g.tmem_cols < 4 * g.NB) g.tmem_cols <<= 1;
     g.first_cta = plan.d_first_cta;
     g.err = err;
     LAUNCH(prof, st, KC_GEMM, 2.0 * (double)plan.N * (double)plan.K,
-           (launch_k(gemm_tc_kernel, plan.grid, GEMM_THREADS, smem, st, w_blocks, map_hi, map_lo, g)));
+           (launch_k(gemm_tc_kernel<MODEL>, plan.grid, GEMM_THREADS, smem, st, (const unsigned char*)w, map_hi, map_lo, g)));
     CUDA_TRY(cudaGetLastError());
     return ANPD_OK;
+}
+
+anpd_status gemm_tc_enqueue(const GemmPlan& plan, const bf16* w_blocks, const CUtensorMap& map_hi, const CUtensorMap& map_lo,
+                            int rows, int NB, float* part, size_t seg_stride, int ld_part, int* err, cudaStream_t st,
+                            Profiler* prof) {
+    GemmArgs g{};
+    g.rows = rows; g.NB = NB;
+    return launch_tc<false>(plan, w_blocks, map_hi, map_lo, g, part, seg_stride, ld_part, err, st, prof);
+}
+
+anpd_status gemm_tc_model_enqueue(const GemmPlan& plan, const ClPlan& storage, const unsigned char* w, const unsigned char* act, int rows, float* part,
+                                  size_t seg_stride, int ld_part, int* err, cudaStream_t st, Profiler* prof) {
+    GemmArgs g{};
+    g.rows = rows; g.NB = rows; g.act = act; g.plan = storage;
+    const CUtensorMap none{};
+    return launch_tc<true>(plan, w, none, none, g, part, seg_stride, ld_part, err, st, prof);
 }

@@ -333,7 +333,7 @@ constexpr int PREFILL_ROWS_MAX = 2048; // most rows of one prompt pass (sizes th
 // SM count only): tile t is started by CTA first_cta[t] and covered by seg_count[t] consecutive CTAs,
 // each of which leaves one partial sum; consumers add them in that order.
 struct GemmPlan {
-    int N, K, m_tiles, k_blocks, grid, max_segs;
+    int N, K, m_tiles, k_blocks, grid, max_segs, min_segs;
     int max_count;                    // most (tile, k-block) blocks any CTA owns
     std::vector<int> first_cta, seg_count;
     int* d_first_cta;
@@ -572,6 +572,12 @@ anpd_status gemm_retile_enqueue(const GemmPlan& p, const void* src, bool src_is_
 anpd_status gemm_tc_enqueue(const GemmPlan& plan, const __nv_bfloat16* w_blocks, const CUtensorMap& map_hi, const CUtensorMap& map_lo,
                             int rows, int NB, float* part, size_t seg_stride, int ld_part, int* err, cudaStream_t st,
                             Profiler* prof);
+// The same kernel on the model's storage and an operand image of `rows` rows (a multiple of 8, 16 to 128):
+// part[segment][row][feature], plan.d_seg_count[storage tile of 128 positions] of them, added by the consumer.
+anpd_status gemm_tc_model_enqueue(const GemmPlan& plan, const ClPlan& storage, const unsigned char* w, const unsigned char* act, int rows, float* part,
+                                  size_t seg_stride, int ld_part, int* err, cudaStream_t st, Profiler* prof);
+bool tc_model_fits(const GemmPlan& plan, int rows);
+const GemmPlan* tc_model_plan(const anpd_model* m, int kind, int rows);      // its cut, null where the cluster form is the better one
 // gemm_pf.cu: the projection of a prompt pass (many rows, bound by the tensor cores): out[row][n], complete sums
 // out[part][row][n]: partial sums per output, seg_stride elements apart.  How the output tiles (feature pair x row tile, row
 // tile fastest) are cut along K: tiles [0, tail_from) into `ksplit` equal parts each, tiles [tail_from, end) - those that would
