@@ -1168,7 +1168,7 @@ static anpd_status debug_gemm_step(const uint16_t* w_bf16, int N, int K, const f
         } else if (sweep) {
             ANPD_TRY(gemm_tc_model_enqueue(tc, plan, dW, dimg, rows, dout, (size_t)rows * N, N, derr, 0, nullptr));
         } else {
-            ANPD_TRY(cl_partial_enqueue(plan, dW, dimg, rows, dout, (size_t)rows * N, N, nullptr, nullptr, 0, 0, derr, 0, nullptr));
+            ANPD_TRY(cl_partial_enqueue(plan, dW, dimg, rows, dout, (size_t)rows * N, N, derr, 0, nullptr));
         }
         CUDA_TRY(cudaDeviceSynchronize());
         int err = 0;

@@ -33,6 +33,7 @@ namespace {
 
 using namespace tc;
 
+constexpr int AD_MAX_CLUSTER = 4;
 constexpr int AD_KEYS = 16;              // keys per block
 constexpr int AD_MAX_CHUNKS = 6;
 constexpr int AD_SMEM_PAIR = 111 * 1024; // two CTAs share an SM: another one of these, or one of the projection before or after
@@ -45,7 +46,6 @@ template <int HD, int G> struct AdCfg {
     static constexpr int WARPS = 8;                          // compute warps, each with 16 keys of a page; one more loads
     static constexpr int COMPUTE = 32 * WARPS, THREADS = COMPUTE + 32;
     static constexpr int REGS = 112;
-    static constexpr int C_MAX = 4;                          // CTAs of a cluster
     static constexpr int OP = HD + 4;                        // padded row
     static constexpr int QP = HD * 2 + 16;                   // bytes per staged query row
     static constexpr int QROWS = STACK ? 16 : 32;
@@ -375,6 +375,18 @@ __global__ void __launch_bounds__((AdCfg<HD, G>::THREADS)) __maxnreg__((AdCfg<HD
     }
 }
 
+// CTAs per head, and clusters that share a kv head (see AdArgs)
+int ad_cluster(const anpd_model* m, int heads) {
+    const int resident = m->num_sms * 7 / 8;
+    int cluster = AD_MAX_CLUSTER;
+    while (cluster > 1 && heads * cluster > resident) cluster /= 2;
+    return cluster;
+}
+int ad_split(const anpd_model_config& c) {
+    const int group = c.n_q_heads / c.n_kv_heads;
+    return c.head_dim == 64 && group > 1 ? group / 2 : group;
+}
+
 template <int HD, int G>
 anpd_status launch_attn_dec(anpd_model* m, anpd_kv* kv, AdArgs& a) {
     typedef AdCfg<HD, G> Cfg;
@@ -385,9 +397,7 @@ anpd_status launch_attn_dec(anpd_model* m, anpd_kv* kv, AdArgs& a) {
     // step with four CTAs per head, 1072 with two; at 4000 tokens 1255 and 1223; eight 1.1B sequences 1337 and 1230 (two, one); four
     // 7B sequences of 600 tokens (8 layers) 915 and 880, of 2000 tokens 1088 and 1040.  Never more than four: sixteen clusters of
     // eight crowd the O projection out (1.1B at 512 keys: 894, with four 800).
-    const int heads = a.Hkv * a.split * kv->batch, resident = m->num_sms * 7 / 8;
-    int cluster = Cfg::C_MAX;
-    while (cluster > 1 && heads * cluster > resident) cluster /= 2;
+    const int cluster = ad_cluster(m, a.Hkv * a.split * kv->batch);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(cluster, a.Hkv * a.split, kv->batch); cfg.blockDim = dim3(Cfg::THREADS); cfg.dynamicSmemBytes = Cfg::SMEM; cfg.stream = m->stream;
     cudaLaunchAttribute attr[2];
@@ -404,6 +414,11 @@ anpd_status launch_attn_dec(anpd_model* m, anpd_kv* kv, AdArgs& a) {
 
 }  // namespace
 
+int attn_dec_ctas(const anpd_model* m) {
+    const int heads = m->cfg.n_kv_heads * ad_split(m->cfg);
+    return heads * ad_cluster(m, heads);
+}
+
 anpd_status attn_dec_enqueue(anpd_model* m, anpd_kv* kv, int layer, bool tree) {
     const anpd_model_config& c = m->cfg;
     Workspace& ws = kv->ws;
@@ -414,15 +429,11 @@ anpd_status attn_dec_enqueue(anpd_model* m, anpd_kv* kv, int layer, bool tree) {
     a.pages_per_seq = kv->pages_per_seq; a.Hkv = c.n_kv_heads; a.rows = kv->batch * ANPD_ROWS;
     a.layer_page0 = layer * kv->total_pages;
     a.img = ws.ci_ao; a.err = ws.gemm_err;
+    a.split = ad_split(c);
     switch (c.head_dim * 16 + c.n_q_heads / c.n_kv_heads) {
-        case 64 * 16 + 1: a.split = 1; return launch_attn_dec<64, 1>(m, kv, a);
-        case 64 * 16 + 2: a.split = 1; return launch_attn_dec<64, 2>(m, kv, a);
-        case 64 * 16 + 4: a.split = 2; return launch_attn_dec<64, 2>(m, kv, a);
-        case 64 * 16 + 8: a.split = 4; return launch_attn_dec<64, 2>(m, kv, a);
-        case 128 * 16 + 1: a.split = 1; return launch_attn_dec<128, 1>(m, kv, a);
-        case 128 * 16 + 2: a.split = 2; return launch_attn_dec<128, 1>(m, kv, a);
-        case 128 * 16 + 4: a.split = 4; return launch_attn_dec<128, 1>(m, kv, a);
-        case 128 * 16 + 8: a.split = 8; return launch_attn_dec<128, 1>(m, kv, a);
+        case 64 * 16 + 1: return launch_attn_dec<64, 1>(m, kv, a);
+        case 64 * 16 + 2: case 64 * 16 + 4: case 64 * 16 + 8: return launch_attn_dec<64, 2>(m, kv, a);
+        case 128 * 16 + 1: case 128 * 16 + 2: case 128 * 16 + 4: case 128 * 16 + 8: return launch_attn_dec<128, 1>(m, kv, a);
     }
     return ANPD_ERR_ARG;
 }

@@ -1097,13 +1097,8 @@ anpd_status gemm_enqueue(anpd_model* m, anpd_kv* kv, int kind, int layer, int ro
         }
         *seg_count_out = nullptr;
         *seg_min_out = CL_CTAS;
-        // the projection after this one, whose first weights are fetched into L2 under the small kernels between the two
-        const bool last = layer + 1 == m->cfg.n_layers;
-        const int next = kind == GK_QKV ? GK_O : kind == GK_O ? GK_GU : kind == GK_GU ? GK_DOWN : last ? GK_LM : GK_QKV;
-        const LayerW& lw = m->layers[layer];
-        const unsigned char* next_w = kind == GK_QKV ? lw.wo : kind == GK_O ? lw.wgu : kind == GK_GU ? lw.wd : last ? m->lm_head : m->layers[layer + 1].wqkv;
-        return cl_partial_enqueue(plan, W, act, rows, ws.part, (size_t)rows * ws.ld[kind], ws.ld[kind], kind == GK_LM || (next == GK_LM && rows != kv->batch * ANPD_ROWS) ? nullptr : &m->cl[next], next_w,
-                                  CL_LEAD, kind == GK_QKV && layer == 0 ? 0 : CL_LEAD, ws.gemm_err, m->stream, &m->prof);
+        // (no L2 prefetch for the projection after this one: two sequences, 13B, 8 layers 1103 -> 1066 us without, 7B 754 -> 746, larger batches equal)
+        return cl_partial_enqueue(plan, W, act, rows, ws.part, (size_t)rows * ws.ld[kind], ws.ld[kind], ws.gemm_err, m->stream, &m->prof);
     }
     // a prompt pass: complete sums, or several per output
     const int m_tiles = m->plan[kind].m_tiles;
@@ -1269,12 +1264,12 @@ static anpd_status forward_rr_enqueue(anpd_model* m, anpd_kv* kv, int max_pos, b
 }
 
 // The vocabulary projection of the 8 rows whose operand image is ws.ci_h, and its argmax candidates.
-static anpd_status lm_head_cl_enqueue(anpd_model* m, anpd_kv* kv, const float* ss, int n_parts, bool want_logits, unsigned own_lead = 0) {
+static anpd_status lm_head_cl_enqueue(anpd_model* m, anpd_kv* kv, const float* ss, int n_parts, bool want_logits, bool ahead = false, unsigned own_lead = 0) {
     const anpd_model_config& c = m->cfg;
     Workspace& ws = kv->ws;
     ClEpilogue lm;
     lm.ss_in = ss; lm.n_parts = n_parts; lm.inv_d = 1.0f / (float)c.d_model; lm.eps = c.rms_eps;
-    lm.own_lead = own_lead;
+    lm.ahead = ahead; lm.own_lead = own_lead;
     lm.out = want_logits ? ws.logits : nullptr; lm.amax_val = ws.amax_val_cl; lm.amax_idx = ws.amax_idx_cl;
     ANPD_TRY(cl_enqueue(m->cl[GK_LM], m->lm_head, ws.ci_h, lm, ws.gemm_err, m->stream, &m->prof));
     ws.amax_nblk = cl_parts(m->cl[GK_LM]);
@@ -1295,14 +1290,17 @@ static anpd_status forward_cl_enqueue(anpd_model* m, anpd_kv* kv, int max_pos, b
     LAUNCH(pf, st, KC_OTHER, 0, (launch_k(embed_cl_kernel, rows, NORM_THREADS, 0, st, m->embed, ws.row_tok, m->layers[0].attn_norm, d, ws.x,
                                           ws.ci_h, rows, ws.ss_cl_a)));
     int parts_a = 1;                                   // sums of squares behind ci_h: one after the embedding, then the down projection's
-    // Each projection brings the first weights of the next one into L2 while its own tail and the hand-over leave HBM idle.
-    auto chain = [&](ClEpilogue& e, unsigned own, int next, const unsigned char* w) {
-        e.own_lead = own; e.next = &m->cl[next]; e.next_w = w; e.next_lead = CL_LEAD;
-    };
-    // Where the O projection's weights fit its first ring of copies, HBM has nothing left to read when the gate-up CTAs start
-    // beside it: these then fetch more of their own weights at once (1.1B: 885 -> 853 us per step; the 7B model, whose O
-    // projection still streams at that point, lost 20 of 2850 us by the same).
+    // A projection brings the first weights of the next one into L2 while its own tail and the hand-over leave HBM idle, and runs ahead
+    // of its own copies there, where that pays: where the attention leaves half of the SMs to the projections around it and the
+    // gate-up weights are more than these take at once (1.1B, 64 attention CTAs: 803 -> 777 us per step).  Elsewhere the same traffic
+    // stands in front of the activations and of the other CTAs' last copies; without it, 7B (16 layers) at 77 keys 1370 -> 1348 us, at
+    // 1536 1437 -> 1416, 13B (8 layers) 1040 -> 991, 1.1B's widths with 32 kv heads (12 layers) 486 -> 479, 1024 wide (16 layers) 457 -> 450.
     const bool o_in_ring = cl_storage_bytes(m->cl[GK_O]) <= CL_RING_SHARE * CL_CTAS * m->cl[GK_O].ncl;
+    const bool lead = o_in_ring && kv->attn_dec && 2 * attn_dec_ctas(m) <= m->num_sms && cl_storage_bytes(m->cl[GK_GU]) > (size_t)2 * CL_BURST * CL_CTAS * m->cl[GK_GU].ncl;
+    auto chain = [&](ClEpilogue& e, unsigned own, int next, const unsigned char* w) {
+        if (!lead) return;
+        e.ahead = true; e.own_lead = own; e.next = &m->cl[next]; e.next_w = w; e.next_lead = CL_LEAD;
+    };
     for (int l = 0; l < c.n_layers; ++l) {
         const LayerW& w = m->layers[l];
         ClEpilogue q;
@@ -1323,7 +1321,7 @@ static anpd_status forward_cl_enqueue(anpd_model* m, anpd_kv* kv, int max_pos, b
         ClEpilogue gu;
         gu.ss_in = ws.ss_cl_b; gu.n_parts = cl_parts(m->cl[GK_O]); gu.inv_d = 1.0f / (float)d; gu.eps = c.rms_eps; gu.act_out = ws.ci_act;
         chain(gu, CL_LEAD, GK_DOWN, w.wd);
-        gu.own_burst = o_in_ring ? CL_BURST : 0;
+        gu.own_burst = lead ? CL_BURST : 0;               // the O projection's weights are in its ring: HBM has nothing else to read (885 -> 853 us)
         ANPD_TRY(cl_enqueue(m->cl[GK_GU], w.wgu, ws.ci_h2, gu, ws.gemm_err, st, pf));
         ClEpilogue dn;
         dn.x = ws.x; dn.gain = (l + 1 < c.n_layers) ? m->layers[l + 1].attn_norm : m->final_norm; dn.ss_out = ws.ss_cl_a; dn.d = d;
@@ -1333,7 +1331,7 @@ static anpd_status forward_cl_enqueue(anpd_model* m, anpd_kv* kv, int max_pos, b
         ANPD_TRY(cl_enqueue(m->cl[GK_DOWN], w.wd, ws.ci_act, dn, ws.gemm_err, st, pf));
         parts_a = cl_parts(m->cl[GK_DOWN]);
     }
-    ANPD_TRY(lm_head_cl_enqueue(m, kv, ws.ss_cl_a, parts_a, want_logits, CL_LEAD));
+    ANPD_TRY(lm_head_cl_enqueue(m, kv, ws.ss_cl_a, parts_a, want_logits, lead, CL_LEAD));
     CUDA_TRY(cudaGetLastError());
     return ANPD_OK;
 }

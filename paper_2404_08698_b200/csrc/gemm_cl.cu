@@ -15,7 +15,7 @@
 // four projections alone: 7B 405 MB in 76 us (copy rate of the device: 62 us), 1.1B 88 MB in 32 us (13.5 us).
 //
 // Roles.  A weight thread keeps a ring of copies in flight; the first ring goes out at once, while the kernel before is still
-// running (weights depend on nothing), and it runs ahead of the ring with L2 prefetches.  An activation thread follows behind the
+// running (weights depend on nothing), and, where that pays, it runs ahead of the ring with L2 prefetches.  An activation thread follows behind the
 // dependency wait.  An MMA thread multiplies tiles of up to 128 features with the rows of the step (N operand: hi terms, then lo
 // terms of the activations) into tensor memory.  Four warps read the accumulators and push each partial sum to the CTA that
 // finishes its feature (st.async: data and arrival in one), eight add the parts in CTA order and apply the epilogue.
@@ -39,7 +39,7 @@ namespace {
 using namespace tc;
 
 // warp 0: weights, warp 1: MMA issuer + tensor-memory owner, warp 2: activations, warps from 4 on: exchange and epilogue
-constexpr int cl_threads(int R) { return R ? 384 : 256; }
+__host__ __device__ constexpr int cl_threads(int R) { return R ? 384 : 256; }
 constexpr int CL_MAX_STAGES = 16;
 constexpr int CL_MAX_ACT = 8;
 constexpr int CL_MAX_TILES = 8;          // tiles of 128 features a pass may hold
@@ -48,6 +48,12 @@ constexpr int CL_STAGE_MAX = 16384;      // one copy: at most 16 groups of 8 fea
 constexpr int CL_SMEM_PAIR = 112 * 1024; // two CTAs of this size share an SM
 constexpr int CL_SMEM_MAX = 216 * 1024;
 constexpr int CL_RING_BYTES = 8 * CL_STAGE_MAX;      // copies in flight per SM
+// A CTA that has its SM for itself starts as the one before leaves, when the activations are about to be ready: its first ring, 128 KB
+// requested at once, would stand in front of them (2.3 us at the device's rate).  So it requests a few stages and the others once the
+// first activations are on their way, or after a while, where the kernel before still has its tail to run.  7B, 16 layers: 77 keys
+// 1339 -> 1321 us per step, 1536 keys 1412 -> 1391 (two stages 1326 and 1395, four 1333 and 1400).
+constexpr int CL_FIRST = 3;
+constexpr int CL_HOLD = 1500;            // cycles
 constexpr int CL_ERR_TIMEOUT = 207;
 
 struct ClArgs {
@@ -56,10 +62,10 @@ struct ClArgs {
     int kb, gpu, n_units, ncl;
     int seg, next_seg;                   // segments of the storage: ncl or 1
     int rows, passes, copies, two, kps, stages, stage_bytes, akb, act_slots, tmem_cols, acc_bufs, acc_cols;
-    int f_own_max;
+    int f_own_max, first;                // first: stages requested ahead of the activations
     // the projection after this one: its storage and cut, and how many bytes per CTA are fetched into L2 ahead (own: already done)
     const unsigned char* next_w;
-    int next_kb, next_gpu, next_units, next_passes;
+    int next_kb, next_gpu, next_units;
     unsigned own_lead, own_burst, next_lead;
     // RMSNorm of the input
     const float* ss_in; int n_parts; float inv_d, eps;
@@ -145,14 +151,15 @@ __device__ __forceinline__ void split2(float a, float b, uint32_t& hi, uint32_t&
     lo = (uint32_t)__bfloat16_as_ushort(la) | ((uint32_t)__bfloat16_as_ushort(lb) << 16);
 }
 
-// R: 8 = a step of one sequence (8 rows, one pass, one chunk); 0 = rows, passes and chunks from the arguments
-template <int EPI, int R>
+// R: 8 = a step of one sequence (8 rows, one pass, one chunk); 0 = rows, passes and chunks from the arguments.  LEAD: runs ahead in L2
+template <int EPI, int R, bool LEAD>
 __global__ void __launch_bounds__(cl_threads(R), 1) gemm_cl_kernel(const __grid_constant__ ClArgs g) {
+    constexpr bool LATE = R && !LEAD;                  // its CTAs start late (see CL_FIRST)
     extern __shared__ __align__(1024) unsigned char cl_smem_raw[];
     __shared__ uint64_t w_full[CL_MAX_STAGES], w_empty[CL_MAX_STAGES], a_full[CL_MAX_ACT], a_empty[CL_MAX_ACT];
     __shared__ uint64_t acc_full[2], acc_empty[2], red_full;
     __shared__ uint32_t tmem_slot;
-    __shared__ int abort_flag, s_issued[2];
+    __shared__ int abort_flag, s_issued[2], s_acts;
     __shared__ float s_rstd[8], s_part[8][8];
     __shared__ int s_pos[8], s_slot[8], s_page[8], s_idx[8][8];
 
@@ -217,19 +224,23 @@ __global__ void __launch_bounds__(cl_threads(R), 1) gemm_cl_kernel(const __grid_
 
     if (warp == 0) {
         if (elect_one()) {
-            abort_flag = 0; s_issued[0] = 0; s_issued[1] = 0;
+            if (!LATE) { abort_flag = 0; s_issued[0] = 0; s_issued[1] = 0; }
             for (int s = 0; s < g.stages; ++s) { mbar_init(&w_full[s], 1); mbar_init(&w_empty[s], 1); }
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             // the weights depend on nothing: the first ring is requested before anything else happens
             w_enter();
-            for (; w_count < g.stages && w_p < passes; ++w_count) w_issue(w_count);
+            for (; w_count < (LATE ? g.first : g.stages) && w_p < passes; ++w_count) w_issue(w_count);
         }
         __syncwarp();
-    } else if (threadIdx.x == 64) {
-        for (int s = 0; s < g.act_slots; ++s) { mbar_init(&a_full[s], 1); mbar_init(&a_empty[s], 1); }
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    } else if (LATE ? warp == 2 : threadIdx.x == 64) {
+        if (!LATE || elect_one()) {
+            if (LATE) { abort_flag = 0; s_issued[0] = 0; s_issued[1] = 0; s_acts = 0; }
+            for (int s = 0; s < g.act_slots; ++s) { mbar_init(&a_full[s], 1); mbar_init(&a_empty[s], 1); }
+            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        }
+        if (LATE) __syncwarp();
     } else if (threadIdx.x == 96) {
         for (int b = 0; b < 2; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], 4); }
         mbar_init(&red_full, 1);
@@ -241,10 +252,14 @@ __global__ void __launch_bounds__(cl_threads(R), 1) gemm_cl_kernel(const __grid_
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     tc_fence_before();
-    __syncthreads();
+    // Where CTAs start late the activation thread goes on at once, past the allocation of tensor memory (7B, 16 layers, 77 keys: 1329 ->
+    // 1323 us; 1.1B, which runs ahead, lost 0.5 %, its batches 4 %).
+    if (!LATE) __syncthreads();
+    else if (warp == 2) asm volatile("bar.arrive 2, %0;" ::"n"(cl_threads(R)) : "memory");
+    else asm volatile("bar.sync 2, %0;" ::"n"(cl_threads(R)) : "memory");
     tc_fence_after();
     // Only now may the next kernel start beside this one: its tensor-memory allocation must not come before this CTA's.
-    pdl_trigger();
+    if (!LATE || warp != 2) pdl_trigger();
     if (R) cluster_arrive();                           // waited for before the first push: every CTA's barriers are initialised then
     const uint32_t tmem_base = *((volatile uint32_t*)&tmem_slot);
     volatile int* abortp = &abort_flag;
@@ -252,29 +267,33 @@ __global__ void __launch_bounds__(cl_threads(R), 1) gemm_cl_kernel(const __grid_
     if (warp == 0) {
         // ---------------- weights ----------------
         if (elect_one()) {
+            if (LATE && g.first < g.stages) {
+                for (const long long t = clock64(); !*(volatile int*)&s_acts && clock64() - t < CL_HOLD;) {}
+                for (; w_count < g.stages && w_p < passes; ++w_count) w_issue(w_count);
+            }
             int stage = 0;
             uint32_t phase = 0;
-            // L2 prefetch: through this CTA's own weights (where one pass reads them in storage order), then its share of the next
-            // projection's first pass, k-block by k-block
-            const unsigned end = passes == 1 ? (unsigned)(Gc * nk) << 10 : 0u, own_piece = g.seg == 1 ? (unsigned)Gc << 10 : end;      // piece: contiguous
+            // One sequence, L2 prefetch: through this CTA's own weights, then its share of the next projection's, k-block by k-block
+            const unsigned end = LEAD ? (unsigned)(Gc * nk) << 10 : 0u, own_piece = g.seg == 1 ? (unsigned)Gc << 10 : end;      // piece: contiguous
             unsigned cur = g.own_lead, left = 0, own_done = 0, nxt_piece = 0, nxt_done = 0;
             const unsigned char *own = nullptr, *nxt = nullptr;
             size_t nxt_step = 0;
-            if (cur < end) {
+            if constexpr (LEAD) if (cur < end) {
                 const unsigned k = cur / own_piece;
                 own_done = cur - k * own_piece;
                 own = g.w + ((size_t)ulo * g.gpu * (g.seg == 1 ? 1 : g.kb) + (size_t)GS * (kb_lo + (int)k)) * 1024;
             }
-            if (g.next_w) {
+            if (LEAD && g.next_w) {
                 const int nu0 = (int)((long long)cluster * g.next_units / g.ncl), nu1 = (int)((long long)(cluster + 1) * g.next_units / g.ncl);
-                const int ng0 = (nu1 - nu0) / g.next_passes * g.next_gpu, ns = (g.next_seg == 1 ? g.next_units : nu1 - nu0) * g.next_gpu;
+                const int ng0 = (nu1 - nu0) * g.next_gpu, ns = (g.next_seg == 1 ? g.next_units : nu1 - nu0) * g.next_gpu;
                 const int k0 = rank * g.next_kb / C, k1 = (rank + 1) * g.next_kb / C;
                 nxt = g.next_w + ((size_t)nu0 * g.next_gpu * (g.next_seg == 1 ? 1 : g.next_kb) + (size_t)ns * k0) * 1024;
                 nxt_piece = (unsigned)ng0 << 10; nxt_step = (size_t)ns << 10;
                 left = min(g.next_lead, (unsigned)(ng0 * (k1 - k0)) << 10);
             }
             auto ahead = [&](unsigned bytes) {
-                if (cur < end) {
+                if constexpr (!LEAD) return;
+                else if (cur < end) {
                     while (bytes > 0 && cur < end) {
                         const unsigned n = min(bytes, own_piece - own_done);
                         l2_prefetch(own + own_done, n);
@@ -289,7 +308,7 @@ __global__ void __launch_bounds__(cl_threads(R), 1) gemm_cl_kernel(const __grid_
                 }
             };
             for (int i = 0; i < w_count; ++i) ahead((unsigned)g.stage_bytes);
-            for (unsigned b = 0; b < g.own_burst && cur < end; b += g.stage_bytes) ahead((unsigned)g.stage_bytes);
+            for (unsigned b = 0; LEAD && b < g.own_burst; b += g.stage_bytes) ahead((unsigned)g.stage_bytes);
             while (w_p < passes) {
                 if (!mbar_wait(&w_empty[stage], phase, abortp)) break;
                 w_issue(stage);
@@ -319,6 +338,7 @@ __global__ void __launch_bounds__(cl_threads(R), 1) gemm_cl_kernel(const __grid_
                     const uint32_t bytes = (uint32_t)(min(g.akb, nk - k) * rows) * 256u;
                     mbar_expect_tx(&a_full[slot], bytes);
                     bulk_load(abuf + slot * act_slot, g.act + (size_t)(kb_lo + k) * rows * 256, bytes, &a_full[slot], pol_a);
+                    if (LATE && count == 0) *(volatile int*)&s_acts = 1;
                     ++count;
                     if (++slot == g.act_slots) { slot = 0; phase ^= 1u; }
                 }
@@ -720,12 +740,12 @@ __global__ void cl_image_kernel(const float* __restrict__ a, int rows, int K, un
     }
 }
 
-template <int EPI, int R>
+template <int EPI, int R, bool LEAD = false>
 anpd_status launch_cl(const ClArgs& g, int smem, cudaStream_t st, Profiler* prof, double bytes) {
     static bool attr_set[64] = {false};
     if (first_call_on_device(attr_set)) {
-        CUDA_TRY(cudaFuncSetAttribute(gemm_cl_kernel<EPI, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, CL_SMEM_MAX));
-        CUDA_TRY(cudaFuncSetAttribute(gemm_cl_kernel<EPI, R>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared));
+        CUDA_TRY(cudaFuncSetAttribute(gemm_cl_kernel<EPI, R, LEAD>, cudaFuncAttributeMaxDynamicSharedMemorySize, CL_SMEM_MAX));
+        CUDA_TRY(cudaFuncSetAttribute(gemm_cl_kernel<EPI, R, LEAD>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared));
     }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(g.ncl * CL_CTAS); cfg.blockDim = dim3(cl_threads(R)); cfg.dynamicSmemBytes = smem; cfg.stream = st;
@@ -743,7 +763,7 @@ anpd_status launch_cl(const ClArgs& g, int smem, cudaStream_t st, Profiler* prof
     }
     cfg.attrs = attr;
     cfg.numAttrs = n;
-    LAUNCH(prof, st, KC_GEMM, bytes, (cudaLaunchKernelEx(&cfg, gemm_cl_kernel<EPI, R>, g)));
+    LAUNCH(prof, st, KC_GEMM, bytes, (cudaLaunchKernelEx(&cfg, gemm_cl_kernel<EPI, R, LEAD>, g)));
     CUDA_TRY(cudaGetLastError());
     return ANPD_OK;
 }
@@ -753,7 +773,7 @@ anpd_status launch_cl(const ClArgs& g, int smem, cudaStream_t st, Profiler* prof
 // Clusters that can be resident together, at most 32: the decoder family's dimensions are multiples of 32 units, so 32 clusters
 // get equal shares, where the 33 a B200's 148 SMs hold would leave some with a unit more than the rest.
 int cl_clusters() {
-    if (cudaFuncSetAttribute(gemm_cl_kernel<CL_RAW, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, CL_SMEM_MAX) != cudaSuccess) { cudaGetLastError(); return 0; }
+    if (cudaFuncSetAttribute(gemm_cl_kernel<CL_RAW, 8, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, CL_SMEM_MAX) != cudaSuccess) { cudaGetLastError(); return 0; }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(32 * CL_CTAS); cfg.blockDim = dim3(cl_threads(8)); cfg.dynamicSmemBytes = CL_SMEM_MAX;
     cudaLaunchAttribute attr[1];
@@ -761,7 +781,7 @@ int cl_clusters() {
     attr[0].val.clusterDim.x = CL_CTAS; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr; cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, gemm_cl_kernel<CL_RAW, 8>, &cfg) != cudaSuccess) { cudaGetLastError(); return 0; }
+    if (cudaOccupancyMaxActiveClusters(&n, gemm_cl_kernel<CL_RAW, 8, false>, &cfg) != cudaSuccess) { cudaGetLastError(); return 0; }
     return std::min(n, 32);
 }
 
@@ -856,6 +876,7 @@ static anpd_status cl_args(ClArgs* g, const ClPlan& p, const unsigned char* w, c
     g->stages = std::min(CL_MAX_STAGES, std::min(room, CL_RING_BYTES) / g->stage_bytes);
     if (g->stages < 2) return ANPD_ERR_CAPACITY;
     // the M = 128 instruction reads 16 KB from the last tile of the last stage on, whatever the tile holds
+    g->first = one && !pair ? std::min(CL_FIRST, g->stages) : g->stages;
     const int need = g->stages * g->stage_bytes + std::max(rest, CL_STAGE_MAX + 1024);
     // Two CTAs that share an SM take half of its shared memory each, whatever they need: with unequal halves the next kernel's
     // CTA finds the space its predecessor's predecessor left too small.
@@ -877,28 +898,25 @@ anpd_status cl_enqueue(const ClPlan& p, const unsigned char* w, const unsigned c
     g.q_hi = e.q_hi; g.q_lo = e.q_lo; g.kpool = e.kpool_l; g.vpool = e.vpool_l;
     g.x = e.x; g.gain = e.gain; g.ss_out = e.ss_out; g.d = e.d; g.act_out = e.act_out;
     g.out = e.out; g.amax_val = e.amax_val; g.amax_idx = e.amax_idx;
-    if (e.next) { g.next_w = e.next_w; g.next_kb = e.next->kb; g.next_gpu = e.next->gpu; g.next_units = e.next->n_units; g.next_passes = 1; g.next_seg = e.next->seg; g.next_lead = e.next_lead; }
+    if (e.next) { g.next_w = e.next_w; g.next_kb = e.next->kb; g.next_gpu = e.next->gpu; g.next_units = e.next->n_units; g.next_seg = e.next->seg; g.next_lead = e.next_lead; }
     g.own_lead = e.own_lead; g.own_burst = e.own_burst;
     g.err = err;
     const double bytes = 2.0 * (double)p.N * (double)p.K;
     switch (p.kind) {
         case CL_RAW: return launch_cl<CL_RAW, 8>(g, smem, st, prof, bytes);
-        case CL_QKV: return launch_cl<CL_QKV, 8>(g, smem, st, prof, bytes);
-        case CL_RESID: return launch_cl<CL_RESID, 8>(g, smem, st, prof, bytes);
-        case CL_GU: return launch_cl<CL_GU, 8>(g, smem, st, prof, bytes);
-        case CL_LM: return launch_cl<CL_LM, 8>(g, smem, st, prof, bytes);
+        case CL_QKV: return e.ahead ? launch_cl<CL_QKV, 8, true>(g, smem, st, prof, bytes) : launch_cl<CL_QKV, 8>(g, smem, st, prof, bytes);
+        case CL_RESID: return e.ahead ? launch_cl<CL_RESID, 8, true>(g, smem, st, prof, bytes) : launch_cl<CL_RESID, 8>(g, smem, st, prof, bytes);
+        case CL_GU: return e.ahead ? launch_cl<CL_GU, 8, true>(g, smem, st, prof, bytes) : launch_cl<CL_GU, 8>(g, smem, st, prof, bytes);
+        case CL_LM: return e.ahead ? launch_cl<CL_LM, 8, true>(g, smem, st, prof, bytes) : launch_cl<CL_LM, 8>(g, smem, st, prof, bytes);
     }
     return ANPD_ERR_ARG;
 }
 
 anpd_status cl_partial_enqueue(const ClPlan& p, const unsigned char* w, const unsigned char* act, int rows, float* part, size_t part_stride, int ld_part,
-                               const ClPlan* next, const unsigned char* next_w, unsigned next_lead, unsigned own_lead, int* err, cudaStream_t st,
-                               Profiler* prof) {
+                               int* err, cudaStream_t st, Profiler* prof) {
     ClArgs g;
     int smem = 0;
     ANPD_TRY(cl_args(&g, p, w, act, rows, cl_passes(p, rows), 0, &smem));
-    if (next) { g.next_w = next_w; g.next_kb = next->kb; g.next_gpu = next->gpu; g.next_units = next->n_units; g.next_passes = cl_passes(*next, rows); g.next_seg = next->seg; g.next_lead = next_lead; }
-    g.own_lead = own_lead; g.own_burst = 0;
     g.part = part; g.part_stride = part_stride; g.ld_part = ld_part; g.plan = p;
     g.err = err;
     return launch_cl<CL_RAW, 0>(g, smem, st, prof, 2.0 * (double)p.N * (double)p.K);

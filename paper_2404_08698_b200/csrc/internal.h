@@ -233,9 +233,7 @@ anpd_status rr_enqueue(int epi, const RRPlan& p, const unsigned char* w, const u
 // What a projection does with its results: plain output, rotary embedding + append, residual add, SwiGLU, vocabulary argmax.
 enum ClKind { CL_RAW = 0, CL_QKV = 1, CL_RESID = 2, CL_GU = 3, CL_LM = 4 };
 constexpr int CL_CTAS = 4;             // CTAs per cluster
-// Bytes per CTA fetched into L2 ahead of the next projection, while the tail of this one, the hand-over and what lies between
-// leave HBM idle.  7B, four projections per layer in sequence: 78.8 us without, 76.4 at 64 KB, 77.5 at 128 KB and 84 at 512 KB
-// (the prefetches of CTAs that are through then delay the others' last copies).  13B, eight sequences: no gain beyond 64 KB.
+// Bytes per CTA fetched into L2 ahead of the next projection, where that pays (see forward_cl_enqueue).
 constexpr int CL_PROMPT_ROWS = 128;       // prompt passes of up to this many rows use the decode projections
 constexpr unsigned CL_LEAD = 64 * 1024;
 constexpr unsigned CL_BURST = 128 * 1024;
@@ -306,6 +304,7 @@ struct ClEpilogue {                    // only the fields of the projection's ki
     float* out = nullptr; float* amax_val = nullptr; int* amax_idx = nullptr;
     // weights the projection fetches into L2 for the one after it, per CTA, and what was fetched for it the same way
     const ClPlan* next = nullptr; const unsigned char* next_w = nullptr; unsigned next_lead = 0, own_lead = 0;
+    bool ahead = false;                 // whether it runs ahead of its own copies in L2, from own_lead on
     unsigned own_burst = 0;             // what the projection fetches into L2 of its own weights at its start, beyond that
 };
 int cl_clusters();                      // clusters the current device runs at once, at most 32 (0: none, or no device)
@@ -320,8 +319,7 @@ anpd_status cl_image_enqueue(const float* a_dev, int rows, int K, unsigned char*
 anpd_status cl_enqueue(const ClPlan& p, const unsigned char* w, const unsigned char* act, const ClEpilogue& e, int* err, cudaStream_t st, Profiler* prof);
 // any number of rows (a multiple of 8, at most 128): CL_CTAS partial sums per output, part[k][row][feature], added by the consumer
 anpd_status cl_partial_enqueue(const ClPlan& p, const unsigned char* w, const unsigned char* act, int rows, float* part, size_t part_stride, int ld_part,
-                               const ClPlan* next, const unsigned char* next_w, unsigned next_lead, unsigned own_lead, int* err, cudaStream_t st,
-                               Profiler* prof);
+                               int* err, cudaStream_t st, Profiler* prof);
 
 // ---------------------------------------------------------------------------------------------
 // model, KV cache and workspace
@@ -542,6 +540,7 @@ anpd_status accept_enqueue(anpd_model* m, anpd_kv* kv, int mode, const NgramDev*
 // tree: the rows carry cache slots and hidden slot ranges of their own (two-candidate steps)
 anpd_status attn_tc_enqueue(anpd_model* m, anpd_kv* kv, int layer, int rows, int max_pos, bool tree = false);
 // attn_dec.cu: attention of a decode step, written straight to the O projection's operand image
+int attn_dec_ctas(const anpd_model* m);          // its CTAs for a single sequence
 anpd_status attn_dec_enqueue(anpd_model* m, anpd_kv* kv, int layer, bool tree);
 // attn_pf.cu: attention of a prompt pass with 128 query rows per CTA (head dimension 128, one query head per kv head)
 anpd_status attn_pf_enqueue(anpd_model* m, anpd_kv* kv, int layer, int rows, unsigned char* img, int n_seq);
