@@ -792,12 +792,12 @@ __global__ void __launch_bounds__(32 * COMBINE_SLICES) attn_combine_wide_kernel(
 // a time; seg_count, null where all tiles have as many, tells of more.  Bound by those sums' way through L2; two chunks where the
 // rows fill the device, one where parallelism is short.
 template <int CH>
-__global__ void __launch_bounds__(256, CH == 1 ? 4 : 5) swiglu_kernel(const float* __restrict__ part, const int* __restrict__ seg_count, size_t split_stride, int ld_part, int F,
+__global__ void __launch_bounds__(256, CH == 1 ? 4 : 5) swiglu_kernel(const float* __restrict__ part, const int* __restrict__ seg_count, size_t split_stride, int ld_part, int F, int from,
                                                      bf16* __restrict__ act_hi, bf16* __restrict__ act_lo, int ns_min, unsigned char* __restrict__ img) {
-    // img: an operand image of gridDim.y rows instead of act_hi and act_lo
+    // img: an operand image of gridDim.y rows instead of act_hi and act_lo; from: the projection has finished the features before it
     pdl_trigger();
     pdl_wait();
-    const int row = blockIdx.y, j0 = 4 * (CH * blockIdx.x * blockDim.x + threadIdx.x);
+    const int row = blockIdx.y, j0 = from + 4 * (CH * blockIdx.x * blockDim.x + threadIdx.x);
     constexpr int AT = CH == 1 ? 4 : 1;
     const float* pr = part + (size_t)row * ld_part;
     if (blockIdx.x == 0) cl_img_clear_row_tail(img, gridDim.y, row, F);
@@ -1073,14 +1073,16 @@ static bool cl_rows(const anpd_model* m, const anpd_kv* kv, int rows) {
 }
 
 // One projection of a prompt pass, of a step of several sequences or, with the plain GEMM, of any forward.  Returns how many
-// partial sums every output has and, where some 128-feature storage tiles have more, all tiles' counts.
-anpd_status gemm_enqueue(anpd_model* m, anpd_kv* kv, int kind, int layer, int rows, const int** seg_count_out, int* seg_min_out) {
+// partial sums every output has and, where some 128-feature storage tiles have more, all tiles' counts.  finished: of a gate-up
+// projection, the activations that it has written itself.
+anpd_status gemm_enqueue(anpd_model* m, anpd_kv* kv, int kind, int layer, int rows, const int** seg_count_out, int* seg_min_out, int* finished = nullptr) {
     Workspace& ws = kv->ws;
     const ClPlan& plan = m->cl[kind];
     const unsigned char* W = kind == GK_LM ? m->lm_head : (kind == GK_QKV ? m->layers[layer].wqkv : kind == GK_O ? m->layers[layer].wo
                                                           : kind == GK_GU ? m->layers[layer].wgu : m->layers[layer].wd);
     const bf16 *a_hi = ws.h_hi, *a_lo = ws.h_lo;
     const CUtensorMap* maps = ws.map_h;
+    if (finished) *finished = 0;
     if (kind == GK_O) { a_hi = ws.ao_hi; a_lo = ws.ao_lo; maps = ws.map_ao; }
     if (kind == GK_DOWN) { a_hi = ws.act_hi; a_lo = ws.act_lo; maps = ws.map_act; }
     if (m->plain_gemm) {
@@ -1120,7 +1122,9 @@ anpd_status gemm_enqueue(anpd_model* m, anpd_kv* kv, int kind, int layer, int ro
         *seg_count_out = nullptr;
     }
     *seg_min_out = sched.ksplit;
-    return gemm_pf_enqueue(plan, W, maps[0], maps[1], rows, ws.part, ws.ld[kind], (size_t)rows * ws.ld[kind], sched, m->num_sms,
+    // a pair of storage tiles holds 128 gate features and their up features
+    if (finished && sched.ksplit == 1) *finished = std::min(m->cfg.d_ffn, sched.tail_split > 1 ? 128 * (sched.tail_from / sched.n_tt) : m->cfg.d_ffn);
+    return gemm_pf_enqueue(plan, W, maps[0], maps[1], rows, ws.part, ws.ld[kind], (size_t)rows * ws.ld[kind], finished ? ws.act_hi : nullptr, finished ? ws.act_lo : nullptr, sched, m->num_sms,
                            ws.gemm_err, m->stream, &m->prof);
 }
 
@@ -1393,13 +1397,14 @@ anpd_status forward_enqueue(anpd_model* m, anpd_kv* kv, int rows, int max_pos, b
         LAUNCH(pf, st, KC_OTHER, 0,
                (launch_k(resid_norm, rows, NORM_THREADS, 0, st, ws.x, ws.part, segs, sstride(GK_O), ws.ld[GK_O], w.ffn_norm, c.rms_eps, d,
                                                        ws.h_hi, ws.h_lo, seg_min, slab ? ws.ci_h : nullptr)));
-        ANPD_TRY(gemm_enqueue(m, kv, GK_GU, l, rows, &segs, &seg_min));
-        if (rows >= 256) LAUNCH(pf, st, KC_OTHER, 0,
-               (launch_k(swiglu_kernel<2>, dim3((F / 4 + 511) / 512, rows), 256, 0, st, ws.part, segs, sstride(GK_GU), ws.ld[GK_GU], F, ws.act_hi, ws.act_lo,
-                         seg_min, slab ? ws.ci_act : nullptr)));
-        else LAUNCH(pf, st, KC_OTHER, 0,
-               (launch_k(swiglu_kernel<1>, dim3((F / 4 + 255) / 256, rows), 256, 0, st, ws.part, segs, sstride(GK_GU), ws.ld[GK_GU], F, ws.act_hi, ws.act_lo,
-                         seg_min, slab ? ws.ci_act : nullptr)));
+        int from = 0;
+        ANPD_TRY(gemm_enqueue(m, kv, GK_GU, l, rows, &segs, &seg_min, &from));
+        if (from < F) {
+            const bool many = rows >= 256;
+            LAUNCH(pf, st, KC_OTHER, 0,
+                   (launch_k(many ? swiglu_kernel<2> : swiglu_kernel<1>, dim3(((F - from) / 4 + (many ? 511 : 255)) / (many ? 512 : 256), rows), 256, 0, st, ws.part, segs,
+                             sstride(GK_GU), ws.ld[GK_GU], F, from, ws.act_hi, ws.act_lo, seg_min, slab ? ws.ci_act : nullptr)));
+        }
         ANPD_TRY(gemm_enqueue(m, kv, GK_DOWN, l, rows, &segs, &seg_min));
         const float* next_gain = (l + 1 < c.n_layers) ? m->layers[l + 1].attn_norm : m->final_norm;
         LAUNCH(pf, st, KC_OTHER, 0,

@@ -29,7 +29,7 @@ namespace {
 using namespace tc;
 
 constexpr int PF_TILE_TOK = 256;
-constexpr int PF_THREADS = 192;          // warp 0: producer, warp 1: MMA issuer + tensor-memory owner, warps 2-5: epilogue
+constexpr int PF_THREADS = 320;          // warp 0: producer, warp 1: MMA issuer + tensor-memory owner, warps 2-9: epilogue, four per accumulator
 constexpr int PF_BLOCK = 16384;          // one 128 x 64 bf16 weight tile
 constexpr int PF_BOX = 8192;             // 64 rows x 64 bf16 of the activations
 constexpr int PF_SMEM = 224 * 1024;
@@ -47,6 +47,7 @@ struct PfArgs {
     int tail_from, tail_split;         // output tiles from tail_from on are cut into tail_split parts instead of ksplit
     size_t seg_stride;                 // elements between the partial-sum slabs of two K parts
     ClPlan plan;
+    bf16 *act_hi, *act_lo;             // gate-up: the activations of tiles in one part, [row][F] as two terms
     int* err;
 };
 
@@ -63,6 +64,9 @@ __device__ __forceinline__ void pf_item(const PfArgs& g, int item, int& ot, int&
     else { const int j = item - uniform; ot = g.tail_from + j / g.tail_split; ks = j % g.tail_split; parts = g.tail_split; }
 }
 
+// GU: the gate-up projection.  A tile in one part is finished here: eight lanes hold gate features, the next eight their up features, so
+// that a lane pair turns two rows' sums into one activation each.  That writes a quarter of the sums' bytes and saves the kernel behind.
+template <bool GU>
 __global__ void __launch_bounds__(PF_THREADS, 1)
 gemm_pf_kernel(const unsigned char* __restrict__ w, const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ CUtensorMap map_lo,
                const __grid_constant__ PfArgs g) {
@@ -81,7 +85,7 @@ gemm_pf_kernel(const unsigned char* __restrict__ w, const __grid_constant__ CUte
     if (threadIdx.x == 0) {
         abort_flag = 0;
         for (int s = 0; s < PF_MAX_STAGES; ++s) { mbar_init(&bar_full[s], 1); mbar_init(&bar_empty[s], 1); }
-        mbar_init(&bar_acc_full, 1); mbar_init(&bar_acc_empty, 4);
+        mbar_init(&bar_acc_full, 1); mbar_init(&bar_acc_empty, 8);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
@@ -193,7 +197,7 @@ gemm_pf_kernel(const unsigned char* __restrict__ w, const __grid_constant__ CUte
             }
         }
     } else {
-        const int quad = warp & 3;
+        const int quad = warp & 3, acc = (warp - 2) >> 2;
         int done_tiles = 0;
         bool ok = true;
         pdl_wait();                                        // the sums of the projection before have been read
@@ -205,22 +209,39 @@ gemm_pf_kernel(const unsigned char* __restrict__ w, const __grid_constant__ CUte
             if (!ok) break;
             tc_fence_after();
             const int row0 = tt * g.tile_rows;
+            const int n_pos = cl_groups(g.plan) * 8, pos = (2 * ft + acc) * 128 + quad * 32 + lane;
+            const uint32_t col = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(acc * 256);
+            const int n_rows = (2 * ft + acc) * 128 < n_pos ? min(g.tile_rows, g.rows - row0) : 0;
+            if (GU && parts == 1) {
+                const int side = (lane >> 3) & 1, f = (pos >> 4) * 8 + (pos & 7);               // 0: this lane holds gate sums, 1: up sums
 #pragma unroll 1
-            for (int j = 0; j < 2; ++j) {
-                const int pos0 = (2 * ft + j) * 128, n_pos = cl_groups(g.plan) * 8;
-                if (pos0 >= n_pos) break;
-                const int pos = pos0 + quad * 32 + lane;
+                for (int c0 = 0; c0 < n_rows; c0 += 16) {
+                    float v[16];
+                    tc_ld16(col + (uint32_t)c0, v);
+                    const size_t at = (size_t)(row0 + c0) * g.plan.F + f;
+#pragma unroll
+                    for (int r = 0; r < 16; r += 2) {                                           // the gate lane takes row r, the up lane row r + 1
+                        const float other = __shfl_xor_sync(0xffffffffu, side ? v[r] : v[r + 1], 8);
+                        const float gte = side ? other : v[r], up = side ? v[r + 1] : other;
+                        const float a = gte / (1.0f + expf(-gte)) * up;
+                        if (f < g.plan.F && c0 + r + side < n_rows) {
+                            const bf16 hi = __float2bfloat16_rn(a);
+                            g.act_hi[at + (size_t)(r + side) * g.plan.F] = hi;
+                            g.act_lo[at + (size_t)(r + side) * g.plan.F] = __float2bfloat16_rn(a - __bfloat162float(hi));
+                        }
+                    }
+                }
+            } else {
                 const int n = pos < n_pos ? cl_feature(g.plan, pos) : g.plan.N;
 #pragma unroll 1
-                for (int c0 = 0; c0 < g.tile_rows; c0 += 16) {
-                    if (row0 + c0 >= g.rows) break;
+                for (int c0 = 0; c0 < n_rows; c0 += 16) {
                     float v[16];
-                    tc_ld16(tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(j * 256 + c0), v);
+                    tc_ld16(col + (uint32_t)c0, v);
                     if (n < g.plan.N) {
                         float* out = g.out + (size_t)ks * g.seg_stride + (size_t)(row0 + c0) * g.ld + n;
 #pragma unroll
                         for (int r = 0; r < 16; ++r)
-                            if (row0 + c0 + r < g.rows) out[(size_t)r * g.ld] = v[r];
+                            if (c0 + r < n_rows) out[(size_t)r * g.ld] = v[r];
                     }
                 }
             }
@@ -243,7 +264,8 @@ gemm_pf_kernel(const unsigned char* __restrict__ w, const __grid_constant__ CUte
 }  // namespace
 
 // Cycles on the busiest CTA when the work items go to the CTAs round robin, and of the partial sums' way through memory.
-static long long pf_cost(int n_ft, int rows, int k_blocks, int num_sms, const PfSchedule& s) {
+// finish: tiles in one part leave finished activations, others need a pass of their own (see GU).
+static long long pf_cost(int n_ft, int rows, int k_blocks, int num_sms, const PfSchedule& s, bool finish) {
     const int T = pf_tile_rows(rows, s.n_tt), n_ot = n_ft * s.n_tt, boxes = (T + 63) / 64;
     // a k-block: 16 products of T / 2 cycles, or its bytes at about 48 a cycle and SM; an item: its epilogue and about a microsecond
     const int step = std::max(8 * T, pf_stage_bytes(boxes) / 48), item = 48 * T + 2000;
@@ -256,21 +278,23 @@ static long long pf_cost(int n_ft, int rows, int k_blocks, int num_sms, const Pf
         const int nu = (uniform - i + grid - 1) / grid, n = (uniform + tail - i + grid - 1) / grid;
         worst = std::max(worst, nu * a + (n - nu) * b);
     }
-    // a sum is written, read and added: 8 bytes at about 3000 a cycle for the device
-    const long long sums = (long long)rows * PF_TILE_FT * ((long long)uniform + tail) / std::max(1, s.n_tt) * 8 / 3000;
-    return worst + sums;
+    // a sum is written, read and added: 8 bytes at about 3000 a cycle for the device, a finished one 2; a kernel of its own: a microsecond more (1024
+    // wide, 300 rows: in three parts 1163 us per prompt, whole and finished 1204)
+    const bool whole = finish && s.ksplit == 1;
+    const long long sums = (long long)rows * PF_TILE_FT * ((whole ? uniform / 4 : uniform) + (long long)tail) / std::max(1, s.n_tt) * 8 / 3000;
+    return worst + sums + (finish && (s.ksplit > 1 || tail) ? 2000 : 0);
 }
 
 // The rows' tiles and the cut along K with the least cost: every tile in up to max_parts parts, or the tiles of the last, partly
 // filled round alone in 2 to 4.
-PfSchedule gemm_pf_schedule(int n_ft, int rows, int k_blocks, int num_sms, int max_parts) {
+PfSchedule gemm_pf_schedule(int n_ft, int rows, int k_blocks, int num_sms, int max_parts, bool finish) {
     PfSchedule best{1, n_ft, 1, 1};
     long long best_cost = -1;
     const int least = (rows + PF_TILE_TOK - 1) / PF_TILE_TOK;
     for (int n_tt = least; n_tt <= least + 1; ++n_tt) {
         const int n_ot = n_ft * n_tt, full = n_ot / num_sms;
         auto consider = [&](PfSchedule c) {
-            const long long cost = pf_cost(n_ft, rows, k_blocks, num_sms, c);
+            const long long cost = pf_cost(n_ft, rows, k_blocks, num_sms, c, finish);
             if (best_cost < 0 || cost < best_cost) { best = c; best_cost = cost; }
         };
         for (int s = 1; s <= std::min(max_parts, k_blocks); ++s) consider({s, n_ot, 1, n_tt});
@@ -282,14 +306,15 @@ PfSchedule gemm_pf_schedule(int n_ft, int rows, int k_blocks, int num_sms, int m
 }
 
 PfSchedule prompt_schedule(const anpd_model* m, const Workspace& ws, int kind, int rows) {
-    return gemm_pf_schedule((m->plan[kind].m_tiles + 1) / 2, rows, m->cl[kind].kb, m->num_sms, std::min(PF_MAX_PARTS, 3 * ws.r_max / rows));
+    return gemm_pf_schedule((m->plan[kind].m_tiles + 1) / 2, rows, m->cl[kind].kb, m->num_sms, std::min(PF_MAX_PARTS, 3 * ws.r_max / rows), kind == GK_GU);
 }
 
 anpd_status gemm_pf_enqueue(const ClPlan& plan, const unsigned char* w, const CUtensorMap& map_hi, const CUtensorMap& map_lo, int rows,
-                            float* out, int ld, size_t seg_stride, PfSchedule sched, int num_sms, int* err, cudaStream_t st, Profiler* prof) {
+                            float* out, int ld, size_t seg_stride, bf16* act_hi, bf16* act_lo, PfSchedule sched, int num_sms, int* err, cudaStream_t st, Profiler* prof) {
     static bool attr_set[64] = {false};
     if (first_call_on_device(attr_set)) {
-        CUDA_TRY(cudaFuncSetAttribute(gemm_pf_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, PF_SMEM));
+        CUDA_TRY(cudaFuncSetAttribute(gemm_pf_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, PF_SMEM));
+        CUDA_TRY(cudaFuncSetAttribute(gemm_pf_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, PF_SMEM));
     }
     PfArgs g;
     g.out = out; g.ld = ld; g.rows = rows;
@@ -301,10 +326,11 @@ anpd_status gemm_pf_enqueue(const ClPlan& plan, const unsigned char* w, const CU
     g.stages = std::min(PF_MAX_STAGES, (PF_SMEM - 1024) / pf_stage_bytes(g.boxes));
     const int smem = g.stages * pf_stage_bytes(g.boxes) + 1024;
     g.ksplit = sched.ksplit; g.tail_from = sched.tail_from; g.tail_split = sched.tail_split; g.seg_stride = seg_stride;
+    g.act_hi = act_hi; g.act_lo = act_lo;
     g.err = err;
     const int grid = std::min(num_sms, sched.tail_from * sched.ksplit + (g.n_ft * g.n_tt - sched.tail_from) * sched.tail_split);
     LAUNCH(prof, st, KC_GEMM, 2.0 * (double)plan.N * (double)plan.K,
-           (launch_k(gemm_pf_kernel, grid, PF_THREADS, (size_t)smem, st, w, map_hi, map_lo, g)));
+           (launch_k(act_hi ? gemm_pf_kernel<true> : gemm_pf_kernel<false>, grid, PF_THREADS, (size_t)smem, st, w, map_hi, map_lo, g)));
     CUDA_TRY(cudaGetLastError());
     return ANPD_OK;
 }

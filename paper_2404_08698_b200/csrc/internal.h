@@ -582,11 +582,11 @@ const GemmPlan* tc_model_plan(const anpd_model* m, int kind, int rows);      // 
 // tile fastest) are cut along K: tiles [0, tail_from) into `ksplit` equal parts each, tiles [tail_from, end) - those that would
 // form a last, partly filled round of CTAs - into `tail_split` parts (tail_from == tile count: no such tail; a multiple of the
 // row tile count, so that a feature tile has one part count for all its rows).
-PfSchedule gemm_pf_schedule(int n_ft, int rows, int k_blocks, int num_sms, int max_parts);
+PfSchedule gemm_pf_schedule(int n_ft, int rows, int k_blocks, int num_sms, int max_parts, bool finish);
 PfSchedule prompt_schedule(const anpd_model* m, const Workspace& ws, int kind, int rows);       // the cut a prompt pass of `rows` rows gets
 constexpr int PF_MAX_PARTS = 8;
 anpd_status gemm_pf_enqueue(const ClPlan& plan, const unsigned char* w, const CUtensorMap& map_hi, const CUtensorMap& map_lo, int rows,
-                            float* out, int ld, size_t seg_stride, PfSchedule sched, int num_sms, int* err, cudaStream_t st, Profiler* prof);
+                            float* out, int ld, size_t seg_stride, __nv_bfloat16* act_hi, __nv_bfloat16* act_lo, PfSchedule sched, int num_sms, int* err, cudaStream_t st, Profiler* prof);
 // forward.cu: the plain (one warp per output feature) GEMM, kept as a cross-check
 anpd_status gemm_plain_enqueue(const ClPlan& p, const unsigned char* W, const __nv_bfloat16* a_hi, const __nv_bfloat16* a_lo, int rows,
                                float* part, int ld_part, cudaStream_t st, Profiler* prof);
