@@ -79,13 +79,14 @@ __global__ void plan_prefill_kernel(const int* prompt, int seq, int start, int p
 // one memory round trip.  The sum of squares is reduced in a fixed tree.
 // ---------------------------------------------------------------------------------------------
 constexpr int NORM_THREADS = 1024;
+constexpr int NORM_THREADS_2 = 768;       // of a row of two chunks per thread
 constexpr int NORM_MAX_CHUNKS = 4;        // float4 chunks per thread: rows up to 16384 wide
 
-__device__ __forceinline__ float block_sum_1024(float v, float* red /*[32]*/) {
+__device__ __forceinline__ float block_sum(float v, float* red /*[32]*/) {
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
     __syncthreads();
-    float t = red[threadIdx.x & 31];
+    float t = (threadIdx.x & 31) < blockDim.x >> 5 ? red[threadIdx.x & 31] : 0.0f;
     for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
     __syncthreads();
     return t;
@@ -126,7 +127,7 @@ __global__ void __launch_bounds__(NORM_THREADS) embed_norm_kernel(const bf16* __
         }
     }
     cl_img_clear_row_tail(img, gridDim.x, row, d);
-    const float rstd = rsqrtf(block_sum_1024(ss, red) / (float)d + eps);
+    const float rstd = rsqrtf(block_sum(ss, red) / (float)d + eps);
 #pragma unroll
     for (int u = 0; u < NORM_MAX_CHUNKS; ++u) {
         const int c = threadIdx.x + u * NORM_THREADS;
@@ -162,7 +163,7 @@ __global__ void __launch_bounds__(NORM_THREADS) embed_cl_kernel(const bf16* __re
         acc += v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
     }
     cl_img_clear_row_tail(img, img_rows, row, d);
-    const float t = block_sum_1024(acc, red);
+    const float t = block_sum(acc, red);
     if (threadIdx.x == 0) ss[row] = t;
 }
 
@@ -190,14 +191,18 @@ __global__ void __launch_bounds__(NORM_THREADS) embed_img_kernel(const bf16* __r
         *(uint2*)(img + act_img_offset(row, 4 * c)) = *(const uint2*)hi;               // 4 elements never straddle a 16-byte chunk
         *(uint2*)(img + act_img_offset(ANPD_ROWS + row, 4 * c)) = *(const uint2*)lo;
     }
-    const float t = block_sum_1024(acc, red);
+    const float t = block_sum(acc, red);
     if (threadIdx.x == 0) ss[row] = t;
 }
 
-// x[row] += sum of the tile's partial sums (in segment order); then h = rmsnorm(x) * gain as hi + lo.  NCH chunks of 4096 features;
-// rows of one chunk run two to an SM, so that one row's sums travel while the other's are reduced (1536 rows of 4096: 31 -> 19 us).
+// x[row] += sum of the tile's partial sums (in segment order); then h = rmsnorm(x) * gain as hi + lo.  NCH chunks of four features per
+// thread.  Rows run two and more to an SM, so that one row's sums travel while another's are reduced (1536 rows of 4096: 31 -> 19 us).
+// A wider row takes as few threads as its chunks need: 1024 for 1280 chunks left most of them idle and the SM to one row (13B, ten
+// layers, eight prompts of 512: 33.2 -> 32.2 ms).  Up to 1024 chunks a block of 1024 is the better one even where some idle (1.1B, 333 rows, 2275 against 2340 us).
+inline int norm_chunks(int d) { return d <= 4 * NORM_THREADS ? 1 : d <= 8 * NORM_THREADS_2 ? 2 : NORM_MAX_CHUNKS; }
+inline int norm_threads(int d) { const int n = norm_chunks(d); return n == 1 ? NORM_THREADS : (d / 4 + 32 * n - 1) / (32 * n) * 32; }
 template <int NCH>
-__global__ void __launch_bounds__(NORM_THREADS, NCH == 1 ? 2 : 1) resid_norm_kernel(float* __restrict__ x, const float* __restrict__ part,
+__global__ void __launch_bounds__(NCH == 2 ? NORM_THREADS_2 : NORM_THREADS, NCH <= 2 ? 2 : 1) resid_norm_kernel(float* __restrict__ x, const float* __restrict__ part,
                                                                   const int* __restrict__ seg_count, size_t split_stride, int ld_part,
                                                                   const float* __restrict__ gain, float eps, int d,
                                                                   bf16* __restrict__ h_hi, bf16* __restrict__ h_lo, int ns_min,
@@ -205,21 +210,21 @@ __global__ void __launch_bounds__(NORM_THREADS, NCH == 1 ? 2 : 1) resid_norm_ker
     // img: a decode step's operand image of gridDim.x rows instead of h_hi and h_lo.
     // ns_min: partial sums every tile of this projection has; seg_count: null, or each tile's own count.
     pdl_trigger();
-    constexpr int AT = NCH == 1 ? 4 : 8;
+    constexpr int AT = NCH <= 2 ? 4 : 8;
     __shared__ float red[32];
     const int row = blockIdx.x, chunks = d >> 2;
     float4 v[NCH], gn[NCH];
     // the norm's gain is a weight: nothing of this step writes it, so it is fetched before the dependency wait
 #pragma unroll
     for (int u = 0; u < NCH; ++u) {
-        const int c = threadIdx.x + u * NORM_THREADS;
+        const int c = threadIdx.x + u * blockDim.x;
         gn[u] = (c < chunks) ? *(const float4*)(gain + 4 * c) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
     pdl_wait();
     float ss = 0.0f;
 #pragma unroll
     for (int u = 0; u < NCH; ++u) {
-        const int c = threadIdx.x + u * NORM_THREADS;
+        const int c = threadIdx.x + u * blockDim.x;
         v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
         if (c < chunks) {
             const float* pr = part + (size_t)row * ld_part + 4 * c;
@@ -240,10 +245,10 @@ __global__ void __launch_bounds__(NORM_THREADS, NCH == 1 ? 2 : 1) resid_norm_ker
         }
     }
     cl_img_clear_row_tail(img, gridDim.x, row, d);
-    const float rstd = rsqrtf(block_sum_1024(ss, red) / (float)d + eps);
+    const float rstd = rsqrtf(block_sum(ss, red) / (float)d + eps);
 #pragma unroll
     for (int u = 0; u < NCH; ++u) {
-        const int c = threadIdx.x + u * NORM_THREADS;
+        const int c = threadIdx.x + u * blockDim.x;
         if (c < chunks) {
             const float4 g = gn[u];
             store_split4(make_float4(v[u].x * rstd * g.x, v[u].y * rstd * g.y, v[u].z * rstd * g.z, v[u].w * rstd * g.w),
@@ -1077,12 +1082,12 @@ static bool cl_rows(const anpd_model* m, const anpd_kv* kv, int rows) {
 // projection, the activations that it has written itself.
 anpd_status gemm_enqueue(anpd_model* m, anpd_kv* kv, int kind, int layer, int rows, const int** seg_count_out, int* seg_min_out, int* finished = nullptr) {
     Workspace& ws = kv->ws;
+    if (finished) *finished = 0;
     const ClPlan& plan = m->cl[kind];
     const unsigned char* W = kind == GK_LM ? m->lm_head : (kind == GK_QKV ? m->layers[layer].wqkv : kind == GK_O ? m->layers[layer].wo
                                                           : kind == GK_GU ? m->layers[layer].wgu : m->layers[layer].wd);
     const bf16 *a_hi = ws.h_hi, *a_lo = ws.h_lo;
     const CUtensorMap* maps = ws.map_h;
-    if (finished) *finished = 0;
     if (kind == GK_O) { a_hi = ws.ao_hi; a_lo = ws.ao_lo; maps = ws.map_ao; }
     if (kind == GK_DOWN) { a_hi = ws.act_hi; a_lo = ws.act_lo; maps = ws.map_act; }
     if (m->plain_gemm) {
@@ -1345,7 +1350,8 @@ anpd_status forward_enqueue(anpd_model* m, anpd_kv* kv, int rows, int max_pos, b
     if (m->rr_ready && kv->batch == 1 && rows == ANPD_ROWS && head && !m->plain_gemm && !two_candidates) return forward_rr_enqueue(m, kv, max_pos, want_logits);
     if (kv->step_ready && rows == kv->batch * ANPD_ROWS && head && !m->prof.on && !two_candidates) return step_kernel_enqueue(m, kv, max_pos, want_logits);
     const bool decode = rows == kv->batch * ANPD_ROWS && !m->plain_gemm;           // (or a prompt pass of as many rows)
-    const auto resid_norm = m->cfg.d_model <= 4 * NORM_THREADS ? resid_norm_kernel<1> : m->cfg.d_model <= 8 * NORM_THREADS ? resid_norm_kernel<2> : resid_norm_kernel<NORM_MAX_CHUNKS>;
+    const int norm_n = norm_chunks(m->cfg.d_model), norm_t = norm_threads(m->cfg.d_model);
+    const auto resid_norm = norm_n == 1 ? resid_norm_kernel<1> : norm_n == 2 ? resid_norm_kernel<2> : resid_norm_kernel<NORM_MAX_CHUNKS>;
     const bool slab = cl_rows(m, kv, rows);
     if (decode && kv->batch == 1 && head && m->cl_all_fused) return forward_cl_enqueue(m, kv, max_pos, want_logits, two_candidates);
     const anpd_model_config& c = m->cfg;
@@ -1395,7 +1401,7 @@ anpd_status forward_enqueue(anpd_model* m, anpd_kv* kv, int rows, int max_pos, b
         else ANPD_TRY(attn_enqueue<64>(m, kv, l, rows, max_pos, ao_img, two_candidates, ao_rows, n_seq));
         ANPD_TRY(gemm_enqueue(m, kv, GK_O, l, rows, &segs, &seg_min));
         LAUNCH(pf, st, KC_OTHER, 0,
-               (launch_k(resid_norm, rows, NORM_THREADS, 0, st, ws.x, ws.part, segs, sstride(GK_O), ws.ld[GK_O], w.ffn_norm, c.rms_eps, d,
+               (launch_k(resid_norm, rows, norm_t, 0, st, ws.x, ws.part, segs, sstride(GK_O), ws.ld[GK_O], w.ffn_norm, c.rms_eps, d,
                                                        ws.h_hi, ws.h_lo, seg_min, slab ? ws.ci_h : nullptr)));
         int from = 0;
         ANPD_TRY(gemm_enqueue(m, kv, GK_GU, l, rows, &segs, &seg_min, &from));
@@ -1408,7 +1414,7 @@ anpd_status forward_enqueue(anpd_model* m, anpd_kv* kv, int rows, int max_pos, b
         ANPD_TRY(gemm_enqueue(m, kv, GK_DOWN, l, rows, &segs, &seg_min));
         const float* next_gain = (l + 1 < c.n_layers) ? m->layers[l + 1].attn_norm : m->final_norm;
         LAUNCH(pf, st, KC_OTHER, 0,
-               (launch_k(resid_norm, rows, NORM_THREADS, 0, st, ws.x, ws.part, segs, sstride(GK_DOWN), ws.ld[GK_DOWN], next_gain, c.rms_eps, d,
+               (launch_k(resid_norm, rows, norm_t, 0, st, ws.x, ws.part, segs, sstride(GK_DOWN), ws.ld[GK_DOWN], next_gain, c.rms_eps, d,
                                                        ws.h_hi, ws.h_lo, seg_min, decode || (slab && l + 1 < c.n_layers) ? ws.ci_h : nullptr)));
     }
     if (!head) { CUDA_TRY(cudaGetLastError()); return ANPD_OK; }
