@@ -97,6 +97,7 @@ __device__ __forceinline__ void st_async4(uint32_t addr, uint32_t bar, float a, 
 }
 // Bounded wait for data other CTAs of the cluster wrote.
 __device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
+#pragma unroll 1
     for (unsigned i = 0; i < WAIT_LIMIT; ++i) {
         uint32_t ok;
         asm volatile(
@@ -109,6 +110,18 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity
     }
     *abort_flag = 1;
     return false;
+}
+// by the barrier's address, with little code (see mbar_wait_small)
+__device__ __forceinline__ void wait_at(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
+#pragma unroll 1
+    for (unsigned i = 0; i < WAIT_LIMIT; ++i) {
+        uint32_t ok;
+        asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                     : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+        if (ok) return;
+        if ((i & 1023u) == 1023u && *abort_flag) return;
+    }
+    *abort_flag = 1;
 }
 __device__ __forceinline__ void l2_prefetch(const void* src, uint32_t bytes) {
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory");
@@ -151,10 +164,12 @@ __device__ __forceinline__ void split2(float a, float b, uint32_t& hi, uint32_t&
     lo = (uint32_t)__bfloat16_as_ushort(la) | ((uint32_t)__bfloat16_as_ushort(lb) << 16);
 }
 
-// R: 8 = a step of one sequence (8 rows, one pass, one chunk); 0 = rows, passes and chunks from the arguments.  LEAD: runs ahead in L2
-template <int EPI, int R, bool LEAD>
+// R: 8 = a step of one sequence (8 rows, one pass, one chunk); 0 = rows, passes and chunks from the arguments.  LEAD: runs ahead in L2.
+// TMAX: most tiles of a sequence's step, 1 or CL_MAX_TILES: code is time here (see launch_step)
+template <int EPI, int R, bool LEAD, int TMAX>
 __global__ void __launch_bounds__(cl_threads(R), 1) gemm_cl_kernel(const __grid_constant__ ClArgs g) {
     constexpr bool LATE = R && !LEAD;                  // its CTAs start late (see CL_FIRST)
+    constexpr bool ONE = R && TMAX == 1;
     extern __shared__ __align__(1024) unsigned char cl_smem_raw[];
     __shared__ uint64_t w_full[CL_MAX_STAGES], w_empty[CL_MAX_STAGES], a_full[CL_MAX_ACT], a_empty[CL_MAX_ACT];
     __shared__ uint64_t acc_full[2], acc_empty[2], red_full;
@@ -171,7 +186,7 @@ __global__ void __launch_bounds__(cl_threads(R), 1) gemm_cl_kernel(const __grid_
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     constexpr int C = CL_CTAS;
     const int rank = (int)blockIdx.x % C, cluster = (int)blockIdx.x / C;            // a cluster is C consecutive CTAs
-    const int ulo = (int)((long long)cluster * g.n_units / g.ncl), uhi = (int)((long long)(cluster + 1) * g.n_units / g.ncl);
+    const int ulo = (int)((unsigned)(cluster * g.n_units) / (unsigned)g.ncl), uhi = (int)((unsigned)((cluster + 1) * g.n_units) / (unsigned)g.ncl);     // at most 32 clusters, 2^21 units
     const int Uc = uhi - ulo, Gc = Uc * g.gpu;                                      // units and groups of the cluster
     const int GS = g.seg == 1 ? g.n_units * g.gpu : Gc;                             // groups of a k-block in its segment
     const int kb_lo = rank * g.kb / C, nk = (rank + 1) * g.kb / C - kb_lo;          // this CTA's k-blocks
@@ -185,7 +200,7 @@ __global__ void __launch_bounds__(cl_threads(R), 1) gemm_cl_kernel(const __grid_
         else { u0 = p * Uc / passes; up = (p + 1) * Uc / passes - u0; }
     };
 
-    auto copies_of = [&](int G) { return min(g.copies, G); };       // the same for every cluster and pass, though some have a unit less than others
+    auto copies_of = [&](int G) { return ONE ? min(1, G) : min(g.copies, G); };       // the same for every cluster and pass, though some have a unit less than others
 
     // ---- weight thread's walk over (pass, step, tile) ----
     const unsigned char* w_src = nullptr;
@@ -206,15 +221,15 @@ __global__ void __launch_bounds__(cl_threads(R), 1) gemm_cl_kernel(const __grid_
     const uint64_t pol_w = policy_evict_first();
     auto w_issue = [&](int stage) {                     // load the current item into `stage` and move on
         const int n = min(g.kps, nk - w_k);
-        const uint32_t bytes = (uint32_t)(n * (w_base + (w_t < w_rem ? 1 : 0))) << 10;      // n > 1 only where one tile holds all of the segment's groups
+        const uint32_t bytes = (uint32_t)(n * (ONE ? Gc : w_base + (w_t < w_rem ? 1 : 0))) << 10;      // n > 1 only where one tile holds all of the segment's groups
         mbar_expect_tx(&w_full[stage], bytes);
         bulk_load(ring + stage * g.stage_bytes, w_src, bytes, &w_full[stage], pol_w);
         w_src += bytes;
-        if (++w_t == w_T) {
+        if (ONE || ++w_t == w_T) {
             w_t = 0;
             w_k += n;
-            w_src += (size_t)(GS - w_G) << 10;          // the k-block's other groups
-            if (w_k >= nk) { ++w_p; w_enter(); }
+            w_src += (size_t)(GS - (R ? Gc : w_G)) << 10;          // the k-block's other groups
+            if (w_k >= nk) { ++w_p; if (!R) w_enter(); }
         }
     };
     int w_count = 0;
@@ -225,17 +240,20 @@ __global__ void __launch_bounds__(cl_threads(R), 1) gemm_cl_kernel(const __grid_
     if (warp == 0) {
         if (elect_one()) {
             if (!LATE) { abort_flag = 0; s_issued[0] = 0; s_issued[1] = 0; }
+#pragma unroll 1
             for (int s = 0; s < g.stages; ++s) { mbar_init(&w_full[s], 1); mbar_init(&w_empty[s], 1); }
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             // the weights depend on nothing: the first ring is requested before anything else happens
             w_enter();
+#pragma unroll 1
             for (; w_count < (LATE ? g.first : g.stages) && w_p < passes; ++w_count) w_issue(w_count);
         }
         __syncwarp();
     } else if (LATE ? warp == 2 : threadIdx.x == 64) {
         if (!LATE || elect_one()) {
             if (LATE) { abort_flag = 0; s_issued[0] = 0; s_issued[1] = 0; s_acts = 0; }
+#pragma unroll 1
             for (int s = 0; s < g.act_slots; ++s) { mbar_init(&a_full[s], 1); mbar_init(&a_empty[s], 1); }
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -269,6 +287,7 @@ __global__ void __launch_bounds__(cl_threads(R), 1) gemm_cl_kernel(const __grid_
         if (elect_one()) {
             if (LATE && g.first < g.stages) {
                 for (const long long t = clock64(); !*(volatile int*)&s_acts && clock64() - t < CL_HOLD;) {}
+#pragma unroll 1
                 for (; w_count < g.stages && w_p < passes; ++w_count) w_issue(w_count);
             }
             int stage = 0;
@@ -284,7 +303,7 @@ __global__ void __launch_bounds__(cl_threads(R), 1) gemm_cl_kernel(const __grid_
                 own = g.w + ((size_t)ulo * g.gpu * (g.seg == 1 ? 1 : g.kb) + (size_t)GS * (kb_lo + (int)k)) * 1024;
             }
             if (LEAD && g.next_w) {
-                const int nu0 = (int)((long long)cluster * g.next_units / g.ncl), nu1 = (int)((long long)(cluster + 1) * g.next_units / g.ncl);
+                const int nu0 = (int)((unsigned)(cluster * g.next_units) / (unsigned)g.ncl), nu1 = (int)((unsigned)((cluster + 1) * g.next_units) / (unsigned)g.ncl);
                 const int ng0 = (nu1 - nu0) * g.next_gpu, ns = (g.next_seg == 1 ? g.next_units : nu1 - nu0) * g.next_gpu;
                 const int k0 = rank * g.next_kb / C, k1 = (rank + 1) * g.next_kb / C;
                 nxt = g.next_w + ((size_t)nu0 * g.next_gpu * (g.next_seg == 1 ? 1 : g.next_kb) + (size_t)ns * k0) * 1024;
@@ -307,15 +326,19 @@ __global__ void __launch_bounds__(cl_threads(R), 1) gemm_cl_kernel(const __grid_
                     if (nxt_done == nxt_piece) { nxt_done = 0; nxt += nxt_step; }
                 }
             };
+#pragma unroll 1
             for (int i = 0; i < w_count; ++i) ahead((unsigned)g.stage_bytes);
+#pragma unroll 1
             for (unsigned b = 0; LEAD && b < g.own_burst; b += g.stage_bytes) ahead((unsigned)g.stage_bytes);
+#pragma unroll 1
             while (w_p < passes) {
-                if (!mbar_wait(&w_empty[stage], phase, abortp)) break;
+                if (!mbar_wait_small(&w_empty[stage], phase, abortp)) break;
                 w_issue(stage);
                 ahead((unsigned)g.stage_bytes);
                 ++w_count;
                 if (++stage == g.stages) { stage = 0; phase ^= 1u; }
             }
+#pragma unroll 1
             while (left) ahead(CL_STAGE_MAX);
             s_issued[0] = w_count;
         }
@@ -332,8 +355,9 @@ __global__ void __launch_bounds__(cl_threads(R), 1) gemm_cl_kernel(const __grid_
                 int u0, up;
                 pass_of(p, u0, up);
                 if (up == 0) continue;
+#pragma unroll 1
                 for (int k = 0; k < nk; k += g.akb) {
-                    if (count >= g.act_slots) ok = mbar_wait(&a_empty[slot], phase, abortp);
+                    if (count >= g.act_slots) ok = mbar_wait_small(&a_empty[slot], phase, abortp);
                     if (!ok) break;
                     const uint32_t bytes = (uint32_t)(min(g.akb, nk - k) * rows) * 256u;
                     mbar_expect_tx(&a_full[slot], bytes);
@@ -371,23 +395,25 @@ __global__ void __launch_bounds__(cl_threads(R), 1) gemm_cl_kernel(const __grid_
                 int u0, up;
                 pass_of(p, u0, up);
                 const int G = up * g.gpu, T = copies_of(G), base = !R && T ? G / T : 0, rem = !R && T ? G - base * T : 0;
-                if (p >= g.acc_bufs) mbar_wait(&acc_empty[buf], eph, abortp);
+                if (p >= g.acc_bufs) mbar_wait_small(&acc_empty[buf], eph, abortp);
                 tc_fence_after();
                 const uint32_t d0 = tmem_base + (uint32_t)(buf * g.acc_cols);
                 uint32_t acc = 0;
                 const int k_end = T > 0 ? nk : 0;
+#pragma unroll 1
                 for (int k0 = 0; k0 < k_end; k0 += akb) {
-                    mbar_wait_at(afull, aph, abortp);
+                    wait_at(afull, aph, abortp);
                     const int kend = min(akb, nk - k0);
                     uint32_t a = a_lo;
                     // a tile of fewer than 16 groups: the instruction reads whatever follows for the rows beyond, whose lanes nobody reads
                     if (!R && g.two) {                                  // two tiles of one k-block per stage
+#pragma unroll 1
                         for (int k = 0; k < kend; ++k) {
                             uint32_t d_tmem = d0;
 #pragma unroll 1
                             for (int t = 0; t < T; ++t) {
                                 const uint32_t first = (uint32_t)(base + (t < rem ? 2 : 1)) >> 1;       // groups of the copy's first tile
-                                mbar_wait_at(full, wph, abortp);
+                                wait_at(full, wph, abortp);
                                 tc_fence_after();
                                 tc_mma_k64(d_tmem, w_lo, a, idesc, acc);
                                 tc_mma_k64(d_tmem + (uint32_t)(2 * rows), w_lo + (first << 6), a, idesc, acc);
@@ -397,12 +423,13 @@ __global__ void __launch_bounds__(cl_threads(R), 1) gemm_cl_kernel(const __grid_
                             acc = 1;
                             a += kb_step;
                         }
-                    } else if (T > 1) {                                 // one tile of one k-block per stage
+                    } else if (!ONE && T > 1) {                         // one tile of one k-block per stage
+#pragma unroll 1
                         for (int k = 0; k < kend; ++k) {
                             uint32_t d_tmem = d0;
 #pragma unroll 1
                             for (int t = T; t > 0; --t) {
-                                mbar_wait_at(full, wph, abortp);
+                                wait_at(full, wph, abortp);
                                 tc_fence_after();
                                 tc_mma_k64(d_tmem, w_lo, a, idesc, acc);
                                 next_stage();
@@ -412,8 +439,9 @@ __global__ void __launch_bounds__(cl_threads(R), 1) gemm_cl_kernel(const __grid_
                             a += kb_step;
                         }
                     } else {                                            // kps k-blocks of the only tile per stage
+#pragma unroll 1
                         for (int k = 0; k < kend; k += kps) {
-                            mbar_wait_at(full, wph, abortp);
+                            wait_at(full, wph, abortp);
                             tc_fence_after();
                             tc_mma_k64(d0, w_lo, a, idesc, acc);
                             acc = 1;
@@ -449,13 +477,13 @@ __global__ void __launch_bounds__(cl_threads(R), 1) gemm_cl_kernel(const __grid_
         const int ufirst = ulo + o0, parts_out = (int)gridDim.x;
 
         // where this thread's feature of each tile goes: byte offset in the exchange buffer and the owner's rank
-        uint32_t dst[CL_MAX_TILES];
+        uint32_t dst[TMAX + 1];
         const int tiles = copies_of(Gc);
         if (pushes) {
             const int base = tiles ? Gc / tiles : 0, rem = tiles ? Gc - base * tiles : 0;
             int t0 = 0;
 #pragma unroll
-            for (int t = 0; t < CL_MAX_TILES; ++t) {
+            for (int t = 0; t < TMAX; ++t) {
                 dst[t] = 0xffffffffu;
                 if (t < tiles) {
                     const int gt = base + (t < rem ? 1 : 0);
@@ -506,18 +534,19 @@ __global__ void __launch_bounds__(cl_threads(R), 1) gemm_cl_kernel(const __grid_
         cluster_wait();
 
         if (pushes) {
-            mbar_wait(&acc_full[0], 0, abortp);
+            mbar_wait_small(&acc_full[0], 0, abortp);
             tc_fence_after();
             const uint32_t col0 = tmem_base + ((uint32_t)(quad * 32) << 16);
 #pragma unroll
-            for (int t = 0; t < CL_MAX_TILES; t += 2) {
+            for (int t = 0; t < TMAX; t += 2) {
                 if (t >= tiles) break;
                 // two tiles' columns in one load; the second repeats the first where there is none
                 float v[2][8];
                 const uint32_t ca = col0 + (uint32_t)(t * 16), cb = t + 1 < tiles ? ca + 16u : ca;
-                tc_ld8_sum2(ca, ca + 8u, cb, cb + 8u, v[0], v[1]);
+                if (ONE) tc_ld8_sum(ca, ca + 8u, v[0]);
+                else tc_ld8_sum2(ca, ca + 8u, cb, cb + 8u, v[0], v[1]);
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {
+                for (int h = 0; h < (ONE ? 1 : 2); ++h) {
                     if (nk == 0)
 #pragma unroll
                         for (int r = 0; r < 8; ++r) v[h][r] = 0.0f;
@@ -538,6 +567,8 @@ __global__ void __launch_bounds__(cl_threads(R), 1) gemm_cl_kernel(const __grid_
         };
         if (EPI == CL_RESID) {
             float ssq = 0.0f;
+#pragma unroll 1
+#pragma unroll 1
             for (int idx = ft; idx < on * 32; idx += 256) {
                 const int f = 2 * (idx >> 3), n = ufirst * 8 + f;
                 float2 x = pf, gn = pg;
@@ -563,6 +594,8 @@ __global__ void __launch_bounds__(cl_threads(R), 1) gemm_cl_kernel(const __grid_
             }
         } else if (EPI == CL_GU) {
             const float rs = s_rstd[row];
+#pragma unroll 1
+#pragma unroll 1
             for (int idx = ft; idx < on * 32; idx += 256) {
                 const int ul = idx >> 5, e = 2 * ((idx >> 3) & 3), f = ul * 16 + e, k = (ufirst + ul) * 8 + e;
                 float v[2];
@@ -579,6 +612,8 @@ __global__ void __launch_bounds__(cl_threads(R), 1) gemm_cl_kernel(const __grid_
         } else if (EPI == CL_QKV) {
             const float rs = s_rstd[row];
             const int pos = s_pos[row], slot = s_slot[row], page = s_page[row], upi = g.hd >> 4;
+#pragma unroll 1
+#pragma unroll 1
             for (int idx = ft; idx < on * 32; idx += 256) {
                 const int ul = idx >> 5, e = 2 * ((idx >> 3) & 3), u = ufirst + ul, head = u / upi, i = (u - head * upi) * 8 + e;
                 float a[2], b[2];
@@ -621,6 +656,8 @@ __global__ void __launch_bounds__(cl_threads(R), 1) gemm_cl_kernel(const __grid_
             const float rs = s_rstd[row];
             float best = -CUDART_INF_F;
             int bidx = 0x7fffffff;
+#pragma unroll 1
+#pragma unroll 1
             for (int idx = ft; idx < on * 64; idx += 256) {
                 const int f = idx >> 3, n = ufirst * 8 + f;
                 if (n >= g.n_out) continue;
@@ -655,7 +692,7 @@ __global__ void __launch_bounds__(cl_threads(R), 1) gemm_cl_kernel(const __grid_
             int u0, up;
             pass_of(p, u0, up);
             const int G = up * g.gpu, T = copies_of(G), base = T ? G / T : 0, rem = T ? G - base * T : 0, per = g.two ? 2 : 1;
-            mbar_wait(&acc_full[buf], bph, abortp);
+            mbar_wait_small(&acc_full[buf], bph, abortp);
             tc_fence_after();
             int t0 = (ulo + u0) * g.gpu;                // the tile's first group
             for (int t = 0; t < T * per; ++t) {
@@ -740,12 +777,12 @@ __global__ void cl_image_kernel(const float* __restrict__ a, int rows, int K, un
     }
 }
 
-template <int EPI, int R, bool LEAD = false>
+template <int EPI, int R, bool LEAD = false, int TMAX = CL_MAX_TILES>
 anpd_status launch_cl(const ClArgs& g, int smem, cudaStream_t st, Profiler* prof, double bytes) {
     static bool attr_set[64] = {false};
     if (first_call_on_device(attr_set)) {
-        CUDA_TRY(cudaFuncSetAttribute(gemm_cl_kernel<EPI, R, LEAD>, cudaFuncAttributeMaxDynamicSharedMemorySize, CL_SMEM_MAX));
-        CUDA_TRY(cudaFuncSetAttribute(gemm_cl_kernel<EPI, R, LEAD>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared));
+        CUDA_TRY(cudaFuncSetAttribute(gemm_cl_kernel<EPI, R, LEAD, TMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, CL_SMEM_MAX));
+        CUDA_TRY(cudaFuncSetAttribute(gemm_cl_kernel<EPI, R, LEAD, TMAX>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared));
     }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(g.ncl * CL_CTAS); cfg.blockDim = dim3(cl_threads(R)); cfg.dynamicSmemBytes = smem; cfg.stream = st;
@@ -763,9 +800,18 @@ anpd_status launch_cl(const ClArgs& g, int smem, cudaStream_t st, Profiler* prof
     }
     cfg.attrs = attr;
     cfg.numAttrs = n;
-    LAUNCH(prof, st, KC_GEMM, bytes, (cudaLaunchKernelEx(&cfg, gemm_cl_kernel<EPI, R, LEAD>, g)));
+    LAUNCH(prof, st, KC_GEMM, bytes, (cudaLaunchKernelEx(&cfg, gemm_cl_kernel<EPI, R, LEAD, TMAX>, g)));
     CUDA_TRY(cudaGetLastError());
     return ANPD_OK;
+}
+
+// The instance of a sequence's step: what a kernel does not need is not in it.  Its code comes from a cold instruction cache, layer after
+// layer; with one instance for any tile count and unrolled waits and loops (43 to 54 KB of code, now 25 to 46) us per step were: 1.1B at 512
+// keys 776, now 744, tiny 55, now 48, 1024 wide (16 layers) 428, now 379, 7B (16 layers, 77 keys) 1317, now 1301.
+template <int EPI>
+anpd_status launch_step(const ClArgs& g, bool lead, int smem, cudaStream_t st, Profiler* prof, double bytes) {
+    if (g.copies == 1) return lead ? launch_cl<EPI, 8, true, 1>(g, smem, st, prof, bytes) : launch_cl<EPI, 8, false, 1>(g, smem, st, prof, bytes);
+    return lead ? launch_cl<EPI, 8, true>(g, smem, st, prof, bytes) : launch_cl<EPI, 8>(g, smem, st, prof, bytes);
 }
 
 }  // namespace
@@ -773,7 +819,7 @@ anpd_status launch_cl(const ClArgs& g, int smem, cudaStream_t st, Profiler* prof
 // Clusters that can be resident together, at most 32: the decoder family's dimensions are multiples of 32 units, so 32 clusters
 // get equal shares, where the 33 a B200's 148 SMs hold would leave some with a unit more than the rest.
 int cl_clusters() {
-    if (cudaFuncSetAttribute(gemm_cl_kernel<CL_RAW, 8, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, CL_SMEM_MAX) != cudaSuccess) { cudaGetLastError(); return 0; }
+    if (cudaFuncSetAttribute(gemm_cl_kernel<CL_RAW, 8, false, CL_MAX_TILES>, cudaFuncAttributeMaxDynamicSharedMemorySize, CL_SMEM_MAX) != cudaSuccess) { cudaGetLastError(); return 0; }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(32 * CL_CTAS); cfg.blockDim = dim3(cl_threads(8)); cfg.dynamicSmemBytes = CL_SMEM_MAX;
     cudaLaunchAttribute attr[1];
@@ -781,7 +827,7 @@ int cl_clusters() {
     attr[0].val.clusterDim.x = CL_CTAS; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr; cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, gemm_cl_kernel<CL_RAW, 8, false>, &cfg) != cudaSuccess) { cudaGetLastError(); return 0; }
+    if (cudaOccupancyMaxActiveClusters(&n, gemm_cl_kernel<CL_RAW, 8, false, CL_MAX_TILES>, &cfg) != cudaSuccess) { cudaGetLastError(); return 0; }
     return std::min(n, 32);
 }
 
@@ -903,11 +949,11 @@ anpd_status cl_enqueue(const ClPlan& p, const unsigned char* w, const unsigned c
     g.err = err;
     const double bytes = 2.0 * (double)p.N * (double)p.K;
     switch (p.kind) {
-        case CL_RAW: return launch_cl<CL_RAW, 8>(g, smem, st, prof, bytes);
-        case CL_QKV: return e.ahead ? launch_cl<CL_QKV, 8, true>(g, smem, st, prof, bytes) : launch_cl<CL_QKV, 8>(g, smem, st, prof, bytes);
-        case CL_RESID: return e.ahead ? launch_cl<CL_RESID, 8, true>(g, smem, st, prof, bytes) : launch_cl<CL_RESID, 8>(g, smem, st, prof, bytes);
-        case CL_GU: return e.ahead ? launch_cl<CL_GU, 8, true>(g, smem, st, prof, bytes) : launch_cl<CL_GU, 8>(g, smem, st, prof, bytes);
-        case CL_LM: return e.ahead ? launch_cl<CL_LM, 8, true>(g, smem, st, prof, bytes) : launch_cl<CL_LM, 8>(g, smem, st, prof, bytes);
+        case CL_RAW: return launch_step<CL_RAW>(g, false, smem, st, prof, bytes);
+        case CL_QKV: return launch_step<CL_QKV>(g, e.ahead, smem, st, prof, bytes);
+        case CL_RESID: return launch_step<CL_RESID>(g, e.ahead, smem, st, prof, bytes);
+        case CL_GU: return launch_step<CL_GU>(g, e.ahead, smem, st, prof, bytes);
+        case CL_LM: return launch_step<CL_LM>(g, e.ahead, smem, st, prof, bytes);
     }
     return ANPD_ERR_ARG;
 }
