@@ -267,7 +267,10 @@ __global__ void __launch_bounds__((AdCfg<HD, G>::THREADS)) __maxnreg__((AdCfg<HD
 #pragma unroll
                 for (int d = 0; d < DT; ++d) { o[d][0] *= ra; o[d][1] *= ra; o[d][2] *= rb; o[d][3] *= rb; }
             }
-            mbar_wait_small(&full[cv], par_v, abortp);
+            // rolled, this wait costs head dimension 128 registers it does not have at its cap (24 bytes spilled); 64 has them and loses 0.15 % of a
+            // 1.1B step by the unrolled one's code (7B, 16 layers, 1536 keys: 1368 us per step with the spill, 1366 without, both +- 5)
+            if (HD == 128) mbar_wait(&full[cv], par_v, abortp);
+            else mbar_wait_small(&full[cv], par_v, abortp);
             const uint32_t vr = ring_addr + (uint32_t)cv * (uint32_t)CHUNK + kv_off + (uint32_t)((key_page >> 6) * (HD * 128)) + ((((uint32_t)((key_page & 63) >> 3) + chunk0) ^ (uint32_t)lr) << 4);
 #pragma unroll
             for (int d = 0; d < DT / 2; ++d) {
