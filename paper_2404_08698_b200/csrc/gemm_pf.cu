@@ -263,9 +263,13 @@ gemm_pf_kernel(const unsigned char* __restrict__ w, const __grid_constant__ CUte
 
 }  // namespace
 
-// Cycles on the busiest CTA when the work items go to the CTAs round robin, and of the partial sums' way through memory.
-// finish: tiles in one part leave finished activations, others need a pass of their own (see GU).
-static long long pf_cost(int n_ft, int rows, int k_blocks, int num_sms, const PfSchedule& s, bool finish) {
+// Cycles on the busiest CTA when the work items go to the CTAs round robin, and of the partial sums' way through memory.  The gate-up
+// projection's are counted like the others', although it finishes the tiles that are left whole: a credit for that left tiles whole
+// where they fill few SMs, and what eight warps per SM then do behind the last product costs more than the kernel it saves.  us per
+// prompt with the credit and without: 7B (8 layers) 140 tokens 1580 and 1470, 1.1B 200 tokens 2365 and 2235, 512 wide (8 layers) 290
+// tokens 574 and 472, 4096 wide with 14336 gate features (8 layers) 370 tokens 2610 and 2390; the other way at 200 tokens of the tiny model (126 and 130) and 300 of the
+// last one (2290 and 2360); from 600 rows on the two cut alike nearly everywhere.
+static long long pf_cost(int n_ft, int rows, int k_blocks, int num_sms, const PfSchedule& s) {
     const int T = pf_tile_rows(rows, s.n_tt), n_ot = n_ft * s.n_tt, boxes = (T + 63) / 64;
     // a k-block: 16 products of T / 2 cycles, or its bytes at about 48 a cycle and SM; an item: its epilogue and about a microsecond
     const int step = std::max(8 * T, pf_stage_bytes(boxes) / 48), item = 48 * T + 2000;
@@ -278,23 +282,21 @@ static long long pf_cost(int n_ft, int rows, int k_blocks, int num_sms, const Pf
         const int nu = (uniform - i + grid - 1) / grid, n = (uniform + tail - i + grid - 1) / grid;
         worst = std::max(worst, nu * a + (n - nu) * b);
     }
-    // a sum is written, read and added: 8 bytes at about 3000 a cycle for the device, a finished one 2; a kernel of its own: a microsecond more (1024
-    // wide, 300 rows: in three parts 1163 us per prompt, whole and finished 1204)
-    const bool whole = finish && s.ksplit == 1;
-    const long long sums = (long long)rows * PF_TILE_FT * ((whole ? uniform / 4 : uniform) + (long long)tail) / std::max(1, s.n_tt) * 8 / 3000;
-    return worst + sums + (finish && (s.ksplit > 1 || tail) ? 2000 : 0);
+    // a sum is written, read and added: 8 bytes at about 3000 a cycle for the device
+    const long long sums = (long long)rows * PF_TILE_FT * ((long long)uniform + tail) / std::max(1, s.n_tt) * 8 / 3000;
+    return worst + sums;
 }
 
 // The rows' tiles and the cut along K with the least cost: every tile in up to max_parts parts, or the tiles of the last, partly
 // filled round alone in 2 to 4.
-PfSchedule gemm_pf_schedule(int n_ft, int rows, int k_blocks, int num_sms, int max_parts, bool finish) {
+PfSchedule gemm_pf_schedule(int n_ft, int rows, int k_blocks, int num_sms, int max_parts) {
     PfSchedule best{1, n_ft, 1, 1};
     long long best_cost = -1;
     const int least = (rows + PF_TILE_TOK - 1) / PF_TILE_TOK;
     for (int n_tt = least; n_tt <= least + 1; ++n_tt) {
         const int n_ot = n_ft * n_tt, full = n_ot / num_sms;
         auto consider = [&](PfSchedule c) {
-            const long long cost = pf_cost(n_ft, rows, k_blocks, num_sms, c, finish);
+            const long long cost = pf_cost(n_ft, rows, k_blocks, num_sms, c);
             if (best_cost < 0 || cost < best_cost) { best = c; best_cost = cost; }
         };
         for (int s = 1; s <= std::min(max_parts, k_blocks); ++s) consider({s, n_ot, 1, n_tt});
@@ -306,7 +308,7 @@ PfSchedule gemm_pf_schedule(int n_ft, int rows, int k_blocks, int num_sms, int m
 }
 
 PfSchedule prompt_schedule(const anpd_model* m, const Workspace& ws, int kind, int rows) {
-    return gemm_pf_schedule((m->plan[kind].m_tiles + 1) / 2, rows, m->cl[kind].kb, m->num_sms, std::min(PF_MAX_PARTS, 3 * ws.r_max / rows), kind == GK_GU);
+    return gemm_pf_schedule((m->plan[kind].m_tiles + 1) / 2, rows, m->cl[kind].kb, m->num_sms, std::min(PF_MAX_PARTS, 3 * ws.r_max / rows));
 }
 
 anpd_status gemm_pf_enqueue(const ClPlan& plan, const unsigned char* w, const CUtensorMap& map_hi, const CUtensorMap& map_lo, int rows,

@@ -582,7 +582,7 @@ const GemmPlan* tc_model_plan(const anpd_model* m, int kind, int rows);      // 
 // tile fastest) are cut along K: tiles [0, tail_from) into `ksplit` equal parts each, tiles [tail_from, end) - those that would
 // form a last, partly filled round of CTAs - into `tail_split` parts (tail_from == tile count: no such tail; a multiple of the
 // row tile count, so that a feature tile has one part count for all its rows).
-PfSchedule gemm_pf_schedule(int n_ft, int rows, int k_blocks, int num_sms, int max_parts, bool finish);
+PfSchedule gemm_pf_schedule(int n_ft, int rows, int k_blocks, int num_sms, int max_parts);
 PfSchedule prompt_schedule(const anpd_model* m, const Workspace& ws, int kind, int rows);       // the cut a prompt pass of `rows` rows gets
 constexpr int PF_MAX_PARTS = 8;
 anpd_status gemm_pf_enqueue(const ClPlan& plan, const unsigned char* w, const CUtensorMap& map_hi, const CUtensorMap& map_lo, int rows,
