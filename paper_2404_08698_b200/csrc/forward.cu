@@ -199,10 +199,18 @@ __global__ void __launch_bounds__(NORM_THREADS) embed_img_kernel(const bf16* __r
 // thread.  Rows run two and more to an SM, so that one row's sums travel while another's are reduced (1536 rows of 4096: 31 -> 19 us).
 // A wider row takes as few threads as its chunks need: 1024 for 1280 chunks left most of them idle and the SM to one row (13B, ten
 // layers, eight prompts of 512: 33.2 -> 32.2 ms).  Up to 1024 chunks a block of 1024 is the better one even where some idle (1.1B, 333 rows, 2275 against 2340 us).
-inline int norm_chunks(int d) { return d <= 4 * NORM_THREADS ? 1 : d <= 8 * NORM_THREADS_2 ? 2 : NORM_MAX_CHUNKS; }
-inline int norm_threads(int d) { const int n = norm_chunks(d); return n == 1 ? NORM_THREADS : (d / 4 + 32 * n - 1) / (32 * n) * 32; }
-template <int NCH>
-__global__ void __launch_bounds__(NCH == 2 ? NORM_THREADS_2 : NORM_THREADS, NCH <= 2 ? 2 : 1) resid_norm_kernel(float* __restrict__ x, const float* __restrict__ part,
+// Above 6144 features two rows share an SM with four chunks per thread, which are as many round trips one after the other: where there
+// are SMs enough for the rows, up to 1024 threads with two chunks are faster (8192 wide, two layers: steps of eight sequences 878 -> 850
+// us, 7168 wide, two: 495 -> 488; prompts of 1500 tokens 7185 with four, 7255 with two).
+struct NormShape { int chunks, threads, per_sm; };
+inline NormShape norm_shape(int d, int rows, int num_sms) {
+    if (d <= 4 * NORM_THREADS) return {1, NORM_THREADS, 2};
+    const bool half = d <= 8 * NORM_THREADS_2, room = rows <= num_sms && d <= 8 * NORM_THREADS;
+    const int n = half || room ? 2 : NORM_MAX_CHUNKS;
+    return {n, (d / 4 + 32 * n - 1) / (32 * n) * 32, half ? 2 : 1};
+}
+template <int NCH, int MAX_THREADS, int PER_SM>
+__global__ void __launch_bounds__(MAX_THREADS, PER_SM) resid_norm_kernel(float* __restrict__ x, const float* __restrict__ part,
                                                                   const int* __restrict__ seg_count, size_t split_stride, int ld_part,
                                                                   const float* __restrict__ gain, float eps, int d,
                                                                   bf16* __restrict__ h_hi, bf16* __restrict__ h_lo, int ns_min,
@@ -210,7 +218,7 @@ __global__ void __launch_bounds__(NCH == 2 ? NORM_THREADS_2 : NORM_THREADS, NCH 
     // img: a decode step's operand image of gridDim.x rows instead of h_hi and h_lo.
     // ns_min: partial sums every tile of this projection has; seg_count: null, or each tile's own count.
     pdl_trigger();
-    constexpr int AT = NCH <= 2 ? 4 : 8;
+    constexpr int AT = PER_SM == 2 ? 4 : 8;
     __shared__ float red[32];
     const int row = blockIdx.x, chunks = d >> 2;
     float4 v[NCH], gn[NCH];
@@ -1350,8 +1358,9 @@ anpd_status forward_enqueue(anpd_model* m, anpd_kv* kv, int rows, int max_pos, b
     if (m->rr_ready && kv->batch == 1 && rows == ANPD_ROWS && head && !m->plain_gemm && !two_candidates) return forward_rr_enqueue(m, kv, max_pos, want_logits);
     if (kv->step_ready && rows == kv->batch * ANPD_ROWS && head && !m->prof.on && !two_candidates) return step_kernel_enqueue(m, kv, max_pos, want_logits);
     const bool decode = rows == kv->batch * ANPD_ROWS && !m->plain_gemm;           // (or a prompt pass of as many rows)
-    const int norm_n = norm_chunks(m->cfg.d_model), norm_t = norm_threads(m->cfg.d_model);
-    const auto resid_norm = norm_n == 1 ? resid_norm_kernel<1> : norm_n == 2 ? resid_norm_kernel<2> : resid_norm_kernel<NORM_MAX_CHUNKS>;
+    const NormShape norm = norm_shape(m->cfg.d_model, rows, m->num_sms);
+    const auto resid_norm = norm.chunks == 1 ? resid_norm_kernel<1, NORM_THREADS, 2> : norm.chunks == NORM_MAX_CHUNKS ? resid_norm_kernel<NORM_MAX_CHUNKS, NORM_THREADS, 1>
+                          : norm.per_sm == 2 ? resid_norm_kernel<2, NORM_THREADS_2, 2> : resid_norm_kernel<2, NORM_THREADS, 1>;
     const bool slab = cl_rows(m, kv, rows);
     if (decode && kv->batch == 1 && head && m->cl_all_fused) return forward_cl_enqueue(m, kv, max_pos, want_logits, two_candidates);
     const anpd_model_config& c = m->cfg;
@@ -1401,7 +1410,7 @@ anpd_status forward_enqueue(anpd_model* m, anpd_kv* kv, int rows, int max_pos, b
         else ANPD_TRY(attn_enqueue<64>(m, kv, l, rows, max_pos, ao_img, two_candidates, ao_rows, n_seq));
         ANPD_TRY(gemm_enqueue(m, kv, GK_O, l, rows, &segs, &seg_min));
         LAUNCH(pf, st, KC_OTHER, 0,
-               (launch_k(resid_norm, rows, norm_t, 0, st, ws.x, ws.part, segs, sstride(GK_O), ws.ld[GK_O], w.ffn_norm, c.rms_eps, d,
+               (launch_k(resid_norm, rows, norm.threads, 0, st, ws.x, ws.part, segs, sstride(GK_O), ws.ld[GK_O], w.ffn_norm, c.rms_eps, d,
                                                        ws.h_hi, ws.h_lo, seg_min, slab ? ws.ci_h : nullptr)));
         int from = 0;
         ANPD_TRY(gemm_enqueue(m, kv, GK_GU, l, rows, &segs, &seg_min, &from));
@@ -1414,7 +1423,7 @@ anpd_status forward_enqueue(anpd_model* m, anpd_kv* kv, int rows, int max_pos, b
         ANPD_TRY(gemm_enqueue(m, kv, GK_DOWN, l, rows, &segs, &seg_min));
         const float* next_gain = (l + 1 < c.n_layers) ? m->layers[l + 1].attn_norm : m->final_norm;
         LAUNCH(pf, st, KC_OTHER, 0,
-               (launch_k(resid_norm, rows, norm_t, 0, st, ws.x, ws.part, segs, sstride(GK_DOWN), ws.ld[GK_DOWN], next_gain, c.rms_eps, d,
+               (launch_k(resid_norm, rows, norm.threads, 0, st, ws.x, ws.part, segs, sstride(GK_DOWN), ws.ld[GK_DOWN], next_gain, c.rms_eps, d,
                                                        ws.h_hi, ws.h_lo, seg_min, decode || (slab && l + 1 < c.n_layers) ? ws.ci_h : nullptr)));
     }
     if (!head) { CUDA_TRY(cudaGetLastError()); return ANPD_OK; }

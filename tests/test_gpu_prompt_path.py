@@ -79,8 +79,10 @@ def test_prompts_of_several_sequences_share_a_pass(A, batch, plen, hd, group):
 
 # The gate-up projection finishes the activations of tiles that are not cut along K: all cut (twice), none cut and a ragged end, more tiles
 # than SMs (the last, partly filled round cut in two: 213 tiles of 256 features x 176 rows); residual rows of more than 1024 chunks of
-# four: one over, the most of two chunks per thread, one over that, one over 8192
-@pytest.mark.parametrize("d,F,plen", [(256, 136, 129), (512, 1400, 300), (2048, 9000, 513), (4104, 136, 140), (6144, 136, 140), (6152, 136, 140), (8200, 136, 140), (512, 1400, 1100)])
+# four: one over, the most of two chunks per thread with two rows to an SM, one over that and 8192 (two chunks where there is an SM per row,
+# 144 rows, four beyond, 200), one over 8192
+@pytest.mark.parametrize("d,F,plen", [(256, 136, 129), (512, 1400, 300), (2048, 9000, 513), (4104, 136, 140), (6144, 136, 140), (6152, 136, 140), (8200, 136, 140),
+                                      (512, 1400, 1100), (6152, 136, 200), (8192, 136, 140), (8192, 136, 200)])
 def test_prompt_logits_at_feature_tile_and_row_width_edges(A, d, F, plen):
     shape = ModelShape(1, d, 2, 2, 128, F, 500)
     w = make_weights(shape, 31, False, std=0.02)
