@@ -417,11 +417,6 @@ anpd_status launch_attn_dec(anpd_model* m, anpd_kv* kv, AdArgs& a) {
 
 }  // namespace
 
-int attn_dec_ctas(const anpd_model* m) {
-    const int heads = m->cfg.n_kv_heads * ad_split(m->cfg);
-    return heads * ad_cluster(m, heads);
-}
-
 anpd_status attn_dec_enqueue(anpd_model* m, anpd_kv* kv, int layer, bool tree) {
     const anpd_model_config& c = m->cfg;
     Workspace& ws = kv->ws;

@@ -1281,12 +1281,11 @@ static anpd_status forward_rr_enqueue(anpd_model* m, anpd_kv* kv, int max_pos, b
 }
 
 // The vocabulary projection of the 8 rows whose operand image is ws.ci_h, and its argmax candidates.
-static anpd_status lm_head_cl_enqueue(anpd_model* m, anpd_kv* kv, const float* ss, int n_parts, bool want_logits, bool ahead = false, unsigned own_lead = 0) {
+static anpd_status lm_head_cl_enqueue(anpd_model* m, anpd_kv* kv, const float* ss, int n_parts, bool want_logits) {
     const anpd_model_config& c = m->cfg;
     Workspace& ws = kv->ws;
     ClEpilogue lm;
     lm.ss_in = ss; lm.n_parts = n_parts; lm.inv_d = 1.0f / (float)c.d_model; lm.eps = c.rms_eps;
-    lm.ahead = ahead; lm.own_lead = own_lead;
     lm.out = want_logits ? ws.logits : nullptr; lm.amax_val = ws.amax_val_cl; lm.amax_idx = ws.amax_idx_cl;
     ANPD_TRY(cl_enqueue(m->cl[GK_LM], m->lm_head, ws.ci_h, lm, ws.gemm_err, m->stream, &m->prof));
     ws.amax_nblk = cl_parts(m->cl[GK_LM]);
@@ -1307,17 +1306,10 @@ static anpd_status forward_cl_enqueue(anpd_model* m, anpd_kv* kv, int max_pos, b
     LAUNCH(pf, st, KC_OTHER, 0, (launch_k(embed_cl_kernel, rows, NORM_THREADS, 0, st, m->embed, ws.row_tok, m->layers[0].attn_norm, d, ws.x,
                                           ws.ci_h, rows, ws.ss_cl_a)));
     int parts_a = 1;                                   // sums of squares behind ci_h: one after the embedding, then the down projection's
-    // A projection brings the first weights of the next one into L2 while its own tail and the hand-over leave HBM idle, and runs ahead
-    // of its own copies there, where that pays: where the attention leaves half of the SMs to the projections around it and the
-    // gate-up weights are more than these take at once (1.1B, 64 attention CTAs: 803 -> 777 us per step).  Elsewhere the same traffic
-    // stands in front of the activations and of the other CTAs' last copies; without it, 7B (16 layers) at 77 keys 1370 -> 1348 us, at
-    // 1536 1437 -> 1416, 13B (8 layers) 1040 -> 991, 1.1B's widths with 32 kv heads (12 layers) 486 -> 479, 1024 wide (16 layers) 457 -> 450.
-    const bool o_in_ring = cl_storage_bytes(m->cl[GK_O]) <= CL_RING_SHARE * CL_CTAS * m->cl[GK_O].ncl;
-    const bool lead = o_in_ring && kv->attn_dec && 2 * attn_dec_ctas(m) <= m->num_sms && cl_storage_bytes(m->cl[GK_GU]) > (size_t)2 * CL_BURST * CL_CTAS * m->cl[GK_GU].ncl;
-    auto chain = [&](ClEpilogue& e, unsigned own, int next, const unsigned char* w) {
-        if (!lead) return;
-        e.ahead = true; e.own_lead = own; e.next = &m->cl[next]; e.next_w = w; e.next_lead = CL_LEAD;
-    };
+    // No projection fetches the weights of the next one, or its own beyond its ring, into L2: the traffic stands in front of the activations and
+    // of the other CTAs' last copies, and the code for it is as much as that of a product loop.  us per step with and without: 7B (16
+    // layers) at 77 keys 1370 and 1348, 13B (8 layers) 1040 and 991, 1.1B at 512 keys 747 and 739, at 3000 838 and 834, 1.1B's
+    // widths with 8192 gate features and 16 query heads of 128 (12 layers) 540 and 502; the other way with 16 kv heads of 64 at 600 keys (438 and 443).
     for (int l = 0; l < c.n_layers; ++l) {
         const LayerW& w = m->layers[l];
         ClEpilogue q;
@@ -1326,29 +1318,23 @@ static anpd_status forward_cl_enqueue(anpd_model* m, anpd_kv* kv, int max_pos, b
         q.rope_cos = kv->rope_cos; q.rope_sin = kv->rope_sin; q.page_table = kv->page_table; q.pages_per_seq = kv->pages_per_seq;
         q.Hq = c.n_q_heads; q.Hkv = c.n_kv_heads; q.hd = hd; q.q_scale = 1.4426950408889634f / sqrtf((float)hd);
         q.q_hi = ws.q_hi; q.q_lo = ws.q_lo; q.kpool_l = kv->kpool + l * layer_elems; q.vpool_l = kv->vpool + l * layer_elems;
-        chain(q, l ? CL_LEAD : 0, GK_O, w.wo);
         ANPD_TRY(cl_enqueue(m->cl[GK_QKV], w.wqkv, ws.ci_h, q, ws.gemm_err, st, pf));
         if (kv->attn_dec) ANPD_TRY(attn_dec_enqueue(m, kv, l, two_candidates));
         else if (hd == 128) ANPD_TRY(attn_enqueue<128>(m, kv, l, rows, max_pos, ws.ci_ao, two_candidates, rows));
         else ANPD_TRY(attn_enqueue<64>(m, kv, l, rows, max_pos, ws.ci_ao, two_candidates, rows));
         ClEpilogue o;
         o.x = ws.x; o.gain = w.ffn_norm; o.ss_out = ws.ss_cl_b; o.d = d; o.act_out = ws.ci_h2;
-        chain(o, CL_LEAD, GK_GU, w.wgu);
         ANPD_TRY(cl_enqueue(m->cl[GK_O], w.wo, ws.ci_ao, o, ws.gemm_err, st, pf));
         ClEpilogue gu;
         gu.ss_in = ws.ss_cl_b; gu.n_parts = cl_parts(m->cl[GK_O]); gu.inv_d = 1.0f / (float)d; gu.eps = c.rms_eps; gu.act_out = ws.ci_act;
-        chain(gu, CL_LEAD, GK_DOWN, w.wd);
-        gu.own_burst = lead ? CL_BURST : 0;               // the O projection's weights are in its ring: HBM has nothing else to read (885 -> 853 us)
         ANPD_TRY(cl_enqueue(m->cl[GK_GU], w.wgu, ws.ci_h2, gu, ws.gemm_err, st, pf));
         ClEpilogue dn;
         dn.x = ws.x; dn.gain = (l + 1 < c.n_layers) ? m->layers[l + 1].attn_norm : m->final_norm; dn.ss_out = ws.ss_cl_a; dn.d = d;
         dn.act_out = ws.ci_h;
-        const bool last = l + 1 == c.n_layers;
-        chain(dn, CL_LEAD, last ? GK_LM : GK_QKV, last ? m->lm_head : m->layers[l + 1].wqkv);
         ANPD_TRY(cl_enqueue(m->cl[GK_DOWN], w.wd, ws.ci_act, dn, ws.gemm_err, st, pf));
         parts_a = cl_parts(m->cl[GK_DOWN]);
     }
-    ANPD_TRY(lm_head_cl_enqueue(m, kv, ws.ss_cl_a, parts_a, want_logits, lead, CL_LEAD));
+    ANPD_TRY(lm_head_cl_enqueue(m, kv, ws.ss_cl_a, parts_a, want_logits));
     CUDA_TRY(cudaGetLastError());
     return ANPD_OK;
 }

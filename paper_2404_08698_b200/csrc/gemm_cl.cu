@@ -15,7 +15,7 @@
 // four projections alone: 7B 405 MB in 76 us (copy rate of the device: 62 us), 1.1B 88 MB in 32 us (13.5 us).
 //
 // Roles.  A weight thread keeps a ring of copies in flight; the first ring goes out at once, while the kernel before is still
-// running (weights depend on nothing), and, where that pays, it runs ahead of the ring with L2 prefetches.  An activation thread follows behind the
+// running (weights depend on nothing).  An activation thread follows behind the
 // dependency wait.  An MMA thread multiplies tiles of up to 128 features with the rows of the step (N operand: hi terms, then lo
 // terms of the activations) into tensor memory.  Four warps read the accumulators and push each partial sum to the CTA that
 // finishes its feature (st.async: data and arrival in one), eight add the parts in CTA order and apply the epilogue.
@@ -60,13 +60,9 @@ struct ClArgs {
     const unsigned char* w;              // see ClPlan
     const unsigned char* act;            // operand image [k-block][2 * rows][64]
     int kb, gpu, n_units, ncl;
-    int seg, next_seg;                   // segments of the storage: ncl or 1
+    int seg;                             // segments of the storage: ncl or 1
     int rows, passes, copies, two, kps, stages, stage_bytes, akb, act_slots, tmem_cols, acc_bufs, acc_cols;
     int f_own_max, first;                // first: stages requested ahead of the activations
-    // the projection after this one: its storage and cut, and how many bytes per CTA are fetched into L2 ahead (own: already done)
-    const unsigned char* next_w;
-    int next_kb, next_gpu, next_units;
-    unsigned own_lead, own_burst, next_lead;
     // RMSNorm of the input
     const float* ss_in; int n_parts; float inv_d, eps;
     // rotary + append
@@ -123,9 +119,6 @@ __device__ __forceinline__ void wait_at(uint32_t bar, uint32_t parity, volatile 
     }
     *abort_flag = 1;
 }
-__device__ __forceinline__ void l2_prefetch(const void* src, uint32_t bytes) {
-    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory");
-}
 // eight columns at `hi` and eight at `lo` of this thread's tensor-memory lane, added
 __device__ __forceinline__ void tc_ld8_sum(uint32_t hi, uint32_t lo, float* v) {
     uint32_t a[8], b[8];
@@ -164,11 +157,11 @@ __device__ __forceinline__ void split2(float a, float b, uint32_t& hi, uint32_t&
     lo = (uint32_t)__bfloat16_as_ushort(la) | ((uint32_t)__bfloat16_as_ushort(lb) << 16);
 }
 
-// R: 8 = a step of one sequence (8 rows, one pass, one chunk); 0 = rows, passes and chunks from the arguments.  LEAD: runs ahead in L2.
+// R: 8 = a step of one sequence (8 rows, one pass, one chunk); 0 = rows, passes and chunks from the arguments.
 // TMAX: most tiles of a sequence's step, 1 or CL_MAX_TILES: code is time here (see launch_step)
-template <int EPI, int R, bool LEAD, int TMAX>
+template <int EPI, int R, int TMAX>
 __global__ void __launch_bounds__(cl_threads(R), 1) gemm_cl_kernel(const __grid_constant__ ClArgs g) {
-    constexpr bool LATE = R && !LEAD;                  // its CTAs start late (see CL_FIRST)
+    constexpr bool LATE = R != 0;                      // its CTAs start late (see CL_FIRST)
     constexpr bool ONE = R && TMAX == 1;
     extern __shared__ __align__(1024) unsigned char cl_smem_raw[];
     __shared__ uint64_t w_full[CL_MAX_STAGES], w_empty[CL_MAX_STAGES], a_full[CL_MAX_ACT], a_empty[CL_MAX_ACT];
@@ -271,7 +264,7 @@ __global__ void __launch_bounds__(cl_threads(R), 1) gemm_cl_kernel(const __grid_
     }
     tc_fence_before();
     // Where CTAs start late the activation thread goes on at once, past the allocation of tensor memory (7B, 16 layers, 77 keys: 1329 ->
-    // 1323 us; 1.1B, which runs ahead, lost 0.5 %, its batches 4 %).
+    // 1323 us; 1.1B's batches lost 4 %).
     if (!LATE) __syncthreads();
     else if (warp == 2) asm volatile("bar.arrive 2, %0;" ::"n"(cl_threads(R)) : "memory");
     else asm volatile("bar.sync 2, %0;" ::"n"(cl_threads(R)) : "memory");
@@ -292,54 +285,13 @@ __global__ void __launch_bounds__(cl_threads(R), 1) gemm_cl_kernel(const __grid_
             }
             int stage = 0;
             uint32_t phase = 0;
-            // One sequence, L2 prefetch: through this CTA's own weights, then its share of the next projection's, k-block by k-block
-            const unsigned end = LEAD ? (unsigned)(Gc * nk) << 10 : 0u, own_piece = g.seg == 1 ? (unsigned)Gc << 10 : end;      // piece: contiguous
-            unsigned cur = g.own_lead, left = 0, own_done = 0, nxt_piece = 0, nxt_done = 0;
-            const unsigned char *own = nullptr, *nxt = nullptr;
-            size_t nxt_step = 0;
-            if constexpr (LEAD) if (cur < end) {
-                const unsigned k = cur / own_piece;
-                own_done = cur - k * own_piece;
-                own = g.w + ((size_t)ulo * g.gpu * (g.seg == 1 ? 1 : g.kb) + (size_t)GS * (kb_lo + (int)k)) * 1024;
-            }
-            if (LEAD && g.next_w) {
-                const int nu0 = (int)((unsigned)(cluster * g.next_units) / (unsigned)g.ncl), nu1 = (int)((unsigned)((cluster + 1) * g.next_units) / (unsigned)g.ncl);
-                const int ng0 = (nu1 - nu0) * g.next_gpu, ns = (g.next_seg == 1 ? g.next_units : nu1 - nu0) * g.next_gpu;
-                const int k0 = rank * g.next_kb / C, k1 = (rank + 1) * g.next_kb / C;
-                nxt = g.next_w + ((size_t)nu0 * g.next_gpu * (g.next_seg == 1 ? 1 : g.next_kb) + (size_t)ns * k0) * 1024;
-                nxt_piece = (unsigned)ng0 << 10; nxt_step = (size_t)ns << 10;
-                left = min(g.next_lead, (unsigned)(ng0 * (k1 - k0)) << 10);
-            }
-            auto ahead = [&](unsigned bytes) {
-                if constexpr (!LEAD) return;
-                else if (cur < end) {
-                    while (bytes > 0 && cur < end) {
-                        const unsigned n = min(bytes, own_piece - own_done);
-                        l2_prefetch(own + own_done, n);
-                        cur += n; own_done += n; bytes -= n;
-                        if (own_done == own_piece) { own_done = 0; own += (size_t)GS << 10; }
-                    }
-                } else if (left) {
-                    const unsigned n = min(min(bytes, left), nxt_piece - nxt_done);
-                    l2_prefetch(nxt + nxt_done, n);
-                    left -= n; nxt_done += n;
-                    if (nxt_done == nxt_piece) { nxt_done = 0; nxt += nxt_step; }
-                }
-            };
-#pragma unroll 1
-            for (int i = 0; i < w_count; ++i) ahead((unsigned)g.stage_bytes);
-#pragma unroll 1
-            for (unsigned b = 0; LEAD && b < g.own_burst; b += g.stage_bytes) ahead((unsigned)g.stage_bytes);
 #pragma unroll 1
             while (w_p < passes) {
                 if (!mbar_wait_small(&w_empty[stage], phase, abortp)) break;
                 w_issue(stage);
-                ahead((unsigned)g.stage_bytes);
                 ++w_count;
                 if (++stage == g.stages) { stage = 0; phase ^= 1u; }
             }
-#pragma unroll 1
-            while (left) ahead(CL_STAGE_MAX);
             s_issued[0] = w_count;
         }
         __syncwarp();
@@ -777,12 +729,12 @@ __global__ void cl_image_kernel(const float* __restrict__ a, int rows, int K, un
     }
 }
 
-template <int EPI, int R, bool LEAD = false, int TMAX = CL_MAX_TILES>
+template <int EPI, int R, int TMAX = CL_MAX_TILES>
 anpd_status launch_cl(const ClArgs& g, int smem, cudaStream_t st, Profiler* prof, double bytes) {
     static bool attr_set[64] = {false};
     if (first_call_on_device(attr_set)) {
-        CUDA_TRY(cudaFuncSetAttribute(gemm_cl_kernel<EPI, R, LEAD, TMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, CL_SMEM_MAX));
-        CUDA_TRY(cudaFuncSetAttribute(gemm_cl_kernel<EPI, R, LEAD, TMAX>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared));
+        CUDA_TRY(cudaFuncSetAttribute(gemm_cl_kernel<EPI, R, TMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, CL_SMEM_MAX));
+        CUDA_TRY(cudaFuncSetAttribute(gemm_cl_kernel<EPI, R, TMAX>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared));
     }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(g.ncl * CL_CTAS); cfg.blockDim = dim3(cl_threads(R)); cfg.dynamicSmemBytes = smem; cfg.stream = st;
@@ -800,7 +752,7 @@ anpd_status launch_cl(const ClArgs& g, int smem, cudaStream_t st, Profiler* prof
     }
     cfg.attrs = attr;
     cfg.numAttrs = n;
-    LAUNCH(prof, st, KC_GEMM, bytes, (cudaLaunchKernelEx(&cfg, gemm_cl_kernel<EPI, R, LEAD, TMAX>, g)));
+    LAUNCH(prof, st, KC_GEMM, bytes, (cudaLaunchKernelEx(&cfg, gemm_cl_kernel<EPI, R, TMAX>, g)));
     CUDA_TRY(cudaGetLastError());
     return ANPD_OK;
 }
@@ -809,9 +761,8 @@ anpd_status launch_cl(const ClArgs& g, int smem, cudaStream_t st, Profiler* prof
 // layer; with one instance for any tile count and unrolled waits and loops (43 to 54 KB of code, now 25 to 46) us per step were: 1.1B at 512
 // keys 776, now 744, tiny 55, now 48, 1024 wide (16 layers) 428, now 379, 7B (16 layers, 77 keys) 1317, now 1301.
 template <int EPI>
-anpd_status launch_step(const ClArgs& g, bool lead, int smem, cudaStream_t st, Profiler* prof, double bytes) {
-    if (g.copies == 1) return lead ? launch_cl<EPI, 8, true, 1>(g, smem, st, prof, bytes) : launch_cl<EPI, 8, false, 1>(g, smem, st, prof, bytes);
-    return lead ? launch_cl<EPI, 8, true>(g, smem, st, prof, bytes) : launch_cl<EPI, 8>(g, smem, st, prof, bytes);
+anpd_status launch_step(const ClArgs& g, int smem, cudaStream_t st, Profiler* prof, double bytes) {
+    return g.copies == 1 ? launch_cl<EPI, 8, 1>(g, smem, st, prof, bytes) : launch_cl<EPI, 8>(g, smem, st, prof, bytes);
 }
 
 }  // namespace
@@ -819,7 +770,7 @@ anpd_status launch_step(const ClArgs& g, bool lead, int smem, cudaStream_t st, P
 // Clusters that can be resident together, at most 32: the decoder family's dimensions are multiples of 32 units, so 32 clusters
 // get equal shares, where the 33 a B200's 148 SMs hold would leave some with a unit more than the rest.
 int cl_clusters() {
-    if (cudaFuncSetAttribute(gemm_cl_kernel<CL_RAW, 8, false, CL_MAX_TILES>, cudaFuncAttributeMaxDynamicSharedMemorySize, CL_SMEM_MAX) != cudaSuccess) { cudaGetLastError(); return 0; }
+    if (cudaFuncSetAttribute(gemm_cl_kernel<CL_RAW, 8, CL_MAX_TILES>, cudaFuncAttributeMaxDynamicSharedMemorySize, CL_SMEM_MAX) != cudaSuccess) { cudaGetLastError(); return 0; }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(32 * CL_CTAS); cfg.blockDim = dim3(cl_threads(8)); cfg.dynamicSmemBytes = CL_SMEM_MAX;
     cudaLaunchAttribute attr[1];
@@ -827,7 +778,7 @@ int cl_clusters() {
     attr[0].val.clusterDim.x = CL_CTAS; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr; cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, gemm_cl_kernel<CL_RAW, 8, false, CL_MAX_TILES>, &cfg) != cudaSuccess) { cudaGetLastError(); return 0; }
+    if (cudaOccupancyMaxActiveClusters(&n, gemm_cl_kernel<CL_RAW, 8, CL_MAX_TILES>, &cfg) != cudaSuccess) { cudaGetLastError(); return 0; }
     return std::min(n, 32);
 }
 
@@ -944,16 +895,14 @@ anpd_status cl_enqueue(const ClPlan& p, const unsigned char* w, const unsigned c
     g.q_hi = e.q_hi; g.q_lo = e.q_lo; g.kpool = e.kpool_l; g.vpool = e.vpool_l;
     g.x = e.x; g.gain = e.gain; g.ss_out = e.ss_out; g.d = e.d; g.act_out = e.act_out;
     g.out = e.out; g.amax_val = e.amax_val; g.amax_idx = e.amax_idx;
-    if (e.next) { g.next_w = e.next_w; g.next_kb = e.next->kb; g.next_gpu = e.next->gpu; g.next_units = e.next->n_units; g.next_seg = e.next->seg; g.next_lead = e.next_lead; }
-    g.own_lead = e.own_lead; g.own_burst = e.own_burst;
     g.err = err;
     const double bytes = 2.0 * (double)p.N * (double)p.K;
     switch (p.kind) {
-        case CL_RAW: return launch_step<CL_RAW>(g, false, smem, st, prof, bytes);
-        case CL_QKV: return launch_step<CL_QKV>(g, e.ahead, smem, st, prof, bytes);
-        case CL_RESID: return launch_step<CL_RESID>(g, e.ahead, smem, st, prof, bytes);
-        case CL_GU: return launch_step<CL_GU>(g, e.ahead, smem, st, prof, bytes);
-        case CL_LM: return launch_step<CL_LM>(g, e.ahead, smem, st, prof, bytes);
+        case CL_RAW: return launch_step<CL_RAW>(g, smem, st, prof, bytes);
+        case CL_QKV: return launch_step<CL_QKV>(g, smem, st, prof, bytes);
+        case CL_RESID: return launch_step<CL_RESID>(g, smem, st, prof, bytes);
+        case CL_GU: return launch_step<CL_GU>(g, smem, st, prof, bytes);
+        case CL_LM: return launch_step<CL_LM>(g, smem, st, prof, bytes);
     }
     return ANPD_ERR_ARG;
 }

@@ -233,11 +233,7 @@ anpd_status rr_enqueue(int epi, const RRPlan& p, const unsigned char* w, const u
 // What a projection does with its results: plain output, rotary embedding + append, residual add, SwiGLU, vocabulary argmax.
 enum ClKind { CL_RAW = 0, CL_QKV = 1, CL_RESID = 2, CL_GU = 3, CL_LM = 4 };
 constexpr int CL_CTAS = 4;             // CTAs per cluster
-// Bytes per CTA fetched into L2 ahead of the next projection, where that pays (see forward_cl_enqueue).
 constexpr int CL_PROMPT_ROWS = 128;       // prompt passes of up to this many rows use the decode projections
-constexpr unsigned CL_LEAD = 64 * 1024;
-constexpr unsigned CL_BURST = 128 * 1024;
-constexpr size_t CL_RING_SHARE = 96 * 1024;       // a CTA's weights that go out with the first ring of copies
 // Storage of an [N][K] weight matrix and its cut over the clusters of a decode projection.  The features are kept in an order
 // in which those that make one result together are neighbours: eight rotary pairs (dimensions i.., then i + hd/2..) or eight
 // gate features and their eight up features make a unit of two groups of 8; elsewhere a unit is one group.  Cluster c owns the
@@ -302,10 +298,6 @@ struct ClEpilogue {                    // only the fields of the projection's ki
     float* x = nullptr; const float* gain = nullptr; float* ss_out = nullptr; int d = 0;
     unsigned char* act_out = nullptr;
     float* out = nullptr; float* amax_val = nullptr; int* amax_idx = nullptr;
-    // weights the projection fetches into L2 for the one after it, per CTA, and what was fetched for it the same way
-    const ClPlan* next = nullptr; const unsigned char* next_w = nullptr; unsigned next_lead = 0, own_lead = 0;
-    bool ahead = false;                 // whether it runs ahead of its own copies in L2, from own_lead on
-    unsigned own_burst = 0;             // what the projection fetches into L2 of its own weights at its start, beyond that
 };
 int cl_clusters();                      // clusters the current device runs at once, at most 32 (0: none, or no device)
 void cl_make_plan(ClPlan* p, int kind, int N, int K, int hd, int F, int ncl);
@@ -540,7 +532,6 @@ anpd_status accept_enqueue(anpd_model* m, anpd_kv* kv, int mode, const NgramDev*
 // tree: the rows carry cache slots and hidden slot ranges of their own (two-candidate steps)
 anpd_status attn_tc_enqueue(anpd_model* m, anpd_kv* kv, int layer, int rows, int max_pos, bool tree = false);
 // attn_dec.cu: attention of a decode step, written straight to the O projection's operand image
-int attn_dec_ctas(const anpd_model* m);          // its CTAs for a single sequence
 anpd_status attn_dec_enqueue(anpd_model* m, anpd_kv* kv, int layer, bool tree);
 // attn_pf.cu: attention of a prompt pass with 128 query rows per CTA (head dimension 128, one query head per kv head)
 anpd_status attn_pf_enqueue(anpd_model* m, anpd_kv* kv, int layer, int rows, unsigned char* img, int n_seq);
