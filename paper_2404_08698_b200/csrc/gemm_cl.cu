@@ -49,11 +49,11 @@ constexpr int CL_SMEM_PAIR = 112 * 1024; // two CTAs of this size share an SM
 constexpr int CL_SMEM_MAX = 216 * 1024;
 constexpr int CL_RING_BYTES = 8 * CL_STAGE_MAX;      // copies in flight per SM
 // A CTA that has its SM for itself starts as the one before leaves, when the activations are about to be ready: its first ring, 128 KB
-// requested at once, would stand in front of them (2.3 us at the device's rate).  So it requests a few stages and the others once the
-// first activations are on their way, or after a while, where the kernel before still has its tail to run.  7B, 16 layers: 77 keys
-// 1339 -> 1321 us per step, 1536 keys 1412 -> 1391 (two stages 1326 and 1395, four 1333 and 1400).
+// requested at once, would stand in front of them (2.3 us at the device's rate).  So it requests a few stages, and the others once tensor
+// memory is allocated, by when the activation thread is past its wait or about to be (a further wait for its first copy, of 500 to 6000
+// cycles at most, changed nothing).  us per step against the whole ring at once: 7B (16 layers) at 77 keys 1311 -> 1295, at 1536 1389 ->
+// 1374, 3072 wide (12 layers) 722 -> 712; 13B (8 layers) 987 -> 995.  Four stages give the same, two lost 5 us at 7B.
 constexpr int CL_FIRST = 3;
-constexpr int CL_HOLD = 1500;            // cycles
 constexpr int CL_ERR_TIMEOUT = 207;
 
 struct ClArgs {
@@ -62,7 +62,7 @@ struct ClArgs {
     int kb, gpu, n_units, ncl;
     int seg;                             // segments of the storage: ncl or 1
     int rows, passes, copies, two, kps, stages, stage_bytes, akb, act_slots, tmem_cols, acc_bufs, acc_cols;
-    int f_own_max, first;                // first: stages requested ahead of the activations
+    int f_own_max, first;                // first: stages requested before tensor memory is allocated
     // RMSNorm of the input
     const float* ss_in; int n_parts; float inv_d, eps;
     // rotary + append
@@ -161,13 +161,12 @@ __device__ __forceinline__ void split2(float a, float b, uint32_t& hi, uint32_t&
 // TMAX: most tiles of a sequence's step, 1 or CL_MAX_TILES: code is time here (see launch_step)
 template <int EPI, int R, int TMAX>
 __global__ void __launch_bounds__(cl_threads(R), 1) gemm_cl_kernel(const __grid_constant__ ClArgs g) {
-    constexpr bool LATE = R != 0;                      // its CTAs start late (see CL_FIRST)
     constexpr bool ONE = R && TMAX == 1;
     extern __shared__ __align__(1024) unsigned char cl_smem_raw[];
     __shared__ uint64_t w_full[CL_MAX_STAGES], w_empty[CL_MAX_STAGES], a_full[CL_MAX_ACT], a_empty[CL_MAX_ACT];
     __shared__ uint64_t acc_full[2], acc_empty[2], red_full;
     __shared__ uint32_t tmem_slot;
-    __shared__ int abort_flag, s_issued[2], s_acts;
+    __shared__ int abort_flag, s_issued[2];
     __shared__ float s_rstd[8], s_part[8][8];
     __shared__ int s_pos[8], s_slot[8], s_page[8], s_idx[8][8];
 
@@ -232,26 +231,26 @@ __global__ void __launch_bounds__(cl_threads(R), 1) gemm_cl_kernel(const __grid_
 
     if (warp == 0) {
         if (elect_one()) {
-            if (!LATE) { abort_flag = 0; s_issued[0] = 0; s_issued[1] = 0; }
+            if (!R) { abort_flag = 0; s_issued[0] = 0; s_issued[1] = 0; }
 #pragma unroll 1
             for (int s = 0; s < g.stages; ++s) { mbar_init(&w_full[s], 1); mbar_init(&w_empty[s], 1); }
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            // the weights depend on nothing: the first ring is requested before anything else happens
+            // the weights depend on nothing: the first of them are requested before anything else happens
             w_enter();
 #pragma unroll 1
-            for (; w_count < (LATE ? g.first : g.stages) && w_p < passes; ++w_count) w_issue(w_count);
+            for (; w_count < (R && !ONE ? g.first : g.stages) && w_p < passes; ++w_count) w_issue(w_count);
         }
         __syncwarp();
-    } else if (LATE ? warp == 2 : threadIdx.x == 64) {
-        if (!LATE || elect_one()) {
-            if (LATE) { abort_flag = 0; s_issued[0] = 0; s_issued[1] = 0; s_acts = 0; }
+    } else if (R ? warp == 2 : threadIdx.x == 64) {
+        if (!R || elect_one()) {
+            if (R) { abort_flag = 0; s_issued[0] = 0; s_issued[1] = 0; }
 #pragma unroll 1
             for (int s = 0; s < g.act_slots; ++s) { mbar_init(&a_full[s], 1); mbar_init(&a_empty[s], 1); }
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         }
-        if (LATE) __syncwarp();
+        if (R) __syncwarp();
     } else if (threadIdx.x == 96) {
         for (int b = 0; b < 2; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], 4); }
         mbar_init(&red_full, 1);
@@ -263,14 +262,14 @@ __global__ void __launch_bounds__(cl_threads(R), 1) gemm_cl_kernel(const __grid_
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     tc_fence_before();
-    // Where CTAs start late the activation thread goes on at once, past the allocation of tensor memory (7B, 16 layers, 77 keys: 1329 ->
+    // In a sequence's step the activation thread goes on at once, past the allocation of tensor memory (7B, 16 layers, 77 keys: 1329 ->
     // 1323 us; 1.1B's batches lost 4 %).
-    if (!LATE) __syncthreads();
+    if (!R) __syncthreads();
     else if (warp == 2) asm volatile("bar.arrive 2, %0;" ::"n"(cl_threads(R)) : "memory");
     else asm volatile("bar.sync 2, %0;" ::"n"(cl_threads(R)) : "memory");
     tc_fence_after();
     // Only now may the next kernel start beside this one: its tensor-memory allocation must not come before this CTA's.
-    if (!LATE || warp != 2) pdl_trigger();
+    if (!R || warp != 2) pdl_trigger();
     if (R) cluster_arrive();                           // waited for before the first push: every CTA's barriers are initialised then
     const uint32_t tmem_base = *((volatile uint32_t*)&tmem_slot);
     volatile int* abortp = &abort_flag;
@@ -278,8 +277,7 @@ __global__ void __launch_bounds__(cl_threads(R), 1) gemm_cl_kernel(const __grid_
     if (warp == 0) {
         // ---------------- weights ----------------
         if (elect_one()) {
-            if (LATE && g.first < g.stages) {
-                for (const long long t = clock64(); !*(volatile int*)&s_acts && clock64() - t < CL_HOLD;) {}
+            if constexpr (R && !ONE) {                  // (one tile: the CTA is beside another, and the ring has gone out)
 #pragma unroll 1
                 for (; w_count < g.stages && w_p < passes; ++w_count) w_issue(w_count);
             }
@@ -314,7 +312,6 @@ __global__ void __launch_bounds__(cl_threads(R), 1) gemm_cl_kernel(const __grid_
                     const uint32_t bytes = (uint32_t)(min(g.akb, nk - k) * rows) * 256u;
                     mbar_expect_tx(&a_full[slot], bytes);
                     bulk_load(abuf + slot * act_slot, g.act + (size_t)(kb_lo + k) * rows * 256, bytes, &a_full[slot], pol_a);
-                    if (LATE && count == 0) *(volatile int*)&s_acts = 1;
                     ++count;
                     if (++slot == g.act_slots) { slot = 0; phase ^= 1u; }
                 }
