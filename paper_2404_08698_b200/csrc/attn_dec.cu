@@ -157,7 +157,7 @@ __global__ void __launch_bounds__((AdCfg<HD, G>::THREADS)) __maxnreg__((AdCfg<HD
                 if (!waited && (p + 1) * KV_PAGE > first_new) { pdl_wait(); waited = true; }       // holds rows the kernel before writes
 #pragma unroll
                 for (int half = 0; half < 2; ++half) {
-                    if (count >= CHUNKS && ok) ok = mbar_wait_small(&empty[stage], phase, abortp);
+                    if (count >= CHUNKS && ok) ok = mbar_wait<1>(&empty[stage], phase, abortp);
                     if (!ok) break;
                     unsigned char* dst = ring + (size_t)stage * CHUNK;
                     mbar_expect_tx(&full[stage], CHUNK);
@@ -269,8 +269,7 @@ __global__ void __launch_bounds__((AdCfg<HD, G>::THREADS)) __maxnreg__((AdCfg<HD
             }
             // rolled, this wait costs head dimension 128 registers it does not have at its cap (24 bytes spilled); 64 has them and loses 0.15 % of a
             // 1.1B step by the unrolled one's code (7B, 16 layers, 1536 keys: 1368 us per step with the spill, 1366 without, both +- 5)
-            if (HD == 128) mbar_wait(&full[cv], par_v, abortp);
-            else mbar_wait_small(&full[cv], par_v, abortp);
+            mbar_wait<HD == 128 ? 16 : 1>(&full[cv], par_v, abortp);
             const uint32_t vr = ring_addr + (uint32_t)cv * (uint32_t)CHUNK + kv_off + (uint32_t)((key_page >> 6) * (HD * 128)) + ((((uint32_t)((key_page & 63) >> 3) + chunk0) ^ (uint32_t)lr) << 4);
 #pragma unroll
             for (int d = 0; d < DT / 2; ++d) {
@@ -295,9 +294,9 @@ __global__ void __launch_bounds__((AdCfg<HD, G>::THREADS)) __maxnreg__((AdCfg<HD
             const int cv = stage;
             const uint32_t par_v = par;
             if (++stage == CHUNKS) { stage = 0; par ^= 1u; }
-            mbar_wait_small(&full[ck], par_k, abortp);
+            mbar_wait<1>(&full[ck], par_k, abortp);
             if (p * KV_PAGE + warp * AD_KEYS <= pos_hi) block(ck, cv, par_v, warp * AD_KEYS, p);
-            else { if (lane == 0) mbar_arrive(&empty[ck]); mbar_wait_small(&full[cv], par_v, abortp); }
+            else { if (lane == 0) mbar_arrive(&empty[ck]); mbar_wait<1>(&full[cv], par_v, abortp); }
             __syncwarp();
             if (lane == 0) mbar_arrive(&empty[cv]);
         }

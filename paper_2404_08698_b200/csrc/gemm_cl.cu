@@ -107,18 +107,6 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity
     *abort_flag = 1;
     return false;
 }
-// by the barrier's address, with little code (see mbar_wait_small)
-__device__ __forceinline__ void wait_at(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
-#pragma unroll 1
-    for (unsigned i = 0; i < WAIT_LIMIT; ++i) {
-        uint32_t ok;
-        asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-                     : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-        if (ok) return;
-        if ((i & 1023u) == 1023u && *abort_flag) return;
-    }
-    *abort_flag = 1;
-}
 // eight columns at `hi` and eight at `lo` of this thread's tensor-memory lane, added
 __device__ __forceinline__ void tc_ld8_sum(uint32_t hi, uint32_t lo, float* v) {
     uint32_t a[8], b[8];
@@ -285,7 +273,7 @@ __global__ void __launch_bounds__(cl_threads(R), 1) gemm_cl_kernel(const __grid_
             uint32_t phase = 0;
 #pragma unroll 1
             while (w_p < passes) {
-                if (!mbar_wait_small(&w_empty[stage], phase, abortp)) break;
+                if (!mbar_wait<1>(&w_empty[stage], phase, abortp)) break;
                 w_issue(stage);
                 ++w_count;
                 if (++stage == g.stages) { stage = 0; phase ^= 1u; }
@@ -307,7 +295,7 @@ __global__ void __launch_bounds__(cl_threads(R), 1) gemm_cl_kernel(const __grid_
                 if (up == 0) continue;
 #pragma unroll 1
                 for (int k = 0; k < nk; k += g.akb) {
-                    if (count >= g.act_slots) ok = mbar_wait_small(&a_empty[slot], phase, abortp);
+                    if (count >= g.act_slots) ok = mbar_wait<1>(&a_empty[slot], phase, abortp);
                     if (!ok) break;
                     const uint32_t bytes = (uint32_t)(min(g.akb, nk - k) * rows) * 256u;
                     mbar_expect_tx(&a_full[slot], bytes);
@@ -344,14 +332,14 @@ __global__ void __launch_bounds__(cl_threads(R), 1) gemm_cl_kernel(const __grid_
                 int u0, up;
                 pass_of(p, u0, up);
                 const int G = up * g.gpu, T = copies_of(G), base = !R && T ? G / T : 0, rem = !R && T ? G - base * T : 0;
-                if (p >= g.acc_bufs) mbar_wait_small(&acc_empty[buf], eph, abortp);
+                if (p >= g.acc_bufs) mbar_wait<1>(&acc_empty[buf], eph, abortp);
                 tc_fence_after();
                 const uint32_t d0 = tmem_base + (uint32_t)(buf * g.acc_cols);
                 uint32_t acc = 0;
                 const int k_end = T > 0 ? nk : 0;
 #pragma unroll 1
                 for (int k0 = 0; k0 < k_end; k0 += akb) {
-                    wait_at(afull, aph, abortp);
+                    mbar_wait_at<1>(afull, aph, abortp);
                     const int kend = min(akb, nk - k0);
                     uint32_t a = a_lo;
                     // a tile of fewer than 16 groups: the instruction reads whatever follows for the rows beyond, whose lanes nobody reads
@@ -362,7 +350,7 @@ __global__ void __launch_bounds__(cl_threads(R), 1) gemm_cl_kernel(const __grid_
 #pragma unroll 1
                             for (int t = 0; t < T; ++t) {
                                 const uint32_t first = (uint32_t)(base + (t < rem ? 2 : 1)) >> 1;       // groups of the copy's first tile
-                                wait_at(full, wph, abortp);
+                                mbar_wait_at<1>(full, wph, abortp);
                                 tc_fence_after();
                                 tc_mma_k64(d_tmem, w_lo, a, idesc, acc);
                                 tc_mma_k64(d_tmem + (uint32_t)(2 * rows), w_lo + (first << 6), a, idesc, acc);
@@ -378,7 +366,7 @@ __global__ void __launch_bounds__(cl_threads(R), 1) gemm_cl_kernel(const __grid_
                             uint32_t d_tmem = d0;
 #pragma unroll 1
                             for (int t = T; t > 0; --t) {
-                                wait_at(full, wph, abortp);
+                                mbar_wait_at<1>(full, wph, abortp);
                                 tc_fence_after();
                                 tc_mma_k64(d_tmem, w_lo, a, idesc, acc);
                                 next_stage();
@@ -390,7 +378,7 @@ __global__ void __launch_bounds__(cl_threads(R), 1) gemm_cl_kernel(const __grid_
                     } else {                                            // kps k-blocks of the only tile per stage
 #pragma unroll 1
                         for (int k = 0; k < kend; k += kps) {
-                            wait_at(full, wph, abortp);
+                            mbar_wait_at<1>(full, wph, abortp);
                             tc_fence_after();
                             tc_mma_k64(d0, w_lo, a, idesc, acc);
                             acc = 1;
@@ -483,7 +471,7 @@ __global__ void __launch_bounds__(cl_threads(R), 1) gemm_cl_kernel(const __grid_
         cluster_wait();
 
         if (pushes) {
-            mbar_wait_small(&acc_full[0], 0, abortp);
+            mbar_wait<1>(&acc_full[0], 0, abortp);
             tc_fence_after();
             const uint32_t col0 = tmem_base + ((uint32_t)(quad * 32) << 16);
 #pragma unroll
@@ -517,7 +505,6 @@ __global__ void __launch_bounds__(cl_threads(R), 1) gemm_cl_kernel(const __grid_
         if (EPI == CL_RESID) {
             float ssq = 0.0f;
 #pragma unroll 1
-#pragma unroll 1
             for (int idx = ft; idx < on * 32; idx += 256) {
                 const int f = 2 * (idx >> 3), n = ufirst * 8 + f;
                 float2 x = pf, gn = pg;
@@ -544,7 +531,6 @@ __global__ void __launch_bounds__(cl_threads(R), 1) gemm_cl_kernel(const __grid_
         } else if (EPI == CL_GU) {
             const float rs = s_rstd[row];
 #pragma unroll 1
-#pragma unroll 1
             for (int idx = ft; idx < on * 32; idx += 256) {
                 const int ul = idx >> 5, e = 2 * ((idx >> 3) & 3), f = ul * 16 + e, k = (ufirst + ul) * 8 + e;
                 float v[2];
@@ -561,7 +547,6 @@ __global__ void __launch_bounds__(cl_threads(R), 1) gemm_cl_kernel(const __grid_
         } else if (EPI == CL_QKV) {
             const float rs = s_rstd[row];
             const int pos = s_pos[row], slot = s_slot[row], page = s_page[row], upi = g.hd >> 4;
-#pragma unroll 1
 #pragma unroll 1
             for (int idx = ft; idx < on * 32; idx += 256) {
                 const int ul = idx >> 5, e = 2 * ((idx >> 3) & 3), u = ufirst + ul, head = u / upi, i = (u - head * upi) * 8 + e;
@@ -606,7 +591,6 @@ __global__ void __launch_bounds__(cl_threads(R), 1) gemm_cl_kernel(const __grid_
             float best = -CUDART_INF_F;
             int bidx = 0x7fffffff;
 #pragma unroll 1
-#pragma unroll 1
             for (int idx = ft; idx < on * 64; idx += 256) {
                 const int f = idx >> 3, n = ufirst * 8 + f;
                 if (n >= g.n_out) continue;
@@ -641,7 +625,7 @@ __global__ void __launch_bounds__(cl_threads(R), 1) gemm_cl_kernel(const __grid_
             int u0, up;
             pass_of(p, u0, up);
             const int G = up * g.gpu, T = copies_of(G), base = T ? G / T : 0, rem = T ? G - base * T : 0, per = g.two ? 2 : 1;
-            mbar_wait_small(&acc_full[buf], bph, abortp);
+            mbar_wait<1>(&acc_full[buf], bph, abortp);
             tc_fence_after();
             int t0 = (ulo + u0) * g.gpu;                // the tile's first group
             for (int t = 0; t < T * per; ++t) {
