@@ -14,10 +14,10 @@
 // one's first activation load, 0.5 us for that load, 1.5 us from the last product to the last store.  Measured per layer, the
 // four projections alone: 7B 405 MB in 76 us (copy rate of the device: 62 us), 1.1B 88 MB in 32 us (13.5 us).
 //
-// Roles.  A weight thread keeps a ring of copies in flight; the first ring goes out at once, while the kernel before is still
-// running (weights depend on nothing).  An activation thread follows behind the
-// dependency wait.  An MMA thread multiplies tiles of up to 128 features with the rows of the step (N operand: hi terms, then lo
-// terms of the activations) into tensor memory.  Four warps read the accumulators and push each partial sum to the CTA that
+// Roles.  A weight thread keeps a ring of copies in flight; the first of them go out while the kernel before is still running (weights
+// depend on nothing): all that the ring holds where CTAs share an SM, three where a step's CTA has one for itself (see CL_FIRST).
+// An activation thread follows behind the dependency wait.  An MMA thread multiplies tiles of up to 128 features with the rows of
+// the step (N operand: hi terms, then lo terms of the activations) into tensor memory.  Four warps read the accumulators and push each partial sum to the CTA that
 // finishes its feature (st.async: data and arrival in one), eight add the parts in CTA order and apply the epilogue.
 // The single threads must keep up with a 16 KB copy every 600 cycles: they are elected, not picked by lane number (see elect_one),
 // walk their sequences with additions only (an integer division costs about a hundred cycles there) and keep only the low words
@@ -853,8 +853,8 @@ static anpd_status cl_args(ClArgs* g, const ClPlan& p, const unsigned char* w, c
     const int room = (pair ? CL_SMEM_PAIR : CL_SMEM_MAX) - rest;
     g->stages = std::min(CL_MAX_STAGES, std::min(room, CL_RING_BYTES) / g->stage_bytes);
     if (g->stages < 2) return ANPD_ERR_CAPACITY;
-    // the M = 128 instruction reads 16 KB from the last tile of the last stage on, whatever the tile holds
     g->first = one && !pair ? std::min(CL_FIRST, g->stages) : g->stages;
+    // the M = 128 instruction reads 16 KB from the last tile of the last stage on, whatever the tile holds
     const int need = g->stages * g->stage_bytes + std::max(rest, CL_STAGE_MAX + 1024);
     // Two CTAs that share an SM take half of its shared memory each, whatever they need: with unequal halves the next kernel's
     // CTA finds the space its predecessor's predecessor left too small.

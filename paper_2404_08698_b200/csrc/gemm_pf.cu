@@ -65,7 +65,7 @@ __device__ __forceinline__ void pf_item(const PfArgs& g, int item, int& ot, int&
 }
 
 // GU: the gate-up projection.  A tile in one part is finished here: eight lanes hold gate features, the next eight their up features, so
-// that a lane pair turns two rows' sums into one activation each.  That writes a quarter of the sums' bytes and saves the kernel behind.
+// that a lane pair turns two rows' sums into one activation each.  That writes half of the sums' bytes, and nobody reads the sums again.
 template <bool GU>
 __global__ void __launch_bounds__(PF_THREADS, 1)
 gemm_pf_kernel(const unsigned char* __restrict__ w, const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ CUtensorMap map_lo,
