@@ -1309,7 +1309,8 @@ static anpd_status forward_cl_enqueue(anpd_model* m, anpd_kv* kv, int max_pos, b
     // No projection fetches the weights of the next one, or its own beyond its ring, into L2: the traffic stands in front of the activations and
     // of the other CTAs' last copies, and the code for it is as much as that of a product loop.  us per step with and without: 7B (16
     // layers) at 77 keys 1370 and 1348, 13B (8 layers) 1040 and 991, 1.1B at 512 keys 747 and 739, at 3000 838 and 834, 1.1B's
-    // widths with 8192 gate features and 16 query heads of 128 (12 layers) 540 and 502; the other way with 16 kv heads of 64 at 600 keys (438 and 443).
+    // widths with 8192 gate features and 16 query heads of 128 (12 layers) 540 and 502; with 16 kv heads of 64 at 600 keys no more than the runs' own
+    // spread (438 and 431 to 443).
     for (int l = 0; l < c.n_layers; ++l) {
         const LayerW& w = m->layers[l];
         ClEpilogue q;
