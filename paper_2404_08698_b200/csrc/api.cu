@@ -429,6 +429,7 @@ anpd_status anpd_kv_create(const anpd_model* cm, int max_len, int batch, int shu
     kv->attn_pf = kv->attn_dec && std::getenv("ANPD_ATTN_PROMPT_TILE16") == nullptr;
     for (int k = 0; k < GK_COUNT; ++k) ws.ld[k] = (m->plan[k].N + 127) / 128 * 128;
     ws.pf_rows = 0;
+    ws.xch_bytes = kv->attn_dec ? step_cl_bytes(m, batch) : 0;
     ws.amax_nblk = ws.amax_blocks = (c.vocab + 1023) / 1024;
     const size_t d = c.d_model, F = c.d_ffn, V = c.vocab, hd = c.head_dim, half = hd / 2;
     const size_t pool = (size_t)c.n_layers * kv->total_pages * c.n_kv_heads * KV_PAGE * hd * 2;
@@ -466,6 +467,7 @@ anpd_status anpd_kv_create(const anpd_model* cm, int max_len, int batch, int shu
             {(void**)&ws.ci_ao, cl_img_bytes(S, m->dq)}, {(void**)&ws.ci_act, cl_img_bytes(S, c.d_ffn)},
             {(void**)&ws.ss_cl_a, (size_t)cl_parts(m->cl[GK_DOWN]) * ANPD_ROWS * 4}, {(void**)&ws.ss_cl_b, (size_t)cl_parts(m->cl[GK_O]) * ANPD_ROWS * 4},
             {(void**)&ws.amax_val_cl, (size_t)cl_parts(m->cl[GK_LM]) * ANPD_ROWS * 4}, {(void**)&ws.amax_idx_cl, (size_t)cl_parts(m->cl[GK_LM]) * ANPD_ROWS * 4},
+            {(void**)&ws.xch, ws.xch_bytes},
             {(void**)&ws.ss_a, (size_t)m->num_sms * ANPD_ROWS * 4}, {(void**)&ws.ss_b, (size_t)m->num_sms * ANPD_ROWS * 4},
             {(void**)&ws.amax_val_rr, (size_t)m->num_sms * ANPD_ROWS * 4}, {(void**)&ws.amax_idx_rr, (size_t)m->num_sms * ANPD_ROWS * 4},
         };
@@ -547,6 +549,7 @@ anpd_status anpd_kv_create(const anpd_model* cm, int max_len, int batch, int shu
     }
     cudaStream_t st = m->stream;
     bool ok = cudaMemsetAsync(kv->slab, 0, kv->slab_bytes, st) == cudaSuccess;
+    if (ws.xch_bytes) ok = ok && cudaMemsetAsync(ws.xch, 0xff, ws.xch_bytes, st) == cudaSuccess;
     ok = ok && cudaMemcpyAsync(kv->page_table, pt.data(), pt.size() * 4, cudaMemcpyHostToDevice, st) == cudaSuccess;
     ok = ok && cudaMemcpyAsync(kv->rope_cos, hc.data(), hc.size() * 4, cudaMemcpyHostToDevice, st) == cudaSuccess;
     ok = ok && cudaMemcpyAsync(kv->rope_sin, hs.data(), hs.size() * 4, cudaMemcpyHostToDevice, st) == cudaSuccess;
@@ -686,7 +689,7 @@ static anpd_status read_seqs(anpd_kv* kv, float* logits_host = nullptr, int rows
     CUDA_TRY(cudaStreamSynchronize(kv->m->stream));
     for (int b = 0; b < kv->batch; ++b) { kv->h_kv_len[b] = kv->h_seq[b].kv_len; kv->h_len_stale[b] = 0; }
     if (*h_err != 0) {
-        std::snprintf(g_last_error, sizeof(g_last_error), "a kernel gave up waiting on a barrier (code %d: 201 GEMM, 202 attention, 204 step kernel, 205 prompt GEMM, 206 prompt attention, 207 decode projection, 208 decode attention)", *h_err);
+        std::snprintf(g_last_error, sizeof(g_last_error), "a kernel gave up waiting on a barrier (code %d: 201 GEMM, 202 attention, 204 step kernel, 205 prompt GEMM, 206 prompt attention, 207 decode projection, 208 decode attention, 209 step)", *h_err);
         return ANPD_ERR_CUDA;
     }
     return ANPD_OK;

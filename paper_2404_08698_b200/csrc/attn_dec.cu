@@ -21,7 +21,7 @@
 // enter as two bf16 terms; with one query head the two terms of the 8 rows are the tile's 16 rows.  The scores are summed in two
 // chains, which halves the wait for the products (7B at 1536 keys: 1104 -> 1089 us for 12 layers and the head).
 #include "internal.h"
-#include "tc_ptx.cuh"
+#include "step_dev.cuh"
 
 #include <math_constants.h>
 
@@ -29,11 +29,23 @@
 
 typedef __nv_bfloat16 bf16;
 
+// CTAs per head, and clusters that share a kv head
+constexpr int AD_MAX_CLUSTER = 4;
+int ad_cluster(const anpd_model* m, int heads) {
+    const int resident = m->num_sms * 7 / 8;
+    int cluster = AD_MAX_CLUSTER;
+    while (cluster > 1 && heads * cluster > resident) cluster /= 2;
+    return cluster;
+}
+int ad_split(const anpd_model_config& c) {
+    const int group = c.n_q_heads / c.n_kv_heads;
+    return c.head_dim == 64 && group > 1 ? group / 2 : group;
+}
+
 namespace {
 
 using namespace tc;
 
-constexpr int AD_MAX_CLUSTER = 4;
 constexpr int AD_KEYS = 16;              // keys per block
 constexpr int AD_MAX_CHUNKS = 6;
 constexpr int AD_SMEM_PAIR = 111 * 1024; // two CTAs share an SM: another one of these, or one of the projection before or after
@@ -70,35 +82,7 @@ struct AdArgs {
     int* err;
 };
 
-__device__ __forceinline__ void ad_mma(float* c, const uint32_t* a, uint32_t b0, uint32_t b1) {
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
-                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-__device__ __forceinline__ void ad_ldm4(uint32_t addr, uint32_t* r) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
-}
-__device__ __forceinline__ uint32_t ad_split(float x, float y, uint32_t& lo) {
-    const bf16 hx = __float2bfloat16_rn(x), hy = __float2bfloat16_rn(y);
-    const bf16 lx = __float2bfloat16_rn(x - __bfloat162float(hx)), ly = __float2bfloat16_rn(y - __bfloat162float(hy));
-    lo = (uint32_t)__bfloat16_as_ushort(lx) | ((uint32_t)__bfloat16_as_ushort(ly) << 16);
-    return (uint32_t)__bfloat16_as_ushort(hx) | ((uint32_t)__bfloat16_as_ushort(hy) << 16);
-}
-__device__ __forceinline__ uint32_t ad_map(const void* p, uint32_t cta) {
-    uint32_t r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_u32(p)), "r"(cta));
-    return r;
-}
 template <int N> __device__ __forceinline__ void ad_bar() { asm volatile("bar.sync 1, %0;" ::"n"(N) : "memory"); }
-
-// a part (maximum pm, sum pl, values p) into the running result
-__device__ __forceinline__ void ad_fold(float& m, float& l, float4& a, float pm, float pl, float4 p) {
-    const float mn = fmaxf(m, pm);
-    const float so = m == -CUDART_INF_F ? 0.0f : exp2f(m - mn), sp = pm == -CUDART_INF_F ? 0.0f : exp2f(pm - mn);
-    a.x = fmaf(p.x, sp, a.x * so); a.y = fmaf(p.y, sp, a.y * so); a.z = fmaf(p.z, sp, a.z * so); a.w = fmaf(p.w, sp, a.w * so);
-    l = fmaf(pl, sp, l * so);
-    m = mn;
-}
 
 template <int HD, int G>
 __global__ void __launch_bounds__((AdCfg<HD, G>::THREADS)) __maxnreg__((AdCfg<HD, G>::REGS)) attn_dec_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v, const AdArgs g) {
@@ -375,18 +359,6 @@ __global__ void __launch_bounds__((AdCfg<HD, G>::THREADS)) __maxnreg__((AdCfg<HD
             for (unsigned spin = 0; spin < WAIT_LIMIT && !mbar_try_wait(&full[i % CHUNKS], (uint32_t)((i / CHUNKS) & 1)); ++spin) {}
         atomicExch(g.err, AD_ERR_TIMEOUT);
     }
-}
-
-// CTAs per head, and clusters that share a kv head (see AdArgs)
-int ad_cluster(const anpd_model* m, int heads) {
-    const int resident = m->num_sms * 7 / 8;
-    int cluster = AD_MAX_CLUSTER;
-    while (cluster > 1 && heads * cluster > resident) cluster /= 2;
-    return cluster;
-}
-int ad_split(const anpd_model_config& c) {
-    const int group = c.n_q_heads / c.n_kv_heads;
-    return c.head_dim == 64 && group > 1 ? group / 2 : group;
 }
 
 template <int HD, int G>

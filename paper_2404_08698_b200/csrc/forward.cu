@@ -1305,6 +1305,7 @@ static anpd_status forward_cl_enqueue(anpd_model* m, anpd_kv* kv, int max_pos, b
     const size_t layer_elems = (size_t)kv->total_pages * c.n_kv_heads * KV_PAGE * hd;
     LAUNCH(pf, st, KC_OTHER, 0, (launch_k(embed_cl_kernel, rows, NORM_THREADS, 0, st, m->embed, ws.row_tok, m->layers[0].attn_norm, d, ws.x,
                                           ws.ci_h, rows, ws.ss_cl_a)));
+    if (ws.xch_bytes && !pf->on) return step_cl_enqueue(m, kv, want_logits, two_candidates);
     int parts_a = 1;                                   // sums of squares behind ci_h: one after the embedding, then the down projection's
     // No projection fetches the weights of the next one, or its own beyond its ring, into L2: the traffic stands in front of the activations and
     // of the other CTAs' last copies, and the code for it is as much as that of a product loop.  us per step with and without: 7B (16

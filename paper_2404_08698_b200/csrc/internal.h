@@ -408,6 +408,8 @@ struct Workspace {
     unsigned char *ci_h, *ci_h2, *ci_ao, *ci_act;
     float *ss_cl_a, *ss_cl_b;
     float* amax_val_cl; int* amax_idx_cl;
+    unsigned char* xch;               // what the CTAs of step_cl.cu exchange; xch_bytes of it, 0: such a step is not available
+    size_t xch_bytes;
     int amax_nblk;                    // argmax candidates per row left by the last forward (depends on the path it took)
     float* amax_val_use; int* amax_idx_use;   // ... and the arrays that hold them
     int* gemm_err;                    // device flag set by a GEMM kernel that gave up waiting
@@ -533,6 +535,12 @@ anpd_status accept_enqueue(anpd_model* m, anpd_kv* kv, int mode, const NgramDev*
 anpd_status attn_tc_enqueue(anpd_model* m, anpd_kv* kv, int layer, int rows, int max_pos, bool tree = false);
 // attn_dec.cu: attention of a decode step, written straight to the O projection's operand image
 anpd_status attn_dec_enqueue(anpd_model* m, anpd_kv* kv, int layer, bool tree);
+int ad_cluster(const anpd_model* m, int heads);         // CTAs that share the pages of an item
+int ad_split(const anpd_model_config& c);               // items that share a kv head
+// step_cl.cu: everything of a single sequence's step between the embedding and the argmax, in one kernel.  Bytes of the buffers its CTAs
+// exchange results through (Workspace::xch, all ones at first), 0 where the shape or the handle is not one for it.
+size_t step_cl_bytes(const anpd_model* m, int batch);
+anpd_status step_cl_enqueue(anpd_model* m, anpd_kv* kv, bool want_logits, bool tree);
 // attn_pf.cu: attention of a prompt pass with 128 query rows per CTA (head dimension 128, one query head per kv head)
 anpd_status attn_pf_enqueue(anpd_model* m, anpd_kv* kv, int layer, int rows, unsigned char* img, int n_seq);
 // attention of a prompt pass (one query head per kv head), written straight to the O projection's input
