@@ -7,7 +7,7 @@
 // five hand-overs per layer.  As a kernel per projection a hand-over took about 3 us: the last CTA's exit and the boundary behind it, tensor
 // memory and barriers set up again, code from a cold instruction cache, a weight ring that starts empty or half an SM wide.  Here the ring runs
 // through: the weight thread walks all layers' weights, and the cache's pages between them, and never waits for an activation.  us per step:
-// 1.1B at 512 keys 729 -> 618, 1024 wide (16 layers) 380 -> 292, 7B (16 layers and the head) at 77 keys 1294 -> 1151, at 1536 1382 -> 1232, tiny
+// 1.1B at 512 keys 729 -> 597, 1024 wide (16 layers) 380 -> 264, 7B (16 layers and the head) at 77 keys 1294 -> 1138, at 1536 1382 -> 1216, tiny
 // (2 x 256) 48 -> 43.
 //
 // Hand-over.  The exchange buffers hold nothing but all-ones words until their values are written, and no value is one (a NaN that
@@ -20,10 +20,17 @@
 // So are the others protected: a CTA's pushes of phase p + 2 into the region of the exchange that phase p used need results of
 // phase p + 1 that need all results of phase p.  This needs every cluster to own features and every CTA k-blocks of every projection.
 //
+// Wide projections.  A cluster's features come in tiles of up to 128 and the weights tile by tile, each through all of K: a tile's sums are
+// exchanged and finished (a quarter of its units by each CTA, the quarters taking turns) while the next one's weights still arrive, and only
+// the last one's exchange stands behind the phase.  The activations of up to 24 k-blocks stay in their slots meanwhile; beyond
+// that the tiles take turns every 24.  us per step against all tiles of a k-block together: 1.1B 627 -> 597, 1024 wide 291 -> 264,
+// 7B (16 layers) at 77 keys 1147 -> 1138, 13B (8 layers) 947 -> 931.
+//
 // The keys and values of the step itself reach the attention the same way; the pages are copied in before they can hold them (any time:
 // they are as old as the step before), and the rows are put into the copy.
 //
-// Values are those of gemm_cl.cu and attn_dec.cu bit for bit: the same cut of K, the same order of parts, pages, warps and CTAs.
+// Values are those of gemm_cl.cu and attn_dec.cu: the same cut of K, the same order of parts, pages, warps and CTAs.  They are equal bit for
+// bit up to 4096 features; beyond (two tiles of the residual stream) a row's sum of squares comes in other groups.
 // Every wait is bounded and reports through the error flag; a handle that has failed once refuses all further results.
 #include "step_dev.cuh"
 
@@ -41,6 +48,7 @@ constexpr int SC_MAX_STAGES = 12;
 constexpr int SC_SMEM = 220 * 1024;      // of dynamic shared memory; the static arrays take 7 KB
 constexpr int SC_AKB = 8, SC_ACT_SLOTS = 3;      // k-blocks of an activation slot, slots
 constexpr int SC_ACT_SLOT = SC_AKB * ANPD_ROWS * 256;
+constexpr int SC_CHUNK = SC_AKB * SC_ACT_SLOTS;  // k-blocks whose activations are there at once: tile by tile through all of them
 constexpr int SC_MAX_TILES = 8;          // tiles of 128 features a projection may hold
 constexpr unsigned SC_POLL_LIMIT = 1u << 21;
 constexpr int SC_ERR_TIMEOUT = 209;
@@ -58,8 +66,11 @@ template <int HD, int G> struct ScCfg {                      // G: query heads a
     static_assert(SLOTS + QROWS * QP <= SC_ACT_SLOTS * SC_ACT_SLOT, "attention's buffers take the activations' place");
 };
 
-struct ScKind { int kb, gpu, n_units, seg, copies, kps, K, f_own_max, shift, red; };
-struct ScGeo { int Uc, Gc, T, base, rem, nk, kb_lo, n_st, on, ufirst, skip; unsigned long long w_off; };
+struct ScKind { int kb, gpu, n_units, seg, tiles, kps, K, f_own_max, shift, red; };
+// a projection as this cluster and CTA see it: tiles, k-blocks, where the weights start and the bytes from a k-block to the next
+struct ScGeo { int T, nk, kb_lo, n_st, step; unsigned long long w_off; };
+// a tile: its groups, the first one (of the cluster's), the units that each rank has finished before it, this CTA's units of it
+struct ScTile { short groups, g0, before[CL_CTAS], own_n; int own_first; };
 
 struct ScArgs {
     ScKind k[GK_COUNT];
@@ -104,7 +115,22 @@ __device__ __forceinline__ void work_bar() { asm volatile("bar.sync 1, 256;" :::
 __device__ __forceinline__ void st_async2(uint32_t addr, uint32_t bar, float a, float b) {
     asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];" ::"r"(addr), "f"(a), "f"(b), "r"(bar) : "memory");
 }
+// four columns at `hi` and four at `lo` of this thread's tensor-memory lane, added
+__device__ __forceinline__ void tc_ld4_sum(uint32_t hi, uint32_t lo, float* v) {
+    uint32_t a[4], b[4];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%8];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%4, %5, %6, %7}, [%9];\n\t"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3]), "=r"(b[0]), "=r"(b[1]), "=r"(b[2]), "=r"(b[3])
+        : "r"(hi), "r"(lo) : "memory");
+#pragma unroll
+    for (int i = 0; i < 4; ++i) v[i] = __uint_as_float(a[i]) + __uint_as_float(b[i]);
+}
 __device__ __forceinline__ void fence_async_cta() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+
+// Units of tile t of a cluster's Uc.  Each rank finishes a quarter of every tile's units, the quarters taking turns.
+__host__ __device__ inline int sc_tile_units(int Uc, int tiles, int t) { return Uc / tiles + (t < Uc % tiles ? 1 : 0); }
 
 template <int HD, int G>
 __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v, const __grid_constant__ ScArgs g) {
@@ -115,12 +141,14 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
     constexpr int CC = CL_CTAS, rows = ANPD_ROWS;
     extern __shared__ __align__(1024) unsigned char sc_smem[];
     __shared__ uint64_t w_full[SC_MAX_STAGES], w_empty[SC_MAX_STAGES], p_empty[SC_MAX_STAGES], a_full[SC_ACT_SLOTS], a_empty[SC_ACT_SLOTS];
-    __shared__ uint64_t acc_full, red_full[2], att_full, jan_done;
+    __shared__ uint64_t acc_full[SC_MAX_TILES], red_full[2][SC_MAX_TILES], att_full, jan_done;
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag, s_issued;
     __shared__ float s_rstd[8], s_part[8][8];
     __shared__ int s_pos[8], s_slot[8], s_page[8], s_raw[8], s_idx[8][8];
     __shared__ ScGeo s_geo[GK_COUNT];
+    __shared__ ScTile s_tile[GK_COUNT][SC_MAX_TILES];
+    __shared__ int s_own[GK_COUNT];                     // units this CTA finishes
     __shared__ float2 rc[NV];                           // [CTA][VO] maximum and sum of the cluster's parts of this CTA's vectors
     __shared__ float sm_m[WARPS * NV], sm_l[WARPS * NV];
     __shared__ __align__(16) float recv[NV * HD];       // [CTA][VO][HD]
@@ -137,24 +165,35 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
     if (threadIdx.x < GK_COUNT) {                       // how this cluster and CTA cut each projection
         const ScKind& k = g.k[threadIdx.x];
         ScGeo e;
-        const int ulo = cluster * k.n_units / g.ncl, uhi = (cluster + 1) * k.n_units / g.ncl;
-        e.Uc = uhi - ulo; e.Gc = e.Uc * k.gpu;
-        e.T = min(k.copies, e.Gc);
-        e.base = e.Gc / e.T; e.rem = e.Gc - e.base * e.T;
+        const int ulo = cluster * k.n_units / g.ncl, uhi = (cluster + 1) * k.n_units / g.ncl, Uc = uhi - ulo, Gc = Uc * k.gpu;
+        e.T = k.tiles;
         e.kb_lo = rank * k.kb / CC; e.nk = (rank + 1) * k.kb / CC - e.kb_lo;
         e.n_st = e.T == 1 ? (e.nk + k.kps - 1) / k.kps : e.nk * e.T;
-        const int o0 = rank * e.Uc / CC;
-        e.on = (rank + 1) * e.Uc / CC - o0; e.ufirst = ulo + o0;
-        const int GS = k.seg == 1 ? k.n_units * k.gpu : e.Gc;             // groups of a k-block in its segment
-        e.skip = (GS - e.Gc) << 10;
+        const int GS = k.seg == 1 ? k.n_units * k.gpu : Gc;               // groups of a k-block in its segment
+        e.step = GS << 10;
         e.w_off = ((unsigned long long)ulo * k.gpu * (k.seg == 1 ? 1 : k.kb) + (unsigned long long)GS * e.kb_lo) * 1024;
+        int before[CC] = {0, 0, 0, 0};
+        for (int t = 0, u0 = 0; t < k.tiles; ++t) {
+            ScTile& w = s_tile[threadIdx.x][t];
+            const int un = sc_tile_units(Uc, k.tiles, t);
+            w.groups = (short)(un * k.gpu); w.g0 = (short)(u0 * k.gpu);
+            for (int r = 0; r < CC; ++r) {
+                const int q = (r + t) & (CC - 1), lo = q * un / CC, n = (q + 1) * un / CC - lo;
+                w.before[r] = (short)before[r];
+                if (r == rank) { w.own_first = ulo + u0 + lo; w.own_n = (short)n; }
+                before[r] += n;
+            }
+            u0 += un;
+        }
+        s_own[threadIdx.x] = before[rank];
         s_geo[threadIdx.x] = e;
     }
     if (threadIdx.x == 64) {
         abort_flag = 0; s_issued = 0;
         for (int s = 0; s < g.stages; ++s) { mbar_init(&w_full[s], 1); mbar_init(&w_empty[s], 1); mbar_init(&p_empty[s], WARPS); }
         for (int s = 0; s < SC_ACT_SLOTS; ++s) { mbar_init(&a_full[s], 8); mbar_init(&a_empty[s], 1); }
-        mbar_init(&acc_full, 1); mbar_init(&red_full[0], 1); mbar_init(&red_full[1], 1); mbar_init(&att_full, 1); mbar_init(&jan_done, 1);
+        for (int t = 0; t < SC_MAX_TILES; ++t) { mbar_init(&acc_full[t], 1); mbar_init(&red_full[0][t], 1); mbar_init(&red_full[1][t], 1); }
+        mbar_init(&att_full, 1); mbar_init(&jan_done, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         fence_async_cta();
     }
@@ -195,21 +234,25 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
             };
             auto next = [&]() { ++count; if (++stage == g.stages) stage = 0; };
             auto weights = [&](int kd, const unsigned char* w) {
-                const int nk = s_geo[kd].nk, T = s_geo[kd].T, Gc = s_geo[kd].Gc, base = s_geo[kd].base, rem = s_geo[kd].rem, skip = s_geo[kd].skip, kps = T == 1 ? g.k[kd].kps : 1;
-                const unsigned char* src = w + s_geo[kd].w_off;
+                const int nk = s_geo[kd].nk, T = s_geo[kd].T, step = s_geo[kd].step, kps = g.k[kd].kps;
+                const unsigned char* src0 = w + s_geo[kd].w_off;
 #pragma unroll 1
-                for (int k = 0; k < nk && ok; k += kps) {
-                    const int n = min(kps, nk - k);
+                for (int k0 = 0; k0 < nk && ok; k0 += SC_CHUNK, src0 += (size_t)SC_CHUNK * step) {
+                    const int kn = min(SC_CHUNK, nk - k0);
 #pragma unroll 1
-                    for (int t = 0; t < T; ++t) {
-                        const uint32_t bytes = (uint32_t)(T == 1 ? n * Gc : base + (t < rem ? 1 : 0)) << 10;
-                        if (!take(false)) break;
-                        mbar_expect_tx(&w_full[stage], bytes);
-                        bulk_load(ring + stage * SC_STAGE, src, bytes, &w_full[stage], pol_w);
-                        src += bytes;
-                        next();
+                    for (int t = 0; t < T && ok; ++t) {
+                        const unsigned char* src = src0 + ((int)s_tile[kd][t].g0 << 10);
+                        const uint32_t kb_bytes = (uint32_t)s_tile[kd][t].groups << 10;
+#pragma unroll 1
+                        for (int k = 0; k < kn; k += kps) {
+                            const uint32_t bytes = (uint32_t)min(kps, kn - k) * kb_bytes;       // kps > 1 only where one tile holds all of the segment's groups
+                            if (!take(false)) break;
+                            mbar_expect_tx(&w_full[stage], bytes);
+                            bulk_load(ring + stage * SC_STAGE, src, bytes, &w_full[stage], pol_w);
+                            src += kps > 1 ? bytes : (uint32_t)step;
+                            next();
+                        }
                     }
-                    src += skip;
                 }
             };
 #pragma unroll 1
@@ -259,54 +302,49 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
             int kd = GK_QKV, l = 0;
 #pragma unroll 1
             while (true) {
-                const int nk = s_geo[kd].nk, T = s_geo[kd].T, Gc = s_geo[kd].Gc, kps = g.k[kd].kps;
+                const int nk = s_geo[kd].nk, T = s_geo[kd].T, kps = g.k[kd].kps;
                 uint32_t acc = 0;
 #pragma unroll 1
-                for (int k0 = 0; k0 < nk; k0 += SC_AKB) {
-                    mbar_wait_at<1>(afull, aph, abortp);
-                    tc_fence_after();
-                    const int kend = min(SC_AKB, nk - k0);
-                    uint32_t a = a_lo;
-                    // a tile of fewer than 16 groups: the instruction reads whatever follows for the rows beyond, whose lanes nobody reads
-                    if (T > 1) {                                        // one tile of one k-block per stage
+                for (int k0 = 0; k0 < nk; k0 += SC_CHUNK) {
+                    const int kn = min(SC_CHUNK, nk - k0);
+                    uint32_t d_tmem = tmem_base;
 #pragma unroll 1
-                        for (int k = 0; k < kend; ++k) {
-                            uint32_t d_tmem = tmem_base;
+                    for (int t = 0; t < T; ++t) {
+                        const uint32_t kb_words = (uint32_t)s_tile[kd][t].groups << 6;
+                        uint32_t af = afull, ap = aph, alo = a_lo, accumulate = acc;
 #pragma unroll 1
-                            for (int t = T; t > 0; --t) {
+                        for (int ks = 0; ks < kn; ks += SC_AKB) {
+                            if (t == 0) { mbar_wait_at<1>(af, ap, abortp); tc_fence_after(); }
+                            const int kend = min(SC_AKB, kn - ks);
+                            uint32_t a = alo;
+                            // a tile of fewer than 16 groups: the instruction reads whatever follows for the rows beyond, whose lanes nobody reads
+#pragma unroll 1
+                            for (int k = 0; k < kend; k += kps) {
                                 mbar_wait_at<1>(full, wph, abortp);
                                 tc_fence_after();
-                                tc_mma_k64(d_tmem, w_lo, a, idesc, acc);
-                                next_stage();
-                                d_tmem += (uint32_t)(2 * rows);
-                            }
-                            acc = 1;
-                            a += kb_step;
-                        }
-                    } else {                                            // kps k-blocks of the only tile per stage
-#pragma unroll 1
-                        for (int k = 0; k < kend; k += kps) {
-                            mbar_wait_at<1>(full, wph, abortp);
-                            tc_fence_after();
-                            tc_mma_k64(tmem_base, w_lo, a, idesc, acc);
-                            acc = 1;
-                            a += kb_step;
-                            uint32_t w = w_lo;
-#pragma unroll 1
-                            for (int j = min(kps, kend - k); j > 1; --j) {
-                                w += (uint32_t)(Gc << 6);
-                                tc_mma_k64(tmem_base, w, a, idesc, 1u);
+                                tc_mma_k64(d_tmem, w_lo, a, idesc, accumulate);
+                                accumulate = 1;
                                 a += kb_step;
+                                uint32_t w = w_lo;
+#pragma unroll 1
+                                for (int j = min(kps, kend - k); j > 1; --j) {
+                                    w += kb_words;
+                                    tc_mma_k64(d_tmem, w, a, idesc, 1u);
+                                    a += kb_step;
+                                }
+                                next_stage();
                             }
-                            next_stage();
+                            if (t == T - 1) tc_commit_at(af + aempty_off);
+                            alo += act_step;
+                            af += 8u;
+                            if (af == af_end) { af = af0; ap ^= 1u; alo = act_lo; }
                         }
+                        if (k0 + kn == nk) tc_commit(&acc_full[t]);
+                        d_tmem += (uint32_t)(2 * rows);
+                        if (t == T - 1) { afull = af; aph = ap; a_lo = alo; }
                     }
-                    tc_commit_at(afull + aempty_off);
-                    a_lo += act_step;
-                    afull += 8u;
-                    if (afull == af_end) { afull = af0; aph ^= 1u; a_lo = act_lo; }
+                    acc = 1;
                 }
-                tc_commit(&acc_full);
                 if (kd == GK_LM) break;
                 if (kd == GK_QKV) {                                     // the pages' stages are the workers'
                     int st = (int)((full - full0) >> 3) + pg_st;
@@ -340,12 +378,7 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
         const int half = HD >> 1, upi = HD >> 4;
         const uint32_t red_addr = smem_u32(redbuf);
         const int VO = NV / g.C;                                                     // vectors a CTA finishes
-        auto red_bytes = [&](int kd) { const int on = s_geo[kd].on; return (uint32_t)(on ? (on << g.k[kd].shift) * CC * 32 : CC * 16); };
-        if (ft == 0) {
-            mbar_expect_tx(&red_full[0], red_bytes(GK_QKV));
-            mbar_expect_tx(&red_full[1], red_bytes(GK_O));
-            mbar_expect_tx(&att_full, (uint32_t)(g.C * VO * (HD * 4 + 8)));
-        }
+        if (ft == 0) mbar_expect_tx(&att_full, (uint32_t)(g.C * VO * (HD * 4 + 8)));
         if (ft < 8) {
             const int slot = g.row_slot[ft];
             s_pos[ft] = g.row_pos[ft];
@@ -354,12 +387,28 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
             s_page[ft] = g.page_table[(size_t)g.row_seq[ft] * g.pages_per_seq + slot / KV_PAGE];
         }
         pdl_wait();                                     // what the embedding left
-        for (int idx = ft; idx < s_geo[GK_O].on * 32; idx += SC_WORKERS) s_x[idx] = *(const float2*)(g.x0 + (size_t)row * g.d + s_geo[GK_O].ufirst * 8 + 2 * (idx >> 3));
+        // A CTA's results in the order of its units over all tiles, 32 pairs each: item idx is thread idx % 256's.  The unit of an item
+        // of tile t, and the features of the residual stream:
+        auto unit_of = [&](int kd, int t, int idx) { return s_tile[kd][t].own_first + (idx >> 5) - s_tile[kd][t].before[rank]; };
+        auto tile_of = [&](int kd, int idx) {
+            int t = 0;
+            while (t + 1 < s_geo[kd].T && (idx >> 5) >= s_tile[kd][t + 1].before[rank]) ++t;
+            return t;
+        };
+        auto resid_feature = [&](int idx) { return unit_of(GK_O, tile_of(GK_O, idx), idx) * 8 + 2 * ((idx >> 3) & 3); };
+        for (int idx = ft; idx < s_own[GK_O] * 32; idx += SC_WORKERS) s_x[idx] = *(const float2*)(g.x0 + (size_t)row * g.d + resid_feature(idx));
+        float2 cs0 = make_float2(0.f, 0.f), sn0 = cs0;         // the rotation of this thread's first item of QKV, the same in every layer
+        if (ft < s_own[GK_QKV] * 32) {
+            const int u = unit_of(GK_QKV, tile_of(GK_QKV, ft), ft);
+            const size_t at = (size_t)g.row_pos[row] * half + (u % upi) * 8 + 2 * ((ft >> 3) & 3);
+            cs0 = *(const float2*)(g.rope_cos + at);
+            sn0 = *(const float2*)(g.rope_sin + at);
+        }
         work_bar();
         cluster_wait();
 
         int a_slot = 0, a_count = 0, p_st = 0;
-        uint32_t a_ph = 1, p_par = 0, acc_par = 0, red_par = 0, att_par = 0;       // red_par: a bit per region
+        uint32_t a_ph = 1, p_par = 0, acc_par = 0, red_par = 0, att_par = 0;       // acc_par: a bit per tile; red_par: per region and tile
         const int st_rest = s_geo[GK_O].n_st + s_geo[GK_GU].n_st + s_geo[GK_DOWN].n_st + s_geo[GK_QKV].n_st;
         auto adv = [&](int n) {                          // stages consumed by others
             p_st += n;
@@ -651,14 +700,18 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
                 if (att) attention(l, copy);
                 adv(st_rest);
             }
-            const int Uc = s_geo[kd].Uc, on = s_geo[kd].on, ufirst = s_geo[kd].ufirst, shift = g.k[kd].shift, f_own_max = g.k[kd].f_own_max;
+            const int T = s_geo[kd].T, shift = g.k[kd].shift, f_own_max = g.k[kd].f_own_max;
             const bool resid = kd == GK_O || kd == GK_DOWN;
             const int region = resid ? 1 : 0;
             float2 gn = make_float2(0.f, 0.f);
             const float* gain = nullptr;
             if (resid) {
                 gain = kd == GK_O ? (const float*)((const char*)g.ffn_norm + (size_t)l * g.layer_step) : l + 1 < g.L ? (const float*)((const char*)g.attn_norm + (size_t)(l + 1) * g.layer_step) : g.final_norm;
-                if (ft < on * 32) gn = *(const float2*)(gain + ufirst * 8 + 2 * (ft >> 3));
+                if (ft < s_own[kd] * 32) gn = *(const float2*)(gain + resid_feature(ft));
+            }
+            if (ft < T) {                                // what the cluster will send here for each tile
+                const int n = s_tile[kd][ft].own_n;
+                mbar_expect_tx(&red_full[region][ft], (uint32_t)(n ? (n << shift) * CC * 32 : CC * 16));
             }
             load_acts(kd == GK_QKV ? (l ? prev : g.img0) : kd == GK_LM ? fin : copy + (kd == GK_O ? g.o_ao : kd == GK_GU ? g.o_h2 : g.o_act), kd);
             // 1 / RMS of every row: a warp per row, 32 interleaved sums over the parts, then a tree over the lanes
@@ -685,82 +738,130 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
                 for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
                 if (lane == 0) s_rstd[fw] = rsqrtf(s * g.inv_d + g.eps);
             }
-            if (pushes) {
-                // where this thread's feature of each tile goes: byte offset in the exchange buffer and the owner's rank
-                const int T = s_geo[kd].T, base = s_geo[kd].base, rem = s_geo[kd].rem;
-                uint32_t dst[SC_MAX_TILES];
-                int t0 = 0;
-#pragma unroll
-                for (int t = 0; t < SC_MAX_TILES; ++t) {
-                    dst[t] = SC_EMPTY;
-                    if (t < T) {
-                        const int gt = base + (t < rem ? 1 : 0);
-                        if (quad * 32 + lane < gt * 8) {
-                            const int f = t0 * 8 + quad * 32 + lane, u = f >> shift, owner = ((u + 1) * CC - 1) / Uc;
-                            const int local = f - ((owner * Uc / CC) << shift);
-                            dst[t] = ((uint32_t)owner << 24) | (uint32_t)(g.k[kd].red + (rank * f_own_max + local) * 32);
-                        }
-                        t0 += gt;
-                    }
-                }
-                // the buffers of the layer before are empty again before anything that the next layer waits for leaves this CTA
-                if (kd == GK_DOWN) mbar_wait<1>(&jan_done, (uint32_t)l & 1u, abortp);
-                mbar_wait<1>(&acc_full, acc_par, abortp);
-                tc_fence_after();
-                const uint32_t bar0 = smem_u32(&red_full[region]);
-                const uint32_t col0 = tmem_base + ((uint32_t)(quad * 32) << 16);
-#pragma unroll
-                for (int t = 0; t < SC_MAX_TILES; t += 2) {
-                    if (t >= T) break;
-                    // two tiles' columns in one load; the second repeats the first where there is none
-                    float v[2][8];
-                    const uint32_t ca = col0 + (uint32_t)(t * 16), cb = t + 1 < T ? ca + 16u : ca;
-                    tc_ld8_sum2(ca, ca + 8u, cb, cb + 8u, v[0], v[1]);
-#pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        if (dst[t + h] != SC_EMPTY) {
-                            const uint32_t owner = dst[t + h] >> 24, to = map_to_cta(red_addr + (dst[t + h] & 0xffffffu), owner), bar = map_to_cta(bar0, owner);
-                            st_async4(to, bar, v[h][0], v[h][1], v[h][2], v[h][3]);
-                            st_async4(to + 16u, bar, v[h][4], v[h][5], v[h][6], v[h][7]);
-                        }
-                    }
-                }
-                // a CTA that finishes nothing hears from the others all the same: it is then behind them
-                if (ft < CC && (ft + 1) * Uc / CC == ft * Uc / CC) st_async4(map_to_cta(red_addr + (uint32_t)g.k[kd].red + (uint32_t)rank * 16u, (uint32_t)ft), map_to_cta(bar0, (uint32_t)ft), 0.f, 0.f, 0.f, 0.f);
-                tc_fence_before();
-            }
-            acc_par ^= 1u;
             if (!resid) work_bar();                      // the rows' 1 / RMS
-            mbar_wait_cluster(&red_full[region], (red_par >> region) & 1u, abortp);
-            red_par ^= 1u << region;
-            if (ft == 0) {                               // what the next exchange through this region will send here
-                if (kd == GK_QKV) mbar_expect_tx(&red_full[0], red_bytes(GK_GU));
-                else if (kd == GK_O) mbar_expect_tx(&red_full[1], red_bytes(GK_DOWN));
-                else if (kd == GK_GU) mbar_expect_tx(&red_full[0], red_bytes(l + 1 < g.L ? GK_QKV : GK_LM));
-                else if (kd == GK_DOWN && l + 1 < g.L) mbar_expect_tx(&red_full[1], red_bytes(GK_O));
-            }
+            // the buffers of the layer before are empty again before anything that the next layer waits for leaves this CTA
+            if (kd == GK_DOWN) mbar_wait<1>(&jan_done, (uint32_t)l & 1u, abortp);
             const float* red = (const float*)(redbuf + g.k[kd].red);
             const int part_step = f_own_max * 8;
             auto sum = [&](int f) {                      // feature f of this CTA's share, this thread's row, parts in CTA order
                 const float* s = red + f * 8 + row;
                 return ((s[0] + s[part_step]) + s[2 * part_step]) + s[3 * part_step];
             };
-            if (resid) {
-                unsigned char* act = kd == GK_O ? copy + g.o_h2 : l + 1 < g.L ? copy : fin;
-                float ssq = 0.0f;
+            // Tile by tile: this CTA's sums go to whoever finishes the features, as soon as the products are through; then it finishes its own of
+            // the tile before, whose parts have come in meanwhile.
+            float ssq = 0.0f, best = -CUDART_INF_F;
+            int bidx = 0x7fffffff;
+            unsigned char* act = kd == GK_O ? copy + g.o_h2 : kd == GK_GU ? copy + g.o_act : l + 1 < g.L ? copy : fin;
+            const float rs = resid ? 1.0f : s_rstd[row];
+            auto finish = [&](int t) {
+                const int lo = s_tile[kd][t].before[rank] * (kd == GK_LM ? 64 : 32), hi_ = lo + s_tile[kd][t].own_n * (kd == GK_LM ? 64 : 32);
+                mbar_wait_cluster(&red_full[region][t], (red_par >> (region * SC_MAX_TILES + t)) & 1u, abortp);
 #pragma unroll 1
-                for (int idx = ft; idx < on * 32; idx += SC_WORKERS) {
-                    const int f = 2 * (idx >> 3), n = ufirst * 8 + f;
-                    if (idx != ft) gn = *(const float2*)(gain + n);
-                    float2 x = s_x[idx];
-                    x.x += sum(f); x.y += sum(f + 1);
-                    s_x[idx] = x;
-                    ssq += x.x * x.x + x.y * x.y;
-                    uint32_t hi, lo;
-                    split2(x.x * gn.x, x.y * gn.y, hi, lo);
-                    st_relaxed1(act + cl_img_offset(rows, row, n), hi);
-                    st_relaxed1(act + cl_img_offset(rows, rows + row, n), lo);
+                for (int idx = lo + ((ft - lo) & (SC_WORKERS - 1)); idx < hi_; idx += SC_WORKERS) {
+                    if (resid) {
+                        const int f = 2 * (idx >> 3), n = unit_of(kd, t, idx) * 8 + (f & 7);
+                        if (idx != ft) gn = *(const float2*)(gain + n);
+                        float2 x = s_x[idx];
+                        x.x += sum(f); x.y += sum(f + 1);
+                        s_x[idx] = x;
+                        ssq += x.x * x.x + x.y * x.y;
+                        uint32_t hi, lo2;
+                        split2(x.x * gn.x, x.y * gn.y, hi, lo2);
+                        st_relaxed1(act + cl_img_offset(rows, row, n), hi);
+                        st_relaxed1(act + cl_img_offset(rows, rows + row, n), lo2);
+                    } else if (kd == GK_GU) {
+                        const int e = 2 * ((idx >> 3) & 3), f = (idx >> 5) * 16 + e, k = unit_of(kd, t, idx) * 8 + e;
+                        float v[2];
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            const float gte = sum(f + h) * rs, upv = sum(f + 8 + h) * rs;
+                            v[h] = gte / (1.0f + expf(-gte)) * upv;
+                        }
+                        uint32_t hi, lo2;
+                        split2(v[0], v[1], hi, lo2);
+                        st_relaxed1(act + cl_img_offset(rows, row, k), hi);
+                        st_relaxed1(act + cl_img_offset(rows, rows + row, k), lo2);
+                    } else if (kd == GK_QKV) {
+                        const int ul = idx >> 5, e = 2 * ((idx >> 3) & 3), u = unit_of(kd, t, idx), head = u / upi, i = (u - head * upi) * 8 + e;
+                        float a[2], b[2];
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) { a[h] = sum(ul * 16 + e + h) * rs; b[h] = sum(ul * 16 + 8 + e + h) * rs; }
+                        if (head < g.Hq + g.Hkv) {
+                            float2 cs = cs0, sn = sn0;
+                            if (idx != ft) {
+                                const size_t at = (size_t)s_pos[row] * half + i;
+                                cs = *(const float2*)(g.rope_cos + at);
+                                sn = *(const float2*)(g.rope_sin + at);
+                            }
+                            const float a0 = a[0] * cs.x - b[0] * sn.x, b0 = b[0] * cs.x + a[0] * sn.x;
+                            const float a1 = a[1] * cs.y - b[1] * sn.y, b1 = b[1] * cs.y + a[1] * sn.y;
+                            a[0] = a0; b[0] = b0; a[1] = a1; b[1] = b1;
+                        }
+                        if (head < g.Hq) {
+                            // queries leave as two bf16 terms, already multiplied by log2(e) / sqrt(hd): [head][term][row][dim]
+                            unsigned char* q = copy + g.o_q + ((size_t)(head * 2) * rows + row) * (HD * 2) + i * 2;
+                            uint32_t hi, lo2;
+                            split2(a[0] * g.q_scale, a[1] * g.q_scale, hi, lo2);
+                            st_relaxed1(q, hi); st_relaxed1(q + rows * HD * 2, lo2);
+                            split2(b[0] * g.q_scale, b[1] * g.q_scale, hi, lo2);
+                            st_relaxed1(q + half * 2, hi); st_relaxed1(q + rows * HD * 2 + half * 2, lo2);
+                        } else {
+                            const bool is_k = head < g.Hq + g.Hkv;
+                            const int kh = is_k ? head - g.Hq : head - g.Hq - g.Hkv, slot = s_slot[row];
+                            const __nv_bfloat162 va = __floats2bfloat162_rn(a[0], a[1]), vb = __floats2bfloat162_rn(b[0], b[1]);
+                            // for this step's attention [kv head][K, V][row][dim], and into the cache for later ones
+                            unsigned char* n = copy + g.o_kv + ((size_t)(kh * 2 + (is_k ? 0 : 1)) * rows + row) * (HD * 2) + i * 2;
+                            st_relaxed1(n, *(const uint32_t*)&va); st_relaxed1(n + half * 2, *(const uint32_t*)&vb);
+                            if (slot >= 0) {
+                                bf16* pg = (is_k ? g.kpool : g.vpool) + (((size_t)l * g.total_pages + s_page[row]) * g.Hkv + kh) * KV_PAGE * HD;
+                                if (is_k) {                                   // K page: [position][dim]
+                                    bf16* at = pg + (size_t)(slot % KV_PAGE) * HD + i;
+                                    *(__nv_bfloat162*)at = va;
+                                    *(__nv_bfloat162*)(at + half) = vb;
+                                } else {                                      // V page, transposed: [dim][position]
+                                    bf16* at = pg + (size_t)i * KV_PAGE + (slot % KV_PAGE);
+                                    at[0] = va.x;
+                                    at[KV_PAGE] = va.y;
+                                    at[(size_t)half * KV_PAGE] = vb.x;
+                                    at[(size_t)(half + 1) * KV_PAGE] = vb.y;
+                                }
+                            }
+                        }
+                    } else {                                                   // vocabulary: a unit is 64 items
+                        const int f = idx >> 3, n = (s_tile[kd][t].own_first + (idx >> 6) - s_tile[kd][t].before[rank]) * 8 + (f & 7);
+                        if (n >= g.n_out) continue;
+                        const float v = sum(f) * rs;
+                        if (g.out) g.out[(size_t)row * g.n_out + n] = v;
+                        if (v > best) { best = v; bidx = n; }                   // ascending n: strict > keeps the lowest id
+                    }
                 }
+            };
+#pragma unroll 1
+            for (int t = 0; t <= T; ++t) {
+                if (t < T) {
+                    // thread: a feature (tensor-memory lane) and four of the rows
+                    const int un = s_tile[kd][t].groups >> (shift - 3), pos = quad * 32 + lane, u = pos >> shift;
+                    const int b1 = un / 4, b2 = un / 2, b3 = 3 * un / 4, q = (u >= b1) + (u >= b2) + (u >= b3), owner = (q - t) & (CC - 1);
+                    const int local = ((s_tile[kd][t].before[owner] + u - (q * un) / CC) << shift) + (pos & ((1 << shift) - 1));
+                    mbar_wait<1>(&acc_full[t], (acc_par >> t) & 1u, abortp);
+                    tc_fence_after();
+                    float v[4];
+                    const uint32_t col = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(t * 2 * rows + (pushes ? 0 : 4));
+                    tc_ld4_sum(col, col + 8u, v);
+                    const uint32_t bar0 = smem_u32(&red_full[region][t]), to = red_addr + (uint32_t)(g.k[kd].red + (rank * f_own_max + local) * 32 + (pushes ? 0 : 16));
+                    if (pos < (int)s_tile[kd][t].groups * 8) st_async4(map_to_cta(to, (uint32_t)owner), map_to_cta(bar0, (uint32_t)owner), v[0], v[1], v[2], v[3]);
+                    // a CTA that finishes nothing of the tile hears from the others all the same: it is then behind them
+                    if (ft < CC && (ft + 1) * un / CC == ft * un / CC) {
+                        const uint32_t o = (uint32_t)((ft - t) & (CC - 1));
+                        st_async4(map_to_cta(red_addr + (uint32_t)(g.k[kd].red + rank * 16), o), map_to_cta(bar0, o), 0.f, 0.f, 0.f, 0.f);
+                    }
+                    tc_fence_before();
+                }
+                if (t > 0) finish(t - 1);
+            }
+            acc_par ^= (1u << T) - 1u;
+            red_par ^= ((1u << T) - 1u) << (region * SC_MAX_TILES);
+            if (resid) {
                 // the row's sum of squares over this CTA's features: one part
                 ssq += __shfl_xor_sync(0xffffffffu, ssq, 8);
                 ssq += __shfl_xor_sync(0xffffffffu, ssq, 16);
@@ -774,83 +875,7 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
                     st_relaxed1(ss + ((size_t)ft * ncta + bid) * 4, __float_as_uint(s));
                 }
                 if (kd == GK_O) asm volatile("bar.arrive 3, 288;" ::: "memory");
-            } else if (kd == GK_GU) {
-                unsigned char* act = copy + g.o_act;
-                const float rs = s_rstd[row];
-#pragma unroll 1
-                for (int idx = ft; idx < on * 32; idx += SC_WORKERS) {
-                    const int ul = idx >> 5, e = 2 * ((idx >> 3) & 3), f = ul * 16 + e, k = (ufirst + ul) * 8 + e;
-                    float v[2];
-#pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        const float gte = sum(f + h) * rs, upv = sum(f + 8 + h) * rs;
-                        v[h] = gte / (1.0f + expf(-gte)) * upv;
-                    }
-                    uint32_t hi, lo;
-                    split2(v[0], v[1], hi, lo);
-                    st_relaxed1(act + cl_img_offset(rows, row, k), hi);
-                    st_relaxed1(act + cl_img_offset(rows, rows + row, k), lo);
-                }
-            } else if (kd == GK_QKV) {
-                const float rs = s_rstd[row];
-                const int pos = s_pos[row], slot = s_slot[row], page = s_page[row];
-                const size_t layer_at = (size_t)l * g.total_pages * g.Hkv * KV_PAGE * HD;
-#pragma unroll 1
-                for (int idx = ft; idx < on * 32; idx += SC_WORKERS) {
-                    const int ul = idx >> 5, e = 2 * ((idx >> 3) & 3), u = ufirst + ul, head = u / upi, i = (u - head * upi) * 8 + e;
-                    float a[2], b[2];
-#pragma unroll
-                    for (int h = 0; h < 2; ++h) { a[h] = sum(ul * 16 + e + h) * rs; b[h] = sum(ul * 16 + 8 + e + h) * rs; }
-                    if (head < g.Hq + g.Hkv) {
-                        const size_t at = (size_t)pos * half + i;
-                        const float2 cs = *(const float2*)(g.rope_cos + at), sn = *(const float2*)(g.rope_sin + at);
-                        const float a0 = a[0] * cs.x - b[0] * sn.x, b0 = b[0] * cs.x + a[0] * sn.x;
-                        const float a1 = a[1] * cs.y - b[1] * sn.y, b1 = b[1] * cs.y + a[1] * sn.y;
-                        a[0] = a0; b[0] = b0; a[1] = a1; b[1] = b1;
-                    }
-                    if (head < g.Hq) {
-                        // queries leave as two bf16 terms, already multiplied by log2(e) / sqrt(hd): [head][term][row][dim]
-                        unsigned char* q = copy + g.o_q + ((size_t)(head * 2) * rows + row) * (HD * 2) + i * 2;
-                        uint32_t hi, lo;
-                        split2(a[0] * g.q_scale, a[1] * g.q_scale, hi, lo);
-                        st_relaxed1(q, hi); st_relaxed1(q + rows * HD * 2, lo);
-                        split2(b[0] * g.q_scale, b[1] * g.q_scale, hi, lo);
-                        st_relaxed1(q + half * 2, hi); st_relaxed1(q + rows * HD * 2 + half * 2, lo);
-                    } else {
-                        const bool is_k = head < g.Hq + g.Hkv;
-                        const int kh = is_k ? head - g.Hq : head - g.Hq - g.Hkv;
-                        const __nv_bfloat162 va = __floats2bfloat162_rn(a[0], a[1]), vb = __floats2bfloat162_rn(b[0], b[1]);
-                        // for this step's attention [kv head][K, V][row][dim], and into the cache for later ones
-                        unsigned char* n = copy + g.o_kv + ((size_t)(kh * 2 + (is_k ? 0 : 1)) * rows + row) * (HD * 2) + i * 2;
-                        st_relaxed1(n, *(const uint32_t*)&va); st_relaxed1(n + half * 2, *(const uint32_t*)&vb);
-                        if (slot >= 0) {
-                            bf16* pg = (is_k ? g.kpool : g.vpool) + layer_at + ((size_t)page * g.Hkv + kh) * KV_PAGE * HD;
-                            if (is_k) {                                   // K page: [position][dim]
-                                bf16* at = pg + (size_t)(slot % KV_PAGE) * HD + i;
-                                *(__nv_bfloat162*)at = va;
-                                *(__nv_bfloat162*)(at + half) = vb;
-                            } else {                                      // V page, transposed: [dim][position]
-                                bf16* at = pg + (size_t)i * KV_PAGE + (slot % KV_PAGE);
-                                at[0] = va.x;
-                                at[KV_PAGE] = va.y;
-                                at[(size_t)half * KV_PAGE] = vb.x;
-                                at[(size_t)(half + 1) * KV_PAGE] = vb.y;
-                            }
-                        }
-                    }
-                }
-            } else {                                                       // vocabulary
-                const float rs = s_rstd[row];
-                float best = -CUDART_INF_F;
-                int bidx = 0x7fffffff;
-#pragma unroll 1
-                for (int idx = ft; idx < on * 64; idx += SC_WORKERS) {
-                    const int f = idx >> 3, n = ufirst * 8 + f;
-                    if (n >= g.n_out) continue;
-                    const float v = sum(f) * rs;
-                    if (g.out) g.out[(size_t)row * g.n_out + n] = v;
-                    if (v > best) { best = v; bidx = n; }                   // ascending n: strict > keeps the lowest id
-                }
+            } else if (kd == GK_LM) {
                 for (int o = 8; o <= 16; o <<= 1) {
                     const float ov = __shfl_xor_sync(0xffffffffu, best, o);
                     const int oi = __shfl_xor_sync(0xffffffffu, bidx, o);
@@ -939,10 +964,19 @@ bool sc_args(const anpd_model* m, ScArgs* g, int* smem) {
         if (p.n_units < g->ncl || p.kb < CL_CTAS) return false;
         const int groups = p.u_max * p.gpu, tiles = (groups + 15) / 16;
         if (tiles > SC_MAX_TILES) return false;
-        s.kb = p.kb; s.gpu = p.gpu; s.n_units = p.n_units; s.seg = p.seg; s.copies = tiles; s.K = p.K;
+        s.kb = p.kb; s.gpu = p.gpu; s.n_units = p.n_units; s.seg = p.seg; s.tiles = tiles; s.K = p.K;
         s.kps = tiles == 1 && p.seg == p.ncl ? std::max(1, std::min(4, 16 / groups)) : 1;
         if (s.kps == 3) s.kps = 2;                       // a stage never straddles two activation slots
-        s.f_own_max = (p.u_max + CL_CTAS - 1) / CL_CTAS * 8 * p.gpu;
+        if (tiles > 1 && p.n_units / g->ncl < tiles * CL_CTAS) return false;              // every CTA finishes units of every tile
+        // the most units a CTA finishes, of the smaller and of the larger clusters
+        int own_max = 0;
+        for (int Uc = p.n_units / g->ncl; Uc <= p.u_max; ++Uc)
+            for (int r = 0; r < CL_CTAS; ++r) {
+                int own = 0;
+                for (int t = 0; t < tiles; ++t) { const int un = sc_tile_units(Uc, tiles, t), q = (r + t) % CL_CTAS; own += (q + 1) * un / CL_CTAS - q * un / CL_CTAS; }
+                own_max = std::max(own_max, own);
+            }
+        s.f_own_max = own_max * 8 * p.gpu;
         s.shift = p.gpu == 2 ? 4 : 3;
         s.red = k == GK_O || k == GK_DOWN ? 1 : 0;
         red[s.red] = std::max(red[s.red], CL_CTAS * s.f_own_max * 32);
