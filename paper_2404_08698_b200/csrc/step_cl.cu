@@ -140,7 +140,7 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
     constexpr int KS = HD / 16, DT = HD / 8, NR = STACK ? 1 : 2;      // NR: query vectors per thread
     constexpr int CC = CL_CTAS, rows = ANPD_ROWS;
     extern __shared__ __align__(1024) unsigned char sc_smem[];
-    __shared__ uint64_t w_full[SC_MAX_STAGES], w_empty[SC_MAX_STAGES], p_empty[SC_MAX_STAGES], a_full[SC_ACT_SLOTS], a_empty[SC_ACT_SLOTS];
+    __shared__ uint64_t w_full[SC_MAX_STAGES], w_empty[SC_MAX_STAGES], a_full[SC_ACT_SLOTS], a_empty[SC_ACT_SLOTS];
     __shared__ uint64_t acc_full[SC_MAX_TILES], red_full[2][SC_MAX_TILES], att_full, jan_done;
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag, s_issued;
@@ -190,7 +190,7 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
     }
     if (threadIdx.x == 64) {
         abort_flag = 0; s_issued = 0;
-        for (int s = 0; s < g.stages; ++s) { mbar_init(&w_full[s], 1); mbar_init(&w_empty[s], 1); mbar_init(&p_empty[s], WARPS); }
+        for (int s = 0; s < g.stages; ++s) { mbar_init(&w_full[s], 1); mbar_init(&w_empty[s], WARPS); }
         for (int s = 0; s < SC_ACT_SLOTS; ++s) { mbar_init(&a_full[s], 8); mbar_init(&a_empty[s], 1); }
         for (int t = 0; t < SC_MAX_TILES; ++t) { mbar_init(&acc_full[t], 1); mbar_init(&red_full[0][t], 1); mbar_init(&red_full[1][t], 1); }
         mbar_init(&att_full, 1); mbar_init(&jan_done, 1);
@@ -220,19 +220,16 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
         if (elect_one()) {
             const uint64_t pol_w = policy_evict_first(), pol_p = g.split > 1 ? policy_evict_last() : pol_w;       // pages are read again by the items that share the head
             const int* pages = g.page_table + (size_t)seq * g.pages_per_seq;
-            int stage = 0, count = 0;
-            uint32_t wpar = 0, ppar = 0, is_page = 0;
+            // by address, with as few instructions per copy as it takes: 16 KB are due every 560 cycles, and faster behind a full ring
+            const uint32_t full0 = smem_u32(&w_full[0]), empty_off = smem_u32(&w_empty[0]) - full0, full_end = full0 + 8u * (uint32_t)g.stages, ring0 = smem_u32(ring);
+            uint32_t full = full0, dst = ring0, eph = 1;        // (a fresh barrier is through with the phase before its first)
+            int turns = 0;
             bool ok = true;
-            auto take = [&](bool page) {                // the next stage, free to be written
-                const uint32_t bit = 1u << stage;
-                if (count >= g.stages) {
-                    if (is_page & bit) { ok = mbar_wait<1>(&p_empty[stage], (ppar >> stage) & 1u, abortp); ppar ^= bit; }
-                    else { ok = mbar_wait<1>(&w_empty[stage], (wpar >> stage) & 1u, abortp); wpar ^= bit; }
-                }
-                is_page = page ? is_page | bit : is_page & ~bit;
-                return ok;
+            auto next = [&]() {
+                full += 8u;
+                dst += SC_STAGE;
+                if (full == full_end) { full = full0; dst = ring0; eph ^= 1u; ++turns; }
             };
-            auto next = [&]() { ++count; if (++stage == g.stages) stage = 0; };
             auto weights = [&](int kd, const unsigned char* w) {
                 const int nk = s_geo[kd].nk, T = s_geo[kd].T, step = s_geo[kd].step, kps = g.k[kd].kps;
                 const unsigned char* src0 = w + s_geo[kd].w_off;
@@ -243,13 +240,15 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
                     for (int t = 0; t < T && ok; ++t) {
                         const unsigned char* src = src0 + ((int)s_tile[kd][t].g0 << 10);
                         const uint32_t kb_bytes = (uint32_t)s_tile[kd][t].groups << 10;
+                        uint32_t bytes = (uint32_t)kps * kb_bytes;
+                        const uint32_t src_step = kps > 1 ? bytes : (uint32_t)step;       // kps > 1 only where one tile holds all of the segment's groups
 #pragma unroll 1
-                        for (int k = 0; k < kn; k += kps) {
-                            const uint32_t bytes = (uint32_t)min(kps, kn - k) * kb_bytes;       // kps > 1 only where one tile holds all of the segment's groups
-                            if (!take(false)) break;
-                            mbar_expect_tx(&w_full[stage], bytes);
-                            bulk_load(ring + stage * SC_STAGE, src, bytes, &w_full[stage], pol_w);
-                            src += kps > 1 ? bytes : (uint32_t)step;
+                        for (int k = kn; k > 0; k -= kps) {
+                            if (k < kps) bytes = (uint32_t)k * kb_bytes;
+                            if (!mbar_wait_at<1>(full + empty_off, eph, abortp)) { ok = false; break; }
+                            bulk_load_at(dst, src, bytes, full, pol_w);
+                            mbar_arrive_at(full + empty_off, WARPS - 1);       // a page's stage is given back by eight warps, a weight stage by one commit
+                            src += src_step;
                             next();
                         }
                     }
@@ -265,19 +264,19 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
                     for (int i = 0, p = arank; i < my_pages && ok; ++i, p += g.C) {
                         const int row = (l * g.total_pages + pages[p]) * g.Hkv + kvh;
 #pragma unroll 1
-                        for (int s = 0; s < 2 * KST && ok; ++s) {
-                            if (!take(true)) break;
-                            unsigned char* dst = ring + stage * SC_STAGE;
-                            mbar_expect_tx(&w_full[stage], SC_STAGE);
-                            if (s < KST) tma_load_2d(dst, &map_k, s * 64, row * KV_PAGE, &w_full[stage], pol_p);
-                            else if (HD == 128) tma_load_2d(dst, &map_v, (s - KST) * 64, row * HD, &w_full[stage], pol_p);
-                            else { tma_load_2d(dst, &map_v, 0, row * HD, &w_full[stage], pol_p); tma_load_2d(dst + HD * 128, &map_v, 64, row * HD, &w_full[stage], pol_p); }
+                        for (int s = 0; s < 2 * KST; ++s) {
+                            if (!mbar_wait_at<1>(full + empty_off, eph, abortp)) { ok = false; break; }
+                            mbar_expect_tx_at(full, SC_STAGE);
+                            if (s < KST) tma_load_2d_at(dst, &map_k, s * 64, row * KV_PAGE, full, pol_p);
+                            else if (HD == 128) tma_load_2d_at(dst, &map_v, (s - KST) * 64, row * HD, full, pol_p);
+                            else { tma_load_2d_at(dst, &map_v, 0, row * HD, full, pol_p); tma_load_2d_at(dst + HD * 128, &map_v, 64, row * HD, full, pol_p); }
                             next();
                         }
                     }
                 }
             }
             if (ok) weights(GK_LM, g.w[GK_LM]);
+            const int count = turns * g.stages + (int)((full - full0) >> 3);
             s_issued = count;
         }
         __syncwarp();
@@ -564,7 +563,7 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
                     __syncwarp();
                     if (lane == 0) {
 #pragma unroll
-                        for (int s = 0; s < KST; ++s) mbar_arrive(&p_empty[st(s)]);
+                        for (int s = 0; s < KST; ++s) mbar_arrive(&w_empty[st(s)]);
                     }
                     uint32_t ph[4], pl[4];
                     float resc[NR];
@@ -618,14 +617,14 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
                 } else {
                     if (lane == 0) {
 #pragma unroll
-                        for (int s = 0; s < KST; ++s) mbar_arrive(&p_empty[st(s)]);
+                        for (int s = 0; s < KST; ++s) mbar_arrive(&w_empty[st(s)]);
                     }
                     mbar_wait<1>(&w_full[vst], vpar, abortp);
                 }
                 __syncwarp();
                 if (lane == 0) {
 #pragma unroll
-                    for (int s = KST; s < 2 * KST; ++s) mbar_arrive(&p_empty[st(s)]);
+                    for (int s = KST; s < 2 * KST; ++s) mbar_arrive(&w_empty[st(s)]);
                 }
             }
             // ---- the warps, in order ----
