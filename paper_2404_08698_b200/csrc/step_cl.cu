@@ -7,7 +7,7 @@
 // five hand-overs per layer.  As a kernel per projection a hand-over took about 3 us: the last CTA's exit and the boundary behind it, tensor
 // memory and barriers set up again, code from a cold instruction cache, a weight ring that starts empty or half an SM wide.  Here the ring runs
 // through: the weight thread walks all layers' weights, and the cache's pages between them, and never waits for an activation.  us per step:
-// 1.1B at 512 keys 729 -> 597, 1024 wide (16 layers) 380 -> 264, 7B (16 layers and the head) at 77 keys 1294 -> 1138, at 1536 1382 -> 1216, tiny
+// 1.1B at 512 keys 729 -> 553, 1024 wide (16 layers) 380 -> 264, 7B (16 layers and the head) at 77 keys 1294 -> 1075, at 1536 1382 -> 1216, tiny
 // (2 x 256) 48 -> 43.
 //
 // Hand-over.  The exchange buffers hold nothing but all-ones words until their values are written, and no value is one (a NaN that
@@ -41,7 +41,7 @@ namespace {
 
 using namespace tc;
 
-constexpr int SC_THREADS = 352;          // warp 0: weights and pages, 1: products, 2: exchange buffers, 3-10: workers
+constexpr int SC_THREADS = 384;          // warp 0: weights and pages, 1: products, 2: exchange buffers, 3-10: workers, 11: L2 prefetch
 constexpr int SC_WORKERS = 256;
 constexpr int SC_STAGE = 16384;          // one slot of the ring: at most 16 groups of 8 features x 64 inputs, or part of a page
 constexpr int SC_MAX_STAGES = 12;
@@ -77,7 +77,8 @@ struct ScArgs {
     const unsigned char* w[GK_COUNT];    // the first layer's; the others follow `layer_step` bytes apart
     const float *attn_norm, *ffn_norm, *final_norm;
     size_t layer_step;
-    int L, ncl, stages, tmem_cols, red_bytes;
+    unsigned* entered;                   // CTAs that have requested all weights before a projection, over all steps
+    int L, ncl, stages, tmem_cols, red_bytes, ahead;
     // what the embedding left
     const unsigned char* img0;
     const float *x0, *ss0;
@@ -143,6 +144,7 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
     __shared__ uint64_t w_full[SC_MAX_STAGES], w_empty[SC_MAX_STAGES], a_full[SC_ACT_SLOTS], a_empty[SC_ACT_SLOTS];
     __shared__ uint64_t acc_full[SC_MAX_TILES], red_full[2][SC_MAX_TILES], att_full, jan_done;
     __shared__ uint32_t tmem_slot;
+    __shared__ volatile int s_requested, s_phase, s_quit;         // copies of weights requested so far; all of them, or none will follow
     __shared__ int abort_flag, s_issued;
     __shared__ float s_rstd[8], s_part[8][8];
     __shared__ int s_pos[8], s_slot[8], s_page[8], s_raw[8], s_idx[8][8];
@@ -189,7 +191,7 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
         s_geo[threadIdx.x] = e;
     }
     if (threadIdx.x == 64) {
-        abort_flag = 0; s_issued = 0;
+        abort_flag = 0; s_issued = 0; s_requested = 0; s_phase = 0; s_quit = 0;
         for (int s = 0; s < g.stages; ++s) { mbar_init(&w_full[s], 1); mbar_init(&w_empty[s], WARPS); }
         for (int s = 0; s < SC_ACT_SLOTS; ++s) { mbar_init(&a_full[s], 8); mbar_init(&a_empty[s], 1); }
         for (int t = 0; t < SC_MAX_TILES; ++t) { mbar_init(&acc_full[t], 1); mbar_init(&red_full[0][t], 1); mbar_init(&red_full[1][t], 1); }
@@ -223,7 +225,7 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
             // by address, with as few instructions per copy as it takes: 16 KB are due every 560 cycles, and faster behind a full ring
             const uint32_t full0 = smem_u32(&w_full[0]), empty_off = smem_u32(&w_empty[0]) - full0, full_end = full0 + 8u * (uint32_t)g.stages, ring0 = smem_u32(ring);
             uint32_t full = full0, dst = ring0, eph = 1;        // (a fresh barrier is through with the phase before its first)
-            int turns = 0;
+            int turns = 0, requested = 0;
             bool ok = true;
             auto next = [&]() {
                 full += 8u;
@@ -249,6 +251,7 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
                             bulk_load_at(dst, src, bytes, full, pol_w);
                             mbar_arrive_at(full + empty_off, WARPS - 1);       // a page's stage is given back by eight warps, a weight stage by one commit
                             src += src_step;
+                            s_requested = ++requested;
                             next();
                         }
                     }
@@ -259,25 +262,30 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
 #pragma unroll 1
                 for (int kd = 0; kd < 4 && ok; ++kd) {
                     weights(kd, g.w[kd] + (size_t)l * g.layer_step);
-                    if (kd != GK_QKV) continue;
+                    if (kd == GK_QKV) {
 #pragma unroll 1
-                    for (int i = 0, p = arank; i < my_pages && ok; ++i, p += g.C) {
-                        const int row = (l * g.total_pages + pages[p]) * g.Hkv + kvh;
+                        for (int i = 0, p = arank; i < my_pages && ok; ++i, p += g.C) {
+                            const int row = (l * g.total_pages + pages[p]) * g.Hkv + kvh;
 #pragma unroll 1
-                        for (int s = 0; s < 2 * KST; ++s) {
-                            if (!mbar_wait_at<1>(full + empty_off, eph, abortp)) { ok = false; break; }
-                            mbar_expect_tx_at(full, SC_STAGE);
-                            if (s < KST) tma_load_2d_at(dst, &map_k, s * 64, row * KV_PAGE, full, pol_p);
-                            else if (HD == 128) tma_load_2d_at(dst, &map_v, (s - KST) * 64, row * HD, full, pol_p);
-                            else { tma_load_2d_at(dst, &map_v, 0, row * HD, full, pol_p); tma_load_2d_at(dst + HD * 128, &map_v, 64, row * HD, full, pol_p); }
-                            next();
+                            for (int s = 0; s < 2 * KST; ++s) {
+                                if (!mbar_wait_at<1>(full + empty_off, eph, abortp)) { ok = false; break; }
+                                mbar_expect_tx_at(full, SC_STAGE);
+                                if (s < KST) tma_load_2d_at(dst, &map_k, s * 64, row * KV_PAGE, full, pol_p);
+                                else if (HD == 128) tma_load_2d_at(dst, &map_v, (s - KST) * 64, row * HD, full, pol_p);
+                                else { tma_load_2d_at(dst, &map_v, 0, row * HD, full, pol_p); tma_load_2d_at(dst + HD * 128, &map_v, 64, row * HD, full, pol_p); }
+                                s_requested = ++requested;
+                                next();
+                            }
                         }
                     }
+                    atomicAdd(g.entered + 4 * l + kd + 1, 1u);
+                    s_phase = 4 * l + kd + 1;
                 }
             }
             if (ok) weights(GK_LM, g.w[GK_LM]);
             const int count = turns * g.stages + (int)((full - full0) >> 3);
             s_issued = count;
+            s_quit = 1;
         }
         __syncwarp();
     } else if (warp == 1) {
@@ -369,6 +377,54 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
             __syncwarp();
             if (lane == 0) mbar_arrive(&jan_done);
         }
+    } else if (warp == 11) {
+        // ---------------- into L2 what the ring will ask for ----------------
+        // While results go from phase to phase the ring is full and HBM would idle (7B: 10 us of a layer's 67); what is prefetched meanwhile comes in at
+        // L2's rate behind the hand-over.  `ahead` copies at most beyond those requested, across projections - but into the one being requested only
+        // once every CTA has requested all before it: CTAs are spread unevenly over the two dies (56 and 72 on one GPU, 60 and 68 on another), and those
+        // of the emptier die would run ahead at the others' expense (7B at 1536 keys 1181 -> 1156 us).  us per step without prefetch and with: 1.1B at 512 keys
+        // 590 -> 553, at 3000 683 -> 652, 7B (16 layers) at 77 keys 1142 -> 1075, from 1536 on the same within the runs' spread (1225, 1290).
+        if (elect_one() && g.ahead > 0) {
+            uint32_t all = ld_relaxed1(g.entered + 4 * g.L) + (uint32_t)ncta;       // the last phase's count is that of the step before
+            int opened = 0;
+            int idx = 0;                                // the walk's copy, of all weights
+            auto prefetch = [](const void* src, uint32_t bytes) { asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory"); };
+            auto turn = [&]() {                         // waits until copy idx is near enough; false: it has been requested
+                if (idx < s_requested) return false;
+                while (true) {
+                    const int pr = s_requested, ph = s_phase;
+                    if (idx < pr || s_quit) return false;
+                    if (idx < pr + g.ahead) {
+                        if (ph > opened && (int)(ld_relaxed1(g.entered + ph) - all) >= 0) opened = ph;
+                        if (ph == opened) return true;
+                    }
+                    __nanosleep(40);
+                }
+            };
+            int kd = GK_QKV, l = 0;
+#pragma unroll 1
+            while (!s_quit) {
+                const int nk = s_geo[kd].nk, T = s_geo[kd].T, step = s_geo[kd].step, kps = g.k[kd].kps;
+                const unsigned char* src0 = g.w[kd] + (kd == GK_LM ? 0 : (size_t)l * g.layer_step) + s_geo[kd].w_off;
+#pragma unroll 1
+                for (int k0 = 0; k0 < nk; k0 += SC_CHUNK, src0 += (size_t)SC_CHUNK * step) {
+                    const int kn = min(SC_CHUNK, nk - k0);
+#pragma unroll 1
+                    for (int t = 0; t < T; ++t) {
+                        const unsigned char* src = src0 + ((int)s_tile[kd][t].g0 << 10);
+                        const uint32_t kb_bytes = (uint32_t)s_tile[kd][t].groups << 10, src_step = kps > 1 ? (uint32_t)kps * kb_bytes : (uint32_t)step;
+#pragma unroll 1
+                        for (int k = kn; k > 0; k -= kps, src += src_step, ++idx) {
+                            if (turn()) prefetch(src, (uint32_t)min(k, kps) * kb_bytes);
+                        }
+                    }
+                }
+                if (kd == GK_QKV) idx += pg_st;         // the pages are left to the ring (prefetched too, 7B steps at 1536 keys took 1 % longer)
+                if (kd == GK_LM) break;
+                if (kd == GK_DOWN) { ++l; kd = l == g.L ? GK_LM : GK_QKV; } else ++kd;
+            }
+        }
+        __syncwarp();
     } else {
         // ---------------- workers ----------------
         const int fw = warp - 3, ft = fw * 32 + lane, row = ft & 7;                  // worker warp and thread, its row
@@ -898,7 +954,7 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
 
     // Leaving: nothing is under way to a CTA that is through its last epilogue; the barrier only keeps a CTA whose wait ran out from leaving
     // under the others.
-    if (warp < 3) cluster_wait();
+    if (warp < 3 || warp == 11) cluster_wait();
     tc_fence_before();
     __syncthreads();
     if (warp == 1) {
@@ -989,6 +1045,16 @@ bool sc_args(const anpd_model* m, ScArgs* g, int* smem) {
     g->stages = std::min(SC_MAX_STAGES, (SC_SMEM - rest) / SC_STAGE);
     if (g->stages < 5) return false;                     // a page and a stage of weights
     *smem = rest + g->stages * SC_STAGE;
+    // How far the prefetch reaches, in copies: half a layer's, at most 24 (50 MB for all CTAs).  us per step with none, 16,
+    // 24, 32 and 48: 1.1B (47 copies a layer and CTA) 592, 550, 553, 562, 662; 7B, 16 layers (203) 1136, 1055, 1043, 1034, 1035; 13B, 8 layers (368)
+    // 903, 888, 870, 861, 865; 7B at 3000 keys 1287, -, 1290, 1320 (there the pages take what the prefetch takes).  A layer of less than 28 copies, three to four rings full, is better off without: 1280 wide (25) 227 -> 230, 1024 wide
+    // (16) 263 -> 273, but 1536 wide (29) 262 -> 258.
+    int copies = 0;
+    for (int k = 0; k < GK_LM; ++k) {
+        const int nk = (g->k[k].kb + CL_CTAS - 1) / CL_CTAS;
+        copies += g->k[k].tiles == 1 ? (nk + g->k[k].kps - 1) / g->k[k].kps : nk * g->k[k].tiles;
+    }
+    g->ahead = copies < 28 ? 0 : std::min(24, copies / 2);
     g->L = c.n_layers; g->d = c.d_model; g->Hq = c.n_q_heads; g->Hkv = c.n_kv_heads; g->n_out = c.vocab;
     g->inv_d = 1.0f / (float)c.d_model; g->eps = c.rms_eps; g->q_scale = 1.4426950408889634f / sqrtf((float)c.head_dim);
     // the layers' tensors lie at one distance
@@ -1028,7 +1094,7 @@ size_t step_cl_bytes(const anpd_model* m, int batch) {
     int smem = 0;
     if (batch != 1 || !m->cl_all_fused || m->plain_gemm || std::getenv("ANPD_STEP_CHAIN") || !sc_args(m, &g, &smem)) return 0;
     const bool ok = sc_form(m->cfg) == 2 ? fits_step_cl<128, 1>(g.ncl, smem) : sc_form(m->cfg) == 1 ? fits_step_cl<64, 2>(g.ncl, smem) : fits_step_cl<64, 1>(g.ncl, smem);
-    return ok ? 2 * (size_t)g.copy_bytes + g.fin_bytes : 0;
+    return ok ? 2 * (size_t)g.copy_bytes + g.fin_bytes + 4 * (4 * (size_t)g.L + 1) : 0;
 }
 
 anpd_status step_cl_enqueue(anpd_model* m, anpd_kv* kv, bool want_logits, bool tree) {
@@ -1038,6 +1104,7 @@ anpd_status step_cl_enqueue(anpd_model* m, anpd_kv* kv, bool want_logits, bool t
     if (!sc_args(m, &g, &smem)) return ANPD_ERR_STATE;
     g.img0 = ws.ci_h; g.x0 = ws.x; g.ss0 = ws.ss_cl_a;
     g.xch = ws.xch;
+    g.entered = (unsigned*)(ws.xch + 2 * (size_t)g.copy_bytes + g.fin_bytes);
     g.row_pos = ws.row_pos; g.row_slot = ws.row_slot; g.row_seq = ws.row_seq; g.row_ok = ws.row_ok; g.hole_lo = ws.row_hole_lo; g.hole_hi = ws.row_hole_hi;
     g.tree = tree ? 1 : 0;
     g.rope_cos = kv->rope_cos; g.rope_sin = kv->rope_sin;
