@@ -26,11 +26,17 @@
 // that the tiles take turns every 24.  us per step against all tiles of a k-block together: 1.1B 627 -> 597, 1024 wide 291 -> 264,
 // 7B (16 layers) at 77 keys 1147 -> 1138, 13B (8 layers) 947 -> 931.
 //
+// Narrow tiles.  A product reads 128 rows of weights from shared memory whatever they hold, beside the copies that fill the ring (350 cycles per
+// 16 KB stage then, 160 alone).  Where a cluster has 64 or 32 features of the residual stream, the two or four k-blocks of a stage are rows of one
+// product, its columns the activations of all of them, and the sums that count lie where a k-block's rows meet its columns: a half or a quarter
+// of the products.  1.1B: O 2185 -> 1665 cycles, down 6344 -> 4856, 551 -> 539 us per step; 1024 wide 264 -> 262.
+//
 // The keys and values of the step itself reach the attention the same way; the pages are copied in before they can hold them (any time:
 // they are as old as the step before), and the rows are put into the copy.
 //
-// Values are those of gemm_cl.cu and attn_dec.cu: the same cut of K, the same order of parts, pages, warps and CTAs.  They are equal bit for
-// bit up to 4096 features; beyond (two tiles of the residual stream) a row's sum of squares comes in other groups.
+// Values are those of gemm_cl.cu and attn_dec.cu: the same cut of K, the same order of parts, pages, warps and CTAs, and so equal bit for bit -
+// but where products are packed (their k-blocks' sums meet at the end), beyond 4096 features (two tiles of the residual stream: a row's sum of
+// squares comes in other groups).
 // Every wait is bounded and reports through the error flag; a handle that has failed once refuses all further results.
 #include "step_dev.cuh"
 
@@ -66,7 +72,8 @@ template <int HD, int G> struct ScCfg {                      // G: query heads a
     static_assert(SLOTS + QROWS * QP <= SC_ACT_SLOTS * SC_ACT_SLOT, "attention's buffers take the activations' place");
 };
 
-struct ScKind { int kb, gpu, n_units, seg, tiles, kps, K, f_own_max, shift, red; };
+// kps: k-blocks of a stage; pack: how many of them one product takes side by side (see the kernel), 1 or kps
+struct ScKind { int kb, gpu, n_units, seg, tiles, kps, pack, K, f_own_max, shift, red; };
 // a projection as this cluster and CTA see it: tiles, k-blocks, where the weights start and the bytes from a k-block to the next
 struct ScGeo { int T, nk, kb_lo, n_st, step; unsigned long long w_off; };
 // a tile: its groups, the first one (of the cluster's), the units that each rank has finished before it, this CTA's units of it
@@ -293,23 +300,25 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
         if (elect_one()) {
             // fp32 accumulate, bf16 x bf16, both operands K-major, M = 128 features, N = 16 (hi terms, then lo terms)
             const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)((2 * rows) >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
-            const uint32_t ring_lo = smem_desc_lo(smem_u32(ring)), act_lo = smem_desc_lo(smem_u32(abuf));
+            const uint64_t ring_d = make_smem_desc(smem_u32(ring)), act_d = make_smem_desc(smem_u32(abuf));
             const uint32_t stage_step = SC_STAGE >> 4, act_step = SC_ACT_SLOT >> 4, kb_step = (uint32_t)(rows * 256) >> 4;
             const uint32_t full0 = smem_u32(&w_full[0]), empty_off = smem_u32(&w_empty[0]) - full0, full_end = full0 + 8u * (uint32_t)g.stages;
-            uint32_t full = full0, wph = 0, w_lo = ring_lo;
+            uint32_t full = full0, wph = 0;
+            uint64_t w_d = ring_d;
             const uint32_t af0 = smem_u32(&a_full[0]), aempty_off = smem_u32(&a_empty[0]) - af0, af_end = af0 + 8u * SC_ACT_SLOTS;
-            uint32_t afull = af0, aph = 0, a_lo = act_lo;
+            uint32_t afull = af0, aph = 0;
+            uint64_t a_d = act_d;
             // A wait that gave up has set the abort flag; the loops run on with whatever the buffers hold (every later wait is short then).
             auto next_stage = [&]() {
                 tc_commit_at(full + empty_off);
-                w_lo += stage_step;
+                w_d += stage_step;
                 full += 8u;
-                if (full == full_end) { full = full0; wph ^= 1u; w_lo = ring_lo; }
+                if (full == full_end) { full = full0; wph ^= 1u; w_d = ring_d; }
             };
             int kd = GK_QKV, l = 0;
 #pragma unroll 1
             while (true) {
-                const int nk = s_geo[kd].nk, T = s_geo[kd].T, kps = g.k[kd].kps;
+                const int nk = s_geo[kd].nk, T = s_geo[kd].T, kps = g.k[kd].kps, pack = g.k[kd].pack;
                 uint32_t acc = 0;
 #pragma unroll 1
                 for (int k0 = 0; k0 < nk; k0 += SC_CHUNK) {
@@ -318,37 +327,44 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
 #pragma unroll 1
                     for (int t = 0; t < T; ++t) {
                         const uint32_t kb_words = (uint32_t)s_tile[kd][t].groups << 6;
-                        uint32_t af = afull, ap = aph, alo = a_lo, accumulate = acc;
+                        uint32_t af = afull, ap = aph, accumulate = acc;
+                        uint64_t ad = a_d;
 #pragma unroll 1
                         for (int ks = 0; ks < kn; ks += SC_AKB) {
                             if (t == 0) { mbar_wait_at<1>(af, ap, abortp); tc_fence_after(); }
                             const int kend = min(SC_AKB, kn - ks);
-                            uint32_t a = alo;
+                            uint64_t a = ad;
                             // a tile of fewer than 16 groups: the instruction reads whatever follows for the rows beyond, whose lanes nobody reads
 #pragma unroll 1
                             for (int k = 0; k < kend; k += kps) {
                                 mbar_wait_at<1>(full, wph, abortp);
                                 tc_fence_after();
-                                tc_mma_k64(d_tmem, w_lo, a, idesc, accumulate);
+                                const int n = min(kps, kend - k);
+                                // packed: the stage's k-blocks are rows of one product, side by side, and its columns are the activations of all of
+                                // them; of the sums, those count where a k-block's rows meet its own columns
+                                tc_mma_k64(d_tmem, w_d, a, pack > 1 ? idesc + ((uint32_t)(n - 1) << 18) : idesc, accumulate);
                                 accumulate = 1;
-                                a += kb_step;
-                                uint32_t w = w_lo;
-#pragma unroll 1
-                                for (int j = min(kps, kend - k); j > 1; --j) {
-                                    w += kb_words;
-                                    tc_mma_k64(d_tmem, w, a, idesc, 1u);
+                                if (pack > 1) a += (uint32_t)n * kb_step;
+                                else {
                                     a += kb_step;
+                                    uint64_t w = w_d;
+#pragma unroll 1
+                                    for (int j = n; j > 1; --j) {
+                                        w += kb_words;
+                                        tc_mma_k64(d_tmem, w, a, idesc, 1u);
+                                        a += kb_step;
+                                    }
                                 }
                                 next_stage();
                             }
                             if (t == T - 1) tc_commit_at(af + aempty_off);
-                            alo += act_step;
+                            ad += act_step;
                             af += 8u;
-                            if (af == af_end) { af = af0; ap ^= 1u; alo = act_lo; }
+                            if (af == af_end) { af = af0; ap ^= 1u; ad = act_d; }
                         }
                         if (k0 + kn == nk) tc_commit(&acc_full[t]);
                         d_tmem += (uint32_t)(2 * rows);
-                        if (t == T - 1) { afull = af; aph = ap; a_lo = alo; }
+                        if (t == T - 1) { afull = af; aph = ap; a_d = ad; }
                     }
                     acc = 1;
                 }
@@ -358,7 +374,7 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
                     wph ^= (uint32_t)(st / g.stages) & 1u;
                     st %= g.stages;
                     full = full0 + 8u * (uint32_t)st;
-                    w_lo = ring_lo + stage_step * (uint32_t)st;
+                    w_d = ring_d + stage_step * (uint32_t)st;
                 }
                 if (kd == GK_DOWN) { ++l; kd = l == g.L ? GK_LM : GK_QKV; } else ++kd;
             }
@@ -755,7 +771,7 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
                 if (att) attention(l, copy);
                 adv(st_rest);
             }
-            const int T = s_geo[kd].T, shift = g.k[kd].shift, f_own_max = g.k[kd].f_own_max;
+            const int T = s_geo[kd].T, shift = g.k[kd].shift, f_own_max = g.k[kd].f_own_max, pack = g.k[kd].pack;
             const bool resid = kd == GK_O || kd == GK_DOWN;
             const int region = resid ? 1 : 0;
             float2 gn = make_float2(0.f, 0.f);
@@ -766,7 +782,7 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
             }
             if (ft < T) {                                // what the cluster will send here for each tile
                 const int n = s_tile[kd][ft].own_n;
-                mbar_expect_tx(&red_full[region][ft], (uint32_t)(n ? (n << shift) * CC * 32 : CC * 16));
+                mbar_expect_tx(&red_full[region][ft], (uint32_t)(n ? (n << shift) * CC * pack * 32 : CC * 16));
             }
             load_acts(kd == GK_QKV ? (l ? prev : g.img0) : kd == GK_LM ? fin : copy + (kd == GK_O ? g.o_ao : kd == GK_GU ? g.o_h2 : g.o_act), kd);
             // 1 / RMS of every row: a warp per row, 32 interleaved sums over the parts, then a tree over the lanes
@@ -817,7 +833,10 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
                         const int f = 2 * (idx >> 3), n = unit_of(kd, t, idx) * 8 + (f & 7);
                         if (idx != ft) gn = *(const float2*)(gain + n);
                         float2 x = s_x[idx];
-                        x.x += sum(f); x.y += sum(f + 1);
+                        float2 v = make_float2(sum(f), sum(f + 1));
+#pragma unroll 1
+                        for (int q = 1; q < pack; ++q) { v.x += sum(f + q * CC * f_own_max); v.y += sum(f + 1 + q * CC * f_own_max); }
+                        x.x += v.x; x.y += v.y;
                         s_x[idx] = x;
                         ssq += x.x * x.x + x.y * x.y;
                         uint32_t hi, lo2;
@@ -895,16 +914,18 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
             for (int t = 0; t <= T; ++t) {
                 if (t < T) {
                     // thread: a feature (tensor-memory lane) and four of the rows
-                    const int un = s_tile[kd][t].groups >> (shift - 3), pos = quad * 32 + lane, u = pos >> shift;
+                    // (packed: the lanes of the second k-block's rows hold the same features' sums over other k-blocks, in columns of their own)
+                    const int lanes = (int)s_tile[kd][t].groups * 8, part = pack > 1 ? quad * 32 / lanes : 0;
+                    const int un = s_tile[kd][t].groups >> (shift - 3), pos = quad * 32 + lane - part * lanes, u = pos >> shift;
                     const int b1 = un / 4, b2 = un / 2, b3 = 3 * un / 4, q = (u >= b1) + (u >= b2) + (u >= b3), owner = (q - t) & (CC - 1);
                     const int local = ((s_tile[kd][t].before[owner] + u - (q * un) / CC) << shift) + (pos & ((1 << shift) - 1));
                     mbar_wait<1>(&acc_full[t], (acc_par >> t) & 1u, abortp);
                     tc_fence_after();
                     float v[4];
-                    const uint32_t col = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(t * 2 * rows + (pushes ? 0 : 4));
+                    const uint32_t col = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)((t + part) * 2 * rows + (pushes ? 0 : 4));
                     tc_ld4_sum(col, col + 8u, v);
-                    const uint32_t bar0 = smem_u32(&red_full[region][t]), to = red_addr + (uint32_t)(g.k[kd].red + (rank * f_own_max + local) * 32 + (pushes ? 0 : 16));
-                    if (pos < (int)s_tile[kd][t].groups * 8) st_async4(map_to_cta(to, (uint32_t)owner), map_to_cta(bar0, (uint32_t)owner), v[0], v[1], v[2], v[3]);
+                    const uint32_t bar0 = smem_u32(&red_full[region][t]), to = red_addr + (uint32_t)(g.k[kd].red + ((part * CC + rank) * f_own_max + local) * 32 + (pushes ? 0 : 16));
+                    if (pos < lanes) st_async4(map_to_cta(to, (uint32_t)owner), map_to_cta(bar0, (uint32_t)owner), v[0], v[1], v[2], v[3]);
                     // a CTA that finishes nothing of the tile hears from the others all the same: it is then behind them
                     if (ft < CC && (ft + 1) * un / CC == ft * un / CC) {
                         const uint32_t o = (uint32_t)((ft - t) & (CC - 1));
@@ -1033,9 +1054,11 @@ bool sc_args(const anpd_model* m, ScArgs* g, int* smem) {
             }
         s.f_own_max = own_max * 8 * p.gpu;
         s.shift = p.gpu == 2 ? 4 : 3;
+        // a stage's k-blocks fill whole warps' lanes, in every cluster alike, and every CTA has a full stage of them
+        s.pack = (k == GK_O || k == GK_DOWN) && s.kps > 1 && p.n_units % g->ncl == 0 && groups % 4 == 0 && groups * s.kps <= 16 && p.kb >= CL_CTAS * s.kps ? s.kps : 1;
         s.red = k == GK_O || k == GK_DOWN ? 1 : 0;
-        red[s.red] = std::max(red[s.red], CL_CTAS * s.f_own_max * 32);
-        tiles_max = std::max(tiles_max, tiles);
+        red[s.red] = std::max(red[s.red], CL_CTAS * s.pack * s.f_own_max * 32);
+        tiles_max = std::max(tiles_max, tiles * s.pack);
     }
     for (int k = 0; k < GK_COUNT; ++k) g->k[k].red = g->k[k].red ? red[0] : 0;
     g->red_bytes = red[0] + red[1];

@@ -108,6 +108,32 @@ __device__ __forceinline__ void tc_mma_bf16(uint32_t d_tmem, uint64_t a_desc, ui
         "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, {%5, %5, %5, %5}, p;\n\t}"
         ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(0u) : "memory");
 }
+// Shared-memory operand descriptor: K-major tile, 128-byte swizzle, rows of 128 bytes, groups of
+// 8 rows 1024 bytes apart (the layout a TMA load with the 128B swizzle mode produces).
+__device__ __forceinline__ uint64_t make_smem_desc(uint32_t saddr) {
+    uint64_t d = (uint64_t)((saddr >> 4) & 0x3FFFu);
+    d |= (uint64_t)1 << 16;               // leading byte offset (unused for swizzled K-major), 16-byte units
+    d |= (uint64_t)(1024 >> 4) << 32;     // stride byte offset between 8-row groups
+    d |= (uint64_t)1 << 46;               // descriptor version of this architecture
+    d |= (uint64_t)2 << 61;               // 128-byte swizzle
+    return d;
+}
+// One product by its operands' descriptors, and the four along a 64-wide k-block (32 bytes = 2 units per 16 inputs).  With the descriptors as
+// 64-bit values the four take their issuing thread 156 cycles (92 with 64 rows), 168 with a wait and a commit; put together from halves
+// inside one statement, 243 and 329.
+__device__ __forceinline__ void tc_mma_desc(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+        ::"r"(d_tmem), "l"(a), "l"(b), "r"(idesc), "r"(accumulate) : "memory");
+}
+__device__ __forceinline__ void tc_mma_k64(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accumulate) {
+    tc_mma_desc(d_tmem, a, b, idesc, accumulate);
+    tc_mma_desc(d_tmem, a + 2, b + 2, idesc, 1u);
+    tc_mma_desc(d_tmem, a + 4, b + 4, idesc, 1u);
+    tc_mma_desc(d_tmem, a + 6, b + 6, idesc, 1u);
+}
 // One 128-feature x 64-input weight tile times the step's rows: four MMAs along K.  The descriptors differ in their low words
 // only (32 bytes = 2 units per 16 inputs), so that is all a caller keeps: a thread that issues these back to back is bound by
 // its own few instructions per tile, each of several cycles.
@@ -220,16 +246,6 @@ __device__ __forceinline__ void tc_st16(uint32_t taddr, const float* v) {
         : "memory");
 }
 
-// Shared-memory operand descriptor: K-major tile, 128-byte swizzle, rows of 128 bytes, groups of
-// 8 rows 1024 bytes apart (the layout a TMA load with the 128B swizzle mode produces).
-__device__ __forceinline__ uint64_t make_smem_desc(uint32_t saddr) {
-    uint64_t d = (uint64_t)((saddr >> 4) & 0x3FFFu);
-    d |= (uint64_t)1 << 16;               // leading byte offset (unused for swizzled K-major), 16-byte units
-    d |= (uint64_t)(1024 >> 4) << 32;     // stride byte offset between 8-row groups
-    d |= (uint64_t)1 << 46;               // descriptor version of this architecture
-    d |= (uint64_t)2 << 61;               // 128-byte swizzle
-    return d;
-}
 
 
 }  // namespace tc
