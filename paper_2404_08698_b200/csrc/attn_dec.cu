@@ -29,17 +29,13 @@
 
 typedef __nv_bfloat16 bf16;
 
-// CTAs per head, and clusters that share a kv head
+// CTAs per item.
 constexpr int AD_MAX_CLUSTER = 4;
 int ad_cluster(const anpd_model* m, int heads) {
     const int resident = m->num_sms * 7 / 8;
     int cluster = AD_MAX_CLUSTER;
     while (cluster > 1 && heads * cluster > resident) cluster /= 2;
     return cluster;
-}
-int ad_split(const anpd_model_config& c) {
-    const int group = c.n_q_heads / c.n_kv_heads;
-    return c.head_dim == 64 && group > 1 ? group / 2 : group;
 }
 
 namespace {
@@ -359,6 +355,12 @@ __global__ void __launch_bounds__((AdCfg<HD, G>::THREADS)) __maxnreg__((AdCfg<HD
             for (unsigned spin = 0; spin < WAIT_LIMIT && !mbar_try_wait(&full[i % CHUNKS], (uint32_t)((i / CHUNKS) & 1)); ++spin) {}
         atomicExch(g.err, AD_ERR_TIMEOUT);
     }
+}
+
+// Clusters that share a kv head.
+int ad_split(const anpd_model_config& c) {
+    const int group = c.n_q_heads / c.n_kv_heads;
+    return c.head_dim == 64 && group > 1 ? group / 2 : group;
 }
 
 template <int HD, int G>

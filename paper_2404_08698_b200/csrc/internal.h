@@ -536,7 +536,6 @@ anpd_status attn_tc_enqueue(anpd_model* m, anpd_kv* kv, int layer, int rows, int
 // attn_dec.cu: attention of a decode step, written straight to the O projection's operand image
 anpd_status attn_dec_enqueue(anpd_model* m, anpd_kv* kv, int layer, bool tree);
 int ad_cluster(const anpd_model* m, int heads);         // CTAs that share the pages of an item
-int ad_split(const anpd_model_config& c);               // items that share a kv head
 // step_cl.cu: everything of a single sequence's step between the embedding and the argmax, in one kernel.  Bytes of the buffers its CTAs
 // exchange results through (Workspace::xch, all ones at first), 0 where the shape or the handle is not one for it.
 size_t step_cl_bytes(const anpd_model* m, int batch);

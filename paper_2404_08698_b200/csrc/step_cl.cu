@@ -7,8 +7,8 @@
 // five hand-overs per layer.  As a kernel per projection a hand-over took about 3 us: the last CTA's exit and the boundary behind it, tensor
 // memory and barriers set up again, code from a cold instruction cache, a weight ring that starts empty or half an SM wide.  Here the ring runs
 // through: the weight thread walks all layers' weights, and the cache's pages between them, and never waits for an activation.  us per step:
-// 1.1B at 512 keys 729 -> 553, 1024 wide (16 layers) 380 -> 264, 7B (16 layers and the head) at 77 keys 1294 -> 1075, at 1536 1382 -> 1216, tiny
-// (2 x 256) 48 -> 43.
+// 1.1B at 512 keys 729 -> 522, 1024 wide (16 layers) 380 -> 262, 7B (16 layers and the head) at 77 keys 1294 -> 1075, at 1536 1382 -> 1216, tiny
+// (2 x 256) 48 -> 42.
 //
 // Hand-over.  The exchange buffers hold nothing but all-ones words until their values are written, and no value is one (a NaN that
 // arithmetic or a rounding to bf16 leaves has its top bit clear): the words are their own flags.  A reader polls the very data it needs, with
@@ -36,7 +36,8 @@
 //
 // Values are those of gemm_cl.cu and attn_dec.cu: the same cut of K, the same order of parts, pages, warps and CTAs, and so equal bit for bit -
 // but where products are packed (their k-blocks' sums meet at the end), beyond 4096 features (two tiles of the residual stream: a row's sum of
-// squares comes in other groups).
+// squares comes in other groups),
+// and for query heads of dimension 64 that share a kv head (a warp takes the products of one of them, not of two).
 // Every wait is bounded and reports through the error flag; a handle that has failed once refuses all further results.
 #include "step_dev.cuh"
 
@@ -59,17 +60,16 @@ constexpr int SC_MAX_TILES = 8;          // tiles of 128 features a projection m
 constexpr unsigned SC_POLL_LIMIT = 1u << 21;
 constexpr int SC_ERR_TIMEOUT = 209;
 
-template <int HD, int G> struct ScCfg {                      // G: query heads a CTA takes (1 or 2 of those that share a kv head)
-    static constexpr bool STACK = G == 1;                    // hi and lo terms of the 8 vectors share a tile
-    static constexpr int NV = STACK ? 8 : 16;                // query vectors of the CTA: one tile
-    static constexpr int WARPS = 8;                          // each with 16 keys of a page
+// Attention: a query head per item, 8 query vectors (with two heads of dimension 64 that share a kv head per item only half of the CTAs have
+// one where there are 32: 1.1B at 512 keys 541 -> 525 us per step, at 3000 638 -> 575; 1536 wide 260 -> 250); the hi and lo terms of the queries, and of the weights, are the 16 rows of a tile.
+template <int HD> struct ScCfg {
+    static constexpr int NV = 8, WARPS = 8;                  // query vectors; warps, each with 16 keys of a page
     static constexpr int OP = HD + 4;                        // padded row
     static constexpr int QP = HD * 2 + 16;                   // bytes per staged query row
-    static constexpr int QROWS = STACK ? 16 : 32;
     static constexpr int V4 = HD / 4;
     static constexpr int KST = HD / 64;                      // ring stages of a page's K; as many of its V^T
     static constexpr int SLOTS = WARPS * NV * OP * 4;        // the warps' results and the queries lie where the activations go
-    static_assert(SLOTS + QROWS * QP <= SC_ACT_SLOTS * SC_ACT_SLOT, "attention's buffers take the activations' place");
+    static_assert(SLOTS + 2 * NV * QP <= SC_ACT_SLOTS * SC_ACT_SLOT, "attention's buffers take the activations' place");
 };
 
 // kps: k-blocks of a stage; pack: how many of them one product takes side by side (see the kernel), 1 or kps
@@ -100,7 +100,7 @@ struct ScArgs {
     const int* page_table;
     int pages_per_seq, total_pages;
     bf16 *kpool, *vpool;
-    int C, split, items;                 // attention: CTAs per item, items that share a kv head, items
+    int C, split, items;                 // attention: CTAs per item, items (query heads) that share a kv head, items
     float* out; float* amax_val; int* amax_idx;
     int* err;
 };
@@ -140,12 +140,11 @@ __device__ __forceinline__ void fence_async_cta() { asm volatile("fence.proxy.as
 // Units of tile t of a cluster's Uc.  Each rank finishes a quarter of every tile's units, the quarters taking turns.
 __host__ __device__ inline int sc_tile_units(int Uc, int tiles, int t) { return Uc / tiles + (t < Uc % tiles ? 1 : 0); }
 
-template <int HD, int G>
+template <int HD>
 __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v, const __grid_constant__ ScArgs g) {
-    typedef ScCfg<HD, G> Cfg;
-    constexpr bool STACK = Cfg::STACK;
+    typedef ScCfg<HD> Cfg;
     constexpr int NV = Cfg::NV, WARPS = Cfg::WARPS, OP = Cfg::OP, QP = Cfg::QP, V4 = Cfg::V4, KST = Cfg::KST;
-    constexpr int KS = HD / 16, DT = HD / 8, NR = STACK ? 1 : 2;      // NR: query vectors per thread
+    constexpr int KS = HD / 16, DT = HD / 8;
     constexpr int CC = CL_CTAS, rows = ANPD_ROWS;
     extern __shared__ __align__(1024) unsigned char sc_smem[];
     __shared__ uint64_t w_full[SC_MAX_STAGES], w_empty[SC_MAX_STAGES], a_full[SC_ACT_SLOTS], a_empty[SC_ACT_SLOTS];
@@ -539,10 +538,10 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
             const bool own_new = my_pages > 0 && arank + (my_pages - 1) * g.C >= first_new;
             uint4 vnew;
             const int which = ft / HD, nr = (ft % HD) / (HD / 8), nc = (ft % HD) % (HD / 8);      // K or V, row, 16-byte chunk
-            const bool has_q = ft < Cfg::QROWS * (HD / 8), has_n = own_new && ft < 2 * HD;
+            const bool has_q = ft < 2 * NV * (HD / 8), has_n = own_new && ft < 2 * HD;
             {
                 const int qrow = ft / (HD / 8), c = ft % (HD / 8), vec = qrow & (NV - 1), term = qrow >= NV ? 1 : 0;
-                const unsigned char* qp = qsrc + (((size_t)(hv * G + vec % G) * 2 + term) * rows + vec / G) * (HD * 2) + c * 16;
+                const unsigned char* qp = qsrc + (((size_t)hv * 2 + term) * rows + vec) * (HD * 2) + c * 16;
                 const unsigned char* np = kvsrc + (((size_t)kvh * 2 + which) * rows + nr) * (HD * 2) + nc * 16;
                 uint4 vq = make_uint4(0u, 0u, 0u, 0u), vn = vq;
                 bool tq = has_q, tn = has_n;
@@ -556,14 +555,7 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
                 if (has_q) *(uint4*)(Qs + qrow * QP + c * 16) = vq;
             vnew = vn;
             }
-            int qpos[NR], qhl[NR], qhh[NR];
-#pragma unroll
-            for (int h = 0; h < NR; ++h) {
-                const int r = (gid + 8 * h) / G;
-                qpos[h] = g.tree ? s_raw[r] : pos_lo + r;
-                qhl[h] = g.tree ? g.hole_lo[r] : 0;
-                qhh[h] = g.tree ? g.hole_hi[r] : 0;
-            }
+            const int qpos = g.tree ? s_raw[gid] : pos_lo + gid, qhl = g.tree ? g.hole_lo[gid] : 0, qhh = g.tree ? g.hole_hi[gid] : 0;       // of this thread's row
             work_bar();
             // lane offsets of the ldmatrix addresses: matrix (lane / 8) of four
             const int mi = lane >> 3, lr = lane & 7;
@@ -572,9 +564,7 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
             const uint32_t ring_addr = smem_u32(ring);
             const int key_page = fw * 16;
 
-            float m_run[NR], l_run[NR], o[DT][4];
-#pragma unroll
-            for (int h = 0; h < NR; ++h) { m_run[h] = -CUDART_INF_F; l_run[h] = 0.0f; }
+            float m_run = -CUDART_INF_F, l_run = 0.0f, o[DT][4];
 #pragma unroll
             for (int d = 0; d < DT; ++d) { o[d][0] = 0.f; o[d][1] = 0.f; o[d][2] = 0.f; o[d][3] = 0.f; }
 #pragma unroll 1
@@ -608,7 +598,7 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
                 const int vst = st(vs);
                 const uint32_t vpar = par(vs);
                 if (p * KV_PAGE + key_page <= pos_hi) {
-                    // two chains of products, added at the end: even and odd steps, or hi and lo terms
+                    // two chains of products, added at the end: even and odd steps
                     float c[2][4], c2[2][4];
 #pragma unroll
                     for (int j = 0; j < 2; ++j)
@@ -620,13 +610,8 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
                         const uint32_t kr = ring_addr + (uint32_t)st(k >> 2) * SC_STAGE + kv_off + (uint32_t)key_page * 128u;
                         ad_ldm4(kr + ((((uint32_t)((k & 3) * 2) + chunk0) ^ (uint32_t)lr) << 4), b);
                         ad_ldm4(q_addr + (uint32_t)(k * 32), a);
-                        ad_mma(STACK && (k & 1) ? c2[0] : c[0], a, b[0], b[1]);
-                        ad_mma(STACK && (k & 1) ? c2[1] : c[1], a, b[2], b[3]);
-                        if (!STACK) {
-                            ad_ldm4(q_addr + (uint32_t)(16 * QP + k * 32), a);
-                            ad_mma(c2[0], a, b[0], b[1]);
-                            ad_mma(c2[1], a, b[2], b[3]);
-                        }
+                        ad_mma(k & 1 ? c2[0] : c[0], a, b[0], b[1]);
+                        ad_mma(k & 1 ? c2[1] : c[1], a, b[2], b[3]);
                     }
 #pragma unroll
                     for (int j = 0; j < 2; ++j)
@@ -637,44 +622,33 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
 #pragma unroll
                         for (int s = 0; s < KST; ++s) mbar_arrive(&w_empty[st(s)]);
                     }
-                    uint32_t ph[4], pl[4];
-                    float resc[NR];
+                    float w[2][2], mx = -CUDART_INF_F;
 #pragma unroll
-                    for (int h = 0; h < NR; ++h) {
-                        float w[2][2], mx = -CUDART_INF_F;
+                    for (int j = 0; j < 2; ++j)
 #pragma unroll
-                        for (int j = 0; j < 2; ++j)
-#pragma unroll
-                            for (int e = 0; e < 2; ++e) {
-                                const int key = p * KV_PAGE + key_page + 8 * j + 2 * t + e;
-                                const float s = STACK ? c[j][e] + c[j][2 + e] : c[j][2 * h + e];
-                                w[j][e] = (key <= qpos[h] && !(key >= qhl[h] && key < qhh[h])) ? s : -CUDART_INF_F;
-                                mx = fmaxf(mx, w[j][e]);
-                            }
-                        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-                        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-                        const float m_new = fmaxf(m_run[h], mx);
-                        const bool none = m_new == -CUDART_INF_F;
-                        resc[h] = none ? 1.0f : exp2f(m_run[h] - m_new);
-                        float sum = 0.0f;
-#pragma unroll
-                        for (int j = 0; j < 2; ++j)
-#pragma unroll
-                            for (int e = 0; e < 2; ++e) { w[j][e] = none ? 0.0f : exp2f(w[j][e] - m_new); sum += w[j][e]; }
-                        l_run[h] = l_run[h] * resc[h] + sum;        // this lane's keys; the four lanes of a row are added at the end
-                        m_run[h] = m_new;
-#pragma unroll
-                        for (int j = 0; j < 2; ++j) {
-                            uint32_t lo;
-                            const uint32_t hi = ad_split(w[j][0], w[j][1], lo);
-                            if (STACK) { ph[2 * j] = hi; ph[2 * j + 1] = lo; }       // rows gid: hi terms, rows gid + 8: lo terms
-                            else { ph[2 * j + h] = hi; pl[2 * j + h] = lo; }
+                        for (int e = 0; e < 2; ++e) {
+                            const int key = p * KV_PAGE + key_page + 8 * j + 2 * t + e;
+                            w[j][e] = (key <= qpos && !(key >= qhl && key < qhh)) ? c[j][e] + c[j][2 + e] : -CUDART_INF_F;
+                            mx = fmaxf(mx, w[j][e]);
                         }
-                    }
-                    const float ra = resc[0], rb = resc[NR - 1];
-                    if (__any_sync(0xffffffffu, ra != 1.0f || rb != 1.0f)) {        // multiplying by 1 changes nothing
+                    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+                    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+                    const float m_new = fmaxf(m_run, mx);
+                    const bool none = m_new == -CUDART_INF_F;
+                    const float resc = none ? 1.0f : exp2f(m_run - m_new);
+                    float wsum = 0.0f;
 #pragma unroll
-                        for (int d = 0; d < DT; ++d) { o[d][0] *= ra; o[d][1] *= ra; o[d][2] *= rb; o[d][3] *= rb; }
+                    for (int j = 0; j < 2; ++j)
+#pragma unroll
+                        for (int e = 0; e < 2; ++e) { w[j][e] = none ? 0.0f : exp2f(w[j][e] - m_new); wsum += w[j][e]; }
+                    l_run = l_run * resc + wsum;                    // this lane's keys; the four lanes of a row are added at the end
+                    m_run = m_new;
+                    uint32_t ph[4];                                 // rows gid: hi terms, rows gid + 8: lo terms
+#pragma unroll
+                    for (int j = 0; j < 2; ++j) ph[2 * j] = ad_split(w[j][0], w[j][1], ph[2 * j + 1]);
+                    if (__any_sync(0xffffffffu, resc != 1.0f)) {    // multiplying by 1 changes nothing
+#pragma unroll
+                        for (int d = 0; d < DT; ++d) { o[d][0] *= resc; o[d][1] *= resc; o[d][2] *= resc; o[d][3] *= resc; }
                     }
                     mbar_wait<1>(&w_full[vst], vpar, abortp);
                     const uint32_t vr = ring_addr + (uint32_t)vst * SC_STAGE + kv_off + (HD == 128 ? 0u : (uint32_t)((key_page >> 6) * (HD * 128))) + ((((uint32_t)((key_page & 63) >> 3) + chunk0) ^ (uint32_t)lr) << 4);
@@ -684,7 +658,6 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
                         ad_ldm4(vr + (uint32_t)(d * 16 * 128), b);
                         ad_mma(o[2 * d], ph, b[0], b[1]);
                         ad_mma(o[2 * d + 1], ph, b[2], b[3]);
-                        if (!STACK) { ad_mma(o[2 * d], pl, b[0], b[1]); ad_mma(o[2 * d + 1], pl, b[2], b[3]); }
                     }
                 } else {
                     if (lane == 0) {
@@ -700,31 +673,22 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
                 }
             }
             // ---- the warps, in order ----
-#pragma unroll
-            for (int h = 0; h < NR; ++h) {
-                l_run[h] += __shfl_xor_sync(0xffffffffu, l_run[h], 1);
-                l_run[h] += __shfl_xor_sync(0xffffffffu, l_run[h], 2);
-                if (t == 0) { sm_m[fw * NV + gid + 8 * h] = m_run[h]; sm_l[fw * NV + gid + 8 * h] = l_run[h]; }
-            }
+            l_run += __shfl_xor_sync(0xffffffffu, l_run, 1);
+            l_run += __shfl_xor_sync(0xffffffffu, l_run, 2);
+            if (t == 0) { sm_m[fw * NV + gid] = m_run; sm_l[fw * NV + gid] = l_run; }
             float* mine = sm_o + (size_t)fw * NV * OP;
 #pragma unroll
-            for (int d = 0; d < DT; ++d) {
-                if (STACK) *(float2*)(mine + gid * OP + 8 * d + 2 * t) = make_float2(o[d][0] + o[d][2], o[d][1] + o[d][3]);
-                else {
-                    *(float2*)(mine + gid * OP + 8 * d + 2 * t) = make_float2(o[d][0], o[d][1]);
-                    *(float2*)(mine + (gid + 8) * OP + 8 * d + 2 * t) = make_float2(o[d][2], o[d][3]);
-                }
-            }
+            for (int d = 0; d < DT; ++d) *(float2*)(mine + gid * OP + 8 * d + 2 * t) = make_float2(o[d][0] + o[d][2], o[d][1] + o[d][3]);
             work_bar();
             // the result, as hi + lo terms in the O projection's operand image
             unsigned char* img = copy + g.o_ao;
             auto store = [&](int vec, int d4, float l_, float4 a) {
-                const int r = vec / G, k = (hv * G + vec % G) * HD + 4 * d4;
+                const int k = hv * HD + 4 * d4;
                 uint2 hi, lo;
                 hi.x = ad_split(a.x / l_, a.y / l_, lo.x);
                 hi.y = ad_split(a.z / l_, a.w / l_, lo.y);
-                st_relaxed2(img + cl_img_offset(rows, r, k), hi);
-                st_relaxed2(img + cl_img_offset(rows, rows + r, k), lo);
+                st_relaxed2(img + cl_img_offset(rows, vec, k), hi);
+                st_relaxed2(img + cl_img_offset(rows, rows + vec, k), lo);
             };
             for (int idx = ft; idx < NV * V4; idx += SC_WORKERS) {
                 const int vec = idx / V4, d4 = idx % V4;
@@ -993,7 +957,7 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
     cluster_wait();
 }
 
-template <int HD, int G>
+template <int HD>
 anpd_status launch_step_cl(const anpd_kv* kv, const ScArgs& g, int smem, cudaStream_t st, Profiler* prof) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(g.ncl * CL_CTAS); cfg.blockDim = dim3(SC_THREADS); cfg.dynamicSmemBytes = smem; cfg.stream = st;
@@ -1006,15 +970,15 @@ anpd_status launch_step_cl(const anpd_kv* kv, const ScArgs& g, int smem, cudaStr
     attr[2].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = (g_use_pdl && !t_no_pdl) ? 3 : 2;
-    LAUNCH(prof, st, KC_GEMM, kv->m->streamed_bytes, (cudaLaunchKernelEx(&cfg, step_cl_kernel<HD, G>, kv->map_k, kv->map_v, g)));
+    LAUNCH(prof, st, KC_GEMM, kv->m->streamed_bytes, (cudaLaunchKernelEx(&cfg, step_cl_kernel<HD>, kv->map_k, kv->map_v, g)));
     CUDA_TRY(cudaGetLastError());
     return ANPD_OK;
 }
 
 // The kernel's function attributes on the current device, and whether the device holds all of its CTAs at once.
-template <int HD, int G>
+template <int HD>
 bool fits_step_cl(int ncl, int smem) {
-    if (cudaFuncSetAttribute(step_cl_kernel<HD, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) { cudaGetLastError(); return false; }
+    if (cudaFuncSetAttribute(step_cl_kernel<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) { cudaGetLastError(); return false; }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(ncl * CL_CTAS); cfg.blockDim = dim3(SC_THREADS); cfg.dynamicSmemBytes = smem;
     cudaLaunchAttribute attr[1];
@@ -1022,7 +986,7 @@ bool fits_step_cl(int ncl, int smem) {
     attr[0].val.clusterDim.x = CL_CTAS; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr; cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, step_cl_kernel<HD, G>, &cfg) != cudaSuccess) { cudaGetLastError(); return false; }
+    if (cudaOccupancyMaxActiveClusters(&n, step_cl_kernel<HD>, &cfg) != cudaSuccess) { cudaGetLastError(); return false; }
     return n >= ncl;
 }
 
@@ -1091,8 +1055,8 @@ bool sc_args(const anpd_model* m, ScArgs* g, int* smem) {
         if (v.wqkv != w.wqkv + at || v.wo != w.wo + at || v.wgu != w.wgu + at || v.wd != w.wd + at || (const char*)v.attn_norm != (const char*)w.attn_norm + at ||
             (const char*)v.ffn_norm != (const char*)w.ffn_norm + at) return false;
     }
-    g->split = ad_split(c);
-    g->items = c.n_kv_heads * g->split;
+    g->split = c.n_q_heads / c.n_kv_heads;
+    g->items = c.n_q_heads;
     g->C = ad_cluster(m, g->items);
     if (g->items * g->C > ncta) return false;
     // exchange buffers
@@ -1108,7 +1072,6 @@ bool sc_args(const anpd_model* m, ScArgs* g, int* smem) {
     return true;
 }
 
-int sc_form(const anpd_model_config& c) { return c.head_dim == 128 ? 2 : c.n_q_heads == c.n_kv_heads ? 0 : 1; }
 
 }  // namespace
 
@@ -1116,7 +1079,7 @@ size_t step_cl_bytes(const anpd_model* m, int batch) {
     ScArgs g;
     int smem = 0;
     if (batch != 1 || !m->cl_all_fused || m->plain_gemm || std::getenv("ANPD_STEP_CHAIN") || !sc_args(m, &g, &smem)) return 0;
-    const bool ok = sc_form(m->cfg) == 2 ? fits_step_cl<128, 1>(g.ncl, smem) : sc_form(m->cfg) == 1 ? fits_step_cl<64, 2>(g.ncl, smem) : fits_step_cl<64, 1>(g.ncl, smem);
+    const bool ok = m->cfg.head_dim == 128 ? fits_step_cl<128>(g.ncl, smem) : fits_step_cl<64>(g.ncl, smem);
     return ok ? 2 * (size_t)g.copy_bytes + g.fin_bytes + 4 * (4 * (size_t)g.L + 1) : 0;
 }
 
@@ -1138,9 +1101,5 @@ anpd_status step_cl_enqueue(anpd_model* m, anpd_kv* kv, bool want_logits, bool t
     ws.amax_nblk = g.ncl * CL_CTAS;
     ws.amax_val_use = ws.amax_val_cl;
     ws.amax_idx_use = ws.amax_idx_cl;
-    switch (sc_form(m->cfg)) {
-        case 0: return launch_step_cl<64, 1>(kv, g, smem, m->stream, &m->prof);
-        case 1: return launch_step_cl<64, 2>(kv, g, smem, m->stream, &m->prof);
-        default: return launch_step_cl<128, 1>(kv, g, smem, m->stream, &m->prof);
-    }
+    return m->cfg.head_dim == 128 ? launch_step_cl<128>(kv, g, smem, m->stream, &m->prof) : launch_step_cl<64>(kv, g, smem, m->stream, &m->prof);
 }
