@@ -384,10 +384,11 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
         const unsigned slice = g.copy_bytes / (unsigned)ncta, fslice = g.fin_bytes / (unsigned)ncta;
 #pragma unroll 1
         for (int l = 0; l <= g.L; ++l) {
-            asm volatile("bar.sync 3, 288;" ::: "memory");             // this CTA is through the O projection of layer l (the vocabulary)
+            asm volatile("bar.sync 3, 288;" ::: "memory");             // this CTA is through the O projection of layer l (or has heard from every CTA's last layer)
             unsigned char* at = l ? g.xch + (size_t)((l - 1) & 1) * g.copy_bytes + (size_t)bid * slice : g.xch + 2 * (size_t)g.copy_bytes + (size_t)bid * fslice;
             const unsigned n = l ? slice : fslice;
             for (unsigned i = lane * 16u; i < n; i += 512u) *(uint4*)(at + i) = make_uint4(SC_EMPTY, SC_EMPTY, SC_EMPTY, SC_EMPTY);
+            if (l == g.L) break;                                       // (the kernel's end makes these visible)
             __threadfence();
             __syncwarp();
             if (lane == 0) mbar_arrive(&jan_done);
@@ -456,7 +457,6 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
             s_slot[ft] = g.row_ok[ft] ? slot : -1;
             s_page[ft] = g.page_table[(size_t)g.row_seq[ft] * g.pages_per_seq + slot / KV_PAGE];
         }
-        pdl_wait();                                     // what the embedding left
         // A CTA's results in the order of its units over all tiles, 32 pairs each: item idx is thread idx % 256's.  The unit of an item
         // of tile t, and the features of the residual stream:
         auto unit_of = [&](int kd, int t, int idx) { return s_tile[kd][t].own_first + (idx >> 5) - s_tile[kd][t].before[rank]; };
@@ -466,7 +466,6 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
             return t;
         };
         auto resid_feature = [&](int idx) { return unit_of(GK_O, tile_of(GK_O, idx), idx) * 8 + 2 * ((idx >> 3) & 3); };
-        for (int idx = ft; idx < s_own[GK_O] * 32; idx += SC_WORKERS) s_x[idx] = *(const float2*)(g.x0 + (size_t)row * g.d + resid_feature(idx));
         float2 cs0 = make_float2(0.f, 0.f), sn0 = cs0;         // the rotation of this thread's first item of QKV, the same in every layer
         if (ft < s_own[GK_QKV] * 32) {
             const int u = unit_of(GK_QKV, tile_of(GK_QKV, ft), ft);
@@ -476,6 +475,8 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
         }
         work_bar();
         cluster_wait();
+        pdl_wait();                                     // what the embedding left
+        for (int idx = ft; idx < s_own[GK_O] * 32; idx += SC_WORKERS) s_x[idx] = *(const float2*)(g.x0 + (size_t)row * g.d + resid_feature(idx));
 
         int a_slot = 0, a_count = 0, p_st = 0;
         uint32_t a_ph = 1, p_par = 0, acc_par = 0, red_par = 0, att_par = 0;       // acc_par: a bit per tile; red_par: per region and tile
@@ -774,6 +775,7 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
                 if (lane == 0) s_rstd[fw] = rsqrtf(s * g.inv_d + g.eps);
             }
             if (!resid) work_bar();                      // the rows' 1 / RMS
+            if (kd == GK_LM) asm volatile("bar.arrive 3, 288;" ::: "memory");        // (whose parts come from every CTA's last result)
             // the buffers of the layer before are empty again before anything that the next layer waits for leaves this CTA
             if (kd == GK_DOWN) mbar_wait<1>(&jan_done, (uint32_t)l & 1u, abortp);
             const float* red = (const float*)(redbuf + g.k[kd].red);
@@ -930,7 +932,6 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
                     g.amax_val[(size_t)ft * ncta + bid] = best;
                     g.amax_idx[(size_t)ft * ncta + bid] = bidx;
                 }
-                asm volatile("bar.arrive 3, 288;" ::: "memory");
                 break;
             }
             if (kd == GK_DOWN) { ++l; kd = l == g.L ? GK_LM : GK_QKV; } else ++kd;
