@@ -34,6 +34,9 @@
 // The keys and values of the step itself reach the attention the same way; the pages are copied in before they can hold them (any time:
 // they are as old as the step before), and the rows are put into the copy.
 //
+// Code.  A worker runs through some 60 KB of code per layer, so loops stay rolled unless they index registers (1.1B 520 -> 517 us per step);
+// results' places worked out once and kept (3 KB of code more) or before the parts arrive lost 0.7 and 3 %.
+//
 // Values are those of gemm_cl.cu and attn_dec.cu: the same cut of K, the same order of parts, pages, warps and CTAs, and so equal bit for bit -
 // but where products are packed (their k-blocks' sums meet at the end), beyond 4096 features (two tiles of the residual stream: a row's sum of
 // squares comes in other groups),
@@ -181,6 +184,7 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
         e.step = GS << 10;
         e.w_off = ((unsigned long long)ulo * k.gpu * (k.seg == 1 ? 1 : k.kb) + (unsigned long long)GS * e.kb_lo) * 1024;
         int before[CC] = {0, 0, 0, 0};
+#pragma unroll 1
         for (int t = 0, u0 = 0; t < k.tiles; ++t) {
             ScTile& w = s_tile[threadIdx.x][t];
             const int un = sc_tile_units(Uc, k.tiles, t);
@@ -198,6 +202,7 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
     }
     if (threadIdx.x == 64) {
         abort_flag = 0; s_issued = 0; s_requested = 0; s_phase = 0; s_quit = 0;
+#pragma unroll 1
         for (int s = 0; s < g.stages; ++s) { mbar_init(&w_full[s], 1); mbar_init(&w_empty[s], WARPS); }
         for (int s = 0; s < SC_ACT_SLOTS; ++s) { mbar_init(&a_full[s], 8); mbar_init(&a_empty[s], 1); }
         for (int t = 0; t < SC_MAX_TILES; ++t) { mbar_init(&acc_full[t], 1); mbar_init(&red_full[0][t], 1); mbar_init(&red_full[1][t], 1); }
@@ -387,6 +392,7 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
             asm volatile("bar.sync 3, 288;" ::: "memory");             // this CTA is through the O projection of layer l (or has heard from every CTA's last layer)
             unsigned char* at = l ? g.xch + (size_t)((l - 1) & 1) * g.copy_bytes + (size_t)bid * slice : g.xch + 2 * (size_t)g.copy_bytes + (size_t)bid * fslice;
             const unsigned n = l ? slice : fslice;
+#pragma unroll 1
             for (unsigned i = lane * 16u; i < n; i += 512u) *(uint4*)(at + i) = make_uint4(SC_EMPTY, SC_EMPTY, SC_EMPTY, SC_EMPTY);
             if (l == g.L) break;                                       // (the kernel's end makes these visible)
             __threadfence();
@@ -407,6 +413,7 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
             auto prefetch = [](const void* src, uint32_t bytes) { asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory"); };
             auto turn = [&]() {                         // waits until copy idx is near enough; false: it has been requested
                 if (idx < s_requested) return false;
+#pragma unroll 1
                 while (true) {
                     const int pr = s_requested, ph = s_phase;
                     if (idx < pr || s_quit) return false;
@@ -462,6 +469,7 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
         auto unit_of = [&](int kd, int t, int idx) { return s_tile[kd][t].own_first + (idx >> 5) - s_tile[kd][t].before[rank]; };
         auto tile_of = [&](int kd, int idx) {
             int t = 0;
+#pragma unroll 1
             while (t + 1 < s_geo[kd].T && (idx >> 5) >= s_tile[kd][t + 1].before[rank]) ++t;
             return t;
         };
@@ -476,6 +484,7 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
         work_bar();
         cluster_wait();
         pdl_wait();                                     // what the embedding left
+#pragma unroll 1
         for (int idx = ft; idx < s_own[GK_O] * 32; idx += SC_WORKERS) s_x[idx] = *(const float2*)(g.x0 + (size_t)row * g.d + resid_feature(idx));
 
         int a_slot = 0, a_count = 0, p_st = 0;
@@ -512,6 +521,7 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
                     // columns behind the last input meet zero weights: nobody writes them, they are zero here
                     if (c < chunks && (kb_lo + k0 + (c >> 7)) * 64 + (((c & 7) ^ ((c >> 3) & 7)) << 3) < K) todo |= 1u << j;
                 }
+#pragma unroll 1
                 for (unsigned i = 0; todo; ++i) {
 #pragma unroll
                     for (int j = 0; j < 4; ++j) if (todo >> j & 1u) v[j] = ld_relaxed4(src + j * (SC_WORKERS * 16));
@@ -546,6 +556,7 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
                 const unsigned char* np = kvsrc + (((size_t)kvh * 2 + which) * rows + nr) * (HD * 2) + nc * 16;
                 uint4 vq = make_uint4(0u, 0u, 0u, 0u), vn = vq;
                 bool tq = has_q, tn = has_n;
+#pragma unroll 1
                 for (unsigned i = 0; tq || tn; ++i) {
                     if (tq) vq = ld_relaxed4(qp);
                     if (tn) vn = ld_relaxed4(np);
@@ -691,6 +702,7 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
                 st_relaxed2(img + cl_img_offset(rows, vec, k), hi);
                 st_relaxed2(img + cl_img_offset(rows, rows + vec, k), lo);
             };
+#pragma unroll 1
             for (int idx = ft; idx < NV * V4; idx += SC_WORKERS) {
                 const int vec = idx / V4, d4 = idx % V4;
                 float mx = -CUDART_INF_F;
@@ -715,6 +727,7 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
                 mbar_wait_cluster(&att_full, att_par, abortp);
                 att_par ^= 1u;
                 if (ft == 0 && l + 1 < g.L) mbar_expect_tx(&att_full, (uint32_t)(g.C * VO * (HD * 4 + 8)));
+#pragma unroll 1
                 for (int idx = ft; idx < VO * V4; idx += SC_WORKERS) {
                     const int vo = idx / V4, d4 = idx % V4;
                     float m = -CUDART_INF_F, lsum = 0.0f;
@@ -761,6 +774,7 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
 #pragma unroll
                     for (int j = 0; j < 4; ++j) if (lane + 32 * j < ncta) todo |= 1u << j;
                     const uint32_t mine = todo;
+#pragma unroll 1
                     for (unsigned i = 0; todo; ++i) {
 #pragma unroll
                         for (int j = 0; j < 4; ++j) if (todo >> j & 1u) v[j] = ld_relaxed1(src + j * 128);
@@ -771,6 +785,7 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
 #pragma unroll
                     for (int j = 0; j < 4; ++j) if (mine >> j & 1u) s += __uint_as_float(v[j]);
                 }
+#pragma unroll 1
                 for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
                 if (lane == 0) s_rstd[fw] = rsqrtf(s * g.inv_d + g.eps);
             }
@@ -918,6 +933,7 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
                 }
                 if (kd == GK_O) asm volatile("bar.arrive 3, 288;" ::: "memory");
             } else if (kd == GK_LM) {
+#pragma unroll 1
                 for (int o = 8; o <= 16; o <<= 1) {
                     const float ov = __shfl_xor_sync(0xffffffffu, best, o);
                     const int oi = __shfl_xor_sync(0xffffffffu, bidx, o);
@@ -949,7 +965,9 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
     }
     if (threadIdx.x == 0 && abort_flag) {
         // gave up: let every copy already issued land before the CTA may exit
+#pragma unroll 1
         for (int i = max(0, s_issued - g.stages); i < s_issued; ++i)
+#pragma unroll 1
             for (unsigned spin = 0; spin < WAIT_LIMIT && !mbar_try_wait(&w_full[i % g.stages], (uint32_t)((i / g.stages) & 1)); ++spin) {}
         atomicExch(g.err, SC_ERR_TIMEOUT);
     }
@@ -998,6 +1016,7 @@ bool sc_args(const anpd_model* m, ScArgs* g, int* smem) {
     g->ncl = m->cl[GK_QKV].ncl;
     const int ncta = g->ncl * CL_CTAS;
     int tiles_max = 1, red[2] = {0, 0};
+#pragma unroll 1
     for (int k = 0; k < GK_COUNT; ++k) {
         const ClPlan& p = m->cl[k];
         ScKind& s = g->k[k];
@@ -1011,9 +1030,12 @@ bool sc_args(const anpd_model* m, ScArgs* g, int* smem) {
         if (tiles > 1 && p.n_units / g->ncl < tiles * CL_CTAS) return false;              // every CTA finishes units of every tile
         // the most units a CTA finishes, of the smaller and of the larger clusters
         int own_max = 0;
+#pragma unroll 1
         for (int Uc = p.n_units / g->ncl; Uc <= p.u_max; ++Uc)
+#pragma unroll 1
             for (int r = 0; r < CL_CTAS; ++r) {
                 int own = 0;
+#pragma unroll 1
                 for (int t = 0; t < tiles; ++t) { const int un = sc_tile_units(Uc, tiles, t), q = (r + t) % CL_CTAS; own += (q + 1) * un / CL_CTAS - q * un / CL_CTAS; }
                 own_max = std::max(own_max, own);
             }
@@ -1025,9 +1047,11 @@ bool sc_args(const anpd_model* m, ScArgs* g, int* smem) {
         red[s.red] = std::max(red[s.red], CL_CTAS * s.pack * s.f_own_max * 32);
         tiles_max = std::max(tiles_max, tiles * s.pack);
     }
+#pragma unroll 1
     for (int k = 0; k < GK_COUNT; ++k) g->k[k].red = g->k[k].red ? red[0] : 0;
     g->red_bytes = red[0] + red[1];
     g->tmem_cols = 32;
+#pragma unroll 1
     while (g->tmem_cols < tiles_max * 2 * ANPD_ROWS) g->tmem_cols <<= 1;
     const int rest = SC_ACT_SLOTS * SC_ACT_SLOT + g->red_bytes + g->k[GK_O].f_own_max / 8 * 32 * (int)sizeof(float2) + 1024;
     g->stages = std::min(SC_MAX_STAGES, (SC_SMEM - rest) / SC_STAGE);
@@ -1038,6 +1062,7 @@ bool sc_args(const anpd_model* m, ScArgs* g, int* smem) {
     // 903, 888, 870, 861, 865; 7B at 3000 keys 1287, -, 1290, 1320 (there the pages take what the prefetch takes).  A layer of less than 28 copies, three to four rings full, is better off without: 1280 wide (25) 227 -> 230, 1024 wide
     // (16) 263 -> 273, but 1536 wide (29) 262 -> 258.
     int copies = 0;
+#pragma unroll 1
     for (int k = 0; k < GK_LM; ++k) {
         const int nk = (g->k[k].kb + CL_CTAS - 1) / CL_CTAS;
         copies += g->k[k].tiles == 1 ? (nk + g->k[k].kps - 1) / g->k[k].kps : nk * g->k[k].tiles;
@@ -1050,6 +1075,7 @@ bool sc_args(const anpd_model* m, ScArgs* g, int* smem) {
     g->w[GK_QKV] = w.wqkv; g->w[GK_O] = w.wo; g->w[GK_GU] = w.wgu; g->w[GK_DOWN] = w.wd; g->w[GK_LM] = m->lm_head;
     g->attn_norm = w.attn_norm; g->ffn_norm = w.ffn_norm; g->final_norm = m->final_norm;
     if (c.n_layers > 1) g->layer_step = (size_t)(m->layers[1].wqkv - w.wqkv);
+#pragma unroll 1
     for (int l = 1; l < c.n_layers; ++l) {
         const LayerW& v = m->layers[l];
         const size_t at = (size_t)l * g->layer_step;
