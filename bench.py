@@ -753,7 +753,8 @@ def main() -> None:
     A.anpd_profile_enable(model, False)
     peak, peak_kind = measured_hbm_peak()
     gemm_gbs = prof["gemm_bytes"] / (prof["ms_gemm"] * 1e-3) / 1e9 if prof["ms_gemm"] > 0 else 0.0
-    roofline = {"bound": "hbm", "kernel": "weight-streaming GEMM (all projections + LM head)",
+    # (profiling launches a kernel per projection; otherwise a single sequence's step is one kernel: "verify_step" below)
+    roofline = {"bound": "hbm", "kernel": "weight-streaming GEMM (all projections + LM head), a launch each; verify_step has the step as one kernel",
                 "achieved": gemm_gbs, "peak": peak, "peak_kind": f"of {peak_kind}", "unit": "GB/s",
                 "frac": gemm_gbs / peak, "traffic": gemm_traffic_per_launch(wl),
                 "launches": prof["n_gemm"], "avg_launch_us": prof["ms_gemm"] * 1e3 / max(prof["n_gemm"], 1),

@@ -88,3 +88,24 @@ def test_sums_in_another_order(A, monkeypatch, shape):
     for a, b in zip(*_both(A, monkeypatch, shape, run)):
         # fp32 sums of two-term products (2^-17 of a term) in another order, through one layer whose cached keys and values are the same
         assert float(np.abs(a - b).max()) <= 2.0 ** -12 * max(1.0, float(np.abs(a).max()))
+
+
+def test_a_kernel_per_projection_under_nsight_compute(A, monkeypatch):
+    """A profiler that runs launches again does not get a kernel whose CTAs wait for one another."""
+    shape = ModelShape(1, 256, 4, 4, 64, 256, 256)
+    m = gpu_model(A, shape, make_weights(shape, 21, True), new_stream())
+    launches = []
+    try:
+        for var in ("ANPD_STEP_CHAIN", "NV_COMPUTE_PROFILER_PERFWORKS_DIR"):
+            with monkeypatch.context() as env:
+                env.delenv("NV_COMPUTE_PROFILER_PERFWORKS_DIR", raising=False)
+                env.setenv(var, "1")
+                kv = A.anpd_kv_create(m, 64)
+            last = A.anpd_prefill(m, kv, [1, 2, 3])
+            A.anpd_launch_count(True)
+            A.anpd_verify(m, kv, last, DRAFT[:3])
+            launches.append(A.anpd_launch_count())
+            A.anpd_kv_destroy(kv)
+    finally:
+        A.anpd_model_destroy(m)
+    assert launches[0] == launches[1]
