@@ -29,7 +29,12 @@ namespace {
 using namespace tc;
 
 constexpr int PF_TILE_TOK = 256;
-constexpr int PF_THREADS = 320;          // warp 0: producer, warp 1: MMA issuer + tensor-memory owner, warps 2-9: epilogue, four per accumulator
+// Epilogue warps.  A finishing epilogue (below) is an exponential and a division per value and stands between two tiles' products, whose accumulators
+// take all of tensor memory: sixteen warps, four per scheduler, hide each other's latencies.  us per prompt with eight and with sixteen: 1.1B 300
+// tokens 2189 -> 2142, 512 3001 -> 2928, 1500 6493 -> 6256; 7B (8 layers) 1536 tokens 8140 -> 7950, 2000 10900 -> 10450; 1024 wide 600 tokens 1721 -> 1663.  Where sums are
+// only stored, sixteen win nothing at 256 rows and lose 1 to 2 % at 100 (more threads to start, the same stores).
+__host__ __device__ constexpr int pf_epi_warps(bool gu) { return gu ? 16 : 8; }
+__host__ __device__ constexpr int pf_threads(bool gu) { return 64 + 32 * pf_epi_warps(gu); }          // warp 0: producer, warp 1: MMA issuer + tensor-memory owner, the others: epilogue
 constexpr int PF_BLOCK = 16384;          // one 128 x 64 bf16 weight tile
 constexpr int PF_BOX = 8192;             // 64 rows x 64 bf16 of the activations
 constexpr int PF_SMEM = 224 * 1024;
@@ -67,7 +72,7 @@ __device__ __forceinline__ void pf_item(const PfArgs& g, int item, int& ot, int&
 // GU: the gate-up projection.  A tile in one part is finished here: eight lanes hold gate features, the next eight their up features, so
 // that a lane pair turns two rows' sums into one activation each.  That writes half of the sums' bytes, and nobody reads the sums again.
 template <bool GU>
-__global__ void __launch_bounds__(PF_THREADS, 1)
+__global__ void __launch_bounds__(pf_threads(GU), 1)
 gemm_pf_kernel(const unsigned char* __restrict__ w, const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ CUtensorMap map_lo,
                const __grid_constant__ PfArgs g) {
     extern __shared__ __align__(1024) unsigned char pf_smem_raw[];
@@ -85,7 +90,7 @@ gemm_pf_kernel(const unsigned char* __restrict__ w, const __grid_constant__ CUte
     if (threadIdx.x == 0) {
         abort_flag = 0;
         for (int s = 0; s < PF_MAX_STAGES; ++s) { mbar_init(&bar_full[s], 1); mbar_init(&bar_empty[s], 1); }
-        mbar_init(&bar_acc_full, 1); mbar_init(&bar_acc_empty, 8);
+        mbar_init(&bar_acc_full, 1); mbar_init(&bar_acc_empty, pf_epi_warps(GU));
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
@@ -197,7 +202,8 @@ gemm_pf_kernel(const unsigned char* __restrict__ w, const __grid_constant__ CUte
             }
         }
     } else {
-        const int quad = warp & 3, acc = (warp - 2) >> 2;
+        // an accumulator's 16 rows at a time are one warp's of each lane quarter, in turn
+        const int quad = warp & 3, acc = ((warp - 2) >> 2) & 1, first = (warp - 2) >> 3 << 4, step = 2 * pf_epi_warps(GU);
         int done_tiles = 0;
         bool ok = true;
         pdl_wait();                                        // the sums of the projection before have been read
@@ -215,7 +221,7 @@ gemm_pf_kernel(const unsigned char* __restrict__ w, const __grid_constant__ CUte
             if (GU && parts == 1) {
                 const int side = (lane >> 3) & 1, f = (pos >> 4) * 8 + (pos & 7);               // 0: this lane holds gate sums, 1: up sums
 #pragma unroll 1
-                for (int c0 = 0; c0 < n_rows; c0 += 16) {
+                for (int c0 = first; c0 < n_rows; c0 += step) {
                     float v[16];
                     tc_ld16(col + (uint32_t)c0, v);
                     const size_t at = (size_t)(row0 + c0) * g.plan.F + f;
@@ -234,7 +240,7 @@ gemm_pf_kernel(const unsigned char* __restrict__ w, const __grid_constant__ CUte
             } else {
                 const int n = pos < n_pos ? cl_feature(g.plan, pos) : g.plan.N;
 #pragma unroll 1
-                for (int c0 = 0; c0 < n_rows; c0 += 16) {
+                for (int c0 = first; c0 < n_rows; c0 += step) {
                     float v[16];
                     tc_ld16(col + (uint32_t)c0, v);
                     if (n < g.plan.N) {
@@ -330,9 +336,10 @@ anpd_status gemm_pf_enqueue(const ClPlan& plan, const unsigned char* w, const CU
     g.ksplit = sched.ksplit; g.tail_from = sched.tail_from; g.tail_split = sched.tail_split; g.seg_stride = seg_stride;
     g.act_hi = act_hi; g.act_lo = act_lo;
     g.err = err;
+    const bool gu = act_hi && sched.ksplit == 1;            // (with every tile cut along K there is nothing to finish)
     const int grid = std::min(num_sms, sched.tail_from * sched.ksplit + (g.n_ft * g.n_tt - sched.tail_from) * sched.tail_split);
     LAUNCH(prof, st, KC_GEMM, 2.0 * (double)plan.N * (double)plan.K,
-           (launch_k(act_hi ? gemm_pf_kernel<true> : gemm_pf_kernel<false>, grid, PF_THREADS, (size_t)smem, st, w, map_hi, map_lo, g)));
+           (launch_k(gu ? gemm_pf_kernel<true> : gemm_pf_kernel<false>, grid, pf_threads(gu), (size_t)smem, st, w, map_hi, map_lo, g)));
     CUDA_TRY(cudaGetLastError());
     return ANPD_OK;
 }

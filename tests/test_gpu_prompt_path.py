@@ -93,3 +93,28 @@ def test_prompt_logits_at_feature_tile_and_row_width_edges(A, d, F, plen):
     finally:
         A.anpd_kv_destroy(kv)
         A.anpd_model_destroy(m)
+
+
+# whole tiles of gate-up, finished by the projection: an odd number of 16-row chunks, a last tile's chunks that are partly or not there
+@pytest.mark.parametrize("plen", [129, 150, 182, 340, 393])
+def test_gate_up_tiles_finished_by_the_projection(A, plen):
+    shape = ModelShape(2, 256, 2, 2, 128, 9608, 300)               # (the second layer reads every row of the first)
+    w = make_weights(shape, 31, False, std=0.03)
+    m = gpu_model(A, shape, w, new_stream())
+    kv = A.anpd_kv_create(m, plen + 16)
+    prompt = markov_prompt(plen, shape.vocab, 2, 500 + plen).tolist()
+    draft = [int(t) for t in markov_prompt(7, shape.vocab, 2, 501 + plen)]
+    try:
+        first = A.anpd_prefill(m, kv, prompt)
+        got = torch.from_numpy(A.anpd_verify_logits(m, kv, first, draft, shape.vocab)).double()
+    finally:
+        A.anpd_kv_destroy(kv)
+        A.anpd_model_destroy(m)
+    dec = Decoder(shape, as_bf16_values(w), torch.float64, kv_dtype=torch.bfloat16)
+    cache = dec.new_cache()
+    lp = dec.forward(prompt, cache)
+    if top2_margin(lp[-1]) > 5e-2:
+        assert first == argmax_lowest(lp[-1])
+    want = dec.forward([first] + draft, cache)
+    err = float((got - want).abs().max())
+    assert err <= 2 ** -8 * max(1.0, float(want.abs().max())), err          # (the bound of the row tile edges above)
