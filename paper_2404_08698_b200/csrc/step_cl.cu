@@ -7,8 +7,8 @@
 // five hand-overs per layer.  As a kernel per projection a hand-over took about 3 us: the last CTA's exit and the boundary behind it, tensor
 // memory and barriers set up again, code from a cold instruction cache, a weight ring that starts empty or half an SM wide.  Here the ring runs
 // through: the weight thread walks all layers' weights, and the cache's pages between them, and never waits for an activation.  us per step:
-// 1.1B at 512 keys 729 -> 522, 1024 wide (16 layers) 380 -> 262, 7B (16 layers and the head) at 77 keys 1294 -> 1075, at 1536 1382 -> 1216, tiny
-// (2 x 256) 48 -> 42.
+// 1.1B at 512 keys 729 -> 516, 1024 wide (16 layers) 380 -> 259, 7B (16 layers and the head) at 77 keys 1294 -> 1047 to 1080, at 1536 1382 -> 1200 to
+// 1240, tiny (2 x 256) 48 -> 41.6.
 //
 // Hand-over.  The exchange buffers hold nothing but all-ones words until their values are written, and no value is one (a NaN that
 // arithmetic or a rounding to bf16 leaves has its top bit clear): the words are their own flags.  A reader polls the very data it needs, with
