@@ -994,10 +994,11 @@ anpd_status launch_step_cl(const anpd_kv* kv, const ScArgs& g, int smem, cudaStr
     return ANPD_OK;
 }
 
-// The kernel's function attributes on the current device, and whether the device holds all of its CTAs at once.
+// The kernel's function attributes on the current device, and whether the device holds all of its CTAs at once.  The limit of shared memory
+// is the function's, for the handles of all models: the bound of every shape's need, so that no handle takes it from another.
 template <int HD>
 bool fits_step_cl(int ncl, int smem) {
-    if (cudaFuncSetAttribute(step_cl_kernel<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) { cudaGetLastError(); return false; }
+    if (cudaFuncSetAttribute(step_cl_kernel<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, SC_SMEM) != cudaSuccess) { cudaGetLastError(); return false; }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(ncl * CL_CTAS); cfg.blockDim = dim3(SC_THREADS); cfg.dynamicSmemBytes = smem;
     cudaLaunchAttribute attr[1];
