@@ -15,8 +15,12 @@
 // relaxed loads from L2, and no fence stands between a store and its use.  Measured with 16 KB per CTA, a round of store, poll and copy takes
 // 1.2 us (1.5 to 2.0 beside a saturated weight stream); through flags with release and acquire it took 2.9, beside the stream 10.  After use
 // the words are set back, by a warp that does nothing else and fences: there are two copies, by the layer's parity, and the copy of
-// layer l - 1 is set back while layer l's gate-up runs (every CTA's O results are in by then, so everybody has read everything of l - 1),
-// and nothing that leads to layer l + 1 leaves this CTA before that is done (jan_done).
+// layer l - 1 is set back while layer l's gate-up runs.  Everybody has read all of it by then: this CTA's O results need its cluster's four
+// quarters of the attention, these every cluster's QKV results, and no CTA pushes sums of QKV before it has read what l - 1 left.  And no
+// sums of layer l's down projection leave this CTA before that is done (jan_done): every CTA's QKV of layer l + 1, the next to write there,
+// needs them.  What the last layer leaves is set back in layer 0 (its readers were the kernel before) and written by the last layer's down
+// projection, which needs layer 0's if there are several.  With one layer it is that same projection, and another cluster's needs this CTA's
+// gate-up sums but not its down sums: there it is the gate-up sums that wait.
 // So are the others protected: a CTA's pushes of phase p + 2 into the region of the exchange that phase p used need results of
 // phase p + 1 that need all results of phase p.  This needs every cluster to own features and every CTA k-blocks of every projection.
 //
@@ -791,8 +795,8 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
             }
             if (!resid) work_bar();                      // the rows' 1 / RMS
             if (kd == GK_LM) asm volatile("bar.arrive 3, 288;" ::: "memory");        // (whose parts come from every CTA's last result)
-            // the buffers of the layer before are empty again before anything that the next layer waits for leaves this CTA
-            if (kd == GK_DOWN) mbar_wait<1>(&jan_done, (uint32_t)l & 1u, abortp);
+            // the buffers set back in this layer are empty again before anything that their next writers wait for leaves this CTA
+            if (kd == (g.L == 1 ? GK_GU : GK_DOWN)) mbar_wait<1>(&jan_done, (uint32_t)l & 1u, abortp);
             const float* red = (const float*)(redbuf + g.k[kd].red);
             const int part_step = f_own_max * 8;
             auto sum = [&](int f) {                      // feature f of this CTA's share, this thread's row, parts in CTA order

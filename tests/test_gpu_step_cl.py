@@ -18,9 +18,9 @@ def A():
     return binding
 
 
-def _both(A, monkeypatch, shape, run):
+def _both(A, monkeypatch, shape, run, stream=None):
     """run(kv) on a handle of either kind: its results, and the kernels it launched."""
-    m = gpu_model(A, shape, make_weights(shape, 21, True), new_stream())
+    m = gpu_model(A, shape, make_weights(shape, 21, True), stream or new_stream())
     got, launches = [], []
     try:
         for chain in (True, False):
@@ -88,6 +88,33 @@ def test_sums_in_another_order(A, monkeypatch, shape):
     for a, b in zip(*_both(A, monkeypatch, shape, run)):
         # fp32 sums of two-term products (2^-17 of a term) in another order, through one layer whose cached keys and values are the same
         assert float(np.abs(a - b).max()) <= 2.0 ** -12 * max(1.0, float(np.abs(a).max()))
+
+
+# What one step leaves in the exchange buffers, the next must not find: many steps, of one layer (its down projection writes what the same
+# layer sets back) and of the fewest that alternate between the copies.
+@pytest.mark.parametrize("shape", [
+    ModelShape(1, 256, 4, 4, 64, 256, 256), ModelShape(1, 4096, 32, 32, 128, 1024, 500), ModelShape(2, 256, 2, 2, 128, 4096, 300),
+], ids=_id)
+def test_many_steps_one_after_the_other(A, monkeypatch, shape):
+    prompt = markov_prompt(200, shape.vocab, 2, 31).tolist()
+    stream = new_stream()
+
+    def run(m, kv):
+        ctx = A.anpd_ngram_create(2, 4, 1200, 0, stream)
+        res = []
+        for n, K in ((3, 0), (200, 5)):                                # one launch for all steps
+            res.append(A.anpd_generate(m, kv, ctx, prompt[:n], 900, K)[0])
+        A.anpd_ngram_destroy(ctx)
+        A.anpd_kv_truncate(kv, 0, 0)
+        last = A.anpd_prefill(m, kv, prompt)
+        for i in range(60):
+            res.append(A.anpd_verify_logits(m, kv, last, DRAFT[:i % 8], shape.vocab))
+            res.append(np.array(A.anpd_verify(m, kv, last, DRAFT[:i % 3])))
+            last = int(res[-1][1])
+        return res
+
+    for a, b in zip(*_both(A, monkeypatch, shape, run, stream)):
+        assert np.array_equal(a, b)
 
 
 # The handle of a model that takes more shared memory than the one whose handle is made after it, in either instance of the kernel (223488 and
