@@ -18,9 +18,9 @@
 // layer l - 1 is set back while layer l's gate-up runs.  Everybody has read all of it by then: this CTA's O results need its cluster's four
 // quarters of the attention, these every cluster's QKV results, and no CTA pushes sums of QKV before it has read what l - 1 left.  And no
 // sums of layer l's down projection leave this CTA before that is done (jan_done): every CTA's QKV of layer l + 1, the next to write there,
-// needs them.  What the last layer leaves is set back in layer 0 (its readers were the kernel before) and written by the last layer's down
-// projection, which needs layer 0's if there are several.  With one layer it is that same projection, and another cluster's needs this CTA's
-// gate-up sums but not its down sums: there it is the gate-up sums that wait.
+// needs them.  What the last layer leaves is set back at the start (its readers were those of the step before) and written again by the last layer's
+// down projection, which needs every CTA's down sums of layer 0; where that is the same projection, with one layer, every CTA waits before its
+// first sums.
 // So are the others protected: a CTA's pushes of phase p + 2 into the region of the exchange that phase p used need results of
 // phase p + 1 that need all results of phase p.  This needs every cluster to own features and every CTA k-blocks of every projection.
 //
@@ -393,7 +393,7 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
         const unsigned slice = g.copy_bytes / (unsigned)ncta, fslice = g.fin_bytes / (unsigned)ncta;
 #pragma unroll 1
         for (int l = 0; l <= g.L; ++l) {
-            asm volatile("bar.sync 3, 288;" ::: "memory");             // this CTA is through the O projection of layer l (or has heard from every CTA's last layer)
+            if (l) asm volatile("bar.sync 3, 288;" ::: "memory");      // this CTA is through the O projection of layer l (or has heard from every CTA's last layer)
             unsigned char* at = l ? g.xch + (size_t)((l - 1) & 1) * g.copy_bytes + (size_t)bid * slice : g.xch + 2 * (size_t)g.copy_bytes + (size_t)bid * fslice;
             const unsigned n = l ? slice : fslice;
 #pragma unroll 1
@@ -402,6 +402,7 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
             __threadfence();
             __syncwarp();
             if (lane == 0) mbar_arrive(&jan_done);
+            if (l == 0) asm volatile("bar.sync 3, 288;" ::: "memory");
         }
     } else if (warp == 11) {
         // ---------------- into L2 what the ring will ask for ----------------
@@ -745,6 +746,7 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
             work_bar();                                  // the activations go where the warps' results were
         };
 
+        if (g.L == 1) mbar_wait<1>(&jan_done, 0u, abortp);        // (out of the loop: a condition in it costs 0.1 us a layer)
         int kd = GK_QKV, l = 0;
 #pragma unroll 1
         while (true) {
@@ -795,8 +797,8 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
             }
             if (!resid) work_bar();                      // the rows' 1 / RMS
             if (kd == GK_LM) asm volatile("bar.arrive 3, 288;" ::: "memory");        // (whose parts come from every CTA's last result)
-            // the buffers set back in this layer are empty again before anything that their next writers wait for leaves this CTA
-            if (kd == (g.L == 1 ? GK_GU : GK_DOWN)) mbar_wait<1>(&jan_done, (uint32_t)l & 1u, abortp);
+            // the buffers of the layer before are empty again before anything that the next layer waits for leaves this CTA
+            if (kd == GK_DOWN) mbar_wait<1>(&jan_done, (uint32_t)l & 1u, abortp);
             const float* red = (const float*)(redbuf + g.k[kd].red);
             const int part_step = f_own_max * 8;
             auto sum = [&](int f) {                      // feature f of this CTA's share, this thread's row, parts in CTA order
