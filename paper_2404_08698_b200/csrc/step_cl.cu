@@ -18,9 +18,9 @@
 // layer l - 1 is set back while layer l's gate-up runs.  Everybody has read all of it by then: this CTA's O results need its cluster's four
 // quarters of the attention, these every cluster's QKV results, and no CTA pushes sums of QKV before it has read what l - 1 left.  And no
 // sums of layer l's down projection leave this CTA before that is done (jan_done): every CTA's QKV of layer l + 1, the next to write there,
-// needs them.  What the last layer leaves is set back at the start (its readers were those of the step before) and written again by the last layer's
-// down projection, which needs every CTA's down sums of layer 0; where that is the same projection, with one layer, every CTA waits before its
-// first sums.
+// needs them.  What the last layer leaves is set back at the start (its readers were those of the step before), ahead of this CTA's first sums of
+// QKV, which every later result needs.  The workers meet that warp at the start and, without waiting for it, behind every O projection and at the
+// vocabulary; they wait for jan_done between any two of these, so that no meeting begins before the one before is over.
 // So are the others protected: a CTA's pushes of phase p + 2 into the region of the exchange that phase p used need results of
 // phase p + 1 that need all results of phase p.  This needs every cluster to own features and every CTA k-blocks of every projection.
 //
@@ -401,8 +401,11 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
             if (l == g.L) break;                                       // (the kernel's end makes these visible)
             __threadfence();
             __syncwarp();
+            if (l == 0) {
+                asm volatile("bar.sync 3, 288;" ::: "memory");         // the workers start
+                asm volatile("bar.sync 3, 288;" ::: "memory");         // and are through the O projection
+            }
             if (lane == 0) mbar_arrive(&jan_done);
-            if (l == 0) asm volatile("bar.sync 3, 288;" ::: "memory");
         }
     } else if (warp == 11) {
         // ---------------- into L2 what the ring will ask for ----------------
@@ -486,7 +489,7 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
             cs0 = *(const float2*)(g.rope_cos + at);
             sn0 = *(const float2*)(g.rope_sin + at);
         }
-        work_bar();
+        asm volatile("bar.sync 3, 288;" ::: "memory");       // (in the place of work_bar: the last layer's results are set back too)
         cluster_wait();
         pdl_wait();                                     // what the embedding left
 #pragma unroll 1
@@ -746,7 +749,6 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
             work_bar();                                  // the activations go where the warps' results were
         };
 
-        if (g.L == 1) mbar_wait<1>(&jan_done, 0u, abortp);        // (out of the loop: a condition in it costs 0.1 us a layer)
         int kd = GK_QKV, l = 0;
 #pragma unroll 1
         while (true) {
