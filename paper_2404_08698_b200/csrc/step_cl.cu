@@ -264,7 +264,7 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
                             if (k < kps) bytes = (uint32_t)k * kb_bytes;
                             if (!mbar_wait_at<1>(full + empty_off, eph, abortp)) { ok = false; break; }
                             bulk_load_at(dst, src, bytes, full, pol_w);
-                            mbar_arrive_at(full + empty_off, WARPS - 1);       // a page's stage is given back by eight warps, a weight stage by one commit
+                            mbar_arrive_at(full + empty_off, WARPS - 1);       // a page's stage is given back by its eight or four warps, a weight stage by one commit
                             src += src_step;
                             s_requested = ++requested;
                             next();
@@ -288,6 +288,7 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
                                 if (s < KST) tma_load_2d_at(dst, &map_k, s * 64, row * KV_PAGE, full, pol_p);
                                 else if (HD == 128) tma_load_2d_at(dst, &map_v, (s - KST) * 64, row * HD, full, pol_p);
                                 else { tma_load_2d_at(dst, &map_v, 0, row * HD, full, pol_p); tma_load_2d_at(dst + HD * 128, &map_v, 64, row * HD, full, pol_p); }
+                                if (HD == 128 && s >= KST) mbar_arrive_at(full + empty_off, WARPS / 2);       // half of the warps read it and give it back
                                 s_requested = ++requested;
                                 next();
                             }
@@ -686,11 +687,9 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
                     }
                     mbar_wait<1>(&w_full[vst], vpar, abortp);
                 }
+                // only the stage that this warp has waited for: it counts towards the phase of this page, whatever lay there before
                 __syncwarp();
-                if (lane == 0) {
-#pragma unroll
-                    for (int s = KST; s < 2 * KST; ++s) mbar_arrive(&w_empty[st(s)]);
-                }
+                if (lane == 0) mbar_arrive(&w_empty[vst]);
             }
             // ---- the warps, in order ----
             l_run += __shfl_xor_sync(0xffffffffu, l_run, 1);

@@ -18,7 +18,7 @@ def A():
     return binding
 
 
-def _both(A, monkeypatch, shape, run, stream=None):
+def _both(A, monkeypatch, shape, run, stream=None, max_len=1200):
     """run(kv) on a handle of either kind: its results, and the kernels it launched."""
     m = gpu_model(A, shape, make_weights(shape, 21, True), stream or new_stream())
     got, launches = [], []
@@ -28,7 +28,7 @@ def _both(A, monkeypatch, shape, run, stream=None):
                 monkeypatch.setenv("ANPD_STEP_CHAIN", "1")
             else:
                 monkeypatch.delenv("ANPD_STEP_CHAIN")
-            kv = A.anpd_kv_create(m, 1200, 1, True)                    # shuffled pages
+            kv = A.anpd_kv_create(m, max_len, 1, True)                 # shuffled pages
             A.anpd_launch_count(True)
             got.append(run(m, kv))
             launches.append(A.anpd_launch_count())
@@ -88,6 +88,24 @@ def test_sums_in_another_order(A, monkeypatch, shape):
     for a, b in zip(*_both(A, monkeypatch, shape, run)):
         # fp32 sums of two-term products (2^-17 of a term) in another order, through one layer whose cached keys and values are the same
         assert float(np.abs(a - b).max()) <= 2.0 ** -12 * max(1.0, float(np.abs(a).max()))
+
+
+# A page of head dimension 128 is four stages of the ring, of ten, nine and eight stages here: which stage of an earlier page lies where a
+# stage goes differs from page to page.  A dozen pages per CTA, and one CTA for all of a head's.
+@pytest.mark.parametrize("shape, n", [
+    (ModelShape(2, 256, 2, 2, 128, 688, 300), 6000), (ModelShape(2, 256, 2, 2, 128, 688, 16000), 6000), (ModelShape(2, 256, 2, 2, 128, 688, 32000), 6000),
+    (ModelShape(1, 1024, 80, 10, 128, 1024, 300), 2000),
+], ids=["10", "9", "8", "one-cta"])
+def test_many_pages_through_a_short_ring(A, monkeypatch, shape, n):
+    prompt = markov_prompt(n, shape.vocab, 2, 31).tolist()
+
+    def run(m, kv):
+        last = A.anpd_prefill(m, kv, prompt)
+        return [A.anpd_verify_logits(m, kv, last, DRAFT[:i % 8], shape.vocab) for i in range(50)]
+
+    for a, b in zip(*_both(A, monkeypatch, shape, run, max_len=n + 16)):
+        # 1024 wide: sums in another order, with the bound above; else bit for bit
+        assert np.array_equal(a, b) if shape.d_model == 256 else float(np.abs(a - b).max()) <= 2.0 ** -12 * max(1.0, float(np.abs(a).max()))
 
 
 # What one step leaves in the exchange buffers, the next must not find: many steps, of one layer (its down projection writes what the same
