@@ -227,6 +227,11 @@ anpd_status anpd_verify_stage(anpd_model* m, anpd_kv* kv, const int32_t* last_to
 anpd_status anpd_verify_enqueue(anpd_model* m, anpd_kv* kv);
 anpd_status anpd_verify_result(anpd_model* m, anpd_kv* kv, int* accepted_len, int32_t* next_tok);
 
+/* Test hook: one step of a handle of batch 1 whose inputs never come.  Its waits run out after a second or two and the call
+ * returns what every later one on this handle returns, ANPD_ERR_CUDA; ANPD_ERR_STATE (and nothing is done) where the handle's
+ * steps are not one kernel. */
+anpd_status anpd_debug_lost_step(anpd_model* m, anpd_kv* kv);
+
 /* ---- Algorithm 1 ------------------------------------------------------------------------
  * prompt -> Initialize + prefill -> repeat {commit, Update, draft K, verify, accept} until
  * max_new tokens are out; the result is cut to max_new.  K == 0 is plain greedy decoding

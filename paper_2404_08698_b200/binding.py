@@ -86,6 +86,7 @@ SIGNATURES = {
     "anpd_verify_two_candidates": (C.c_int, [_P, _P, C.c_int32, _I32P, C.c_int, _I32P, C.c_int, _IP, _I32P, _IP, C.POINTER(C.c_float)]),
     "anpd_verify_stage": (C.c_int, [_P, _P, _I32P, _I32P, _IP]),
     "anpd_verify_enqueue": (C.c_int, [_P, _P]),
+    "anpd_debug_lost_step": (C.c_int, [_P, _P]),
     "anpd_verify_result": (C.c_int, [_P, _P, _IP, _I32P]),
     "anpd_generate": (C.c_int, [_P, _P, _P, _I32P, C.c_int, C.c_int, C.c_int, _I32P, _IP, C.POINTER(Stats)]),
     "anpd_generate_dev": (C.c_int, [_P, _P, _P, _P, C.c_int, C.c_int, C.c_int, _P, _IP, C.POINTER(Stats)]),
@@ -297,6 +298,10 @@ def anpd_verify_stage(m: int, kv: int, last_tok, drafts) -> None:
 
 def anpd_verify_enqueue(m: int, kv: int) -> None:
     _check(lib().anpd_verify_enqueue(_P(m), _P(kv)), "anpd_verify_enqueue")
+
+
+def anpd_debug_lost_step(m: int, kv: int) -> None:
+    _check(lib().anpd_debug_lost_step(_P(m), _P(kv)), "anpd_debug_lost_step")
 
 
 def anpd_verify_result(m: int, kv: int, batch: int = 1) -> tuple[list[int], list[int]]:

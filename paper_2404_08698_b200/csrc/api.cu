@@ -717,6 +717,16 @@ anpd_status anpd_prefill(anpd_model* m, anpd_kv* kv, int seq, const int32_t* pro
     return ANPD_OK;
 }
 
+anpd_status anpd_debug_lost_step(anpd_model* m, anpd_kv* kv) {
+    if (!m || !kv || kv->m != m) return ANPD_ERR_ARG;
+    ANPD_TRY(check_device(m));
+    if (!kv->ws.xch_bytes) return ANPD_ERR_STATE;
+    ANPD_TRY(plan_decode_enqueue(m, kv, false));
+    CUDA_TRY(cudaMemsetAsync(kv->ws.ci_h, 0xff, cl_img_bytes(ANPD_ROWS, m->cfg.d_model), m->stream));       // what a word not yet written looks like
+    ANPD_TRY(step_cl_enqueue(m, kv, false, false));
+    return read_seqs(kv);
+}
+
 // ---------------------------------------------------------------------------------------------
 // verify
 // ---------------------------------------------------------------------------------------------

@@ -45,7 +45,11 @@
 // but where products are packed (their k-blocks' sums meet at the end), beyond 4096 features (two tiles of the residual stream: a row's sum of
 // squares comes in other groups),
 // and for query heads of dimension 64 that share a kv head (a warp takes the products of one of them, not of two).
-// Every wait is bounded and reports through the error flag; a handle that has failed once refuses all further results.
+// Every wait is bounded and reports through the error flag; a handle that has failed once refuses all further results.  What can fail is to hear from
+// another CTA: a wait for the cluster's sums that runs out raises abort_flag, a poll the handle's error too, and all others of either kind look at both.
+// The CTA then goes through the rest of the step as ever, with whatever its buffers hold: ring, products and the setting back wait for nobody else,
+// are in order whatever the values, and leave no copy or product under way behind them.  Only the exchange in the cluster stops, so that no
+// barrier is counted on that has not come round.
 #include "step_dev.cuh"
 
 #include <algorithm>
@@ -142,6 +146,32 @@ __device__ __forceinline__ void tc_ld4_sum(uint32_t hi, uint32_t lo, float* v) {
 #pragma unroll
     for (int i = 0; i < 4; ++i) v[i] = __uint_as_float(a[i]) + __uint_as_float(b[i]);
 }
+// Bounded wait for something in this CTA, not begun where another one has run out.  (The flag is read ahead of the loop: 1.1B 515 -> 509 us per step.)
+__device__ __forceinline__ bool sc_wait_at(uint32_t bar, uint32_t parity, volatile int* stuck_flag) {
+    if (mbar_try_wait_at(bar, parity)) return true;
+    if (*stuck_flag) return false;
+#pragma unroll 1
+    for (unsigned i = 0; i < WAIT_LIMIT; ++i)
+        if (mbar_try_wait_at(bar, parity)) return true;
+    *stuck_flag = 1;
+    return false;
+}
+__device__ __forceinline__ bool sc_wait(uint64_t* bar, uint32_t parity, volatile int* stuck_flag) { return sc_wait_at(smem_u32(bar), parity, stuck_flag); }
+// Bounded wait for what other CTAs of the cluster send: ends as soon as anybody in this CTA has given up, and soon after anybody at all has.
+__device__ __forceinline__ void sc_wait_cluster(uint64_t* bar, uint32_t parity, volatile int* abort_flag, volatile int* err) {
+#pragma unroll 1
+    for (unsigned i = 0; i < WAIT_LIMIT; ++i) {
+        uint32_t ok;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
+        if (ok) return;
+        if (*abort_flag || ((i & 255u) == 255u && *err)) break;
+    }
+    *abort_flag = 1;
+}
 __device__ __forceinline__ void fence_async_cta() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
 // Units of tile t of a cluster's Uc.  Each rank finishes a quarter of every tile's units, the quarters taking turns.
@@ -158,7 +188,7 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
     __shared__ uint64_t acc_full[SC_MAX_TILES], red_full[2][SC_MAX_TILES], att_full, jan_done;
     __shared__ uint32_t tmem_slot;
     __shared__ volatile int s_requested, s_phase, s_quit;         // copies of weights requested so far; all of them, or none will follow
-    __shared__ int abort_flag, s_issued;
+    __shared__ int abort_flag, stuck_flag, s_issued;    // another CTA was not heard from; a wait inside this CTA ran out
     __shared__ float s_rstd[8], s_part[8][8];
     __shared__ int s_pos[8], s_slot[8], s_page[8], s_raw[8], s_idx[8][8];
     __shared__ ScGeo s_geo[GK_COUNT];
@@ -174,7 +204,7 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
     float2* s_x = (float2*)(redbuf + g.red_bytes);      // this CTA's part of the residual stream, in pairs
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int bid = (int)blockIdx.x, rank = bid % CC, cluster = bid / CC, ncta = g.ncl * CC;
-    volatile int* abortp = &abort_flag;
+    volatile int *abortp = &abort_flag, *stuckp = &stuck_flag;
 
     pdl_trigger();
     if (threadIdx.x < GK_COUNT) {                       // how this cluster and CTA cut each projection
@@ -205,7 +235,7 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
         s_geo[threadIdx.x] = e;
     }
     if (threadIdx.x == 64) {
-        abort_flag = 0; s_issued = 0; s_requested = 0; s_phase = 0; s_quit = 0;
+        abort_flag = 0; stuck_flag = 0; s_issued = 0; s_requested = 0; s_phase = 0; s_quit = 0;
 #pragma unroll 1
         for (int s = 0; s < g.stages; ++s) { mbar_init(&w_full[s], 1); mbar_init(&w_empty[s], WARPS); }
         for (int s = 0; s < SC_ACT_SLOTS; ++s) { mbar_init(&a_full[s], 8); mbar_init(&a_empty[s], 1); }
@@ -262,7 +292,7 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
 #pragma unroll 1
                         for (int k = kn; k > 0; k -= kps) {
                             if (k < kps) bytes = (uint32_t)k * kb_bytes;
-                            if (!mbar_wait_at<1>(full + empty_off, eph, abortp)) { ok = false; break; }
+                            if (!sc_wait_at(full + empty_off, eph, stuckp)) { ok = false; break; }
                             bulk_load_at(dst, src, bytes, full, pol_w);
                             mbar_arrive_at(full + empty_off, WARPS - 1);       // a page's stage is given back by its eight or four warps, a weight stage by one commit
                             src += src_step;
@@ -283,7 +313,7 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
                             const int row = (l * g.total_pages + pages[p]) * g.Hkv + kvh;
 #pragma unroll 1
                             for (int s = 0; s < 2 * KST; ++s) {
-                                if (!mbar_wait_at<1>(full + empty_off, eph, abortp)) { ok = false; break; }
+                                if (!sc_wait_at(full + empty_off, eph, stuckp)) { ok = false; break; }
                                 mbar_expect_tx_at(full, SC_STAGE);
                                 if (s < KST) tma_load_2d_at(dst, &map_k, s * 64, row * KV_PAGE, full, pol_p);
                                 else if (HD == 128) tma_load_2d_at(dst, &map_v, (s - KST) * 64, row * HD, full, pol_p);
@@ -317,7 +347,6 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
             const uint32_t af0 = smem_u32(&a_full[0]), aempty_off = smem_u32(&a_empty[0]) - af0, af_end = af0 + 8u * SC_ACT_SLOTS;
             uint32_t afull = af0, aph = 0;
             uint64_t a_d = act_d;
-            // A wait that gave up has set the abort flag; the loops run on with whatever the buffers hold (every later wait is short then).
             auto next_stage = [&]() {
                 tc_commit_at(full + empty_off);
                 w_d += stage_step;
@@ -340,13 +369,13 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
                         uint64_t ad = a_d;
 #pragma unroll 1
                         for (int ks = 0; ks < kn; ks += SC_AKB) {
-                            if (t == 0) { mbar_wait_at<1>(af, ap, abortp); tc_fence_after(); }
+                            if (t == 0) { sc_wait_at(af, ap, stuckp); tc_fence_after(); }
                             const int kend = min(SC_AKB, kn - ks);
                             uint64_t a = ad;
                             // a tile of fewer than 16 groups: the instruction reads whatever follows for the rows beyond, whose lanes nobody reads
 #pragma unroll 1
                             for (int k = 0; k < kend; k += kps) {
-                                mbar_wait_at<1>(full, wph, abortp);
+                                sc_wait_at(full, wph, stuckp);
                                 tc_fence_after();
                                 const int n = min(kps, kend - k);
                                 // packed: the stage's k-blocks are rows of one product, side by side, and its columns are the activations of all of
@@ -507,8 +536,8 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
         };
         adv(s_geo[GK_QKV].n_st);
         auto gave_up = [&](unsigned i) {                // a poll that lasts: has anybody failed?
-            if ((i & 1023u) != 1023u) return false;
-            if (*abortp || *(volatile int*)g.err || i >= SC_POLL_LIMIT) { *abortp = 1; return true; }
+            if ((i & 255u) != 255u) return false;
+            if (*abortp || *(volatile int*)g.err || i >= SC_POLL_LIMIT) { *abortp = 1; *(volatile int*)g.err = SC_ERR_TIMEOUT; return true; }
             return false;
         };
 
@@ -517,7 +546,7 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
             const int nk = s_geo[kd].nk, kb_lo = s_geo[kd].kb_lo, K = g.k[kd].K;
 #pragma unroll 1
             for (int k0 = 0; k0 < nk; k0 += SC_AKB) {
-                if (a_count >= SC_ACT_SLOTS) mbar_wait<1>(&a_empty[a_slot], a_ph, abortp);
+                if (a_count >= SC_ACT_SLOTS) sc_wait(&a_empty[a_slot], a_ph, stuckp);
                 const int chunks = min(SC_AKB, nk - k0) * 128;                       // of 16 bytes
                 const unsigned char* src = img + (size_t)(kb_lo + k0) * (rows * 256) + ft * 16;
                 unsigned char* dst = abuf + a_slot * SC_ACT_SLOT + ft * 16;
@@ -597,11 +626,11 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
                 p_par = par(2 * KST);
                 p_st = st(2 * KST);
 #pragma unroll
-                for (int s = 0; s < KST; ++s) mbar_wait<1>(&w_full[st(s)], par(s), abortp);
+                for (int s = 0; s < KST; ++s) sc_wait(&w_full[st(s)], par(s), stuckp);
                 const int vs = HD == 128 ? KST + (key_page >> 6) : KST;
                 if (p >= first_new) {                   // the cache's page is from before this step: the step's own rows go in here
 #pragma unroll
-                    for (int s = KST; s < 2 * KST; ++s) mbar_wait<1>(&w_full[st(s)], par(s), abortp);
+                    for (int s = KST; s < 2 * KST; ++s) sc_wait(&w_full[st(s)], par(s), stuckp);
                     const int slot = s_slot[nr];
                     if (has_n && slot >= 0 && slot / KV_PAGE == p) {
                         const int at = slot % KV_PAGE, box = at >> 6;
@@ -671,7 +700,7 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
 #pragma unroll
                         for (int d = 0; d < DT; ++d) { o[d][0] *= resc; o[d][1] *= resc; o[d][2] *= resc; o[d][3] *= resc; }
                     }
-                    mbar_wait<1>(&w_full[vst], vpar, abortp);
+                    sc_wait(&w_full[vst], vpar, stuckp);
                     const uint32_t vr = ring_addr + (uint32_t)vst * SC_STAGE + kv_off + (HD == 128 ? 0u : (uint32_t)((key_page >> 6) * (HD * 128))) + ((((uint32_t)((key_page & 63) >> 3) + chunk0) ^ (uint32_t)lr) << 4);
 #pragma unroll
                     for (int d = 0; d < DT / 2; ++d) {
@@ -685,7 +714,7 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
 #pragma unroll
                         for (int s = 0; s < KST; ++s) mbar_arrive(&w_empty[st(s)]);
                     }
-                    mbar_wait<1>(&w_full[vst], vpar, abortp);
+                    sc_wait(&w_full[vst], vpar, stuckp);
                 }
                 // only the stage that this warp has waited for: it counts towards the phase of this page, whatever lay there before
                 __syncwarp();
@@ -731,9 +760,9 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
                 if (d4 == 0) st_async2(map_to_cta(smem_u32(&rc[at]), cta), bar, mx, lsum);
             }
             if (g.C > 1) {
-                mbar_wait_cluster(&att_full, att_par, abortp);
+                sc_wait_cluster(&att_full, att_par, abortp, g.err);
                 att_par ^= 1u;
-                if (ft == 0 && l + 1 < g.L) mbar_expect_tx(&att_full, (uint32_t)(g.C * VO * (HD * 4 + 8)));
+                if (ft == 0 && l + 1 < g.L && !*abortp) mbar_expect_tx(&att_full, (uint32_t)(g.C * VO * (HD * 4 + 8)));
 #pragma unroll 1
                 for (int idx = ft; idx < VO * V4; idx += SC_WORKERS) {
                     const int vo = idx / V4, d4 = idx % V4;
@@ -765,7 +794,7 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
                 gain = kd == GK_O ? (const float*)((const char*)g.ffn_norm + (size_t)l * g.layer_step) : l + 1 < g.L ? (const float*)((const char*)g.attn_norm + (size_t)(l + 1) * g.layer_step) : g.final_norm;
                 if (ft < s_own[kd] * 32) gn = *(const float2*)(gain + resid_feature(ft));
             }
-            if (ft < T) {                                // what the cluster will send here for each tile
+            if (ft < T && !*abortp) {                    // what the cluster will send here for each tile
                 const int n = s_tile[kd][ft].own_n;
                 mbar_expect_tx(&red_full[region][ft], (uint32_t)(n ? (n << shift) * CC * pack * 32 : CC * 16));
             }
@@ -799,7 +828,7 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
             if (!resid) work_bar();                      // the rows' 1 / RMS
             if (kd == GK_LM) asm volatile("bar.arrive 3, 288;" ::: "memory");        // (whose parts come from every CTA's last result)
             // the buffers of the layer before are empty again before anything that the next layer waits for leaves this CTA
-            if (kd == GK_DOWN) mbar_wait<1>(&jan_done, (uint32_t)l & 1u, abortp);
+            if (kd == GK_DOWN) sc_wait(&jan_done, (uint32_t)l & 1u, stuckp);
             const float* red = (const float*)(redbuf + g.k[kd].red);
             const int part_step = f_own_max * 8;
             auto sum = [&](int f) {                      // feature f of this CTA's share, this thread's row, parts in CTA order
@@ -814,7 +843,7 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
             const float rs = resid ? 1.0f : s_rstd[row];
             auto finish = [&](int t) {
                 const int lo = s_tile[kd][t].before[rank] * (kd == GK_LM ? 64 : 32), hi_ = lo + s_tile[kd][t].own_n * (kd == GK_LM ? 64 : 32);
-                mbar_wait_cluster(&red_full[region][t], (red_par >> (region * SC_MAX_TILES + t)) & 1u, abortp);
+                sc_wait_cluster(&red_full[region][t], (red_par >> (region * SC_MAX_TILES + t)) & 1u, abortp, g.err);
 #pragma unroll 1
                 for (int idx = lo + ((ft - lo) & (SC_WORKERS - 1)); idx < hi_; idx += SC_WORKERS) {
                     if (resid) {
@@ -907,15 +936,16 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
                     const int un = s_tile[kd][t].groups >> (shift - 3), pos = quad * 32 + lane - part * lanes, u = pos >> shift;
                     const int b1 = un / 4, b2 = un / 2, b3 = 3 * un / 4, q = (u >= b1) + (u >= b2) + (u >= b3), owner = (q - t) & (CC - 1);
                     const int local = ((s_tile[kd][t].before[owner] + u - (q * un) / CC) << shift) + (pos & ((1 << shift) - 1));
-                    mbar_wait<1>(&acc_full[t], (acc_par >> t) & 1u, abortp);
+                    const bool send = !*abortp;
+                    sc_wait(&acc_full[t], (acc_par >> t) & 1u, stuckp);
                     tc_fence_after();
                     float v[4];
                     const uint32_t col = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)((t + part) * 2 * rows + (pushes ? 0 : 4));
                     tc_ld4_sum(col, col + 8u, v);
                     const uint32_t bar0 = smem_u32(&red_full[region][t]), to = red_addr + (uint32_t)(g.k[kd].red + ((part * CC + rank) * f_own_max + local) * 32 + (pushes ? 0 : 16));
-                    if (pos < lanes) st_async4(map_to_cta(to, (uint32_t)owner), map_to_cta(bar0, (uint32_t)owner), v[0], v[1], v[2], v[3]);
+                    if (pos < lanes && send) st_async4(map_to_cta(to, (uint32_t)owner), map_to_cta(bar0, (uint32_t)owner), v[0], v[1], v[2], v[3]);
                     // a CTA that finishes nothing of the tile hears from the others all the same: it is then behind them
-                    if (ft < CC && (ft + 1) * un / CC == ft * un / CC) {
+                    if (ft < CC && send && (ft + 1) * un / CC == ft * un / CC) {
                         const uint32_t o = (uint32_t)((ft - t) & (CC - 1));
                         st_async4(map_to_cta(red_addr + (uint32_t)(g.k[kd].red + rank * 16), o), map_to_cta(bar0, o), 0.f, 0.f, 0.f, 0.f);
                     }
@@ -970,13 +1000,15 @@ __global__ void __launch_bounds__(SC_THREADS, 1) step_cl_kernel(const __grid_con
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"((uint32_t)g.tmem_cols) : "memory");
     }
-    if (threadIdx.x == 0 && abort_flag) {
+    if (threadIdx.x == 0 && (abort_flag || stuck_flag)) {
         // gave up: let every copy already issued land before the CTA may exit
 #pragma unroll 1
         for (int i = max(0, s_issued - g.stages); i < s_issued; ++i)
 #pragma unroll 1
             for (unsigned spin = 0; spin < WAIT_LIMIT && !mbar_try_wait(&w_full[i % g.stages], (uint32_t)((i / g.stages) & 1)); ++spin) {}
         atomicExch(g.err, SC_ERR_TIMEOUT);
+#pragma unroll 1
+        for (int i = 0; i < 20; ++i) __nanosleep(20000);        // ... and what went to the cluster's other CTAs, for which nobody may be waiting, arrive
     }
     __syncwarp();
     cluster_arrive();

@@ -1,5 +1,7 @@
 """A single sequence's step as one kernel (csrc/step_cl.cu) against the same step as a kernel per projection, which the other tests
 hold to the oracle."""
+import time
+
 import numpy as np
 import pytest
 
@@ -163,6 +165,29 @@ def test_handles_of_two_models_do_not_disturb_each_other(A, first, second):
             A.anpd_kv_destroy(kv)
         for m in models:
             A.anpd_model_destroy(m)
+
+
+# A step whose inputs never come ends by itself, soon, and with an error that stays with its handle.
+@pytest.mark.parametrize("shape", [
+    ModelShape(2, 256, 4, 4, 64, 256, 256), ModelShape(16, 2048, 16, 16, 128, 2048, 8000),
+], ids=_id)
+def test_a_step_that_hears_nothing(A, shape):
+    m = gpu_model(A, shape, make_weights(shape, 21, True), new_stream())
+    kvs = [A.anpd_kv_create(m, 600) for _ in range(2)]
+    try:
+        last = [A.anpd_prefill(m, kv, markov_prompt(500, shape.vocab, 2, 31).tolist()) for kv in kvs][0]
+        want = [A.anpd_verify_logits(m, kv, last, DRAFT, shape.vocab) for kv in kvs][0]
+        t0 = time.perf_counter()
+        with pytest.raises(A.AnpdError, match="209"):
+            A.anpd_debug_lost_step(m, kvs[0])
+        assert time.perf_counter() - t0 < 20.0                         # 2^21 polls, and what is left of the step
+        with pytest.raises(A.AnpdError, match="209"):
+            A.anpd_verify_logits(m, kvs[0], last, DRAFT, shape.vocab)
+        assert np.array_equal(A.anpd_verify_logits(m, kvs[1], last, DRAFT, shape.vocab), want)
+    finally:
+        for kv in kvs:
+            A.anpd_kv_destroy(kv)
+        A.anpd_model_destroy(m)
 
 
 def test_a_kernel_per_projection_under_nsight_compute(A, monkeypatch):
