@@ -28,6 +28,11 @@
  *     the CUDA stream given at creation (0 = the default stream).  Calls that return results
  *     in host memory synchronise that stream before returning; calls marked "asynchronous"
  *     only enqueue work.
+ *   - A step of one sequence is for most shapes a single kernel, launched cooperatively: its blocks (128 on a
+ *     B200, each with an SM to itself) wait for one another, so that it starts when so many SMs are free at one moment.
+ *     Steps of several models on one GPU therefore take turns.  A program that keeps a kernel of its own on
+ *     more than 20 of a B200's 148 SMs until a step has ended has to create its kv handles with ANPD_STEP_CHAIN=1 in the
+ *     environment: such a handle steps with a kernel per projection, whose blocks wait for their own cluster of four only.
  *   - There is no CPU implementation behind any of these calls: without a CUDA device
  *     every call that needs one returns ANPD_ERR_CUDA.
  *   - Limits: draft length K <= ANPD_K_MAX (a step verifies at most K+1 = 8 rows per
@@ -227,7 +232,7 @@ anpd_status anpd_verify_stage(anpd_model* m, anpd_kv* kv, const int32_t* last_to
 anpd_status anpd_verify_enqueue(anpd_model* m, anpd_kv* kv);
 anpd_status anpd_verify_result(anpd_model* m, anpd_kv* kv, int* accepted_len, int32_t* next_tok);
 
-/* Test hook: one step of a handle of batch 1 whose inputs never come.  Its waits run out after a second or two and the call
+/* Test hook: one step of a handle of batch 1 whose inputs never come.  Its waits run out within seconds and the call
  * returns what every later one on this handle returns, ANPD_ERR_CUDA; ANPD_ERR_STATE (and nothing is done) where the handle's
  * steps are not one kernel. */
 anpd_status anpd_debug_lost_step(anpd_model* m, anpd_kv* kv);

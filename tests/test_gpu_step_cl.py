@@ -1,6 +1,7 @@
 """A single sequence's step as one kernel (csrc/step_cl.cu) against the same step as a kernel per projection, which the other tests
 hold to the oracle."""
 import time
+from concurrent.futures import ThreadPoolExecutor
 
 import numpy as np
 import pytest
@@ -160,6 +161,37 @@ def test_handles_of_two_models_do_not_disturb_each_other(A, first, second):
         for _ in range(2):
             for m, kv, shape, alone in zip(models, kvs, (first, second), want):
                 assert all(np.array_equal(x, y) for x, y in zip(steps(m, kv, shape.vocab), alone))
+    finally:
+        for kv in kvs:
+            A.anpd_kv_destroy(kv)
+        for m in models:
+            A.anpd_model_destroy(m)
+
+
+def test_two_models_step_at_the_same_time(A):
+    """Either model's kernel needs most of the GPU: on two streams, from two threads, they take turns."""
+    shapes = [ModelShape(3, 512, 8, 8, 64, 1376, 2000), ModelShape(2, 1024, 8, 8, 128, 2816, 3000)]
+    models, kvs = [], []
+    try:
+        for shape in shapes:
+            models.append(gpu_model(A, shape, make_weights(shape, 21, True), new_stream()))
+            kvs.append(A.anpd_kv_create(models[-1], 512))
+
+        def steps(i):
+            res = []
+            for _ in range(20):
+                A.anpd_kv_truncate(kvs[i], 0, 0)
+                last = A.anpd_prefill(models[i], kvs[i], [1, 2, 3])
+                for k in range(30):                                    # the first are launched, the others replay a graph
+                    res.append(A.anpd_verify_logits(models[i], kvs[i], last, DRAFT[:k % 8], shapes[i].vocab))
+                    last = A.anpd_verify(models[i], kvs[i], last, DRAFT[:k % 3])[1]
+            return res
+
+        alone = [steps(i) for i in range(2)]
+        with ThreadPoolExecutor(2) as pool:
+            together = list(pool.map(steps, range(2)))
+        for a, b in zip(alone, together):
+            assert all(np.array_equal(x, y) for x, y in zip(a, b))
     finally:
         for kv in kvs:
             A.anpd_kv_destroy(kv)
