@@ -5,6 +5,7 @@ from concurrent.futures import ThreadPoolExecutor
 
 import numpy as np
 import pytest
+import torch
 
 from helpers import gpu_model, new_stream, require_gpu
 from workloads import ModelShape, make_weights, markov_prompt
@@ -21,9 +22,9 @@ def A():
     return binding
 
 
-def _both(A, monkeypatch, shape, run, stream=None, max_len=1200):
+def _both(A, monkeypatch, shape, run, stream=None, max_len=1200, weights=None):
     """run(kv) on a handle of either kind: its results, and the kernels it launched."""
-    m = gpu_model(A, shape, make_weights(shape, 21, True), stream or new_stream())
+    m = gpu_model(A, shape, weights or make_weights(shape, 21, True), stream or new_stream())
     got, launches = [], []
     try:
         for chain in (True, False):
@@ -91,6 +92,56 @@ def test_sums_in_another_order(A, monkeypatch, shape):
     for a, b in zip(*_both(A, monkeypatch, shape, run)):
         # fp32 sums of two-term products (2^-17 of a term) in another order, through one layer whose cached keys and values are the same
         assert float(np.abs(a - b).max()) <= 2.0 ** -12 * max(1.0, float(np.abs(a).max()))
+
+
+# Words that are all ones mean "not written yet" between the CTAs: infinities and NaN of that pattern go through a step like any other value.
+@pytest.mark.parametrize("where", ["embed", "l1.attn_norm", "l1.ffn_norm", "final_norm", "l0.wv"])
+@pytest.mark.parametrize("shape", [ModelShape(3, 328, 6, 6, 64, 904, 1037), ModelShape(2, 512, 4, 4, 128, 1000, 5000)], ids=_id)
+def test_infinities_and_nan(A, monkeypatch, shape, where):
+    w = make_weights(shape, 21, True)
+    ones = {2: torch.tensor([-1], dtype=torch.int16).view(torch.bfloat16), 4: torch.tensor([-1], dtype=torch.int32).view(torch.float32)}
+    t = w[where]
+    if where == "embed":
+        t[7, 3], t[9, 4:6], t[2, 5] = float("inf"), ones[2], float("-inf")
+    elif t.dim() == 2:
+        t[5, 11] = float("inf")
+    else:
+        t[8:10], t[17] = ones[4], float("-inf")
+
+    def run(m, kv):
+        res = []
+        for n in (3, 126, 300):
+            A.anpd_kv_truncate(kv, 0, 0)
+            A.anpd_prefill(m, kv, markov_prompt(n, shape.vocab, 2, 31).tolist())
+            for k in (7, 0, 3):                                        # the rows' keys and values stay in the cache
+                res.append(A.anpd_verify_logits(m, kv, 3, DRAFT[:k], shape.vocab))
+                A.anpd_verify(m, kv, 3, DRAFT[:k])
+        return res
+
+    chain, one = _both(A, monkeypatch, shape, run, weights=w)
+    assert any(np.isnan(a).any() for a in chain)
+    for a, b in zip(chain, one):
+        assert np.array_equal(a, b, equal_nan=True)
+
+
+# Two-tile and packed projections and grouped heads of dimension 64 over several layers: the step's results against the chain's.  A layer
+# changes what it is given by no more than rounding; sums in another order differ by 2^-17 of a term, of which the residual stream holds three per layer.
+@pytest.mark.parametrize("shape", [ModelShape(4, 2048, 32, 4, 64, 5632, 3200), ModelShape(3, 5120, 40, 40, 128, 1024, 500)], ids=_id)
+def test_several_layers_in_another_order(A, monkeypatch, shape):
+    prompt = markov_prompt(600, shape.vocab, 2, 31).tolist()
+
+    def run(m, kv):
+        res = []
+        for n in (9, 128, 590):
+            A.anpd_kv_truncate(kv, 0, 0)
+            A.anpd_prefill(m, kv, prompt[:n])
+            for k in (7, 2, 7):
+                res.append(A.anpd_verify_logits(m, kv, 3, DRAFT[:k], shape.vocab))
+        return res
+
+    for a, b in zip(*_both(A, monkeypatch, shape, run)):
+        # the step's own keys and values are rounded to bf16: a sum next to a boundary falls to either side, 2^-8 of that one element
+        assert float(np.abs(a - b).max()) <= 2.0 ** -9 * max(1.0, float(np.abs(a).max()))
 
 
 # A page of head dimension 128 is four stages of the ring, of ten, nine and eight stages here: which stage of an earlier page lies where a
@@ -241,3 +292,10 @@ def test_a_kernel_per_projection_under_nsight_compute(A, monkeypatch):
     finally:
         A.anpd_model_destroy(m)
     assert launches[0] == launches[1]
+
+
+def test_the_one_kernel_elsewhere(A, monkeypatch):
+    """The shape of the test above, with neither variable: fewer kernels than with either."""
+    monkeypatch.delenv("NV_COMPUTE_PROFILER_PERFWORKS_DIR", raising=False)
+    shape = ModelShape(1, 256, 4, 4, 64, 256, 256)
+    _both(A, monkeypatch, shape, lambda m, kv: [A.anpd_verify(m, kv, A.anpd_prefill(m, kv, [1, 2, 3]), DRAFT[:3])])

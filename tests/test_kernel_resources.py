@@ -18,3 +18,7 @@ def test_no_register_spills(source):
     kernels = re.findall(r"Compiling entry function '(\w+)'(?:.*\n)*?.*?(\d+) bytes spill stores, (\d+) bytes spill loads", r.stderr)
     assert kernels
     assert [k for k in kernels if k[1] != "0" or k[2] != "0"] == []
+
+
+def test_no_register_spills_in_the_one_kernel_step():
+    test_no_register_spills("step_cl.cu")
