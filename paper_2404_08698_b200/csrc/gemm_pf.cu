@@ -271,10 +271,10 @@ gemm_pf_kernel(const unsigned char* __restrict__ w, const __grid_constant__ CUte
 
 // Cycles on the busiest CTA when the work items go to the CTAs round robin, and of the partial sums' way through memory.  The gate-up
 // projection's are counted like the others', although it finishes the tiles that are left whole: a credit for that left tiles whole
-// where they fill few SMs, and what eight warps per SM then do behind the last product costs more than the kernel it saves.  us per
-// prompt with the credit and without: 7B (8 layers) 140 tokens 1580 and 1470, 1.1B 200 tokens 2365 and 2235, 512 wide (8 layers) 290
-// tokens 574 and 472, 4096 wide with 14336 gate features (8 layers) 370 tokens 2610 and 2390; the other way at 200 tokens of the tiny model (126 and 130) and 300 of the
-// last one (2290 and 2360); from 600 rows on the two cut alike nearly everywhere.
+// where they fill few SMs, and what sixteen warps per SM then do behind the last product costs more than the kernel it saves.  us per
+// prompt with the credit and without: 7B (8 layers) 140 tokens 1585 and 1489, 1.1B 200 tokens 2000 and 1915, 512 wide (8 layers) 290
+// tokens 568 and 503, 4096 wide with 14336 gate features (8 layers) 370 tokens 2790 and 2640 (runs differ by 4 %); equal within the runs' spread at 200 tokens of the
+// tiny model and 300 of the last one; from 600 rows on the two cut alike nearly everywhere.
 static long long pf_cost(int n_ft, int rows, int k_blocks, int num_sms, const PfSchedule& s) {
     const int T = pf_tile_rows(rows, s.n_tt), n_ot = n_ft * s.n_tt, boxes = (T + 63) / 64;
     // a k-block: 16 products of T / 2 cycles, or its bytes at about 48 a cycle and SM; an item: its epilogue and about a microsecond
