@@ -62,7 +62,7 @@ using namespace tc;
 constexpr int SC_THREADS = 384;          // warp 0: weights and pages, 1: products, 2: exchange buffers, 3-10: workers, 11: L2 prefetch
 constexpr int SC_WORKERS = 256;
 constexpr int SC_STAGE = 16384;          // one slot of the ring: at most 16 groups of 8 features x 64 inputs, or part of a page
-constexpr int SC_MAX_STAGES = 12;
+constexpr int SC_MAX_STAGES = 10;        // (what the shared memory holds beside the activations)
 constexpr int SC_SMEM = 220 * 1024;      // of dynamic shared memory; the static arrays take 7 KB
 constexpr int SC_AKB = 8, SC_ACT_SLOTS = 3;      // k-blocks of an activation slot, slots
 constexpr int SC_ACT_SLOT = SC_AKB * ANPD_ROWS * 256;
